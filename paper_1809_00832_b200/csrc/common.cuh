@@ -127,6 +127,13 @@ struct treelstm {
   int tc_resident_ctas = 0;             // CTAs of the grid-wide bf16 kernel the device holds at once
   bool tail_skip = false;               // the last forward whose control block was read back had no tail worth a hand-over
 
+  // TreeRNN / RNTN: how the tree kernels (rec_trees.cu) run for the context's sizes
+  struct RecTrees {
+    bool ok = false;
+    int cs = 1, Q = 0, R = 0, JS = 0, SP = 0, max_nodes = 0;   // cluster size, product rows, rows, units per CTA, row stride
+    float* W = nullptr;      // RNTN: [R][H], symmetric products added up (TreeRNN: Wcat as it is)
+  } rt;
+
   tl::Options opt;
 
   // what the last forward call saw (needed by roots / backward / status_sync)
@@ -195,6 +202,13 @@ int launch_forward_rec(treelstm* ctx, int n, const int32_t* left, const int32_t*
                        float* h, const int32_t* order, const int32_t* level_offset_dev,
                        const int32_t* level_offset_host, int n_levels_host, int flags, void* ws,
                        const WsLayout& lay, cudaStream_t stream);
+
+// rec_trees.cu (TreeRNN / RNTN, trees dealt out to clusters)
+int init_rec_trees(treelstm* ctx, cudaStream_t stream);
+int launch_forward_rec_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token,
+                             float* h, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
+int launch_backward_rec_trees(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb_rows, const int* tok_slot,
+                              cudaStream_t stream);
 
 // gemm_tc.cu
 int pack_weights_bf16(treelstm* ctx, cudaStream_t stream);
