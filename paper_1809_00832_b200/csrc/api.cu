@@ -62,6 +62,8 @@ int copy_params(treelstm* ctx, const float* emb, const float* W, const float* b,
     int rc = pack_weights_bf16(ctx, s);
     if (rc != TREELSTM_OK) return rc;
   }
+  const int rc = init_trees(ctx, s);
+  if (rc != TREELSTM_OK) return rc;
   TL_CUDA(ctx, cudaStreamSynchronize(s));
   return TREELSTM_OK;
 }
@@ -248,7 +250,7 @@ int treelstm_create_recursive(treelstm_t** out, int cell, int H, int vocab, cons
       cudaMemcpyAsync(ctx->b, b, sizeof(float) * Hs, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return fail(TREELSTM_ERR_CUDA);
   rc = pack_weights_rec(ctx, W, V, s);
-  if (rc == TREELSTM_OK) rc = init_rec_trees(ctx, s);
+  if (rc == TREELSTM_OK) rc = init_trees(ctx, s);
   if (rc != TREELSTM_OK) return fail(rc);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(TREELSTM_ERR_CUDA);
   *out = ctx;
@@ -616,7 +618,8 @@ int treelstm_last_cuda_error(const treelstm_t* ctx) { return ctx ? ctx->cuda_err
 
 int treelstm_destroy(treelstm_t* ctx) {
   if (!ctx) return TREELSTM_OK;
-  cudaFree(ctx->emb); cudaFree(ctx->W); cudaFree(ctx->b); cudaFree(ctx->Wc); cudaFree(ctx->bc); cudaFree(ctx->Wcat); cudaFree(ctx->rt.W);
+  cudaFree(ctx->emb); cudaFree(ctx->W); cudaFree(ctx->b); cudaFree(ctx->Wc); cudaFree(ctx->bc); cudaFree(ctx->Wcat); 
+  cudaFree(ctx->trees.Wf); cudaFree(ctx->trees.Wb); cudaFree(ctx->trees.pairs);
   cudaFree(ctx->emb_bf); cudaFree(ctx->Wp_h); cudaFree(ctx->Wp_x); cudaFree(ctx->bp_h); cudaFree(ctx->bp_x);
   if (ctx->host_level_offset) cudaFreeHost(ctx->host_level_offset);
   if (ctx->host_status) cudaFreeHost(ctx->host_status);

@@ -890,6 +890,68 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
   TL_STAMP(trace, kTraceLevels - 1, 8);
 }
 
+// What precedes the walk over the trees (trees_fp32.cu), in one cooperative launch: outputs cleared | leaf tokens
+// marked | tokens counted beside the classifier | tokens placed.  The level table stays on the device.
+struct GradSizes { size_t dW, db, dV; };   // floats
+__global__ void __launch_bounds__(256, 2)
+k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, long long wait_limit) {
+  extern __shared__ float s_cls[];
+  __shared__ __align__(16) unsigned int s_mask[1024];
+  __shared__ int s_flag;
+  // the kernel behind this one may set itself up: it waits for this grid before it reads dh
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (ld_volatile(&p.st->status) != 0) return;
+  const int n_levels = p.st->n_levels, H = p.H, C = p.C;
+  p.n_leaves = n_levels > 0 ? level_offset[1] : 0;
+  const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, gthreads = (size_t)gridDim.x * blockDim.x;
+  unsigned int arrivals = 0;
+  auto barrier = [&]() {
+    arrivals += gridDim.x;
+    return grid_barrier(p.st, arrivals, wait_limit, &s_flag, true, &p.st->barrier_bwd);
+  };
+  if (gtid == 0) { *p.loss = 0.f; *p.n_touched = 0; }
+  zero_range(p.dW, sizes.dW, gtid, gthreads);
+  zero_range(p.db, sizes.db, gtid, gthreads);
+  zero_range(dV, sizes.dV, gtid, gthreads);
+  zero_range(p.dWc, (size_t)H * C, gtid, gthreads);
+  zero_range(p.dbc, (size_t)C, gtid, gthreads);
+  zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
+  zero_range(p.dEmb_rows, (size_t)p.n_leaves * p.E, gtid, gthreads);
+  if (!barrier()) return;
+  for (size_t r = gtid; r < (size_t)p.n_leaves; r += gthreads)
+    p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[r], p.n)], p.vocab)] = 1;
+  if (!barrier()) return;
+  int* const group_count = p.tok_slot + p.vocab + 4;
+  if (gridDim.x == 1) {
+    scan_tokens(p, s_mask, 1024);
+    classifier_groups(p, 0, 1, s_cls);
+  } else {
+    scan_count_groups(p, group_count);
+    classifier_groups(p, blockIdx.x, gridDim.x, s_cls);
+    if (!barrier()) return;
+    scan_place_groups(p, group_count);
+  }
+}
+
+int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, cudaStream_t stream) {
+  const size_t smem = sizeof(float) * ((size_t)p.H * p.C + p.C);
+  if (smem > 160 * 1024) return TREELSTM_ERR_UNSUPPORTED;
+  if (smem > 40 * 1024)
+    TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_begin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_begin, 256, smem));
+  if (per_sm < 1) return TREELSTM_ERR_UNSUPPORTED;
+  int grid = ctx->sm_count * (per_sm < 2 ? per_sm : 2);
+  if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
+  TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, sizeof(unsigned int), stream));
+  const int* lvl_off = ctx->last.level_offset;
+  long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
+  void* args[] = {&p, &dV, &sizes, &lvl_off, &wait_limit};
+  TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_begin, dim3(grid), dim3(256), args, smem, stream));
+  ctx->launches += 1;
+  return TREELSTM_OK;
+}
+
 }  // namespace
 
 int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW, float* db,
@@ -938,6 +1000,12 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
       TL_CUDA(ctx, cudaMemsetAsync(dbc, 0, sizeof(float) * C, stream));
       TL_CUDA(ctx, cudaMemsetAsync(n_touched, 0, sizeof(int), stream));
       return TREELSTM_OK;
+    }
+    if (ctx->opt.dw_tensor_cores && trees_take(ctx, n)) {
+      int rc = launch_bwd_begin(ctx, p, nullptr, {(E + 2 * (size_t)H) * J, J, 0}, stream);
+      if (rc == TREELSTM_OK) rc = launch_backward_trees(ctx, stream);
+      return rc != TREELSTM_OK ? rc : launch_dweight_tc(ctx, n, L.order, L.level_offset, L.token, L.left, L.right, L.h, p.dz, dW, db,
+                                                        p.tok_slot, dEmb_rows, p.st, stream);
     }
     const size_t smem = ((sizeof(BwdSmem) + 3) / 4) * 4 + cls_smem;
     TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1104,76 +1172,12 @@ __global__ void k_rec_bwd_dv(RecBwd p) {
 
 }  // namespace
 
-// What precedes the walk over the trees (rec_trees.cu), in one cooperative launch: outputs cleared | leaf tokens
-// marked | tokens counted beside the classifier | tokens placed.  The level table stays on the device.
-__global__ void __launch_bounds__(256, 2)
-k_rec_bwd_begin(BwdParams p, float* dV, size_t dv_words, const int* level_offset, long long wait_limit) {
-  extern __shared__ float s_cls[];
-  __shared__ __align__(16) unsigned int s_mask[1024];
-  __shared__ int s_flag;
-  // the kernel behind this one may set itself up: it waits for this grid before it reads dh
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (ld_volatile(&p.st->status) != 0) return;
-  const int n_levels = p.st->n_levels, H = p.H, C = p.C;
-  p.n_leaves = n_levels > 0 ? level_offset[1] : 0;
-  const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, gthreads = (size_t)gridDim.x * blockDim.x;
-  unsigned int arrivals = 0;
-  auto barrier = [&]() {
-    arrivals += gridDim.x;
-    return grid_barrier(p.st, arrivals, wait_limit, &s_flag, true, &p.st->barrier_bwd);
-  };
-  if (gtid == 0) { *p.loss = 0.f; *p.n_touched = 0; }
-  zero_range(p.dW, 2 * (size_t)H * H, gtid, gthreads);
-  zero_range(p.db, (size_t)H, gtid, gthreads);
-  zero_range(dV, dv_words, gtid, gthreads);
-  zero_range(p.dWc, (size_t)H * C, gtid, gthreads);
-  zero_range(p.dbc, (size_t)C, gtid, gthreads);
-  zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
-  zero_range(p.dEmb_rows, (size_t)p.n_leaves * H, gtid, gthreads);
-  if (!barrier()) return;
-  for (size_t r = gtid; r < (size_t)p.n_leaves; r += gthreads)
-    p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[r], p.n)], p.vocab)] = 1;
-  if (!barrier()) return;
-  int* const group_count = p.tok_slot + p.vocab + 4;
-  if (gridDim.x == 1) {
-    scan_tokens(p, s_mask, 1024);
-    classifier_groups(p, 0, 1, s_cls);
-  } else {
-    scan_count_groups(p, group_count);
-    classifier_groups(p, blockIdx.x, gridDim.x, s_cls);
-    if (!barrier()) return;
-    scan_place_groups(p, group_count);
-  }
-}
-
-// Backward of a context whose cells run on clusters: three launches, nothing read back.
-int launch_backward_rec_resident(treelstm* ctx, BwdParams& p, float* dV, cudaStream_t stream) {
-  auto& L = ctx->last;
-  const size_t H = ctx->H, dv_words = ctx->cell == TREELSTM_CELL_RNTN ? 4 * H * H * H : 0;
-  const size_t smem = sizeof(float) * (H * p.C + p.C);
-  if (smem > 48 * 1024)
-    TL_CUDA(ctx, cudaFuncSetAttribute(k_rec_bwd_begin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int per_sm = 0;
-  TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rec_bwd_begin, 256, smem));
-  if (per_sm < 1) return TREELSTM_ERR_UNSUPPORTED;
-  int grid = ctx->sm_count * (per_sm < 2 ? per_sm : 2);
-  if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
-  TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, sizeof(unsigned int), stream));
-  const int* lvl_off = L.level_offset;
-  long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
-  size_t words = dv_words;
-  void* args[] = {&p, &dV, &words, &lvl_off, &wait_limit};
-  TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_rec_bwd_begin, dim3(grid), dim3(256), args, smem, stream));
-  ctx->launches += 1;
-  return launch_backward_rec_trees(ctx, p.dW, p.db, dV, p.dEmb_rows, p.tok_slot, stream);
-}
-
 int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float* dW, float* db, float* dV,
                         float* dWc, float* dbc, int32_t* touched_ids, float* dEmb_rows, int32_t* n_touched,
                         cudaStream_t stream) {
   auto& L = ctx->last;
   L.stream = stream;
-  if (L.n > 0 && !L.host_levels_valid && ctx->rt.ok && L.n <= ctx->rt.max_nodes) {
+  if (L.n > 0 && !L.host_levels_valid && trees_take(ctx, L.n)) {
     char* base = static_cast<char*>(L.ws);
     BwdParams p{};
     p.n = L.n; p.H = p.E = ctx->H; p.C = ctx->C; p.vocab = ctx->vocab;
@@ -1185,7 +1189,10 @@ int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float
     p.tok_slot = reinterpret_cast<int*>(base + L.lay.tok_slot);
     p.touched_ids = touched_ids; p.n_touched = n_touched;
     p.st = reinterpret_cast<DevStatus*>(base + L.lay.status);
-    return launch_backward_rec_resident(ctx, p, dV, stream);
+    const size_t H = ctx->H;
+    int rc = launch_bwd_begin(ctx, p, dV, {2 * H * H, H, ctx->cell == TREELSTM_CELL_RNTN ? 4 * H * H * H : 0}, stream);
+    if (rc == TREELSTM_OK) rc = launch_backward_trees(ctx, stream);
+    return rc != TREELSTM_OK ? rc : launch_rec_grads(ctx, dW, db, dV, dEmb_rows, p.tok_slot, stream);
   }
   int rc = ensure_host_levels(ctx);      // one read of the level table (a persistent forward left it on the device)
   if (rc != TREELSTM_OK) return rc;

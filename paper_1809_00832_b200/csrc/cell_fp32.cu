@@ -478,6 +478,11 @@ int launch_forward_fp32(treelstm* ctx, int n, const int32_t* left, const int32_t
                         const int32_t* level_offset_dev, const int32_t* level_offset_host,
                         int n_levels_host, int flags, void* ws, const WsLayout& lay,
                         cudaStream_t stream) {
+  if ((flags & TREELSTM_PERSISTENT) && trees_take(ctx, n)) {
+    const int single_max = ctx->opt.sched_single_cta_max < kSchedSingleMaxNodes ? ctx->opt.sched_single_cta_max : kSchedSingleMaxNodes;
+    return launch_forward_trees(ctx, n, left, right, token, h, c, (flags & TREELSTM_SAVE_FOR_BACKWARD) != 0, ws, lay,
+                                ctx->opt.overlap_launch && n <= single_max, stream);
+  }
   char* base = static_cast<char*>(ws);
   FwdParams p;
   p.n = n; p.H = ctx->H; p.E = ctx->E; p.n_sms = ctx->sm_count; p.vocab = ctx->vocab;

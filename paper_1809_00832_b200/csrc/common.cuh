@@ -90,6 +90,15 @@ struct SubforestPlan {
   int cluster_size = 0, groups_per_cta = 0, smem_bytes = 0, n_parts = 0;
 };
 
+// How the fp32 tree kernels (trees_fp32.cu) run for a context's sizes: CTAs per cluster, units per CTA; forward: outputs
+// per thread, threads over the outputs (lane groups), segments of the inputs, 16-byte chunks of inputs in all and per
+// segment; backward: threads, segments, chunks per segment, RNTN: threads per row.
+struct TreesShape {
+  int cs = 0, JS = 0;
+  int U = 0, JL = 0, nseg = 0, chunks = 0, nc = 0;
+  int bthreads = 0, bseg = 0, BC = 0, TPA = 0;
+};
+
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 inline size_t round_up_sz(size_t x, size_t m) { return (x + m - 1) / m * m; }
 
@@ -127,12 +136,14 @@ struct treelstm {
   int tc_resident_ctas = 0;             // CTAs of the grid-wide bf16 kernel the device holds at once
   bool tail_skip = false;               // the last forward whose control block was read back had no tail worth a hand-over
 
-  // TreeRNN / RNTN: how the tree kernels (rec_trees.cu) run for the context's sizes
-  struct RecTrees {
-    bool ok = false;
-    int cs = 1, Q = 0, R = 0, JS = 0, SP = 0, max_nodes = 0;   // cluster size, product rows, rows, units per CTA, row stride
-    float* W = nullptr;      // RNTN: [R][H], symmetric products added up (TreeRNN: Wcat as it is)
-  } rt;
+  // the fp32 tree kernels (trees_fp32.cu)
+  struct Trees {
+    bool ok = false, known = false;
+    tl::TreesShape s;
+    float *Wf = nullptr, *Wb = nullptr;                 // register images of the weights
+    int clusters = 0, clusters_bwd = 0;                 // that the device holds at once
+    ushort2* pairs = nullptr;                           // RNTN: operands of every input chunk
+  } trees;
 
   tl::Options opt;
 
@@ -203,12 +214,13 @@ int launch_forward_rec(treelstm* ctx, int n, const int32_t* left, const int32_t*
                        const int32_t* level_offset_host, int n_levels_host, int flags, void* ws,
                        const WsLayout& lay, cudaStream_t stream);
 
-// rec_trees.cu (TreeRNN / RNTN, trees dealt out to clusters)
-int init_rec_trees(treelstm* ctx, cudaStream_t stream);
-int launch_forward_rec_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token,
-                             float* h, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
-int launch_backward_rec_trees(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb_rows, const int* tok_slot,
-                              cudaStream_t stream);
+// trees_fp32.cu (all cells in fp32, trees dealt out to clusters)
+int init_trees(treelstm* ctx, cudaStream_t stream);      // shapes and register images; again after the weights changed
+bool trees_take(const treelstm* ctx, int n);
+int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
+                         float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
+int launch_backward_trees(treelstm* ctx, cudaStream_t stream);   // dz of every node (TreeRNN / RNTN: and dh of the leaves) from dh
+int launch_rec_grads(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb_rows, const int* tok_slot, cudaStream_t stream);
 
 // gemm_tc.cu
 int pack_weights_bf16(treelstm* ctx, cudaStream_t stream);

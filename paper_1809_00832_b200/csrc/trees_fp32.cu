@@ -1,0 +1,1222 @@
+// fp32 evaluation and backpropagation of all three cells (TreeLSTM, TreeRNN, RNTN), one thread-block cluster
+// per group of trees, with the recurrent weights held in REGISTERS.
+//
+// Trees are independent (Section 2.2), so a cluster walks its own trees depth by depth and waits for nobody
+// else.  A depth is then a handful of matrix-vector products, and its cost is a chain: weights to the
+// multipliers, sum over the inputs, activation, state to whoever reads it, barrier.
+//   - Weights.  From shared memory the 32 k weights of a TreeRNN with H = 128 take 1 k cycles per pass (2.1 k
+//     measured); the register files of the cluster hold them all.
+//   - Product.  A thread holds U outputs x a few inputs.  Shared memory gives a thread one word per lane and cycle,
+//     broadcast or not, so U decides: with one output per thread a TreeRNN node costs 1.1 k cycles and a TreeLSTM node
+//     (H = 150, eight CTAs) 1.65 k, all of it operand reads; the price of a large U is partial sums per output
+//     (512 U / outputs).  Four or five outputs balance the two.  (A warp per unit with shuffles instead of partial
+//     sums needs no CTA barrier, but every warp then issues the activations of a few values: 2.6 k cycles.)
+//   - State.  A node has one caller, so its h is stored straight into the caller's operand row [h_l | h_r] in the
+//     shared memory of every CTA of the cluster (distributed shared memory); the cell state stays with the unit's
+//     owner.  If the rows of the cluster's trees do not fit, states go through L2.
+//
+// Split.  CTA r of a cluster of cs owns hidden units [r JS, (r + 1) JS); cs is the smallest power of two whose
+// slice fits the registers of one CTA.  Backward is the same product with inputs (the CTA's own gate gradients) and
+// outputs (the 2H units of the children) exchanged; partial sums go straight to the unit's owner, who adds them.
+//
+// Order.  The schedule that callers see (level, order) is the scheduler's.  A cluster needs only "children
+// before parents"; deepest depth first is such an order with the same number of steps.  It finds roots and depths
+// itself, from the child arrays in shared memory, so nothing here waits for the scheduler before its end.  (A
+// malformed forest is the scheduler's to report; here every index is clamped and every list bounded, so that
+// whatever the arrays hold the walk ends.)  Clusters take roots q, q + Q, ... in id order.
+#include <new>
+#include <type_traits>
+
+#include "common.cuh"
+
+namespace tl {
+namespace {
+
+constexpr int NT = 4;                     // nodes per pass of the forward
+constexpr int kFwdT = 512, kBwdT = 640;   // threads of a CTA (backward: at most)
+constexpr int kSmemMax = 224 * 1024;
+constexpr int kLstm = 0, kRnn = TREELSTM_CELL_TREERNN, kRntn = TREELSTM_CELL_RNTN;
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kND = 16;                   // backward: nodes between two cluster barriers at most
+constexpr int kRntnBC = 2, kRntnJS = 8, kRntnMaxH = 32, kRntnT = 512;   // RNTN backward: columns and units per thread
+constexpr int kRntnBwdWords = 4 * kRntnBC * kRntnJS + kRntnJS;
+
+__device__ __forceinline__ float sigmoid_acc(float x) { return 1.0f / (1.0f + expf(-x)); }
+__device__ __forceinline__ uint32_t cta_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// every thread of the cluster; what any of them wrote before is visible to all of them afterwards
+__device__ __forceinline__ void cluster_sync(int cs) {
+  if (cs > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+__device__ __forceinline__ uint32_t peer_addr(uint32_t smem_addr, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Four sums over each group of LANES lanes: v[0] of a lane becomes the sum of value value_of_lane(lane) - every
+// exchange halves the values a lane still carries.
+template <int LANES>
+__device__ __forceinline__ void lane_sums4(float (&v)[4], int lane) {
+  const bool up = (lane & (LANES / 2)) != 0, up2 = (lane & (LANES / 4)) != 0;
+  const float s0 = up ? v[0] : v[2], s1 = up ? v[1] : v[3];
+  v[0] = (up ? v[2] : v[0]) + __shfl_xor_sync(kFull, s0, LANES / 2);
+  v[1] = (up ? v[3] : v[1]) + __shfl_xor_sync(kFull, s1, LANES / 2);
+  const float s2 = up2 ? v[0] : v[1];
+  v[0] = (up2 ? v[1] : v[0]) + __shfl_xor_sync(kFull, s2, LANES / 4);
+#pragma unroll
+  for (int d = LANES / 8; d > 0; d /= 2) v[0] += __shfl_xor_sync(kFull, v[0], d);
+}
+template <int LANES>
+__device__ __forceinline__ int value_of_lane(int lane) { return ((lane & (LANES / 2)) ? 2 : 0) + ((lane & (LANES / 4)) ? 1 : 0); }
+
+struct TreesParams {
+  int n, H, E, vocab;
+  int Hp;                                 // H rounded up to 4: half an operand row in shared memory
+  TreesShape s;
+  int* chk_counts;
+  const int *left, *right, *token;
+  const float *emb, *W, *b;               // W: register image [rank][word][thread]; b [G H]
+  const ushort2* pairs;                   // RNTN: the two operands of every input chunk
+  float *h, *c, *gates, *dh, *dc, *dz;
+  DevStatus* st;
+  long long* trace;                       // cycle stamps of the first CTA (trace builds), else nullptr
+};
+
+// ---- which weight a thread holds where (host and device; the register images are packed once) ------- //
+struct WeightAt { long long i0, i1; };    // index into the fp32 weights, -1: padding; i1 >= 0: a second one is added
+__host__ __device__ inline int real_input(int padded, int H, int Hp) {   // entry of [h_l | h_r] behind a padded one, -1: padding
+  const int side = padded >= Hp, k = padded - side * Hp;
+  return k < H ? side * H + k : -1;
+}
+// Forward word (c * 4 + i) * U + u of a thread (lane group t % JL, segment t / JL): input i of the segment's chunk c,
+// output u: the unit's gate u (TreeLSTM), unit u JL + lane (the others).
+__host__ __device__ inline WeightAt fwd_weight(int cell, int H, int E, const TreesShape& s, int rank, int t, int w, const ushort2* pairs) {
+  const WeightAt none{-1, -1};
+  const int Hp = (H + 3) & ~3, u = w % s.U, i = (w / s.U) % 4, c = w / (4 * s.U), lane = t % s.JL, seg = t / s.JL;
+  // RNTN segments interleave their chunks (the rows of one operand pair lie side by side), the others take runs
+  const int ch = cell == kRntn ? seg + s.nseg * c : seg * s.nc + c;
+  if (seg >= s.nseg || ch >= s.chunks) return none;
+  const int unit = cell == kLstm ? lane : u * s.JL + lane, gate = cell == kLstm ? u : 0;
+  const int j = rank * s.JS + unit;
+  if (unit >= s.JS || j >= H || gate > 4) return none;
+  if (cell != kRntn) {
+    const int r = real_input(4 * ch + i, H, Hp);
+    if (r < 0) return none;
+    return cell == kLstm ? WeightAt{((long long)E + r) * 5 * H + (long long)gate * H + j, -1} : WeightAt{(long long)r * H + j, -1};
+  }
+  const int K = 2 * H, bp = pairs[ch].y + i, b = real_input(bp, H, Hp);
+  if (b < 0) return none;
+  if (pairs[ch].x == 0xFFFF) return {((long long)K * K + b) * H + j, -1};      // linear part behind the 4H^2 product rows
+  if (bp < pairs[ch].x) return none;                                           // b < a: counted in the other half
+  const int a = real_input(pairs[ch].x, H, Hp);
+  const long long ab = ((long long)a * K + b) * H + j;
+  return {ab, a != b ? ((long long)b * K + a) * H + j : -1};
+}
+// Backward word (c * 4 + i) * 4 + u: output 4 (t / bseg) + u, input 4 (t % bseg + bseg c) + i of the CTA's gate gradients
+// (gate JS + unit).
+__host__ __device__ inline WeightAt bwd_weight(int cell, int H, int E, const TreesShape& s, int rank, int t, int w) {
+  const WeightAt none{-1, -1};
+  if (cell == kRntn) {
+    // thread (row a of x, q of TPA): word (c * 4 + i) * 8 + u: entry (a, b) of the symmetric S_u, then the linear part
+    const int K = 2 * H, Hp = (H + 3) & ~3, tpa = s.TPA, a = t / tpa, q = t % tpa;
+    if (a >= K) return none;
+    const int u = w % kRntnJS, j = rank * s.JS + u;
+    if (u >= s.JS || j >= H) return none;
+    if (w >= 4 * kRntnBC * kRntnJS) return u % tpa == q ? WeightAt{((long long)K * K + a) * H + j, -1} : none;
+    const int i = (w / kRntnJS) % 4, c = w / (4 * kRntnJS), bp = 4 * (q + tpa * c) + i;
+    const int b = bp < 2 * Hp ? real_input(bp, H, Hp) : -1;
+    if (b < 0) return none;
+    return {((long long)a * K + b) * H + j, ((long long)b * K + a) * H + j};   // V_ab + V_ba, twice V_aa
+  }
+  const int out = 4 * (t / s.bseg) + w % 4, c = w / 16, in = 4 * (t % s.bseg + s.bseg * c) + (w / 4) % 4;
+  if (out >= 2 * H || c >= s.BC) return none;
+  const int gate = in / s.JS, unit = in - gate * s.JS, j = rank * s.JS + unit;
+  if (gate >= (cell == kLstm ? 5 : 1) || j >= H) return none;
+  return cell == kLstm ? WeightAt{((long long)E + out) * 5 * H + (long long)gate * H + j, -1} : WeightAt{(long long)out * H + j, -1};
+}
+
+// ---- shared memory -------------------------------------------------------------------------------- //
+// Offsets in 4-byte words.  What is left behind `state` holds the states of the cluster's nodes, if they fit.
+struct TreesSmem {
+  int buf, kids, child, list, start, par, leaf, leaf_par, state, state_words;
+};
+__host__ __device__ inline TreesSmem trees_smem(int n, int buf_words) {
+  TreesSmem s{};
+  int off = 0;
+  auto take = [&](int words) { const int o = off; off += (words + 3) & ~3; return o; };
+  s.buf = take(buf_words);
+  s.kids = take(n);
+  s.child = take(n / 32 + 1);             // a bit per node: it has a caller
+  const int half = n / 4 + 8;             // uint16 entries for the internal nodes (fewer than n / 2)
+  s.list = take(half);
+  s.start = take(half);
+  s.par = take(half);
+  s.leaf = take(n / 2 + 8);               // (a forest of single-leaf trees has n leaves)
+  s.leaf_par = take(n / 2 + 8);
+  s.state = off;
+  s.state_words = kSmemMax / 4 - off;
+  return s;
+}
+// forward: partial sums [nseg][NT][outs], gate values [NT][outs], operand rows and cell states of a pass (states in L2)
+__host__ __device__ inline int fwd_outs(const TreesShape& s) { return s.U * s.JL; }
+__host__ __device__ inline int fwd_parts(int cell, const TreesShape& s) { return ((cell == kRntn ? kFwdT / 32 : s.nseg) + 7) & ~7; }
+__host__ __device__ inline int fwd_buf_words(int cell, int H, const TreesShape& s) {
+  return (fwd_parts(cell, s) + 1) * NT * fwd_outs(s) + NT * (2 * ((H + 3) & ~3) + 2 * ((s.JS + 3) & ~3));
+}
+// backward: gate gradients of a round [kND][in_row], then the sums that came in [2][cs][kND][2 JS] (RNTN: and x)
+__host__ __device__ inline int bwd_in_row(int cell, const TreesShape& s) { return cell == kRntn ? kRntnJS : 4 * s.bseg * s.BC; }
+__host__ __device__ inline int bwd_buf_words(int cell, int H, const TreesShape& s) {
+  return kND * bwd_in_row(cell, s) + 2 * s.cs * kND * 2 * s.JS + (cell == kRntn ? kND * 2 * ((H + 3) & ~3) : 0);
+}
+
+// Child table entry of a node: left | right << 16 (ids below 32768), or the top bit and the token of a leaf.  Ids and
+// tokens are clamped: nothing has been validated yet.
+constexpr unsigned kLeafBit = 0x80000000u;
+__device__ __forceinline__ bool is_leaf(unsigned kids) { return (kids & kLeafBit) != 0; }
+__device__ __forceinline__ void load_kids(const TreesParams& p, const TreesSmem& s, float* sm) {
+  unsigned* kids = reinterpret_cast<unsigned*>(sm + s.kids);
+  unsigned* child = reinterpret_cast<unsigned*>(sm + s.child);
+  for (int k = threadIdx.x; k < p.n / 32 + 1; k += blockDim.x) child[k] = 0u;
+  __syncthreads();
+  for (int k = threadIdx.x; k < p.n; k += blockDim.x) {
+    const int l = p.left[k], r = p.right[k], t = p.token[k];
+    if (l < 0) {
+      kids[k] = kLeafBit | (unsigned)min(max(t, 0), p.vocab - 1);
+    } else {
+      const unsigned a = (unsigned)min(l, p.n - 1), b = (unsigned)min(max(r, 0), p.n - 1);
+      kids[k] = a | (b << 16);
+      atomicOr(child + (a >> 5), 1u << (a & 31));
+      atomicOr(child + (b >> 5), 1u << (b & 31));
+    }
+  }
+  __syncthreads();
+}
+
+// The cluster's trees by depth: internal node number q is list[q], depth d is [start[d], start[d + 1]), the leaves are
+// in leaf[]; par[q] and leaf_par[] say whose child a node is: 2 x number of the caller + side, kNoCaller for a root.  One
+// warp; every CTA of the cluster gets the same lists.
+constexpr unsigned short kNoCaller = 0xFFFF;
+struct Walk { int depths, internal, leaves; };
+__device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, Walk* out) {
+  const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
+  const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
+  unsigned short* list = reinterpret_cast<unsigned short*>(sm + s.list);
+  unsigned short* start = reinterpret_cast<unsigned short*>(sm + s.start);
+  unsigned short* par = reinterpret_cast<unsigned short*>(sm + s.par);
+  unsigned short* leaf = reinterpret_cast<unsigned short*>(sm + s.leaf);
+  unsigned short* leaf_par = reinterpret_cast<unsigned short*>(sm + s.leaf_par);
+  const int lane = threadIdx.x & 31, n = p.n;
+  const unsigned below = (1u << lane) - 1u;
+  const int max_internal = n / 2, max_leaves = n;
+  int count = 0, leaves = 0, depth = 0, lo = 0, rank0 = 0;
+  auto scan = [&](int v) {                // inclusive over the lanes
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int t = __shfl_up_sync(kFull, v, d);
+      if (lane >= d) v += t;
+    }
+    return v;
+  };
+  for (int w0 = 0; w0 * 32 < n; w0 += 32) {   // roots: nodes without a caller, 32 words of 32 ids at a time
+    const int w = w0 + lane, base = w * 32;
+    unsigned m = base < n ? ~child[w] : 0u;
+    if (base < n && n - base < 32) m &= (1u << (n - base)) - 1u;
+    const int roots = __popc(m), incl = scan(roots);
+    int rank = rank0 + incl - roots, mi = 0, ml = 0;
+    rank0 += __shfl_sync(kFull, incl, 31);
+    for (unsigned b = m; b; b &= b - 1, ++rank)
+      if (rank % parts == part) (is_leaf(kids[base + __ffs(b) - 1]) ? ml : mi) += 1;
+    const int ii = scan(mi), il = scan(ml);
+    int ci = count + ii - mi, cl = leaves + il - ml;
+    rank = rank0 - __shfl_sync(kFull, incl, 31) + incl - roots;
+    for (unsigned b = m; b; b &= b - 1, ++rank)
+      if (rank % parts == part) {
+        const int node = base + __ffs(b) - 1;
+        if (is_leaf(kids[node])) { leaf[cl] = (unsigned short)node; leaf_par[cl++] = kNoCaller; }
+        else if (ci < max_internal) { list[ci] = (unsigned short)node; par[ci++] = kNoCaller; }
+      }
+    count = min(count + __shfl_sync(kFull, ii, 31), max_internal);
+    leaves += __shfl_sync(kFull, il, 31);
+  }
+  bool fits = true;
+  if (lane == 0) start[0] = 0;
+  __syncwarp();
+  while (lo < count && fits) {
+    const int hi = count;
+    ++depth;
+    if (lane == 0) start[depth] = (unsigned short)hi;
+    for (int i0 = lo; i0 < hi; i0 += 32) {
+      const bool have = i0 + lane < hi;
+      const unsigned kd = have ? kids[list[i0 + lane]] : 0u;
+      const int l = (int)(kd & 0xFFFFu), r = (int)(kd >> 16);
+      const bool ll = is_leaf(kids[l]), lr = is_leaf(kids[r]);
+      const unsigned il = __ballot_sync(kFull, have && !ll), ir = __ballot_sync(kFull, have && !lr);
+      const unsigned fl = __ballot_sync(kFull, have && ll), fr = __ballot_sync(kFull, have && lr);
+      // only arrays that are no forest of trees can run over
+      if (count + __popc(il) + __popc(ir) > max_internal || leaves + __popc(fl) + __popc(fr) > max_leaves) { fits = false; break; }
+      if (have) {
+        const int al = ll ? leaves + __popc(fl & below) : count + __popc(il & below);
+        const int ar = lr ? leaves + __popc(fl) + __popc(fr & below) : count + __popc(il) + __popc(ir & below);
+        (ll ? leaf : list)[al] = (unsigned short)l;
+        (lr ? leaf : list)[ar] = (unsigned short)r;
+        (ll ? leaf_par : par)[al] = (unsigned short)(2 * (i0 + lane));
+        (lr ? leaf_par : par)[ar] = (unsigned short)(2 * (i0 + lane) + 1);
+      }
+      count += __popc(il) + __popc(ir);
+      leaves += __popc(fl) + __popc(fr);
+      __syncwarp();
+    }
+    lo = hi;
+  }
+  if (lane == 0) *out = fits ? Walk{depth, count, leaves} : Walk{0, 0, 0};
+}
+
+// ---- forward -------------------------------------------------------------------------------------- //
+template <int CELL, int U, int RC>
+__global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constant__ TreesParams p) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ Walk s_walk;
+  const int cs = p.s.cs, rank = cs > 1 ? (int)cta_rank() : 0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int part = blockIdx.x / cs, parts = gridDim.x / cs;
+  const int H = p.H, Hp = p.Hp, JS = p.s.JS, JS4 = (JS + 3) & ~3, JL = p.s.JL, outs = U * JL, j0 = rank * JS;
+  const TreesSmem s = trees_smem(p.n, fwd_buf_words(CELL, H, p.s));
+#ifdef TREELSTM_TRACE
+  long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;   // row d: depth d; last row: set-up
+#endif
+  TL_STAMP(trace, kTraceLevels - 1, 0);
+  float w[RC * 4 * U];
+#pragma unroll
+  for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
+  load_kids(p, s, sm);
+  TL_STAMP(trace, kTraceLevels - 1, 1);
+  if (warp == 0) walk_trees(p, s, sm, part, parts, &s_walk);
+#pragma unroll
+  for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
+  __syncthreads();
+  TL_STAMP(trace, kTraceLevels - 1, 2);
+  const Walk walk = s_walk;
+  const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
+  const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
+  const unsigned short* start = reinterpret_cast<const unsigned short*>(sm + s.start);
+  const unsigned short* par = reinterpret_cast<const unsigned short*>(sm + s.par);
+  const unsigned short* leaf = reinterpret_cast<const unsigned short*>(sm + s.leaf);
+  const unsigned short* leaf_par = reinterpret_cast<const unsigned short*>(sm + s.leaf_par);
+  // operand rows [h_l | h_r] of the internal nodes, padded to whole segments; then (TreeLSTM) the children's c of the
+  // CTA's own units
+  const int row = CELL == kRntn ? 2 * Hp : 4 * p.s.nseg * RC, crow = CELL == kLstm ? 2 * JS4 : 0;
+  const bool resident = (long long)walk.internal * (row + crow) <= s.state_words;
+  float* const red = sm + s.buf;
+  float* const act = red + fwd_parts(CELL, p.s) * NT * outs;
+  float* const xrow = act + NT * outs;                   // states in L2: operand rows and cell states of a pass
+  float* const state = resident ? sm + s.state : xrow;
+  float* const cstate = state + (resident ? walk.internal * row : NT * 2 * Hp);
+  const uint32_t state_addr = smem_u32(state);
+  const int xstride = resident ? row : 2 * Hp;           // (the padding behind an L2 row is the next row: finite, times zero)
+  for (int e = tid; e < (resident ? walk.internal * (row - 2 * H) : NT * (2 * Hp + 2 * JS4)); e += kFwdT) {
+    if (resident) {
+      const int q = e / (row - 2 * H), k = e - q * (row - 2 * H);
+      state[q * row + (k < Hp - H ? H + k : H + k + H)] = 0.f;
+    } else {
+      xrow[e] = 0.f;
+    }
+  }
+  for (int e = tid; e < fwd_parts(CELL, p.s) * NT * outs; e += kFwdT) red[e] = 0.f;   // (sums beyond the segments stay zero)
+  if (CELL == kLstm) asm volatile("griddepcontrol.wait;" ::: "memory"); // the leaves' states come from the kernel ahead
+  cluster_sync(cs);                                      // every CTA of the cluster runs: its shared memory may be written
+  for (int q = warp; q < walk.leaves; q += kFwdT / 32) {
+    const int node = leaf[q];
+    const unsigned code = leaf_par[q];
+    const bool keep = resident && code != kNoCaller;
+    const float* src = CELL == kLstm ? p.h + (size_t)node * H : p.emb + (size_t)(kids[node] & ~kLeafBit) * H;
+    float* dst = state + (code >> 1) * row + (code & 1) * Hp;
+    const bool copy = CELL != kLstm && q % cs == rank;   // a leaf's state is its word vector
+    if (keep || copy)
+      for (int k = lane; k < H; k += 32) {
+        const float v = CELL == kLstm ? __ldcg(src + k) : __ldg(src + k);
+        if (keep) dst[k] = v;
+        if (copy) {
+          p.h[(size_t)node * H + k] = v;
+          count_write(p.chk_counts, node, 1);
+        }
+      }
+    if (CELL == kLstm && keep)
+      for (int u = lane; u < JS && j0 + u < H; u += 32)
+        cstate[(code >> 1) * crow + (code & 1) * JS4 + u] = __ldcg(p.c + (size_t)node * H + j0 + u);
+  }
+  // the thread's first chunk, or (RNTN) its chunks' operands: b in bits 8.., a below, 255: the linear part
+  const int lane_out = tid % JL, seg = tid / JL;
+  const bool works = seg < p.s.nseg;
+  int ops[CELL == kRntn ? RC : 1];
+  if constexpr (CELL == kRntn) {
+#pragma unroll
+    for (int c = 0; c < RC; ++c) {
+      const ushort2 ab = p.pairs[min(seg + p.s.nseg * c, p.s.chunks - 1)];
+      ops[c] = ((int)ab.y << 8) | (ab.x & 255);
+    }
+  } else {
+    ops[0] = 4 * min(seg, p.s.nseg - 1) * RC;
+  }
+  // what this thread adds up (node red_i of a pass, output red_o; further ones kFwdT entries on) and updates
+  const int step_i = kFwdT / outs, step_o = kFwdT - step_i * outs;
+  const int red_i = tid / outs, red_o = tid - red_i * outs;
+  const float red_bias = __ldg(p.b + (CELL == kLstm ? min(red_o / JS, 4) * H + min(j0 + red_o % JS, H - 1) : min(j0 + red_o, H - 1)));
+  const int red_g = CELL == kLstm ? red_o / JS : 0, red_u = CELL == kLstm ? red_o - red_g * JS : red_o;
+  const int sets = max(1, kFwdT / (NT * JS)), cell_set = tid / (NT * JS), cell_q = tid - cell_set * NT * JS;
+  const int cell_i = cell_q / JS, cell_u = cell_q - cell_i * JS;
+  (void)cell_i; (void)cell_u; (void)sets;
+  const int parts_sum = fwd_parts(CELL, p.s);
+  cluster_sync(cs);                                      // the leaves' states are in place
+  TL_STAMP(trace, kTraceLevels - 1, 3);
+  for (int d = walk.depths - 1; d >= 0; --d) {
+    for (int lo = start[d], hi = start[d + 1]; lo < hi; lo += NT) {
+      const int cnt = min(NT, hi - lo);
+      TL_STAMP(trace, d, 0);
+      if (!resident) {
+        // the children's states from L2 (a leaf of TreeRNN / RNTN: from the table itself)
+        __syncthreads();
+        for (int i = warp; i < 2 * cnt; i += kFwdT / 32) {
+          const unsigned kd = kids[list[lo + (i >> 1)]];
+          const int child = (int)((i & 1) ? kd >> 16 : kd & 0xFFFFu);
+          const unsigned ck = kids[child];
+          const bool table = CELL != kLstm && is_leaf(ck);
+          const float* src = table ? p.emb + (size_t)(ck & ~kLeafBit) * H : p.h + (size_t)child * H;
+          for (int k = lane; k < H; k += 32) xrow[i * Hp + k] = table ? __ldg(src + k) : __ldcg(src + k);
+          if (CELL == kLstm)
+            for (int u = lane; u < JS && j0 + u < H; u += 32) cstate[i * JS4 + u] = __ldcg(p.c + (size_t)child * H + j0 + u);
+        }
+        __syncthreads();
+      }
+      const float* const x0 = state + (resident ? lo * row : 0);
+      auto multiply = [&](auto n_const) {
+        constexpr int N = decltype(n_const)::value;
+        float acc[N][U];
+        const float* xb[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          xb[i] = x0 + min(i, cnt - 1) * xstride + (CELL == kRntn ? 0 : ops[0]);
+#pragma unroll
+          for (int u = 0; u < U; ++u) acc[i][u] = 0.f;
+        }
+#pragma unroll
+        for (int c = 0; c < RC; ++c) {
+          float4 x[N];
+#pragma unroll
+          for (int i = 0; i < N; ++i) {
+            if constexpr (CELL == kRntn) {
+              x[i] = *reinterpret_cast<const float4*>(xb[i] + (ops[c] >> 8));
+              const int a = ops[c] & 255;
+              const float f = a == 255 ? 1.f : xb[i][a];
+              x[i].x *= f; x[i].y *= f; x[i].z *= f; x[i].w *= f;
+            } else {
+              x[i] = *reinterpret_cast<const float4*>(xb[i] + 4 * c);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              acc[i][u] = fmaf(x[i].x, w[(c * 4 + 0) * U + u], acc[i][u]);
+              acc[i][u] = fmaf(x[i].y, w[(c * 4 + 1) * U + u], acc[i][u]);
+              acc[i][u] = fmaf(x[i].z, w[(c * 4 + 2) * U + u], acc[i][u]);
+              acc[i][u] = fmaf(x[i].w, w[(c * 4 + 3) * U + u], acc[i][u]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            if constexpr (CELL == kRntn) {               // JL is a power of two: a warp adds its own segments first
+              float v = acc[i][u];
+              for (int dd = JL; dd < 32; dd <<= 1) v += __shfl_xor_sync(kFull, v, dd);
+              if (lane < JL) red[(warp * NT + i) * outs + u * JL + lane_out] = v;
+            } else if (works) {
+              red[(seg * NT + i) * outs + u * JL + lane_out] = acc[i][u];
+            }
+          }
+      };
+      if (cnt == 1) multiply(std::integral_constant<int, 1>{});
+      else if (cnt == 2) multiply(std::integral_constant<int, 2>{});
+      else multiply(std::integral_constant<int, NT>{});
+      __syncthreads();
+      TL_STAMP(trace, d, 1);
+      auto put_h = [&](int q, int unit, float hv, int first, int by) {   // into the caller's row, in every CTA (or every by-th)
+        const unsigned code = par[q];
+        if (!resident || code == kNoCaller) return;
+        const int at = (int)(code >> 1) * row + (int)(code & 1) * Hp + unit;
+        if (cs == 1) state[at] = hv;
+        else
+          for (int c = first; c < cs; c += by) st_cluster(peer_addr(state_addr + 4u * (uint32_t)at, (uint32_t)c), hv);
+      };
+      for (int i = red_i, o = red_o; i < cnt;) {
+        const bool own = o == red_o;                     // else: a second output of this thread (JS > 128 / gates)
+        const int g = CELL == kLstm ? (own ? red_g : o / JS) : 0, u = CELL == kLstm ? (own ? red_u : o - g * JS) : o;
+        float z = own ? red_bias : __ldg(p.b + min(g, 4) * H + min(j0 + u, H - 1));
+        const float* r = red + i * outs + o;
+        for (int q = 0; q < parts_sum; q += 8, r += 8 * NT * outs) {   // eight reads in flight (the sums are padded to eights)
+          float v[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) v[k] = r[k * NT * outs];
+          z += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        }
+        if constexpr (CELL == kLstm) {
+          const float a = g == 4 ? tanhf(z) : sigmoid_acc(z);
+          act[i * outs + o] = a;
+          if (p.gates && j0 + u < H) p.gates[(size_t)list[lo + i] * 5 * H + g * H + j0 + u] = a;
+        } else if (u < JS && j0 + u < H) {
+          const float hv = tanhf(z);
+          const int node = list[lo + i];
+          put_h(lo + i, j0 + u, hv, 0, 1);
+          p.h[(size_t)node * H + j0 + u] = hv;
+          count_write(p.chk_counts, node, 1);
+        }
+        i += step_i;
+        o += step_o;
+        if (o >= outs) { o -= outs; ++i; }
+      }
+      TL_STAMP(trace, d, 2);
+      if constexpr (CELL == kLstm) {
+        __syncthreads();
+        // cell update; several sets of threads repeat the same few operations and share the stores to the CTAs
+        if (cell_i < cnt && j0 + cell_u < H && cell_set < sets) {
+          const int q = lo + cell_i, node = list[q];
+          const float* a = act + cell_i * outs + cell_u;
+          const float* cc = cstate + (resident ? q : cell_i) * crow + cell_u;
+          const float cv = a[0] * a[4 * JS] + a[JS] * cc[0] + a[2 * JS] * cc[JS4];
+          const float hv = a[3 * JS] * tanhf(cv);
+          put_h(q, j0 + cell_u, hv, cell_set, sets);
+          if (cell_set == 0) {
+            const unsigned code = par[q];
+            if (resident && code != kNoCaller) cstate[(code >> 1) * crow + (code & 1) * JS4 + cell_u] = cv;
+            p.c[(size_t)node * H + j0 + cell_u] = cv;
+            p.h[(size_t)node * H + j0 + cell_u] = hv;
+            count_write(p.chk_counts, node, 1);
+          }
+        }
+      }
+      if (CELL != kLstm && lo + NT < hi) __syncthreads();   // the next pass's partial sums overwrite these
+      TL_STAMP(trace, d, 3);
+    }
+    cluster_sync(cs);                                    // the depth's states are in place (and no CTA leaves while a peer still writes to it)
+    TL_STAMP(trace, d, 4);
+  }
+  // what follows on the stream waits for this grid only: it must not end before the scheduler ahead of it has
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// ---- TreeLSTM leaves ------------------------------------------------------------------------------ //
+// Their states need no schedule, so this kernel runs beside the scheduler, over the whole GPU.  A CTA takes 2 ROWS consecutive
+// node ids, the leaves among them (half, in a forest of any shape) in tiles of ROWS, and 32 hidden units x the
+// three gates a leaf has.  Thread (unit, row group): ROWS / 8 rows x 3 gates; the rows are read as broadcasts,
+// the weights one word per lane, the next chunk is fetched into registers meanwhile.
+constexpr int kLeafT = 256, kLeafU = 32, kLeafK = 32;
+struct LeafParams {
+  int n, H, E, vocab;
+  int* chk_counts;
+  const int *left, *token;
+  const float *emb, *W, *b;
+  float *h, *c, *gates;
+};
+template <int ROWS>
+__global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
+  constexpr int RPT = ROWS / 8, AL = ROWS * kLeafK / kLeafT, WL = 3 * kLeafU * kLeafK / kLeafT;
+  __shared__ __align__(16) float As[2][ROWS][kLeafK + 4];
+  __shared__ float Ws[2][kLeafK][3 * kLeafU];
+  __shared__ int s_node[2 * ROWS], s_tok[2 * ROWS], s_count;
+  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5, H = p.H, E = p.E;
+  const int tiles_u = (H + kLeafU - 1) / kLeafU;
+  const int id0 = (int)(blockIdx.x / tiles_u) * 2 * ROWS, u0 = (int)(blockIdx.x % tiles_u) * kLeafU;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tid < 32) {                                        // the leaves among the CTA's node ids, ascending
+    int count = 0;
+#pragma unroll
+    for (int q = 0; q < 2 * ROWS / 32; ++q) {
+      const int k = id0 + 32 * q + tid;
+      const bool lf = k < p.n && p.left[min(k, p.n - 1)] < 0;
+      const unsigned m = __ballot_sync(0xffffffffu, lf);
+      if (lf) {
+        const int at = count + __popc(m & ((1u << tid) - 1u));
+        s_node[at] = k;
+        s_tok[at] = min(max(p.token[k], 0), p.vocab - 1);   // nothing has been validated yet
+      }
+      count += __popc(m);
+    }
+    if (tid == 0) s_count = count;
+  }
+  __syncthreads();
+  const int count = s_count;
+  const int u = min(u0 + tx, H - 1);
+  const float bi = __ldg(p.b + u), bo = __ldg(p.b + 3 * H + u), bu = __ldg(p.b + 4 * H + u);
+  for (int r0 = 0; r0 < count; r0 += ROWS) {
+    float acc[RPT][3] = {}, ra[AL], rw[WL];
+    auto fetch = [&](int k0) {
+#pragma unroll
+      for (int j = 0; j < AL; ++j) {
+        const int e = tid + j * kLeafT, i = e / kLeafK, k = min(k0 + e % kLeafK, E - 1);
+        ra[j] = __ldg(p.emb + (size_t)s_tok[min(r0 + i, count - 1)] * E + k);
+      }
+#pragma unroll
+      for (int j = 0; j < WL; ++j) {
+        const int e = tid + j * kLeafT, kk = e / (3 * kLeafU), g = (e / kLeafU) % 3, uu = e % kLeafU;
+        rw[j] = __ldg(p.W + (size_t)min(k0 + kk, E - 1) * 5 * H + (g ? g + 2 : 0) * H + min(u0 + uu, H - 1));
+      }
+    };
+    auto stash = [&](int buf, int k0) {                  // zeros beyond the contraction (other padding is never stored)
+#pragma unroll
+      for (int j = 0; j < AL; ++j) {
+        const int e = tid + j * kLeafT;
+        As[buf][e / kLeafK][e % kLeafK] = k0 + e % kLeafK < E ? ra[j] : 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < WL; ++j) {
+        const int e = tid + j * kLeafT, kk = e / (3 * kLeafU);
+        Ws[buf][kk][e % (3 * kLeafU)] = k0 + kk < E ? rw[j] : 0.f;
+      }
+    };
+    fetch(0);
+    __syncthreads();                                     // the previous tile's readers are done
+    stash(0, 0);
+    __syncthreads();
+    const int chunks = (E + kLeafK - 1) / kLeafK;
+    for (int ch = 0; ch < chunks; ++ch) {
+      const int buf = ch & 1;
+      if (ch + 1 < chunks) fetch((ch + 1) * kLeafK);
+#pragma unroll
+      for (int kk = 0; kk < kLeafK; kk += 4) {
+        float w[4][3];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int g = 0; g < 3; ++g) w[q][g] = Ws[buf][kk + q][g * kLeafU + tx];
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+          const float4 a = *reinterpret_cast<const float4*>(&As[buf][ty * RPT + i][kk]);
+#pragma unroll
+          for (int g = 0; g < 3; ++g) {
+            acc[i][g] = fmaf(a.x, w[0][g], acc[i][g]);
+            acc[i][g] = fmaf(a.y, w[1][g], acc[i][g]);
+            acc[i][g] = fmaf(a.z, w[2][g], acc[i][g]);
+            acc[i][g] = fmaf(a.w, w[3][g], acc[i][g]);
+          }
+        }
+      }
+      if (ch + 1 < chunks) stash(buf ^ 1, (ch + 1) * kLeafK);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      const int at = r0 + ty * RPT + i;
+      if (at >= count || u0 + tx >= H) continue;
+      const int node = s_node[at];
+      const float gi = sigmoid_acc(acc[i][0] + bi), go = sigmoid_acc(acc[i][1] + bo), gu = tanhf(acc[i][2] + bu);
+      const float cv = gi * gu;
+      p.c[(size_t)node * H + u] = cv;
+      p.h[(size_t)node * H + u] = go * tanhf(cv);
+      count_write(p.chk_counts, node, 1);
+      if (p.gates) {
+        float* g = p.gates + (size_t)node * 5 * H + u;
+        g[0] = gi; g[3 * H] = go; g[4 * H] = gu;
+      }
+    }
+  }
+  // the kernel behind this one waits for this grid only: it must not end before the scheduler ahead of it has
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+
+// ---- backward: dz of every node (TreeRNN / RNTN: dh of the leaves) from the classifier's dh --------- //
+// TreeLSTM   dc += dh o (1 - tanh^2 c);  dz_o = dh tanh(c) o (1 - o),  dz_i = dc u i (1 - i),  dz_u = dc i (1 - u^2),
+//            dz_f = dc c_child f (1 - f),  dc_child = dc f;  dh_children += W_h dz
+// TreeRNN    dz = dh (1 - h^2);  dh_children += W dz
+// RNTN       the same dz;  dh_children += W dz + sum_b x_b sum_j dz_j (V_j[a][b] + V_j[b][a])
+// A round is up to kND nodes of one depth: gate gradients of the CTA's own units (a thread each) | products, SEG lanes
+// per four outputs, sums sent to the owners of the units | cluster barrier | the owner adds what came to dh.
+// What a round needs from global memory and no ancestor changes is fetched a round ahead.
+template <int CELL, int SEG, int BC, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constant__ TreesParams p) {
+  constexpr int G = CELL == kLstm ? 5 : 1;
+  constexpr int kWords = CELL == kRntn ? kRntnBwdWords : BC * 16;
+  extern __shared__ __align__(16) float sm[];
+  __shared__ Walk s_walk;
+  const int cs = p.s.cs, rank = cs > 1 ? (int)cta_rank() : 0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+  const int part = blockIdx.x / cs, parts = gridDim.x / cs;
+  const int H = p.H, Hp = p.Hp, JS = p.s.JS, j0 = rank * JS, jn = max(0, min(JS, H - j0));
+  const int in_row = bwd_in_row(CELL, p.s), nd = min(kND, nt / JS);
+  const TreesSmem s = trees_smem(p.n, bwd_buf_words(CELL, H, p.s));
+#ifdef TREELSTM_TRACE
+  long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;
+#endif
+  TL_STAMP(trace, kTraceLevels - 1, 0);
+  float w[kWords];
+#pragma unroll
+  for (int q = 0; q < kWords; ++q) w[q] = __ldg(p.W + ((size_t)rank * kWords + q) * nt + tid);
+  load_kids(p, s, sm);
+  float* const in = sm + s.buf;                          // [kND][in_row]
+  float* const dx = in + kND * in_row;                   // [2][cs][kND][2 JS]
+  float* const xs = dx + 2 * cs * kND * 2 * JS;          // RNTN: [kND][2 Hp]
+  for (int e = tid; e < kND * in_row; e += nt) in[e] = 0.f;
+  if (CELL == kRntn)
+    for (int e = tid; e < kND * 2 * Hp; e += nt) xs[e] = 0.f;
+  TL_STAMP(trace, kTraceLevels - 1, 1);
+  if (warp == 0) walk_trees(p, s, sm, part, parts, &s_walk);
+#pragma unroll
+  for (int q = 0; q < kWords; ++q) asm volatile("" : "+f"(w[q]));       // held in registers: not to be loaded again where it is used
+  __syncthreads();
+  TL_STAMP(trace, kTraceLevels - 1, 2);
+  const Walk walk = s_walk;
+  const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
+  const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
+  const unsigned short* start = reinterpret_cast<const unsigned short*>(sm + s.start);
+  const unsigned short* par = reinterpret_cast<const unsigned short*>(sm + s.par);
+  const unsigned short* leaf = reinterpret_cast<const unsigned short*>(sm + s.leaf);
+  const unsigned short* leaf_par = reinterpret_cast<const unsigned short*>(sm + s.leaf_par);
+  // by caller: dh (and behind it dc) of its two children, the CTA's own units: in shared memory if they fit
+  const int row = CELL == kLstm ? 4 * JS : 2 * JS;
+  const bool resident = (long long)walk.internal * row <= s.state_words;
+  float* const state = sm + s.state;
+  const int my_i = tid / JS, my_u = tid - my_i * JS;     // the thread's node of a round and unit
+  const bool mine = my_i < nd && my_u < jn;
+  float g[G] = {}, cn = 0.f, cl = 0.f, cr = 0.f, xv[2] = {0.f, 0.f};    // of the next round: gates and cell states, or h; x
+  auto fetch = [&](int lo) {
+    if (lo >= walk.internal) return;
+    if (mine) {
+      const int node = list[min(lo + my_i, walk.internal - 1)];
+      const size_t at = (size_t)node * H + j0 + my_u;
+      if constexpr (CELL == kLstm) {
+        const unsigned kd = kids[node];
+        const float* gp = p.gates + (size_t)node * 5 * H + j0 + my_u;
+#pragma unroll
+        for (int q = 0; q < G; ++q) g[q] = __ldg(gp + q * H);
+        cn = __ldg(p.c + at);
+        cl = __ldg(p.c + (size_t)(kd & 0xFFFFu) * H + j0 + my_u);
+        cr = __ldg(p.c + (size_t)(kd >> 16) * H + j0 + my_u);
+      } else {
+        cn = __ldg(p.h + at);
+      }
+    }
+    if constexpr (CELL == kRntn) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int e = tid + q * nt, i = e / (2 * H), k = e - i * 2 * H;
+        const unsigned kd = kids[list[min(lo + i, walk.internal - 1)]];
+        xv[q] = __ldg(p.h + (size_t)(k >= H ? kd >> 16 : kd & 0xFFFFu) * H + (k >= H ? k - H : k));
+      }
+    }
+  };
+  fetch(0);
+  // where this thread's output goes: the owner of unit k of a child, [rank][0][side JS + u] of its buffer
+  const int out = CELL == kRntn ? tid / p.s.TPA : 4 * (tid / SEG) + value_of_lane<SEG>(lane);
+  const bool sends = out < 2 * H && (CELL == kRntn ? tid % p.s.TPA == 0 : (lane & (SEG / 4 - 1)) == 0);
+  uint32_t send_addr = 0;
+  if (sends) {
+    const int side = out >= H, k = out - side * H, owner = k / JS;
+    const uint32_t local = smem_u32(dx) + 4u * (uint32_t)(rank * kND * 2 * JS + side * JS + k - owner * JS);
+    send_addr = cs > 1 ? peer_addr(local, (uint32_t)owner) : local;
+  }
+  const uint32_t send_turn = 4u * (uint32_t)(cs * kND * 2 * JS), send_node = 4u * (uint32_t)(2 * JS);
+  const int sum_i0 = tid / (2 * JS), sum_k0 = tid - sum_i0 * 2 * JS, sum_di = nt / (2 * JS), sum_dk = nt - sum_di * 2 * JS;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  TL_STAMP(trace, kTraceLevels - 1, 3);
+  if (resident)
+    for (int e = tid; e < walk.internal * 2 * JS; e += nt) {
+      const int q = e / (2 * JS), k = e - q * 2 * JS, side = k >= JS, u = k - side * JS;
+      const unsigned kd = kids[list[q]];
+      state[q * row + k] = u < jn ? __ldcg(p.dh + (size_t)(side ? kd >> 16 : kd & 0xFFFFu) * H + j0 + u) : 0.f;
+    }
+  // generic pointers: shared or global memory, written by this CTA only.  A root's dh is the classifier's.
+  auto dh_at = [&](unsigned code, int node, int u) -> float* {
+    return resident && code != kNoCaller ? state + (code >> 1) * row + (code & 1) * JS + u : p.dh + (size_t)node * H + j0 + u;
+  };
+  auto dc_at = [&](unsigned code, int node, int u) -> float* {
+    return resident ? state + (code >> 1) * row + 2 * JS + (code & 1) * JS + u : p.dc + (size_t)node * H + j0 + u;
+  };
+  cluster_sync(cs);                                      // every CTA of the cluster runs: its shared memory may be written
+  TL_STAMP(trace, kTraceLevels - 1, 4);
+  int turn = 0;
+  for (int d = 0; d < walk.depths; ++d) {
+    const int hi = start[d + 1];
+    for (int lo = start[d]; lo < hi; lo += nd, turn ^= 1) {
+      const int cnt = min(nd, hi - lo);
+      TL_STAMP(trace, d, 0);
+      if (mine && my_i < cnt) {
+        const int q = lo + my_i, node = list[q];
+        const unsigned code = par[q];
+        const float dhn = *dh_at(code, node, my_u);
+        float* z = in + my_i * in_row + my_u;
+        float* dz = p.dz + (size_t)node * G * H + j0 + my_u;
+        if constexpr (CELL == kLstm) {
+          const float gi = g[0], gl = g[1], gr = g[2], go = g[3], gu = g[4];
+          const float tc = tanhf(cn);
+          const float dcn = (d == 0 ? 0.f : *dc_at(code, node, my_u)) + dhn * go * (1.f - tc * tc);
+          const float v[5] = {dcn * gu * gi * (1.f - gi), dcn * cl * gl * (1.f - gl), dcn * cr * gr * (1.f - gr),
+                              dhn * tc * go * (1.f - go), dcn * gi * (1.f - gu * gu)};
+#pragma unroll
+          for (int k = 0; k < 5; ++k) { z[k * JS] = v[k]; dz[k * H] = v[k]; }
+          const unsigned kd = kids[node];
+          *dc_at(2u * q, (int)(kd & 0xFFFFu), my_u) = dcn * gl;          // every node has exactly one caller: plain stores
+          *dc_at(2u * q + 1u, (int)(kd >> 16), my_u) = dcn * gr;
+        } else {
+          const float v = dhn * (1.f - cn * cn);
+          z[0] = v;
+          dz[0] = v;
+        }
+      }
+      if constexpr (CELL == kRntn) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int e = tid + q * nt, i = e / (2 * H), k = e - i * 2 * H;
+          if (i < kND) xs[i * 2 * Hp + (k >= H ? Hp + k - H : k)] = xv[q];
+        }
+      }
+      fetch(lo + cnt);
+      __syncthreads();
+      TL_STAMP(trace, d, 1);
+      const uint32_t to = send_addr + (uint32_t)turn * send_turn;
+      auto send = [&](int i, float v) {
+        if (!sends) return;
+        if (cs > 1) st_cluster(to + (uint32_t)i * send_node, v);
+        else asm volatile("st.shared.f32 [%0], %1;" ::"r"(to + (uint32_t)i * send_node), "f"(v) : "memory");
+      };
+      if constexpr (CELL == kRntn) {
+        // thread (row a of x, every TPA-th chunk of columns): M_ab = sum_u S_u[a][b] dz_u, then sum_b M_ab x_b
+        const int tpa = p.s.TPA, q = tid % tpa;
+        for (int i = 0; i < cnt; ++i) {
+          const float4 z0 = *reinterpret_cast<const float4*>(in + i * in_row), z1 = *reinterpret_cast<const float4*>(in + i * in_row + 4);
+          const float z[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+          float v = 0.f;
+#pragma unroll
+          for (int c = 0; c < kRntnBC; ++c) {
+            const float4 x4 = *reinterpret_cast<const float4*>(xs + i * 2 * Hp + min(4 * (q + tpa * c), 2 * Hp - 4));
+            const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              float m = 0.f;
+#pragma unroll
+              for (int u = 0; u < kRntnJS; ++u) m = fmaf(w[(c * 4 + k) * kRntnJS + u], z[u], m);
+              v = fmaf(m, x[k], v);
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < kRntnJS; ++u) v = fmaf(w[4 * kRntnBC * kRntnJS + u], z[u], v);
+          for (int dd = tpa / 2; dd > 0; dd >>= 1) v += __shfl_xor_sync(kFull, v, dd);
+          send(i, v);
+        }
+      } else {
+        const float* const zin = in + 4 * (tid % SEG);
+        auto nodes = [&](auto n_const, int i0) {
+          constexpr int N = decltype(n_const)::value;
+          float acc[N][4];
+#pragma unroll
+          for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[i][u] = 0.f;
+#pragma unroll
+          for (int c = 0; c < BC; ++c) {
+            if (c >= p.s.BC) break;                      // the same for every thread
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+              const float4 x = *reinterpret_cast<const float4*>(zin + (i0 + i) * in_row + 4 * SEG * c);
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                acc[i][u] = fmaf(x.x, w[16 * c + u], acc[i][u]); acc[i][u] = fmaf(x.y, w[16 * c + 4 + u], acc[i][u]);
+                acc[i][u] = fmaf(x.z, w[16 * c + 8 + u], acc[i][u]); acc[i][u] = fmaf(x.w, w[16 * c + 12 + u], acc[i][u]);
+              }
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < N; ++i) {
+            lane_sums4<SEG>(acc[i], lane);
+            send(i0 + i, acc[i][0]);
+          }
+        };
+        int i = 0;
+        for (; i + 1 < cnt; i += 2) nodes(std::integral_constant<int, 2>{}, i);
+        if (i < cnt) nodes(std::integral_constant<int, 1>{}, i);
+      }
+      TL_STAMP(trace, d, 2);
+      cluster_sync(cs);
+      TL_STAMP(trace, d, 3);
+      const float* got = dx + turn * cs * kND * 2 * JS;
+      for (int i = sum_i0, k = sum_k0; i < cnt;) {
+        const int side = k >= JS, u = k - side * JS;
+        float v = 0.f;
+#pragma unroll 8
+        for (int c = 0; c < cs; ++c) v += got[(c * kND + i) * 2 * JS + k];
+        const unsigned kd = resident ? 0u : kids[list[lo + i]];
+        float* at = dh_at((unsigned)(2 * (lo + i) + side), (int)(side ? kd >> 16 : kd & 0xFFFFu), u);
+        if (u < jn) *at = *at + v;
+        i += sum_di;
+        k += sum_dk;
+        if (k >= 2 * JS) { k -= 2 * JS; ++i; }
+      }
+      TL_STAMP(trace, d, 4);
+    }
+    __syncthreads();                                     // the next depth's dh (this CTA's units) is complete
+    TL_STAMP(trace, d, 5);
+  }
+  // leaves: their own gate gradients (no forget gates), or for the other cells dh where the gradient kernel reads it
+  for (int e = tid; e < walk.leaves * JS; e += nt) {
+    const int q = e / JS, u = e - q * JS;
+    if (u >= jn) continue;
+    const unsigned code = leaf_par[q];
+    const int node = leaf[q];
+    const size_t at = (size_t)node * H + j0 + u;
+    if constexpr (CELL == kLstm) {
+      const float* gp = p.gates + (size_t)node * 5 * H + j0 + u;
+      const float gi = __ldg(gp), go = __ldg(gp + 3 * H), gu = __ldg(gp + 4 * H), tc = tanhf(__ldg(p.c + at));
+      const float dhn = *dh_at(code, node, u);
+      const float dcn = (code == kNoCaller ? 0.f : *dc_at(code, node, u)) + dhn * go * (1.f - tc * tc);
+      float* dz = p.dz + (size_t)node * 5 * H + j0 + u;
+      dz[0] = dcn * gu * gi * (1.f - gi);
+      dz[H] = 0.f;
+      dz[2 * H] = 0.f;
+      dz[3 * H] = dhn * tc * go * (1.f - go);
+      dz[4 * H] = dcn * gi * (1.f - gu * gu);
+    } else if (resident) {
+      p.dh[at] = *dh_at(code, node, u);
+    }
+  }
+  cluster_sync(cs);                                      // no CTA leaves while a peer may still write to it
+}
+
+// ---- dW, db, dV and the embedding rows ------------------------------------------------------------ //
+// One tile of gradient rows (32 of the R rows) x 32 units per CTA and run of nodes: sum over the internal
+// nodes of P_r dz_j.  A product row's sum belongs to V_j[a][b] and V_j[b][a] alike.  The runs are as long
+// as two CTAs per SM allow, because every run ends in one atomic add per element.  CTAs behind the tiles
+// add dh of the leaves to the rows of their tokens.
+constexpr int GR = 32, GU = 32, GN = 64, kGT = 256;
+struct GradParams {
+  int n, H, K, Q, R, tiles_u, tiles, splits, vocab;
+  const int *left, *right, *token, *order, *level_offset, *tok_slot;
+  const float *h, *dh, *dz;
+  float *dW, *db, *dV, *dEmb_rows;
+  DevStatus* st;
+};
+__global__ void __launch_bounds__(kGT) k_rec_grads(GradParams p) {
+  __shared__ float As[GN][GR];
+  __shared__ __align__(16) float Ds[GN][GU];
+  __shared__ int s_node[GN], s_l[GN], s_r[GN];
+  __shared__ int s_a[GR], s_b[GR];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = p.H, K = p.K;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (p.st->n_levels < 1 || (ld_volatile(&p.st->status) != 0 && ld_volatile(&p.st->status) != TREELSTM_ERR_LABEL_OUT_OF_RANGE)) return;
+  const int n_leaves = p.level_offset[1];
+  const int grad_ctas = p.tiles * p.splits;
+  if ((int)blockIdx.x >= grad_ctas) {
+    const int warps = ((int)gridDim.x - grad_ctas) * (kGT / 32);
+    for (int q = ((int)blockIdx.x - grad_ctas) * (kGT / 32) + warp; q < n_leaves; q += warps) {
+      const int node = chk(p.st, p.order[q], p.n);
+      const int row = p.tok_slot[chk(p.st, p.token[node], p.vocab)];
+      for (int u = lane; u < H; u += 32) atomicAdd(p.dEmb_rows + (size_t)row * H + u, __ldg(p.dh + (size_t)node * H + u));
+    }
+    return;
+  }
+  const int tile = (int)blockIdx.x % p.tiles, split = (int)blockIdx.x / p.tiles;
+  const int r0 = (tile / p.tiles_u) * GR, u0 = (tile % p.tiles_u) * GU;
+  const int internal = p.n - n_leaves, per = (internal + p.splits - 1) / p.splits;
+  const int q_lo = n_leaves + split * per, q_hi = min(p.n, q_lo + per);
+  if (tid < GR) {                          // the two entries of x behind a row (b < 0: a linear row)
+    int r = r0 + tid, a = -1, b = -1;
+    if (r < p.Q) {
+      a = 0;
+      while (r >= K - a) { r -= K - a; ++a; }
+      b = a + r;
+    } else if (r < p.R) {
+      a = r - p.Q;
+    }
+    s_a[tid] = a; s_b[tid] = b;
+  }
+  float acc[4] = {}, accb[4] = {};
+  for (int q0 = q_lo; q0 < q_hi; q0 += GN) {
+    __syncthreads();
+    if (tid < GN) {
+      const int node = chk(p.st, p.order[min(q0 + tid, q_hi - 1)], p.n);
+      s_node[tid] = node; s_l[tid] = chk(p.st, p.left[node], p.n); s_r[tid] = chk(p.st, p.right[node], p.n);
+    }
+    __syncthreads();
+    const int a = s_a[lane], b = s_b[lane];
+    float va[GN / 8], vb[GN / 8], vd[GN / 8];
+#pragma unroll
+    for (int e = 0; e < GN / 8; ++e) {     // loads first
+      const int i = warp + 8 * e;
+      const int aa = max(a, 0), bb = max(b, 0);
+      va[e] = __ldg(p.h + (size_t)(aa < H ? s_l[i] : s_r[i]) * H + (aa < H ? aa : aa - H));
+      vb[e] = p.Q ? __ldg(p.h + (size_t)(bb < H ? s_l[i] : s_r[i]) * H + (bb < H ? bb : bb - H)) : 1.f;
+      vd[e] = __ldg(p.dz + (size_t)s_node[i] * H + min(u0 + lane, H - 1));
+    }
+#pragma unroll
+    for (int e = 0; e < GN / 8; ++e) {
+      const int i = warp + 8 * e;
+      const bool in = q0 + i < q_hi;
+      As[i][lane] = in && a >= 0 ? (b >= 0 ? va[e] * vb[e] : va[e]) : 0.f;
+      Ds[i][lane] = in && u0 + lane < H ? vd[e] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int i = 0; i < GN; ++i) {         // thread: row `lane`, units 4 warp .. 4 warp + 3
+      const float x = As[i][lane];
+      const float4 d = *reinterpret_cast<const float4*>(&Ds[i][4 * warp]);
+      acc[0] = fmaf(x, d.x, acc[0]); acc[1] = fmaf(x, d.y, acc[1]);
+      acc[2] = fmaf(x, d.z, acc[2]); acc[3] = fmaf(x, d.w, acc[3]);
+      accb[0] += d.x; accb[1] += d.y; accb[2] += d.z; accb[3] += d.w;
+    }
+  }
+  if (q_lo >= q_hi) return;
+  const int a = s_a[lane], b = s_b[lane];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int u = u0 + 4 * warp + q;
+    if (u >= H || a < 0) continue;
+    if (b < 0) {
+      atomicAdd(p.dW + (size_t)a * H + u, acc[q]);
+      if (a == 0) atomicAdd(p.db + u, accb[q]);
+    } else {
+      float* v = p.dV + (size_t)u * K * K;
+      atomicAdd(v + (size_t)a * K + b, acc[q]);
+      if (a != b) atomicAdd(v + (size_t)b * K + a, acc[q]);
+    }
+  }
+}
+
+
+// ---- register images and launches ------------------------------------------------------------------ //
+__global__ void k_trees_pack(int backward, int cell, int H, int E, int words, int threads, TreesShape s, const ushort2* pairs,
+                             const float* src, float* out) {
+  const int total = s.cs * words * threads;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const int t = i % threads, w = (i / threads) % words, rank = i / threads / words;
+    const WeightAt at = backward ? bwd_weight(cell, H, E, s, rank, t, w) : fwd_weight(cell, H, E, s, rank, t, w, pairs);
+    float v = 0.f;
+    if (at.i0 >= 0) v = src[at.i0];
+    if (at.i1 >= 0) v += src[at.i1];
+    out[i] = v;
+  }
+}
+
+constexpr int kLstmRC = 4, kRnnRC = 4, kRntnRC = 3;       // forward chunks per thread (U = 5, 4, 4)
+int fwd_words(int cell) { return cell == kLstm ? 20 * kLstmRC : (cell == kRnn ? 16 * kRnnRC : 16 * kRntnRC); }
+int bwd_chunks(int cell, const TreesShape& s) { return cell == kLstm && s.bseg == 4 ? 5 : 4; }
+int bwd_words(int cell, const TreesShape& s) { return cell == kRntn ? kRntnBwdWords : 16 * bwd_chunks(cell, s); }
+
+// One cluster size: does the slice fit the registers?
+bool shape_fits(int cell, int H, int cs, TreesShape& s) {
+  const int Hp = round_up(H, 4), G = cell == kLstm ? 5 : 1;
+  s.cs = cs;
+  s.JS = (H + cs - 1) / cs;
+  s.U = cell == kLstm ? 5 : 4;
+  if (NT * s.JS > kFwdT) return false;
+  if (cell == kRntn) {
+    for (s.JL = 1; 4 * s.JL < s.JS; s.JL *= 2) {}
+    s.nc = kRntnRC;
+    s.nseg = (s.chunks + s.nc - 1) / s.nc;
+    if (s.nseg * s.JL > kFwdT) return false;
+    s.bthreads = kRntnT; s.bseg = 1; s.BC = kRntnBC;
+    for (s.TPA = 32; s.TPA * 2 * H > kRntnT; s.TPA /= 2) {}
+    return s.JS <= kRntnJS;
+  }
+  s.chunks = 2 * Hp / 4;
+  s.JL = cell == kLstm ? s.JS : (s.JS + 3) / 4;
+  s.nc = cell == kLstm ? kLstmRC : kRnnRC;                // whole segments: as few partial sums as the registers allow
+  s.nseg = (s.chunks + s.nc - 1) / s.nc;
+  if (s.nseg * s.JL > kFwdT) return false;
+  // backward: eight lanes per four outputs where the threads allow it
+  const int groups = (2 * H + 3) / 4;
+  s.bseg = groups * 8 <= kBwdT ? 8 : 4;
+  if (groups * s.bseg > kBwdT) return false;
+  s.bthreads = round_up(groups * s.bseg, 32);
+  if (s.bthreads < s.JS) s.bthreads = round_up(s.JS, 32);
+  s.BC = ((G * s.JS + 3) / 4 + s.bseg - 1) / s.bseg;
+  return s.BC <= bwd_chunks(cell, s);
+}
+
+using TreesKernel = void (*)(const TreesParams);
+TreesKernel forward_kernel(int cell) {
+  return cell == kRntn ? k_trees_forward<kRntn, 4, kRntnRC> : (cell == kRnn ? k_trees_forward<kRnn, 4, kRnnRC> : k_trees_forward<kLstm, 5, kLstmRC>);
+}
+TreesKernel backward_kernel(int cell, const TreesShape& s) {
+  if (cell == kRntn) return k_trees_backward<kRntn, 8, 1, kRntnT>;
+  if (cell == kRnn) return s.bseg == 8 ? k_trees_backward<kRnn, 8, 4, kBwdT> : k_trees_backward<kRnn, 4, 4, 512>;
+  return s.bseg == 8 ? k_trees_backward<kLstm, 8, 4, kBwdT> : k_trees_backward<kLstm, 4, 5, 512>;
+}
+
+TreesParams trees_params(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
+                         float* c, void* ws, const WsLayout& lay) {
+  char* base = static_cast<char*>(ws);
+  TreesParams p{};
+  p.n = n; p.H = ctx->H; p.E = ctx->E; p.vocab = ctx->vocab; p.Hp = round_up(ctx->H, 4); p.s = ctx->trees.s;
+  p.chk_counts = check_counters(ws, lay);
+  p.left = left; p.right = right; p.token = token;
+  p.emb = ctx->emb; p.b = ctx->b; p.pairs = ctx->trees.pairs;
+  p.h = h; p.c = c;
+  p.dh = reinterpret_cast<float*>(base + lay.dh);
+  p.dc = reinterpret_cast<float*>(base + lay.dc);
+  p.dz = reinterpret_cast<float*>(base + lay.dz);
+  p.st = reinterpret_cast<DevStatus*>(base + lay.status);
+  p.trace = nullptr;
+#ifdef TREELSTM_TRACE
+  p.trace = reinterpret_cast<long long*>(base + lay.trace);   // forward: first table, backward: second
+#endif
+  return p;
+}
+
+// As many clusters as the device holds at once (they do not wait for one another, but trees dealt to a cluster that
+// starts late end late).  `after_running`: the kernel may start while the one ahead of it on the stream still runs (it
+// waits on the device for its end).
+int launch_trees(treelstm* ctx, TreesKernel kernel, const TreesParams& p, int threads, int clusters, bool after_running, cudaStream_t stream) {
+  const int cap = ctx->opt.max_ctas / p.s.cs;
+  if (ctx->opt.max_ctas > 0 && clusters > cap) clusters = cap;
+  if (clusters > p.n) clusters = p.n;                    // (a tree is a node at least)
+  if (clusters < 1) clusters = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(clusters * p.s.cs); cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = kSmemMax; cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = p.s.cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = after_running ? 1 : 0;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, kernel, p));
+  ctx->launches += 1;
+  return TREELSTM_OK;
+}
+
+}  // namespace
+
+int init_trees(treelstm* ctx, cudaStream_t stream) {
+  auto& t = ctx->trees;
+  auto& s = t.s;
+  const int H = ctx->H, E = ctx->E, cell = ctx->cell;
+  if (!t.known) {
+    t.known = true;
+    t.ok = false;
+    if (H > (cell == kRntn ? kRntnMaxH : 256)) return TREELSTM_OK;   // the level kernels stream the weights instead
+    if (cell == kRntn) {
+      const int Hp = round_up(H, 4), K = 2 * Hp;
+      ushort2* pairs = new (std::nothrow) ushort2[(size_t)(K + 1) * (K / 4)];
+      if (!pairs) return TREELSTM_ERR_INVALID_ARG;
+      for (int a = 0; a < K; ++a)                        // products x_a x_b, b >= a, four b at a time; then x itself
+        for (int b4 = a / 4 * 4; a % Hp < H && b4 < K; b4 += 4) pairs[s.chunks++] = make_ushort2((unsigned short)a, (unsigned short)b4);
+      for (int b4 = 0; b4 < K; b4 += 4) pairs[s.chunks++] = make_ushort2(0xFFFF, (unsigned short)b4);
+      cudaError_t e = cudaMalloc((void**)&t.pairs, sizeof(ushort2) * s.chunks);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(t.pairs, pairs, sizeof(ushort2) * s.chunks, cudaMemcpyHostToDevice, stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+      delete[] pairs;
+      TL_CUDA(ctx, e);
+    }
+    // (TreeRNN: four CTAs at least from H = 64 on: 25 trees, H = 128, forward / backward on clusters of 1, 2, 4, 8 CTAs:
+    // 58.6 / 142, 60.6 / 133, 56.0 / 124, 67.2 / 122 us)
+    for (int cs = cell == kRnn && H >= 64 ? 4 : 1; cs <= 16 && !t.ok; cs *= 2) t.ok = shape_fits(cell, H, cs, s);
+    if (!t.ok) return TREELSTM_OK;
+    for (int back = 0; back < 2; ++back) {
+      TreesKernel k = back ? backward_kernel(cell, s) : forward_kernel(cell);
+      TL_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
+      if (s.cs > 8) TL_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = s.cs; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+      cfg.gridDim = dim3(s.cs); cfg.blockDim = dim3(back ? s.bthreads : kFwdT); cfg.dynamicSmemBytes = kSmemMax;
+      cfg.attrs = &at; cfg.numAttrs = 1;
+      int clusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) != cudaSuccess || clusters < 1) {
+        cudaGetLastError();
+        t.ok = false;
+        return TREELSTM_OK;
+      }
+      (back ? t.clusters_bwd : t.clusters) = clusters;
+    }
+    const size_t cta = sizeof(float) * (size_t)s.cs;
+    TL_CUDA(ctx, cudaMalloc((void**)&t.Wf, cta * kFwdT * fwd_words(cell)));
+    TL_CUDA(ctx, cudaMalloc((void**)&t.Wb, cta * s.bthreads * bwd_words(cell, s)));
+  }
+  if (!t.ok) return TREELSTM_OK;
+  const float* src = cell == kLstm ? ctx->W : ctx->Wcat;
+  k_trees_pack<<<592, 256, 0, stream>>>(0, cell, H, E, fwd_words(cell), kFwdT, s, t.pairs, src, t.Wf);
+  k_trees_pack<<<592, 256, 0, stream>>>(1, cell, H, E, bwd_words(cell, s), s.bthreads, s, t.pairs, src, t.Wb);
+  TL_CUDA(ctx, cudaGetLastError());
+  return TREELSTM_OK;
+}
+
+// Forests whose tables fit shared memory; beyond that the level kernels are used.
+bool trees_take(const treelstm* ctx, int n) {
+  const auto& s = ctx->trees.s;
+  return ctx->trees.ok && n >= 1 && n <= 32767 && trees_smem(n, fwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0 &&
+         trees_smem(n, bwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0;
+}
+
+int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
+                         float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream) {
+  const auto& s = ctx->trees.s;
+  TreesParams p = trees_params(ctx, n, left, right, token, h, c, ws, lay);
+  p.W = ctx->trees.Wf;
+  p.gates = save_gates ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
+  if (ctx->cell == kLstm) {
+    LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->W, ctx->b, h, c, p.gates};
+    const int tiles_u = (ctx->H + kLeafU - 1) / kLeafU;
+    const int small = (n + 63) / 64 * tiles_u;           // 32-row tiles until they take several rounds
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kLeafT); cfg.stream = stream;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = after_running ? 1 : 0;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    if (small <= 4 * ctx->sm_count) {
+      cfg.gridDim = dim3(small);
+      TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_leaves_fp32<32>, q));
+    } else {
+      cfg.gridDim = dim3((n + 127) / 128 * tiles_u);
+      TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_leaves_fp32<64>, q));
+    }
+    ctx->launches += 1;
+  }
+  return launch_trees(ctx, forward_kernel(ctx->cell), p, kFwdT, after_running ? max(1, (ctx->sm_count - 1) / s.cs < ctx->trees.clusters ? (ctx->sm_count - 1) / s.cs : ctx->trees.clusters) : ctx->trees.clusters, after_running, stream);
+}
+
+int launch_backward_trees(treelstm* ctx, cudaStream_t stream) {
+  const auto& L = ctx->last;
+  TreesParams p = trees_params(ctx, L.n, L.left, L.right, L.token, L.h, L.c, L.ws, L.lay);
+  p.W = ctx->trees.Wb;
+  p.gates = reinterpret_cast<float*>(static_cast<char*>(L.ws) + L.lay.gates);
+  if (p.trace) p.trace += kTraceSlots * kTraceLevels;
+  return launch_trees(ctx, backward_kernel(ctx->cell, p.s), p, p.s.bthreads, ctx->trees.clusters_bwd, true, stream);
+}
+
+int launch_rec_grads(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb_rows, const int* tok_slot, cudaStream_t stream) {
+  const auto& L = ctx->last;
+  char* base = static_cast<char*>(L.ws);
+  GradParams g{};
+  g.n = L.n; g.H = ctx->H; g.K = 2 * ctx->H; g.Q = ctx->cell == kRntn ? g.K * (g.K + 1) / 2 : 0; g.R = g.Q + g.K; g.vocab = ctx->vocab;
+  g.left = L.left; g.right = L.right; g.token = L.token; g.order = L.order; g.level_offset = L.level_offset;
+  g.tok_slot = tok_slot; g.h = L.h;
+  g.dh = reinterpret_cast<const float*>(base + L.lay.dh); g.dz = reinterpret_cast<const float*>(base + L.lay.dz);
+  g.dW = dW; g.db = db; g.dV = dV; g.dEmb_rows = dEmb_rows;
+  g.st = reinterpret_cast<DevStatus*>(base + L.lay.status);
+  g.tiles_u = (ctx->H + GU - 1) / GU;
+  g.tiles = ((g.R + GR - 1) / GR) * g.tiles_u;
+  const int most = (L.n / 2 + GN - 1) / GN;               // runs of at least one chunk
+  g.splits = 2 * ctx->sm_count / g.tiles;
+  if (g.splits > most) g.splits = most;
+  if (g.splits < 1) g.splits = 1;
+  const int leaf_ctas = L.n / 16 < 64 ? L.n / 16 + 1 : 64;
+  k_rec_grads<<<g.tiles * g.splits + leaf_ctas, kGT, 0, stream>>>(g);
+  TL_CUDA(ctx, cudaGetLastError());
+  ctx->launches += 1;
+  return TREELSTM_OK;
+}
+
+}  // namespace tl

@@ -162,3 +162,20 @@ def test_training_step_on_small_grids(ctas):
     model.set_option(binding.OPT_MAX_CTAS, ctas)
     res = _train_step(model, forest, labels, binding.PERSISTENT)
     _compare(res, ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("H,E,n_trees,hi", [(25, 9, 40, 30), (103, 40, 20, 30), (161, 30, 12, 24), (256, 70, 8, 20), (257, 20, 3, 12), (150, 520, 2, 600)])
+def test_training_step_at_the_limits_of_the_tree_kernels(H, E, n_trees, hi):
+    """hidden sizes at which the cluster grows and at which the tree kernels end; more trees than clusters; states
+    that do not fit the shared memory of a cluster; long embedding rows"""
+    rng = np.random.default_rng(800 + H)
+    params = fg.draw_params(rng, H, E, 90, emb_dist="normal", emb_scale=0.3, w_scale=1.0 / np.sqrt(H), n_classes=3)
+    forest = fg.concat_forests([fg.random_forest(rng, n_trees, 1 if hi < 100 else hi - 1, hi, 90),
+                                fg.forest_from_shapes([fg.left_chain_shape(9), fg.balanced_shape(32)], rng, 90)])
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    res = _train_step(model, forest, labels, binding.PERSISTENT)
+    assert util.max_abs(res["h"], ref["h"]) < util.TOL["fp32"]
+    _compare(res, ref, util.TOL["fp32"])

@@ -175,3 +175,25 @@ def test_recursive_training_edge_cases():
     with pytest.raises(binding.TreeLSTMError):
         model.backward(util.to_dev(np.zeros(forest.n_nodes, np.int32)), forest.n_leaves)
     model.close()
+
+
+@pytest.mark.parametrize("cell,H,n_trees,hi", [
+    (binding.CELL_TREERNN, 63, 9, 40), (binding.CELL_TREERNN, 64, 9, 40), (binding.CELL_TREERNN, 254, 6, 30), (binding.CELL_TREERNN, 257, 6, 30),
+    (binding.CELL_TREERNN, 128, 300, 12), (binding.CELL_RNTN, 1, 5, 9), (binding.CELL_RNTN, 32, 60, 20), (binding.CELL_RNTN, 33, 5, 20)])
+def test_training_step_at_the_limits_of_the_tree_kernels(cell, H, n_trees, hi):
+    """sizes at which the cluster grows and at which the tree kernels end; more trees than clusters; a depth wider
+    than a pass; single leaves and chains among the trees"""
+    rng = np.random.default_rng(600 + H)
+    tensor = cell == binding.CELL_RNTN
+    p = fg.draw_recursive_params(rng, H, 90, tensor=tensor, emb_scale=0.8, w_scale=1.0 / np.sqrt(2 * H), v_scale=1.0 / (2 * H))
+    forest = fg.concat_forests([fg.random_forest(rng, n_trees, 1, hi, 90),
+                                fg.forest_from_shapes([fg.left_chain_shape(17), fg.balanced_shape(32)], rng, 90)])
+    _training_step(cell, p, forest, binding.PERSISTENT)
+
+
+def test_states_that_do_not_fit_shared_memory():
+    """two trees of a thousand leaves each: the states of a cluster go through L2"""
+    rng = np.random.default_rng(700)
+    p = fg.draw_recursive_params(rng, 130, 90, tensor=False, emb_scale=0.8, w_scale=1.0 / np.sqrt(260))
+    forest = fg.random_forest(rng, 2, 1000, 1001, 90)
+    _training_step(binding.CELL_TREERNN, p, forest, binding.PERSISTENT)
