@@ -1,6 +1,7 @@
 // extern "C" entry points of libtreelstm_b200 (declared in include/treelstm.h): argument checks,
 // parameter copies, workspace layout and the launch sequence of one forward / backward call.
 #include <new>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -62,7 +63,7 @@ int copy_params(treelstm* ctx, const float* emb, const float* W, const float* b,
     int rc = pack_weights_bf16(ctx, s);
     if (rc != TREELSTM_OK) return rc;
   }
-  const int rc = init_trees(ctx, s);
+  const int rc = pack_trees(ctx, s);
   if (rc != TREELSTM_OK) return rc;
   TL_CUDA(ctx, cudaStreamSynchronize(s));
   return TREELSTM_OK;
@@ -192,19 +193,31 @@ int treelstm_create(treelstm_t** out, int H, int E, int vocab, const float* emb,
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const size_t Hs = H, Es = E, V = vocab;
   auto fail = [&](int rc) { treelstm_destroy(ctx); return rc; };
-  if (cudaMalloc((void**)&ctx->emb, sizeof(float) * V * Es) != cudaSuccess ||
-      cudaMalloc((void**)&ctx->W, sizeof(float) * (Es + 2 * Hs) * 5 * Hs) != cudaSuccess ||
-      cudaMalloc((void**)&ctx->b, sizeof(float) * 5 * Hs) != cudaSuccess ||
-      cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess)
-    return fail(TREELSTM_ERR_CUDA);
-  if (precision == TREELSTM_BF16) {
-    const size_t Hp = ctx->Hp, Ep = ctx->Ep, groups = Hp / kUnitGroup;
-    if (cudaMalloc((void**)&ctx->emb_bf, 2 * V * Ep) != cudaSuccess ||
-        cudaMalloc((void**)&ctx->Wp_h, 2 * groups * 40 * 2 * Hp) != cudaSuccess ||
-        cudaMalloc((void**)&ctx->Wp_x, 2 * groups * 24 * Ep) != cudaSuccess ||
-        cudaMalloc((void**)&ctx->bp_h, 4 * groups * 40) != cudaSuccess ||
-        cudaMalloc((void**)&ctx->bp_x, 4 * groups * 24) != cudaSuccess)
+  const size_t Hp = ctx->Hp, Ep = ctx->Ep, groups = Hp / kUnitGroup;
+  const size_t trees = plan_trees(ctx);
+  // one allocation (a call costs about a millisecond for every couple of megabytes it maps)
+  for (int pass = 0; pass < 2; ++pass) {
+    size_t off = 0;
+    auto take = [&](auto& ptr, size_t bytes) {
+      if (pass) ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(ctx->memory + off);
+      off += round_up_sz(bytes, 256);
+    };
+    unsigned char* images = nullptr;
+    take(ctx->emb, sizeof(float) * V * Es);
+    take(ctx->W, sizeof(float) * (Es + 2 * Hs) * 5 * Hs);
+    take(ctx->b, sizeof(float) * 5 * Hs);
+    if (precision == TREELSTM_BF16) {
+      take(ctx->emb_bf, 2 * V * Ep);
+      take(ctx->Wp_h, 2 * groups * 40 * 2 * Hp);
+      take(ctx->Wp_x, 2 * groups * 24 * Ep);
+      take(ctx->bp_h, 4 * groups * 40);
+      take(ctx->bp_x, 4 * groups * 24);
+    }
+    take(images, trees);
+    if (!pass && (cudaMalloc((void**)&ctx->memory, off) != cudaSuccess ||
+                  cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess))
       return fail(TREELSTM_ERR_CUDA);
+    if (pass && init_trees(ctx, images, s) != TREELSTM_OK) return fail(TREELSTM_ERR_CUDA);
   }
   int rc = init_schedule_attributes(ctx);
   if (rc == TREELSTM_OK && precision == TREELSTM_BF16) rc = init_tc_attributes(ctx);
@@ -239,18 +252,22 @@ int treelstm_create_recursive(treelstm_t** out, int cell, int H, int vocab, cons
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const size_t Hs = H, V_ = vocab, K2 = 2 * Hs, KQ = cell == TREELSTM_CELL_RNTN ? K2 * K2 : 0;
   auto fail = [&](int rc) { treelstm_destroy(ctx); return rc; };
-  if (cudaMalloc((void**)&ctx->emb, sizeof(float) * V_ * Hs) != cudaSuccess ||
-      cudaMalloc((void**)&ctx->Wcat, sizeof(float) * (KQ + K2) * Hs) != cudaSuccess ||
-      cudaMalloc((void**)&ctx->b, sizeof(float) * Hs) != cudaSuccess ||
+  const size_t trees = plan_trees(ctx), emb_bytes = round_up_sz(sizeof(float) * V_ * Hs, 256),
+               w_bytes = round_up_sz(sizeof(float) * (KQ + K2) * Hs, 256), b_bytes = round_up_sz(sizeof(float) * Hs, 256);
+  if (cudaMalloc((void**)&ctx->memory, emb_bytes + w_bytes + b_bytes + trees) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess)
     return fail(TREELSTM_ERR_CUDA);
+  ctx->emb = reinterpret_cast<float*>(ctx->memory);
+  ctx->Wcat = reinterpret_cast<float*>(ctx->memory + emb_bytes);
+  ctx->b = reinterpret_cast<float*>(ctx->memory + emb_bytes + w_bytes);
+  if (init_trees(ctx, ctx->memory + emb_bytes + w_bytes + b_bytes, s) != TREELSTM_OK) return fail(TREELSTM_ERR_CUDA);
   int rc = init_schedule_attributes(ctx);
   if (rc != TREELSTM_OK) return fail(rc);
   if (cudaMemcpyAsync(ctx->emb, emb, sizeof(float) * V_ * Hs, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
       cudaMemcpyAsync(ctx->b, b, sizeof(float) * Hs, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return fail(TREELSTM_ERR_CUDA);
   rc = pack_weights_rec(ctx, W, V, s);
-  if (rc == TREELSTM_OK) rc = init_trees(ctx, s);
+  if (rc == TREELSTM_OK) rc = pack_trees(ctx, s);
   if (rc != TREELSTM_OK) return fail(rc);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(TREELSTM_ERR_CUDA);
   *out = ctx;
@@ -618,9 +635,7 @@ int treelstm_last_cuda_error(const treelstm_t* ctx) { return ctx ? ctx->cuda_err
 
 int treelstm_destroy(treelstm_t* ctx) {
   if (!ctx) return TREELSTM_OK;
-  cudaFree(ctx->emb); cudaFree(ctx->W); cudaFree(ctx->b); cudaFree(ctx->Wc); cudaFree(ctx->bc); cudaFree(ctx->Wcat); 
-  cudaFree(ctx->trees.Wf); cudaFree(ctx->trees.Wb); cudaFree(ctx->trees.pairs);
-  cudaFree(ctx->emb_bf); cudaFree(ctx->Wp_h); cudaFree(ctx->Wp_x); cudaFree(ctx->bp_h); cudaFree(ctx->bp_x);
+  cudaFree(ctx->memory); cudaFree(ctx->Wc); cudaFree(ctx->bc);
   if (ctx->host_level_offset) cudaFreeHost(ctx->host_level_offset);
   if (ctx->host_status) cudaFreeHost(ctx->host_status);
   free_host_path(ctx);

@@ -112,6 +112,8 @@ struct treelstm {
   int device = 0;
   int sm_count = 0;
 
+  unsigned char* memory = nullptr;  // one allocation: everything the library owns on the device but the classifier
+
   // fp32 parameters (library-owned device copies)
   float* emb = nullptr;  // [vocab][E]
   float* W = nullptr;    // [E+2H][5H]
@@ -138,7 +140,7 @@ struct treelstm {
 
   // the fp32 tree kernels (trees_fp32.cu)
   struct Trees {
-    bool ok = false, known = false;
+    bool ok = false;
     tl::TreesShape s;
     float *Wf = nullptr, *Wb = nullptr;                 // register images of the weights
     int clusters = 0, clusters_bwd = 0;                 // that the device holds at once
@@ -215,7 +217,9 @@ int launch_forward_rec(treelstm* ctx, int n, const int32_t* left, const int32_t*
                        const WsLayout& lay, cudaStream_t stream);
 
 // trees_fp32.cu (all cells in fp32, trees dealt out to clusters)
-int init_trees(treelstm* ctx, cudaStream_t stream);      // shapes and register images; again after the weights changed
+size_t plan_trees(treelstm* ctx);                        // bytes of the register images of the weights (0: not available)
+int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream);
+int pack_trees(treelstm* ctx, cudaStream_t stream);      // after the weights have changed
 bool trees_take(const treelstm* ctx, int n);
 int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
                          float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);

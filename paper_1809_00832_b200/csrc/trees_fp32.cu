@@ -24,7 +24,6 @@
 // itself, from the child arrays in shared memory, so nothing here waits for the scheduler before its end.  (A
 // malformed forest is the scheduler's to report; here every index is clamped and every list bounded, so that
 // whatever the arrays hold the walk ends.)  Clusters take roots q, q + Q, ... in id order.
-#include <new>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1053,6 +1052,21 @@ TreesKernel backward_kernel(int cell, const TreesShape& s) {
   return s.bseg == 8 ? k_trees_backward<kLstm, 8, 4, kBwdT> : k_trees_backward<kLstm, 4, 5, 512>;
 }
 
+// RNTN chunks of row a of x: products x_a x_b, b >= a, four b at a time; a = 2 Hp stands for x itself
+__host__ __device__ inline int pair_chunks(int a, int H, int Hp) { return a == 2 * Hp ? Hp / 2 : (a % Hp < H ? Hp / 2 - a / 4 : 0); }
+__global__ void k_trees_pairs(int H, ushort2* pairs) {
+  const int Hp = (H + 3) & ~3;
+  for (int a = 0, at = 0; a <= 2 * Hp; ++a)
+    for (int c = 0, n = pair_chunks(a, H, Hp); c < n; ++c)
+      pairs[at++] = a == 2 * Hp ? make_ushort2(0xFFFF, (unsigned short)(4 * c)) : make_ushort2((unsigned short)a, (unsigned short)(4 * (a / 4 + c)));
+}
+size_t images_bytes(const treelstm* ctx, int what) {     // forward image, backward image, chunk operands
+  const auto& s = ctx->trees.s;
+  const size_t cta = sizeof(float) * (size_t)s.cs;
+  return round_up_sz(what == 0 ? cta * kFwdT * fwd_words(ctx->cell) : (what == 1 ? cta * s.bthreads * bwd_words(ctx->cell, s)
+                                                                               : sizeof(ushort2) * (ctx->cell == kRntn ? s.chunks : 0)), 256);
+}
+
 TreesParams trees_params(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
                          float* c, void* ws, const WsLayout& lay) {
   char* base = static_cast<char*>(ws);
@@ -1097,54 +1111,52 @@ int launch_trees(treelstm* ctx, TreesKernel kernel, const TreesParams& p, int th
 
 }  // namespace
 
-int init_trees(treelstm* ctx, cudaStream_t stream) {
+// Chooses the shapes and says how much device memory the register images take (0: the level kernels stream the
+// weights instead).
+size_t plan_trees(treelstm* ctx) {
   auto& t = ctx->trees;
   auto& s = t.s;
-  const int H = ctx->H, E = ctx->E, cell = ctx->cell;
-  if (!t.known) {
-    t.known = true;
-    t.ok = false;
-    if (H > (cell == kRntn ? kRntnMaxH : 256)) return TREELSTM_OK;   // the level kernels stream the weights instead
-    if (cell == kRntn) {
-      const int Hp = round_up(H, 4), K = 2 * Hp;
-      ushort2* pairs = new (std::nothrow) ushort2[(size_t)(K + 1) * (K / 4)];
-      if (!pairs) return TREELSTM_ERR_INVALID_ARG;
-      for (int a = 0; a < K; ++a)                        // products x_a x_b, b >= a, four b at a time; then x itself
-        for (int b4 = a / 4 * 4; a % Hp < H && b4 < K; b4 += 4) pairs[s.chunks++] = make_ushort2((unsigned short)a, (unsigned short)b4);
-      for (int b4 = 0; b4 < K; b4 += 4) pairs[s.chunks++] = make_ushort2(0xFFFF, (unsigned short)b4);
-      cudaError_t e = cudaMalloc((void**)&t.pairs, sizeof(ushort2) * s.chunks);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(t.pairs, pairs, sizeof(ushort2) * s.chunks, cudaMemcpyHostToDevice, stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-      delete[] pairs;
-      TL_CUDA(ctx, e);
-    }
-    // (TreeRNN: four CTAs at least from H = 64 on: 25 trees, H = 128, forward / backward on clusters of 1, 2, 4, 8 CTAs:
-    // 58.6 / 142, 60.6 / 133, 56.0 / 124, 67.2 / 122 us)
-    for (int cs = cell == kRnn && H >= 64 ? 4 : 1; cs <= 16 && !t.ok; cs *= 2) t.ok = shape_fits(cell, H, cs, s);
-    if (!t.ok) return TREELSTM_OK;
-    for (int back = 0; back < 2; ++back) {
-      TreesKernel k = back ? backward_kernel(cell, s) : forward_kernel(cell);
-      TL_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
-      if (s.cs > 8) TL_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute at;
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = s.cs; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-      cfg.gridDim = dim3(s.cs); cfg.blockDim = dim3(back ? s.bthreads : kFwdT); cfg.dynamicSmemBytes = kSmemMax;
-      cfg.attrs = &at; cfg.numAttrs = 1;
-      int clusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) != cudaSuccess || clusters < 1) {
-        cudaGetLastError();
-        t.ok = false;
-        return TREELSTM_OK;
-      }
-      (back ? t.clusters_bwd : t.clusters) = clusters;
-    }
-    const size_t cta = sizeof(float) * (size_t)s.cs;
-    TL_CUDA(ctx, cudaMalloc((void**)&t.Wf, cta * kFwdT * fwd_words(cell)));
-    TL_CUDA(ctx, cudaMalloc((void**)&t.Wb, cta * s.bthreads * bwd_words(cell, s)));
+  const int H = ctx->H, cell = ctx->cell;
+  if (H > (cell == kRntn ? kRntnMaxH : 256)) return 0;
+  if (cell == kRntn)
+    for (int a = 0, Hp = round_up(H, 4); a <= 2 * Hp; ++a) s.chunks += pair_chunks(a, H, Hp);
+  // (TreeRNN: four CTAs at least from H = 64 on: 25 trees, H = 128, forward / backward on clusters of 1, 2, 4, 8 CTAs:
+  // 58.6 / 142, 60.6 / 133, 56.0 / 124, 67.2 / 122 us)
+  for (int cs = cell == kRnn && H >= 64 ? 4 : 1; cs <= 16 && !t.ok; cs *= 2) t.ok = shape_fits(cell, H, cs, s);
+  for (int back = 0; back < 2 && t.ok; ++back) {
+    TreesKernel k = back ? backward_kernel(cell, s) : forward_kernel(cell);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = s.cs; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(s.cs); cfg.blockDim = dim3(back ? s.bthreads : kFwdT); cfg.dynamicSmemBytes = kSmemMax;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    int clusters = 0;
+    t.ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) == cudaSuccess &&
+           (s.cs <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+           cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) == cudaSuccess && clusters >= 1;
+    (back ? t.clusters_bwd : t.clusters) = clusters;
   }
+  if (!t.ok) { cudaGetLastError(); return 0; }
+  return images_bytes(ctx, 0) + images_bytes(ctx, 1) + images_bytes(ctx, 2);
+}
+
+int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream) {
+  auto& t = ctx->trees;
   if (!t.ok) return TREELSTM_OK;
+  t.Wf = reinterpret_cast<float*>(memory);
+  t.Wb = reinterpret_cast<float*>(memory + images_bytes(ctx, 0));
+  t.pairs = reinterpret_cast<ushort2*>(memory + images_bytes(ctx, 0) + images_bytes(ctx, 1));
+  if (ctx->cell == kRntn) k_trees_pairs<<<1, 1, 0, stream>>>(ctx->H, t.pairs);
+  TL_CUDA(ctx, cudaGetLastError());
+  return TREELSTM_OK;
+}
+
+int pack_trees(treelstm* ctx, cudaStream_t stream) {
+  const auto& t = ctx->trees;
+  const auto& s = t.s;
+  if (!t.ok) return TREELSTM_OK;
+  const int H = ctx->H, E = ctx->E, cell = ctx->cell;
   const float* src = cell == kLstm ? ctx->W : ctx->Wcat;
   k_trees_pack<<<592, 256, 0, stream>>>(0, cell, H, E, fwd_words(cell), kFwdT, s, t.pairs, src, t.Wf);
   k_trees_pack<<<592, 256, 0, stream>>>(1, cell, H, E, bwd_words(cell, s), s.bthreads, s, t.pairs, src, t.Wb);
