@@ -479,9 +479,8 @@ int launch_forward_fp32(treelstm* ctx, int n, const int32_t* left, const int32_t
                         int n_levels_host, int flags, void* ws, const WsLayout& lay,
                         cudaStream_t stream) {
   if ((flags & TREELSTM_PERSISTENT) && trees_take(ctx, n)) {
-    const int single_max = ctx->opt.sched_single_cta_max < kSchedSingleMaxNodes ? ctx->opt.sched_single_cta_max : kSchedSingleMaxNodes;
     return launch_forward_trees(ctx, n, left, right, token, h, c, (flags & TREELSTM_SAVE_FOR_BACKWARD) != 0, ws, lay,
-                                ctx->opt.overlap_launch && n <= single_max, stream);
+                                ctx->opt.overlap_launch && scheduler_lets_start(ctx, n), stream);
   }
   char* base = static_cast<char*>(ws);
   FwdParams p;
@@ -527,8 +526,7 @@ int launch_forward_fp32(treelstm* ctx, int n, const int32_t* left, const int32_t
                                                                kThreads, smem));
     // Started under the single-CTA scheduler (see launch_forward_bf16 for the two ways to launch a
     // kernel with a grid barrier): the scheduler keeps its SM.
-    const int single_max = ctx->opt.sched_single_cta_max < kSchedSingleMaxNodes ? ctx->opt.sched_single_cta_max : kSchedSingleMaxNodes;
-    const bool overlap = ctx->opt.overlap_launch && n <= single_max && per_sm >= 1 && ctx->sm_count > 1;
+    const bool overlap = ctx->opt.overlap_launch && scheduler_lets_start(ctx, n) && per_sm >= 1 && ctx->sm_count > 1;
     p.early_start = overlap ? 1 : 0;
     int grid = per_sm * (overlap ? ctx->sm_count - 1 : ctx->sm_count);
     const int want = ((n + TMS - 1) / TMS + 1) * tiles_u;   // never more CTAs than the widest level has tiles

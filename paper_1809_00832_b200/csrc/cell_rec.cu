@@ -177,8 +177,7 @@ int launch_forward_rec(treelstm* ctx, int n, const int32_t* left, const int32_t*
                        const int32_t* level_offset_host, int n_levels_host, int flags, void* ws,
                        const WsLayout& lay, cudaStream_t stream) {
   if ((flags & TREELSTM_PERSISTENT) && trees_take(ctx, n)) {
-    const int single_max = ctx->opt.sched_single_cta_max < kSchedSingleMaxNodes ? ctx->opt.sched_single_cta_max : kSchedSingleMaxNodes;
-    return launch_forward_trees(ctx, n, left, right, token, h, nullptr, false, ws, lay, ctx->opt.overlap_launch && n <= single_max, stream);
+    return launch_forward_trees(ctx, n, left, right, token, h, nullptr, false, ws, lay, ctx->opt.overlap_launch && scheduler_lets_start(ctx, n), stream);
   }
   RecParams p;
   p.n = n; p.H = ctx->H; p.cell = ctx->cell; p.vocab = ctx->vocab;

@@ -60,6 +60,7 @@ struct Options {
 constexpr int kRadixBins = 256;
 constexpr int kRadixChunk = 1024;        // items per single-warp CTA of the multi-CTA sort
 constexpr int kSchedSingleMaxNodes = 32768;
+constexpr int kClusterMinNodes = 1024;      // smallest forest that one cluster schedules instead of one CTA
 constexpr int kSchedPartMaxNodes = 24576;   // largest forest the single-CTA scheduler can also deal out to sub-forests
 constexpr int kMaxParts = 32;               // upper bound on the number of sub-forests (co-resident clusters)
 
@@ -111,6 +112,7 @@ struct treelstm {
   int Hp = 0, Ep = 0;  // bf16 path: H padded to a multiple of 64, E padded to a multiple of 64
   int device = 0;
   int sm_count = 0;
+  int sched_cluster = 0;   // CTAs of the scheduling cluster (0: none fits the device)
 
   unsigned char* memory = nullptr;  // one allocation: everything the library owns on the device but the classifier
 
@@ -195,6 +197,8 @@ WsLayout ws_layout(const treelstm* ctx, int n, bool with_backward);
 // Per-device kernel attributes (the opt-in to more than 48 KB of dynamic shared memory belongs to the
 // device that is current when it is set): called by treelstm_create with the context's device current.
 int init_schedule_attributes(treelstm* ctx);   // schedule.cu
+bool schedules_on_cluster(const treelstm* ctx, int n);
+bool scheduler_lets_start(const treelstm* ctx, int n);
 int init_tc_attributes(treelstm* ctx);         // gemm_tc.cu
 
 // schedule.cu: enqueue the on-device ready-set construction.  Returns a treelstm_status.

@@ -941,16 +941,17 @@ int launch_forward_bf16(treelstm* ctx, int n, const int32_t* left, const int32_t
   p.tail_launched = with_tail ? 1 : 0;
   // Started under the single-CTA scheduler, the kernel takes the leaves first (the scratch of the
   // multi-CTA scheduler, unused then, holds its leaf order).
-  const int single_max = ctx->opt.sched_single_cta_max < kSchedSingleMaxNodes ? ctx->opt.sched_single_cta_max : kSchedSingleMaxNodes;
+  const bool on_cluster = schedules_on_cluster(ctx, n);
   int grid_persistent = ctx->sm_count;                 // one CTA per SM (shared and tensor memory)
   if (ctx->opt.max_ctas > 0 && grid_persistent > ctx->opt.max_ctas) grid_persistent = ctx->opt.max_ctas;
-  const bool overlap = (flags & TREELSTM_PERSISTENT) && ctx->opt.overlap_launch && n <= single_max &&
+  const bool overlap = (flags & TREELSTM_PERSISTENT) && ctx->opt.overlap_launch && scheduler_lets_start(ctx, n) &&
                        ctx->tc_resident_ctas >= ctx->sm_count && ctx->sm_count > 1 && ctx->sm_count <= kThreads;
-  if (overlap && grid_persistent > ctx->sm_count - 1) grid_persistent = ctx->sm_count - 1;   // the scheduler keeps its SM
-  p.leaves_first = overlap && n >= ctx->opt.leaves_first_min_nodes ? 1 : 0;
+  // (a single scheduling CTA keeps its SM; the CTAs of a scheduling cluster are gone before the first grid barrier counts)
+  if (overlap && !on_cluster && grid_persistent > ctx->sm_count - 1) grid_persistent = ctx->sm_count - 1;
+  p.leaves_first = overlap && !on_cluster && n >= ctx->opt.leaves_first_min_nodes ? 1 : 0;
   p.pre_counts = reinterpret_cast<int*>(base + lay.pre);
   p.pre_order = reinterpret_cast<int*>(base + lay.pending);
-  if (overlap) p.sched_ctas = ctx->sm_count - 1;   // the tile plans count on the CTAs that run
+  if (overlap && !on_cluster) p.sched_ctas = ctx->sm_count - 1;   // the tile plans count on the CTAs that run
   p.trace = nullptr;
 #ifdef TREELSTM_TRACE
   p.trace = reinterpret_cast<long long*>(base + lay.trace);
