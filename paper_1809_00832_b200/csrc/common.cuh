@@ -60,7 +60,7 @@ struct Options {
 constexpr int kRadixBins = 256;
 constexpr int kRadixChunk = 1024;        // items per single-warp CTA of the multi-CTA sort
 constexpr int kSchedSingleMaxNodes = 32768;
-constexpr int kClusterMinNodes = 1024;      // smallest forest that one cluster schedules instead of one CTA
+constexpr int kClusterMinNodes = 4096;      // smallest forest that one cluster schedules instead of one CTA
 constexpr int kSchedPartMaxNodes = 24576;   // largest forest the single-CTA scheduler can also deal out to sub-forests
 constexpr int kMaxParts = 32;               // upper bound on the number of sub-forests (co-resident clusters)
 

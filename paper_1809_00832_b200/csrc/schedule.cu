@@ -530,24 +530,35 @@ k_schedule_single(int n, const int* __restrict__ left, const int* __restrict__ r
 // ------------------------------------------------------------------------------------------ //
 // One cluster schedules the whole forest in its shared memory.
 //
-// The same algorithm as the single CTA's, with the nodes dealt out to the CTAs in contiguous id ranges and the
-// links, reports and climbs going through distributed shared memory (a parser numbers the nodes of a tree side
-// by side: most of them stay in the CTA).  What bounds the single CTA is its issue slots - every node takes part in
-// half a dozen passes - so sixteen of them take 14 k nodes from 31 us to the time of the longest climb.
+// The same algorithm as the single CTA's, with the nodes dealt out to the CTAs in contiguous id ranges (a power of two,
+// so that a node's CTA is a shift) and the links, reports and climbs going through distributed shared memory.  What
+// bounds the single CTA is its issue slots - every node takes part in half a dozen passes - and it takes 31 us for
+// 14 k nodes; here the longest climb counts: two round trips per level, 300 to 650 cycles depending on whether a
+// tree's nodes lie in one CTA's range.  Measured (trace build, cycles): 14.6 k nodes, 15 levels 25 k (single CTA 57 k);
+// 57 k nodes 30 k (before: ten launches, 145 us); of it linking 3 to 5 k, climbs 10 k, ordering 8 to 10 k.
 //
-// Order: LSD passes of kClBits bits.  Thread t of CTA c owns a contiguous run of positions of the pass's input;
-// tab[b][t] counts its items of bin b, a warp per bin turns the counts into prefixes over the threads, the CTAs
-// exchange their totals per bin, and every thread hands out places in its items' order.  The items are staged in
-// the order of the CTA's places, so that the stores to global memory run along whole lines.
-constexpr int kClBits = 6, kClBins = 1 << kClBits, kClMax = 16;
+// Order: LSD passes of kClBits bits.  A warp owns a contiguous run of positions of the pass's input and ranks its
+// items 32 at a time by matching bins; a warp per bin turns the warps' counts into prefixes, the CTAs exchange their
+// totals per bin.  The items are staged in the order of the CTA's places, so that the stores to global memory run
+// along whole lines.
+constexpr int kClBits = 6, kClBins = 1 << kClBits, kClMax = 16, kClGroups = 8;
+constexpr int kClMaxPer = 32 * 32 * kClGroups;           // nodes per CTA: a warp keeps its items' ranks in registers
 constexpr unsigned int kClDone = 0x80000000u, kClNone = 0xFFFFFFFFu;
-__host__ __device__ inline int cl_per(int n, int cs) { return (n + cs - 1) / cs; }
-// dependency word and caller per node, queue of climbs (later the staged order), counts, totals
-__host__ __device__ inline size_t cl_smem_bytes(int n, int cs) {
-  const size_t per = cl_per(n, cs);
-  return 4 * ((2 * per + per / 2 + 1 + 3) / 4 * 4) + 2 * (size_t)(kClBins + 1) * kSingleThreads + 4 * (size_t)(kClMax + 2) * (kClBins + 1) + 64;
+struct ClSmem {                                          // behind it: uint32 state[per], caller[per], uint16 staged[per]
+  int hist[kClBins + 1][33];                             // items of a bin per warp, then before the warp; last row: roots
+  int totals[kClMax][kClBins + 1];                       // items of a bin per CTA
+  int local[kClBins + 1];                                // first staged place of a bin
+  int place[kClBins + 1];                                // place in the output minus staged place
+  int scan[8];
+  int err, max_level, qhead, qtail;
+};
+inline int cl_shift(int n, int cs) {
+  int sh = 5;
+  while (((long long)cs << sh) < n) ++sh;
+  return sh;
 }
-__device__ __forceinline__ uint32_t cl_addr(uint32_t smem_addr, int rank) {
+inline size_t cl_smem_bytes(int sh) { return round_up_sz(sizeof(ClSmem), 16) + ((size_t)10 << sh); }
+__device__ __forceinline__ uint32_t cl_addr(uint32_t smem_addr, unsigned rank) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
   return a;
@@ -579,44 +590,34 @@ __device__ __forceinline__ void cl_sync() {
 __global__ void __launch_bounds__(kSingleThreads, 1)
 k_schedule_cluster(int n, const int* __restrict__ left, const int* __restrict__ right, const int* __restrict__ token,
                    int vocab, int* level, int* order, int* order_tmp, int* level_offset, int* roots, int* n_levels_out,
-                   DevStatus* st, int per) {
-  extern __shared__ __align__(16) unsigned int cl_smem[];
-  __shared__ int s_err, s_max, s_qhead, s_qtail, s_scan[32];
+                   DevStatus* st, int sh) {
+  extern __shared__ __align__(16) unsigned char cl_smem[];
+  ClSmem& sm = *reinterpret_cast<ClSmem*>(cl_smem);
   uint32_t cs, rank;
   asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(cs));
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned int* const w = cl_smem;                       // [per] dependency words
-  unsigned int* const par = w + per;                     // [per] caller of every node
-  unsigned short* const queue = reinterpret_cast<unsigned short*>(par + per);   // [per] leaves whose callers start a climb
-  unsigned short* const tab = reinterpret_cast<unsigned short*>(w + (2 * per + per / 2 + 1 + 3) / 4 * 4);   // [bins + 1][threads]
-  int* const totals = reinterpret_cast<int*>(tab + (kClBins + 1) * kSingleThreads);   // [CTA][bins + 1], exchanged
-  int* const local = totals + kClMax * (kClBins + 1);    // first staged place of a bin
-  int* const place = local + kClBins + 1;                // first place of a bin's items of this CTA in the output
-  const uint32_t w_addr = (uint32_t)__cvta_generic_to_shared(w), par_addr = (uint32_t)__cvta_generic_to_shared(par);
-  const uint32_t err_addr = (uint32_t)__cvta_generic_to_shared(&s_err), max_addr = (uint32_t)__cvta_generic_to_shared(&s_max);
-  const int base = (int)rank * per, mine = max(0, min(per, n - base));
+  const int per = 1 << sh, base = (int)rank << sh, mine = max(0, min(per, n - base));
+  unsigned int* const state = reinterpret_cast<unsigned int*>(cl_smem + (sizeof(ClSmem) + 15) / 16 * 16);
+  unsigned int* const caller = state + per;
+  unsigned short* const queue = reinterpret_cast<unsigned short*>(caller + per);   // leaves whose callers start a climb; later staged items
+  const uint32_t state_addr = (uint32_t)__cvta_generic_to_shared(state), to_caller = 4u << sh;   // distance of the two words of a node
+  const uint32_t err_addr = cl_addr((uint32_t)__cvta_generic_to_shared(&sm.err), 0), max_addr = cl_addr((uint32_t)__cvta_generic_to_shared(&sm.max_level), 0);
+#ifdef TREELSTM_TRACE
+  const long long t_start = clock64();
+#define TL_CL_STAMP(i) do { if (tid == 0 && rank == 0) st->pad[i] = (int)(clock64() - t_start); } while (0)
+#else
+#define TL_CL_STAMP(i) do { } while (0)
+#endif
   if (rank == 0 && tid < (int)(sizeof(DevStatus) / sizeof(int))) reinterpret_cast<int*>(st)[tid] = 0;
-  if (tid == 0) { s_err = 0; s_max = 0; s_qhead = 0; s_qtail = 0; }
-  for (int k = tid; k < mine; k += kSingleThreads) { w[k] = 0u; par[k] = kClNone; }
+  if (tid == 0) { sm.err = 0; sm.max_level = 0; sm.qhead = 0; sm.qtail = 0; }
+  for (int k = tid; k < mine; k += kSingleThreads) { state[k] = 0u; caller[k] = kClNone; }
   if (rank == 0) __threadfence();
   cl_sync();
+  TL_CL_STAMP(0);   // cleared
   // a kernel launched behind this one as its programmatic dependent may start now (see k_schedule_single)
   if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // where a node lives: CTA node / per (the quotient by multiplication: the ids are below 2^22)
-  const float inv_per = 1.0f / (float)per;
-  auto home = [&](int k, int& at) {
-    int c = (int)((float)k * inv_per);
-    at = k - c * per;
-    if (at < 0) { --c; at += per; }
-    if (at >= per) { ++c; at -= per; }
-    return c;
-  };
-  auto word_of = [&](uint32_t local_addr, int k) {
-    int at;
-    const int c = home(k, at);
-    return cl_addr(local_addr + 4u * (uint32_t)at, c);
-  };
+  auto node_at = [&](unsigned k) { return cl_addr(state_addr + 4u * (k & (unsigned)(per - 1)), k >> sh); };
   // validate; a child's word gets its caller (a second caller finds the first one there)
   for (int k0 = tid; k0 < mine; k0 += 4 * kSingleThreads) {
     int l[4], r[4], t[4];
@@ -635,64 +636,70 @@ k_schedule_cluster(int n, const int* __restrict__ left, const int* __restrict__ 
       if (l[j] < 0 && r[j] < 0) {
         if (l[j] != -1 || r[j] != -1) err = TREELSTM_ERR_INVALID_FOREST;
         else if (t[j] < 0 || t[j] >= vocab) err = TREELSTM_ERR_TOKEN_OUT_OF_RANGE;
-        else w[k] = kClDone;
+        else state[k] = kClDone;
       } else if (l[j] < 0 || r[j] < 0 || l[j] >= n || r[j] >= n || l[j] == r[j] || l[j] == id || r[j] == id) {
         err = TREELSTM_ERR_INVALID_FOREST;
       } else {
-        const unsigned int a = cl_exch(word_of(par_addr, l[j]), (unsigned int)id), b = cl_exch(word_of(par_addr, r[j]), (unsigned int)id);
+        const unsigned int a = cl_exch(node_at((unsigned)l[j]) + to_caller, (unsigned int)id), b = cl_exch(node_at((unsigned)r[j]) + to_caller, (unsigned int)id);
         if (a != kClNone || b != kClNone) err = TREELSTM_ERR_INVALID_FOREST;
       }
-      if (err) cl_min(cl_addr(err_addr, 0), err);
+      if (err) cl_min(err_addr, err);
     }
   }
   cl_sync();
-  if ((int)cl_ld(cl_addr(err_addr, 0)) == 0) {
+  TL_CL_STAMP(1);   // validated and linked
+  if ((int)cl_ld(err_addr) == 0) {
     // every leaf reports to its caller; a caller whose second child reports here starts a climb
     for (int k = tid; k < mine; k += kSingleThreads) {
-      if (w[k] != kClDone) continue;
-      const unsigned int p = par[k];
-      if (p == kClNone) continue;
-      const uint32_t a = word_of(w_addr, (int)p);
+      const unsigned int p = caller[k];
+      if (state[k] != kClDone || p == kClNone) continue;
+      const uint32_t a = node_at(p);
       const unsigned int old = cl_exch(a, 1u);           // 1 + the level of the other child, if that was there first
       if (old != 0u) {
         cl_st(a, kClDone | old);
-        queue[atomicAdd(&s_qtail, 1)] = (unsigned short)k;
+        queue[atomicAdd(&sm.qtail, 1)] = (unsigned short)k;
       }
     }
     __syncthreads();
+    TL_CL_STAMP(2);   // leaves reported
     for (;;) {
-      const int q = atomicAdd(&s_qhead, 1);
-      if (q >= s_qtail) break;
-      int cur = (int)par[queue[q]], lvl = (int)(cl_ld(word_of(w_addr, cur)) & ~kClDone);
-      for (int step = 0; step < n; ++step) {             // a path to the root has fewer than n edges
-        const unsigned int p = cl_ld(word_of(par_addr, cur));
-        if (p == kClNone) break;
-        const uint32_t a = word_of(w_addr, (int)p);
-        const unsigned int old = cl_exch(a, (unsigned int)lvl + 1u);
+      const int q = atomicAdd(&sm.qhead, 1);
+      if (q >= sm.qtail) break;
+      const uint32_t first = node_at(caller[queue[q]]);
+      unsigned int lvl = cl_ld(first) & ~kClDone, p = cl_ld(first + to_caller);
+      for (int step = 0; p != kClNone && step < n; ++step) {   // a path to the root has fewer than n edges
+        const uint32_t a = node_at(p);
+        const unsigned int old = cl_exch(a, lvl + 1u);
         if (old == 0u) break;                            // sibling subtree still unresolved
-        lvl = 1 + max(lvl, (int)old - 1);
-        cl_st(a, kClDone | (unsigned int)lvl);
-        cur = (int)p;
+        lvl = 1u + max(lvl, old - 1u);
+        cl_st(a, kClDone | lvl);
+        p = cl_ld(a + to_caller);
       }
     }
   }
+  TL_CL_STAMP(3);
   cl_sync();
+  TL_CL_STAMP(4);   // climbed
+  // A warp's contiguous run of positions, 32 at a time: its items (positions within the CTA) and their levels.
+  const int wper = (((mine + 31) / 32) + 31) & ~31;
+  const int w_begin = min(mine, warp * wper), w_end = min(mine, w_begin + wper);
   {
     int top = 0, bad = 0;
-    for (int k = tid; k < mine; k += kSingleThreads) {
-      const unsigned int v = w[k];
+    for (int k = w_begin + lane; k < w_end; k += 32) {
+      const unsigned int v = state[k];
       bad |= !(v & kClDone);                             // on a cycle: never ready
       const int lvl = (int)(v & ~kClDone);
       level[base + k] = lvl;
       top = max(top, lvl);
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) top = max(top, __shfl_xor_sync(kFull, top, d));
-    if (lane == 0) cl_max(cl_addr(max_addr, 0), top);
-    if (bad) cl_min(cl_addr(err_addr, 0), (int)TREELSTM_ERR_INVALID_FOREST);
+    top = __reduce_max_sync(kFull, top);
+    if (lane == 0) cl_max(max_addr, top);
+    if (bad) cl_min(err_addr, (int)TREELSTM_ERR_INVALID_FOREST);
   }
+  for (int i = tid; i < (kClBins + 1) * 33; i += kSingleThreads) (&sm.hist[0][0])[i] = 0;
   cl_sync();
-  const int err = (int)cl_ld(cl_addr(err_addr, 0)), n_levels = (int)cl_ld(cl_addr(max_addr, 0)) + 1;
+  const int err = (int)cl_ld(err_addr), n_levels = (int)cl_ld(max_addr) + 1;
+  TL_CL_STAMP(5);   // levels written
   if (err != 0) {
     if (rank == 0 && tid == 0) { report(st, err); *n_levels_out = 0; }
     cl_sync();                                           // rank 0's words are read until here
@@ -700,109 +707,103 @@ k_schedule_cluster(int n, const int* __restrict__ left, const int* __restrict__ 
   }
   int passes = 1;
   while ((n_levels - 1) >> (kClBits * passes)) ++passes;
-  const int npt = ((per + kSingleThreads - 1) / kSingleThreads) | 1;   // odd: the threads' runs start in different banks
-  const int k0 = min(mine, tid * npt), k1 = min(mine, k0 + npt);
-  unsigned short* const staged16 = queue;
   for (int pass = 0; pass < passes; ++pass) {
     int* const dst = ((passes - 1 - pass) & 1) ? order_tmp : order;
     const int* const src = pass == 0 ? nullptr : (dst == order ? order_tmp : order);
     const int shift = kClBits * pass, bins = min(kClBins, ((n_levels - 1) >> shift) + 1);
-    const bool with_roots = pass == 0;                   // one more bin: nodes without a caller, counted beside their own bin
-    if (pass > 0)                                        // this CTA's items of the last pass's output and their levels
+    if (pass > 0) {                                      // this CTA's items of the last pass's output and their levels
       for (int k = tid; k < mine; k += kSingleThreads) {
         const int item = *(volatile const int*)(src + base + k);
-        par[k] = (unsigned int)item;
-        w[k] = (unsigned int)*(volatile const int*)(level + item);
+        state[k] = (unsigned int)*(volatile const int*)(level + item);
+        caller[k] = (unsigned int)item;
       }
-    {
-      uint4* z = reinterpret_cast<uint4*>(tab);
-      for (int i = tid; i < (bins + 1) * kSingleThreads * 2 / 16; i += kSingleThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
+      for (int i = tid; i < (kClBins + 1) * 33; i += kSingleThreads) (&sm.hist[0][0])[i] = 0;
+      __syncthreads();
     }
-    __syncthreads();
-    int my_roots = 0;
-    for (int k = k0; k < k1; ++k) {
-      const int b = (int)((w[k] & ~kClDone) >> shift) & (kClBins - 1);
-      tab[b * kSingleThreads + tid] += 1;
-      my_roots += with_roots && par[k] == kClNone;
-    }
-    tab[bins * kSingleThreads + tid] = (unsigned short)my_roots;
-    __syncthreads();
-    for (int b = warp; b <= bins; b += 32) {             // row b -> exclusive prefix over the threads; its total to every CTA
-      unsigned short* row = tab + b * kSingleThreads + lane * 32;
-      int sum = 0;
-      for (int q = 0; q < 32; q += 8) {
-        uint4 x = *reinterpret_cast<uint4*>(row + q);
-        unsigned int* x4 = reinterpret_cast<unsigned int*>(&x);
+    // rank of every item among the warp's items of its bin (and of every root among the warp's roots)
+    unsigned int ranks[kClGroups];                       // rank | bin << 16 | root rank << 22, per group of 32
+    int warp_roots = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int lo = (int)(x4[j] & 0xFFFFu), hi = (int)(x4[j] >> 16);
-          x4[j] = (unsigned int)sum | ((unsigned int)(sum + lo) << 16);
-          sum += lo + hi;
-        }
-        *reinterpret_cast<uint4*>(row + q) = x;
-      }
-      int incl = sum;
+    for (int g = 0; g < kClGroups; ++g) {
+      const int k = w_begin + 32 * g + lane;
+      ranks[g] = 0u;
+      if (w_begin + 32 * g >= w_end) continue;           // the same for the whole warp
+      const bool valid = k < w_end;
+      const int bin = valid ? (int)((state[k] & ~kClDone) >> shift) & (kClBins - 1) : kClBins;
+      const bool root = pass == 0 && valid && caller[k] == kClNone;
+      const unsigned peers = __match_any_sync(kFull, bin), rmask = __ballot_sync(kFull, root);
+      const int before = valid ? sm.hist[bin][warp] : 0;
+      __syncwarp();
+      if (valid && lane == __ffs(peers) - 1) sm.hist[bin][warp] = before + __popc(peers);
+      ranks[g] = (unsigned)(before + __popc(peers & lanemask_lt())) | ((unsigned)bin << 16) |
+                 ((unsigned)(warp_roots + __popc(rmask & lanemask_lt())) << 23);
+      warp_roots += __popc(rmask);
+      __syncwarp();
+    }
+    if (lane == 0) sm.hist[kClBins][warp] = warp_roots;
+    __syncthreads();
+    for (int b = warp; b <= kClBins; b += 32) {          // counts of the warps -> prefixes; the bin's total to every CTA
+      if (b >= bins && b != kClBins) continue;
+      const int v = sm.hist[b][lane];
+      int incl = v;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
         const int t = __shfl_up_sync(kFull, incl, d);
         if (lane >= d) incl += t;
       }
-      const unsigned int before = (unsigned int)(incl - sum), both = before | (before << 16);
-      for (int q = 0; q < 32; q += 8) {
-        uint4 x = *reinterpret_cast<uint4*>(row + q);
-        x.x += both; x.y += both; x.z += both; x.w += both;
-        *reinterpret_cast<uint4*>(row + q) = x;
-      }
+      sm.hist[b][lane] = incl - v;
       const int total = __shfl_sync(kFull, incl, 31);
-      if (lane < (int)cs)
-        cl_st(cl_addr((uint32_t)__cvta_generic_to_shared(totals + (int)rank * (kClBins + 1) + b), lane), (unsigned int)total);
+      if (lane < (int)cs) cl_st(cl_addr((uint32_t)__cvta_generic_to_shared(&sm.totals[rank][b]), lane), (unsigned int)total);
     }
+    TL_CL_STAMP(6);   // counted
     cl_sync();
+    TL_CL_STAMP(7);
     // places: bins before it in the whole forest, then CTAs before this one
-    if (tid < 128) {
-      int all = 0, before = 0, own = 0;
-      if (tid <= bins)
-        for (int c = 0; c < (int)cs; ++c) {
-          const int v = totals[c * (kClBins + 1) + tid];
-          all += v;
-          before += c < (int)rank ? v : 0;
-          own = c == (int)rank ? v : own;
-        }
-      const bool bin = tid < bins;
-      int ga = bin ? all : 0, la = bin ? own : 0;
+    if (warp < 2) {
+      const int b = tid;
+      int all = 0, before = 0;
+#pragma unroll
+      for (int c = 0; c < kClMax; ++c) {
+        const int v = c < (int)cs && b < bins ? sm.totals[c][b] : 0;
+        all += v;
+        before += c < (int)rank ? v : 0;
+      }
+      const int own = b < bins ? sm.totals[rank][b] : 0;
+      int ga = all, la = own;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
-        const int a = __shfl_up_sync(kFull, ga, d), b = __shfl_up_sync(kFull, la, d);
-        if (lane >= d) { ga += a; la += b; }
+        const int x = __shfl_up_sync(kFull, ga, d), y = __shfl_up_sync(kFull, la, d);
+        if (lane >= d) { ga += x; la += y; }
       }
-      if (lane == 31) { s_scan[warp] = ga; s_scan[8 + warp] = la; }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      int g0 = 0, l0 = 0;
-      for (int q = 0; q < warp; ++q) { g0 += s_scan[q]; l0 += s_scan[8 + q]; }
-      if (bin) {
-        const int first = g0 + ga - all;
-        place[tid] = first + before;
-        local[tid] = l0 + la - own;
-        if (rank == 0 && passes == 1) level_offset[tid] = first;
-      } else if (tid == bins) {
-        place[bins] = before;                            // roots
-        if (rank == 0 && with_roots) st->n_roots = all;
+      if (tid == 31) { sm.scan[0] = ga; sm.scan[1] = la; }
+      asm volatile("bar.sync 1, 64;" ::: "memory");
+      const int first = ga - all + (warp ? sm.scan[0] : 0), local = la - own + (warp ? sm.scan[1] : 0);
+      sm.local[b] = local;
+      sm.place[b] = first + before - local;
+      if (rank == 0 && passes == 1 && b < bins) level_offset[b] = first;
+    } else if (warp == 2 && pass == 0) {
+      const int v = lane < (int)cs ? sm.totals[lane][kClBins] : 0;
+      const int before = __reduce_add_sync(kFull, lane < (int)rank ? v : 0), all = __reduce_add_sync(kFull, v);
+      if (lane == 0) {
+        sm.place[kClBins] = before;
+        if (rank == 0) st->n_roots = all;
       }
     }
     __syncthreads();
-    int root_at = place[bins] + tab[bins * kSingleThreads + tid];
-    for (int k = k0; k < k1; ++k) {
-      const int b = (int)((w[k] & ~kClDone) >> shift) & (kClBins - 1);
-      unsigned short* cell = tab + b * kSingleThreads + tid;
-      staged16[local[b] + *cell] = (unsigned short)k;
-      *cell += 1;
-      if (with_roots && par[k] == kClNone) roots[root_at++] = base + k;
+    const int root_at = sm.place[kClBins] + sm.hist[kClBins][warp];
+#pragma unroll
+    for (int g = 0; g < kClGroups; ++g) {
+      const int k = w_begin + 32 * g + lane;
+      if (k >= w_end) break;
+      const int bin = (int)(ranks[g] >> 16) & (kClBins - 1);
+      queue[sm.local[bin] + sm.hist[bin][warp] + (int)(ranks[g] & 0xFFFFu)] = (unsigned short)k;
+      if (pass == 0 && caller[k] == kClNone) roots[root_at + (int)(ranks[g] >> 23)] = base + k;
     }
     __syncthreads();
-    // a staged place q of bin b goes to place[b] + q - local[b]
+    TL_CL_STAMP(8);   // staged
     for (int q = tid; q < mine; q += kSingleThreads) {
-      const int k = staged16[q], b = (int)((w[k] & ~kClDone) >> shift) & (kClBins - 1);
-      dst[place[b] + q - local[b]] = pass == 0 ? base + k : (int)par[k];
+      const int k = queue[q];
+      dst[sm.place[(int)((state[k] & ~kClDone) >> shift) & (kClBins - 1)] + q] = pass == 0 ? base + k : (int)caller[k];
     }
     if (pass + 1 < passes) {
       __threadfence();
@@ -818,6 +819,7 @@ k_schedule_cluster(int n, const int* __restrict__ left, const int* __restrict__ 
     }
   }
   if (rank == 0 && tid == 0) { level_offset[n_levels] = n; st->n_levels = n_levels; *n_levels_out = n_levels; }
+  TL_CL_STAMP(9);
   cl_sync();                                             // no CTA leaves while a peer may still read its words
 }
 
@@ -1028,7 +1030,7 @@ int init_schedule_attributes(treelstm* ctx) {
   TL_CUDA(ctx, cudaFuncSetAttribute(k_schedule_single, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)single_smem_bytes(kSchedSingleMaxNodes, false)));
   // sixteen CTAs where the device has room for such a cluster, else the portable eight
-  constexpr int kMost = 224 * 1024;
+  const int kMost = (int)cl_smem_bytes(13);              // 8192 nodes per CTA
   TL_CUDA(ctx, cudaFuncSetAttribute(k_schedule_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost));
   TL_CUDA(ctx, cudaFuncSetAttribute(k_schedule_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   for (int cs = 16; cs >= 8 && ctx->sched_cluster == 0; cs /= 2) {
@@ -1051,12 +1053,12 @@ bool scheduler_lets_start(const treelstm* ctx, int n) {
 }
 
 // Forests scheduled by one cluster: from kClusterMinNodes nodes on (below that a single CTA is done before the CTAs of
-// a cluster have met a few times), as long as a CTA's share fits its shared memory and 16-bit places.  A lowered
+// a cluster have met a few times), as long as a warp can keep its share in registers.  A lowered
 // TREELSTM_OPT_SCHED_SINGLE_CTA_MAX asks for the multi-CTA path.
 bool schedules_on_cluster(const treelstm* ctx, int n) {
   const int cs = ctx->sched_cluster;
-  return cs > 0 && n >= kClusterMinNodes && ctx->opt.sched_single_cta_max >= kSchedSingleMaxNodes && n < (1 << 22) &&
-         cl_per(n, cs) < 65536 && cl_smem_bytes(n, cs) <= 224 * 1024;
+  return cs > 0 && n >= kClusterMinNodes && ctx->opt.sched_single_cta_max >= kSchedSingleMaxNodes &&
+         n <= (long long)cs * kClMaxPer;
 }
 
 int launch_schedule(treelstm* ctx, int n, const int32_t* left, const int32_t* right,
@@ -1078,10 +1080,10 @@ int launch_schedule(treelstm* ctx, int n, const int32_t* left, const int32_t* ri
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = cs; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-    cfg.gridDim = dim3(cs); cfg.blockDim = dim3(kSingleThreads); cfg.dynamicSmemBytes = cl_smem_bytes(n, cs); cfg.stream = stream;
+    cfg.gridDim = dim3(cs); cfg.blockDim = dim3(kSingleThreads); cfg.dynamicSmemBytes = cl_smem_bytes(cl_shift(n, cs)); cfg.stream = stream;
     cfg.attrs = &at; cfg.numAttrs = 1;
     TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_schedule_cluster, n, left, right, token, ctx->vocab, level, order, order_tmp,
-                                    level_offset, roots, n_levels_out, st, cl_per(n, cs)));
+                                    level_offset, roots, n_levels_out, st, cl_shift(n, cs)));
     ctx->launches += 1;
     return TREELSTM_OK;
   }

@@ -216,3 +216,63 @@ def test_fp32_persistent_odd_and_large_hidden_sizes(H, E):
         res = util.gpu_forward(model, forest, flags)
         assert util.max_abs(res["h"], h) < util.TOL["fp32"]
         assert util.max_abs(res["c"], c) < util.TOL["fp32"]
+
+
+@pytest.mark.parametrize("kind", ["threshold", "permuted", "64 levels", "65 levels", "4200 levels", "single leaves", "largest", "beyond"])
+def test_schedule_of_one_cluster(kind):
+    """forests that one cluster schedules: the smallest, shuffled ids (every link crosses CTAs), one to three sorting
+    passes, ids that fill the last CTA's range partly, the largest forest and the first one beyond it; roots in order"""
+    rng = np.random.default_rng(21)
+    params = fg.draw_params(rng, 2, 2, 50, emb_dist="uniform", emb_scale=0.1, w_scale=0.1)
+    cap = 16 * 8192
+    if kind in ("largest", "beyond"):          # chains of 3 nodes, built directly: left leaf, right leaf, their caller
+        n = cap - cap % 3 + (3 if kind == "beyond" else 0)
+        k = np.arange(n, dtype=np.int32)
+        inner = k % 3 == 2
+        forest = fg.Forest(np.where(inner, k - 2, -1).astype(np.int32), np.where(inner, k - 1, -1).astype(np.int32),
+                           np.where(inner, -1, k % 50).astype(np.int32), k[inner], k // 3)
+    elif kind == "single leaves":
+        forest = fg.forest_from_shapes([None] * 4097, rng, 50)
+    elif kind.endswith("levels"):
+        depth = int(kind.split()[0])
+        forest = fg.concat_forests([fg.random_forest(rng, 70, 40, 60, 50), fg.forest_from_shapes([fg.left_chain_shape(depth)], rng, 50)])
+    else:
+        forest = fg.random_forest(rng, 75, 20, 36, 50)
+        forest = fg.concat_forests([forest, fg.forest_from_shapes([None] * (4096 - forest.n_nodes), rng, 50)]) if forest.n_nodes < 4096 else forest
+        if kind == "permuted":
+            forest, _ = fg.permute_node_ids(forest, rng)
+    status, _, level, order, off = orc.schedule(forest.left, forest.right)
+    model = util.make_model(params, "fp32")
+    res = util.gpu_forward(model, forest, binding.PERSISTENT)
+    util.check_schedule(res, dict(level=level, order=order, level_offset=off), forest.n_nodes)
+    roots = model.roots(forest.n_trees)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(roots["root_ids"].cpu().numpy(), np.sort(forest.roots))
+
+
+def test_malformed_forests_on_the_scheduling_cluster():
+    """two callers for one node, a cycle, a child out of range, a bad token: the same codes as on any other path"""
+    rng = np.random.default_rng(22)
+    params = fg.draw_params(rng, 4, 4, 50, emb_dist="uniform", emb_scale=0.1, w_scale=0.1)
+    base = fg.random_forest(rng, 120, 30, 50, 50)
+    inner = np.flatnonzero(base.left >= 0)
+    model = util.make_model(params, "fp32")
+
+    def code(change):
+        arrays = [base.left.copy(), base.right.copy(), base.token.copy()]
+        change(*arrays)
+        with pytest.raises(binding.TreeLSTMError) as err:
+            model.forward(*[util.to_dev(a) for a in arrays], flags=binding.PERSISTENT)
+        return err.value.code
+
+    def twice(l, r, t): l[inner[7]] = l[inner[900]]
+    def cycle(l, r, t):                        # top -> p -> q becomes top -> q's old child, and p and q point at each other
+        top = next(k for k in inner[::-1] if l[k] >= 0 and l[l[k]] >= 0 and l[l[l[k]]] >= 0)
+        p, q = l[top], l[l[top]]
+        l[top], l[q] = l[q], p
+    def out_of_range(l, r, t): r[inner[3]] = base.n_nodes
+    def token(l, r, t): t[np.flatnonzero(base.left < 0)[-1]] = 50
+    assert code(twice) == code(out_of_range) == binding.ERR_INVALID_FOREST
+    assert code(cycle) == binding.ERR_INVALID_FOREST
+    assert code(token) == binding.ERR_TOKEN_OUT_OF_RANGE
+    util.gpu_forward(model, base, binding.PERSISTENT)
