@@ -108,7 +108,7 @@ def load_library(variant: Optional[str] = None) -> ctypes.CDLL:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
@@ -117,8 +117,8 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
     return t
 
 
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())   # (no Stream object is made for it)
 
 
 STATIC_MAX_NODES = 16384
@@ -181,7 +181,9 @@ class TreeLSTM:
             raise TreeLSTMError(rc, "treelstm_create")
         self.handle = handle
         self._ws: Optional[torch.Tensor] = None
+        self._ws_nodes, self._ws_backward = -1, False   # what the workspace was last found large enough for
         self._host_staging: Optional[torch.Tensor] = None
+        self._host_nodes = -1
         self._keep = None
 
     @classmethod
@@ -205,7 +207,9 @@ class TreeLSTM:
             raise TreeLSTMError(rc, "treelstm_create_recursive")
         self.handle = handle
         self._ws = None
+        self._ws_nodes, self._ws_backward = -1, False
         self._host_staging = None
+        self._host_nodes = -1
         self._keep = None
         return self
 
@@ -244,9 +248,11 @@ class TreeLSTM:
         return int(self.lib.treelstm_workspace_bytes(self.handle, max_nodes, int(with_backward)))
 
     def _workspace(self, n: int, with_backward: bool) -> torch.Tensor:
-        need = self.workspace_bytes(n, with_backward)
-        if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+        if self._ws is None or n > self._ws_nodes or (with_backward and not self._ws_backward):
+            need = self.workspace_bytes(n, with_backward)
+            if self._ws is None or self._ws.numel() < need + 256:
+                self._ws = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+            self._ws_nodes, self._ws_backward = n, with_backward
         return self._ws
 
     # -- forward ------------------------------------------------------------------------------
@@ -273,7 +279,7 @@ class TreeLSTM:
         rc = self.lib.treelstm_forward(self.handle, n, _ptr(left), _ptr(right), _ptr(token), _ptr(out["h"]),
                                        _ptr(out.get("c")), _ptr(out["level"]), _ptr(out["order"]),
                                        _ptr(out["level_offset"]), _ptr(out["n_levels"]), flags,
-                                       ctypes.c_void_p(aligned), ws.numel() - (aligned - base), _stream())
+                                       aligned, ws.numel() - (aligned - base), _stream())
         if rc != OK:
             raise TreeLSTMError(rc, "treelstm_forward")
         self._keep = (left, right, token, out)
@@ -306,11 +312,11 @@ class TreeLSTM:
         H, E, C = self.H, self.E, self.C
         f32 = dict(dtype=torch.float32, device="cuda")
         out = dict(
-            loss=torch.zeros(1, **f32), dW=torch.empty((E + 2 * H, 5 * H), **f32), db=torch.empty(5 * H, **f32),
+            loss=torch.empty(1, **f32), dW=torch.empty((E + 2 * H, 5 * H), **f32), db=torch.empty(5 * H, **f32),
             dWc=torch.empty((H, C), **f32), dbc=torch.empty(C, **f32),
             touched_ids=torch.empty(max(n_leaves, 1), dtype=torch.int32, device="cuda"),
             dEmb_rows=torch.empty((max(n_leaves, 1), E), **f32),
-            n_touched=torch.zeros(1, dtype=torch.int32, device="cuda"),
+            n_touched=torch.empty(1, dtype=torch.int32, device="cuda"),
         )
         rc = self.lib.treelstm_backward(self.handle, _ptr(labels), _ptr(out["loss"]), _ptr(out["dW"]),
                                         _ptr(out["db"]), _ptr(out["dWc"]), _ptr(out["dbc"]),
@@ -329,11 +335,11 @@ class TreeLSTM:
         H, C = self.H, self.C
         f32 = dict(dtype=torch.float32, device="cuda")
         out = dict(
-            loss=torch.zeros(1, **f32), dW=torch.empty((2 * H, H), **f32), db=torch.empty(H, **f32),
+            loss=torch.empty(1, **f32), dW=torch.empty((2 * H, H), **f32), db=torch.empty(H, **f32),
             dWc=torch.empty((H, C), **f32), dbc=torch.empty(C, **f32),
             touched_ids=torch.empty(max(n_leaves, 1), dtype=torch.int32, device="cuda"),
             dEmb_rows=torch.empty((max(n_leaves, 1), H), **f32),
-            n_touched=torch.zeros(1, dtype=torch.int32, device="cuda"),
+            n_touched=torch.empty(1, dtype=torch.int32, device="cuda"),
         )
         if self.cell == CELL_RNTN:
             out["dV"] = torch.empty((H, 2 * H, 2 * H), **f32)
@@ -357,7 +363,7 @@ class TreeLSTM:
             if t.is_cuda or t.dtype != torch.int32 or not t.is_contiguous():
                 raise ValueError("forest arrays must be contiguous CPU int32 tensors")
         # device staging is torch's memory too: hand the library a buffer large enough for this forest
-        need = int(self.lib.treelstm_host_staging_bytes(self.handle, n))
+        need = 0 if n <= self._host_nodes else int(self.lib.treelstm_host_staging_bytes(self.handle, n))
         if self._host_staging is None or self._host_staging.numel() < need + 256:
             grown = torch.empty(need + need // 4 + 256, dtype=torch.uint8, device="cuda")
             base = grown.data_ptr()
@@ -367,6 +373,7 @@ class TreeLSTM:
             if rc != OK:
                 raise TreeLSTMError(rc, "treelstm_set_host_staging")
             self._host_staging = grown
+        self._host_nodes = max(n, self._host_nodes)
         if out is None:
             pin = dict(pin_memory=True)
             out = dict(n_levels=torch.zeros(1, dtype=torch.int32, **pin),

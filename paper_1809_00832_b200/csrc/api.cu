@@ -159,6 +159,24 @@ void learn_tail_hint(treelstm* ctx) {
   ctx->tail_skip = hs->tail_from >= hs->n_levels;
 }
 
+// Waits for the stream of the last call, whose control block is then in ctx->host_status, and says what it holds.
+int finish_status(treelstm* ctx) {
+  auto& L = ctx->last;
+  TL_CUDA(ctx, cudaStreamSynchronize(L.stream));
+  const int st = reinterpret_cast<const DevStatus*>(ctx->host_status)->status;
+  if (st != 0) L.valid = false;
+  else learn_tail_hint(ctx);
+  return st;
+}
+
+// Whether a kernel may write to host memory at `ptr` (pinned, at the same address on the device); NULL: nothing to write.
+bool gpu_writable(const void* ptr) {
+  if (!ptr) return true;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) { cudaGetLastError(); return false; }
+  return a.type == cudaMemoryTypeHost && a.devicePointer == ptr;
+}
+
 // used by backward.cu
 int ensure_host_levels(treelstm* ctx) {
   if (ctx->last.host_levels_valid) return TREELSTM_OK;
@@ -432,18 +450,14 @@ int treelstm_status_sync(treelstm_t* ctx) {
   char* base = static_cast<char*>(L.ws);
   TL_CUDA(ctx, cudaMemcpyAsync(ctx->host_status, base + L.lay.status, sizeof(DevStatus),
                                cudaMemcpyDeviceToHost, L.stream));
-  TL_CUDA(ctx, cudaStreamSynchronize(L.stream));
-  const int st = reinterpret_cast<const DevStatus*>(ctx->host_status)->status;
-  if (st != 0) L.valid = false;
-  else learn_tail_hint(ctx);
-  return st;
+  return finish_status(ctx);
 }
 
 int treelstm_roots(treelstm_t* ctx, int max_roots, int32_t* root_ids, float* root_h, float* root_c,
                    int32_t* n_roots, void* stream) {
   if (!ctx || max_roots < 0 || !n_roots) return TREELSTM_ERR_INVALID_ARG;
   if (!ctx->last.valid) return TREELSTM_ERR_STATE;
-  return launch_gather_roots(ctx, max_roots, root_ids, root_h, root_c, n_roots,
+  return launch_gather_roots(ctx, max_roots, root_ids, root_h, root_c, n_roots, nullptr,
                              static_cast<cudaStream_t>(stream));
 }
 
@@ -547,8 +561,12 @@ int treelstm_forward_host(treelstm_t* ctx, int n_nodes, const int32_t* left, con
   p.root_ids = reinterpret_cast<int32_t*>(p.roots_pack);
   p.root_h = reinterpret_cast<float*>(p.root_ids + max_r);
   p.root_c = p.root_h + (size_t)max_r * H;
+  // Roots whose destinations are pinned are written there by the gathering kernel itself, and so is the control
+  // block: two copies less behind it on the stream.
+  const bool direct = want_roots && max_r > 0 && gpu_writable(root_ids) && gpu_writable(root_h) && gpu_writable(root_c);
   if (want_roots) {
-    rc = launch_gather_roots(ctx, max_r, p.root_ids, p.root_h, p.root_c, p.n_roots, s);
+    rc = direct ? launch_gather_roots(ctx, max_r, root_ids, root_h, root_c, nullptr, ctx->host_status, s)
+                : launch_gather_roots(ctx, max_r, p.root_ids, p.root_h, p.root_c, p.n_roots, nullptr, s);
     if (rc != TREELSTM_OK) return rc;
   }
   if (n_nodes > 0) {
@@ -557,7 +575,7 @@ int treelstm_forward_host(treelstm_t* ctx, int n_nodes, const int32_t* left, con
     if (level) TL_CUDA(ctx, cudaMemcpyAsync(level, p.level, nb, cudaMemcpyDeviceToHost, s));
     if (order) TL_CUDA(ctx, cudaMemcpyAsync(order, p.order, nb, cudaMemcpyDeviceToHost, s));
   }
-  if (want_roots && max_r > 0) {
+  if (want_roots && max_r > 0 && !direct) {
     // the number of roots is not known on the host yet: copy max_r rows (rows past n_roots are
     // unspecified) - callers pass the number of trees they submitted
     if (root_ids && root_h && root_c && max_r == max_roots &&
@@ -570,7 +588,7 @@ int treelstm_forward_host(treelstm_t* ctx, int n_nodes, const int32_t* left, con
     }
   }
   // the level and root counts come back with the control block that the status read copies anyway
-  rc = treelstm_status_sync(ctx);
+  rc = direct ? finish_status(ctx) : treelstm_status_sync(ctx);
   const DevStatus* hs = reinterpret_cast<const DevStatus*>(ctx->host_status);
   const bool ok = rc == TREELSTM_OK;
   if (n_levels) *n_levels = ok ? hs->n_levels : 0;

@@ -286,7 +286,7 @@ inline int* check_counters(void* ws, const WsLayout& lay) {
 
 // roots (schedule.cu)
 int launch_gather_roots(treelstm* ctx, int max_roots, int32_t* root_ids, float* root_h,
-                        float* root_c, int32_t* n_roots, cudaStream_t stream);
+                        float* root_c, int32_t* n_roots, int* status_out, cudaStream_t stream);
 
 #define TL_CUDA(ctx, expr)                                  \
   do {                                                      \

@@ -1000,9 +1000,12 @@ __global__ void k_sched_offsets(int n, const int* level, const int* order, int* 
 
 __global__ void k_gather_roots(int max_roots, int H, const int* roots, const float* h,
                                const float* c, int* root_ids, float* root_h, float* root_c,
-                               int* n_roots_out, const DevStatus* st) {
+                               int* n_roots_out, const DevStatus* st, int* status_out) {
   const int n_roots = st->status == 0 ? min(st->n_roots, max_roots) : 0;
   if (blockIdx.x == 0 && threadIdx.x == 0 && n_roots_out) *n_roots_out = n_roots;
+  // the control block to pinned host memory (the destinations may lie there as well): no copy behind this kernel
+  if (blockIdx.x == 0 && status_out && threadIdx.x < sizeof(DevStatus) / sizeof(int))
+    status_out[threadIdx.x] = reinterpret_cast<const int*>(st)[threadIdx.x];
   for (int t = blockIdx.x; t < n_roots; t += gridDim.x) {
     const int node = roots[t];   // written by the scheduler from ids below n
     if (threadIdx.x == 0 && root_ids) root_ids[t] = node;
@@ -1182,14 +1185,14 @@ int launch_check_counts(treelstm* ctx, int n, const int32_t* rows, const int32_t
 }
 
 int launch_gather_roots(treelstm* ctx, int max_roots, int32_t* root_ids, float* root_h,
-                        float* root_c, int32_t* n_roots, cudaStream_t stream) {
+                        float* root_c, int32_t* n_roots, int* status_out, cudaStream_t stream) {
   const auto& L = ctx->last;
   char* base = static_cast<char*>(L.ws);
   const DevStatus* st = reinterpret_cast<const DevStatus*>(base + L.lay.status);
   const int* roots = reinterpret_cast<const int*>(base + L.lay.roots);
   int blocks = max_roots < 1 ? 1 : (max_roots < 1184 ? max_roots : 1184);
   k_gather_roots<<<blocks, 128, 0, stream>>>(max_roots, ctx->H, roots, L.h, L.c, root_ids, root_h,
-                                             L.c ? root_c : nullptr, n_roots, st);
+                                             L.c ? root_c : nullptr, n_roots, st, status_out);
   ctx->launches += 1;
   TL_CUDA(ctx, cudaGetLastError());
   return TREELSTM_OK;
