@@ -743,12 +743,15 @@ __device__ __forceinline__ void zero_range(T* ptr, size_t count, size_t gtid, si
   for (size_t i = gtid; i < count; i += gthreads) ptr[i] = T(0);
 }
 __global__ void __launch_bounds__(256, 2)
-k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int with_dweight) {
+k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int with_dweight, int tree_parts) {
   extern __shared__ float4 s_dyn4[];
   BwdSmem& sm = *reinterpret_cast<BwdSmem*>(s_dyn4);
   float* s_cls = reinterpret_cast<float*>(s_dyn4) + (sizeof(BwdSmem) + 3) / 4;
   __shared__ int s_flag;
   if (ld_volatile(&p.st->status) != 0) return;
+  // behind k_bwd_begin and the tree kernel: classifier and token table are done, and only forests that trees_pay() leaves
+  const bool after_begin = tree_parts > 0;
+  if (after_begin && trees_pay(p.n, p.st->n_roots, p.H, tree_parts)) return;
   const int n_levels = p.st->n_levels;
   const int n = p.n, H = p.H, E = p.E, C = p.C, J = 5 * H;
 #ifdef TREELSTM_TRACE
@@ -762,20 +765,24 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
   unsigned int arrivals = 0;
   auto barrier = [&]() {
     arrivals += gridDim.x;
-    return grid_barrier(p.st, arrivals, wait_limit, &s_flag, true, &p.st->barrier_bwd);
+    return grid_barrier(p.st, arrivals, wait_limit, &s_flag, true, after_begin ? &p.st->barrier_levels : &p.st->barrier_bwd);
   };
-  if (gtid == 0) { *p.loss = 0.f; *p.n_touched = 0; }
-  zero_range(p.dW, (size_t)(E + 2 * H) * J, gtid, gthreads);
-  zero_range(p.db, (size_t)J, gtid, gthreads);
-  zero_range(p.dWc, (size_t)H * C, gtid, gthreads);
-  zero_range(p.dbc, (size_t)C, gtid, gthreads);
-  zero_range(p.dc, (size_t)n * H, gtid, gthreads);
-  zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
-  zero_range(p.dEmb_rows, (size_t)p.n_leaves * E, gtid, gthreads);
-  if (!barrier()) return;
-  TL_STAMP(trace, kTraceLevels - 1, 1);   // outputs and scratch cleared
-  for (size_t r = gtid; r < (size_t)p.n_leaves; r += gthreads)
-    p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[r], p.n)], p.vocab)] = 1;
+  if (after_begin) {
+    zero_range(p.dc, (size_t)n * H, gtid, gthreads);
+  } else {
+    if (gtid == 0) { *p.loss = 0.f; *p.n_touched = 0; }
+    zero_range(p.dW, (size_t)(E + 2 * H) * J, gtid, gthreads);
+    zero_range(p.db, (size_t)J, gtid, gthreads);
+    zero_range(p.dWc, (size_t)H * C, gtid, gthreads);
+    zero_range(p.dbc, (size_t)C, gtid, gthreads);
+    zero_range(p.dc, (size_t)n * H, gtid, gthreads);
+    zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
+    zero_range(p.dEmb_rows, (size_t)p.n_leaves * E, gtid, gthreads);
+    if (!barrier()) return;
+    TL_STAMP(trace, kTraceLevels - 1, 1);   // outputs and scratch cleared
+    for (size_t r = gtid; r < (size_t)p.n_leaves; r += gthreads)
+      p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[r], p.n)], p.vocab)] = 1;
+  }
   for (size_t r = (size_t)p.n_leaves + gtid; r < (size_t)n; r += gthreads) {   // children by ready position
     const int node = chk(p.st, p.order[r], p.n);
     p.pos_left[r] = p.left[node];
@@ -787,7 +794,8 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
   unsigned int* const s_mask = reinterpret_cast<unsigned int*>(s_dyn4);
   const int mask_cap = (int)(sizeof(BwdSmem) / sizeof(unsigned int));
   int* const group_count = p.tok_slot + p.vocab + 4;   // behind the table and its spare entries
-  if (gridDim.x == 1) {
+  if (after_begin) {
+  } else if (gridDim.x == 1) {
     scan_tokens(p, s_mask, mask_cap);
     classifier_groups(p, 0, 1, s_cls);
   } else {
@@ -795,9 +803,9 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
     classifier_groups(p, blockIdx.x, gridDim.x, s_cls);
   }
   TL_STAMP(trace, kTraceLevels - 1, 3);   // this CTA's part (the first one: the token scan) done
-  if (!barrier()) return;
+  if (!after_begin && !barrier()) return;
   TL_STAMP(trace, kTraceLevels - 1, 4);   // classifier, loss and token scan done everywhere
-  if (gridDim.x > 1) scan_place_groups(p, group_count);   // needs nothing but the counts; its results are read after the kernel
+  if (!after_begin && gridDim.x > 1) scan_place_groups(p, group_count);   // needs nothing but the counts; its results are read after the kernel
   // the first wavefront boundaries in shared memory: no dependent global load after every barrier
   // (filled here, ordered before its first use by the CTA barriers inside the grid barrier above)
   constexpr int kOffCache = 256;
@@ -943,7 +951,7 @@ int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, cu
   if (per_sm < 1) return TREELSTM_ERR_UNSUPPORTED;
   int grid = ctx->sm_count * (per_sm < 2 ? per_sm : 2);
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
-  TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, sizeof(unsigned int), stream));
+  TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, 2 * sizeof(unsigned int), stream));   // and barrier_levels behind it
   const int* lvl_off = ctx->last.level_offset;
   long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
   void* args[] = {&p, &dV, &sizes, &lvl_off, &wait_limit};
@@ -953,6 +961,22 @@ int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, cu
 }
 
 }  // namespace
+
+static int launch_bwd_persistent(treelstm* ctx, BwdParams& p, size_t cls_smem, int with_dweight, int tree_parts, cudaStream_t stream) {
+  const size_t smem = ((sizeof(BwdSmem) + 3) / 4) * 4 + cls_smem;
+  TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_persistent, 256, smem));
+  if (per_sm < 1) return TREELSTM_ERR_UNSUPPORTED;
+  int grid = ctx->sm_count * (per_sm < 2 ? per_sm : 2);
+  if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
+  const int* lvl_off = ctx->last.level_offset;
+  long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
+  void* args[] = {&p, &lvl_off, &wait_limit, &with_dweight, &tree_parts};
+  TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_persistent, dim3(grid), dim3(256), args, smem, stream));
+  ctx->launches += 1;
+  return TREELSTM_OK;
+}
 
 int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW, float* db,
                     float* dWc, float* dbc, int32_t* touched_ids, float* dEmb_rows,
@@ -1004,24 +1028,15 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
     if (ctx->opt.dw_tensor_cores && trees_take(ctx, n)) {
       int rc = launch_bwd_begin(ctx, p, nullptr, {(E + 2 * (size_t)H) * J, J, 0}, stream);
       if (rc == TREELSTM_OK) rc = launch_backward_trees(ctx, stream);
+      const int tree_parts = trees_parts(ctx, n, true, true);
+      if (rc == TREELSTM_OK && !trees_always_pay(n, H, tree_parts)) rc = launch_bwd_persistent(ctx, p, cls_smem, 0, tree_parts, stream);
       return rc != TREELSTM_OK ? rc : launch_dweight_tc(ctx, n, L.order, L.level_offset, L.token, L.left, L.right, L.h, p.dz, dW, db,
                                                         p.tok_slot, dEmb_rows, p.st, stream);
     }
-    const size_t smem = ((sizeof(BwdSmem) + 3) / 4) * 4 + cls_smem;
-    TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0;
-    TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_persistent, 256, smem));
-    if (per_sm < 1) return TREELSTM_ERR_UNSUPPORTED;
-    int grid = ctx->sm_count * (per_sm < 2 ? per_sm : 2);
-    if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
-    DevStatus* st = p.st;
-    TL_CUDA(ctx, cudaMemsetAsync(&st->barrier_bwd, 0, sizeof(unsigned int), stream));
-    const int* lvl_off = L.level_offset;
-    long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
-    int with_dweight = ctx->opt.dw_tensor_cores ? 0 : 1;
-    void* args[] = {&p, &lvl_off, &wait_limit, &with_dweight};
-    TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_persistent, dim3(grid), dim3(256), args, smem, stream));
-    ctx->launches += 1;
+    TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, sizeof(unsigned int), stream));
+    const int with_dweight = ctx->opt.dw_tensor_cores ? 0 : 1;
+    const int rc = launch_bwd_persistent(ctx, p, cls_smem, with_dweight, 0, stream);
+    if (rc != TREELSTM_OK) return rc;
     if (!with_dweight)
       return launch_dweight_tc(ctx, n, L.order, L.level_offset, L.token, L.left, L.right, L.h, p.dz, dW, db, p.tok_slot,
                                dEmb_rows, p.st, stream);

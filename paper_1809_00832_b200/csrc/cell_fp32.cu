@@ -27,6 +27,7 @@ struct FwdParams {
   DevStatus* st;
   long long wait_limit;
   int w_stationary, a_row, w_row;   // persistent kernel: W_h slice resident in shared memory; row strides (floats)
+  int tree_parts = 0;               // > 0: launched behind the tree kernels, leaves done; takes the forests that trees_pay() leaves to it
   int early_start = 0;              // persistent kernel: launched under the scheduler, waits for it on the device
   long long* trace = nullptr;       // cycle stamps of the persistent kernel (trace builds), else nullptr
 };
@@ -367,6 +368,10 @@ k_fwd_fp32_persistent(FwdParams p) {
   // Launched as a programmatic dependent of the ready-set construction (p.early_start), the kernel
   // gets here while that one still runs: the weight slice needs nothing from it and is fetched first.
   int n_levels = 0;
+  if (p.tree_parts > 0) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (ld_volatile(&p.st->status) != 0 || trees_pay(p.n, p.st->n_roots, p.H, p.tree_parts)) return;
+  }
   if (!p.early_start) {
     if (ld_volatile(&p.st->status) != 0) return;
     n_levels = p.st->n_levels;
@@ -383,7 +388,8 @@ k_fwd_fp32_persistent(FwdParams p) {
       Ws[col * w_row + k] = v;
     }
   }
-  {
+  const int first_level = p.tree_parts > 0 ? 1 : 0;
+  if (first_level == 0) {
     // The leaf wavefront streams W_x and the leaves' embedding rows chunk by chunk, one dependent fetch per
     // chunk: asked into L2 now (which nodes are leaves and their tokens are the caller's arrays, readable
     // before the schedule exists; tokens are clamped, nothing has been validated yet), those fetches find
@@ -419,7 +425,7 @@ k_fwd_fp32_persistent(FwdParams p) {
   __syncthreads();
   auto level_begin = [&](int l) { return l < kOffCache ? s_off[l] : p.level_offset[l]; };
   bool ids_ahead = false;   // uniform: the row ids of this CTA's first tile of the wavefront are in shared memory
-  for (int lvl = 0; lvl < n_levels; ++lvl) {
+  for (int lvl = first_level; lvl < n_levels; ++lvl) {
     const int begin = level_begin(lvl), end = level_begin(lvl + 1);
     const int tmr = rows_per_tile(end - begin, tiles_u, p.n_sms);
     const int tiles = ((end - begin + tmr - 1) / tmr) * tiles_u;
@@ -447,7 +453,7 @@ k_fwd_fp32_persistent(FwdParams p) {
       // ids of this CTA's first tile of the next wavefront while the barrier is pending (three
       // dependent loads off the path that follows the barrier).
       const bool passed = grid_barrier_with(
-          p.st, (unsigned)(lvl + 1) * gridDim.x, p.wait_limit, &s_flag, true, nullptr, nullptr, [&]() {
+          p.st, (unsigned)(lvl + 1 - first_level) * gridDim.x, p.wait_limit, &s_flag, true, nullptr, nullptr, [&]() {
             if (!p.w_stationary) return;
             const int i = (int)threadIdx.x - 32;
             if (i >= TM) return;
@@ -478,9 +484,13 @@ int launch_forward_fp32(treelstm* ctx, int n, const int32_t* left, const int32_t
                         const int32_t* level_offset_dev, const int32_t* level_offset_host,
                         int n_levels_host, int flags, void* ws, const WsLayout& lay,
                         cudaStream_t stream) {
+  int tree_parts = 0;
   if ((flags & TREELSTM_PERSISTENT) && trees_take(ctx, n)) {
-    return launch_forward_trees(ctx, n, left, right, token, h, c, (flags & TREELSTM_SAVE_FOR_BACKWARD) != 0, ws, lay,
-                                ctx->opt.overlap_launch && scheduler_lets_start(ctx, n), stream);
+    const bool running = ctx->opt.overlap_launch && scheduler_lets_start(ctx, n);
+    const int rc = launch_forward_trees(ctx, n, left, right, token, h, c, (flags & TREELSTM_SAVE_FOR_BACKWARD) != 0, ws, lay, running, stream);
+    if (rc != TREELSTM_OK) return rc;
+    tree_parts = trees_parts(ctx, n, false, running);
+    if (trees_always_pay(n, ctx->H, tree_parts)) return TREELSTM_OK;
   }
   char* base = static_cast<char*>(ws);
   FwdParams p;
@@ -494,6 +504,7 @@ int launch_forward_fp32(treelstm* ctx, int n, const int32_t* left, const int32_t
   p.st = reinterpret_cast<DevStatus*>(base + lay.status);
   p.wait_limit = ctx->opt.wait_limit_kcycles * 1024;
   p.w_stationary = 0; p.a_row = 0; p.w_row = 0;
+  p.tree_parts = tree_parts;
 #ifdef TREELSTM_TRACE
   p.trace = reinterpret_cast<long long*>(base + lay.trace) + kTraceSlots * kTraceLevels;   // second table: the backward clears the first
   if (flags & TREELSTM_PERSISTENT)

@@ -20,8 +20,9 @@ struct DevStatus {
   unsigned int barrier;  // arrival counter of the persistent kernels' grid barrier
   int n_touched;         // distinct leaf tokens (backward)
   unsigned int barrier_bwd;  // arrival counter of the one-launch backward pass (cleared by its launch)
+  unsigned int barrier_levels;  // the same of its wavefronts alone, behind k_bwd_begin
   int tail_from;         // persistent bf16 forward: first wavefront the cluster kernel takes (or would take), n_levels if none
-  int pad[56];
+  int pad[55];
 };
 static_assert(sizeof(DevStatus) == 256, "control block is one 256-byte line group");
 
@@ -99,6 +100,19 @@ struct TreesShape {
   int U = 0, JL = 0, nseg = 0, chunks = 0, nc = 0;
   int bthreads = 0, bseg = 0, BC = 0, TPA = 0;
 };
+
+// Whether a TreeLSTM forest of n nodes and n_roots trees goes to the tree kernels (trees_fp32.cu) or to the kernels that
+// take a wavefront over the whole GPU.  A cluster takes about 1600 cycles per internal node (H = 150 and 256 alike: the
+// slice per CTA is), a grid-wide wavefront 9000 and more: at least 13 of them are assumed, and 12 TFLOP/s behind them.
+// The host knows neither count, so both kernels are launched and ask here.
+__host__ __device__ inline bool trees_pay(int n, int n_roots, int H, int clusters) {
+  const int internal = (n - n_roots) / 2, busy = n_roots < clusters ? n_roots : clusters;
+  if (internal <= 0 || busy <= 0) return true;
+  return 1600.f * (float)internal / (float)busy < 117000.f + (float)internal * (float)H * (float)H * 3.2e-3f;
+}
+
+// The same for every number of trees: forests so small that one cluster alone is faster.
+inline bool trees_always_pay(int n, int H, int clusters) { return clusters > 0 && trees_pay(n, 1, H, 1); }
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 inline size_t round_up_sz(size_t x, size_t m) { return (x + m - 1) / m * m; }
@@ -225,6 +239,7 @@ size_t plan_trees(treelstm* ctx);                        // bytes of the registe
 int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream);
 int pack_trees(treelstm* ctx, cudaStream_t stream);      // after the weights have changed
 bool trees_take(const treelstm* ctx, int n);
+int trees_parts(const treelstm* ctx, int n, bool backward, bool after_running);   // clusters that a launch takes
 int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
                          float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
 int launch_backward_trees(treelstm* ctx, cudaStream_t stream);   // dz of every node (TreeRNN / RNTN: and dh of the leaves) from dh

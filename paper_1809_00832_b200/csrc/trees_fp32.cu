@@ -208,7 +208,7 @@ __device__ __forceinline__ void load_kids(const TreesParams& p, const TreesSmem&
 // in leaf[]; par[q] and leaf_par[] say whose child a node is: 2 x number of the caller + side, kNoCaller for a root.  One
 // warp; every CTA of the cluster gets the same lists.
 constexpr unsigned short kNoCaller = 0xFFFF;
-struct Walk { int depths, internal, leaves; };
+struct Walk { int depths, internal, leaves, roots; };   // roots: of the whole forest
 __device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, Walk* out) {
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
@@ -280,7 +280,7 @@ __device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem
     }
     lo = hi;
   }
-  if (lane == 0) *out = fits ? Walk{depth, count, leaves} : Walk{0, 0, 0};
+  if (lane == 0) *out = fits ? Walk{depth, count, leaves, rank0} : Walk{0, 0, 0, rank0};
 }
 
 // ---- forward -------------------------------------------------------------------------------------- //
@@ -307,7 +307,8 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   __syncthreads();
   TL_STAMP(trace, kTraceLevels - 1, 2);
-  const Walk walk = s_walk;
+  Walk walk = s_walk;
+  if (CELL == kLstm && !trees_pay(p.n, walk.roots, p.H, parts)) walk = Walk{0, 0, 0, walk.roots};   // the grid-wide kernel's forest
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
   const unsigned short* start = reinterpret_cast<const unsigned short*>(sm + s.start);
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     TL_STAMP(trace, d, 4);
   }
   // what follows on the stream waits for this grid only: it must not end before the scheduler ahead of it has
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---- TreeLSTM leaves ------------------------------------------------------------------------------ //
@@ -631,8 +632,9 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
       }
     }
   }
-  // the kernel behind this one waits for this grid only: it must not end before the scheduler ahead of it has
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // the kernel behind this one waits for this grid only: it must not end before the scheduler ahead of it has (one CTA
+  // is enough for that; the others make room for that kernel)
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 
@@ -660,6 +662,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;
 #endif
   TL_STAMP(trace, kTraceLevels - 1, 0);
+  if (CELL == kLstm && !trees_pay(p.n, p.st->n_roots, p.H, parts)) {   // the grid-wide kernel's forest (the schedule is the forward's)
+    if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   float w[kWords];
 #pragma unroll
   for (int q = 0; q < kWords; ++q) w[q] = __ldg(p.W + ((size_t)rank * kWords + q) * nt + tid);
@@ -1091,10 +1097,6 @@ TreesParams trees_params(treelstm* ctx, int n, const int32_t* left, const int32_
 // starts late end late).  `after_running`: the kernel may start while the one ahead of it on the stream still runs (it
 // waits on the device for its end).
 int launch_trees(treelstm* ctx, TreesKernel kernel, const TreesParams& p, int threads, int clusters, bool after_running, cudaStream_t stream) {
-  const int cap = ctx->opt.max_ctas / p.s.cs;
-  if (ctx->opt.max_ctas > 0 && clusters > cap) clusters = cap;
-  if (clusters > p.n) clusters = p.n;                    // (a tree is a node at least)
-  if (clusters < 1) clusters = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * p.s.cs); cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = kSmemMax; cfg.stream = stream;
@@ -1171,6 +1173,15 @@ bool trees_take(const treelstm* ctx, int n) {
          trees_smem(n, bwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0;
 }
 
+int trees_parts(const treelstm* ctx, int n, bool backward, bool after_running) {
+  const auto& t = ctx->trees;
+  int clusters = backward ? t.clusters_bwd : t.clusters;
+  if (after_running && !backward && (ctx->sm_count - 1) / t.s.cs < clusters) clusters = (ctx->sm_count - 1) / t.s.cs;   // a single scheduling CTA keeps its SM
+  if (ctx->opt.max_ctas > 0 && ctx->opt.max_ctas / t.s.cs < clusters) clusters = ctx->opt.max_ctas / t.s.cs;
+  if (clusters > n) clusters = n;                        // (a tree is a node at least)
+  return clusters < 1 ? 1 : clusters;
+}
+
 int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
                          float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream) {
   const auto& s = ctx->trees.s;
@@ -1196,7 +1207,7 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
     }
     ctx->launches += 1;
   }
-  return launch_trees(ctx, forward_kernel(ctx->cell), p, kFwdT, after_running ? max(1, (ctx->sm_count - 1) / s.cs < ctx->trees.clusters ? (ctx->sm_count - 1) / s.cs : ctx->trees.clusters) : ctx->trees.clusters, after_running, stream);
+  return launch_trees(ctx, forward_kernel(ctx->cell), p, kFwdT, trees_parts(ctx, n, false, after_running), after_running, stream);
 }
 
 int launch_backward_trees(treelstm* ctx, cudaStream_t stream) {
@@ -1205,7 +1216,7 @@ int launch_backward_trees(treelstm* ctx, cudaStream_t stream) {
   p.W = ctx->trees.Wb;
   p.gates = reinterpret_cast<float*>(static_cast<char*>(L.ws) + L.lay.gates);
   if (p.trace) p.trace += kTraceSlots * kTraceLevels;
-  return launch_trees(ctx, backward_kernel(ctx->cell, p.s), p, p.s.bthreads, ctx->trees.clusters_bwd, true, stream);
+  return launch_trees(ctx, backward_kernel(ctx->cell, p.s), p, p.s.bthreads, trees_parts(ctx, L.n, true, true), true, stream);
 }
 
 int launch_rec_grads(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb_rows, const int* tok_slot, cudaStream_t stream) {
