@@ -40,6 +40,14 @@ WsLayout ws_layout(const treelstm* ctx, int n, bool with_backward) {
     L.tok_slot = take(4 * ((size_t)ctx->vocab + 4 + ((size_t)ctx->vocab + 127) / 128));   // vocab + 1 entries in use, the scan
                                                                    // reads whole quads; then one count per 128 ids
   }
+  L.img_dz = L.img_x0 = L.img_x1 = L.img_end = off;
+  // forests that one cluster may be too slow for: operands of the backward pass split into bf16 pieces
+  if (with_backward && ctx->wsp && !trees_always_pay((int)nn, ctx->H, 1)) {
+    L.img_dz = take(image_bytes((int)nn, 5 * ctx->H));
+    L.img_x0 = take(image_bytes((int)nn, ctx->E + 1));
+    L.img_x1 = take(image_bytes((int)nn, 2 * ctx->H + 1));
+    L.img_end = off;
+  }
   L.trace = off;
 #ifdef TREELSTM_TRACE
   L.trace = take(2 * sizeof(long long) * kTraceSlots * kTraceLevels);   // grid kernel | cluster kernel
@@ -63,7 +71,8 @@ int copy_params(treelstm* ctx, const float* emb, const float* W, const float* b,
     int rc = pack_weights_bf16(ctx, s);
     if (rc != TREELSTM_OK) return rc;
   }
-  const int rc = pack_trees(ctx, s);
+  int rc = pack_trees(ctx, s);
+  if (rc == TREELSTM_OK) rc = pack_wide_backward(ctx, s);
   if (rc != TREELSTM_OK) return rc;
   TL_CUDA(ctx, cudaStreamSynchronize(s));
   return TREELSTM_OK;
@@ -232,6 +241,7 @@ int treelstm_create(treelstm_t** out, int H, int E, int vocab, const float* emb,
       take(ctx->bp_x, 4 * groups * 24);
     }
     take(images, trees);
+    if (const size_t split = wide_backward_bytes(ctx)) take(ctx->wsp, split);
     if (!pass && (cudaMalloc((void**)&ctx->memory, off) != cudaSuccess ||
                   cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess))
       return fail(TREELSTM_ERR_CUDA);

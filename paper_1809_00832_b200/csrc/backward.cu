@@ -11,7 +11,7 @@
 //   dz_o = dh tanh(c) o(1-o)   dz_i = dc u i(1-i)   dz_u = dc i (1-u^2)   dz_f* = dc c_* f*(1-f*)
 //   dIn  = W dz  (rows [0,E): embedding row of a leaf; rows [E,E+2H): dh of the two children)
 //   dW   = sum_n in_n (x) dz_n,   db = sum_n dz_n
-#include "common.cuh"
+#include "split_tc.cuh"
 
 namespace tl {
 
@@ -398,10 +398,10 @@ __device__ void dinput_block(const BwdParams& p, int row_begin, int row_end, int
 // How many CTAs share the contraction of one dIn tile.  A 64 x 64 tile costs about 4 k cycles per
 // 32-wide chunk of the contraction whatever the number of valid rows, so a wavefront with few tiles
 // spreads the chunks over as many CTAs as there are (about two per SM), down to one chunk each.
-__host__ __device__ inline int dinput_splits(int tiles, int J) {
+__host__ __device__ inline int dinput_splits(int tiles, int J, int blocks = 296) {
   const int chunks_all = (J + BK - 1) / BK;
-  if (tiles >= 148) return 1;
-  int s = 296 / (tiles > 0 ? tiles : 1);
+  if (tiles >= blocks / 2) return 1;
+  int s = blocks / (tiles > 0 ? tiles : 1);
   if (s < 6) s = 6;
   return s < chunks_all ? s : chunks_all;
 }
@@ -491,7 +491,7 @@ __device__ __forceinline__ int gate_of_column(int j, int H) { return (j >= H) + 
 // branch (rows and columns beyond the block are clamped onto valid ones and discarded afterwards), so that
 // they are in flight together: one round trip instead of one per element; then the arithmetic and the stores.
 __device__ __forceinline__ void fused_gate_gradients(const BwdParams& p, const FusedItem& it, DinputSmem& sm, int ib,
-                                                     int buf, int j0) {
+                                                     int buf, int j0, unsigned char* image) {
   const int H = p.H, J = 5 * H, tid = threadIdx.x;
   float dhn[kLd], dci[kLd], go[kLd], cn[kLd], g1[kLd], g2[kLd];
 #pragma unroll
@@ -529,7 +529,11 @@ __device__ __forceinline__ void fused_gate_gradients(const BwdParams& p, const F
         const float gi = g1[q], gu = g2[q];
         dz = g == 0 ? dcn * gu * gi * (1.f - gi) : dcn * gi * (1.f - gu * gu);
       }
-      if (keep) p.dz[(size_t)node * J + j] = dz;
+      if (keep) {
+        const int pos = it.row0 + i;
+        if (image) split_store1_unit(image + ((size_t)(pos >> 6) * img_units(J) + (j >> 6)) * kUnitBytes, pos & 63, j & 63, dz);
+        else p.dz[(size_t)node * J + j] = dz;
+      }
     }
     sm.As[buf][i][e % BK] = dz;
   }
@@ -558,9 +562,11 @@ __device__ __forceinline__ void fused_chunk(const DinputSmem& sm, int buf, int t
 // One block.  fetched: `f` holds the block's index triples and first weight chunk (fused_fetch was called before
 // the grid barrier) and no thread of the CTA still reads the operand buffers.
 // buffers_free() runs once, when the block no longer needs the operand buffers and before its results go out.
+// image: dz goes there, split (k_bwd_wide), instead of to the fp32 rows.
 template <class FreeFn>
 __device__ __forceinline__ void dinput_fused(const BwdParams& p, const FusedItem& it, DinputSmem& sm, int ib, bool fetched,
-                                             FusedFetch& f, long long* trace, int lvl, FreeFn buffers_free) {
+                                             FusedFetch& f, long long* trace, int lvl, FreeFn buffers_free,
+                                             unsigned char* image = nullptr) {
   (void)trace; (void)lvl;
   if (it.c_lo >= it.chunks) { buffers_free(); return; }   // the same for every thread of the CTA
   const int H = p.H, K = 2 * H;
@@ -573,7 +579,7 @@ __device__ __forceinline__ void dinput_fused(const BwdParams& p, const FusedItem
   __syncthreads();
   TL_STAMP(trace, lvl, 8);   // index triples and first weight chunk in shared memory
   float acc[4][4] = {};
-  fused_gate_gradients(p, it, sm, ib, it.c_lo & 1, it.c_lo * BK);
+  fused_gate_gradients(p, it, sm, ib, it.c_lo & 1, it.c_lo * BK, image);
   __syncthreads();
   TL_STAMP(trace, lvl, 5);   // gate gradients of the first chunk formed by all warps
   const int ni = (it.rows + 15) / 16;   // 16-row groups of the tile that hold nodes
@@ -586,7 +592,7 @@ __device__ __forceinline__ void dinput_fused(const BwdParams& p, const FusedItem
     else if (ni == 3) fused_chunk<3>(sm, buf, tx, ty, acc);
     else fused_chunk<4>(sm, buf, tx, ty, acc);
     if (more) {
-      fused_gate_gradients(p, it, sm, ib, buf ^ 1, (cidx + 1) * BK);
+      fused_gate_gradients(p, it, sm, ib, buf ^ 1, (cidx + 1) * BK, image);
     }
     __syncthreads();
   }
@@ -898,6 +904,273 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
   TL_STAMP(trace, kTraceLevels - 1, 8);
 }
 
+// ---- the wavefronts of a forest that is wide, on the tensor cores ------------------------------ //
+// Behind k_bwd_begin, for the forests that trees_pay() leaves.  A wavefront of more than kFusedMaxRows nodes is
+// dIn = dz W^T with hundreds of rows: on fp32 units that contraction was 600 of the 880 us of the backward pass of
+// 14.6 k nodes (H = 256).  Here its dz is written as split bf16 pieces (BwdImages, the layout the tensor core reads),
+// and tiles of 128 positions x 128 outputs are multiplied with W split once per set of weights: one thread asks for
+// blocks (plain bulk copies of whole tiles), one issues the MMAs, eight warps add the tile to the children's dh.  The
+// contraction is cut into as many pieces as leave no CTA without a tile.  The leaves' dIn (their rows of dEmb) is one
+// more such wavefront.  Narrow wavefronts form their gate gradients inside an fp32 contraction as in k_bwd_persistent.
+// The images stay for the weight gradient.
+constexpr int kWideSmem = 2 * kSpStageBytes + 1024;
+struct WideArgs {
+  const int* level_offset;
+  long long wait_limit;
+  int tree_parts;
+  BwdImages img;
+};
+
+// dz of rows [row0, row0 + cnt) of the ready order (at most eight) -> image; s_dz [8][J]
+__device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& img, int row0, int cnt, int leaf, float* s_dz) {
+  const int H = p.H, J = 5 * H, ju = img_units(J), tid = threadIdx.x;
+  __syncthreads();                                       // the previous rows have left shared memory
+  for (int e = tid; e < cnt * H; e += 256) {
+    const int i = e / H, u = e - i * H;
+    const int node = chk(p.st, p.order[row0 + i], p.n);
+    const int l = leaf ? 0 : chk(p.st, p.pos_left[row0 + i], p.n), r = leaf ? 0 : chk(p.st, p.pos_right[row0 + i], p.n);
+    const float* g = p.gates + (size_t)node * J + u;
+    const float gi = g[0], gl = leaf ? 0.f : g[H], gr = leaf ? 0.f : g[2 * H], go = g[3 * H], gu = g[4 * H];
+    const float cn = p.c[(size_t)node * H + u], dhn = p.dh[(size_t)node * H + u], dci = p.dc[(size_t)node * H + u];
+    const float cl = leaf ? 0.f : p.c[(size_t)l * H + u], cr = leaf ? 0.f : p.c[(size_t)r * H + u];
+    const float tc = tanhf(cn);
+    const float dcn = dci + dhn * go * (1.f - tc * tc);
+    float* z = s_dz + i * J + u;
+    z[0] = dcn * gu * gi * (1.f - gi);
+    z[H] = dcn * cl * gl * (1.f - gl);
+    z[2 * H] = dcn * cr * gr * (1.f - gr);
+    z[3 * H] = dhn * tc * go * (1.f - go);
+    z[4 * H] = dcn * gi * (1.f - gu * gu);
+    if (!leaf) {
+      p.dc[(size_t)l * H + u] = dcn * gl;                // every node has exactly one caller: plain stores
+      p.dc[(size_t)r * H + u] = dcn * gr;
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < cnt * ju * 8; e += 256) {
+    const int i = e / (ju * 8), ch = e - i * ju * 8, pos = row0 + i;
+    float x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = ch * 8 + k < J ? s_dz[i * J + min(ch * 8 + k, J - 1)] : 0.f;
+    split_store8_unit(img.dz + ((size_t)(pos >> 6) * ju + (ch >> 3)) * kUnitBytes, pos & 63, ch & 7, x);
+  }
+}
+
+__global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
+  extern __shared__ unsigned char wide_dyn[];
+  __shared__ __align__(8) uint64_t s_bars[6];            // full, empty (two stages each), accumulator, drain
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort, s_flag;
+  __shared__ int s_da[kSpTile], s_db[kSpTile];
+  if (ld_volatile(&p.st->status) != 0 || (a.tree_parts > 0 && trees_pay(p.n, p.st->n_roots, p.H, a.tree_parts))) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  unsigned char* const tiles = wide_dyn + ((1024u - (smem_u32(wide_dyn) & 1023u)) & 1023u);
+  DinputSmem& di = *reinterpret_cast<DinputSmem*>(tiles);
+  const uint32_t tiles_addr = smem_u32(tiles), full0 = smem_u32(&s_bars[0]), empty0 = smem_u32(&s_bars[2]),
+                 acc_bar = smem_u32(&s_bars[4]), drain_bar = smem_u32(&s_bars[5]);
+  if (tid == 0) {
+    for (int s = 0; s < 6; ++s) mbar_init(smem_u32(&s_bars[s]), 1);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kSpTile);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = s_tmem;
+  const int n_levels = p.st->n_levels, n = p.n, H = p.H, E = p.E, J = 5 * H, ju = img_units(J);
+  p.n_leaves = n_levels > 0 ? a.level_offset[1] : 0;
+  const int n_leaves = p.n_leaves;
+  const size_t gtid = (size_t)blockIdx.x * 256 + tid, gthreads = (size_t)gridDim.x * 256;
+  unsigned int arrivals = 0;
+  auto barrier = [&]() {
+    arrivals += gridDim.x;
+    return grid_barrier(p.st, arrivals, a.wait_limit, &s_flag, true, &p.st->barrier_levels);
+  };
+  bool ok = true;
+  // ---- set-up: dc of the roots, children by position, the inputs' images, zeros behind the last position
+  zero_range(p.dc, (size_t)n * H, gtid, gthreads);
+  for (size_t r = (size_t)n_leaves + gtid; r < (size_t)n; r += gthreads) {
+    const int node = chk(p.st, p.order[r], p.n);
+    p.pos_left[r] = p.left[node];
+    p.pos_right[r] = p.right[node];
+  }
+  {
+    const int xu0 = img_units(E + 1), xu1 = img_units(2 * H + 1), pb1 = n_leaves / 64, pbs = (n + 63) / 64;
+    const int units0 = (n_leaves + 63) / 64 * xu0, units1 = n > n_leaves ? (pbs - pb1) * xu1 : 0;
+    const int r = tid >> 2, c0 = (tid & 3) * 2;
+    for (int q = blockIdx.x; q < units0 + units1; q += gridDim.x) {
+      const int part = q >= units0, qq = part ? q - units0 : q, xu = part ? xu1 : xu0;
+      const int pb = (part ? pb1 : 0) + qq / xu, fb = qq % xu, pos = pb * 64 + r, feats = part ? 2 * H : E;
+      const bool in = part ? pos >= n_leaves && pos < n : pos < n_leaves;
+      const float *s0 = nullptr, *s1 = nullptr;
+      if (in) {
+        const int node = chk(p.st, p.order[pos], p.n);
+        if (part) {
+          s0 = p.h + (size_t)chk(p.st, p.left[node], p.n) * H;
+          s1 = p.h + (size_t)chk(p.st, p.right[node], p.n) * H - H;
+        } else {
+          s0 = p.emb + (size_t)chk(p.st, p.token[node], p.vocab) * E;
+        }
+      }
+#pragma unroll
+      for (int c = c0; c < c0 + 2; ++c) {
+        float x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int f = fb * 64 + c * 8 + k, fc = min(f, feats - 1);
+          x[k] = in ? (f < feats ? (part && fc >= H ? s1 : s0)[fc] : (f == feats ? 1.f : 0.f)) : 0.f;
+        }
+        split_store8_unit(a.img.x[part] + ((size_t)pb * xu + fb) * kUnitBytes, r, c, x);
+      }
+    }
+    const float zero[8] = {};
+    for (size_t q = gtid; q < (size_t)(pbs * 64 - n) * ju * 8; q += gthreads) {
+      const int pos = n + (int)(q / (ju * 8)), ch = (int)(q % (ju * 8));
+      split_store8_unit(a.img.dz + ((size_t)(pos >> 6) * ju + (ch >> 3)) * kUnitBytes, pos & 63, ch & 7, zero);
+    }
+  }
+  ok = barrier();
+  uint32_t put = 0, got = 0, done = 0;
+  bool prepared = false;
+  FusedItem pre_item{};
+  FusedFetch pre_fetch;
+  const int splits_for = 2 * (int)gridDim.x;             // pieces of a narrow contraction over all CTAs
+  auto level_begin = [&](int l) { return a.level_offset[l]; };
+  auto is_fused = [&](int l) { return l > 0 && level_begin(l + 1) - level_begin(l) <= kFusedMaxRows; };
+  for (int lvl = n_levels - 1; lvl >= 0 && ok; --lvl) {
+    const int begin = level_begin(lvl), end = level_begin(lvl + 1), leaf = lvl == 0 ? 1 : 0;
+    if (is_fused(lvl)) {
+      const int ntiles = dinput_tiles(end - begin, 2 * H), nsplits = dinput_splits(ntiles, J, splits_for);
+      for (int vb = blockIdx.x; vb < ntiles * nsplits; vb += gridDim.x) {
+        const bool ready = prepared && vb == (int)blockIdx.x;
+        const FusedItem item = ready ? pre_item : fused_item(p, begin, end, vb % ntiles, vb / ntiles, nsplits);
+        dinput_fused(p, item, di, lvl & 1, ready, pre_fetch, nullptr, lvl, []() {}, a.img.dz);
+      }
+      prepared = false;
+      if (lvl > 1 && is_fused(lvl - 1)) {                // the next wavefront's first block, fetched while the barrier is pending
+        const int b = level_begin(lvl - 1), e = level_begin(lvl), nt = dinput_tiles(e - b, 2 * H), ns = dinput_splits(nt, J, splits_for);
+        if ((int)blockIdx.x < nt * ns) {
+          pre_item = fused_item(p, b, e, blockIdx.x % nt, blockIdx.x / nt, ns);
+          if (pre_item.c_lo < pre_item.chunks) {
+            fused_fetch(p, pre_item, pre_item.c_lo * BK, pre_fetch);
+            prepared = true;
+          }
+        }
+      }
+      ok = barrier();
+      continue;
+    }
+    prepared = false;
+    for (int r0 = begin + 8 * (int)blockIdx.x; r0 < end; r0 += 8 * (int)gridDim.x)
+      wide_gates(p, a.img, r0, min(8, end - r0), leaf, reinterpret_cast<float*>(tiles));
+    asm volatile("fence.proxy.async;" ::: "memory");     // the image is read by bulk copies (and this shared memory written by them)
+    if (!(ok = barrier())) break;
+    asm volatile("fence.proxy.async;" ::: "memory");
+    // dIn: tiles of 128 positions (from a multiple of 64 on) x 128 outputs, the column blocks cut into pieces
+    const int base = begin & ~63, K = leaf ? E : 2 * H, tr = (end - base + 127) / 128, to = (K + 127) / 128;
+    const int all = wsp_kblocks(H);
+    int skip_first = all, skip = 0;                      // a leaf's forget gates are zero: blocks inside [H, 3H) are left out
+    if (leaf) {
+      skip_first = (H + 63) / 64;
+      const int skip_end = 3 * H / 64;
+      skip = skip_end > skip_first ? skip_end - skip_first : 0;
+    }
+    const int kbs = all - skip;
+    int pieces = (int)gridDim.x / (tr * to);
+    pieces = pieces < 1 ? 1 : (pieces > kbs / 2 ? (kbs / 2 < 1 ? 1 : kbs / 2) : pieces);
+    const int per = (kbs + pieces - 1) / pieces;
+    for (int item = blockIdx.x; item < tr * to * pieces && ok; item += gridDim.x) {
+      const int ot = item % to, rt = (item / to) % tr, k0 = item / (to * tr) * per, nk = min(per, kbs - k0);
+      if (nk <= 0) continue;
+      const int pos0 = base + rt * 128;
+      if (tid < kSpTile) {                               // where the rows go
+        const int pos = pos0 + tid;
+        int da = -1, db = 0;
+        if (pos >= begin && pos < end) {
+          if (leaf) da = chk(p.st, p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[pos], p.n)], p.vocab)], p.n_leaves);
+          else { da = chk(p.st, p.pos_left[pos], p.n); db = chk(p.st, p.pos_right[pos], p.n); }
+        }
+        s_da[tid] = da; s_db[tid] = db;
+      }
+      const unsigned char* wt = a.img.w + (size_t)((leaf ? 0 : wsp_tiles_x(E)) + ot) * all * kSpOperandBytes;
+      if (tid == 0) {
+        for (int k = 0; k < nk && ok; ++k, ++put) {
+          const uint32_t stage = put & 1u, dst = tiles_addr + stage * kSpStageBytes, bar = full0 + 8 * stage;
+          if (put >= 2) ok = mbar_wait(empty0 + 8 * stage, ((put >> 1) - 1) & 1u, &s_abort, a.wait_limit, p.st);
+          if (!ok) break;
+          const int kk = k0 + k, kb = kk < skip_first ? kk : kk + skip;
+          mbar_arrive_expect_tx(bar, kSpStageBytes);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < kSpPieces; ++q)
+              bulk_load(dst + q * kSpTileBytes + h * kUnitPieceBytes,
+                        a.img.dz + ((size_t)((pos0 >> 6) + h) * ju + kb) * kUnitBytes + q * kUnitPieceBytes, kUnitPieceBytes, bar);
+          bulk_load(dst + kSpOperandBytes, wt + (size_t)kb * kSpOperandBytes, kSpOperandBytes, bar);
+        }
+      } else if (tid == 32) {
+        for (int k = 0; k < nk && ok; ++k, ++got) {
+          const uint32_t stage = got & 1u, src = tiles_addr + stage * kSpStageBytes;
+          ok = mbar_wait(full0 + 8 * stage, (got >> 1) & 1u, &s_abort, a.wait_limit, p.st);
+          if (!ok) break;
+          tc_fence_after();
+          split_mmas(tmem_base, src, src + kSpOperandBytes, umma_idesc(kSpTile), k == 0);
+          umma_commit(empty0 + 8 * stage);
+          if (k == nk - 1) umma_commit(acc_bar);
+        }
+      }
+      __syncwarp();
+      ok = mbar_wait(acc_bar, done & 1u, &s_abort, a.wait_limit, p.st) && ok;
+      ++done;
+      if (__syncthreads_or(!ok)) { ok = false; break; }
+      tc_fence_after();
+      constexpr int kRowStride = kSpTile + 4;
+      float* stage_out = reinterpret_cast<float*>(tiles);
+      {
+        const int quad = warp & 3, half = warp >> 2;
+        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 64);
+        uint32_t v[64];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
+        tmem_ld_wait();
+        tc_fence_before();
+        float* dst = stage_out + (size_t)(quad * 32 + lane) * kRowStride + half * 64;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
+                                                                __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+      }
+      __syncthreads();
+      for (int r = warp; r < kSpTile; r += 8) {
+        if (s_da[r] < 0) continue;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int c = lane + 32 * i, k = ot * 128 + c;
+          if (k >= K) continue;
+          float* out = leaf ? p.dEmb_rows + (size_t)s_da[r] * E + k
+                            : p.dh + (size_t)(k < H ? s_da[r] : s_db[r]) * H + (k < H ? k : k - H);
+          atomicAdd(out, stage_out[(size_t)r * kRowStride + c]);
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the next bulk copies overwrite the staging rows
+      __syncthreads();
+    }
+    if (ok && lvl > 0) ok = barrier();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (s_abort) {                                         // what was asked for gets a bounded time to land, the MMAs to retire
+    if (tid == 32) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
+    if (tid == 0) for (int s = 0; s < 2; ++s) mbar_drain(full0 + 8 * s, 0);
+    __syncthreads();
+  }
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, kSpTile);
+  }
+}
+
 // What precedes the walk over the trees (trees_fp32.cu), in one cooperative launch: outputs cleared | leaf tokens
 // marked | tokens counted beside the classifier | tokens placed.  The level table stays on the device.
 struct GradSizes { size_t dW, db, dV; };   // floats
@@ -978,6 +1251,17 @@ static int launch_bwd_persistent(treelstm* ctx, BwdParams& p, size_t cls_smem, i
   return TREELSTM_OK;
 }
 
+static int launch_bwd_wide(treelstm* ctx, BwdParams& p, const BwdImages& img, int tree_parts, cudaStream_t stream) {
+  TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmem));
+  int grid = ctx->sm_count;
+  if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
+  WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, tree_parts, img};
+  void* args[] = {&p, &a};
+  TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_wide, dim3(grid), dim3(256), args, kWideSmem, stream));
+  ctx->launches += 1;
+  return TREELSTM_OK;
+}
+
 int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW, float* db,
                     float* dWc, float* dbc, int32_t* touched_ids, float* dEmb_rows,
                     int32_t* n_touched, cudaStream_t stream) {
@@ -1025,13 +1309,23 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
       TL_CUDA(ctx, cudaMemsetAsync(n_touched, 0, sizeof(int), stream));
       return TREELSTM_OK;
     }
-    if (ctx->opt.dw_tensor_cores && trees_take(ctx, n)) {
+    const bool trees = trees_take(ctx, n), wide = L.lay.img_dz != L.lay.img_end;
+    if (ctx->opt.dw_tensor_cores && (trees || wide)) {
       int rc = launch_bwd_begin(ctx, p, nullptr, {(E + 2 * (size_t)H) * J, J, 0}, stream);
-      if (rc == TREELSTM_OK) rc = launch_backward_trees(ctx, stream);
-      const int tree_parts = trees_parts(ctx, n, true, true);
-      if (rc == TREELSTM_OK && !trees_always_pay(n, H, tree_parts)) rc = launch_bwd_persistent(ctx, p, cls_smem, 0, tree_parts, stream);
+      if (rc == TREELSTM_OK && trees) rc = launch_backward_trees(ctx, stream);
+      const int tree_parts = trees ? trees_parts(ctx, n, true, true) : 0;
+      BwdImages img;
+      if (rc == TREELSTM_OK && wide) {
+        img.dz = reinterpret_cast<unsigned char*>(base + L.lay.img_dz);
+        img.x[0] = reinterpret_cast<unsigned char*>(base + L.lay.img_x0);
+        img.x[1] = reinterpret_cast<unsigned char*>(base + L.lay.img_x1);
+        img.w = ctx->wsp;
+        rc = launch_bwd_wide(ctx, p, img, tree_parts, stream);
+      } else if (rc == TREELSTM_OK && !trees_always_pay(n, H, tree_parts)) {
+        rc = launch_bwd_persistent(ctx, p, cls_smem, 0, tree_parts, stream);
+      }
       return rc != TREELSTM_OK ? rc : launch_dweight_tc(ctx, n, L.order, L.level_offset, L.token, L.left, L.right, L.h, p.dz, dW, db,
-                                                        p.tok_slot, dEmb_rows, p.st, stream);
+                                                        p.tok_slot, dEmb_rows, p.st, &img, tree_parts, stream);
     }
     TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, sizeof(unsigned int), stream));
     const int with_dweight = ctx->opt.dw_tensor_cores ? 0 : 1;
@@ -1039,7 +1333,7 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
     if (rc != TREELSTM_OK) return rc;
     if (!with_dweight)
       return launch_dweight_tc(ctx, n, L.order, L.level_offset, L.token, L.left, L.right, L.h, p.dz, dW, db, p.tok_slot,
-                               dEmb_rows, p.st, stream);
+                               dEmb_rows, p.st, nullptr, 0, stream);
     return TREELSTM_OK;
   }
   TL_CUDA(ctx, cudaMemsetAsync(loss, 0, sizeof(float), stream));

@@ -29,7 +29,7 @@ static_assert(sizeof(DevStatus) == 256, "control block is one 256-byte line grou
 // Offsets (bytes) of the regions inside the workspace for a forest of up to n nodes.
 struct WsLayout {
   size_t status, parent, pending, order_tmp, level_offset, roots, table, slot, part_order, part_offset,
-      part_spill, xin, ain, cin, gates, dh, dc, dz, tok_slot, trace, check, pre, total;
+      part_spill, xin, ain, cin, gates, dh, dc, dz, tok_slot, trace, check, pre, img_dz, img_x0, img_x1, img_end, total;
 };
 
 // Cycle stamps of the wavefront kernels (builds with -DTREELSTM_TRACE only): kTraceSlots stamps per
@@ -134,6 +134,7 @@ struct treelstm {
   float* emb = nullptr;  // [vocab][E]
   float* W = nullptr;    // [E+2H][5H]
   float* b = nullptr;    // [5H]
+  unsigned char* wsp = nullptr;   // W split into bf16 pieces for the wide backward (split_tc.cuh), nullptr: not kept
   float* Wcat = nullptr; // TreeRNN / RNTN: [4H^2 + 2H][H] (tensor slices transposed, then W) or [2H][H]
   float* Wc = nullptr;   // [H][C]
   float* bc = nullptr;   // [C]
@@ -279,11 +280,16 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
                     float* dWc, float* dbc, int32_t* touched_ids, float* dEmb_rows,
                     int32_t* n_touched, cudaStream_t stream);
 
+struct BwdImages;   // split_tc.cuh
 // dweight_tc.cu: dW += In^T dZ, db += sum dZ, dEmb_rows += dz_leaves W_x^T on the tensor cores (three bf16 pieces per fp32 value)
 int init_dweight_tc_attributes(treelstm* ctx);
+size_t wide_backward_bytes(const treelstm* ctx);         // split image of W (0: not kept)
+int pack_wide_backward(treelstm* ctx, cudaStream_t stream);
+size_t image_bytes(int n, int features);
 int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t* level_offset, const int32_t* token,
                       const int32_t* left, const int32_t* right, const float* h, const float* dz, float* dW, float* db,
-                      const int* tok_slot, float* dEmb_rows, DevStatus* st, cudaStream_t stream);
+                      const int* tok_slot, float* dEmb_rows, DevStatus* st, const BwdImages* img, int tree_parts,
+                      cudaStream_t stream);
 
 // Checked build: clears the per-row write counters before a forward / compares them after it
 // (schedule.cu); both do nothing in the normal build.  Counters: [h per node | Ain per position | Cin per position].

@@ -20,19 +20,17 @@
 // Two stages of tiles: block b + 1 is built while the MMAs of block b run.  Partial sums of the node
 // runs meet in dW by atomic adds (dW and db are cleared before), whole rows at a time through a
 // shared-memory copy of the accumulator.
-#include "tc_ptx.cuh"
+#include "split_tc.cuh"
 
 namespace tl {
 namespace {
 
-constexpr int kDwThreads = 256;
-constexpr int kDwTile = 128;                     // rows of either operand tile (UMMA M and N)
-constexpr int kDwBlock = 64;                     // nodes per block of the contraction (one swizzle span of bf16)
-constexpr int kDwPieces = 3;                     // bf16 pieces per value
-constexpr int kDwTileBytes = kDwTile * 128;      // one piece of one operand tile: 16 KB
-constexpr int kDwStageBytes = 2 * kDwPieces * kDwTileBytes;   // A and B, three pieces each: 96 KB
+constexpr int kDwThreads = 512;
+constexpr int kDwTile = kSpTile;                 // rows of either operand tile (UMMA M and N)
+constexpr int kDwBlock = kSpBlock;               // nodes per block of the contraction (one swizzle span of bf16)
+constexpr int kDwStageBytes = kSpStageBytes;     // A and B, three pieces each: 96 KB
 constexpr int kDwStages = 2;
-constexpr int kDwMaxRun = 8;                     // blocks per work item at most (index tables in shared memory)
+constexpr int kDwMaxRun = 16;                    // blocks per work item at most (index tables in shared memory)
 constexpr int kDwSmemBytes = kDwStages * kDwStageBytes + 1024;   // + alignment slack
 
 struct DwParams {
@@ -45,25 +43,9 @@ struct DwParams {
   float *dW, *db, *dEmb_rows;   // dEmb_rows == nullptr: the leaves' input gradients are not formed here
   DevStatus* st;
   long long wait_limit;
+  BwdImages img;                // operands split beforehand (forests that went to the grid-wide wavefront kernel)
+  int tree_parts;               // > 0: the tree kernels took the forest if trees_pay() says so, and img holds nothing
 };
-
-// (x, y) -> three words of two bf16 pieces each (x in the low half): x = x0 + x1 + x2, y likewise
-__device__ __forceinline__ void split3_pair(float x, float y, uint32_t& w0, uint32_t& w1, uint32_t& w2) {
-  auto pack = [](float a, float b) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&v);
-  };
-  w0 = pack(x, y);
-  x -= __uint_as_float(w0 << 16);  y -= __uint_as_float(w0 & 0xFFFF0000u);
-  w1 = pack(x, y);
-  x -= __uint_as_float(w1 << 16);  y -= __uint_as_float(w1 & 0xFFFF0000u);
-  w2 = pack(x, y);
-}
-
-// byte offset of the 16-byte piece (row r, nodes 8 c .. 8 c + 7) inside a K-major tile with the 128-byte swizzle
-__device__ __forceinline__ uint32_t swz_piece(int r, int c) {
-  return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4));
-}
 
 // One operand tile (128 rows x 64 nodes, three pieces) of block `kb` of the work item, in two steps: the
 // fp32 values into registers (tile_load: nothing but loads, so all of a block's are in flight together),
@@ -72,16 +54,16 @@ __device__ __forceinline__ uint32_t swz_piece(int r, int c) {
 // nodes ([h_l | h_r], then the row of ones), 2: gate columns (dz).  row0: first row of the tile within its
 // operand.  s_node / s_ia / s_ib: per node of the item its id and where its input row comes from (token; left,
 // right child); entries behind the item's last node are 0 and their values are discarded.  Warp w takes the
-// nodes 8 w .. 8 w + 7 of the block, lane l the rows l, l + 32, l + 64, l + 96.
+// nodes 8 (w mod 8) .. + 7 of the block, lane l the rows l and l + 32 of the tile's lower (w < 8) or upper half.
 template <int kKind>
 __device__ __forceinline__ void tile_load(const DwParams& p, int row0, const int* s_node, const int* s_ia,
-                                          const int* s_ib, int kb, float (&v)[4][8]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                                          const int* s_ib, int kb, float (&v)[2][8]) {
+  const int warp = (threadIdx.x >> 5) & 7, half = threadIdx.x >> 8, lane = threadIdx.x & 31;
   const int H = p.H, E = p.E, J = 5 * H;
   const int rows = kKind == 0 ? E : (kKind == 1 ? 2 * H : J);
 #pragma unroll
-  for (int rg = 0; rg < 4; ++rg) {
-    const int fc = min(row0 + rg * 32 + lane, rows - 1);
+  for (int rg = 0; rg < 2; ++rg) {
+    const int fc = min(row0 + half * 64 + rg * 32 + lane, rows - 1);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = kb * kDwBlock + 8 * warp + i;
@@ -95,61 +77,46 @@ __device__ __forceinline__ void tile_load(const DwParams& p, int row0, const int
 }
 template <int kKind>
 __device__ __forceinline__ void tile_store(const DwParams& p, unsigned char* tile, int row0, int valid_nodes,
-                                           const float (&v)[4][8]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                                           const float (&v)[2][8]) {
+  const int warp = (threadIdx.x >> 5) & 7, half = threadIdx.x >> 8, lane = threadIdx.x & 31;
   const int rows = kKind == 0 ? p.E : (kKind == 1 ? 2 * p.H : 5 * p.H);   // row `rows` of an input operand is the ones
 #pragma unroll
-  for (int rg = 0; rg < 4; ++rg) {
-    const int r = rg * 32 + lane, f = row0 + r;
-    uint32_t w0[4], w1[4], w2[4];
+  for (int rg = 0; rg < 2; ++rg) {
+    const int r = half * 64 + rg * 32 + lane, f = row0 + r;
+    float x[8];
 #pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-      float x[2];
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const bool node_ok = 8 * warp + i + e < valid_nodes;
-        x[e] = node_ok && f < rows ? v[rg][i + e] : 0.f;
-        if (kKind != 2 && node_ok && f == rows) x[e] = 1.f;
-      }
-      split3_pair(x[0], x[1], w0[i >> 1], w1[i >> 1], w2[i >> 1]);
+    for (int i = 0; i < 8; ++i) {
+      const bool node_ok = 8 * warp + i < valid_nodes;
+      x[i] = node_ok && f < rows ? v[rg][i] : 0.f;
+      if (kKind != 2 && node_ok && f == rows) x[i] = 1.f;
     }
-    unsigned char* dst = tile + swz_piece(r, warp);
-    *reinterpret_cast<uint4*>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-    *reinterpret_cast<uint4*>(dst + kDwTileBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-    *reinterpret_cast<uint4*>(dst + 2 * kDwTileBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
+    split_store8(tile, r, warp, x);
   }
 }
 
 // The third kind of work item, dEmb_rows += dz_leaves W_x^T, contracts over the gate columns, which are
 // contiguous in both operands (a leaf's dz row, a row of W): no transposition, a thread takes eight
-// consecutive columns of one row - one 16-byte piece - for four rows.  row_ptr(r): start of tile row r in
+// consecutive columns of one row - one 16-byte piece - for two rows.  row_ptr(r): start of tile row r in
 // global memory or nullptr; j0: first column of the block; J: columns in a row.
 template <class RowFn>
-__device__ __forceinline__ void rows_load(RowFn row_ptr, int j0, int J, float (&v)[4][8]) {
+__device__ __forceinline__ void rows_load(RowFn row_ptr, int j0, int J, float (&v)[2][8]) {
   const int c = threadIdx.x & 7;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float* row = row_ptr((threadIdx.x >> 3) + 32 * i);
+  for (int i = 0; i < 2; ++i) {
+    const float* row = row_ptr((threadIdx.x >> 3) + 64 * i);
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[i][e] = row[min(j0 + 8 * c + e, J - 1)];
   }
 }
-__device__ __forceinline__ void rows_store(unsigned char* tile, int rows_valid, int j0, int J, const float (&v)[4][8]) {
+__device__ __forceinline__ void rows_store(unsigned char* tile, int rows_valid, int j0, int J, const float (&v)[2][8]) {
   const int c = threadIdx.x & 7;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = (threadIdx.x >> 3) + 32 * i;
-    uint32_t w0[4], w1[4], w2[4];
+  for (int i = 0; i < 2; ++i) {
+    const int r = (threadIdx.x >> 3) + 64 * i;
+    float x[8];
 #pragma unroll
-    for (int e = 0; e < 8; e += 2) {
-      const float x = r < rows_valid && j0 + 8 * c + e < J ? v[i][e] : 0.f;
-      const float y = r < rows_valid && j0 + 8 * c + e + 1 < J ? v[i][e + 1] : 0.f;
-      split3_pair(x, y, w0[e >> 1], w1[e >> 1], w2[e >> 1]);
-    }
-    unsigned char* dst = tile + swz_piece(r, c);
-    *reinterpret_cast<uint4*>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-    *reinterpret_cast<uint4*>(dst + kDwTileBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-    *reinterpret_cast<uint4*>(dst + 2 * kDwTileBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
+    for (int e = 0; e < 8; ++e) x[e] = r < rows_valid && j0 + 8 * c + e < J ? v[i][e] : 0.f;
+    split_store8(tile, r, c, x);
   }
 }
 
@@ -192,10 +159,102 @@ __host__ __device__ inline int dw_run(int n, int n_leaves, int H, int E, bool le
   return run;
 }
 
+// The sums over the nodes where the wavefront kernel has left both operands split (BwdImages): no thread touches a
+// value before the accumulator.  One thread asks for the units of a block, one issues its MMAs, two stages; bound by the
+// shared-memory reads of the MMAs (8 KB per 64 cycles of tensor pipe) and the 96 KB of a block on their way in.
+// (Splitting inside this kernel instead converts every value of dz once per row tile: 335 us for 14.6 k nodes,
+// H = 256, tensor pipe 24 % active, 43 % of the issue slots taken by conversions.)
+__device__ void dw_from_images(const DwParams& p, int n_leaves, unsigned char* tiles, uint32_t full_bar0, uint32_t empty_bar0,
+                               uint32_t acc_bar, uint32_t tmem_base, int* s_abort_) {
+  volatile int* s_abort = s_abort_;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int H = p.H, E = p.E, J = 5 * H;
+  const int ju = img_units(J), xu[2] = {img_units(E + 1), img_units(2 * H + 1)};
+  const int n_tiles = (J + kDwTile - 1) / kDwTile;
+  const int m_tiles[2] = {(E + 1 + kDwTile - 1) / kDwTile, (2 * H + 1 + kDwTile - 1) / kDwTile};
+  const int pb_lo[2] = {0, n_leaves / 64}, pb_hi[2] = {(n_leaves + 63) / 64, p.n > n_leaves ? (p.n + 63) / 64 : n_leaves / 64};
+  // runs of blocks as long as leave every CTA about two items (each ends in an atomic add per output)
+  int run = 1, items[2];
+  for (;; run *= 2) {
+    for (int q = 0; q < 2; ++q) items[q] = m_tiles[q] * n_tiles * ((pb_hi[q] - pb_lo[q] + run - 1) / run);
+    if (items[0] + items[1] <= 2 * (int)gridDim.x || run >= 256) break;
+  }
+  const uint32_t tiles_addr = smem_u32(tiles), idesc = umma_idesc_mn(kDwTile);
+  uint32_t put = 0, got = 0;             // blocks asked for / multiplied so far (thread 0 / thread 32)
+  uint32_t done = 0;
+  bool failed = false;
+  for (int item = blockIdx.x; item < items[0] + items[1] && !failed; item += gridDim.x, ++done) {
+    const int part = item < items[0] ? 0 : 1;
+    int it = item - (part ? items[0] : 0);
+    const int nt = it % n_tiles; it /= n_tiles;
+    const int mt = it % m_tiles[part], b0 = pb_lo[part] + it / m_tiles[part] * run;
+    const int nblk = min(run, pb_hi[part] - b0);
+    bool ok = true;
+    if (tid == 0) {
+      const unsigned char* xi = p.img.x[part];
+      for (int b = 0; b < nblk && ok; ++b, ++put) {
+        const uint32_t stage = put & 1u, dst = tiles_addr + stage * kDwStageBytes, bar = full_bar0 + 8 * stage;
+        if (put >= 2) ok = mbar_wait(empty_bar0 + 8 * stage, ((put >> 1) - 1) & 1u, s_abort, p.wait_limit, p.st);
+        if (!ok) break;
+        const size_t pb = b0 + b;
+        // (the last tile of either operand may have one unit only: the other half keeps what it holds, its outputs are dropped)
+        const int ma = min(2, xu[part] - 2 * mt), mb = min(2, ju - 2 * nt);
+        mbar_arrive_expect_tx(bar, (uint32_t)(ma + mb) * kUnitBytes);
+        bulk_load(dst, xi + (pb * xu[part] + 2 * mt) * kUnitBytes, (uint32_t)ma * kUnitBytes, bar);
+        bulk_load(dst + kSpOperandBytes, p.img.dz + (pb * ju + 2 * nt) * kUnitBytes, (uint32_t)mb * kUnitBytes, bar);
+      }
+    } else if (tid == 32) {
+      for (int b = 0; b < nblk && ok; ++b, ++got) {
+        const uint32_t stage = got & 1u, src = tiles_addr + stage * kDwStageBytes;
+        ok = mbar_wait(full_bar0 + 8 * stage, (got >> 1) & 1u, s_abort, p.wait_limit, p.st);
+        if (!ok) break;
+        tc_fence_after();
+        split_mmas_mn(tmem_base, src, src + kSpOperandBytes, idesc, b == 0);
+        umma_commit(empty_bar0 + 8 * stage);
+        if (b == nblk - 1) umma_commit(acc_bar);
+      }
+    }
+    __syncwarp();
+    ok = mbar_wait(acc_bar, done & 1u, s_abort, p.wait_limit, p.st) && ok;
+    if (__syncthreads_or(!ok)) { failed = true; break; }
+    tc_fence_after();
+    // tensor memory -> row segments: a warp reads 32 rows x 32 columns, lane = row; adds go out along the row through a transposition
+    {
+      const int quad = warp & 3, quarter = warp >> 2;
+      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(quarter * 32);
+      uint32_t v[32];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
+      tmem_ld_wait();
+      tc_fence_before();
+      constexpr int kRowStride = kDwTile + 4;
+      float* stage_out = reinterpret_cast<float*>(tiles);   // both stages are idle: every block asked for has been multiplied
+      float* dst = stage_out + (size_t)(quad * 32 + lane) * kRowStride + quarter * 32;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
+                                                              __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+      __syncthreads();
+      const int rows = part ? 2 * H : E, m0 = mt * kDwTile, j0 = nt * kDwTile, cols_valid = min(kDwTile, J - j0);
+      for (int r = warp; r < min(kDwTile, rows + 1 - m0); r += kDwThreads / 32) {
+        const int f = m0 + r;
+        float* out = f == rows ? p.db + j0 : p.dW + (size_t)((part ? E : 0) + f) * J + j0;
+#pragma unroll
+        for (int i = 0; i < kDwTile / 32; ++i) {
+          const int c = lane + 32 * i;
+          if (c < cols_valid) atomicAdd(out + c, stage_out[(size_t)r * kRowStride + c]);
+        }
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the next item's bulk copies overwrite the staging rows
+    __syncthreads();
+  }
+}
+
 __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
   extern __shared__ unsigned char dw_dyn[];
   __shared__ int s_node[kDwMaxRun * kDwBlock], s_ia[kDwMaxRun * kDwBlock], s_ib[kDwMaxRun * kDwBlock];
-  __shared__ __align__(8) uint64_t s_bars[kDwStages + 2];
+  __shared__ __align__(8) uint64_t s_bars[2 * kDwStages + 2];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
   if (ld_volatile(&p.st->status) != 0) return;   // the passes before failed: nothing here may be trusted
@@ -206,6 +265,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
                  drain_bar = smem_u32(&s_bars[kDwStages + 1]);
   if (tid == 0) {
     for (int s = 0; s < kDwStages; ++s) mbar_init(stage_bar0 + 8 * s, 1);
+    for (int s = 0; s < kDwStages; ++s) mbar_init(smem_u32(&s_bars[kDwStages + 2 + s]), 1);
     mbar_init(acc_bar, 1);
     mbar_init(drain_bar, 1);
     s_abort = 0;
@@ -218,6 +278,21 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
   const uint32_t tmem_base = s_tmem;
   const int H = p.H, E = p.E, J = 5 * H;
   const int n_leaves = p.st->n_levels > 0 ? min(p.n, max(0, p.level_offset[1])) : 0;
+  if (p.img.dz != nullptr && !(p.tree_parts > 0 && trees_pay(p.n, p.st->n_roots, H, p.tree_parts))) {
+    dw_from_images(p, n_leaves, tiles, stage_bar0, smem_u32(&s_bars[kDwStages + 2]), acc_bar, tmem_base, &s_abort);
+    tc_fence_before();
+    __syncthreads();
+    if (s_abort) {                         // what was asked for gets a bounded time to land, the MMAs a bounded time to retire
+      if (tid == 32) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
+      if (tid == 0) for (int s = 0; s < kDwStages; ++s) mbar_drain(stage_bar0 + 8 * s, 0);
+      __syncthreads();
+    }
+    if (warp == 0) {
+      tc_fence_after();
+      tmem_dealloc(tmem_base, kDwTile);
+    }
+    return;
+  }
   const bool leaf_dinput = p.dEmb_rows != nullptr;
   const int run = dw_run(p.n, n_leaves, H, E, leaf_dinput, (int)gridDim.x);   // the host does not know the number of leaves
   const DwShape sh = dw_shape(p.n, n_leaves, H, E, run, leaf_dinput);
@@ -264,45 +339,45 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
       }
     }
     __syncthreads();
+    // The fp32 values of block b + 1 are on their way into registers while block b is split, stored and multiplied.
+    auto block_col = [&](int b) {        // part 2: first gate column of the block
+      const int kb = kb0 + b;
+      return (kb < sh.skip_first ? kb : kb + sh.skip_count) * kDwBlock;
+    };
+    float va[2][8], vb[2][8], na[2][8], nb[2][8];
+    auto load_block = [&](int b) {
+      if (part == 0) tile_load<0>(p, m0, s_node, s_ia, s_ib, b, na);
+      else if (part == 1) tile_load<1>(p, m0, s_node, s_ia, s_ib, b, na);
+      else rows_load([&](int r) { return p.dz + (size_t)s_node[r] * J; }, block_col(b), J, na);
+      if (part < 2) tile_load<2>(p, j0, s_node, s_ia, s_ib, b, nb);
+      else rows_load([&](int r) { return p.W + (size_t)min(j0 + r, E - 1) * J; }, block_col(b), J, nb);
+    };
+    load_block(0);
     for (int b = 0; b < nblk; ++b, ++built) {
       const uint32_t stage = built & 1u, use = built >> 1;
       unsigned char* st_tiles = tiles + stage * kDwStageBytes;
       const int valid_nodes = min(kDwBlock, pos_end - pos0 - b * kDwBlock);
-      int kcol = 0;                      // part 2: first gate column of the block
-      if (part == 2) {
-        const int kb = kb0 + b;
-        kcol = (kb < sh.skip_first ? kb : kb + sh.skip_count) * kDwBlock;
-      }
-      float va[4][8], vb[4][8];
-      if (part == 0) tile_load<0>(p, m0, s_node, s_ia, s_ib, b, va);
-      else if (part == 1) tile_load<1>(p, m0, s_node, s_ia, s_ib, b, va);
-      else rows_load([&](int r) { return p.dz + (size_t)s_node[r] * J; }, kcol, J, va);
-      if (part < 2) tile_load<2>(p, j0, s_node, s_ia, s_ib, b, vb);
-      else rows_load([&](int r) { return p.W + (size_t)min(j0 + r, E - 1) * J; }, kcol, J, vb);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) { va[i][e] = na[i][e]; vb[i][e] = nb[i][e]; }
+      if (b + 1 < nblk) load_block(b + 1);
       bool ok = true;
       if (use >= 1)   // the MMAs that read this stage two blocks ago must have retired before it is overwritten
         ok = mbar_wait(stage_bar0 + 8 * stage, (use - 1) & 1u, &s_abort, p.wait_limit, p.st);
       if (__syncthreads_or(!ok)) { failed = true; break; }
       if (part == 0) tile_store<0>(p, st_tiles, m0, valid_nodes, va);
       else if (part == 1) tile_store<1>(p, st_tiles, m0, valid_nodes, va);
-      else rows_store(st_tiles, rows_here, kcol, J, va);
-      if (part < 2) tile_store<2>(p, st_tiles + kDwPieces * kDwTileBytes, j0, valid_nodes, vb);
-      else rows_store(st_tiles + kDwPieces * kDwTileBytes, min(kDwTile, E - j0), kcol, J, vb);
+      else rows_store(st_tiles, rows_here, block_col(b), J, va);
+      if (part < 2) tile_store<2>(p, st_tiles + kSpOperandBytes, j0, valid_nodes, vb);
+      else rows_store(st_tiles + kSpOperandBytes, min(kDwTile, E - j0), block_col(b), J, vb);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the tensor core
       tc_fence_before();
       __syncthreads();
       if (tid == 0) {
         tc_fence_after();
-        const uint32_t a_addr = tiles_addr + stage * kDwStageBytes, b_addr = a_addr + kDwPieces * kDwTileBytes;
-        // (piece of the input operand, piece of dz), the small products first: (0,2) (2,0) (1,1) (0,1) (1,0) (0,0)
-#pragma unroll
-        for (int k = 0; k < kDwBlock / 16; ++k)     // UMMA K = 16 bf16 = 32 bytes = 2 descriptor units
-#pragma unroll
-          for (int q = 0; q < 6; ++q) {
-            const int pa = (0x010120 >> (4 * q)) & 0xF, pb = (0x001102 >> (4 * q)) & 0xF;
-            umma_bf16(tmem_base, umma_desc(a_addr + pa * kDwTileBytes) + 2 * k,
-                      umma_desc(b_addr + pb * kDwTileBytes) + 2 * k, idesc, !(b == 0 && k == 0 && q == 0));
-          }
+        const uint32_t a_addr = tiles_addr + stage * kDwStageBytes;
+        split_mmas(tmem_base, a_addr, a_addr + kSpOperandBytes, idesc, b == 0);
         umma_commit(stage_bar0 + 8 * stage);
         if (b == nblk - 1) umma_commit(acc_bar);
       }
@@ -316,17 +391,17 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
     constexpr int kRowStride = kDwTile + 4;                 // floats; 16-byte stores of a warp's 32 rows spread over all banks
     float* stage_out = reinterpret_cast<float*>(tiles);     // every MMA that read the operand stages has retired
     {
-      const int quad = warp & 3, half = warp >> 2;          // a warp reads the tensor-memory lanes of quadrant (warp id mod 4)
+      const int quad = warp & 3, quarter = warp >> 2;       // a warp reads the tensor-memory lanes of quadrant (warp id mod 4)
       const int r = quad * 32 + lane;
-      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 64);
-      uint32_t v[64];
+      const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(quarter * 32);
+      uint32_t v[32];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
+      for (int i = 0; i < 8; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
       tmem_ld_wait();
       tc_fence_before();
-      float* dst = stage_out + (size_t)r * kRowStride + half * 64;
+      float* dst = stage_out + (size_t)r * kRowStride + quarter * 32;
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
+      for (int i = 0; i < 8; ++i)
         *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
                                                               __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
     }
@@ -365,6 +440,35 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
 
 }  // namespace
 
+// W -> its split image (see wsp_bytes)
+__global__ void k_split_w(int H, int E, const float* W, unsigned char* out) {
+  const int J = 5 * H, kbs = wsp_kblocks(H), tx = wsp_tiles_x(E), tiles = tx + wsp_tiles_h(H);
+  const int total = tiles * kbs * kSpTile * 8;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
+    const int c = q & 7, r = (q >> 3) % kSpTile, kb = (q >> 3) / kSpTile % kbs, t = (q >> 3) / kSpTile / kbs;
+    const int row = t < tx ? t * kSpTile + r : (t - tx) * kSpTile + r;
+    const bool in = row < (t < tx ? E : 2 * H);
+    float x[8];
+    for (int e = 0; e < 8; ++e) {
+      const int j = kb * kSpBlock + 8 * c + e;
+      x[e] = in && j < J ? W[(size_t)(t < tx ? row : E + row) * J + j] : 0.f;
+    }
+    split_store8(out + (size_t)(t * kbs + kb) * kSpOperandBytes, r, c, x);
+  }
+}
+size_t wide_backward_bytes(const treelstm* ctx) {
+  if (ctx->cell != 0 || ctx->H > 512 || ctx->E > 1024) return 0;
+  return round_up_sz(wsp_bytes(ctx->H, ctx->E), 1024);
+}
+int pack_wide_backward(treelstm* ctx, cudaStream_t stream) {
+  if (!ctx->wsp) return TREELSTM_OK;
+  k_split_w<<<592, 256, 0, stream>>>(ctx->H, ctx->E, ctx->W, ctx->wsp);
+  TL_CUDA(ctx, cudaGetLastError());
+  return TREELSTM_OK;
+}
+// bytes of the images of n positions x `features` features (one unit row more than needed: tiles of 128 positions)
+size_t image_bytes(int n, int features) { return (size_t)((n + 63) / 64 + 1) * img_units(features) * kUnitBytes; }
+
 int init_dweight_tc_attributes(treelstm* ctx) {
   TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_dweight_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmemBytes));
   return TREELSTM_OK;
@@ -374,8 +478,10 @@ int init_dweight_tc_attributes(treelstm* ctx) {
 // stream before; dz holds the gate gradients of every node.
 int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t* level_offset, const int32_t* token,
                       const int32_t* left, const int32_t* right, const float* h, const float* dz, float* dW, float* db,
-                      const int* tok_slot, float* dEmb_rows, DevStatus* st, cudaStream_t stream) {
+                      const int* tok_slot, float* dEmb_rows, DevStatus* st, const BwdImages* img, int tree_parts, cudaStream_t stream) {
   DwParams p;
+  if (img) p.img = *img;
+  p.tree_parts = tree_parts;
   p.n = n; p.n_leaves = 0; p.H = ctx->H; p.E = ctx->E; p.vocab = ctx->vocab; p.run = 0;
   p.order = order; p.level_offset = level_offset; p.token = token; p.left = left; p.right = right;
   p.emb = ctx->emb; p.h = h; p.dz = dz; p.W = ctx->W; p.dW = dW; p.db = db; p.st = st;

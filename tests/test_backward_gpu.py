@@ -179,3 +179,30 @@ def test_training_step_at_the_limits_of_the_tree_kernels(H, E, n_trees, hi):
     res = _train_step(model, forest, labels, binding.PERSISTENT)
     assert util.max_abs(res["h"], ref["h"]) < util.TOL["fp32"]
     _compare(res, ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("H,E,shapes", [
+    (40, 30, "balanced"), (72, 127, "bushy"), (150, 64, "bushy"), (33, 128, "leaves"), (128, 63, "exact"), (256, 300, "bushy"), (300, 20, "balanced")])
+def test_training_step_of_wide_forests(H, E, shapes):
+    """forests whose wavefronts go over the whole GPU, their contractions on split bf16 pieces: wavefronts around 64,
+    128 and 256 positions that start inside a block, ragged outputs and gate columns, the boundary between leaves and
+    internal nodes inside a block or on it, narrow wavefronts on top, single leaves, sizes beyond the tree kernels"""
+    rng = np.random.default_rng(900 + H)
+    vocab = 70
+    params = fg.draw_params(rng, H, E, vocab, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    if shapes == "balanced":
+        forest = fg.forest_from_shapes([fg.balanced_shape(512)] * 2 + [None] * 3, rng, vocab)
+    elif shapes == "exact":
+        forest = fg.forest_from_shapes([fg.balanced_shape(1024)], rng, vocab)
+    elif shapes == "leaves":
+        forest = fg.forest_from_shapes([fg.balanced_shape(256)] * 2 + [None] * 600 + [fg.left_chain_shape(150)], rng, vocab)
+    else:
+        forest = fg.forest_from_shapes([fg.random_split_shape(rng, 701), fg.random_split_shape(rng, 390)], rng, vocab)
+    forest, _ = fg.permute_node_ids(forest, rng)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    res = _train_step(model, forest, labels, binding.PERSISTENT)
+    _compare(res, ref, util.TOL["fp32"])
+    _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
