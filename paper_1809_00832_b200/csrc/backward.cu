@@ -186,6 +186,97 @@ __global__ void __launch_bounds__(1024) k_bwd_scan_tokens(BwdParams p) {
 constexpr int kClsWarps = 8;
 constexpr int kClsNodesPerCta = 8;    // one node per warp and group: the chains of dependent loads of a node are long
 
+// Up to 256 hidden units and 8 classes (instantiations for the units per lane): a lane keeps its units' part of dWc in
+// registers over all nodes of its warp.  (One shared-memory add per node, unit and class instead is an add of
+// floats in a compare-and-swap loop: 70 us for 14.6 k nodes, H = 256, 5 classes.)
+// Wider states take at most five classes, which is what the registers of two CTAs per SM hold.
+template <int NJ, int kClsRegC>
+__device__ __forceinline__ void classifier_nodes(const BwdParams& p, int warp_first, int warp_step, float* s_dWc) {
+  const int lane = threadIdx.x & 31, H = p.H, C = p.C;
+  const float inv_n = 1.0f / (float)p.n;
+  float wc[NJ][kClsRegC], acc[NJ][kClsRegC], loss = 0.f, acc_b = 0.f;
+#pragma unroll
+  for (int t = 0; t < NJ; ++t)
+#pragma unroll
+    for (int k = 0; k < kClsRegC; ++k) {
+      const int j = lane + 32 * t;
+      wc[t][k] = j < H && k < C ? __ldg(p.Wc + j * C + k) : 0.f;
+      acc[t][k] = 0.f;
+    }
+  const float my_bias = lane < C ? __ldg(p.bc + lane) : 0.f;
+  float hn[NJ];
+  int y = 0;
+  auto fetch = [&](int node) {           // the next node's states and label, while this one is worked on
+    if (node >= p.n) return;
+    y = p.labels[node];
+#pragma unroll
+    for (int t = 0; t < NJ; ++t) hn[t] = p.h[(size_t)node * H + min(lane + 32 * t, H - 1)];
+  };
+  fetch(warp_first);
+  for (int node = warp_first; node < p.n; node += warp_step) {
+    float h[NJ];
+    const int label = y;
+#pragma unroll
+    for (int t = 0; t < NJ; ++t) h[t] = lane + 32 * t < H ? hn[t] : 0.f;
+    fetch(node + warp_step);
+    float part[kClsRegC];
+#pragma unroll
+    for (int k = 0; k < kClsRegC; ++k) {
+      part[k] = 0.f;
+      if (k < C) {
+#pragma unroll
+        for (int t = 0; t < NJ; ++t) part[k] = fmaf(h[t], wc[t][k], part[k]);
+      }
+    }
+    float logit = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kClsRegC; ++k)
+      if (k < C) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) part[k] += __shfl_xor_sync(kFull, part[k], d);
+        if (lane == k) logit = part[k] + my_bias;
+      }
+    float m = logit;
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, d));   // the classes sit in the first eight lanes
+    m = __shfl_sync(kFull, m, 0);
+    const float e = lane < C ? expf(logit - m) : 0.f;
+    float sum = e;
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) sum += __shfl_xor_sync(kFull, sum, d);
+    sum = __shfl_sync(kFull, sum, 0);
+    const bool y_ok = label >= 0 && label < C;
+    if (!y_ok && lane == 0) report(p.st, TREELSTM_ERR_LABEL_OUT_OF_RANGE);
+    const float logit_y = __shfl_sync(kFull, logit, y_ok ? label : 0);
+    if (y_ok) loss += m + logf(sum) - logit_y;
+    const float dlogit = lane < C ? (e / sum - (lane == label ? 1.f : 0.f)) * inv_n : 0.f;
+    acc_b += dlogit;
+    float dh[NJ];
+#pragma unroll
+    for (int t = 0; t < NJ; ++t) dh[t] = 0.f;
+#pragma unroll
+    for (int k = 0; k < kClsRegC; ++k)
+      if (k < C) {
+        const float dk = __shfl_sync(kFull, dlogit, k);
+#pragma unroll
+        for (int t = 0; t < NJ; ++t) {
+          dh[t] = fmaf(wc[t][k], dk, dh[t]);
+          acc[t][k] = fmaf(h[t], dk, acc[t][k]);
+        }
+      }
+#pragma unroll
+    for (int t = 0; t < NJ; ++t)
+      if (lane + 32 * t < H) p.dh[(size_t)node * H + lane + 32 * t] = dh[t];
+  }
+#pragma unroll
+  for (int t = 0; t < NJ; ++t)
+#pragma unroll
+    for (int k = 0; k < kClsRegC; ++k)
+      if (lane + 32 * t < H && k < C) atomicAdd(&s_dWc[(lane + 32 * t) * C + k], acc[t][k]);
+  if (lane < C) atomicAdd(&s_dWc[H * C + lane], acc_b);
+  if (lane == 0 && loss != 0.f) atomicAdd(p.loss, loss * inv_n);
+}
+
 // The CTA takes the node groups vb_first, vb_first + vb_step, ...; s_dWc [H][C] + [C] collects its partial sums.
 __device__ void classifier_groups(const BwdParams& p, int vb_first, int vb_step, float* s_dWc) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -198,6 +289,12 @@ __device__ void classifier_groups(const BwdParams& p, int vb_first, int vb_step,
   TL_STAMP(ctrace, kTraceLevels - 1, 11);
   const float inv_n = 1.0f / (float)p.n;
   const int n_groups = (p.n + kClsNodesPerCta - 1) / kClsNodesPerCta;
+  if (C <= (H <= 64 ? 8 : 5) && H <= 256) {
+    const int first = vb_first * kClsWarps + warp, step = vb_step * kClsWarps;
+    if (H <= 64) classifier_nodes<2, 8>(p, first, step, s_dWc);
+    else if (H <= 160) classifier_nodes<5, 5>(p, first, step, s_dWc);
+    else classifier_nodes<8, 5>(p, first, step, s_dWc);
+  } else {
   for (int vb = vb_first; vb < n_groups; vb += vb_step)
   for (int q = warp; q < kClsNodesPerCta; q += kClsWarps) {
     const int node0 = vb * kClsNodesPerCta;
@@ -241,6 +338,7 @@ __device__ void classifier_groups(const BwdParams& p, int vb_first, int vb_step,
       if (j < H) p.dh[(size_t)node * H + j] = dhj;
     }
     TL_STAMP(ctrace, kTraceLevels - 1, 12);   // first warp: a node done
+  }
   }
   __syncthreads();
   TL_STAMP(ctrace, kTraceLevels - 1, 13);     // all warps: nodes done
@@ -925,25 +1023,44 @@ struct WideArgs {
 __device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& img, int row0, int cnt, int leaf, float* s_dz) {
   const int H = p.H, J = 5 * H, ju = img_units(J), tid = threadIdx.x;
   __syncthreads();                                       // the previous rows have left shared memory
-  for (int e = tid; e < cnt * H; e += 256) {
-    const int i = e / H, u = e - i * H;
-    const int node = chk(p.st, p.order[row0 + i], p.n);
-    const int l = leaf ? 0 : chk(p.st, p.pos_left[row0 + i], p.n), r = leaf ? 0 : chk(p.st, p.pos_right[row0 + i], p.n);
-    const float* g = p.gates + (size_t)node * J + u;
-    const float gi = g[0], gl = leaf ? 0.f : g[H], gr = leaf ? 0.f : g[2 * H], go = g[3 * H], gu = g[4 * H];
-    const float cn = p.c[(size_t)node * H + u], dhn = p.dh[(size_t)node * H + u], dci = p.dc[(size_t)node * H + u];
-    const float cl = leaf ? 0.f : p.c[(size_t)l * H + u], cr = leaf ? 0.f : p.c[(size_t)r * H + u];
-    const float tc = tanhf(cn);
-    const float dcn = dci + dhn * go * (1.f - tc * tc);
-    float* z = s_dz + i * J + u;
-    z[0] = dcn * gu * gi * (1.f - gi);
-    z[H] = dcn * cl * gl * (1.f - gl);
-    z[2 * H] = dcn * cr * gr * (1.f - gr);
-    z[3 * H] = dhn * tc * go * (1.f - go);
-    z[4 * H] = dcn * gi * (1.f - gu * gu);
-    if (!leaf) {
-      p.dc[(size_t)l * H + u] = dcn * gl;                // every node has exactly one caller: plain stores
-      p.dc[(size_t)r * H + u] = dcn * gr;
+  // eight rows at a time, a thread's four elements together: index loads, then value loads, then the arithmetic
+  constexpr int kG = 4;
+  for (int e0 = tid; e0 < cnt * H; e0 += 256 * kG) {
+    int node[kG], l[kG], r[kG], u[kG];
+#pragma unroll
+    for (int q = 0; q < kG; ++q) {
+      const int e = min(e0 + 256 * q, cnt * H - 1), i = e / H;
+      u[q] = e - i * H;
+      node[q] = chk(p.st, p.order[row0 + i], p.n);
+      l[q] = leaf ? node[q] : chk(p.st, p.pos_left[row0 + i], p.n);
+      r[q] = leaf ? node[q] : chk(p.st, p.pos_right[row0 + i], p.n);
+    }
+    float gi[kG], gl[kG], gr[kG], go[kG], gu[kG], cn[kG], dhn[kG], dci[kG], cl[kG], cr[kG];
+#pragma unroll
+    for (int q = 0; q < kG; ++q) {
+      const float* g = p.gates + (size_t)node[q] * J + u[q];
+      const size_t at = (size_t)node[q] * H + u[q];
+      gi[q] = g[0]; go[q] = g[3 * H]; gu[q] = g[4 * H];
+      gl[q] = leaf ? 0.f : g[H]; gr[q] = leaf ? 0.f : g[2 * H];
+      cn[q] = p.c[at]; dhn[q] = p.dh[at]; dci[q] = p.dc[at];
+      cl[q] = leaf ? 0.f : p.c[(size_t)l[q] * H + u[q]]; cr[q] = leaf ? 0.f : p.c[(size_t)r[q] * H + u[q]];
+    }
+#pragma unroll
+    for (int q = 0; q < kG; ++q) {
+      const int e = e0 + 256 * q;
+      if (e >= cnt * H) break;
+      const float tc = tanhf(cn[q]);
+      const float dcn = dci[q] + dhn[q] * go[q] * (1.f - tc * tc);
+      float* z = s_dz + e / H * J + u[q];
+      z[0] = dcn * gu[q] * gi[q] * (1.f - gi[q]);
+      z[H] = dcn * cl[q] * gl[q] * (1.f - gl[q]);
+      z[2 * H] = dcn * cr[q] * gr[q] * (1.f - gr[q]);
+      z[3 * H] = dhn[q] * tc * go[q] * (1.f - go[q]);
+      z[4 * H] = dcn * gi[q] * (1.f - gu[q] * gu[q]);
+      if (!leaf) {
+        p.dc[(size_t)l[q] * H + u[q]] = dcn * gl[q];     // every node has exactly one caller: plain stores
+        p.dc[(size_t)r[q] * H + u[q]] = dcn * gr[q];
+      }
     }
   }
   __syncthreads();
@@ -982,6 +1099,9 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
   p.n_leaves = n_levels > 0 ? a.level_offset[1] : 0;
   const int n_leaves = p.n_leaves;
   const size_t gtid = (size_t)blockIdx.x * 256 + tid, gthreads = (size_t)gridDim.x * 256;
+#ifdef TREELSTM_TRACE
+  long long* const trace = gtid == 0 ? p.trace : nullptr;
+#endif
   unsigned int arrivals = 0;
   auto barrier = [&]() {
     arrivals += gridDim.x;
@@ -989,6 +1109,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
   };
   bool ok = true;
   // ---- set-up: dc of the roots, children by position, the inputs' images, zeros behind the last position
+  TL_STAMP(trace, kTraceLevels - 1, 0);
   zero_range(p.dc, (size_t)n * H, gtid, gthreads);
   for (size_t r = (size_t)n_leaves + gtid; r < (size_t)n; r += gthreads) {
     const int node = chk(p.st, p.order[r], p.n);
@@ -996,14 +1117,15 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
     p.pos_right[r] = p.right[node];
   }
   {
+    // a warp per four rows (eight lanes each: one 16-byte piece of a unit per lane and step), a row's units one after the
+    // other: its index chain is resolved once, the loads of two units are in flight together
     const int xu0 = img_units(E + 1), xu1 = img_units(2 * H + 1), pb1 = n_leaves / 64, pbs = (n + 63) / 64;
-    const int units0 = (n_leaves + 63) / 64 * xu0, units1 = n > n_leaves ? (pbs - pb1) * xu1 : 0;
-    const int r = tid >> 2, c0 = (tid & 3) * 2;
-    for (int q = blockIdx.x; q < units0 + units1; q += gridDim.x) {
-      const int part = q >= units0, qq = part ? q - units0 : q, xu = part ? xu1 : xu0;
-      const int pb = (part ? pb1 : 0) + qq / xu, fb = qq % xu, pos = pb * 64 + r, feats = part ? 2 * H : E;
+    const int rows0 = (n_leaves + 63) / 64 * 64, rows1 = n > n_leaves ? (pbs - pb1) * 64 : 0;
+    for (int q = (int)(gtid >> 3); q < rows0 + rows1; q += (int)(gthreads >> 3)) {
+      const int part = q >= rows0, xu = part ? xu1 : xu0, pos = part ? pb1 * 64 + q - rows0 : q, feats = part ? 2 * H : E;
       const bool in = part ? pos >= n_leaves && pos < n : pos < n_leaves;
-      const float *s0 = nullptr, *s1 = nullptr;
+      const int c = tid & 7;
+      const float *s0 = p.h, *s1 = p.h;
       if (in) {
         const int node = chk(p.st, p.order[pos], p.n);
         if (part) {
@@ -1013,15 +1135,26 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
           s0 = p.emb + (size_t)chk(p.st, p.token[node], p.vocab) * E;
         }
       }
+      unsigned char* row = a.img.x[part] + (size_t)(pos >> 6) * xu * kUnitBytes;
+      for (int fb = 0; fb < xu; fb += 2) {
+        float x[2][8];
 #pragma unroll
-      for (int c = c0; c < c0 + 2; ++c) {
-        float x[8];
+        for (int v = 0; v < 2; ++v)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int f = fb * 64 + c * 8 + k, fc = min(f, feats - 1);
-          x[k] = in ? (f < feats ? (part && fc >= H ? s1 : s0)[fc] : (f == feats ? 1.f : 0.f)) : 0.f;
+          for (int k = 0; k < 8; ++k) {
+            const int fc = min((fb + v) * 64 + c * 8 + k, feats - 1);
+            x[v][k] = (part && fc >= H ? s1 : s0)[in ? fc : 0];
+          }
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          if (fb + v >= xu) break;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int f = (fb + v) * 64 + c * 8 + k;
+            x[v][k] = in ? (f < feats ? x[v][k] : (f == feats ? 1.f : 0.f)) : 0.f;
+          }
+          split_store8_unit(row + (size_t)(fb + v) * kUnitBytes, pos & 63, c, x[v]);
         }
-        split_store8_unit(a.img.x[part] + ((size_t)pb * xu + fb) * kUnitBytes, r, c, x);
       }
     }
     const float zero[8] = {};
@@ -1030,7 +1163,9 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
       split_store8_unit(a.img.dz + ((size_t)(pos >> 6) * ju + (ch >> 3)) * kUnitBytes, pos & 63, ch & 7, zero);
     }
   }
+  TL_STAMP(trace, kTraceLevels - 1, 1);   // operand images of this CTA written
   ok = barrier();
+  TL_STAMP(trace, kTraceLevels - 1, 2);
   uint32_t put = 0, got = 0, done = 0;
   bool prepared = false;
   FusedItem pre_item{};
@@ -1040,6 +1175,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
   auto is_fused = [&](int l) { return l > 0 && level_begin(l + 1) - level_begin(l) <= kFusedMaxRows; };
   for (int lvl = n_levels - 1; lvl >= 0 && ok; --lvl) {
     const int begin = level_begin(lvl), end = level_begin(lvl + 1), leaf = lvl == 0 ? 1 : 0;
+    TL_STAMP(trace, lvl, 0);
     if (is_fused(lvl)) {
       const int ntiles = dinput_tiles(end - begin, 2 * H), nsplits = dinput_splits(ntiles, J, splits_for);
       for (int vb = blockIdx.x; vb < ntiles * nsplits; vb += gridDim.x) {
@@ -1058,15 +1194,19 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
           }
         }
       }
+      TL_STAMP(trace, lvl, 3);            // own blocks done
       ok = barrier();
+      TL_STAMP(trace, lvl, 4);
       continue;
     }
     prepared = false;
     for (int r0 = begin + 8 * (int)blockIdx.x; r0 < end; r0 += 8 * (int)gridDim.x)
       wide_gates(p, a.img, r0, min(8, end - r0), leaf, reinterpret_cast<float*>(tiles));
+    TL_STAMP(trace, lvl, 1);              // own gate gradients stored
     asm volatile("fence.proxy.async;" ::: "memory");     // the image is read by bulk copies (and this shared memory written by them)
     if (!(ok = barrier())) break;
     asm volatile("fence.proxy.async;" ::: "memory");
+    TL_STAMP(trace, lvl, 2);
     // dIn: tiles of 128 positions (from a multiple of 64 on) x 128 outputs, the column blocks cut into pieces
     const int base = begin & ~63, K = leaf ? E : 2 * H, tr = (end - base + 127) / 128, to = (K + 127) / 128;
     const int all = wsp_kblocks(H);
@@ -1123,6 +1263,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
       __syncwarp();
       ok = mbar_wait(acc_bar, done & 1u, &s_abort, a.wait_limit, p.st) && ok;
       ++done;
+      TL_STAMP(trace, lvl, 5);            // a tile accumulated
       if (__syncthreads_or(!ok)) { ok = false; break; }
       tc_fence_after();
       constexpr int kRowStride = kSpTile + 4;
@@ -1142,6 +1283,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
                                                                 __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
       }
       __syncthreads();
+      TL_STAMP(trace, lvl, 6);            // and read back
       for (int r = warp; r < kSpTile; r += 8) {
         if (s_da[r] < 0) continue;
 #pragma unroll
@@ -1156,7 +1298,9 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the next bulk copies overwrite the staging rows
       __syncthreads();
     }
+    TL_STAMP(trace, lvl, 3);
     if (ok && lvl > 0) ok = barrier();
+    TL_STAMP(trace, lvl, 4);
   }
   tc_fence_before();
   __syncthreads();
