@@ -496,10 +496,10 @@ __device__ void dinput_block(const BwdParams& p, int row_begin, int row_end, int
 // How many CTAs share the contraction of one dIn tile.  A 64 x 64 tile costs about 4 k cycles per
 // 32-wide chunk of the contraction whatever the number of valid rows, so a wavefront with few tiles
 // spreads the chunks over as many CTAs as there are (about two per SM), down to one chunk each.
-__host__ __device__ inline int dinput_splits(int tiles, int J, int blocks = 296) {
+__host__ __device__ inline int dinput_splits(int tiles, int J) {
   const int chunks_all = (J + BK - 1) / BK;
-  if (tiles >= blocks / 2) return 1;
-  int s = blocks / (tiles > 0 ? tiles : 1);
+  if (tiles >= 148) return 1;
+  int s = 296 / (tiles > 0 ? tiles : 1);
   if (s < 6) s = 6;
   return s < chunks_all ? s : chunks_all;
 }
@@ -589,7 +589,7 @@ __device__ __forceinline__ int gate_of_column(int j, int H) { return (j >= H) + 
 // branch (rows and columns beyond the block are clamped onto valid ones and discarded afterwards), so that
 // they are in flight together: one round trip instead of one per element; then the arithmetic and the stores.
 __device__ __forceinline__ void fused_gate_gradients(const BwdParams& p, const FusedItem& it, DinputSmem& sm, int ib,
-                                                     int buf, int j0, unsigned char* image) {
+                                                     int buf, int j0) {
   const int H = p.H, J = 5 * H, tid = threadIdx.x;
   float dhn[kLd], dci[kLd], go[kLd], cn[kLd], g1[kLd], g2[kLd];
 #pragma unroll
@@ -627,11 +627,7 @@ __device__ __forceinline__ void fused_gate_gradients(const BwdParams& p, const F
         const float gi = g1[q], gu = g2[q];
         dz = g == 0 ? dcn * gu * gi * (1.f - gi) : dcn * gi * (1.f - gu * gu);
       }
-      if (keep) {
-        const int pos = it.row0 + i;
-        if (image) split_store1_unit(image + ((size_t)(pos >> 6) * img_units(J) + (j >> 6)) * kUnitBytes, pos & 63, j & 63, dz);
-        else p.dz[(size_t)node * J + j] = dz;
-      }
+      if (keep) p.dz[(size_t)node * J + j] = dz;
     }
     sm.As[buf][i][e % BK] = dz;
   }
@@ -660,11 +656,9 @@ __device__ __forceinline__ void fused_chunk(const DinputSmem& sm, int buf, int t
 // One block.  fetched: `f` holds the block's index triples and first weight chunk (fused_fetch was called before
 // the grid barrier) and no thread of the CTA still reads the operand buffers.
 // buffers_free() runs once, when the block no longer needs the operand buffers and before its results go out.
-// image: dz goes there, split (k_bwd_wide), instead of to the fp32 rows.
 template <class FreeFn>
 __device__ __forceinline__ void dinput_fused(const BwdParams& p, const FusedItem& it, DinputSmem& sm, int ib, bool fetched,
-                                             FusedFetch& f, long long* trace, int lvl, FreeFn buffers_free,
-                                             unsigned char* image = nullptr) {
+                                             FusedFetch& f, long long* trace, int lvl, FreeFn buffers_free) {
   (void)trace; (void)lvl;
   if (it.c_lo >= it.chunks) { buffers_free(); return; }   // the same for every thread of the CTA
   const int H = p.H, K = 2 * H;
@@ -677,7 +671,7 @@ __device__ __forceinline__ void dinput_fused(const BwdParams& p, const FusedItem
   __syncthreads();
   TL_STAMP(trace, lvl, 8);   // index triples and first weight chunk in shared memory
   float acc[4][4] = {};
-  fused_gate_gradients(p, it, sm, ib, it.c_lo & 1, it.c_lo * BK, image);
+  fused_gate_gradients(p, it, sm, ib, it.c_lo & 1, it.c_lo * BK);
   __syncthreads();
   TL_STAMP(trace, lvl, 5);   // gate gradients of the first chunk formed by all warps
   const int ni = (it.rows + 15) / 16;   // 16-row groups of the tile that hold nodes
@@ -690,7 +684,7 @@ __device__ __forceinline__ void dinput_fused(const BwdParams& p, const FusedItem
     else if (ni == 3) fused_chunk<3>(sm, buf, tx, ty, acc);
     else fused_chunk<4>(sm, buf, tx, ty, acc);
     if (more) {
-      fused_gate_gradients(p, it, sm, ib, buf ^ 1, (cidx + 1) * BK, image);
+      fused_gate_gradients(p, it, sm, ib, buf ^ 1, (cidx + 1) * BK);
     }
     __syncthreads();
   }
@@ -1011,7 +1005,8 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
 // contraction is cut into as many pieces as leave no CTA without a tile.  The leaves' dIn (their rows of dEmb) is one
 // more such wavefront.  Narrow wavefronts form their gate gradients inside an fp32 contraction as in k_bwd_persistent.
 // The images stay for the weight gradient.
-constexpr int kWideSmem = 2 * kSpStageBytes + 1024;
+constexpr int kWideSmem = 2 * kSpStageBytes + 1024, kWideThreads = 512;
+constexpr int kDirectRows = 256, kWideOffCache = 512;
 struct WideArgs {
   const int* level_offset;
   long long wait_limit;
@@ -1019,70 +1014,234 @@ struct WideArgs {
   BwdImages img;
 };
 
-// dz of rows [row0, row0 + cnt) of the ready order (at most eight) -> image; s_dz [8][J]
-__device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& img, int row0, int cnt, int leaf, float* s_dz) {
-  const int H = p.H, J = 5 * H, ju = img_units(J), tid = threadIdx.x;
-  __syncthreads();                                       // the previous rows have left shared memory
-  // eight rows at a time, a thread's four elements together: index loads, then value loads, then the arithmetic
-  constexpr int kG = 4;
-  for (int e0 = tid; e0 < cnt * H; e0 += 256 * kG) {
-    int node[kG], l[kG], r[kG], u[kG];
+// How the dIn of a wavefront is cut: tiles of 128 positions (from `base` on) x 128 outputs, each `span` steps long (kbs
+// blocks of 64 gate columns, padded to a multiple of `per`); a CTA takes `per` steps after the other.
+struct WidePlan {
+  int begin, end, base, leaf, direct, to, kbs, span, per, total, skip_first, skip;
+};
+__device__ __forceinline__ WidePlan wide_plan(int begin, int end, int leaf, int H, int E, int grid) {
+  WidePlan w;
+  w.begin = begin; w.end = end; w.leaf = leaf;
+  w.direct = !leaf && end - begin <= kDirectRows;
+  w.base = w.direct ? begin : begin & ~63;
+  w.to = ((leaf ? E : 2 * H) + 127) / 128;
+  const int tiles = (end - w.base + 127) / 128 * w.to, gp = gate_pitch(H);
+  w.kbs = wsp_kblocks(H);
+  w.skip_first = w.kbs; w.skip = 0;
+  if (leaf) {                                            // a leaf's forget gates are zero: blocks inside them are left out
+    w.skip_first = (gp + 63) / 64;
+    w.skip = max(0, 3 * gp / 64 - w.skip_first);
+    w.kbs -= w.skip;
+  }
+  if (w.direct) w.per = tiles * w.kbs <= grid ? 1 : 2;
+  else if (2 * tiles > grid) w.per = (tiles * w.kbs + grid - 1) / grid;   // equal shares, whatever tile they lie in
+  else w.per = (w.kbs + grid / tiles - 1) / (grid / tiles);
+  w.span = !w.direct && 2 * tiles > grid ? w.kbs : (w.kbs + w.per - 1) / w.per * w.per;
+  w.total = tiles * w.span;
+  return w;
+}
+
+// units u0 .. u0 + 7 of a row of H; what lies behind the row repeats units of it.  kVec: 16-byte loads (H a multiple of 4)
+template <bool kVec>
+__device__ __forceinline__ void load8(const float* row, int u0, int H, float (&x)[8]) {
+  if (kVec) {
+    const float4 a = *reinterpret_cast<const float4*>(row + u0), b = *reinterpret_cast<const float4*>(row + min(u0 + 4, H - 4));
+    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+  } else {
 #pragma unroll
-    for (int q = 0; q < kG; ++q) {
-      const int e = min(e0 + 256 * q, cnt * H - 1), i = e / H;
-      u[q] = e - i * H;
-      node[q] = chk(p.st, p.order[row0 + i], p.n);
-      l[q] = leaf ? node[q] : chk(p.st, p.pos_left[row0 + i], p.n);
-      r[q] = leaf ? node[q] : chk(p.st, p.pos_right[row0 + i], p.n);
+    for (int k = 0; k < 8; ++k) x[k] = row[min(u0 + k, H - 1)];
+  }
+}
+template <bool kVec>
+__device__ __forceinline__ void store_units(float* row, int u0, int H, const float (&x)[8]) {
+  if (kVec) {
+    *reinterpret_cast<float4*>(row + u0) = make_float4(x[0], x[1], x[2], x[3]);
+    if (u0 + 4 < H) *reinterpret_cast<float4*>(row + u0 + 4) = make_float4(x[4], x[5], x[6], x[7]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (u0 + k < H) row[u0 + k] = x[k];
+  }
+}
+__device__ __forceinline__ unsigned char* dz_unit(const BwdImages& img, int pos, int kb, int ju) {
+  return img.dz + ((size_t)(pos >> 6) * ju + kb) * kUnitBytes;
+}
+
+// This CTA's share of a wavefront's gate gradients -> image, dc of the children.  A thread forms the five gates of eight
+// units of one node at a time: all its loads are in flight together and every store is a whole 16-byte piece.
+// (One element per thread through shared memory: 12 k cycles for eight nodes per CTA.)
+template <bool kVec>
+__device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& img, const WidePlan& w) {
+  const int H = p.H, J = 5 * H, gp = gate_pitch(H), octs = gp / 8, ju = img_units(5 * gp), tid = threadIdx.x;
+  const long long all = (long long)(w.end - w.begin) * octs;
+  const int share = (int)((all + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
+  const long long lo = (long long)blockIdx.x * share, hi = min(all, lo + share);
+  const int keep_zero = w.leaf ? w.end & ~63 : 0;        // leaves below: nobody reads the blocks of their forget gates
+  for (long long e = lo + tid; e < hi; e += kWideThreads) {
+    const int i = (int)(e / octs), o = (int)(e - (long long)i * octs), u0 = 8 * o, pos = w.begin + i;
+    const int node = chk(p.st, p.order[pos], p.n);
+    const int l = w.leaf ? node : chk(p.st, p.pos_left[pos], p.n), r = w.leaf ? node : chk(p.st, p.pos_right[pos], p.n);
+    const float* g = p.gates + (size_t)node * J;
+    float gi[8], go[8], gu[8], c[8], dh[8], dc[8], z[8];
+    load8<kVec>(p.c + (size_t)node * H, u0, H, c);
+    load8<kVec>(p.dh + (size_t)node * H, u0, H, dh);
+    load8<kVec>(p.dc + (size_t)node * H, u0, H, dc);
+    load8<kVec>(g + 3 * H, u0, H, go);
+    load8<kVec>(g, u0, H, gi);
+    load8<kVec>(g + 4 * H, u0, H, gu);
+    auto put = [&](int gate) {
+      const int j = gate * gp + u0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) z[k] = u0 + k < H ? z[k] : 0.f;
+      split_store8_unit(dz_unit(img, pos, j >> 6, ju), pos & 63, (j >> 3) & 7, z);
+    };
+    float gf[2][8], cc[2][8];
+    if (!w.leaf) {
+      load8<kVec>(g + H, u0, H, gf[0]);
+      load8<kVec>(g + 2 * H, u0, H, gf[1]);
+      load8<kVec>(p.c + (size_t)l * H, u0, H, cc[0]);
+      load8<kVec>(p.c + (size_t)r * H, u0, H, cc[1]);
     }
-    float gi[kG], gl[kG], gr[kG], go[kG], gu[kG], cn[kG], dhn[kG], dci[kG], cl[kG], cr[kG];
 #pragma unroll
-    for (int q = 0; q < kG; ++q) {
-      const float* g = p.gates + (size_t)node[q] * J + u[q];
-      const size_t at = (size_t)node[q] * H + u[q];
-      gi[q] = g[0]; go[q] = g[3 * H]; gu[q] = g[4 * H];
-      gl[q] = leaf ? 0.f : g[H]; gr[q] = leaf ? 0.f : g[2 * H];
-      cn[q] = p.c[at]; dhn[q] = p.dh[at]; dci[q] = p.dc[at];
-      cl[q] = leaf ? 0.f : p.c[(size_t)l[q] * H + u[q]]; cr[q] = leaf ? 0.f : p.c[(size_t)r[q] * H + u[q]];
+    for (int k = 0; k < 8; ++k) {
+      const float tc = tanhf(c[k]);
+      z[k] = dh[k] * tc * go[k] * (1.f - go[k]);
+      dc[k] += dh[k] * go[k] * (1.f - tc * tc);
     }
+    put(3);
 #pragma unroll
-    for (int q = 0; q < kG; ++q) {
-      const int e = e0 + 256 * q;
-      if (e >= cnt * H) break;
-      const float tc = tanhf(cn[q]);
-      const float dcn = dci[q] + dhn[q] * go[q] * (1.f - tc * tc);
-      float* z = s_dz + e / H * J + u[q];
-      z[0] = dcn * gu[q] * gi[q] * (1.f - gi[q]);
-      z[H] = dcn * cl[q] * gl[q] * (1.f - gl[q]);
-      z[2 * H] = dcn * cr[q] * gr[q] * (1.f - gr[q]);
-      z[3 * H] = dhn[q] * tc * go[q] * (1.f - go[q]);
-      z[4 * H] = dcn * gi[q] * (1.f - gu[q] * gu[q]);
-      if (!leaf) {
-        p.dc[(size_t)l[q] * H + u[q]] = dcn * gl[q];     // every node has exactly one caller: plain stores
-        p.dc[(size_t)r[q] * H + u[q]] = dcn * gr[q];
+    for (int k = 0; k < 8; ++k) z[k] = dc[k] * gu[k] * gi[k] * (1.f - gi[k]);
+    put(0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) z[k] = dc[k] * gi[k] * (1.f - gu[k] * gu[k]);
+    put(4);
+    if (!w.leaf) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          z[k] = dc[k] * cc[q][k] * gf[q][k] * (1.f - gf[q][k]);
+          gf[q][k] *= dc[k];
+        }
+        put(1 + q);
+        store_units<kVec>(p.dc + (size_t)(q ? r : l) * H, u0, H, gf[q]);   // every node has exactly one caller: plain stores
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) z[k] = 0.f;
+      for (int q = 1; q < 3; ++q) {
+        const int kb = (q * gp + u0) >> 6;
+        if (pos >= keep_zero || !forget_tile(kb >> 1, gp)) put(q);
       }
     }
-  }
-  __syncthreads();
-  for (int e = tid; e < cnt * ju * 8; e += 256) {
-    const int i = e / (ju * 8), ch = e - i * ju * 8, pos = row0 + i;
-    float x[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) x[k] = ch * 8 + k < J ? s_dz[i * J + min(ch * 8 + k, J - 1)] : 0.f;
-    split_store8_unit(img.dz + ((size_t)(pos >> 6) * ju + (ch >> 3)) * kUnitBytes, pos & 63, ch & 7, x);
+    for (int k = 0; k < 8; ++k) z[k] = 0.f;
+    for (int x = 5 * octs + o; x < 8 * ju; x += octs)    // columns behind the last gate
+      split_store8_unit(dz_unit(img, pos, x >> 3, ju), pos & 63, x & 7, z);
   }
 }
 
-__global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
+// Block kb of a narrow wavefront's gate gradients, formed where the tensor core reads it: rows 0 .. rows - 1 of the
+// tile are the nodes in s_node.  keep: this CTA also stores the block in the image and hands dc to the children.
+template <bool kVec>
+__device__ __forceinline__ void direct_block(const BwdParams& p, const BwdImages& img, unsigned char* tile, int kb, int pos0, int rows,
+                                             bool keep, const int* s_node, const int* s_left, const int* s_right) {
+  const int H = p.H, J = 5 * H, gp = gate_pitch(H), ju = img_units(5 * gp), c = threadIdx.x & 7, j = kb * 64 + 8 * c;
+  const int gate = j / gp, u0 = j - gate * gp;
+  const bool forget = gate == 1 || gate == 2;
+  for (int i = threadIdx.x >> 3; i < rows; i += kWideThreads / 8) {
+    float z[8];
+    if (gate < 5) {
+      const int node = s_node[i], child = gate == 2 ? s_right[i] : s_left[i];
+      const float* g = p.gates + (size_t)node * J;
+      float dh[8], dc[8], go[8], cn[8], g1[8], g2[8];
+      load8<kVec>(p.dh + (size_t)node * H, u0, H, dh);
+      load8<kVec>(p.dc + (size_t)node * H, u0, H, dc);
+      load8<kVec>(g + 3 * H, u0, H, go);
+      load8<kVec>(p.c + (size_t)node * H, u0, H, cn);
+      load8<kVec>(g + (forget ? gate * H : 0), u0, H, g1);                         // f_l / f_r, else i
+      load8<kVec>(forget ? p.c + (size_t)child * H : g + 4 * H, u0, H, g2);       // the child's cell state, else u
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float tc = tanhf(cn[k]), dcn = dc[k] + dh[k] * go[k] * (1.f - tc * tc);
+        const float a = gate == 3 ? dh[k] * tc : dcn * (gate == 4 ? g1[k] : g2[k]);
+        const float b = gate == 3 ? go[k] : (gate == 4 ? 1.f : g1[k]);
+        const float d = gate == 3 ? go[k] : (gate == 4 ? g2[k] * g2[k] : g1[k]);
+        z[k] = u0 + k < H ? a * b * (1.f - d) : 0.f;
+        g1[k] *= dcn;
+      }
+      if (keep && forget) store_units<kVec>(p.dc + (size_t)child * H, u0, H, g1);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) z[k] = 0.f;
+    }
+    split_store8(tile, i, c, z);
+    if (keep) split_store8_unit(dz_unit(img, pos0 + i, kb, ju), (pos0 + i) & 63, c, z);
+  }
+}
+
+// 64 rows of the inputs' images (leaves first: embedding row and a one; then internal nodes: [h_l | h_r] and a one);
+// eight lanes per row, four units in flight
+template <bool kVec>
+__device__ __forceinline__ void input_rows(const BwdParams& p, const BwdImages& img, int chunk, int rows0) {
+  const int H = p.H, E = p.E, n = p.n, c = threadIdx.x & 7;
+  const int q = chunk * 64 + (threadIdx.x >> 3), part = q >= rows0;
+  const int pos = part ? p.n_leaves / 64 * 64 + q - rows0 : q, feats = part ? 2 * H : E, units = img_units(feats + 1);
+  const bool in = part ? pos >= p.n_leaves && pos < n : pos < p.n_leaves;
+  const float *s0 = p.h, *s1 = p.h;
+  if (in) {
+    if (part) {
+      s0 = p.h + (size_t)chk(p.st, p.pos_left[pos], p.n) * H;
+      s1 = p.h + (size_t)chk(p.st, p.pos_right[pos], p.n) * H - H;
+    } else {
+      s0 = p.emb + (size_t)chk(p.st, p.token[chk(p.st, p.order[pos], p.n)], p.vocab) * E;
+    }
+  }
+  unsigned char* row = img.x[part] + (size_t)(pos >> 6) * units * kUnitBytes;
+  constexpr int kF = 4;
+  for (int fb = 0; fb < units; fb += kF) {
+    float x[kF][8];
+#pragma unroll
+    for (int v = 0; v < kF; ++v) {
+      const int f = (fb + v) * 64 + c * 8;
+      if (kVec) {
+#pragma unroll
+        for (int q4 = 0; q4 < 2; ++q4) {
+          const int fc = min(f + 4 * q4, feats - 4);
+          const float4 t = *reinterpret_cast<const float4*>(in ? (part && fc >= H ? s1 : s0) + fc : s0);
+          x[v][4 * q4] = t.x; x[v][4 * q4 + 1] = t.y; x[v][4 * q4 + 2] = t.z; x[v][4 * q4 + 3] = t.w;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int fc = min(f + k, feats - 1);
+          x[v][k] = *(in ? (part && fc >= H ? s1 : s0) + fc : s0);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < kF; ++v) {
+      if (fb + v >= units) break;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int f = (fb + v) * 64 + c * 8 + k;
+        x[v][k] = in ? (f < feats ? x[v][k] : (f == feats ? 1.f : 0.f)) : 0.f;
+      }
+      split_store8_unit(row + (size_t)(fb + v) * kUnitBytes, pos & 63, c, x[v]);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideArgs a) {
   extern __shared__ unsigned char wide_dyn[];
   __shared__ __align__(8) uint64_t s_bars[6];            // full, empty (two stages each), accumulator, drain
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort, s_flag;
-  __shared__ int s_da[kSpTile], s_db[kSpTile];
+  __shared__ int s_node[kSpTile], s_da[kSpTile], s_db[kSpTile];
+  __shared__ int s_off[kWideOffCache];
   if (ld_volatile(&p.st->status) != 0 || (a.tree_parts > 0 && trees_pay(p.n, p.st->n_roots, p.H, a.tree_parts))) return;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grid = (int)gridDim.x;
   unsigned char* const tiles = wide_dyn + ((1024u - (smem_u32(wide_dyn) & 1023u)) & 1023u);
-  DinputSmem& di = *reinterpret_cast<DinputSmem*>(tiles);
   const uint32_t tiles_addr = smem_u32(tiles), full0 = smem_u32(&s_bars[0]), empty0 = smem_u32(&s_bars[2]),
                  acc_bar = smem_u32(&s_bars[4]), drain_bar = smem_u32(&s_bars[5]);
   if (tid == 0) {
@@ -1090,223 +1249,207 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  const int n_levels = p.st->n_levels, n = p.n, H = p.H, E = p.E, gp = gate_pitch(H), ju = img_units(5 * gp);
+  for (int l = tid; l < kWideOffCache && l <= n_levels; l += kWideThreads) s_off[l] = a.level_offset[l];
   if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kSpTile);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = s_tmem;
-  const int n_levels = p.st->n_levels, n = p.n, H = p.H, E = p.E, J = 5 * H, ju = img_units(J);
-  p.n_leaves = n_levels > 0 ? a.level_offset[1] : 0;
-  const int n_leaves = p.n_leaves;
-  const size_t gtid = (size_t)blockIdx.x * 256 + tid, gthreads = (size_t)gridDim.x * 256;
+  auto level_begin = [&](int l) { return l < kWideOffCache ? s_off[l] : a.level_offset[l]; };
+  p.n_leaves = n_levels > 0 ? level_begin(1) : 0;
+  const int n_leaves = p.n_leaves, wsp_kb = wsp_kblocks(H);
+  // 16-byte accesses to rows of H (and E): whether every row starts on a 16-byte boundary
+  const bool vec_h = H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.h) | reinterpret_cast<uintptr_t>(p.c)) & 15) == 0;
+  const bool vec_e = E % 4 == 0 && (reinterpret_cast<uintptr_t>(p.dEmb_rows) & 15) == 0;
+  const bool vec_x = vec_h && E % 4 == 0 && (reinterpret_cast<uintptr_t>(p.emb) & 15) == 0;
 #ifdef TREELSTM_TRACE
-  long long* const trace = gtid == 0 ? p.trace : nullptr;
+  long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;
 #endif
+  TL_STAMP(trace, kTraceLevels - 1, 0);
   unsigned int arrivals = 0;
   auto barrier = [&]() {
     arrivals += gridDim.x;
     return grid_barrier(p.st, arrivals, a.wait_limit, &s_flag, true, &p.st->barrier_levels);
   };
-  bool ok = true;
-  // ---- set-up: dc of the roots, children by position, the inputs' images, zeros behind the last position
-  TL_STAMP(trace, kTraceLevels - 1, 0);
-  zero_range(p.dc, (size_t)n * H, gtid, gthreads);
-  for (size_t r = (size_t)n_leaves + gtid; r < (size_t)n; r += gthreads) {
-    const int node = chk(p.st, p.order[r], p.n);
-    p.pos_left[r] = p.left[node];
-    p.pos_right[r] = p.right[node];
-  }
-  {
-    // a warp per four rows (eight lanes each: one 16-byte piece of a unit per lane and step), a row's units one after the
-    // other: its index chain is resolved once, the loads of two units are in flight together
-    const int xu0 = img_units(E + 1), xu1 = img_units(2 * H + 1), pb1 = n_leaves / 64, pbs = (n + 63) / 64;
-    const int rows0 = (n_leaves + 63) / 64 * 64, rows1 = n > n_leaves ? (pbs - pb1) * 64 : 0;
-    for (int q = (int)(gtid >> 3); q < rows0 + rows1; q += (int)(gthreads >> 3)) {
-      const int part = q >= rows0, xu = part ? xu1 : xu0, pos = part ? pb1 * 64 + q - rows0 : q, feats = part ? 2 * H : E;
-      const bool in = part ? pos >= n_leaves && pos < n : pos < n_leaves;
-      const int c = tid & 7;
-      const float *s0 = p.h, *s1 = p.h;
-      if (in) {
-        const int node = chk(p.st, p.order[pos], p.n);
-        if (part) {
-          s0 = p.h + (size_t)chk(p.st, p.left[node], p.n) * H;
-          s1 = p.h + (size_t)chk(p.st, p.right[node], p.n) * H - H;
-        } else {
-          s0 = p.emb + (size_t)chk(p.st, p.token[node], p.vocab) * E;
-        }
-      }
-      unsigned char* row = a.img.x[part] + (size_t)(pos >> 6) * xu * kUnitBytes;
-      for (int fb = 0; fb < xu; fb += 2) {
-        float x[2][8];
-#pragma unroll
-        for (int v = 0; v < 2; ++v)
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int fc = min((fb + v) * 64 + c * 8 + k, feats - 1);
-            x[v][k] = (part && fc >= H ? s1 : s0)[in ? fc : 0];
-          }
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          if (fb + v >= xu) break;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int f = (fb + v) * 64 + c * 8 + k;
-            x[v][k] = in ? (f < feats ? x[v][k] : (f == feats ? 1.f : 0.f)) : 0.f;
-          }
-          split_store8_unit(row + (size_t)(fb + v) * kUnitBytes, pos & 63, c, x[v]);
-        }
-      }
-    }
+  // The inputs' images are for the kernel behind this one: CTAs without a share of a wavefront write them.
+  const int rows0 = (n_leaves + 63) / 64 * 64, chunks = rows0 / 64 + (n > n_leaves ? (n + 63) / 64 - n_leaves / 64 : 0);
+  int chunks_done = 0;
+  auto input_chunk = [&](int chunk) {
+    if (vec_x) input_rows<true>(p, a.img, chunk, rows0);
+    else input_rows<false>(p, a.img, chunk, rows0);
+  };
+  {                                                      // zeros behind the last position
     const float zero[8] = {};
-    for (size_t q = gtid; q < (size_t)(pbs * 64 - n) * ju * 8; q += gthreads) {
-      const int pos = n + (int)(q / (ju * 8)), ch = (int)(q % (ju * 8));
-      split_store8_unit(a.img.dz + ((size_t)(pos >> 6) * ju + (ch >> 3)) * kUnitBytes, pos & 63, ch & 7, zero);
-    }
+    for (int q = (int)blockIdx.x * kWideThreads + tid; q < ((n + 63) / 64 * 64 - n) * ju * 8; q += grid * kWideThreads)
+      split_store8_unit(dz_unit(a.img, n, q % (ju * 8) >> 3, ju), (n + q / (ju * 8)) & 63, q & 7, zero);
   }
-  TL_STAMP(trace, kTraceLevels - 1, 1);   // operand images of this CTA written
-  ok = barrier();
-  TL_STAMP(trace, kTraceLevels - 1, 2);
-  uint32_t put = 0, got = 0, done = 0;
-  bool prepared = false;
-  FusedItem pre_item{};
-  FusedFetch pre_fetch;
-  const int splits_for = 2 * (int)gridDim.x;             // pieces of a narrow contraction over all CTAs
-  auto level_begin = [&](int l) { return a.level_offset[l]; };
-  auto is_fused = [&](int l) { return l > 0 && level_begin(l + 1) - level_begin(l) <= kFusedMaxRows; };
-  for (int lvl = n_levels - 1; lvl >= 0 && ok; --lvl) {
-    const int begin = level_begin(lvl), end = level_begin(lvl + 1), leaf = lvl == 0 ? 1 : 0;
-    TL_STAMP(trace, lvl, 0);
-    if (is_fused(lvl)) {
-      const int ntiles = dinput_tiles(end - begin, 2 * H), nsplits = dinput_splits(ntiles, J, splits_for);
-      for (int vb = blockIdx.x; vb < ntiles * nsplits; vb += gridDim.x) {
-        const bool ready = prepared && vb == (int)blockIdx.x;
-        const FusedItem item = ready ? pre_item : fused_item(p, begin, end, vb % ntiles, vb / ntiles, nsplits);
-        dinput_fused(p, item, di, lvl & 1, ready, pre_fetch, nullptr, lvl, []() {}, a.img.dz);
+  bool ok = true, fetched = false;
+  uint32_t blk = 0, asked = 0, done = 0;                 // blocks multiplied; asked for (thread 0); tiles
+  auto read_tables = [&](const WidePlan& w, int pos0) {  // the nodes of a tile and where its rows go
+    if (tid >= kSpTile) return;
+    const int pos = pos0 + tid;
+    int node = 0, da = -1, db = 0;
+    if (pos >= w.begin && pos < w.end) {
+      if (w.leaf) {
+        da = chk(p.st, p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[pos], p.n)], p.vocab)], p.n_leaves);
+      } else {
+        if (w.direct) node = chk(p.st, p.order[pos], p.n);
+        da = chk(p.st, p.pos_left[pos], p.n);
+        db = chk(p.st, p.pos_right[pos], p.n);
       }
-      prepared = false;
-      if (lvl > 1 && is_fused(lvl - 1)) {                // the next wavefront's first block, fetched while the barrier is pending
-        const int b = level_begin(lvl - 1), e = level_begin(lvl), nt = dinput_tiles(e - b, 2 * H), ns = dinput_splits(nt, J, splits_for);
-        if ((int)blockIdx.x < nt * ns) {
-          pre_item = fused_item(p, b, e, blockIdx.x % nt, blockIdx.x / nt, ns);
-          if (pre_item.c_lo < pre_item.chunks) {
-            fused_fetch(p, pre_item, pre_item.c_lo * BK, pre_fetch);
-            prepared = true;
+    }
+    s_node[tid] = node; s_da[tid] = da; s_db[tid] = db;
+  };
+  // thread 0: blocks k0 .. k0 + nk - 1 of a tile -> the ring
+  auto ask = [&](const WidePlan& w, int pos0, int ot, int k0, int nk) {
+    const unsigned char* wt = a.img.w + (size_t)((w.leaf ? 0 : wsp_tiles_x(E)) + ot) * wsp_kb * kSpOperandBytes;
+    for (int k = 0; k < nk; ++k) {
+      const uint32_t stage = asked & 1u, dst = tiles_addr + stage * kSpStageBytes, bar = full0 + 8 * stage;
+      if (asked >= 2 && !mbar_wait(empty0 + 8 * stage, ((asked >> 1) - 1) & 1u, &s_abort, a.wait_limit, p.st)) return false;
+      ++asked;
+      const int kk = k0 + k, kb = kk < w.skip_first ? kk : kk + w.skip;
+      mbar_arrive_expect_tx(bar, w.direct ? kSpOperandBytes : kSpStageBytes);
+      if (!w.direct) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int q = 0; q < kSpPieces; ++q)
+            bulk_load(dst + q * kSpTileBytes + h * kUnitPieceBytes, dz_unit(a.img, pos0 + 64 * h, kb, ju) + q * kUnitPieceBytes,
+                      kUnitPieceBytes, bar);
+      }
+      bulk_load(dst + kSpOperandBytes, wt + (size_t)kb * kSpOperandBytes, kSpOperandBytes, bar);
+    }
+    return true;
+  };
+  WidePlan w;
+  if (n_levels > 0) w = wide_plan(level_begin(n_levels - 1), level_begin(n_levels), n_levels == 1, H, E, grid);
+  for (int lvl = n_levels - 1; lvl >= 0 && ok; --lvl) {
+    TL_STAMP(trace, lvl, 0);
+    if (!w.direct) {
+      if (vec_h) wide_gates<true>(p, a.img, w);
+      else wide_gates<false>(p, a.img, w);
+      TL_STAMP(trace, lvl, 1);              // own gate gradients stored
+      asm volatile("fence.proxy.async;" ::: "memory");   // the image is read by bulk copies
+      if (!(ok = barrier())) break;
+      asm volatile("fence.proxy.async;" ::: "memory");
+      TL_STAMP(trace, lvl, 2);
+    }
+    for (int lo = blockIdx.x * w.per; lo < w.total && ok; lo += grid * w.per) {
+      for (int at = lo; at < min(lo + w.per, w.total) && ok;) {
+        const int tile = at / w.span, k0 = at - tile * w.span, len = min(min(lo + w.per, w.total) - at, w.span - k0);
+        const int nk = min(len, w.kbs - k0), ot = tile % w.to, pos0 = w.base + tile / w.to * kSpTile;
+        at += len;
+        if (nk <= 0) continue;
+        if (!fetched) read_tables(w, pos0);
+        if (tid == 0 && !fetched) ok = ask(w, pos0, ot, k0, nk);
+        if (w.direct) {
+          if (!fetched) __syncthreads();
+          for (int k = 0; k < nk; ++k) {
+            unsigned char* dst = tiles + ((blk + k) & 1u) * kSpStageBytes;
+            if (vec_h) direct_block<true>(p, a.img, dst, k0 + k, pos0, min(kSpTile, w.end - pos0), ot == 0, s_node, s_da, s_db);
+            else direct_block<false>(p, a.img, dst, k0 + k, pos0, min(kSpTile, w.end - pos0), ot == 0, s_node, s_da, s_db);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads these rows
+          __syncthreads();
+          TL_STAMP(trace, lvl, 7);          // a tile's gate gradients formed
+        }
+        fetched = false;
+        if (tid == 32) {
+          for (int k = 0; k < nk && ok; ++k) {
+            const uint32_t b = blk + k, stage = b & 1u, src = tiles_addr + stage * kSpStageBytes;
+            ok = mbar_wait(full0 + 8 * stage, (b >> 1) & 1u, &s_abort, a.wait_limit, p.st);
+            if (!ok) break;
+            tc_fence_after();
+            split_mmas(tmem_base, src, src + kSpOperandBytes, umma_idesc(kSpTile), k == 0);
+            umma_commit(empty0 + 8 * stage);
+            if (k == nk - 1) umma_commit(acc_bar);
           }
         }
+        __syncwarp();
+        ok = mbar_wait(acc_bar, done & 1u, &s_abort, a.wait_limit, p.st) && ok;
+        ++done;
+        blk += nk;
+        TL_STAMP(trace, lvl, 5);            // a tile accumulated
+        if (__syncthreads_or(!ok)) { ok = false; break; }
+        tc_fence_after();
+        constexpr int kRowStride = kSpTile + 4;
+        float* stage_out = reinterpret_cast<float*>(tiles);
+        {
+          const int quad = warp & 3, quarter = warp >> 2;
+          const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(quarter * 32);
+          uint32_t v[32];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
+          tmem_ld_wait();
+          tc_fence_before();
+          float* dst = stage_out + (size_t)(quad * 32 + lane) * kRowStride + quarter * 32;
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
+                                                                  __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+        }
+        __syncthreads();
+        TL_STAMP(trace, lvl, 6);            // and read back
+        const int K = w.leaf ? E : 2 * H;
+        auto out_of = [&](int r, int k) {
+          return w.leaf ? p.dEmb_rows + (size_t)s_da[r] * E + k
+                        : p.dh + (size_t)(k < H ? s_da[r] : s_db[r]) * H + (k < H ? k : k - H);
+        };
+        if (w.leaf ? vec_e : vec_h) {
+          const int k = ot * 128 + 4 * lane;
+          if (k < K)
+            for (int r = warp; r < kSpTile; r += kWideThreads / 32)
+              if (s_da[r] >= 0)
+                atomicAdd(reinterpret_cast<float4*>(out_of(r, k)), *reinterpret_cast<const float4*>(stage_out + (size_t)r * kRowStride + 4 * lane));
+        } else {
+          for (int r = warp; r < kSpTile; r += kWideThreads / 32) {
+            if (s_da[r] < 0) continue;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int c = lane + 32 * i, k = ot * 128 + c;
+              if (k < K) atomicAdd(out_of(r, k), stage_out[(size_t)r * kRowStride + c]);
+            }
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the next bulk copies overwrite the staging rows
+        __syncthreads();
       }
-      TL_STAMP(trace, lvl, 3);            // own blocks done
-      ok = barrier();
-      TL_STAMP(trace, lvl, 4);
-      continue;
     }
-    prepared = false;
-    for (int r0 = begin + 8 * (int)blockIdx.x; r0 < end; r0 += 8 * (int)gridDim.x)
-      wide_gates(p, a.img, r0, min(8, end - r0), leaf, reinterpret_cast<float*>(tiles));
-    TL_STAMP(trace, lvl, 1);              // own gate gradients stored
-    asm volatile("fence.proxy.async;" ::: "memory");     // the image is read by bulk copies (and this shared memory written by them)
-    if (!(ok = barrier())) break;
-    asm volatile("fence.proxy.async;" ::: "memory");
-    TL_STAMP(trace, lvl, 2);
-    // dIn: tiles of 128 positions (from a multiple of 64 on) x 128 outputs, the column blocks cut into pieces
-    const int base = begin & ~63, K = leaf ? E : 2 * H, tr = (end - base + 127) / 128, to = (K + 127) / 128;
-    const int all = wsp_kblocks(H);
-    int skip_first = all, skip = 0;                      // a leaf's forget gates are zero: blocks inside [H, 3H) are left out
-    if (leaf) {
-      skip_first = (H + 63) / 64;
-      const int skip_end = 3 * H / 64;
-      skip = skip_end > skip_first ? skip_end - skip_first : 0;
+    if (!ok) break;
+    const int busy = (w.total + w.per - 1) / w.per;
+    if (busy < grid) {
+      if ((int)blockIdx.x >= busy && chunks_done + (int)blockIdx.x - busy < chunks) input_chunk(chunks_done + blockIdx.x - busy);
+      chunks_done += grid - busy;
     }
-    const int kbs = all - skip;
-    int pieces = (int)gridDim.x / (tr * to);
-    pieces = pieces < 1 ? 1 : (pieces > kbs / 2 ? (kbs / 2 < 1 ? 1 : kbs / 2) : pieces);
-    const int per = (kbs + pieces - 1) / pieces;
-    for (int item = blockIdx.x; item < tr * to * pieces && ok; item += gridDim.x) {
-      const int ot = item % to, rt = (item / to) % tr, k0 = item / (to * tr) * per, nk = min(per, kbs - k0);
-      if (nk <= 0) continue;
-      const int pos0 = base + rt * 128;
-      if (tid < kSpTile) {                               // where the rows go
-        const int pos = pos0 + tid;
-        int da = -1, db = 0;
-        if (pos >= begin && pos < end) {
-          if (leaf) da = chk(p.st, p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[pos], p.n)], p.vocab)], p.n_leaves);
-          else { da = chk(p.st, p.pos_left[pos], p.n); db = chk(p.st, p.pos_right[pos], p.n); }
-        }
-        s_da[tid] = da; s_db[tid] = db;
-      }
-      const unsigned char* wt = a.img.w + (size_t)((leaf ? 0 : wsp_tiles_x(E)) + ot) * all * kSpOperandBytes;
-      if (tid == 0) {
-        for (int k = 0; k < nk && ok; ++k, ++put) {
-          const uint32_t stage = put & 1u, dst = tiles_addr + stage * kSpStageBytes, bar = full0 + 8 * stage;
-          if (put >= 2) ok = mbar_wait(empty0 + 8 * stage, ((put >> 1) - 1) & 1u, &s_abort, a.wait_limit, p.st);
-          if (!ok) break;
-          const int kk = k0 + k, kb = kk < skip_first ? kk : kk + skip;
-          mbar_arrive_expect_tx(bar, kSpStageBytes);
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int q = 0; q < kSpPieces; ++q)
-              bulk_load(dst + q * kSpTileBytes + h * kUnitPieceBytes,
-                        a.img.dz + ((size_t)((pos0 >> 6) + h) * ju + kb) * kUnitBytes + q * kUnitPieceBytes, kUnitPieceBytes, bar);
-          bulk_load(dst + kSpOperandBytes, wt + (size_t)kb * kSpOperandBytes, kSpOperandBytes, bar);
-        }
-      } else if (tid == 32) {
-        for (int k = 0; k < nk && ok; ++k, ++got) {
-          const uint32_t stage = got & 1u, src = tiles_addr + stage * kSpStageBytes;
-          ok = mbar_wait(full0 + 8 * stage, (got >> 1) & 1u, &s_abort, a.wait_limit, p.st);
-          if (!ok) break;
-          tc_fence_after();
-          split_mmas(tmem_base, src, src + kSpOperandBytes, umma_idesc(kSpTile), k == 0);
-          umma_commit(empty0 + 8 * stage);
-          if (k == nk - 1) umma_commit(acc_bar);
+    if (lvl == 0) break;
+    w = wide_plan(level_begin(lvl - 1), level_begin(lvl), lvl == 1, H, E, grid);
+    if (w.direct) {                                      // what does not depend on the wavefront above, while the barrier is pending
+      const int lo = blockIdx.x * w.per;
+      if (lo < w.total) {
+        const int tile = lo / w.span, k0 = lo - tile * w.span, nk = min(w.per, w.kbs - k0), pos0 = w.base + tile / w.to * kSpTile;
+        if (nk > 0) {
+          read_tables(w, pos0);
+          if (tid == 0) ask(w, pos0, tile % w.to, k0, nk);
+          fetched = true;
         }
       }
-      __syncwarp();
-      ok = mbar_wait(acc_bar, done & 1u, &s_abort, a.wait_limit, p.st) && ok;
-      ++done;
-      TL_STAMP(trace, lvl, 5);            // a tile accumulated
-      if (__syncthreads_or(!ok)) { ok = false; break; }
-      tc_fence_after();
-      constexpr int kRowStride = kSpTile + 4;
-      float* stage_out = reinterpret_cast<float*>(tiles);
-      {
-        const int quad = warp & 3, half = warp >> 2;
-        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 64);
-        uint32_t v[64];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
-        tmem_ld_wait();
-        tc_fence_before();
-        float* dst = stage_out + (size_t)(quad * 32 + lane) * kRowStride + half * 64;
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
-                                                                __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
-      }
-      __syncthreads();
-      TL_STAMP(trace, lvl, 6);            // and read back
-      for (int r = warp; r < kSpTile; r += 8) {
-        if (s_da[r] < 0) continue;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int c = lane + 32 * i, k = ot * 128 + c;
-          if (k >= K) continue;
-          float* out = leaf ? p.dEmb_rows + (size_t)s_da[r] * E + k
-                            : p.dh + (size_t)(k < H ? s_da[r] : s_db[r]) * H + (k < H ? k : k - H);
-          atomicAdd(out, stage_out[(size_t)r * kRowStride + c]);
-        }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the next bulk copies overwrite the staging rows
-      __syncthreads();
     }
     TL_STAMP(trace, lvl, 3);
-    if (ok && lvl > 0) ok = barrier();
+    ok = barrier();
     TL_STAMP(trace, lvl, 4);
   }
+  if (ok)
+    for (int chunk = chunks_done + (int)blockIdx.x; chunk < chunks; chunk += grid) input_chunk(chunk);
+  TL_STAMP(trace, kTraceLevels - 1, 1);
   tc_fence_before();
-  __syncthreads();
-  if (s_abort) {                                         // what was asked for gets a bounded time to land, the MMAs to retire
+  if (__syncthreads_or(!ok)) {                           // what was asked for gets a bounded time to land, the MMAs to retire
     if (tid == 32) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
-    if (tid == 0) for (int s = 0; s < 2; ++s) mbar_drain(full0 + 8 * s, 0);
+    if (tid == 0)
+      for (uint32_t s = 0; s < 2; ++s) {
+        const uint32_t times = (asked + 1 - s) / 2;      // how often stage s was filled
+        if (times > 0) mbar_drain(full0 + 8 * s, (times - 1) & 1u);
+      }
     __syncthreads();
   }
   if (warp == 0) {
@@ -1319,7 +1462,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_wide(BwdParams p, WideArgs a) {
 // marked | tokens counted beside the classifier | tokens placed.  The level table stays on the device.
 struct GradSizes { size_t dW, db, dV; };   // floats
 __global__ void __launch_bounds__(256, 2)
-k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, long long wait_limit) {
+k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, long long wait_limit, int wide, int tree_parts) {
   extern __shared__ float s_cls[];
   __shared__ __align__(16) unsigned int s_mask[1024];
   __shared__ int s_flag;
@@ -1342,6 +1485,14 @@ k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, lo
   zero_range(p.dbc, (size_t)C, gtid, gthreads);
   zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
   zero_range(p.dEmb_rows, (size_t)p.n_leaves * p.E, gtid, gthreads);
+  if (wide && !(tree_parts > 0 && trees_pay(p.n, p.st->n_roots, H, tree_parts))) {   // k_bwd_wide follows: dc of the roots, children by position
+    zero_range(p.dc, (size_t)p.n * H, gtid, gthreads);
+    for (size_t r = (size_t)p.n_leaves + gtid; r < (size_t)p.n; r += gthreads) {
+      const int node = chk(p.st, p.order[r], p.n);
+      p.pos_left[r] = p.left[node];
+      p.pos_right[r] = p.right[node];
+    }
+  }
   if (!barrier()) return;
   for (size_t r = gtid; r < (size_t)p.n_leaves; r += gthreads)
     p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[r], p.n)], p.vocab)] = 1;
@@ -1358,7 +1509,7 @@ k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, lo
   }
 }
 
-int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, cudaStream_t stream) {
+int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, int wide, int tree_parts, cudaStream_t stream) {
   const size_t smem = sizeof(float) * ((size_t)p.H * p.C + p.C);
   if (smem > 160 * 1024) return TREELSTM_ERR_UNSUPPORTED;
   if (smem > 40 * 1024)
@@ -1371,7 +1522,7 @@ int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, cu
   TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, 2 * sizeof(unsigned int), stream));   // and barrier_levels behind it
   const int* lvl_off = ctx->last.level_offset;
   long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
-  void* args[] = {&p, &dV, &sizes, &lvl_off, &wait_limit};
+  void* args[] = {&p, &dV, &sizes, &lvl_off, &wait_limit, &wide, &tree_parts};
   TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_begin, dim3(grid), dim3(256), args, smem, stream));
   ctx->launches += 1;
   return TREELSTM_OK;
@@ -1401,7 +1552,7 @@ static int launch_bwd_wide(treelstm* ctx, BwdParams& p, const BwdImages& img, in
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
   WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, tree_parts, img};
   void* args[] = {&p, &a};
-  TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_wide, dim3(grid), dim3(256), args, kWideSmem, stream));
+  TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_wide, dim3(grid), dim3(kWideThreads), args, kWideSmem, stream));
   ctx->launches += 1;
   return TREELSTM_OK;
 }
@@ -1455,9 +1606,9 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
     }
     const bool trees = trees_take(ctx, n), wide = L.lay.img_dz != L.lay.img_end;
     if (ctx->opt.dw_tensor_cores && (trees || wide)) {
-      int rc = launch_bwd_begin(ctx, p, nullptr, {(E + 2 * (size_t)H) * J, J, 0}, stream);
-      if (rc == TREELSTM_OK && trees) rc = launch_backward_trees(ctx, stream);
       const int tree_parts = trees ? trees_parts(ctx, n, true, true) : 0;
+      int rc = launch_bwd_begin(ctx, p, nullptr, {(E + 2 * (size_t)H) * J, J, 0}, wide, tree_parts, stream);
+      if (rc == TREELSTM_OK && trees) rc = launch_backward_trees(ctx, stream);
       BwdImages img;
       if (rc == TREELSTM_OK && wide) {
         img.dz = reinterpret_cast<unsigned char*>(base + L.lay.img_dz);
@@ -1643,7 +1794,7 @@ int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float
     p.touched_ids = touched_ids; p.n_touched = n_touched;
     p.st = reinterpret_cast<DevStatus*>(base + L.lay.status);
     const size_t H = ctx->H;
-    int rc = launch_bwd_begin(ctx, p, dV, {2 * H * H, H, ctx->cell == TREELSTM_CELL_RNTN ? 4 * H * H * H : 0}, stream);
+    int rc = launch_bwd_begin(ctx, p, dV, {2 * H * H, H, ctx->cell == TREELSTM_CELL_RNTN ? 4 * H * H * H : 0}, 0, 0, stream);
     if (rc == TREELSTM_OK) rc = launch_backward_trees(ctx, stream);
     return rc != TREELSTM_OK ? rc : launch_rec_grads(ctx, dW, db, dV, dEmb_rows, p.tok_slot, stream);
   }

@@ -281,6 +281,8 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
                     int32_t* n_touched, cudaStream_t stream);
 
 struct BwdImages;   // split_tc.cuh
+// Columns of the images of dz and W: each gate's units padded to whole groups of eight, so that a group has one gate.
+__host__ __device__ inline int gate_pitch(int H) { return (H + 7) / 8 * 8; }
 // dweight_tc.cu: dW += In^T dZ, db += sum dZ, dEmb_rows += dz_leaves W_x^T on the tensor cores (three bf16 pieces per fp32 value)
 int init_dweight_tc_attributes(treelstm* ctx);
 size_t wide_backward_bytes(const treelstm* ctx);         // split image of W (0: not kept)

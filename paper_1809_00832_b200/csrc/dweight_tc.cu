@@ -169,14 +169,16 @@ __device__ void dw_from_images(const DwParams& p, int n_leaves, unsigned char* t
   volatile int* s_abort = s_abort_;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = p.H, E = p.E, J = 5 * H;
-  const int ju = img_units(J), xu[2] = {img_units(E + 1), img_units(2 * H + 1)};
-  const int n_tiles = (J + kDwTile - 1) / kDwTile;
+  const int gp = gate_pitch(H), ju = img_units(5 * gp), xu[2] = {img_units(E + 1), img_units(2 * H + 1)};
+  // column tiles; the leaves' forget gates are zero: tiles inside them [skip_lo, skip_lo + skip) are left out
+  const int skip_lo = (gp + kDwTile - 1) / kDwTile, skip = max(0, 3 * gp / kDwTile - skip_lo);
+  const int all_tiles = (5 * gp + kDwTile - 1) / kDwTile, n_tiles[2] = {all_tiles - skip, all_tiles};
   const int m_tiles[2] = {(E + 1 + kDwTile - 1) / kDwTile, (2 * H + 1 + kDwTile - 1) / kDwTile};
   const int pb_lo[2] = {0, n_leaves / 64}, pb_hi[2] = {(n_leaves + 63) / 64, p.n > n_leaves ? (p.n + 63) / 64 : n_leaves / 64};
   // runs of blocks as long as leave every CTA about two items (each ends in an atomic add per output)
   int run = 1, items[2];
   for (;; run *= 2) {
-    for (int q = 0; q < 2; ++q) items[q] = m_tiles[q] * n_tiles * ((pb_hi[q] - pb_lo[q] + run - 1) / run);
+    for (int q = 0; q < 2; ++q) items[q] = m_tiles[q] * n_tiles[q] * ((pb_hi[q] - pb_lo[q] + run - 1) / run);
     if (items[0] + items[1] <= 2 * (int)gridDim.x || run >= 256) break;
   }
   const uint32_t tiles_addr = smem_u32(tiles), idesc = umma_idesc_mn(kDwTile);
@@ -186,7 +188,8 @@ __device__ void dw_from_images(const DwParams& p, int n_leaves, unsigned char* t
   for (int item = blockIdx.x; item < items[0] + items[1] && !failed; item += gridDim.x, ++done) {
     const int part = item < items[0] ? 0 : 1;
     int it = item - (part ? items[0] : 0);
-    const int nt = it % n_tiles; it /= n_tiles;
+    int nt = it % n_tiles[part]; it /= n_tiles[part];
+    if (!part && nt >= skip_lo) nt += skip;
     const int mt = it % m_tiles[part], b0 = pb_lo[part] + it / m_tiles[part] * run;
     const int nblk = min(run, pb_hi[part] - b0);
     bool ok = true;
@@ -235,14 +238,27 @@ __device__ void dw_from_images(const DwParams& p, int n_leaves, unsigned char* t
         *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
                                                               __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
       __syncthreads();
-      const int rows = part ? 2 * H : E, m0 = mt * kDwTile, j0 = nt * kDwTile, cols_valid = min(kDwTile, J - j0);
-      for (int r = warp; r < min(kDwTile, rows + 1 - m0); r += kDwThreads / 32) {
-        const int f = m0 + r;
-        float* out = f == rows ? p.db + j0 : p.dW + (size_t)((part ? E : 0) + f) * J + j0;
+      const int rows = part ? 2 * H : E, m0 = mt * kDwTile;
+      auto column = [&](int c) {                              // of dW; none behind a gate's last unit
+        const int gate = (nt * kDwTile + c) / gp, u = nt * kDwTile + c - gate * gp;
+        return gate < 5 && u < H ? gate * H + u : -1;
+      };
+      auto row_of = [&](int f) { return f == rows ? p.db : p.dW + (size_t)((part ? E : 0) + f) * J; };
+      const int r_end = min(kDwTile, rows + 1 - m0);
+      if (H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.dW) | reinterpret_cast<uintptr_t>(p.db)) & 15) == 0) {
+        const int j = column(4 * lane);
+        if (j >= 0)
+          for (int r = warp; r < r_end; r += kDwThreads / 32)
+            atomicAdd(reinterpret_cast<float4*>(row_of(m0 + r) + j), *reinterpret_cast<const float4*>(stage_out + (size_t)r * kRowStride + 4 * lane));
+      } else {
+        int j[kDwTile / 32];
 #pragma unroll
-        for (int i = 0; i < kDwTile / 32; ++i) {
-          const int c = lane + 32 * i;
-          if (c < cols_valid) atomicAdd(out + c, stage_out[(size_t)r * kRowStride + c]);
+        for (int i = 0; i < kDwTile / 32; ++i) j[i] = column(lane + 32 * i);
+        for (int r = warp; r < r_end; r += kDwThreads / 32) {
+          float* out = row_of(m0 + r);
+#pragma unroll
+          for (int i = 0; i < kDwTile / 32; ++i)
+            if (j[i] >= 0) atomicAdd(out + j[i], stage_out[(size_t)r * kRowStride + lane + 32 * i]);
         }
       }
     }
@@ -442,7 +458,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
 
 // W -> its split image (see wsp_bytes)
 __global__ void k_split_w(int H, int E, const float* W, unsigned char* out) {
-  const int J = 5 * H, kbs = wsp_kblocks(H), tx = wsp_tiles_x(E), tiles = tx + wsp_tiles_h(H);
+  const int J = 5 * H, gp = gate_pitch(H), kbs = wsp_kblocks(H), tx = wsp_tiles_x(E), tiles = tx + wsp_tiles_h(H);
   const int total = tiles * kbs * kSpTile * 8;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
     const int c = q & 7, r = (q >> 3) % kSpTile, kb = (q >> 3) / kSpTile % kbs, t = (q >> 3) / kSpTile / kbs;
@@ -450,8 +466,8 @@ __global__ void k_split_w(int H, int E, const float* W, unsigned char* out) {
     const bool in = row < (t < tx ? E : 2 * H);
     float x[8];
     for (int e = 0; e < 8; ++e) {
-      const int j = kb * kSpBlock + 8 * c + e;
-      x[e] = in && j < J ? W[(size_t)(t < tx ? row : E + row) * J + j] : 0.f;
+      const int j = kb * kSpBlock + 8 * c, gate = j / gp, u = j - gate * gp + e;
+      x[e] = in && gate < 5 && u < H ? W[(size_t)(t < tx ? row : E + row) * J + gate * H + u] : 0.f;
     }
     split_store8(out + (size_t)(t * kbs + kb) * kSpOperandBytes, r, c, x);
   }

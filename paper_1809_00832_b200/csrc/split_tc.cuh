@@ -56,9 +56,12 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// whether the 128 columns of tile t are a leaf's forget gates, all of them (zero: not computed with)
+__host__ __device__ inline bool forget_tile(int t, int gp) { return t * 128 >= gp && (t + 1) * 128 <= 3 * gp; }
+
 // W split once, in the layout of the tiles: rows of W in tiles of 128 (the input rows [0, E) first, then the 2H state
 // rows), columns in blocks of 64; block (tile, kb) is kSpOperandBytes at ((tile * kblocks) + kb).
-__host__ __device__ inline int wsp_kblocks(int H) { return (5 * H + kSpBlock - 1) / kSpBlock; }
+__host__ __device__ inline int wsp_kblocks(int H) { return (5 * gate_pitch(H) + kSpBlock - 1) / kSpBlock; }
 __host__ __device__ inline int wsp_tiles_x(int E) { return (E + kSpTile - 1) / kSpTile; }
 __host__ __device__ inline int wsp_tiles_h(int H) { return (2 * H + kSpTile - 1) / kSpTile; }
 __host__ __device__ inline size_t wsp_bytes(int H, int E) {
@@ -82,14 +85,6 @@ __device__ __forceinline__ void split_store8_unit(unsigned char* unit, int r, in
   *reinterpret_cast<uint4*>(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
   *reinterpret_cast<uint4*>(dst + kUnitPieceBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
   *reinterpret_cast<uint4*>(dst + 2 * kUnitPieceBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
-}
-__device__ __forceinline__ void split_store1_unit(unsigned char* unit, int r, int col, float x) {
-  uint32_t w0, w1, w2;
-  split3_pair(x, 0.f, w0, w1, w2);
-  unsigned char* dst = unit + swz_piece(r, col >> 3) + 2 * (col & 7);
-  *reinterpret_cast<unsigned short*>(dst) = (unsigned short)w0;
-  *reinterpret_cast<unsigned short*>(dst + kUnitPieceBytes) = (unsigned short)w1;
-  *reinterpret_cast<unsigned short*>(dst + 2 * kUnitPieceBytes) = (unsigned short)w2;
 }
 // MN-major operand of two units side by side (128 of the outer dimension): rows of 128 bytes run along it, groups of
 // eight contraction indices 1024 bytes apart, the second unit kUnitBytes further
