@@ -54,7 +54,7 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
   const float* crow = p.cin + (size_t)t.row * 2 * H;   // [c_l | c_r] of the node at this position
   const bool full_slice = vec && (nt + 1) * G * 8 <= H;   // no padded unit among the tile's columns
   const bool staged = !leaf && full_slice;
-  const bool staged_out = full_slice && p.gates == nullptr && t.allow_staged_out;
+  const bool staged_out = full_slice && t.allow_staged_out;
   const int half = t.half;
   const uint32_t my_c = t.cstage_addr + ((uint32_t)r << t.crow_shift);
   unsigned char* mine = t.cstage_ptr + ((size_t)r << t.crow_shift);
@@ -173,15 +173,15 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
           count_write(p.chk_counts, node, count);
           st_row4(p.h + (size_t)node * H + u0, vec, count, hv);
           st_row4(p.c + (size_t)node * H + u0, vec, count, cv);
-          if (p.gates) {
-            float* gp = p.gates + (size_t)node * 5 * H + u0;
-            st_row4(gp, vec, count, gi);
-            st_row4(gp + H, vec, count, gfl);
-            st_row4(gp + 2 * H, vec, count, gfr);
-            st_row4(gp + 3 * H, vec, count, go);
-            st_row4(gp + 4 * H, vec, count, gu);
-          }
         }
+      }
+      if (p.gates && count > 0) {
+        float* gp = p.gates + (size_t)node * 5 * H + u0;
+        st_row4(gp, vec, count, gi);
+        st_row4(gp + H, vec, count, gfl);
+        st_row4(gp + 2 * H, vec, count, gfr);
+        st_row4(gp + 3 * H, vec, count, go);
+        st_row4(gp + 4 * H, vec, count, gu);
       }
     }
   }
