@@ -257,7 +257,7 @@ __global__ void k_prepare_operands(TcParams p) {
 // only_level >= 0: process that wavefront only (one launch per level; operands prepared before).
 // only_level < 0: prepare the operands, then all wavefronts, separated by the bounded grid barrier (cooperative
 // launch).
-template <bool kLeavesFirst>
+template <bool kLeavesFirst, bool kGates>
 __global__ void __launch_bounds__(kThreads, 1)
 k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
   // kLeavesFirst = false: the instantiation for launches that never take the leaves ahead of the schedule (one
@@ -632,7 +632,7 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
         }
         EpiTile et;
         et.leaf = leaf; et.G = G; et.gcols = gcols; et.ncols = ncols; et.nt = nt;
-        et.row = row; et.node = node; et.slot = slot; et.valid = valid;
+        et.row0 = row0; et.row_end = row_end; et.row = row; et.node = node; et.slot = slot; et.valid = valid;
         et.allow_staged_out = rt == BM;   // a tile of 32 or 64 rows writes so little that it stores straight from registers
         et.r = r; et.e = e; et.quad = quad;
         et.cstage_addr = cstage_addr; et.cstage_ptr = cstage_w; et.crow_shift = 8; et.half = 8;
@@ -645,7 +645,7 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
         // the CTA's first tile of the wavefront stamps slots 1-3, its second one slots 8-10
         if (trace != nullptr && lvl < kTraceLevels && t < 2 * (int)gridDim.x) et.stamp = trace + lvl * kTraceSlots + (t < (int)gridDim.x ? 1 : 8);
 #endif
-        epilogue_tile(p, et, epi_phase, alive, s_abort, [&]() { if (nx_have) nx_slot = valid2 && !ahead ? chk_slot(p.st, p.slot[nx_node], p.n) : -1; });
+        epilogue_tile<kGates>(p, et, epi_phase, alive, s_abort, [&]() { if (nx_have) nx_slot = valid2 && !ahead ? chk_slot(p.st, p.slot[nx_node], p.n) : -1; });
         ++acc_iter;
       }
     }
@@ -862,11 +862,16 @@ int ensure_operand_tmaps(treelstm* ctx, void* ws, int n, const void* xin, const 
   return TREELSTM_OK;
 }
 
+using FwdTcKernel = void (*)(TmapSet, TcParams, int);
+static FwdTcKernel fwd_tc_kernel(bool leaves_first, bool gates) {
+  if (leaves_first) return gates ? k_fwd_tc<true, true> : k_fwd_tc<true, false>;
+  return gates ? k_fwd_tc<false, true> : k_fwd_tc<false, false>;
+}
 int init_tc_attributes(treelstm* ctx) {
-  TL_CUDA(ctx, cudaFuncSetAttribute(k_fwd_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-  TL_CUDA(ctx, cudaFuncSetAttribute(k_fwd_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  for (int i = 0; i < 4; ++i)
+    TL_CUDA(ctx, cudaFuncSetAttribute(fwd_tc_kernel(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
   int per_sm = 0;
-  TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fwd_tc<true>, kThreads, kSmemBytes));
+  TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwd_tc_kernel(true, false), kThreads, kSmemBytes));
   ctx->tc_resident_ctas = per_sm * ctx->sm_count;
   return TREELSTM_OK;
 }
@@ -989,8 +994,7 @@ int launch_forward_bf16(treelstm* ctx, int n, const int32_t* left, const int32_t
       attr.id = cudaLaunchAttributeCooperative; attr.val.cooperative = 1;
     }
     cfg.attrs = &attr; cfg.numAttrs = 1;
-    if (p.leaves_first) TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_fwd_tc<true>, ctx->maps, p, only));
-    else TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_fwd_tc<false>, ctx->maps, p, only));
+    TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, fwd_tc_kernel(p.leaves_first, p.gates != nullptr), ctx->maps, p, only));
     ctx->launches += 1;
     if (with_tail)
       return launch_forward_bf16_tail(ctx, n, left, right, token, h, c, order, level_offset_dev, flags, ws, lay, stream);
@@ -1007,7 +1011,7 @@ int launch_forward_bf16(treelstm* ctx, int n, const int32_t* left, const int32_t
     if (w <= 0) continue;
     const int tiles = choose_tile_plan(w, groups, p.sched_ctas, lvl == 0,
                                        lvl == 0 ? ctx->Ep / kKBlock : 2 * ctx->Hp / kKBlock).tiles;
-    k_fwd_tc<false><<<tiles, kThreads, kSmemBytes, stream>>>(ctx->maps, p, lvl);
+    fwd_tc_kernel(false, p.gates != nullptr)<<<tiles, kThreads, kSmemBytes, stream>>>(ctx->maps, p, lvl);
     ctx->launches += 1;
   }
   TL_CUDA(ctx, cudaGetLastError());

@@ -327,7 +327,7 @@ k_fwd_tc_subforest(const __grid_constant__ TmapSet maps, const __grid_constant__
           if (nx_have) nx_node = valid2 ? chk(p.st, p.order[row + BM], p.n) : 0;
           EpiTile et;
           et.leaf = leaf; et.G = G; et.gcols = gcols; et.ncols = ncols; et.nt = nt;
-          et.row = row; et.node = node; et.slot = slot; et.valid = valid;
+          et.row0 = row0; et.row_end = end; et.row = row; et.node = node; et.slot = slot; et.valid = valid;
           et.allow_staged_out = rows > 64;   // a narrow tile writes so little that it stores straight from registers
           et.r = r; et.e = e; et.quad = quad;
           et.cstage_addr = cstage_addr; et.cstage_ptr = cstage_ptr; et.crow_shift = L.crow_shift;
@@ -340,7 +340,9 @@ k_fwd_tc_subforest(const __grid_constant__ TmapSet maps, const __grid_constant__
 #ifdef TREELSTM_TRACE
           if (tid == 0 && t == 0) TL_STAMP(trace, lvl, 4);
 #endif
-          epilogue_tile(p, et, epi_phase, alive, s_abort, [&]() { if (nx_have) nx_slot = valid2 ? chk_slot(p.st, p.slot[nx_node], p.n) : -1; });
+          auto between = [&]() { if (nx_have) nx_slot = valid2 ? chk_slot(p.st, p.slot[nx_node], p.n) : -1; };
+          if (p.gates) epilogue_tile<true>(p, et, epi_phase, alive, s_abort, between);
+          else epilogue_tile<false>(p, et, epi_phase, alive, s_abort, between);
 #ifdef TREELSTM_TRACE
           if (tid == 0 && t == tiles - 1) TL_STAMP(trace, lvl, 5);
 #endif

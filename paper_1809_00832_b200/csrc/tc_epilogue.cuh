@@ -19,6 +19,7 @@ struct EpiTile {
   // the tile
   bool leaf;
   int G, gcols, ncols, nt;      // unit groups, packed columns per group, columns in use, column tile (units of G groups)
+  int row0, row_end;            // its rows (operand rows of the children)
   int row, node, slot;          // this thread's operand row, its node and delivery slot (2 * pos(caller) + side, -1: root)
   bool valid;                   // the row belongs to the tile
   bool allow_staged_out;        // copy the outputs out through the staging rows (else straight from registers)
@@ -42,9 +43,10 @@ struct EpiTile {
 #define TL_TILE_STAMP(t, k) do { } while (0)
 #endif
 
-// between_fn runs after the cell updates and before the accumulator is handed back (the callers
+// kGates: the gate activations are kept for the backward pass (p.gates).  Code of its own: carrying them through the cell
+// update behind a branch made a forward without them 6 % slower (1000 trees).  between_fn runs after the cell updates and before the accumulator is handed back (the callers
 // fetch row data of their next tile there).
-template <class BetweenFn>
+template <bool kGates, class BetweenFn>
 __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& t, uint32_t& epi_phase, bool& alive,
                                               volatile int* s_abort, BetweenFn between_fn) {
   const int H = p.H, Hp = p.Hp, G = t.G, r = t.r, e = t.e, nt = t.nt, gcols = t.gcols;
@@ -58,7 +60,20 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
   const int half = t.half;
   const uint32_t my_c = t.cstage_addr + ((uint32_t)r << t.crow_shift);
   unsigned char* mine = t.cstage_ptr + ((size_t)r << t.crow_shift);
-  if (staged) {   // the children's cell states of this thread's row, while the MMAs run
+  // The children's cell states, while the MMAs run.  With gates kept, whole tiles fetch them several lanes per row segment:
+  // one row per lane is 32 lines per request, in the queue behind the gates' stores (training step of 256 trees 679 -> 637 us).
+  // Otherwise each thread fetches its own row: the meeting of the threads that the other form needs costs more than
+  // it saves (forward of 1000 trees 235 -> 246 us with it).
+  const bool spread = staged && t.allow_staged_out && kGates && (G & (G - 1)) == 0;
+  if (spread) {
+    const int per = 4 * G, lper = 31 - __clz(per);
+    const float* base = p.cin + (size_t)t.row0 * 2 * H + nt * G * 8;
+    for (int idx = e * BM + r; idx < BM * per; idx += 2 * BM) {
+      const int ro = idx >> lper, k = idx & (per - 1), side = k >= 2 * G, ch = k - side * 2 * G;
+      cp_async16(t.cstage_addr + ((uint32_t)ro << t.crow_shift) + (uint32_t)(((side * half + ch) ^ (ro & 7)) << 4),
+                 base + (size_t)ro * 2 * H + side * H + ch * 4, t.row0 + ro < t.row_end ? 16u : 0u);
+    }
+  } else if (staged) {
     const float* sl = crow + nt * G * 8;
     const float* sr = sl + H;
     const uint32_t nb = valid ? 16u : 0u;
@@ -76,6 +91,12 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
   if (!mbar_wait(t.tfull, t.acc_phase, s_abort, p.wait_limit, p.st)) alive = false;
   alive = __all_sync(kFullMask, alive);
   asm volatile("cp.async.wait_all;" ::: "memory");
+  if (spread) {                                // every thread's pieces are in
+    mbar_arrive(t.epi_bar);
+    if (!mbar_wait(t.epi_bar, epi_phase, s_abort, p.wait_limit, p.st)) alive = false;
+    epi_phase ^= 1;
+    alive = __all_sync(kFullMask, alive);
+  }
   if (!alive) return;
   TL_TILE_STAMP(t, 0);
   tc_fence_after();
@@ -175,7 +196,7 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
           st_row4(p.c + (size_t)node * H + u0, vec, count, cv);
         }
       }
-      if (p.gates && count > 0) {
+      if (kGates && count > 0) {
         float* gp = p.gates + (size_t)node * 5 * H + u0;
         st_row4(gp, vec, count, gi);
         st_row4(gp + H, vec, count, gfl);
