@@ -60,11 +60,10 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
   const int half = t.half;
   const uint32_t my_c = t.cstage_addr + ((uint32_t)r << t.crow_shift);
   unsigned char* mine = t.cstage_ptr + ((size_t)r << t.crow_shift);
-  // The children's cell states, while the MMAs run.  With gates kept, whole tiles fetch them several lanes per row segment:
-  // one row per lane is 32 lines per request, in the queue behind the gates' stores (training step of 256 trees 679 -> 637 us).
-  // Otherwise each thread fetches its own row: the meeting of the threads that the other form needs costs more than
-  // it saves (forward of 1000 trees 235 -> 246 us with it).
-  const bool spread = staged && t.allow_staged_out && kGates && (G & (G - 1)) == 0;
+  // The children's cell states, while the MMAs run: of whole tiles several lanes per row segment (one row per lane is 32
+  // lines per request: forward of 1000 trees 233 -> 231 us, training step of 256 trees, where the requests queue behind
+  // the gates' stores, 679 -> 637 us), of narrow ones each thread its own row (no meeting of the threads behind it).
+  const bool spread = staged && t.allow_staged_out && (G & (G - 1)) == 0;
   if (spread) {
     const int per = 4 * G, lper = 31 - __clz(per);
     const float* base = p.cin + (size_t)t.row0 * 2 * H + nt * G * 8;
