@@ -206,3 +206,30 @@ def test_training_step_of_wide_forests(H, E, shapes):
     res = _train_step(model, forest, labels, binding.PERSISTENT)
     _compare(res, ref, util.TOL["fp32"])
     _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("H,trees", [(260, 256), (260, 257), (258, 257), (264, 128), (257, 129)])
+def test_wide_wavefronts_at_the_limits_of_their_kinds(H, trees):
+    """wavefronts of 256 and 257 nodes (operands formed at the tensor core or stored first), of exactly one and of one more
+    than one tile of 128, in rows that can be read 16 bytes at a time and in rows that cannot"""
+    rng = np.random.default_rng(77 + H + trees)
+    params = fg.draw_params(rng, H, 20, 50, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    forest = fg.forest_from_shapes([fg.balanced_shape(4)] * trees, rng, 50)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("H,classes", [(40, 1), (64, 8), (64, 9), (65, 5), (65, 6), (160, 5), (161, 5), (256, 5), (256, 6), (257, 5)])
+def test_classifier_of_every_width(H, classes):
+    """the classifier's sums in registers up to 64, 160 and 256 units with few classes, in shared memory beyond"""
+    rng = np.random.default_rng(H + classes)
+    params = fg.draw_params(rng, H, 24, 40, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=classes)
+    forest = fg.forest_from_shapes([fg.random_split_shape(rng, 30) for _ in range(4)] + [None], rng, 40)
+    labels = rng.integers(0, classes, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
