@@ -357,8 +357,9 @@ __device__ __forceinline__ void gates_element(const BwdParams& p, int row_begin,
   const int H = p.H;
   const int row = row_begin + (int)(idx / H), u = (int)(idx % H);
   const int node = chk(p.st, p.order[row], p.n);
-  const float* g = p.gates + (size_t)node * 5 * H + u;
-  const float gi = g[0], go = g[3 * H], gu = g[4 * H];
+  const int gs = row_pitch(H);
+  const float* g = p.gates + (size_t)node * 5 * gs + u;
+  const float gi = g[0], go = g[3 * gs], gu = g[4 * gs];
   const float cn = p.c[(size_t)node * H + u];
   const float tc = tanhf(cn);
   const float dhn = p.dh[(size_t)node * H + u];
@@ -372,7 +373,7 @@ __device__ __forceinline__ void gates_element(const BwdParams& p, int row_begin,
     dz[2 * H] = 0.f;
   } else {
     const int l = chk(p.st, p.left[node], p.n), r = chk(p.st, p.right[node], p.n);
-    const float gfl = g[H], gfr = g[2 * H];
+    const float gfl = g[gs], gfr = g[2 * gs];
     dz[H] = dcn * p.c[(size_t)l * H + u] * gfl * (1.f - gfl);
     dz[2 * H] = dcn * p.c[(size_t)r * H + u] * gfr * (1.f - gfr);
     p.dc[(size_t)l * H + u] = dcn * gfl;  // every node has exactly one caller: plain stores
@@ -590,7 +591,7 @@ __device__ __forceinline__ int gate_of_column(int j, int H) { return (j >= H) + 
 // they are in flight together: one round trip instead of one per element; then the arithmetic and the stores.
 __device__ __forceinline__ void fused_gate_gradients(const BwdParams& p, const FusedItem& it, DinputSmem& sm, int ib,
                                                      int buf, int j0) {
-  const int H = p.H, J = 5 * H, tid = threadIdx.x;
+  const int H = p.H, J = 5 * H, gs = row_pitch(H), tid = threadIdx.x;
   float dhn[kLd], dci[kLd], go[kLd], cn[kLd], g1[kLd], g2[kLd];
 #pragma unroll
   for (int q = 0; q < kLd; ++q) {
@@ -599,13 +600,13 @@ __device__ __forceinline__ void fused_gate_gradients(const BwdParams& p, const F
     const int g = gate_of_column(j, H), u = j - g * H;
     const bool forget = g == 1 || g == 2;
     const int child = chk(p.st, g == 2 ? sm.fright[ib][i] : sm.fleft[ib][i], p.n);
-    const float* gt = p.gates + (size_t)node * J + u;
+    const float* gt = p.gates + (size_t)node * 5 * gs + u;
     dhn[q] = p.dh[(size_t)node * H + u];
     dci[q] = p.dc[(size_t)node * H + u];
-    go[q] = gt[3 * H];
+    go[q] = gt[3 * gs];
     cn[q] = p.c[(size_t)node * H + u];
-    g1[q] = gt[forget ? g * H : 0];                                   // f_l / f_r, else i
-    g2[q] = *(forget ? p.c + (size_t)child * H + u : gt + 4 * H);    // the child's cell state, else u
+    g1[q] = gt[forget ? g * gs : 0];                                   // f_l / f_r, else i
+    g2[q] = *(forget ? p.c + (size_t)child * H + u : gt + 4 * gs);   // the child's cell state, else u
   }
   const bool keep = it.k0 == 0;
 #pragma unroll
@@ -1072,7 +1073,7 @@ __device__ __forceinline__ unsigned char* dz_unit(const BwdImages& img, int pos,
 // (One element per thread through shared memory: 12 k cycles for eight nodes per CTA.)
 template <bool kVec>
 __device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& img, const WidePlan& w) {
-  const int H = p.H, J = 5 * H, gp = gate_pitch(H), octs = gp / 8, ju = img_units(5 * gp), tid = threadIdx.x;
+  const int H = p.H, gs = row_pitch(H), gp = gate_pitch(H), octs = gp / 8, ju = img_units(5 * gp), tid = threadIdx.x;
   const long long all = (long long)(w.end - w.begin) * octs;
   const int share = (int)((all + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
   const long long lo = (long long)blockIdx.x * share, hi = min(all, lo + share);
@@ -1081,14 +1082,14 @@ __device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& 
     const int i = (int)(e / octs), o = (int)(e - (long long)i * octs), u0 = 8 * o, pos = w.begin + i;
     const int node = chk(p.st, p.order[pos], p.n);
     const int l = w.leaf ? node : chk(p.st, p.pos_left[pos], p.n), r = w.leaf ? node : chk(p.st, p.pos_right[pos], p.n);
-    const float* g = p.gates + (size_t)node * J;
+    const float* g = p.gates + (size_t)node * 5 * gs;
     float gi[8], go[8], gu[8], c[8], dh[8], dc[8], z[8];
     load8<kVec>(p.c + (size_t)node * H, u0, H, c);
     load8<kVec>(p.dh + (size_t)node * H, u0, H, dh);
     load8<kVec>(p.dc + (size_t)node * H, u0, H, dc);
-    load8<kVec>(g + 3 * H, u0, H, go);
-    load8<kVec>(g, u0, H, gi);
-    load8<kVec>(g + 4 * H, u0, H, gu);
+    load8<true>(g + 3 * gs, u0, gs, go);
+    load8<true>(g, u0, gs, gi);
+    load8<true>(g + 4 * gs, u0, gs, gu);
     auto put = [&](int gate) {
       const int j = gate * gp + u0;
 #pragma unroll
@@ -1097,8 +1098,8 @@ __device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& 
     };
     float gf[2][8], cc[2][8];
     if (!w.leaf) {
-      load8<kVec>(g + H, u0, H, gf[0]);
-      load8<kVec>(g + 2 * H, u0, H, gf[1]);
+      load8<true>(g + gs, u0, gs, gf[0]);
+      load8<true>(g + 2 * gs, u0, gs, gf[1]);
       load8<kVec>(p.c + (size_t)l * H, u0, H, cc[0]);
       load8<kVec>(p.c + (size_t)r * H, u0, H, cc[1]);
     }
@@ -1146,21 +1147,22 @@ __device__ __forceinline__ void wide_gates(const BwdParams& p, const BwdImages& 
 template <bool kVec>
 __device__ __forceinline__ void direct_block(const BwdParams& p, const BwdImages& img, unsigned char* tile, int kb, int pos0, int rows,
                                              bool keep, const int* s_node, const int* s_left, const int* s_right) {
-  const int H = p.H, J = 5 * H, gp = gate_pitch(H), ju = img_units(5 * gp), c = threadIdx.x & 7, j = kb * 64 + 8 * c;
+  const int H = p.H, gs = row_pitch(H), gp = gate_pitch(H), ju = img_units(5 * gp), c = threadIdx.x & 7, j = kb * 64 + 8 * c;
   const int gate = j / gp, u0 = j - gate * gp;
   const bool forget = gate == 1 || gate == 2;
   for (int i = threadIdx.x >> 3; i < rows; i += kWideThreads / 8) {
     float z[8];
     if (gate < 5) {
       const int node = s_node[i], child = gate == 2 ? s_right[i] : s_left[i];
-      const float* g = p.gates + (size_t)node * J;
+      const float* g = p.gates + (size_t)node * 5 * gs;
       float dh[8], dc[8], go[8], cn[8], g1[8], g2[8];
       load8<kVec>(p.dh + (size_t)node * H, u0, H, dh);
       load8<kVec>(p.dc + (size_t)node * H, u0, H, dc);
-      load8<kVec>(g + 3 * H, u0, H, go);
+      load8<true>(g + 3 * gs, u0, gs, go);
       load8<kVec>(p.c + (size_t)node * H, u0, H, cn);
-      load8<kVec>(g + (forget ? gate * H : 0), u0, H, g1);                         // f_l / f_r, else i
-      load8<kVec>(forget ? p.c + (size_t)child * H : g + 4 * H, u0, H, g2);       // the child's cell state, else u
+      load8<true>(g + (forget ? gate * gs : 0), u0, gs, g1);                         // f_l / f_r, else i
+      if (forget) load8<kVec>(p.c + (size_t)child * H, u0, H, g2);                  // the child's cell state, else u
+      else load8<true>(g + 4 * gs, u0, gs, g2);
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const float tc = tanhf(cn[k]), dcn = dc[k] + dh[k] * go[k] * (1.f - tc * tc);

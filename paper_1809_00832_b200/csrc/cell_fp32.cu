@@ -172,8 +172,9 @@ __device__ void fp32_tile(const FwdParams& p, int row0, int row_end, int u0, boo
     p.h[(size_t)node * H + u] = go * tanhf(cn);
     count_write(p.chk_counts, node, 1);
     if (p.gates) {
-      float* g = p.gates + (size_t)node * 5 * H + u;
-      g[0] = gi; g[H] = gfl; g[2 * H] = gfr; g[3 * H] = go; g[4 * H] = gu;
+      const int gs = row_pitch(H);
+      float* g = p.gates + (size_t)node * 5 * gs + u;
+      g[0] = gi; g[gs] = gfl; g[2 * gs] = gfr; g[3 * gs] = go; g[4 * gs] = gu;
     }
   }
 }
@@ -306,8 +307,9 @@ __device__ void fp32_tile_stationary(const FwdParams& p, int row0, int row_end, 
     p.h[(size_t)node * H + u] = go * tanhf(cn);
     count_write(p.chk_counts, node, 1);
     if (p.gates) {
-      float* g = p.gates + (size_t)node * 5 * H + u;
-      g[0] = gi; g[H] = gfl; g[2 * H] = gfr; g[3 * H] = go; g[4 * H] = gu;
+      const int gs = row_pitch(H);
+      float* g = p.gates + (size_t)node * 5 * gs + u;
+      g[0] = gi; g[gs] = gfl; g[2 * gs] = gfr; g[3 * gs] = go; g[4 * gs] = gu;
     }
   };
   if (kSplit) {

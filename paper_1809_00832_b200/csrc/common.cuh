@@ -27,6 +27,9 @@ struct DevStatus {
 static_assert(sizeof(DevStatus) == 256, "control block is one 256-byte line group");
 
 // Offsets (bytes) of the regions inside the workspace for a forest of up to n nodes.
+// Row pitch (floats) of H units in arrays of the workspace: every row starts on a 16-byte boundary whatever H.
+__host__ __device__ inline int row_pitch(int H) { return (H + 3) / 4 * 4; }
+
 struct WsLayout {
   size_t status, parent, pending, order_tmp, level_offset, roots, table, slot, part_order, part_offset,
       part_spill, xin, ain, cin, gates, dh, dc, dz, tok_slot, trace, check, pre, img_dz, img_x0, img_x1, img_end, total;

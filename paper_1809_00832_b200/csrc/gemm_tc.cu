@@ -234,7 +234,7 @@ __device__ __forceinline__ void deliver_leaves(const TcParams& p, int gwarp, int
             __nv_bfloat162 lo = __floats2bfloat162_rn(hv[q][sd][0], hv[q][sd][1]), hi = __floats2bfloat162_rn(hv[q][sd][2], hv[q][sd][3]);
             *reinterpret_cast<uint2*>(p.ain + (row + sd) * Hp + u) =
                 make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-            if (count > 0) st_row4(p.cin + (row + sd) * H + u, vec, count, cv[q][sd]);
+            if (count > 0) st_row4(p.cin + (row + sd) * row_pitch(H) + u, true, 4, cv[q][sd]);
           }
         }
       }

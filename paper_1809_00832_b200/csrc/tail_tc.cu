@@ -249,50 +249,27 @@ k_fwd_tc_tail(const __grid_constant__ TmapSet maps, const __grid_constant__ SfTm
     const int* fresh = s_rows + (b * 3 + 2) * kTailRows;
     __syncwarp();
     asm volatile("bar.sync 2, 64;" ::: "memory");   // the flags written by both fetching warps are in
-    if ((H & 3) == 0) {                             // 16-byte pieces: (row, side) runs of U floats are aligned
-      const int c4 = U / 4, total = rows * 2 * c4;
-      for (int e0 = 0; e0 < total; e0 += 64 * 8) {
-        float4 v[8];
-        bool take[8];
+    // 16-byte pieces: (row, side) runs of U floats
+    const int c4 = U / 4, total = rows * 2 * c4;
+    for (int e0 = 0; e0 < total; e0 += 64 * 8) {
+      float4 v[8];
+      bool take[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int e = e0 + j * 64 + t;
-          v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-          take[j] = false;
-          if (e < total) {
-            const int pair = e / c4, q = e - pair * c4;         // pair = row * 2 + side
-            take[j] = !((fresh[pair >> 1] >> (pair & 1)) & 1);
-            if (take[j] && U0 + 4 * q < H)
-              v[j] = __ldcg(reinterpret_cast<const float4*>(p.cin + (size_t)(2 * begin + pair) * H + U0 + 4 * q));
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int e = e0 + j * 64 + t;
-          if (take[j]) reinterpret_cast<float4*>(dst)[e] = v[j];
+      for (int j = 0; j < 8; ++j) {
+        const int e = e0 + j * 64 + t;
+        v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        take[j] = false;
+        if (e < total) {
+          const int pair = e / c4, q = e - pair * c4;         // pair = row * 2 + side
+          take[j] = !((fresh[pair >> 1] >> (pair & 1)) & 1);
+          if (take[j] && U0 + 4 * q < H)
+            v[j] = __ldcg(reinterpret_cast<const float4*>(p.cin + (size_t)(2 * begin + pair) * row_pitch(H) + U0 + 4 * q));
         }
       }
-    } else {
-      const int total = rows * 2 * U;
-      for (int e0 = 0; e0 < total; e0 += 64 * 8) {
-        float v[8];
-        bool take[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int e = e0 + j * 64 + t;
-          v[j] = 0.f;
-          take[j] = false;
-          if (e < total) {
-            const int pair = e / U, u = e - pair * U;
-            take[j] = !((fresh[pair >> 1] >> (pair & 1)) & 1);
-            if (take[j] && U0 + u < H) v[j] = __ldcg(p.cin + (size_t)(2 * begin + pair) * H + U0 + u);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int e = e0 + j * 64 + t;
-          if (take[j]) dst[e] = v[j];
-        }
+      for (int j = 0; j < 8; ++j) {
+        const int e = e0 + j * 64 + t;
+        if (take[j]) reinterpret_cast<float4*>(dst)[e] = v[j];
       }
     }
   };
@@ -339,7 +316,7 @@ k_fwd_tc_tail(const __grid_constant__ TmapSet maps, const __grid_constant__ SfTm
       p.c[(size_t)node * H + unit] = cn;
       count_write(p.chk_counts, node, 1);
       if (slot >= 0) {
-        if (!((keep_near >> (2 * it)) & 3u)) p.cin[(size_t)slot * H + unit] = cn;
+        if (!((keep_near >> (2 * it)) & 3u)) p.cin[(size_t)slot * row_pitch(H) + unit] = cn;
         count_write(p.chk_counts ? p.chk_counts + p.n : nullptr, slot >> 1, 1);   // handed over, in shared or global memory
         count_write(p.chk_counts ? p.chk_counts + 2 * p.n : nullptr, slot >> 1, 1);
       }
@@ -549,8 +526,9 @@ k_fwd_tc_tail(const __grid_constant__ TmapSet maps, const __grid_constant__ SfTm
             hs[q] = __float2bfloat16_rn(real ? hn : 0.f);
             if (dep1[it] >= 0) cnext[dep1[it]] = real ? cn : 0.f;
             if (p.gates && real) {
-              float* gp = p.gates + (size_t)keep_node[it] * 5 * H + U0 + (q % U);
-              gp[0] = gi; gp[H] = gfl; gp[2 * H] = gfr; gp[3 * H] = go; gp[4 * H] = gu;
+              const int hp4 = row_pitch(H);
+              float* gp = p.gates + (size_t)keep_node[it] * 5 * hp4 + U0 + (q % U);
+              gp[0] = gi; gp[hp4] = gfl; gp[2 * hp4] = gfr; gp[3 * hp4] = go; gp[4 * hp4] = gu;
             }
           }
           kept = n_items;

@@ -49,12 +49,12 @@ struct EpiTile {
 template <bool kGates, class BetweenFn>
 __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& t, uint32_t& epi_phase, bool& alive,
                                               volatile int* s_abort, BetweenFn between_fn) {
-  const int H = p.H, Hp = p.Hp, G = t.G, r = t.r, e = t.e, nt = t.nt, gcols = t.gcols;
+  const int H = p.H, Hp = p.Hp, Hc = row_pitch(H), G = t.G, r = t.r, e = t.e, nt = t.nt, gcols = t.gcols;
   const bool leaf = t.leaf, valid = t.valid;
   const int node = t.node, slot = t.slot;
   const bool vec = (H % 4) == 0;
-  const float* crow = p.cin + (size_t)t.row * 2 * H;   // [c_l | c_r] of the node at this position
-  const bool full_slice = vec && (nt + 1) * G * 8 <= H;   // no padded unit among the tile's columns
+  const float* crow = p.cin + (size_t)t.row * 2 * Hc;   // [c_l | c_r] of the node at this position
+  const bool full_slice = (nt + 1) * G * 8 <= H;   // no padded unit among the tile's columns
   const bool staged = !leaf && full_slice;
   const bool staged_out = full_slice && t.allow_staged_out;
   const int half = t.half;
@@ -66,15 +66,15 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
   const bool spread = staged && t.allow_staged_out && (G & (G - 1)) == 0;
   if (spread) {
     const int per = 4 * G, lper = 31 - __clz(per);
-    const float* base = p.cin + (size_t)t.row0 * 2 * H + nt * G * 8;
+    const float* base = p.cin + (size_t)t.row0 * 2 * Hc + nt * G * 8;
     for (int idx = e * BM + r; idx < BM * per; idx += 2 * BM) {
       const int ro = idx >> lper, k = idx & (per - 1), side = k >= 2 * G, ch = k - side * 2 * G;
       cp_async16(t.cstage_addr + ((uint32_t)ro << t.crow_shift) + (uint32_t)(((side * half + ch) ^ (ro & 7)) << 4),
-                 base + (size_t)ro * 2 * H + side * H + ch * 4, t.row0 + ro < t.row_end ? 16u : 0u);
+                 base + (size_t)ro * 2 * Hc + side * Hc + ch * 4, t.row0 + ro < t.row_end ? 16u : 0u);
     }
   } else if (staged) {
     const float* sl = crow + nt * G * 8;
-    const float* sr = sl + H;
+    const float* sr = sl + Hc;
     const uint32_t nb = valid ? 16u : 0u;
     for (int ch = e; ch < 2 * G; ch += 2) {
       cp_async16(my_c + (uint32_t)((ch ^ (r & 7)) << 4), sl + ch * 4, nb);
@@ -140,7 +140,7 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           cl[j] = j < count ? __ldcg(crow + u0 + j) : 0.f;
-          cr[j] = j < count ? __ldcg(crow + H + u0 + j) : 0.f;
+          cr[j] = j < count ? __ldcg(crow + Hc + u0 + j) : 0.f;
         }
       }
       const float* bq = reinterpret_cast<const float*>(bcur);
@@ -185,7 +185,7 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
             packed[j] = *reinterpret_cast<uint32_t*>(&b2);
           }
           *reinterpret_cast<uint2*>(p.ain + (size_t)slot * Hp + u0) = make_uint2(packed[0], packed[1]);
-          if (count > 0) st_row4(p.cin + (size_t)slot * H + u0, vec, count, cv);
+          if (count > 0) st_row4(p.cin + (size_t)slot * Hc + u0, true, count, cv);
           count_write(p.chk_counts ? p.chk_counts + p.n : nullptr, slot >> 1, count);
           count_write(p.chk_counts ? p.chk_counts + 2 * p.n : nullptr, slot >> 1, count);
         }
@@ -196,12 +196,12 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
         }
       }
       if (kGates && count > 0) {
-        float* gp = p.gates + (size_t)node * 5 * H + u0;
-        st_row4(gp, vec, count, gi);
-        st_row4(gp + H, vec, count, gfl);
-        st_row4(gp + 2 * H, vec, count, gfr);
-        st_row4(gp + 3 * H, vec, count, go);
-        st_row4(gp + 4 * H, vec, count, gu);
+        float* gp = p.gates + (size_t)node * 5 * Hc + u0;
+        st_row4(gp, true, 4, gi);
+        st_row4(gp + Hc, true, 4, gfl);
+        st_row4(gp + 2 * Hc, true, 4, gfr);
+        st_row4(gp + 3 * Hc, true, 4, go);
+        st_row4(gp + 4 * Hc, true, 4, gu);
       }
     }
   }
@@ -225,18 +225,31 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, const EpiTile& 
         const float4 c4 = *reinterpret_cast<const float4*>(src + ((ch ^ (ro & 7)) << 4));
         const float4 h4 = *reinterpret_cast<const float4*>(src + (((half + ch) ^ (ro & 7)) << 4));
         const int uo = nt * G * 8 + 4 * ch;
-        *reinterpret_cast<float4*>(p.h + (size_t)node_o * H + uo) = h4;
-        *reinterpret_cast<float4*>(p.c + (size_t)node_o * H + uo) = c4;
+        if (vec) {
+          *reinterpret_cast<float4*>(p.h + (size_t)node_o * H + uo) = h4;
+          *reinterpret_cast<float4*>(p.c + (size_t)node_o * H + uo) = c4;
+        }
         count_write(p.chk_counts, node_o, 4);
         const int slot_o = t.s_rowslot[ro];
         if (slot_o >= 0) {
           count_write(p.chk_counts ? p.chk_counts + p.n : nullptr, slot_o >> 1, 4);
           count_write(p.chk_counts ? p.chk_counts + 2 * p.n : nullptr, slot_o >> 1, 4);
-          *reinterpret_cast<float4*>(p.cin + (size_t)slot_o * H + uo) = c4;
+          *reinterpret_cast<float4*>(p.cin + (size_t)slot_o * Hc + uo) = c4;
           __nv_bfloat162 lo = __floats2bfloat162_rn(h4.x, h4.y), hi = __floats2bfloat162_rn(h4.z, h4.w);
           *reinterpret_cast<uint2*>(p.ain + (size_t)slot_o * Hp + uo) =
               make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
         }
+      }
+    }
+    if (ok && !vec) {                                   // rows of h and c on any boundary: a unit per lane along them
+      const int U = 8 * G, lu = (G & (G - 1)) == 0 ? 31 - __clz(U) : -1;
+      for (int idx = e * BM + r; idx < BM * U; idx += 2 * BM) {
+        const int ro = lu >= 0 ? idx >> lu : idx / U, u = idx - ro * U, node_o = t.s_rownode[ro];
+        if (node_o < 0) continue;
+        const unsigned char* src = t.cstage_ptr + ((size_t)ro << t.crow_shift) + 4 * (u & 3);
+        const size_t at = (size_t)node_o * H + nt * U + u;
+        p.h[at] = *reinterpret_cast<const float*>(src + (((half + (u >> 2)) ^ (ro & 7)) << 4));
+        p.c[at] = *reinterpret_cast<const float*>(src + (((u >> 2) ^ (ro & 7)) << 4));
       }
     }
     // the staging rows are reused by the next tile's loads of the children's cell states

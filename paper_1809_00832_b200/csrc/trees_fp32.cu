@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
         if constexpr (CELL == kLstm) {
           const float a = g == 4 ? tanhf(z) : sigmoid_acc(z);
           act[i * outs + o] = a;
-          if (p.gates && j0 + u < H) p.gates[(size_t)list[lo + i] * 5 * H + g * H + j0 + u] = a;
+          if (p.gates && j0 + u < H) p.gates[((size_t)list[lo + i] * 5 + g) * row_pitch(H) + j0 + u] = a;
         } else if (u < JS && j0 + u < H) {
           const float hv = tanhf(z);
           const int node = list[lo + i];
@@ -627,8 +627,9 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
       p.h[(size_t)node * H + u] = go * tanhf(cv);
       count_write(p.chk_counts, node, 1);
       if (p.gates) {
-        float* g = p.gates + (size_t)node * 5 * H + u;
-        g[0] = gi; g[3 * H] = go; g[4 * H] = gu;
+        const int gs = row_pitch(H);
+        float* g = p.gates + (size_t)node * 5 * gs + u;
+        g[0] = gi; g[3 * gs] = go; g[4 * gs] = gu;
       }
     }
   }
@@ -703,9 +704,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
       const size_t at = (size_t)node * H + j0 + my_u;
       if constexpr (CELL == kLstm) {
         const unsigned kd = kids[node];
-        const float* gp = p.gates + (size_t)node * 5 * H + j0 + my_u;
+        const float* gp = p.gates + (size_t)node * 5 * row_pitch(H) + j0 + my_u;
 #pragma unroll
-        for (int q = 0; q < G; ++q) g[q] = __ldg(gp + q * H);
+        for (int q = 0; q < G; ++q) g[q] = __ldg(gp + q * row_pitch(H));
         cn = __ldg(p.c + at);
         cl = __ldg(p.c + (size_t)(kd & 0xFFFFu) * H + j0 + my_u);
         cr = __ldg(p.c + (size_t)(kd >> 16) * H + j0 + my_u);
@@ -881,8 +882,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
     const int node = leaf[q];
     const size_t at = (size_t)node * H + j0 + u;
     if constexpr (CELL == kLstm) {
-      const float* gp = p.gates + (size_t)node * 5 * H + j0 + u;
-      const float gi = __ldg(gp), go = __ldg(gp + 3 * H), gu = __ldg(gp + 4 * H), tc = tanhf(__ldg(p.c + at));
+      const int gs = row_pitch(H);
+      const float* gp = p.gates + (size_t)node * 5 * gs + j0 + u;
+      const float gi = __ldg(gp), go = __ldg(gp + 3 * gs), gu = __ldg(gp + 4 * gs), tc = tanhf(__ldg(p.c + at));
       const float dhn = *dh_at(code, node, u);
       const float dcn = (code == kNoCaller ? 0.f : *dc_at(code, node, u)) + dhn * go * (1.f - tc * tc);
       float* dz = p.dz + (size_t)node * 5 * H + j0 + u;
