@@ -163,6 +163,7 @@ struct treelstm {
     bool ok = false;
     tl::TreesShape s;
     float *Wf = nullptr, *Wb = nullptr;                 // register images of the weights
+    float* Wx = nullptr;                                // input weights of the leaves' gates, by slices of units
     int clusters = 0, clusters_bwd = 0;                 // that the device holds at once
     ushort2* pairs = nullptr;                           // RNTN: operands of every input chunk
   } trees;

@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "split_tc.cuh"
 
 namespace tl {
 namespace {
@@ -518,32 +519,83 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
 }
 
 // ---- TreeLSTM leaves ------------------------------------------------------------------------------ //
-// Their states need no schedule, so this kernel runs beside the scheduler, over the whole GPU.  A CTA takes 2 ROWS consecutive
-// node ids, the leaves among them (half, in a forest of any shape) in tiles of ROWS, and 32 hidden units x the
-// three gates a leaf has.  Thread (unit, row group): ROWS / 8 rows x 3 gates; the rows are read as broadcasts,
-// the weights one word per lane, the next chunk is fetched into registers meanwhile.
-constexpr int kLeafT = 256, kLeafU = 32, kLeafK = 32;
+// Their states need no schedule, so this kernel runs beside the scheduler, over the whole GPU.  A CTA takes 64 consecutive node
+// ids, the leaves among them (about half), and 32 hidden units x the three gates a leaf has.  All operands of
+// kLeafK contraction indices are asked for at once - the weights as one bulk copy out of an image kept for it, the
+// embedding rows through registers - because the kernel is bound by the latency of its loads: in chunks of 32 indices,
+// each a round trip behind the one before, 25 trees (H = 150, E = 300) took 43 us with cold caches, this way 28.
+// A warp takes RPT rows and half of the contraction (rows read as broadcasts, weights one word per lane), as many rows
+// as give 16 warps one turn each; the halves meet in shared memory.
+constexpr int kLeafT = 512, kLeafU = 32, kLeafIds = 64, kLeafK = 320;
+constexpr int kLeafSmem = 4 * kLeafK * (3 * kLeafU + kLeafIds);
 struct LeafParams {
   int n, H, E, vocab;
   int* chk_counts;
   const int *left, *token;
-  const float *emb, *W, *b;
+  const float *emb, *Wx, *b;
   float *h, *c, *gates;
+  DevStatus* st;
+  long long wait_limit;
 };
-template <int ROWS>
+// image of the input weights: [slice of 32 units][input unit][gate i, o, u][unit], zeros behind the last unit
+__host__ __device__ inline size_t leaf_image_words(int H, int E) { return (size_t)((H + kLeafU - 1) / kLeafU) * E * 3 * kLeafU; }
+__global__ void k_leaves_pack(int H, int E, const float* W, float* out) {
+  const int total = (int)leaf_image_words(H, E);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const int uu = i % kLeafU, g = i / kLeafU % 3, k = i / (3 * kLeafU) % E, u = i / (3 * kLeafU) / E * kLeafU + uu;
+    out[i] = u < H ? W[(size_t)k * 5 * H + (g ? g + 2 : 0) * H + u] : 0.f;
+  }
+}
+// RPT rows from `rows` on and half of nk contraction indices
+template <int RPT>
+__device__ __forceinline__ void leaf_rows(const float* As, const float* Ws, int pitch, int nk, int rows, int half, int lane, float (&acc)[8][3]) {
+  const int mid = (nk / 2 + 3) & ~3, lo = half ? mid : 0, hi = half ? (nk + 3) & ~3 : mid;
+#pragma unroll 2
+  for (int k = lo; k < hi; k += 4) {
+    float w[4][3];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int g = 0; g < 3; ++g) w[q][g] = Ws[(k + q) * 3 * kLeafU + g * kLeafU + lane];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      const float4 x = *reinterpret_cast<const float4*>(As + (rows + i) * pitch + k);
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        acc[i][g] = fmaf(x.x, w[0][g], acc[i][g]);
+        acc[i][g] = fmaf(x.y, w[1][g], acc[i][g]);
+        acc[i][g] = fmaf(x.z, w[2][g], acc[i][g]);
+        acc[i][g] = fmaf(x.w, w[3][g], acc[i][g]);
+      }
+    }
+  }
+}
 __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
-  constexpr int RPT = ROWS / 8, AL = ROWS * kLeafK / kLeafT, WL = 3 * kLeafU * kLeafK / kLeafT;
-  __shared__ __align__(16) float As[2][ROWS][kLeafK + 4];
-  __shared__ float Ws[2][kLeafK][3 * kLeafU];
-  __shared__ int s_node[2 * ROWS], s_tok[2 * ROWS], s_count;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5, H = p.H, E = p.E;
-  const int tiles_u = (H + kLeafU - 1) / kLeafU;
-  const int id0 = (int)(blockIdx.x / tiles_u) * 2 * ROWS, u0 = (int)(blockIdx.x % tiles_u) * kLeafU;
+  extern __shared__ __align__(16) float leaf_smem[];
+  float* const Ws = leaf_smem;                           // [kLeafK][3 gates][32 units]; then the second halves' sums
+  float* const As = leaf_smem + kLeafK * 3 * kLeafU;     // [rows][pitch]
+  __shared__ int s_node[kLeafIds], s_tok[kLeafIds], s_count, s_abort;
+  __shared__ __align__(8) uint64_t s_bar;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = p.H, E = p.E;
+  const int tiles_u = (H + kLeafU - 1) / kLeafU, slice = (int)blockIdx.x % tiles_u;
+  const int id0 = (int)blockIdx.x / tiles_u * kLeafIds, u0 = slice * kLeafU;
+  const uint32_t bar = smem_u32(&s_bar);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  auto ask = [&](int k0) {                               // one thread: the weights of the next kLeafK indices
+    const uint32_t bytes = (uint32_t)min(kLeafK, E - k0) * 3 * kLeafU * 4;
+    mbar_arrive_expect_tx(bar, bytes);
+    bulk_load(smem_u32(Ws), p.Wx + ((size_t)slice * E + k0) * 3 * kLeafU, bytes, bar);
+  };
+  if (tid == 32) {
+    mbar_init(bar, 1);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    ask(0);
+  }
   if (tid < 32) {                                        // the leaves among the CTA's node ids, ascending
     int count = 0;
 #pragma unroll
-    for (int q = 0; q < 2 * ROWS / 32; ++q) {
+    for (int q = 0; q < kLeafIds / 32; ++q) {
       const int k = id0 + 32 * q + tid;
       const bool lf = k < p.n && p.left[min(k, p.n - 1)] < 0;
       const unsigned m = __ballot_sync(0xffffffffu, lf);
@@ -557,71 +609,66 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
     if (tid == 0) s_count = count;
   }
   __syncthreads();
-  const int count = s_count;
-  const int u = min(u0 + tx, H - 1);
+  const int count = s_count, octant = warp & 7, half = warp >> 3;
+  const int rpt = count <= 32 ? 4 : (count <= 48 ? 6 : 8), row0 = octant * rpt;
+  const int u = min(u0 + lane, H - 1);
   const float bi = __ldg(p.b + u), bo = __ldg(p.b + 3 * H + u), bu = __ldg(p.b + 4 * H + u);
-  for (int r0 = 0; r0 < count; r0 += ROWS) {
-    float acc[RPT][3] = {}, ra[AL], rw[WL];
-    auto fetch = [&](int k0) {
-#pragma unroll
-      for (int j = 0; j < AL; ++j) {
-        const int e = tid + j * kLeafT, i = e / kLeafK, k = min(k0 + e % kLeafK, E - 1);
-        ra[j] = __ldg(p.emb + (size_t)s_tok[min(r0 + i, count - 1)] * E + k);
+  float acc[8][3] = {};
+  bool ok = true;
+  for (int k0 = 0, turn = 0; k0 < E; k0 += kLeafK, ++turn) {
+    const int nk = min(kLeafK, E - k0), pitch = (nk + 3) & ~3;
+    if (turn > 0) {
+      __syncthreads();                                   // the previous indices' readers are done
+      if (tid == 32) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        ask(k0);
       }
-#pragma unroll
-      for (int j = 0; j < WL; ++j) {
-        const int e = tid + j * kLeafT, kk = e / (3 * kLeafU), g = (e / kLeafU) % 3, uu = e % kLeafU;
-        rw[j] = __ldg(p.W + (size_t)min(k0 + kk, E - 1) * 5 * H + (g ? g + 2 : 0) * H + min(u0 + uu, H - 1));
-      }
-    };
-    auto stash = [&](int buf, int k0) {                  // zeros beyond the contraction (other padding is never stored)
-#pragma unroll
-      for (int j = 0; j < AL; ++j) {
-        const int e = tid + j * kLeafT;
-        As[buf][e / kLeafK][e % kLeafK] = k0 + e % kLeafK < E ? ra[j] : 0.f;
-      }
-#pragma unroll
-      for (int j = 0; j < WL; ++j) {
-        const int e = tid + j * kLeafT, kk = e / (3 * kLeafU);
-        Ws[buf][kk][e % (3 * kLeafU)] = k0 + kk < E ? rw[j] : 0.f;
-      }
-    };
-    fetch(0);
-    __syncthreads();                                     // the previous tile's readers are done
-    stash(0, 0);
-    __syncthreads();
-    const int chunks = (E + kLeafK - 1) / kLeafK;
-    for (int ch = 0; ch < chunks; ++ch) {
-      const int buf = ch & 1;
-      if (ch + 1 < chunks) fetch((ch + 1) * kLeafK);
-#pragma unroll
-      for (int kk = 0; kk < kLeafK; kk += 4) {
-        float w[4][3];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int g = 0; g < 3; ++g) w[q][g] = Ws[buf][kk + q][g * kLeafU + tx];
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const float4 a = *reinterpret_cast<const float4*>(&As[buf][ty * RPT + i][kk]);
-#pragma unroll
-          for (int g = 0; g < 3; ++g) {
-            acc[i][g] = fmaf(a.x, w[0][g], acc[i][g]);
-            acc[i][g] = fmaf(a.y, w[1][g], acc[i][g]);
-            acc[i][g] = fmaf(a.z, w[2][g], acc[i][g]);
-            acc[i][g] = fmaf(a.w, w[3][g], acc[i][g]);
-          }
-        }
-      }
-      if (ch + 1 < chunks) stash(buf ^ 1, (ch + 1) * kLeafK);
-      __syncthreads();
     }
+    // rows: a warp takes every 16th; lanes along the row, ten loads in flight; zeros up to the pitch
+    for (int i = warp; i < count; i += kLeafT / 32) {
+      const float* src = p.emb + (size_t)s_tok[i] * E + k0;
+      float v[kLeafK / 32];
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int at = r0 + ty * RPT + i;
-      if (at >= count || u0 + tx >= H) continue;
+      for (int j = 0; j < kLeafK / 32; ++j) v[j] = __ldg(src + min(lane + 32 * j, nk - 1));
+#pragma unroll
+      for (int j = 0; j < kLeafK / 32; ++j)
+        if (lane + 32 * j < pitch) As[i * pitch + lane + 32 * j] = lane + 32 * j < nk ? v[j] : 0.f;
+    }
+    ok = mbar_wait(bar, turn & 1, &s_abort, p.wait_limit, p.st) && ok;
+    // behind the last index, up to a multiple of four: zeros, like the rows' (shared memory may hold anything)
+    if (nk & 3)
+      for (int e = tid; e < (pitch - nk) * 3 * kLeafU; e += kLeafT) Ws[nk * 3 * kLeafU + e] = 0.f;
+    if (__syncthreads_or(!ok)) { ok = false; break; }
+    if (row0 < count) {
+      if (rpt == 4) leaf_rows<4>(As, Ws, pitch, nk, row0, half, lane, acc);
+      else if (rpt == 6) leaf_rows<6>(As, Ws, pitch, nk, row0, half, lane, acc);
+      else leaf_rows<8>(As, Ws, pitch, nk, row0, half, lane, acc);
+    }
+  }
+  if (__syncthreads_or(!ok)) {                           // a wait expired: what was asked for gets a bounded time to land
+    if (tid == 32) { mbar_drain(bar, 0); mbar_drain(bar, 1); }
+    __syncthreads();
+    if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
+  float* const red = Ws;                                 // [row][gate][unit]
+  if (half) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < rpt)
+#pragma unroll
+        for (int g = 0; g < 3; ++g) red[((row0 + i) * 3 + g) * kLeafU + lane] = acc[i][g];
+  }
+  __syncthreads();
+  if (!half && u0 + lane < H) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int at = row0 + i;
+      if (i >= rpt || at >= count) break;
       const int node = s_node[at];
-      const float gi = sigmoid_acc(acc[i][0] + bi), go = sigmoid_acc(acc[i][1] + bo), gu = tanhf(acc[i][2] + bu);
+      const float* r = red + at * 3 * kLeafU + lane;
+      const float gi = sigmoid_acc(acc[i][0] + r[0] + bi), go = sigmoid_acc(acc[i][1] + r[kLeafU] + bo),
+                  gu = tanhf(acc[i][2] + r[2 * kLeafU] + bu);
       const float cv = gi * gu;
       p.c[(size_t)node * H + u] = cv;
       p.h[(size_t)node * H + u] = go * tanhf(cv);
@@ -1068,11 +1115,12 @@ __global__ void k_trees_pairs(int H, ushort2* pairs) {
     for (int c = 0, n = pair_chunks(a, H, Hp); c < n; ++c)
       pairs[at++] = a == 2 * Hp ? make_ushort2(0xFFFF, (unsigned short)(4 * c)) : make_ushort2((unsigned short)a, (unsigned short)(4 * (a / 4 + c)));
 }
-size_t images_bytes(const treelstm* ctx, int what) {     // forward image, backward image, chunk operands
+size_t images_bytes(const treelstm* ctx, int what) {     // forward image, backward image, chunk operands, leaves' weights
   const auto& s = ctx->trees.s;
   const size_t cta = sizeof(float) * (size_t)s.cs;
   return round_up_sz(what == 0 ? cta * kFwdT * fwd_words(ctx->cell) : (what == 1 ? cta * s.bthreads * bwd_words(ctx->cell, s)
-                                                                               : sizeof(ushort2) * (ctx->cell == kRntn ? s.chunks : 0)), 256);
+                                                                               : what == 2 ? sizeof(ushort2) * (ctx->cell == kRntn ? s.chunks : 0)
+                                                                                           : ctx->cell == kLstm ? 4 * leaf_image_words(ctx->H, ctx->E) : 0), 256);
 }
 
 TreesParams trees_params(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
@@ -1142,7 +1190,12 @@ size_t plan_trees(treelstm* ctx) {
     (back ? t.clusters_bwd : t.clusters) = clusters;
   }
   if (!t.ok) { cudaGetLastError(); return 0; }
-  return images_bytes(ctx, 0) + images_bytes(ctx, 1) + images_bytes(ctx, 2);
+  if (cell == kLstm && cudaFuncSetAttribute(k_leaves_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem) != cudaSuccess) {
+    cudaGetLastError();
+    t.ok = false;
+    return 0;
+  }
+  return images_bytes(ctx, 0) + images_bytes(ctx, 1) + images_bytes(ctx, 2) + images_bytes(ctx, 3);
 }
 
 int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream) {
@@ -1151,6 +1204,7 @@ int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream) {
   t.Wf = reinterpret_cast<float*>(memory);
   t.Wb = reinterpret_cast<float*>(memory + images_bytes(ctx, 0));
   t.pairs = reinterpret_cast<ushort2*>(memory + images_bytes(ctx, 0) + images_bytes(ctx, 1));
+  t.Wx = reinterpret_cast<float*>(memory + images_bytes(ctx, 0) + images_bytes(ctx, 1) + images_bytes(ctx, 2));
   if (ctx->cell == kRntn) k_trees_pairs<<<1, 1, 0, stream>>>(ctx->H, t.pairs);
   TL_CUDA(ctx, cudaGetLastError());
   return TREELSTM_OK;
@@ -1164,6 +1218,7 @@ int pack_trees(treelstm* ctx, cudaStream_t stream) {
   const float* src = cell == kLstm ? ctx->W : ctx->Wcat;
   k_trees_pack<<<592, 256, 0, stream>>>(0, cell, H, E, fwd_words(cell), kFwdT, s, t.pairs, src, t.Wf);
   k_trees_pack<<<592, 256, 0, stream>>>(1, cell, H, E, bwd_words(cell, s), s.bthreads, s, t.pairs, src, t.Wb);
+  if (cell == kLstm) k_leaves_pack<<<592, 256, 0, stream>>>(H, E, ctx->W, t.Wx);
   TL_CUDA(ctx, cudaGetLastError());
   return TREELSTM_OK;
 }
@@ -1191,22 +1246,16 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
   p.W = ctx->trees.Wf;
   p.gates = save_gates ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
   if (ctx->cell == kLstm) {
-    LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->W, ctx->b, h, c, p.gates};
-    const int tiles_u = (ctx->H + kLeafU - 1) / kLeafU;
-    const int small = (n + 63) / 64 * tiles_u;           // 32-row tiles until they take several rounds
+    LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->trees.Wx, ctx->b, h, c, p.gates,
+                 p.st, ctx->opt.wait_limit_kcycles * 1024};
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kLeafT); cfg.stream = stream;
+    cfg.gridDim = dim3((n + kLeafIds - 1) / kLeafIds * ((ctx->H + kLeafU - 1) / kLeafU));
+    cfg.blockDim = dim3(kLeafT); cfg.dynamicSmemBytes = kLeafSmem; cfg.stream = stream;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = after_running ? 1 : 0;
     cfg.attrs = &at; cfg.numAttrs = 1;
-    if (small <= 4 * ctx->sm_count) {
-      cfg.gridDim = dim3(small);
-      TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_leaves_fp32<32>, q));
-    } else {
-      cfg.gridDim = dim3((n + 127) / 128 * tiles_u);
-      TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_leaves_fp32<64>, q));
-    }
+    TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_leaves_fp32, q));
     ctx->launches += 1;
   }
   return launch_trees(ctx, forward_kernel(ctx->cell), p, kFwdT, trees_parts(ctx, n, false, after_running), after_running, stream);
