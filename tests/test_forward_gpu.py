@@ -276,3 +276,16 @@ def test_malformed_forests_on_the_scheduling_cluster():
     assert code(cycle) == binding.ERR_INVALID_FOREST
     assert code(token) == binding.ERR_TOKEN_OUT_OF_RANGE
     util.gpu_forward(model, base, binding.PERSISTENT)
+
+
+@pytest.mark.parametrize("H,E,kind", [(32, 320, "leaves"), (33, 321, "leaves"), (31, 5, "half"), (150, 319, "most"), (64, 643, "half"), (1, 1, "leaves")])
+def test_fp32_leaves_at_the_limits_of_their_tiles(H, E, kind):
+    """the leaves' kernel: 64 leaves, 33 to 48 and at most 32 of them among 64 consecutive ids, contractions of one, of exactly one
+    full, of just over one and of three loads of the operands, slices of 32 units with one unit more or less"""
+    rng = np.random.default_rng(H + E)
+    params = fg.draw_params(rng, H, E, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.1)
+    shapes = {"leaves": [None] * 193, "half": [fg.balanced_shape(32)] * 3 + [None], "most": [None, fg.left_chain_shape(4), None] * 25}[kind]
+    forest = fg.forest_from_shapes(shapes, rng, 60)
+    res = util.gpu_forward(util.make_model(params, "fp32"), forest, binding.PERSISTENT)
+    h, c, _ = orc.forward_recursive(forest.left, forest.right, forest.token, params.emb, params.W, params.b)
+    assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
