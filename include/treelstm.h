@@ -130,8 +130,9 @@ typedef enum treelstm_status {
                                             /* order of work of the cooperative launch: their scheduler    */
                                             /* is too short to hide the two extra grid barriers            */
 #define TREELSTM_OPT_DW_TENSOR_CORES 10     /* 1 (default): after a forward that kept its level table on   */
-                                            /* the device, treelstm_backward forms dW, db and the input    */
-                                            /* gradients of the leaves (dEmb_rows) in a second kernel on   */
+                                            /* the device, treelstm_backward forms dW, db, the input       */
+                                            /* gradients of the leaves (dEmb_rows) and, in forests with    */
+                                            /* wide wavefronts, all input gradients in kernels on          */
                                             /* the tensor cores, every fp32 operand split into three bf16  */
                                             /* pieces (six products per term: fp32 accuracy); 0: fp32      */
                                             /* multiply-adds inside the one-launch backward                */
@@ -254,10 +255,11 @@ TREELSTM_API int treelstm_roots(treelstm_t* ctx, int max_roots, int32_t* root_id
  *                Rows past n_touched are unspecified.
  * The forest arrays, h, c, order, level and the workspace of the forward call must still be
  * valid and unchanged.  After a TREELSTM_PERSISTENT or TREELSTM_SUBFORESTS forward the loss and all
- * wavefronts are one cooperative launch that reads the level table on the device (asynchronous, no
- * host round trip; a label out of range is reported by treelstm_status_sync), followed - unless
- * TREELSTM_OPT_DW_TENSOR_CORES is 0 - by one tensor-core launch for dW, db and dEmb_rows (their sums
- * run over all nodes and depend on no wavefront order); after a TREELSTM_PER_LEVEL forward it is one
+ * wavefronts run from the level table on the device (asynchronous, no host round trip; a label out of range
+ * is reported by treelstm_status_sync): with TREELSTM_OPT_DW_TENSOR_CORES = 0 as one cooperative launch, else
+ * as one for the loss, one per way of walking the wavefronts (trees dealt to clusters, or all wavefronts over
+ * the whole GPU on the tensor cores; the one that does not apply exits at once) and a tensor-core launch for
+ * dW, db and dEmb_rows (their sums run over all nodes and depend on no wavefront order); after a TREELSTM_PER_LEVEL forward it is one
  * launch pair per wavefront, driven by the level table the forward already read back.  Computes at
  * fp32 accuracy from the fp32 parameters whatever the forward precision.
  */
@@ -276,9 +278,9 @@ TREELSTM_API int treelstm_backward(treelstm_t* ctx, const int32_t* labels, float
  *   labels, loss, dWc [H][C], dbc [C], touched_ids, n_touched: as for treelstm_backward.
  *   dW [2H][H], db [H]  out;  dV [H][2H][2H] out (RNTN; may be NULL for TreeRNN);
  *   dEmb_rows [n_leaves][H] out: one summed row per touched id.
- * All device pointers; gradients are overwritten.  The level table is read back once (the call
- * synchronises the stream of the forward if that was a TREELSTM_PERSISTENT one), then one launch per
- * phase and wavefront; fp32.  Errors: as treelstm_backward; TREELSTM_ERR_STATE on a TreeLSTM context
+ * All device pointers; gradients are overwritten; fp32.  Up to H = 256 (TreeRNN) and H = 32 (RNTN), after a
+ * TREELSTM_PERSISTENT forward, three launches without a host round trip; else the level table is read back
+ * once (the call synchronises the stream of the forward), then one launch per phase and wavefront.  Errors: as treelstm_backward; TREELSTM_ERR_STATE on a TreeLSTM context
  * (and treelstm_backward returns it on a TreeRNN / RNTN context).
  */
 TREELSTM_API int treelstm_backward_recursive(treelstm_t* ctx, const int32_t* labels, float* loss, float* dW,
