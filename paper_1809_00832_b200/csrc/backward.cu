@@ -998,14 +998,13 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
 }
 
 // ---- the wavefronts of a forest that is wide, on the tensor cores ------------------------------ //
-// Behind k_bwd_begin, for the forests that trees_pay() leaves.  A wavefront of more than kFusedMaxRows nodes is
-// dIn = dz W^T with hundreds of rows: on fp32 units that contraction was 600 of the 880 us of the backward pass of
-// 14.6 k nodes (H = 256).  Here its dz is written as split bf16 pieces (BwdImages, the layout the tensor core reads),
-// and tiles of 128 positions x 128 outputs are multiplied with W split once per set of weights: one thread asks for
-// blocks (plain bulk copies of whole tiles), one issues the MMAs, eight warps add the tile to the children's dh.  The
-// contraction is cut into as many pieces as leave no CTA without a tile.  The leaves' dIn (their rows of dEmb) is one
-// more such wavefront.  Narrow wavefronts form their gate gradients inside an fp32 contraction as in k_bwd_persistent.
-// The images stay for the weight gradient.
+// Behind k_bwd_begin, for the forests that trees_pay() leaves.  On fp32 units the contraction dIn = dz W^T of the wide
+// wavefronts was 600 of the 880 us of the backward pass of 14.6 k nodes (H = 256).  Here dz is split into bf16 pieces
+// (BwdImages, the layout the tensor core reads), and tiles of 128 positions x 128 outputs are multiplied with W split once
+// per set of weights: one thread asks for blocks (plain bulk copies of whole tiles), one issues the MMAs, sixteen warps
+// add the tile to the children's dh.  The leaves' dIn (their rows of dEmb) is one more such wavefront.  The images stay for the weight
+// gradient.  What is left is latency: 10 - 14 k cycles of a narrow wavefront (3.3 k grid barrier, 3.5 k gate gradients, 2.5 k MMAs, 4 k
+// adds), 30 k of one of 300 nodes, 70 k of one of 2.5 k; 315 us in all for 14.6 k nodes, 19 wavefronts.
 constexpr int kWideSmem = 2 * kSpStageBytes + 1024, kWideThreads = 512;
 constexpr int kDirectRows = 256, kWideOffCache = 512;
 struct WideArgs {
