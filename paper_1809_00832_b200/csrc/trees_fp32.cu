@@ -524,10 +524,12 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
 // kLeafK contraction indices are asked for at once - the weights as one bulk copy out of an image kept for it, the
 // embedding rows through registers - because the kernel is bound by the latency of its loads: in chunks of 32 indices,
 // each a round trip behind the one before, 25 trees (H = 150, E = 300) took 43 us with cold caches, this way 28.
-// A warp takes RPT rows and half of the contraction (rows read as broadcasts, weights one word per lane), as many rows
-// as give 16 warps one turn each; the halves meet in shared memory.
+// A warp takes a quarter of the rows (8, 10, 12 or 16) and a quarter of the contraction: rows read as broadcasts, weights one
+// word per lane, 96 multiply-adds per 20 reads.  (Half of the rows and twice the quarters of the contraction, 48 per 16 reads,
+// was bound by shared memory: 15 k cycles for 32 leaves.)  The quarters meet in shared memory, every warp finishes some rows.
 constexpr int kLeafT = 512, kLeafU = 32, kLeafIds = 64, kLeafK = 320;
 constexpr int kLeafSmem = 4 * kLeafK * (3 * kLeafU + kLeafIds);
+static_assert(4 * kLeafIds <= kLeafK, "the sums of the quarters fit where the weights were");
 struct LeafParams {
   int n, H, E, vocab;
   int* chk_counts;
@@ -546,11 +548,12 @@ __global__ void k_leaves_pack(int H, int E, const float* W, float* out) {
     out[i] = u < H ? W[(size_t)k * 5 * H + (g ? g + 2 : 0) * H + u] : 0.f;
   }
 }
-// RPT rows from `rows` on and half of nk contraction indices
+// RPT rows from `rows` on and a quarter of nk contraction indices
 template <int RPT>
-__device__ __forceinline__ void leaf_rows(const float* As, const float* Ws, int pitch, int nk, int rows, int half, int lane, float (&acc)[8][3]) {
-  const int mid = (nk / 2 + 3) & ~3, lo = half ? mid : 0, hi = half ? (nk + 3) & ~3 : mid;
-#pragma unroll 2
+__device__ __forceinline__ void leaf_rows(const float* As, const float* Ws, int pitch, int nk, int rows, int quarter, int lane,
+                                          float (&acc)[16][3]) {
+  const int per = (nk + 15) / 16 * 4, lo = quarter * per, hi = min(lo + per, (nk + 3) & ~3);
+#pragma unroll 1
   for (int k = lo; k < hi; k += 4) {
     float w[4][3];
 #pragma unroll
@@ -609,11 +612,11 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
     if (tid == 0) s_count = count;
   }
   __syncthreads();
-  const int count = s_count, octant = warp & 7, half = warp >> 3;
-  const int rpt = count <= 32 ? 4 : (count <= 48 ? 6 : 8), row0 = octant * rpt;
+  const int count = s_count, quarter = warp >> 2;
+  const int rpt = count <= 32 ? 8 : (count <= 40 ? 10 : (count <= 48 ? 12 : 16)), row0 = (warp & 3) * rpt;
   const int u = min(u0 + lane, H - 1);
   const float bi = __ldg(p.b + u), bo = __ldg(p.b + 3 * H + u), bu = __ldg(p.b + 4 * H + u);
-  float acc[8][3] = {};
+  float acc[16][3] = {};
   bool ok = true;
   for (int k0 = 0, turn = 0; k0 < E; k0 += kLeafK, ++turn) {
     const int nk = min(kLeafK, E - k0), pitch = (nk + 3) & ~3;
@@ -640,9 +643,10 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
       for (int e = tid; e < (pitch - nk) * 3 * kLeafU; e += kLeafT) Ws[nk * 3 * kLeafU + e] = 0.f;
     if (__syncthreads_or(!ok)) { ok = false; break; }
     if (row0 < count) {
-      if (rpt == 4) leaf_rows<4>(As, Ws, pitch, nk, row0, half, lane, acc);
-      else if (rpt == 6) leaf_rows<6>(As, Ws, pitch, nk, row0, half, lane, acc);
-      else leaf_rows<8>(As, Ws, pitch, nk, row0, half, lane, acc);
+      if (rpt == 8) leaf_rows<8>(As, Ws, pitch, nk, row0, quarter, lane, acc);
+      else if (rpt == 10) leaf_rows<10>(As, Ws, pitch, nk, row0, quarter, lane, acc);
+      else if (rpt == 12) leaf_rows<12>(As, Ws, pitch, nk, row0, quarter, lane, acc);
+      else leaf_rows<16>(As, Ws, pitch, nk, row0, quarter, lane, acc);
     }
   }
   if (__syncthreads_or(!ok)) {                           // a wait expired: what was asked for gets a bounded time to land
@@ -651,24 +655,24 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
     if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
-  float* const red = Ws;                                 // [row][gate][unit]
-  if (half) {
+  float* const red = Ws;                                 // [quarter][row][gate][unit]
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (i < rpt)
+  for (int i = 0; i < 16; ++i)
+    if (i < rpt)
 #pragma unroll
-        for (int g = 0; g < 3; ++g) red[((row0 + i) * 3 + g) * kLeafU + lane] = acc[i][g];
-  }
+      for (int g = 0; g < 3; ++g) red[((quarter * kLeafIds + row0 + i) * 3 + g) * kLeafU + lane] = acc[i][g];
   __syncthreads();
-  if (!half && u0 + lane < H) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int at = row0 + i;
-      if (i >= rpt || at >= count) break;
+  if (u0 + lane < H) {
+    for (int at = warp; at < count; at += kLeafT / 32) {
       const int node = s_node[at];
-      const float* r = red + at * 3 * kLeafU + lane;
-      const float gi = sigmoid_acc(acc[i][0] + r[0] + bi), go = sigmoid_acc(acc[i][1] + r[kLeafU] + bo),
-                  gu = tanhf(acc[i][2] + r[2 * kLeafU] + bu);
+      float z[3];
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        const float* r = red + (at * 3 + g) * kLeafU + lane;
+        constexpr int kq = kLeafIds * 3 * kLeafU;
+        z[g] = (r[0] + r[kq]) + (r[2 * kq] + r[3 * kq]);
+      }
+      const float gi = sigmoid_acc(z[0] + bi), go = sigmoid_acc(z[1] + bo), gu = tanhf(z[2] + bu);
       const float cv = gi * gu;
       p.c[(size_t)node * H + u] = cv;
       p.h[(size_t)node * H + u] = go * tanhf(cv);
