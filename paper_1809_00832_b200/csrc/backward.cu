@@ -1356,15 +1356,16 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
           TL_STAMP(trace, lvl, 7);          // a tile's gate gradients formed
         }
         fetched = false;
-        if (tid == 32) {
+        if (warp == 1) {
+          const bool issue = elect_one();
           for (int k = 0; k < nk && ok; ++k) {
             const uint32_t b = blk + k, stage = b & 1u, src = tiles_addr + stage * kSpStageBytes;
-            ok = mbar_wait(full0 + 8 * stage, (b >> 1) & 1u, &s_abort, a.wait_limit, p.st);
+            ok = __all_sync(kFull, mbar_wait(full0 + 8 * stage, (b >> 1) & 1u, &s_abort, a.wait_limit, p.st));
             if (!ok) break;
             tc_fence_after();
-            split_mmas(tmem_base, src, src + kSpOperandBytes, umma_idesc(kSpTile), k == 0);
-            umma_commit(empty0 + 8 * stage);
-            if (k == nk - 1) umma_commit(acc_bar);
+            split_mmas(tmem_base, src, src + kSpOperandBytes, umma_idesc(kSpTile), k == 0, issue);
+            if (issue) umma_commit(empty0 + 8 * stage);
+            if (issue && k == nk - 1) umma_commit(acc_bar);
           }
         }
         __syncwarp();
@@ -1445,7 +1446,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   TL_STAMP(trace, kTraceLevels - 1, 1);
   tc_fence_before();
   if (__syncthreads_or(!ok)) {                           // what was asked for gets a bounded time to land, the MMAs to retire
-    if (tid == 32) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
+    if (warp == 1 && elect_one()) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
     if (tid == 0)
       for (uint32_t s = 0; s < 2; ++s) {
         const uint32_t times = (asked + 1 - s) / 2;      // how often stage s was filled

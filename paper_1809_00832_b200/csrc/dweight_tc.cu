@@ -206,15 +206,16 @@ __device__ void dw_from_images(const DwParams& p, int n_leaves, unsigned char* t
         bulk_load(dst, xi + (pb * xu[part] + 2 * mt) * kUnitBytes, (uint32_t)ma * kUnitBytes, bar);
         bulk_load(dst + kSpOperandBytes, p.img.dz + (pb * ju + 2 * nt) * kUnitBytes, (uint32_t)mb * kUnitBytes, bar);
       }
-    } else if (tid == 32) {
+    } else if (warp == 1) {
+      const bool issue = elect_one();
       for (int b = 0; b < nblk && ok; ++b, ++got) {
         const uint32_t stage = got & 1u, src = tiles_addr + stage * kDwStageBytes;
-        ok = mbar_wait(full_bar0 + 8 * stage, (got >> 1) & 1u, s_abort, p.wait_limit, p.st);
+        ok = __all_sync(0xffffffffu, mbar_wait(full_bar0 + 8 * stage, (got >> 1) & 1u, s_abort, p.wait_limit, p.st));
         if (!ok) break;
         tc_fence_after();
-        split_mmas_mn(tmem_base, src, src + kSpOperandBytes, idesc, b == 0);
-        umma_commit(empty_bar0 + 8 * stage);
-        if (b == nblk - 1) umma_commit(acc_bar);
+        split_mmas_mn(tmem_base, src, src + kSpOperandBytes, idesc, b == 0, issue);
+        if (issue) umma_commit(empty_bar0 + 8 * stage);
+        if (issue && b == nblk - 1) umma_commit(acc_bar);
       }
     }
     __syncwarp();
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
     tc_fence_before();
     __syncthreads();
     if (s_abort) {                         // what was asked for gets a bounded time to land, the MMAs a bounded time to retire
-      if (tid == 32) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
+      if (warp == 1 && elect_one()) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
       if (tid == 0) for (int s = 0; s < kDwStages; ++s) mbar_drain(stage_bar0 + 8 * s, 0);
       __syncthreads();
     }
@@ -390,12 +391,13 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the tensor core
       tc_fence_before();
       __syncthreads();
-      if (tid == 0) {
+      if (warp == 0) {
+        const bool issue = elect_one();
         tc_fence_after();
         const uint32_t a_addr = tiles_addr + stage * kDwStageBytes;
-        split_mmas(tmem_base, a_addr, a_addr + kSpOperandBytes, idesc, b == 0);
-        umma_commit(stage_bar0 + 8 * stage);
-        if (b == nblk - 1) umma_commit(acc_bar);
+        split_mmas(tmem_base, a_addr, a_addr + kSpOperandBytes, idesc, b == 0, issue);
+        if (issue) umma_commit(stage_bar0 + 8 * stage);
+        if (issue && b == nblk - 1) umma_commit(acc_bar);
       }
     }
     if (failed) break;
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
   // teardown: MMAs still in flight after a failed wait get a bounded time to retire before tensor memory goes back
   tc_fence_before();
   __syncthreads();
-  if (failed && tid == 0) {
+  if (failed && warp == 0 && elect_one()) {
     umma_commit(drain_bar);
     mbar_drain(drain_bar, 0);
   }

@@ -39,14 +39,14 @@ __device__ __forceinline__ void split_store8(unsigned char* tiles, int r, int c,
   *reinterpret_cast<uint4*>(dst + kSpTileBytes) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
   *reinterpret_cast<uint4*>(dst + 2 * kSpTileBytes) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
 }
-// The MMAs of one block (one thread): (piece of A, piece of B), the small products first.
-__device__ __forceinline__ void split_mmas(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc, bool first_block) {
+// The MMAs of one block (a whole warp, issued by its elected lane): (piece of A, piece of B), the small products first.
+__device__ __forceinline__ void split_mmas(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc, bool first_block, bool issue) {
 #pragma unroll
   for (int k = 0; k < kSpBlock / 16; ++k)     // UMMA K = 16 bf16 = 32 bytes = 2 descriptor units
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
       const int pa = (0x010120 >> (4 * q)) & 0xF, pb = (0x001102 >> (4 * q)) & 0xF;
-      umma_bf16(d_tmem, umma_desc(a_addr + pa * kSpTileBytes) + 2 * k, umma_desc(b_addr + pb * kSpTileBytes) + 2 * k, idesc,
+      if (issue) umma_bf16(d_tmem, umma_desc(a_addr + pa * kSpTileBytes) + 2 * k, umma_desc(b_addr + pb * kSpTileBytes) + 2 * k, idesc,
                 !(first_block && k == 0 && q == 0));
     }
 }
@@ -99,13 +99,13 @@ __device__ __forceinline__ uint64_t umma_desc_mn(uint32_t smem_addr) {
 }
 __device__ __forceinline__ uint32_t umma_idesc_mn(int n) { return umma_idesc(n) | (1u << 15) | (1u << 16); }
 // one block (64 positions) of In^T dz: both operands MN-major, [unit][piece] in shared memory
-__device__ __forceinline__ void split_mmas_mn(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc, bool first_block) {
+__device__ __forceinline__ void split_mmas_mn(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc, bool first_block, bool issue) {
 #pragma unroll
   for (int k = 0; k < 4; ++k)            // 16 positions = two groups of eight
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
       const int pa = (0x010120 >> (4 * q)) & 0xF, pb = (0x001102 >> (4 * q)) & 0xF;
-      umma_bf16(d_tmem, umma_desc_mn(a_addr + pa * kUnitPieceBytes) + 128 * k, umma_desc_mn(b_addr + pb * kUnitPieceBytes) + 128 * k,
+      if (issue) umma_bf16(d_tmem, umma_desc_mn(a_addr + pa * kUnitPieceBytes) + 128 * k, umma_desc_mn(b_addr + pb * kUnitPieceBytes) + 128 * k,
                 idesc, !(first_block && k == 0 && q == 0));
     }
 }

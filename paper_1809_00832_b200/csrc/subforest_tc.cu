@@ -266,25 +266,25 @@ k_fwd_tc_subforest(const __grid_constant__ TmapSet maps, const __grid_constant__
           alive = __shfl_sync(kFullMask, (int)alive, 0) != 0;
         } else if (warp == 5) {
           // ---------------- MMA issuer ----------------
-          if (lane == 0) {
+          {
+            const bool issue = elect_one();
             const uint32_t acc = acc_iter & 1, acc_phase = (acc_iter >> 1) & 1;
-            if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1, s_abort, p.wait_limit, p.st)) alive = false;
+            alive = mbar_wait(tempty_bar(acc), acc_phase ^ 1, s_abort, p.wait_limit, p.st) && alive;
             if (!leaf && !wres_ready) {
-              if (!mbar_wait(wres_bar, 0, s_abort, p.wait_limit, p.st)) alive = false;
+              alive = mbar_wait(wres_bar, 0, s_abort, p.wait_limit, p.st) && alive;
               wres_ready = true;
             }
+            alive = __all_sync(kFullMask, alive);
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * kAccCols;
             const uint32_t idesc = umma_idesc(ncols_mma);
             bool first = true;
             for (int box = 0; box < n_box && alive; ++box) {
-              if (!mbar_wait(full_bar(stage), (phase_bits >> stage) & 1u, s_abort, p.wait_limit, p.st)) {
-                alive = false;
-                break;
-              }
+              alive = __all_sync(kFullMask, mbar_wait(full_bar(stage), (phase_bits >> stage) & 1u, s_abort, p.wait_limit, p.st));
+              if (!alive) break;
               tc_fence_after();
 #ifdef TREELSTM_TRACE
-              if (t == 0 && box == 0) TL_STAMP(trace, lvl, 2);
+              if (t == 0 && box == 0 && lane == 0) TL_STAMP(trace, lvl, 2);
 #endif
               const uint32_t st_addr = ring_addr + stage * stage_bytes;
               const int nkb = min(kbox, kblocks - box * kbox);
@@ -294,16 +294,16 @@ k_fwd_tc_subforest(const __grid_constant__ TmapSet maps, const __grid_constant__
                 const uint64_t a_desc = umma_desc(st_addr + (uint32_t)kbi * a_bytes), b_desc = umma_desc(b_addr);
 #pragma unroll
                 for (int k = 0; k < kKBlock / 16; ++k)   // UMMA K = 16 bf16 = 32 bytes = 2 descriptor units
-                  umma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, !(first && k == 0));
+                  if (issue) umma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, !(first && k == 0));
                 first = false;
               }
-              umma_commit(empty_bar(stage));             // frees the ring stage when these MMAs retire
+              if (issue) umma_commit(empty_bar(stage));  // frees the ring stage when these MMAs retire
               phase_bits ^= 1u << stage;
               if (++stage == n_stages) stage = 0;
             }
-            if (alive) umma_commit(tfull_bar(acc));      // the accumulator is complete
+            if (alive && issue) umma_commit(tfull_bar(acc));   // the accumulator is complete
 #ifdef TREELSTM_TRACE
-            if (t == tiles - 1) TL_STAMP(trace, lvl, 3);
+            if (t == tiles - 1 && lane == 0) TL_STAMP(trace, lvl, 3);
 #endif
           }
           ++acc_iter;
@@ -380,7 +380,7 @@ k_fwd_tc_subforest(const __grid_constant__ TmapSet maps, const __grid_constant__
       for (uint32_t s = 0; s < (uint32_t)kMaxStages; ++s)
         if (armed & (1u << s)) mbar_drain(full_bar(s), ((phase_bits >> s) & 1u) ^ 1u);
     }
-    if (warp == 5 && lane == 0) {
+    if (warp == 5 && elect_one()) {                  // (a commit covers the MMAs of the thread that makes it)
       umma_commit(drain_bar);
       mbar_drain(drain_bar, 0);
     }

@@ -383,31 +383,31 @@ k_fwd_tc_tail(const __grid_constant__ TmapSet maps, const __grid_constant__ SfTm
       }
     } else if (warp == 9) {
       // ---------------- MMA issuer ----------------
-      if (lane == 0) {
-        if (i == 0 && !mbar_wait(Wb, 0, s_abort, p.wait_limit, p.st)) alive = false;
-        if (alive && !mbar_wait(TLb(cur), use, s_abort, p.wait_limit, p.st)) alive = false;
-        if (alive && !mbar_wait_cluster(XFb(cur), use, s_abort, p.wait_limit, p.st)) alive = false;
-        if (alive && i > 0 && !mbar_wait(TEb, (uint32_t)(i - 1) & 1u, s_abort, p.wait_limit, p.st)) alive = false;
-        if (alive) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // pushed pieces are read by the tensor core
-          tc_fence_after();
+      const bool issue = elect_one();
+      if (i == 0) alive = mbar_wait(Wb, 0, s_abort, p.wait_limit, p.st);
+      alive = alive && mbar_wait(TLb(cur), use, s_abort, p.wait_limit, p.st);
+      alive = alive && mbar_wait_cluster(XFb(cur), use, s_abort, p.wait_limit, p.st);
+      if (i > 0) alive = alive && mbar_wait(TEb, (uint32_t)(i - 1) & 1u, s_abort, p.wait_limit, p.st);
+      alive = __all_sync(kFullMask, alive);
+      if (alive) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // pushed pieces are read by the tensor core
+        tc_fence_after();
 #ifdef TREELSTM_TRACE
-          TL_STAMP(trace, first_level + i, 2);
+        if (lane == 0) TL_STAMP(trace, first_level + i, 2);
 #endif
-          const uint32_t idesc = umma_idesc(n_pad);
-          const uint32_t x_addr = base + L.xop + (uint32_t)cur * L.xop_bytes;
-          for (int kb = 0; kb < kb_int; ++kb) {
-            const uint64_t a_desc = umma_desc(wres_addr + (uint32_t)kb * (uint32_t)m_rows * 128u);
-            const uint64_t b_desc = umma_desc(x_addr + (uint32_t)kb * (uint32_t)kTailRows * 128u);
+        const uint32_t idesc = umma_idesc(n_pad);
+        const uint32_t x_addr = base + L.xop + (uint32_t)cur * L.xop_bytes;
+        for (int kb = 0; kb < kb_int; ++kb) {
+          const uint64_t a_desc = umma_desc(wres_addr + (uint32_t)kb * (uint32_t)m_rows * 128u);
+          const uint64_t b_desc = umma_desc(x_addr + (uint32_t)kb * (uint32_t)kTailRows * 128u);
 #pragma unroll
-            for (int k = 0; k < kKBlock / 16; ++k)
-              umma_bf16(tmem_base, a_desc + 2 * k, b_desc + 2 * k, idesc, !(kb == 0 && k == 0));
-          }
-          umma_commit(TFb);
-#ifdef TREELSTM_TRACE
-          TL_STAMP(trace, first_level + i, 3);
-#endif
+          for (int k = 0; k < kKBlock / 16; ++k)
+            if (issue) umma_bf16(tmem_base, a_desc + 2 * k, b_desc + 2 * k, idesc, !(kb == 0 && k == 0));
         }
+        if (issue) umma_commit(TFb);
+#ifdef TREELSTM_TRACE
+        if (lane == 0) TL_STAMP(trace, first_level + i, 3);
+#endif
       }
     } else if (warp >= 10) {
       // ---------------- tables and older child cell states of the next wavefront ----------------
@@ -597,7 +597,7 @@ k_fwd_tc_tail(const __grid_constant__ TmapSet maps, const __grid_constant__ SfTm
   if (*s_abort) {
     // a wait expired: give what was requested a bounded time to land, the MMAs a bounded time to retire
     if (warp == 8 && lane == 0) { mbar_drain(Wb, 0); }
-    if (warp == 9 && lane == 0) { umma_commit(drainb); mbar_drain(drainb, 0); }
+    if (warp == 9 && elect_one()) { umma_commit(drainb); mbar_drain(drainb, 0); }   // (by the thread that issued the MMAs)
     __syncthreads();
   }
   // no CTA may leave while a peer can still write into its shared memory or signal its barriers
