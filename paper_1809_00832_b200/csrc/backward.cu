@@ -1252,7 +1252,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   }
   const int n_levels = p.st->n_levels, n = p.n, H = p.H, E = p.E, gp = gate_pitch(H), ju = img_units(5 * gp);
   for (int l = tid; l < kWideOffCache && l <= n_levels; l += kWideThreads) s_off[l] = a.level_offset[l];
-  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kSpTile);
+  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kSpTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1380,16 +1380,13 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
         {
           const int quad = warp & 3, quarter = warp >> 2;
           const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(quarter * 32);
-          uint32_t v[32];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
-          tmem_ld_wait();
+          float v[32];
+          split_sum(taddr, v);
           tc_fence_before();
           float* dst = stage_out + (size_t)(quad * 32 + lane) * kRowStride + quarter * 32;
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
-                                                                  __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+            *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
         __syncthreads();
         TL_STAMP(trace, lvl, 6);            // and read back
@@ -1456,7 +1453,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   }
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kSpTile);
+    tmem_dealloc(tmem_base, kSpTmemCols);
   }
 }
 

@@ -226,18 +226,15 @@ __device__ void dw_from_images(const DwParams& p, int n_leaves, unsigned char* t
     {
       const int quad = warp & 3, quarter = warp >> 2;
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(quarter * 32);
-      uint32_t v[32];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
-      tmem_ld_wait();
+      float v[32];
+      split_sum(taddr, v);
       tc_fence_before();
       constexpr int kRowStride = kDwTile + 4;
       float* stage_out = reinterpret_cast<float*>(tiles);   // both stages are idle: every block asked for has been multiplied
       float* dst = stage_out + (size_t)(quad * 32 + lane) * kRowStride + quarter * 32;
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
-                                                              __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+        *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
       __syncthreads();
       const int rows = part ? 2 * H : E, m0 = mt * kDwTile;
       auto column = [&](int c) {                              // of dW; none behind a gate's last unit
@@ -288,7 +285,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kDwTile);   // 128 columns: one 128 x 128 fp32 accumulator
+  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kSpTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -306,7 +303,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
     }
     if (warp == 0) {
       tc_fence_after();
-      tmem_dealloc(tmem_base, kDwTile);
+      tmem_dealloc(tmem_base, kSpTmemCols);
     }
     return;
   }
@@ -412,16 +409,13 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
       const int quad = warp & 3, quarter = warp >> 2;       // a warp reads the tensor-memory lanes of quadrant (warp id mod 4)
       const int r = quad * 32 + lane;
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(quarter * 32);
-      uint32_t v[32];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) tmem_ld4(taddr + 4 * i, v + 4 * i);
-      tmem_ld_wait();
+      float v[32];
+      split_sum(taddr, v);
       tc_fence_before();
       float* dst = stage_out + (size_t)r * kRowStride + quarter * 32;
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
-                                                              __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+        *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
     }
     __syncthreads();
     const int rows_valid = part < 2 ? min(kDwTile, sh.rows[part] + 1 - m0) : rows_here;
@@ -452,7 +446,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kDwTile);
+    tmem_dealloc(tmem_base, kSpTmemCols);
   }
 }
 
