@@ -578,7 +578,7 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
           alive = __all_sync(kFullMask, mbar_wait(tempty_bar(acc), acc_phase ^ 1, s_abort, p.wait_limit, p.st) && alive);
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + acc * kAccCols;
-          const uint32_t idesc = umma_idesc(ncols_mma);
+          const uint32_t idesc = umma_idesc(ncols_mma, rt < BM ? 64 : BM);
           bool first = true;
           for (int box = 0; box < n_box && alive; ++box) {
             alive = __all_sync(kFullMask, mbar_wait(full_bar(stage), (phase_bits >> stage) & 1u, s_abort, p.wait_limit, p.st));
@@ -609,8 +609,11 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
         // warp may only read the tensor-memory lanes of quadrant (warp id mod 4).
         const int e = warp < 4 ? 0 : 1;   // warps 0-3: set 0, warps 6-9: set 1
         const int quad = warp & 3;
-        const int r = quad * 32 + lane;
-        const int row = row0 + r;
+        // An MMA is bound by the reads of its operands (4 KB of rows at M = 128: 48 cycles), so tiles of 32 or 64 rows are
+        // computed with M = 64 (33 cycles alone): 16 rows per quadrant, the other lanes idle (rows behind the tile's).
+        const int r = quad * 32 + lane;               // tensor-memory lane and staging row
+        const int tr = rt == BM ? r : quad * 16 + (lane & 15) + (lane & 16) * 4;   // row of the tile
+        const int row = row0 + tr;
         const bool valid = row < row_end;
         int node, slot;                               // slot: 2 * pos(caller) + side, -1 for a root
         if (nx_have) {
@@ -625,8 +628,8 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
         bool valid2 = false;
         if (nx_have) {
           const int fat2 = t2 < plan.tail_from ? t2 : plan.tail_from + ((t2 - plan.tail_from) >> plan.tail_ls);
-          const int rtile2 = fat2 / ntn, row2 = begin + (rtile2 << plan.lrt) + r;
-          valid2 = r < rt && row2 < end;
+          const int rtile2 = fat2 / ntn, row2 = begin + (rtile2 << plan.lrt) + tr;
+          valid2 = tr < rt && row2 < end;
           nx_node = valid2 ? chk(p.st, order_cur[row2], p.n) : 0;
         }
         EpiTile et;
