@@ -390,7 +390,7 @@ __device__ __forceinline__ bool grid_barrier_with(DevStatus* st, unsigned int ta
     if (lane < 8) {
       const long long t0 = clock64();
       while (clock64() - t0 < 150 * lane) {}
-      for (;;) {
+      for (int turn = 1;; ++turn) {
         if (*(volatile int*)s_flag >= 0) break;          // another lane has the answer
         unsigned int seen;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
@@ -399,7 +399,7 @@ __device__ __forceinline__ bool grid_barrier_with(DevStatus* st, unsigned int ta
           *(volatile int*)s_flag = 1;
           break;
         }
-        if (*(volatile int*)&st->status != 0) {
+        if ((turn & 15) == 0 && *(volatile int*)&st->status != 0) {   // (a round trip of its own: not on every turn)
           if (s_early) *(volatile unsigned int*)s_early = 0xFFFFFFFFu;
           *(volatile int*)s_flag = 0;
           break;
