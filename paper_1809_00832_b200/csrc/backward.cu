@@ -1004,7 +1004,7 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
 // per set of weights: one thread asks for blocks (plain bulk copies of whole tiles), one issues the MMAs, sixteen warps
 // add the tile to the children's dh.  The leaves' dIn (their rows of dEmb) is one more such wavefront.  The images stay for the weight
 // gradient.  What is left is latency: 10 - 14 k cycles of a narrow wavefront (3.3 k grid barrier, 3.5 k gate gradients, 2.5 k MMAs, 4 k
-// adds), 30 k of one of 300 nodes, 70 k of one of 2.5 k; 315 us in all for 14.6 k nodes, 19 wavefronts.
+// adds), 30 k of one of 300 nodes, 70 k of one of 2.5 k; 340 us in all (ncu, cold caches) for 14.6 k nodes, 19 wavefronts.
 constexpr int kWideSmem = 2 * kSpStageBytes + 1024, kWideThreads = 512;
 constexpr int kDirectRows = 256, kWideOffCache = 512;
 struct WideArgs {

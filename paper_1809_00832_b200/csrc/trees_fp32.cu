@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
 // ids, the leaves among them (about half), and 32 hidden units x the three gates a leaf has.  All operands of
 // kLeafK contraction indices are asked for at once - the weights as one bulk copy out of an image kept for it, the
 // embedding rows through registers - because the kernel is bound by the latency of its loads: in chunks of 32 indices,
-// each a round trip behind the one before, 25 trees (H = 150, E = 300) took 43 us with cold caches, this way 28.
+// each a round trip behind the one before, 25 trees (H = 150, E = 300) took 43 us with cold caches, this way 17.
 // A warp takes a quarter of the rows (8, 10, 12 or 16) and a quarter of the contraction: rows read as broadcasts, weights one
 // word per lane, 96 multiply-adds per 20 reads.  (Half of the rows and twice the quarters of the contraction, 48 per 16 reads,
 // was bound by shared memory: 15 k cycles for 32 leaves.)  The quarters meet in shared memory, every warp finishes some rows.
