@@ -971,7 +971,9 @@ __global__ void __launch_bounds__(kGT) k_rec_grads(GradParams p) {
   __shared__ int s_a[GR], s_b[GR];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = p.H, K = p.K;
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (p.st->n_levels < 1 || (ld_volatile(&p.st->status) != 0 && ld_volatile(&p.st->status) != TREELSTM_ERR_LABEL_OUT_OF_RANGE)) return;
+  // On any error the kernels ahead may have stopped half way: with a label out of range some CTAs of k_bwd_begin give up at
+  // their last barrier, and the tokens they would have placed still hold the mark 1, which is no row of dEmb_rows.
+  if (ld_volatile(&p.st->status) != 0 || p.st->n_levels < 1) return;
   const int n_leaves = p.level_offset[1];
   const int grad_ctas = p.tiles * p.splits;
   if ((int)blockIdx.x >= grad_ctas) {

@@ -197,3 +197,37 @@ def test_states_that_do_not_fit_shared_memory():
     p = fg.draw_recursive_params(rng, 130, 90, tensor=False, emb_scale=0.8, w_scale=1.0 / np.sqrt(260))
     forest = fg.random_forest(rng, 2, 1000, 1001, 90)
     _training_step(binding.CELL_TREERNN, p, forest, binding.PERSISTENT)
+
+
+@pytest.mark.parametrize("cell,n_trees,hi", [(binding.CELL_TREERNN, 20, 40), (binding.CELL_TREERNN, 1, 1),
+                                             (binding.CELL_RNTN, 20, 24), (binding.CELL_RNTN, 1, 1)])
+def test_label_out_of_range_reaches_no_gradient(cell, n_trees, hi):
+    """a bad label ends the step before anything is added to a gradient (which tokens had got their row of
+    dEmb_rows by then is a matter of timing): the cleared outputs stay zero, the memory behind the rows of the
+    leaves is not touched, and the context takes the next step"""
+    rng = np.random.default_rng(800 + hi)
+    tensor = cell == binding.CELL_RNTN
+    p = fg.draw_recursive_params(rng, 24, 50, tensor=tensor, emb_scale=0.8, w_scale=0.2, v_scale=0.02)
+    forest = fg.random_forest(rng, n_trees, 1, hi, 50)
+    n, leaves, H, C = forest.n_nodes, forest.n_leaves, p.H, 5
+    model = _model(cell, p)
+    model.set_classifier(util.to_dev(rng.uniform(-0.3, 0.3, size=(H, C)).astype(np.float32)), util.to_dev(np.zeros(C, np.float32)))
+    arrs = [util.to_dev(a) for a in (forest.left, forest.right, forest.token)]
+    labels = np.zeros(n, np.int32)
+    labels[n // 2] = C
+    model.forward(*arrs, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+    f32 = dict(dtype=torch.float32, device="cuda")
+    out = {k: torch.full(shape, 7.0, **f32) for k, shape in dict(loss=(1,), dW=(2 * H, H), db=(H,), dV=(H, 2 * H, 2 * H), dWc=(H, C), dbc=(C,)).items()}
+    rows = torch.full((leaves + 8, H), 7.0, **f32)
+    ids, touched = torch.empty(leaves, dtype=torch.int32, device="cuda"), torch.empty(1, dtype=torch.int32, device="cuda")
+    bad = util.to_dev(labels)
+    ptr = lambda t: t.data_ptr()
+    rc_ = model.lib.treelstm_backward_recursive(model.handle, ptr(bad), ptr(out["loss"]), ptr(out["dW"]), ptr(out["db"]), ptr(out["dV"]),
+                                                ptr(out["dWc"]), ptr(out["dbc"]), ptr(ids), ptr(rows), ptr(touched), None)
+    assert rc_ == binding.OK and model.status_sync() == binding.ERR_LABEL_OUT_OF_RANGE
+    assert bool((rows[leaves:] == 7.0).all()) and not bool(rows[:leaves].any())
+    assert not bool(out["dW"].any()) and not bool(out["db"].any()) and (not tensor or not bool(out["dV"].any()))
+    labels[n // 2] = 0
+    model.forward(*arrs, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+    assert np.isfinite(model.backward_recursive(util.to_dev(labels), leaves)["loss"].item())
+    model.close()
