@@ -41,8 +41,8 @@ WsLayout ws_layout(const treelstm* ctx, int n, bool with_backward) {
                                                                    // reads whole quads; then one count per 128 ids
   }
   L.img_dz = L.img_x0 = L.img_x1 = L.img_end = off;
-  // forests that one cluster may be too slow for: operands of the backward pass split into bf16 pieces
-  if (with_backward && ctx->wsp && !trees_always_pay((int)nn, ctx->H, 1)) {
+  // forests that the tree kernels may be too slow for: operands of the backward pass split into bf16 pieces
+  if (with_backward && ctx->wsp && !trees_always_pay(ctx->cell, ctx->H, (int)nn, true)) {
     L.img_dz = take(image_bytes((int)nn, 5 * gate_pitch(ctx->H)));
     L.img_x0 = take(image_bytes((int)nn, ctx->E + 1));
     L.img_x1 = take(image_bytes((int)nn, 2 * ctx->H + 1));

@@ -842,15 +842,15 @@ __device__ __forceinline__ void zero_range(T* ptr, size_t count, size_t gtid, si
   for (size_t i = gtid; i < count; i += gthreads) ptr[i] = T(0);
 }
 __global__ void __launch_bounds__(256, 2)
-k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int with_dweight, int tree_parts) {
+k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int with_dweight, int after_trees) {
   extern __shared__ float4 s_dyn4[];
   BwdSmem& sm = *reinterpret_cast<BwdSmem*>(s_dyn4);
   float* s_cls = reinterpret_cast<float*>(s_dyn4) + (sizeof(BwdSmem) + 3) / 4;
   __shared__ int s_flag;
   if (ld_volatile(&p.st->status) != 0) return;
-  // behind k_bwd_begin and the tree kernel: classifier and token table are done, and only forests that trees_pay() leaves
-  const bool after_begin = tree_parts > 0;
-  if (after_begin && trees_pay(p.n, p.st->n_roots, p.H, tree_parts)) return;
+  // behind k_bwd_begin and the tree kernel: classifier and token table are done, and only forests that the latter leaves
+  const bool after_begin = after_trees != 0;
+  if (after_begin && p.st->trees_bwd) return;
   const int n_levels = p.st->n_levels;
   const int n = p.n, H = p.H, E = p.E, C = p.C, J = 5 * H;
 #ifdef TREELSTM_TRACE
@@ -998,7 +998,7 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
 }
 
 // ---- the wavefronts of a forest that is wide, on the tensor cores ------------------------------ //
-// Behind k_bwd_begin, for the forests that trees_pay() leaves.  On fp32 units the contraction dIn = dz W^T of the wide
+// Behind k_bwd_begin, for the forests that the tree kernel leaves.  On fp32 units the contraction dIn = dz W^T of the wide
 // wavefronts was 600 of the 880 us of the backward pass of 14.6 k nodes (H = 256).  Here dz is split into bf16 pieces
 // (BwdImages, the layout the tensor core reads), and tiles of 128 positions x 128 outputs are multiplied with W split once
 // per set of weights: one thread asks for blocks (plain bulk copies of whole tiles), one issues the MMAs, sixteen warps
@@ -1010,7 +1010,7 @@ constexpr int kDirectRows = 256, kWideOffCache = 512;
 struct WideArgs {
   const int* level_offset;
   long long wait_limit;
-  int tree_parts;
+  int after_trees;
   BwdImages img;
 };
 
@@ -1240,7 +1240,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   __shared__ int s_abort, s_flag;
   __shared__ int s_node[kSpTile], s_da[kSpTile], s_db[kSpTile];
   __shared__ int s_off[kWideOffCache];
-  if (ld_volatile(&p.st->status) != 0 || (a.tree_parts > 0 && trees_pay(p.n, p.st->n_roots, p.H, a.tree_parts))) return;
+  if (ld_volatile(&p.st->status) != 0 || (a.after_trees && p.st->trees_bwd)) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grid = (int)gridDim.x;
   unsigned char* const tiles = wide_dyn + ((1024u - (smem_u32(wide_dyn) & 1023u)) & 1023u);
   const uint32_t tiles_addr = smem_u32(tiles), full0 = smem_u32(&s_bars[0]), empty0 = smem_u32(&s_bars[2]),
@@ -1461,7 +1461,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
 // marked | tokens counted beside the classifier | tokens placed.  The level table stays on the device.
 struct GradSizes { size_t dW, db, dV; };   // floats
 __global__ void __launch_bounds__(256, 2)
-k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, long long wait_limit, int wide, int tree_parts) {
+k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, long long wait_limit, int wide) {
   extern __shared__ float s_cls[];
   __shared__ __align__(16) unsigned int s_mask[1024];
   __shared__ int s_flag;
@@ -1484,17 +1484,17 @@ k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, lo
   zero_range(p.dbc, (size_t)C, gtid, gthreads);
   zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
   zero_range(p.dEmb_rows, (size_t)p.n_leaves * p.E, gtid, gthreads);
-  if (wide && !(tree_parts > 0 && trees_pay(p.n, p.st->n_roots, H, tree_parts))) {   // k_bwd_wide follows: dc of the roots, children by position
-    zero_range(p.dc, (size_t)p.n * H, gtid, gthreads);
-    for (size_t r = (size_t)p.n_leaves + gtid; r < (size_t)p.n; r += gthreads) {
-      const int node = chk(p.st, p.order[r], p.n);
+  if (wide) zero_range(p.dc, (size_t)p.n * H, gtid, gthreads);   // k_bwd_wide may follow: dc of the roots
+  if (!barrier()) return;
+  for (size_t r = gtid; r < (size_t)(wide ? p.n : p.n_leaves); r += gthreads) {
+    const int node = chk(p.st, p.order[r], p.n);
+    if (r < (size_t)p.n_leaves) {
+      p.tok_slot[chk(p.st, p.token[node], p.vocab)] = 1;
+    } else {                               // children by position, for k_bwd_wide
       p.pos_left[r] = p.left[node];
       p.pos_right[r] = p.right[node];
     }
   }
-  if (!barrier()) return;
-  for (size_t r = gtid; r < (size_t)p.n_leaves; r += gthreads)
-    p.tok_slot[chk(p.st, p.token[chk(p.st, p.order[r], p.n)], p.vocab)] = 1;
   if (!barrier()) return;
   int* const group_count = p.tok_slot + p.vocab + 4;
   if (gridDim.x == 1) {
@@ -1508,7 +1508,7 @@ k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, lo
   }
 }
 
-int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, int wide, int tree_parts, cudaStream_t stream) {
+int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, int wide, cudaStream_t stream) {
   const size_t smem = sizeof(float) * ((size_t)p.H * p.C + p.C);
   if (smem > 160 * 1024) return TREELSTM_ERR_UNSUPPORTED;
   if (smem > 40 * 1024)
@@ -1521,7 +1521,7 @@ int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, in
   TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, 2 * sizeof(unsigned int), stream));   // and barrier_levels behind it
   const int* lvl_off = ctx->last.level_offset;
   long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
-  void* args[] = {&p, &dV, &sizes, &lvl_off, &wait_limit, &wide, &tree_parts};
+  void* args[] = {&p, &dV, &sizes, &lvl_off, &wait_limit, &wide};
   TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_begin, dim3(grid), dim3(256), args, smem, stream));
   ctx->launches += 1;
   return TREELSTM_OK;
@@ -1529,7 +1529,7 @@ int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, in
 
 }  // namespace
 
-static int launch_bwd_persistent(treelstm* ctx, BwdParams& p, size_t cls_smem, int with_dweight, int tree_parts, cudaStream_t stream) {
+static int launch_bwd_persistent(treelstm* ctx, BwdParams& p, size_t cls_smem, int with_dweight, int after_trees, cudaStream_t stream) {
   const size_t smem = ((sizeof(BwdSmem) + 3) / 4) * 4 + cls_smem;
   TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
@@ -1539,17 +1539,17 @@ static int launch_bwd_persistent(treelstm* ctx, BwdParams& p, size_t cls_smem, i
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
   const int* lvl_off = ctx->last.level_offset;
   long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
-  void* args[] = {&p, &lvl_off, &wait_limit, &with_dweight, &tree_parts};
+  void* args[] = {&p, &lvl_off, &wait_limit, &with_dweight, &after_trees};
   TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_persistent, dim3(grid), dim3(256), args, smem, stream));
   ctx->launches += 1;
   return TREELSTM_OK;
 }
 
-static int launch_bwd_wide(treelstm* ctx, BwdParams& p, const BwdImages& img, int tree_parts, cudaStream_t stream) {
+static int launch_bwd_wide(treelstm* ctx, BwdParams& p, const BwdImages& img, int after_trees, cudaStream_t stream) {
   TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmem));
   int grid = ctx->sm_count;
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
-  WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, tree_parts, img};
+  WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, after_trees, img};
   void* args[] = {&p, &a};
   TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_wide, dim3(grid), dim3(kWideThreads), args, kWideSmem, stream));
   ctx->launches += 1;
@@ -1605,8 +1605,7 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
     }
     const bool trees = trees_take(ctx, n), wide = L.lay.img_dz != L.lay.img_end;
     if (ctx->opt.dw_tensor_cores && (trees || wide)) {
-      const int tree_parts = trees ? trees_parts(ctx, n, true, true) : 0;
-      int rc = launch_bwd_begin(ctx, p, nullptr, {(E + 2 * (size_t)H) * J, J, 0}, wide, tree_parts, stream);
+      int rc = launch_bwd_begin(ctx, p, nullptr, {(E + 2 * (size_t)H) * J, J, 0}, wide, stream);
       if (rc == TREELSTM_OK && trees) rc = launch_backward_trees(ctx, stream);
       BwdImages img;
       if (rc == TREELSTM_OK && wide) {
@@ -1614,12 +1613,12 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
         img.x[0] = reinterpret_cast<unsigned char*>(base + L.lay.img_x0);
         img.x[1] = reinterpret_cast<unsigned char*>(base + L.lay.img_x1);
         img.w = ctx->wsp;
-        rc = launch_bwd_wide(ctx, p, img, tree_parts, stream);
-      } else if (rc == TREELSTM_OK && !trees_always_pay(n, H, tree_parts)) {
-        rc = launch_bwd_persistent(ctx, p, cls_smem, 0, tree_parts, stream);
+        rc = launch_bwd_wide(ctx, p, img, trees, stream);
+      } else if (rc == TREELSTM_OK && !trees_always_pay(0, H, n, true)) {
+        rc = launch_bwd_persistent(ctx, p, cls_smem, 0, 1, stream);
       }
       return rc != TREELSTM_OK ? rc : launch_dweight_tc(ctx, n, L.order, L.level_offset, L.token, L.left, L.right, L.h, p.dz, dW, db,
-                                                        p.tok_slot, dEmb_rows, p.st, &img, tree_parts, stream);
+                                                        p.tok_slot, dEmb_rows, p.st, &img, trees, stream);
     }
     TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, sizeof(unsigned int), stream));
     const int with_dweight = ctx->opt.dw_tensor_cores ? 0 : 1;
@@ -1627,7 +1626,7 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
     if (rc != TREELSTM_OK) return rc;
     if (!with_dweight)
       return launch_dweight_tc(ctx, n, L.order, L.level_offset, L.token, L.left, L.right, L.h, p.dz, dW, db, p.tok_slot,
-                               dEmb_rows, p.st, nullptr, 0, stream);
+                               dEmb_rows, p.st, nullptr, false, stream);
     return TREELSTM_OK;
   }
   TL_CUDA(ctx, cudaMemsetAsync(loss, 0, sizeof(float), stream));
@@ -1730,6 +1729,66 @@ __global__ void k_rec_bwd_dx(RecBwd p, int begin, int end) {
   p.dh[(size_t)child * H + (a < H ? a : a - H)] += acc;
 }
 
+// The wavefronts of a forest that the tree kernel leaves (few large trees), in one cooperative launch behind it and behind
+// k_bwd_begin; the gradients are k_rec_grads's either way.  A warp takes one node and kDxUnits of the 2H inputs; its lanes
+// share the units of dz and read rows of W (and V) side by side, so that a wavefront is one chain of loads and one grid barrier.
+constexpr int kDxUnits = 8, kDxThreads = 256, kDxMaxH = 256;   // (the tree kernels end there)
+__global__ void __launch_bounds__(kDxThreads) k_rec_bwd_levels(RecBwd p, const int* level_offset, long long wait_limit) {
+  __shared__ int s_flag;
+  if (ld_volatile(&p.st->status) != 0 || p.st->trees_bwd) return;
+  const int H = p.H, K = 2 * H, lane = threadIdx.x & 31, groups = (K + kDxUnits - 1) / kDxUnits;
+  const long long first = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, step = (long long)gridDim.x * (kDxThreads / 32);
+  unsigned int arrivals = 0;
+  for (int lvl = p.st->n_levels - 1; lvl >= 1; --lvl) {
+    const int begin = level_offset[lvl], end = level_offset[lvl + 1];
+    for (long long i = first; i < (long long)(end - begin) * groups; i += step) {
+      const int node = chk(p.st, p.order[begin + (int)(i / groups)], p.n), a0 = (int)(i % groups) * kDxUnits;
+      const int l = chk(p.st, p.left[node], p.n), r = chk(p.st, p.right[node], p.n);
+      float dz[kDxMaxH / 32];
+#pragma unroll
+      for (int t = 0; t < kDxMaxH / 32; ++t) {
+        const int j = lane + 32 * t;
+        dz[t] = 0.f;
+        if (j < H) {
+          const float hv = __ldg(p.h + (size_t)node * H + j);
+          dz[t] = __ldcg(p.dh + (size_t)node * H + j) * (1.f - hv * hv);
+          if (a0 == 0) p.dz[(size_t)node * H + j] = dz[t];
+        }
+      }
+      float acc[kDxUnits];
+#pragma unroll
+      for (int u = 0; u < kDxUnits; ++u) {
+        acc[u] = 0.f;
+        const int a = min(a0 + u, K - 1);
+#pragma unroll
+        for (int t = 0; t < kDxMaxH / 32; ++t)
+          if (lane + 32 * t < H) acc[u] = fmaf(__ldg(p.W + (size_t)a * H + lane + 32 * t), dz[t], acc[u]);
+        if (p.tensor)
+          for (int b = 0; b < K; ++b) {
+            const float xb = __ldg(p.h + (size_t)(b < H ? l : r) * H + (b < H ? b : b - H));
+#pragma unroll
+            for (int t = 0; t < kDxMaxH / 32; ++t) {
+              const int j = lane + 32 * t;
+              if (j < H) acc[u] = fmaf(xb * dz[t], __ldg(p.Vt + ((size_t)a * K + b) * H + j) + __ldg(p.Vt + ((size_t)b * K + a) * H + j), acc[u]);
+            }
+          }
+      }
+#pragma unroll
+      for (int u = 0; u < kDxUnits; ++u) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) acc[u] += __shfl_xor_sync(kFull, acc[u], d);
+        const int a = a0 + u;
+        if (lane == u && a < K) {                // a child has one caller
+          float* at = p.dh + (size_t)(a < H ? l : r) * H + (a < H ? a : a - H);
+          *at = __ldcg(at) + acc[u];
+        }
+      }
+    }
+    arrivals += gridDim.x;
+    if (lvl > 1 && !grid_barrier(p.st, arrivals, wait_limit, &s_flag, true, &p.st->barrier_levels)) return;
+  }
+}
+
 __global__ void k_rec_bwd_leaves(RecBwd p) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)p.n_leaves * p.H) return;
@@ -1773,6 +1832,16 @@ __global__ void k_rec_bwd_dv(RecBwd p) {
   p.dV[idx] = acc;
 }
 
+RecBwd rec_bwd(const treelstm* ctx, const BwdParams& p, float* dW, float* db, float* dV) {
+  RecBwd q{};
+  const size_t K = 2 * (size_t)p.H;
+  q.n = p.n; q.H = p.H; q.n_leaves = p.n_leaves; q.tensor = ctx->cell == TREELSTM_CELL_RNTN ? 1 : 0;
+  q.left = p.left; q.right = p.right; q.token = p.token; q.order = p.order;
+  q.h = p.h; q.Vt = ctx->Wcat; q.W = ctx->Wcat + (q.tensor ? K * K * p.H : 0);
+  q.dh = p.dh; q.dz = p.dz; q.dW = dW; q.db = db; q.dV = dV; q.dEmb_rows = p.dEmb_rows; q.tok_slot = p.tok_slot; q.st = p.st;
+  return q;
+}
+
 }  // namespace
 
 int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float* dW, float* db, float* dV,
@@ -1793,8 +1862,21 @@ int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float
     p.touched_ids = touched_ids; p.n_touched = n_touched;
     p.st = reinterpret_cast<DevStatus*>(base + L.lay.status);
     const size_t H = ctx->H;
-    int rc = launch_bwd_begin(ctx, p, dV, {2 * H * H, H, ctx->cell == TREELSTM_CELL_RNTN ? 4 * H * H * H : 0}, 0, 0, stream);
+    int rc = launch_bwd_begin(ctx, p, dV, {2 * H * H, H, ctx->cell == TREELSTM_CELL_RNTN ? 4 * H * H * H : 0}, 0, stream);
     if (rc == TREELSTM_OK) rc = launch_backward_trees(ctx, stream);
+    if (rc == TREELSTM_OK && !trees_always_pay(ctx->cell, ctx->H, L.n, true)) {
+      RecBwd q = rec_bwd(ctx, p, dW, db, dV);
+      int per_sm = 0;
+      TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rec_bwd_levels, kDxThreads, 0));
+      if (per_sm < 1) return TREELSTM_ERR_UNSUPPORTED;
+      int grid = ctx->sm_count * (per_sm < 2 ? per_sm : 2);
+      if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
+      const int* lvl_off = L.level_offset;
+      long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
+      void* args[] = {&q, &lvl_off, &wait_limit};
+      TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_rec_bwd_levels, dim3(grid), dim3(kDxThreads), args, 0, stream));
+      ctx->launches += 1;
+    }
     return rc != TREELSTM_OK ? rc : launch_rec_grads(ctx, dW, db, dV, dEmb_rows, p.tok_slot, stream);
   }
   int rc = ensure_host_levels(ctx);      // one read of the level table (a persistent forward left it on the device)
@@ -1835,11 +1917,7 @@ int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float
   k_bwd_classifier<<<(n + kClsNodesPerCta - 1) / kClsNodesPerCta, kClsWarps * 32, cls_smem, stream>>>(p);
   ctx->launches += 3;
 
-  RecBwd q{};
-  q.n = n; q.H = H; q.n_leaves = n_leaves; q.tensor = tensor ? 1 : 0;
-  q.left = L.left; q.right = L.right; q.token = L.token; q.order = L.order;
-  q.h = L.h; q.Vt = ctx->Wcat; q.W = ctx->Wcat + (tensor ? K * K * H : 0);
-  q.dh = p.dh; q.dz = p.dz; q.dW = dW; q.db = db; q.dV = dV; q.dEmb_rows = dEmb_rows; q.tok_slot = p.tok_slot; q.st = p.st;
+  const RecBwd q = rec_bwd(ctx, p, dW, db, dV);
   for (int lvl = n_levels - 1; lvl >= 1; --lvl) {
     const int begin = off[lvl], end = off[lvl + 1];
     const long long e1 = (long long)(end - begin) * H, e2 = (long long)(end - begin) * (long long)K;

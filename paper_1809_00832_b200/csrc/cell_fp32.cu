@@ -27,7 +27,7 @@ struct FwdParams {
   DevStatus* st;
   long long wait_limit;
   int w_stationary, a_row, w_row;   // persistent kernel: W_h slice resident in shared memory; row strides (floats)
-  int tree_parts = 0;               // > 0: launched behind the tree kernels, leaves done; takes the forests that trees_pay() leaves to it
+  int after_trees = 0;              // launched behind the tree kernels, leaves done; takes the forests that they leave to it
   int early_start = 0;              // persistent kernel: launched under the scheduler, waits for it on the device
   long long* trace = nullptr;       // cycle stamps of the persistent kernel (trace builds), else nullptr
 };
@@ -370,9 +370,9 @@ k_fwd_fp32_persistent(FwdParams p) {
   // Launched as a programmatic dependent of the ready-set construction (p.early_start), the kernel
   // gets here while that one still runs: the weight slice needs nothing from it and is fetched first.
   int n_levels = 0;
-  if (p.tree_parts > 0) {
+  if (p.after_trees) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (ld_volatile(&p.st->status) != 0 || trees_pay(p.n, p.st->n_roots, p.H, p.tree_parts)) return;
+    if (ld_volatile(&p.st->status) != 0 || p.st->trees_fwd) return;
   }
   if (!p.early_start) {
     if (ld_volatile(&p.st->status) != 0) return;
@@ -390,7 +390,7 @@ k_fwd_fp32_persistent(FwdParams p) {
       Ws[col * w_row + k] = v;
     }
   }
-  const int first_level = p.tree_parts > 0 ? 1 : 0;
+  const int first_level = p.after_trees ? 1 : 0;
   if (first_level == 0) {
     // The leaf wavefront streams W_x and the leaves' embedding rows chunk by chunk, one dependent fetch per
     // chunk: asked into L2 now (which nodes are leaves and their tokens are the caller's arrays, readable
@@ -486,13 +486,13 @@ int launch_forward_fp32(treelstm* ctx, int n, const int32_t* left, const int32_t
                         const int32_t* level_offset_dev, const int32_t* level_offset_host,
                         int n_levels_host, int flags, void* ws, const WsLayout& lay,
                         cudaStream_t stream) {
-  int tree_parts = 0;
+  bool after_trees = false;
   if ((flags & TREELSTM_PERSISTENT) && trees_take(ctx, n)) {
     const bool running = ctx->opt.overlap_launch && scheduler_lets_start(ctx, n);
     const int rc = launch_forward_trees(ctx, n, left, right, token, h, c, (flags & TREELSTM_SAVE_FOR_BACKWARD) != 0, ws, lay, running, stream);
     if (rc != TREELSTM_OK) return rc;
-    tree_parts = trees_parts(ctx, n, false, running);
-    if (trees_always_pay(n, ctx->H, tree_parts)) return TREELSTM_OK;
+    if (trees_always_pay(0, ctx->H, n, false)) return TREELSTM_OK;
+    after_trees = true;
   }
   char* base = static_cast<char*>(ws);
   FwdParams p;
@@ -506,7 +506,7 @@ int launch_forward_fp32(treelstm* ctx, int n, const int32_t* left, const int32_t
   p.st = reinterpret_cast<DevStatus*>(base + lay.status);
   p.wait_limit = ctx->opt.wait_limit_kcycles * 1024;
   p.w_stationary = 0; p.a_row = 0; p.w_row = 0;
-  p.tree_parts = tree_parts;
+  p.after_trees = after_trees ? 1 : 0;
 #ifdef TREELSTM_TRACE
   p.trace = reinterpret_cast<long long*>(base + lay.trace) + kTraceSlots * kTraceLevels;   // second table: the backward clears the first
   if (flags & TREELSTM_PERSISTENT)

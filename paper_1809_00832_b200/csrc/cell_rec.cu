@@ -30,6 +30,7 @@ struct RecParams {
   float* h;
   DevStatus* st;
   long long wait_limit;
+  int after_trees;            // launched behind the tree kernel: takes the forests that it leaves
 };
 
 // rows [row_begin, row_end) of the ready order (level 0): the word vectors
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(kThreads) k_rec_level(RecParams p, int row_beg
 __global__ void __launch_bounds__(kThreads) k_rec_persistent(RecParams p) {
   extern __shared__ float rec_smem[];
   __shared__ int s_flag;
-  if (ld_volatile(&p.st->status) != 0) return;
+  if (ld_volatile(&p.st->status) != 0 || (p.after_trees && p.st->trees_fwd)) return;
   const int n_levels = p.st->n_levels;
   const int tiles_u = (p.H + RN - 1) / RN;
   for (int lvl = 0; lvl < n_levels; ++lvl) {
@@ -176,10 +177,15 @@ int launch_forward_rec(treelstm* ctx, int n, const int32_t* left, const int32_t*
                        float* h, const int32_t* order, const int32_t* level_offset_dev,
                        const int32_t* level_offset_host, int n_levels_host, int flags, void* ws,
                        const WsLayout& lay, cudaStream_t stream) {
+  bool after_trees = false;
   if ((flags & TREELSTM_PERSISTENT) && trees_take(ctx, n)) {
-    return launch_forward_trees(ctx, n, left, right, token, h, nullptr, false, ws, lay, ctx->opt.overlap_launch && scheduler_lets_start(ctx, n), stream);
+    const int rc = launch_forward_trees(ctx, n, left, right, token, h, nullptr, false, ws, lay,
+                                        ctx->opt.overlap_launch && scheduler_lets_start(ctx, n), stream);
+    if (rc != TREELSTM_OK || trees_always_pay(ctx->cell, ctx->H, n, false)) return rc;
+    after_trees = true;
   }
   RecParams p;
+  p.after_trees = after_trees ? 1 : 0;
   p.n = n; p.H = ctx->H; p.cell = ctx->cell; p.vocab = ctx->vocab;
   p.chk_counts = check_counters(ws, lay);
   p.K = ctx->cell == TREELSTM_CELL_RNTN ? 4 * ctx->H * ctx->H + 2 * ctx->H : 2 * ctx->H;

@@ -22,7 +22,8 @@ struct DevStatus {
   unsigned int barrier_bwd;  // arrival counter of the one-launch backward pass (cleared by its launch)
   unsigned int barrier_levels;  // the same of its wavefronts alone, behind k_bwd_begin
   int tail_from;         // persistent bf16 forward: first wavefront the cluster kernel takes (or would take), n_levels if none
-  int pad[55];
+  int trees_fwd, trees_bwd;   // 1: the tree kernels (trees_fp32.cu) took this forest forward / backward
+  int pad[53];
 };
 static_assert(sizeof(DevStatus) == 256, "control block is one 256-byte line group");
 
@@ -104,18 +105,22 @@ struct TreesShape {
   int bthreads = 0, bseg = 0, BC = 0, TPA = 0;
 };
 
-// Whether a TreeLSTM forest of n nodes and n_roots trees goes to the tree kernels (trees_fp32.cu) or to the kernels that
-// take a wavefront over the whole GPU.  A cluster takes about 1600 cycles per internal node (H = 150 and 256 alike: the
-// slice per CTA is), a grid-wide wavefront 9000 and more: at least 13 of them are assumed, and 12 TFLOP/s behind them.
-// The host knows neither count, so both kernels are launched and ask here.
-__host__ __device__ inline bool trees_pay(int n, int n_roots, int H, int clusters) {
-  const int internal = (n - n_roots) / 2, busy = n_roots < clusters ? n_roots : clusters;
-  if (internal <= 0 || busy <= 0) return true;
-  return 1600.f * (float)internal / (float)busy < 117000.f + (float)internal * (float)H * (float)H * 3.2e-3f;
+// What the two fp32 ways through a forest cost in microseconds: trees dealt out to clusters (trees_fp32.cu), where the
+// fullest cluster sets the time, or every wavefront over the whole GPU (cell_fp32.cu, cell_rec.cu, backward.cu).  The host
+// knows the number of nodes only, so the tree kernel counts (trees_win) and leaves the forest to the kernel behind it, or
+// not; that one reads the outcome in the control block.
+struct WalkCosts {
+  float tree0, node, depth, rest;   // clusters: fixed, per internal node and depth of the fullest one, per internal node of the forest
+  float grid0, wave, each;          // whole GPU: fixed, per wavefront of internal nodes, per internal node
+};
+__host__ __device__ inline float tree_cost(const WalkCosts& c, float nodes, float depth, float internal) {
+  return c.tree0 + c.node * nodes + c.depth * depth + c.rest * internal;
 }
-
-// The same for every number of trees: forests so small that one cluster alone is faster.
-inline bool trees_always_pay(int n, int H, int clusters) { return clusters > 0 && trees_pay(n, 1, H, 1); }
+__host__ __device__ inline float grid_cost(const WalkCosts& c, float waves, float internal) {
+  return c.grid0 + c.wave * waves + c.each * internal;
+}
+WalkCosts walk_costs(int cell, int H, bool backward);        // trees_fp32.cu
+bool trees_always_pay(int cell, int H, int n, bool backward); // forests too small to be worth the second launch
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 inline size_t round_up_sz(size_t x, size_t m) { return (x + m - 1) / m * m; }
@@ -244,7 +249,6 @@ size_t plan_trees(treelstm* ctx);                        // bytes of the registe
 int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream);
 int pack_trees(treelstm* ctx, cudaStream_t stream);      // after the weights have changed
 bool trees_take(const treelstm* ctx, int n);
-int trees_parts(const treelstm* ctx, int n, bool backward, bool after_running);   // clusters that a launch takes
 int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
                          float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
 int launch_backward_trees(treelstm* ctx, cudaStream_t stream);   // dz of every node (TreeRNN / RNTN: and dh of the leaves) from dh
@@ -294,7 +298,7 @@ int pack_wide_backward(treelstm* ctx, cudaStream_t stream);
 size_t image_bytes(int n, int features);
 int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t* level_offset, const int32_t* token,
                       const int32_t* left, const int32_t* right, const float* h, const float* dz, float* dW, float* db,
-                      const int* tok_slot, float* dEmb_rows, DevStatus* st, const BwdImages* img, int tree_parts,
+                      const int* tok_slot, float* dEmb_rows, DevStatus* st, const BwdImages* img, bool after_trees,
                       cudaStream_t stream);
 
 // Checked build: clears the per-row write counters before a forward / compares them after it

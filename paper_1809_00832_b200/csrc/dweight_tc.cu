@@ -44,7 +44,7 @@ struct DwParams {
   DevStatus* st;
   long long wait_limit;
   BwdImages img;                // operands split beforehand (forests that went to the grid-wide wavefront kernel)
-  int tree_parts;               // > 0: the tree kernels took the forest if trees_pay() says so, and img holds nothing
+  int after_trees;              // the tree kernels took the forest if the control block says so, and img holds nothing
 };
 
 // One operand tile (128 rows x 64 nodes, three pieces) of block `kb` of the work item, in two steps: the
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
   const uint32_t tmem_base = s_tmem;
   const int H = p.H, E = p.E, J = 5 * H;
   const int n_leaves = p.st->n_levels > 0 ? min(p.n, max(0, p.level_offset[1])) : 0;
-  if (p.img.dz != nullptr && !(p.tree_parts > 0 && trees_pay(p.n, p.st->n_roots, H, p.tree_parts))) {
+  if (p.img.dz != nullptr && !(p.after_trees && p.st->trees_bwd)) {
     dw_from_images(p, n_leaves, tiles, stage_bar0, smem_u32(&s_bars[kDwStages + 2]), acc_bar, tmem_base, &s_abort);
     tc_fence_before();
     __syncthreads();
@@ -490,10 +490,10 @@ int init_dweight_tc_attributes(treelstm* ctx) {
 // stream before; dz holds the gate gradients of every node.
 int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t* level_offset, const int32_t* token,
                       const int32_t* left, const int32_t* right, const float* h, const float* dz, float* dW, float* db,
-                      const int* tok_slot, float* dEmb_rows, DevStatus* st, const BwdImages* img, int tree_parts, cudaStream_t stream) {
+                      const int* tok_slot, float* dEmb_rows, DevStatus* st, const BwdImages* img, bool after_trees, cudaStream_t stream) {
   DwParams p;
   if (img) p.img = *img;
-  p.tree_parts = tree_parts;
+  p.after_trees = after_trees ? 1 : 0;
   p.n = n; p.n_leaves = 0; p.H = ctx->H; p.E = ctx->E; p.vocab = ctx->vocab; p.run = 0;
   p.order = order; p.level_offset = level_offset; p.token = token; p.left = left; p.right = right;
   p.emb = ctx->emb; p.h = h; p.dz = dz; p.W = ctx->W; p.dW = dW; p.db = db; p.st = st;

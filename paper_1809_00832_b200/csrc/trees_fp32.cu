@@ -24,6 +24,8 @@
 // itself, from the child arrays in shared memory, so nothing here waits for the scheduler before its end.  (A
 // malformed forest is the scheduler's to report; here every index is clamped and every list bounded, so that
 // whatever the arrays hold the walk ends.)  Clusters take roots q, q + Q, ... in id order.
+#include <math.h>
+
 #include <type_traits>
 
 #include "common.cuh"
@@ -90,6 +92,8 @@ struct TreesParams {
   const int *left, *right, *token;
   const float *emb, *W, *b;               // W: register image [rank][word][thread]; b [G H]
   const ushort2* pairs;                   // RNTN: the two operands of every input chunk
+  WalkCosts costs;
+  int choose;                             // 1: the forest may be left to the kernel behind this one (trees_win)
   float *h, *c, *gates, *dh, *dc, *dz;
   DevStatus* st;
   long long* trace;                       // cycle stamps of the first CTA (trace builds), else nullptr
@@ -186,11 +190,16 @@ __host__ __device__ inline int bwd_buf_words(int cell, int H, const TreesShape& 
 // tokens are clamped: nothing has been validated yet.
 constexpr unsigned kLeafBit = 0x80000000u;
 __device__ __forceinline__ bool is_leaf(unsigned kids) { return (kids & kLeafBit) != 0; }
-__device__ __forceinline__ void load_kids(const TreesParams& p, const TreesSmem& s, float* sm) {
+// (up: if given, every node's caller, a root's itself.  Two callers of one child are no forest: which of them is found is a matter of timing, so
+// the answer is true then, the same in every CTA.)
+__device__ __forceinline__ bool load_kids(const TreesParams& p, const TreesSmem& s, float* sm, unsigned short* up) {
   unsigned* kids = reinterpret_cast<unsigned*>(sm + s.kids);
   unsigned* child = reinterpret_cast<unsigned*>(sm + s.child);
   for (int k = threadIdx.x; k < p.n / 32 + 1; k += blockDim.x) child[k] = 0u;
+  if (up)
+    for (int k = threadIdx.x; k < p.n; k += blockDim.x) up[k] = (unsigned short)k;
   __syncthreads();
+  bool twice = false;
   for (int k = threadIdx.x; k < p.n; k += blockDim.x) {
     const int l = p.left[k], r = p.right[k], t = p.token[k];
     if (l < 0) {
@@ -198,19 +207,26 @@ __device__ __forceinline__ void load_kids(const TreesParams& p, const TreesSmem&
     } else {
       const unsigned a = (unsigned)min(l, p.n - 1), b = (unsigned)min(max(r, 0), p.n - 1);
       kids[k] = a | (b << 16);
-      atomicOr(child + (a >> 5), 1u << (a & 31));
-      atomicOr(child + (b >> 5), 1u << (b & 31));
+      if (up) {
+        up[a] = up[b] = (unsigned short)k;
+        const unsigned had_a = atomicOr(child + (a >> 5), 1u << (a & 31)), had_b = atomicOr(child + (b >> 5), 1u << (b & 31));
+        twice = twice || ((had_a >> (a & 31) | had_b >> (b & 31)) & 1u);
+      } else {
+        atomicOr(child + (a >> 5), 1u << (a & 31));
+        atomicOr(child + (b >> 5), 1u << (b & 31));
+      }
     }
   }
-  __syncthreads();
+  return __syncthreads_or(twice) != 0;
 }
 
 // The cluster's trees by depth: internal node number q is list[q], depth d is [start[d], start[d + 1]), the leaves are
 // in leaf[]; par[q] and leaf_par[] say whose child a node is: 2 x number of the caller + side, kNoCaller for a root.  One
 // warp; every CTA of the cluster gets the same lists.
 constexpr unsigned short kNoCaller = 0xFFFF;
-struct Walk { int depths, internal, leaves, roots; };   // roots: of the whole forest
-__device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, Walk* out) {
+struct Walk { int depths, internal, leaves; };
+// `win`: if given, the walk may end where it reads zero.
+__device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, const int* win, Walk* out) {
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
   unsigned short* list = reinterpret_cast<unsigned short*>(sm + s.list);
@@ -256,6 +272,7 @@ __device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem
   __syncwarp();
   while (lo < count && fits) {
     const int hi = count;
+    if (win && hi - lo >= 512 && !__shfl_sync(kFull, *(const volatile int*)win, 0)) break;   // (narrow depths are not worth the look)
     ++depth;
     if (lane == 0) start[depth] = (unsigned short)hi;
     for (int i0 = lo; i0 < hi; i0 += 32) {
@@ -281,7 +298,114 @@ __device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem
     }
     lo = hi;
   }
-  if (lane == 0) *out = fits ? Walk{depth, count, leaves, rank0} : Walk{0, 0, 0, rank0};
+  if (lane == 0) *out = fits ? Walk{depth, count, leaves} : Walk{0, 0, 0};
+}
+
+// Whether this forest is walked faster by clusters than wavefront by wavefront over the whole GPU.  (The average load of a
+// cluster says too little: one tree of 1024 leaves among 24 sentences, H = 150, was 4.5 times slower here than over the whole
+// GPU.)  Every node of a sample - all of them, if there are no more than kClimbs per thread - climbs to its root, which says
+// whose load it is; every CTA takes the same sample and comes to the same answer.  All warps but the first, which walks the
+// trees meanwhile: with all nodes' ancestors doubled by the whole CTA instead, 25 sentences (H = 150) took 104 us, not 92.
+constexpr int kMaxTreeClusters = 192, kClimbs = 3;
+struct TreeLoads { int nodes[kMaxTreeClusters], depth[kMaxTreeClusters], win; };
+// Callers by node id, then (32-bit words) the roots before each word of the bit map: behind the lists if there is room, else
+// in their place (`beside` false: then the walk comes afterwards).
+struct TreeLinks { unsigned short* up; int* before; bool beside; };
+__device__ __forceinline__ TreeLinks tree_links(const TreesSmem& s, float* sm, int n) {
+  const int words = (n + 1) / 2;
+  TreeLinks t;
+  t.beside = s.state_words >= words + n / 32 + 1;
+  float* at = sm + (t.beside ? s.state : s.list);
+  t.up = reinterpret_cast<unsigned short*>(at);
+  t.before = reinterpret_cast<int*>(at + words);
+  return t;
+}
+__device__ void trees_win(const TreesParams& p, const TreesSmem& s, float* sm, const TreeLinks& links, int parts, TreeLoads* out) {
+  const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
+  const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
+  const int tid = (int)threadIdx.x - 32, nt = (int)blockDim.x - 32, lane = tid & 31, n = p.n;
+  auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); };
+  for (int q = tid; q < parts; q += nt) out->nodes[q] = out->depth[q] = 0;
+  if (tid < 32) {
+    int sum = 0;
+    for (int w0 = 0; w0 * 32 < n; w0 += 32) {
+      const int w = w0 + lane, roots = w * 32 < n ? __popc(~child[w]) : 0;   // (ids beyond n come last: nobody counts them)
+      int incl = roots;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, d);
+        if (lane >= d) incl += t;
+      }
+      if (w * 32 < n) links.before[w] = sum + incl - roots;
+      sum += __shfl_sync(kFull, incl, 31);
+    }
+  }
+  const int sample = min(n, nt * kClimbs);
+  int at[kClimbs], depth[kClimbs];
+  bool have[kClimbs];
+#pragma unroll
+  for (int q = 0; q < kClimbs; ++q) {
+    const int i = tid + q * nt;
+    have[q] = i < sample;
+    at[q] = have[q] ? (int)((long long)i * n / sample) : 0;
+    depth[q] = is_leaf(kids[at[q]]) ? 0 : 1;
+  }
+  for (int step = 0; step < n; ++step) {                     // (arrays that are no forest may hold a cycle)
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < kClimbs; ++q) {
+      const int up = links.up[at[q]];
+      if (up != at[q]) { ++depth[q]; any = true; }
+      at[q] = up;
+    }
+    if (!any) break;
+  }
+  sync();
+#pragma unroll
+  for (int q = 0; q < kClimbs; ++q) {
+    const int root = at[q], w = root >> 5;
+    const int part = have[q] ? (links.before[w] + __popc(~child[w] & ((1u << (root & 31)) - 1u))) % parts : -1;
+    const unsigned peers = __match_any_sync(kFull, part);
+    const int deepest = __reduce_max_sync(peers, depth[q]);
+    if (have[q] && lane == __ffs(peers) - 1) {
+      atomicAdd(&out->nodes[part], __popc(peers));
+      atomicMax(&out->depth[part], deepest);
+    }
+  }
+  sync();
+  if (tid < 32) {
+    const int roots = links.before[(n - 1) >> 5] + __popc(~child[(n - 1) >> 5] & (0xFFFFFFFFu >> (31 - ((n - 1) & 31))));
+    const float internal = (float)((n - roots) / 2), share = internal / (float)sample;
+    float cost = 0.f;
+    int waves = 0;
+    for (int q = lane; q < parts; q += 32) {
+      cost = fmaxf(cost, tree_cost(p.costs, share * (float)out->nodes[q], (float)out->depth[q], internal));
+      waves = max(waves, out->depth[q]);
+    }
+    waves = __reduce_max_sync(kFull, waves);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) cost = fmaxf(cost, __shfl_xor_sync(kFull, cost, d));
+    if (lane == 0) *(volatile int*)&out->win = cost < grid_cost(p.costs, (float)waves, internal);
+  }
+}
+// The tables of the forest, then what the cluster has to walk: nothing, if loads->win says that the forest is the next kernel's.
+__device__ __forceinline__ void deal_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, TreeLoads* loads, Walk* walk) {
+  const int warp = (int)threadIdx.x >> 5;
+  if (threadIdx.x == 0) loads->win = 1;
+  if (!p.choose) {
+    load_kids(p, s, sm, nullptr);
+    if (warp == 0) walk_trees(p, s, sm, part, parts, nullptr, walk);
+    __syncthreads();
+    return;
+  }
+  const TreeLinks links = tree_links(s, sm, p.n);
+  const bool forest = !load_kids(p, s, sm, links.up);    // (else: the scheduler reports it, and the walk is bounded)
+  if (forest && warp > 0) trees_win(p, s, sm, links, parts, loads);
+  if (!links.beside) __syncthreads();
+  if (warp == 0) walk_trees(p, s, sm, part, parts, &loads->win, walk);
+  __syncthreads();
+  if (threadIdx.x == 0 && !loads->win) *walk = Walk{0, 0, 0};
+  __syncthreads();
 }
 
 // ---- forward -------------------------------------------------------------------------------------- //
@@ -289,6 +413,7 @@ template <int CELL, int U, int RC>
 __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constant__ TreesParams p) {
   extern __shared__ __align__(16) float sm[];
   __shared__ Walk s_walk;
+  __shared__ TreeLoads s_loads;
   const int cs = p.s.cs, rank = cs > 1 ? (int)cta_rank() : 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int part = blockIdx.x / cs, parts = gridDim.x / cs;
@@ -301,15 +426,11 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   float w[RC * 4 * U];
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
-  load_kids(p, s, sm);
-  TL_STAMP(trace, kTraceLevels - 1, 1);
-  if (warp == 0) walk_trees(p, s, sm, part, parts, &s_walk);
+  deal_trees(p, s, sm, part, parts, &s_loads, &s_walk);
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
-  __syncthreads();
   TL_STAMP(trace, kTraceLevels - 1, 2);
-  Walk walk = s_walk;
-  if (CELL == kLstm && !trees_pay(p.n, walk.roots, p.H, parts)) walk = Walk{0, 0, 0, walk.roots};   // the grid-wide kernel's forest
+  const Walk walk = s_walk;
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
   const unsigned short* start = reinterpret_cast<const unsigned short*>(sm + s.start);
@@ -515,7 +636,10 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     TL_STAMP(trace, d, 4);
   }
   // what follows on the stream waits for this grid only: it must not end before the scheduler ahead of it has
-  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (blockIdx.x == 0) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tid == 0) p.st->trees_fwd = s_loads.win;
+  }
 }
 
 // ---- TreeLSTM leaves ------------------------------------------------------------------------------ //
@@ -704,6 +828,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   constexpr int kWords = CELL == kRntn ? kRntnBwdWords : BC * 16;
   extern __shared__ __align__(16) float sm[];
   __shared__ Walk s_walk;
+  __shared__ TreeLoads s_loads;
   const int cs = p.s.cs, rank = cs > 1 ? (int)cta_rank() : 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
   const int part = blockIdx.x / cs, parts = gridDim.x / cs;
@@ -714,14 +839,23 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;
 #endif
   TL_STAMP(trace, kTraceLevels - 1, 0);
-  if (CELL == kLstm && !trees_pay(p.n, p.st->n_roots, p.H, parts)) {   // the grid-wide kernel's forest (the schedule is the forward's)
-    if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-    return;
+  if (p.choose) {
+    // the schedule is the forward's: where even an equal deal and a chain of the forest's depth would take too long, no
+    // table is set up
+    const int roots = p.st->n_roots, internal = (p.n - roots) / 2, waves = p.st->n_levels - 1, busy = max(1, min(roots, parts));
+    const float least = fmaxf(tree_cost(p.costs, (float)internal / (float)busy, 1.f, (float)internal),
+                              tree_cost(p.costs, (float)waves, (float)waves, (float)internal));
+    if (least >= grid_cost(p.costs, (float)waves, (float)internal)) {
+      if (blockIdx.x == 0) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (tid == 0) p.st->trees_bwd = 0;
+      }
+      return;
+    }
   }
   float w[kWords];
 #pragma unroll
   for (int q = 0; q < kWords; ++q) w[q] = __ldg(p.W + ((size_t)rank * kWords + q) * nt + tid);
-  load_kids(p, s, sm);
   float* const in = sm + s.buf;                          // [kND][in_row]
   float* const dx = in + kND * in_row;                   // [2][cs][kND][2 JS]
   float* const xs = dx + 2 * cs * kND * 2 * JS;          // RNTN: [kND][2 Hp]
@@ -729,10 +863,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   if (CELL == kRntn)
     for (int e = tid; e < kND * 2 * Hp; e += nt) xs[e] = 0.f;
   TL_STAMP(trace, kTraceLevels - 1, 1);
-  if (warp == 0) walk_trees(p, s, sm, part, parts, &s_walk);
+  deal_trees(p, s, sm, part, parts, &s_loads, &s_walk);
 #pragma unroll
   for (int q = 0; q < kWords; ++q) asm volatile("" : "+f"(w[q]));       // held in registers: not to be loaded again where it is used
-  __syncthreads();
   TL_STAMP(trace, kTraceLevels - 1, 2);
   const Walk walk = s_walk;
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
@@ -948,6 +1081,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
       p.dh[at] = *dh_at(code, node, u);
     }
   }
+  if (blockIdx.x == 0 && tid == 0) p.st->trees_bwd = s_loads.win;
   cluster_sync(cs);                                      // no CTA leaves while a peer may still write to it
 }
 
@@ -1169,6 +1303,38 @@ int launch_trees(treelstm* ctx, TreesKernel kernel, const TreesParams& p, int th
 
 }  // namespace
 
+// Fitted to whole calls, each way forced (caches cold; 1, 4, 25, 100 and 250 trees, balanced, chains and sentences, one large tree
+// among 24 sentences; TreeLSTM H = 64 to 256, TreeRNN 64 to 256, RNTN 16 and 32).  Forward / backward in us, clusters against
+// whole GPU: TreeLSTM H = 150, 25 sentences 100 / 163 against 170 / 298, chain of 1024 leaves 3 410 / 3 870 against 7 450 / 8 530,
+// balanced tree of 1024 leaves 945 / 848 against 166 / 240; TreeRNN H = 128, 25 sentences 51 / 112 against 351 / 361, balanced
+// tree of 8192 leaves 3 080 / 3 320 against 590 / 1 330.
+WalkCosts walk_costs(int cell, int H, bool backward) {
+  const float h = (float)H;
+  if (cell == kLstm) {
+    // a wavefront over the whole GPU: with the weights' slice resident in shared memory, or streamed (from H = 165 on)
+    if (!backward)
+      return {10.f, 0.35f + 0.0025f * fminf(h, 200.f), 1.9f, 1.5e-4f * h, 40.f, H <= 164 ? 3.2f + 0.0265f * h : 0.1f * h, fmaxf(0.f, 2.9e-4f * h - 0.0075f)};
+    return {66.f, 0.65f, 2.9f, 2e-4f * h, 105.f, 8.f, 1.5e-4f * h};
+  }
+  if (cell == kRnn) {
+    const float unit = 0.3f + 0.0011f * h;
+    if (!backward) return {15.f, unit, 1.2f, 0.f, 45.f, 1.5f + 0.157f * h, 2.5e-4f * h};
+    return {56.f, unit, 1.7f, 0.f, 85.f, 12.5f, 1.2e-3f * h};
+  }
+  if (!backward) return {18.f, 0.87f, 1.05f, 0.f, 50.f, 0.27f * h * h, 1.1e-4f * h * h};
+  return {56.f, 0.55f, 2.f, 0.f, 85.f, 3.9f * h, 4.2e-4f * h * h};
+}
+// Forests whose calls launch the tree kernels only.  A forest of n nodes gains most from the whole GPU as one balanced tree: it
+// is small if the clusters are the better way even then.  For TreeRNN and RNTN, where a second kernel that only looks and exits
+// would be 3 to 5 us of a call of 50 to 90, they may lose a quarter of the forward (25 sentences of 2 to 56 words have 1 450
+// nodes; TreeRNN, H = 128: up to 1 640), and the backward follows the forward.  TreeLSTM decides for the backward by itself,
+// since the size of its workspace hangs on it.
+bool trees_always_pay(int cell, int H, int n, bool backward) {
+  const WalkCosts c = walk_costs(cell, H, backward && cell == kLstm);
+  const float internal = (float)((n - 1) / 2), depth = ceilf(log2f(internal + 1.f));
+  return tree_cost(c, internal, depth, internal) <= (cell == kLstm ? 1.f : 1.25f) * grid_cost(c, depth, internal);
+}
+
 // Chooses the shapes and says how much device memory the register images take (0: the level kernels stream the
 // weights instead).
 size_t plan_trees(treelstm* ctx) {
@@ -1236,11 +1402,13 @@ bool trees_take(const treelstm* ctx, int n) {
          trees_smem(n, bwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0;
 }
 
-int trees_parts(const treelstm* ctx, int n, bool backward, bool after_running) {
+// clusters that a launch takes
+static int trees_parts(const treelstm* ctx, int n, bool backward, bool after_running) {
   const auto& t = ctx->trees;
   int clusters = backward ? t.clusters_bwd : t.clusters;
   if (after_running && !backward && (ctx->sm_count - 1) / t.s.cs < clusters) clusters = (ctx->sm_count - 1) / t.s.cs;   // a single scheduling CTA keeps its SM
   if (ctx->opt.max_ctas > 0 && ctx->opt.max_ctas / t.s.cs < clusters) clusters = ctx->opt.max_ctas / t.s.cs;
+  if (clusters > kMaxTreeClusters) clusters = kMaxTreeClusters;
   if (clusters > n) clusters = n;                        // (a tree is a node at least)
   return clusters < 1 ? 1 : clusters;
 }
@@ -1250,6 +1418,8 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
   const auto& s = ctx->trees.s;
   TreesParams p = trees_params(ctx, n, left, right, token, h, c, ws, lay);
   p.W = ctx->trees.Wf;
+  p.costs = walk_costs(ctx->cell, ctx->H, false);
+  p.choose = !trees_always_pay(ctx->cell, ctx->H, n, false);
   p.gates = save_gates ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
   if (ctx->cell == kLstm) {
     LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->trees.Wx, ctx->b, h, c, p.gates,
@@ -1271,6 +1441,8 @@ int launch_backward_trees(treelstm* ctx, cudaStream_t stream) {
   const auto& L = ctx->last;
   TreesParams p = trees_params(ctx, L.n, L.left, L.right, L.token, L.h, L.c, L.ws, L.lay);
   p.W = ctx->trees.Wb;
+  p.costs = walk_costs(ctx->cell, ctx->H, true);
+  p.choose = !trees_always_pay(ctx->cell, ctx->H, L.n, true);
   p.gates = reinterpret_cast<float*>(static_cast<char*>(L.ws) + L.lay.gates);
   if (p.trace) p.trace += kTraceSlots * kTraceLevels;
   return launch_trees(ctx, backward_kernel(ctx->cell, p.s), p, p.s.bthreads, trees_parts(ctx, L.n, true, true), true, stream);

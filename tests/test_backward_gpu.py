@@ -233,3 +233,23 @@ def test_classifier_of_every_width(H, classes):
                                  params.bc, labels)
     model = util.make_model(params, "fp32")
     _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("H,shapes", [(40, "one large tree"), (40, "chains"), (33, "leaves"), (150, "chains"), (200, "sentences")])
+def test_large_forests_on_either_way(H, shapes):
+    """forests beyond those that always go to the clusters, decided from the fullest cluster and the depth: one large tree
+    among small ones and wide wavefronts go over the whole GPU, few deep trees and many small ones to the clusters"""
+    rng = np.random.default_rng(1000 + H)
+    params = fg.draw_params(rng, H, 30, 70, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    shape = {"one large tree": lambda: [fg.balanced_shape(512)] + [fg.random_split_shape(rng, 12) for _ in range(20)],
+             "chains": lambda: [fg.left_chain_shape(150), fg.left_chain_shape(70)] + [fg.random_split_shape(rng, 20)],
+             "leaves": lambda: [fg.balanced_shape(256)] * 2 + [None] * 600,
+             "sentences": lambda: [fg.random_split_shape(rng, int(n)) for n in rng.integers(1, 40, size=30)]}[shapes]
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shape(), rng, 70), rng)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    res = _train_step(model, forest, labels, binding.PERSISTENT)
+    assert util.max_abs(res["h"], ref["h"]) < util.TOL["fp32"]
+    _compare(res, ref, util.TOL["fp32"])

@@ -199,6 +199,46 @@ def test_states_that_do_not_fit_shared_memory():
     _training_step(binding.CELL_TREERNN, p, forest, binding.PERSISTENT)
 
 
+LARGE = {"few large trees": lambda rng: [fg.balanced_shape(1024)] + [fg.random_split_shape(rng, 9) for _ in range(7)] + [None],
+         "one chain": lambda rng: [fg.left_chain_shape(900)],
+         "many trees": lambda rng: [fg.random_split_shape(rng, int(n)) for n in rng.integers(1, 30, size=120)],
+         "tables that fill shared memory": lambda rng: [fg.random_split_shape(rng, int(n)) for n in rng.integers(2, 56, size=310)]}
+
+
+@pytest.mark.parametrize("kind", LARGE)
+@pytest.mark.parametrize("cell,H", [(binding.CELL_TREERNN, 20), (binding.CELL_TREERNN, 130), (binding.CELL_RNTN, 8)])
+def test_large_forests_on_either_way(cell, H, kind):
+    """forests beyond those that always go to the clusters: the tree kernel leaves some of them to the kernels that take a
+    wavefront over the whole GPU, forward and backward, and walks the others, from a sample of their nodes"""
+    rng = np.random.default_rng(900 + H)
+    tensor = cell == binding.CELL_RNTN
+    p = fg.draw_recursive_params(rng, H, 90, tensor=tensor, emb_scale=0.8, w_scale=1.0 / np.sqrt(2 * H), v_scale=1.0 / (2 * H))
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(LARGE[kind](rng), rng, 90), rng)
+    _training_step(cell, p, forest, binding.PERSISTENT)
+
+
+@pytest.mark.parametrize("kind", ["two callers", "itself", "cycle"])
+def test_large_malformed_forests_return_errors(kind):
+    """the ways are chosen from the arrays before anything has validated them"""
+    rng = np.random.default_rng(950)
+    p = fg.draw_recursive_params(rng, 20, 90, tensor=False, emb_scale=0.8, w_scale=0.2)
+    forest = fg.forest_from_shapes([fg.balanced_shape(1024)] * 2, rng, 90)
+    left, right = forest.left.copy(), forest.right.copy()
+    inner = np.flatnonzero(left >= 0)
+    if kind == "two callers":
+        left[inner[7]] = left[inner[300]]
+    elif kind == "itself":
+        right[inner[40]] = inner[40]
+    else:                                       # a node below the root calls the root
+        left[inner[3]] = forest.roots[0]
+    model = _model(binding.CELL_TREERNN, p)
+    with pytest.raises(binding.TreeLSTMError) as err:
+        model.forward(util.to_dev(left), util.to_dev(right), util.to_dev(forest.token), flags=binding.PERSISTENT)
+    assert err.value.code == binding.ERR_INVALID_FOREST
+    _check(binding.CELL_TREERNN, p, forest, binding.PERSISTENT)
+    model.close()
+
+
 @pytest.mark.parametrize("cell,n_trees,hi", [(binding.CELL_TREERNN, 20, 40), (binding.CELL_TREERNN, 1, 1),
                                              (binding.CELL_RNTN, 20, 24), (binding.CELL_RNTN, 1, 1)])
 def test_label_out_of_range_reaches_no_gradient(cell, n_trees, hi):
