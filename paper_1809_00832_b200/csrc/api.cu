@@ -42,7 +42,7 @@ WsLayout ws_layout(const treelstm* ctx, int n, bool with_backward) {
   }
   L.img_dz = L.img_x0 = L.img_x1 = L.img_end = off;
   // forests that the tree kernels may be too slow for: operands of the backward pass split into bf16 pieces
-  if (with_backward && ctx->wsp && !trees_always_pay(ctx->cell, ctx->H, (int)nn, true)) {
+  if (with_backward && wide_backward_bytes(ctx) > 0 && !trees_always_pay(ctx->cell, ctx->H, (int)nn, true)) {
     L.img_dz = take(image_bytes((int)nn, 5 * gate_pitch(ctx->H)));
     L.img_x0 = take(image_bytes((int)nn, ctx->E + 1));
     L.img_x1 = take(image_bytes((int)nn, 2 * ctx->H + 1));
@@ -71,11 +71,46 @@ int copy_params(treelstm* ctx, const float* emb, const float* W, const float* b,
     int rc = pack_weights_bf16(ctx, s);
     if (rc != TREELSTM_OK) return rc;
   }
-  int rc = pack_trees(ctx, s);
+  int rc = pack_trees(ctx, true, true, s);
   if (rc == TREELSTM_OK) rc = pack_wide_backward(ctx, s);
   if (rc != TREELSTM_OK) return rc;
   TL_CUDA(ctx, cudaStreamSynchronize(s));
   return TREELSTM_OK;
+}
+
+// Room for a classifier, and the images of the weights that only a backward pass reads: a context that never gets a
+// classifier has none, and treelstm_update_weights keeps them up to date from then on.  One allocation (each costs a third of
+// a millisecond).  The caller waits for `s`.
+int ensure_backward_memory(treelstm* ctx, cudaStream_t s) {
+  if (ctx->memory_bwd) return TREELSTM_OK;
+  const size_t trees = tree_backward_bytes(ctx), wide = wide_backward_bytes(ctx);
+  int dev = -1;
+  TL_CUDA(ctx, cudaGetDevice(&dev));
+  if (dev != ctx->device) {              // the classifier may be set with another device current
+    TL_CUDA(ctx, cudaSetDevice(ctx->device));
+    s = nullptr;
+  }
+  int rc = TREELSTM_OK;
+  const cudaError_t e = cudaMalloc((void**)&ctx->memory_bwd, trees + wide + sizeof(float) * ((size_t)ctx->H + 1) * kMaxClasses);
+  if (e != cudaSuccess) {
+    ctx->cuda_error = (int)e;
+    cudaGetLastError();
+    ctx->memory_bwd = nullptr;
+    rc = TREELSTM_ERR_CUDA;
+  } else {
+    ctx->trees.Wb = trees ? reinterpret_cast<float*>(ctx->memory_bwd) : nullptr;
+    ctx->wsp = wide ? ctx->memory_bwd + trees : nullptr;
+    ctx->Wc = reinterpret_cast<float*>(ctx->memory_bwd + trees + wide);
+    rc = pack_trees(ctx, false, true, s);
+    if (rc == TREELSTM_OK) rc = pack_wide_backward(ctx, s);
+    if (rc == TREELSTM_OK && dev != ctx->device && cudaStreamSynchronize(s) != cudaSuccess) rc = TREELSTM_ERR_CUDA;
+    if (rc != TREELSTM_OK) {
+      cudaFree(ctx->memory_bwd);
+      ctx->memory_bwd = nullptr; ctx->trees.Wb = nullptr; ctx->wsp = nullptr; ctx->Wc = nullptr;
+    }
+  }
+  if (dev != ctx->device) TL_CUDA(ctx, cudaSetDevice(dev));
+  return rc;
 }
 
 void free_host_path(treelstm* ctx) {
@@ -241,7 +276,6 @@ int treelstm_create(treelstm_t** out, int H, int E, int vocab, const float* emb,
       take(ctx->bp_x, 4 * groups * 24);
     }
     take(images, trees);
-    if (const size_t split = wide_backward_bytes(ctx)) take(ctx->wsp, split);
     if (!pass && (cudaMalloc((void**)&ctx->memory, off) != cudaSuccess ||
                   cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess))
       return fail(TREELSTM_ERR_CUDA);
@@ -295,7 +329,7 @@ int treelstm_create_recursive(treelstm_t** out, int cell, int H, int vocab, cons
       cudaMemcpyAsync(ctx->b, b, sizeof(float) * Hs, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return fail(TREELSTM_ERR_CUDA);
   rc = pack_weights_rec(ctx, W, V, s);
-  if (rc == TREELSTM_OK) rc = pack_trees(ctx, s);
+  if (rc == TREELSTM_OK) rc = pack_trees(ctx, true, false, s);
   if (rc != TREELSTM_OK) return fail(rc);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(TREELSTM_ERR_CUDA);
   *out = ctx;
@@ -311,12 +345,13 @@ int treelstm_update_weights(treelstm_t* ctx, const float* emb, const float* W, c
 
 int treelstm_set_classifier(treelstm_t* ctx, int C, const float* Wc, const float* bc, void* stream) {
   if (!ctx || !Wc || !bc || C < 1) return TREELSTM_ERR_INVALID_ARG;
-  if (C > 32) return TREELSTM_ERR_UNSUPPORTED;
+  if (C > kMaxClasses) return TREELSTM_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaFree(ctx->Wc); cudaFree(ctx->bc);
-  ctx->Wc = ctx->bc = nullptr; ctx->C = 0;
-  TL_CUDA(ctx, cudaMalloc((void**)&ctx->Wc, sizeof(float) * ctx->H * C));
-  TL_CUDA(ctx, cudaMalloc((void**)&ctx->bc, sizeof(float) * C));
+  if (ctx->C > 0) TL_CUDA(ctx, cudaDeviceSynchronize());   // a backward on another stream may still read the old one
+  ctx->C = 0;
+  const int rc = ensure_backward_memory(ctx, s);
+  if (rc != TREELSTM_OK) return rc;
+  ctx->bc = ctx->Wc + (size_t)ctx->H * C;
   TL_CUDA(ctx, cudaMemcpyAsync(ctx->Wc, Wc, sizeof(float) * ctx->H * C, cudaMemcpyDeviceToDevice, s));
   TL_CUDA(ctx, cudaMemcpyAsync(ctx->bc, bc, sizeof(float) * C, cudaMemcpyDeviceToDevice, s));
   TL_CUDA(ctx, cudaStreamSynchronize(s));
@@ -663,7 +698,7 @@ int treelstm_last_cuda_error(const treelstm_t* ctx) { return ctx ? ctx->cuda_err
 
 int treelstm_destroy(treelstm_t* ctx) {
   if (!ctx) return TREELSTM_OK;
-  cudaFree(ctx->memory); cudaFree(ctx->Wc); cudaFree(ctx->bc);
+  cudaFree(ctx->memory); cudaFree(ctx->memory_bwd);
   if (ctx->host_level_offset) cudaFreeHost(ctx->host_level_offset);
   if (ctx->host_status) cudaFreeHost(ctx->host_status);
   free_host_path(ctx);

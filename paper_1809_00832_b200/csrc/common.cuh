@@ -62,6 +62,7 @@ struct Options {
   int overlap_launch = 1;      // persistent bf16 forward: the wavefront kernel starts under the scheduler (programmatic dependent launch)
 };
 
+constexpr int kMaxClasses = 32;          // a lane per class
 constexpr int kRadixBins = 256;
 constexpr int kRadixChunk = 1024;        // items per single-warp CTA of the multi-CTA sort
 constexpr int kSchedSingleMaxNodes = 32768;
@@ -137,14 +138,15 @@ struct treelstm {
   int sched_cluster = 0;   // CTAs of the scheduling cluster (0: none fits the device)
 
   unsigned char* memory = nullptr;  // one allocation: everything the library owns on the device but the classifier
+  unsigned char* memory_bwd = nullptr;   // the classifier and the weights as the backward pass wants them: made with the first classifier
 
   // fp32 parameters (library-owned device copies)
   float* emb = nullptr;  // [vocab][E]
   float* W = nullptr;    // [E+2H][5H]
   float* b = nullptr;    // [5H]
-  unsigned char* wsp = nullptr;   // W split into bf16 pieces for the wide backward (split_tc.cuh), nullptr: not kept
+  unsigned char* wsp = nullptr;   // W split into bf16 pieces for the wide backward (split_tc.cuh), in memory_bwd
   float* Wcat = nullptr; // TreeRNN / RNTN: [4H^2 + 2H][H] (tensor slices transposed, then W) or [2H][H]
-  float* Wc = nullptr;   // [H][C]
+  float* Wc = nullptr;   // [H][C], bc behind it (memory_bwd)
   float* bc = nullptr;   // [C]
 
   // bf16 tensor-core path (library-owned)
@@ -167,7 +169,7 @@ struct treelstm {
   struct Trees {
     bool ok = false;
     tl::TreesShape s;
-    float *Wf = nullptr, *Wb = nullptr;                 // register images of the weights
+    float *Wf = nullptr, *Wb = nullptr;                 // register images of the weights: forward (not with bf16), backward (memory_bwd)
     float* Wx = nullptr;                                // input weights of the leaves' gates, by slices of units
     int clusters = 0, clusters_bwd = 0;                 // that the device holds at once
     ushort2* pairs = nullptr;                           // RNTN: operands of every input chunk
@@ -245,9 +247,10 @@ int launch_forward_rec(treelstm* ctx, int n, const int32_t* left, const int32_t*
                        const WsLayout& lay, cudaStream_t stream);
 
 // trees_fp32.cu (all cells in fp32, trees dealt out to clusters)
-size_t plan_trees(treelstm* ctx);                        // bytes of the register images of the weights (0: not available)
+size_t plan_trees(treelstm* ctx);                        // bytes of the forward's images of the weights
+size_t tree_backward_bytes(const treelstm* ctx);         // and of the backward's
 int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream);
-int pack_trees(treelstm* ctx, cudaStream_t stream);      // after the weights have changed
+int pack_trees(treelstm* ctx, bool forward, bool backward, cudaStream_t stream);   // after the weights have changed
 bool trees_take(const treelstm* ctx, int n);
 int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
                          float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
@@ -293,7 +296,7 @@ struct BwdImages;   // split_tc.cuh
 __host__ __device__ inline int gate_pitch(int H) { return (H + 7) / 8 * 8; }
 // dweight_tc.cu: dW += In^T dZ, db += sum dZ, dEmb_rows += dz_leaves W_x^T on the tensor cores (three bf16 pieces per fp32 value)
 int init_dweight_tc_attributes(treelstm* ctx);
-size_t wide_backward_bytes(const treelstm* ctx);         // split image of W (0: not kept)
+size_t wide_backward_bytes(const treelstm* ctx);         // split image of W (0: these sizes have none)
 int pack_wide_backward(treelstm* ctx, cudaStream_t stream);
 size_t image_bytes(int n, int features);
 int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t* level_offset, const int32_t* token,

@@ -665,12 +665,9 @@ struct LeafParams {
 };
 // image of the input weights: [slice of 32 units][input unit][gate i, o, u][unit], zeros behind the last unit
 __host__ __device__ inline size_t leaf_image_words(int H, int E) { return (size_t)((H + kLeafU - 1) / kLeafU) * E * 3 * kLeafU; }
-__global__ void k_leaves_pack(int H, int E, const float* W, float* out) {
-  const int total = (int)leaf_image_words(H, E);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int uu = i % kLeafU, g = i / kLeafU % 3, k = i / (3 * kLeafU) % E, u = i / (3 * kLeafU) / E * kLeafU + uu;
-    out[i] = u < H ? W[(size_t)k * 5 * H + (g ? g + 2 : 0) * H + u] : 0.f;
-  }
+__device__ __forceinline__ float leaf_weight(int H, int E, const float* W, int i) {
+  const int uu = i % kLeafU, g = i / kLeafU % 3, k = i / (3 * kLeafU) % E, u = i / (3 * kLeafU) / E * kLeafU + uu;
+  return u < H ? W[(size_t)k * 5 * H + (g ? g + 2 : 0) * H + u] : 0.f;
 }
 // RPT rows from `rows` on and a quarter of nk contraction indices
 template <int RPT>
@@ -1188,16 +1185,30 @@ __global__ void __launch_bounds__(kGT) k_rec_grads(GradParams p) {
 
 
 // ---- register images and launches ------------------------------------------------------------------ //
-__global__ void k_trees_pack(int backward, int cell, int H, int E, int words, int threads, TreesShape s, const ushort2* pairs,
-                             const float* src, float* out) {
-  const int total = s.cs * words * threads;
+// The images that are wanted (out != nullptr), one after the other in one launch: it belongs to every change of the weights.
+struct PackParams {
+  int cell, H, E, fwd_words, bwd_words;
+  TreesShape s;
+  const ushort2* pairs;
+  const float* src;
+  float *fwd, *bwd, *leaves;
+};
+__global__ void k_trees_pack(const __grid_constant__ PackParams p) {
+  const int n_fwd = p.fwd ? p.s.cs * p.fwd_words * kFwdT : 0, n_bwd = p.bwd ? p.s.cs * p.bwd_words * p.s.bthreads : 0;
+  const int total = n_fwd + n_bwd + (p.leaves ? (int)leaf_image_words(p.H, p.E) : 0);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int t = i % threads, w = (i / threads) % words, rank = i / threads / words;
-    const WeightAt at = backward ? bwd_weight(cell, H, E, s, rank, t, w) : fwd_weight(cell, H, E, s, rank, t, w, pairs);
+    if (i >= n_fwd + n_bwd) {
+      p.leaves[i - n_fwd - n_bwd] = leaf_weight(p.H, p.E, p.src, i - n_fwd - n_bwd);
+      continue;
+    }
+    const bool backward = i >= n_fwd;
+    const int at_i = backward ? i - n_fwd : i, threads = backward ? p.s.bthreads : kFwdT, words = backward ? p.bwd_words : p.fwd_words;
+    const int t = at_i % threads, w = (at_i / threads) % words, rank = at_i / threads / words;
+    const WeightAt at = backward ? bwd_weight(p.cell, p.H, p.E, p.s, rank, t, w) : fwd_weight(p.cell, p.H, p.E, p.s, rank, t, w, p.pairs);
     float v = 0.f;
-    if (at.i0 >= 0) v = src[at.i0];
-    if (at.i1 >= 0) v += src[at.i1];
-    out[i] = v;
+    if (at.i0 >= 0) v = p.src[at.i0];
+    if (at.i1 >= 0) v += p.src[at.i1];
+    (backward ? p.bwd : p.fwd)[at_i] = v;
   }
 }
 
@@ -1249,12 +1260,16 @@ TreesKernel backward_kernel(int cell, const TreesShape& s) {
 
 // RNTN chunks of row a of x: products x_a x_b, b >= a, four b at a time; a = 2 Hp stands for x itself
 __host__ __device__ inline int pair_chunks(int a, int H, int Hp) { return a == 2 * Hp ? Hp / 2 : (a % Hp < H ? Hp / 2 - a / 4 : 0); }
-__global__ void k_trees_pairs(int H, ushort2* pairs) {
-  const int Hp = (H + 3) & ~3;
-  for (int a = 0, at = 0; a <= 2 * Hp; ++a)
-    for (int c = 0, n = pair_chunks(a, H, Hp); c < n; ++c)
-      pairs[at++] = a == 2 * Hp ? make_ushort2(0xFFFF, (unsigned short)(4 * c)) : make_ushort2((unsigned short)a, (unsigned short)(4 * (a / 4 + c)));
+__global__ void k_trees_pairs(int H, ushort2* pairs) {   // a thread per row
+  const int Hp = (H + 3) & ~3, a = threadIdx.x;
+  if (a > 2 * Hp) return;
+  int at = 0;
+  for (int b = 0; b < a; ++b) at += pair_chunks(b, H, Hp);
+  for (int c = 0, n = pair_chunks(a, H, Hp); c < n; ++c)
+    pairs[at + c] = a == 2 * Hp ? make_ushort2(0xFFFF, (unsigned short)(4 * c)) : make_ushort2((unsigned short)a, (unsigned short)(4 * (a / 4 + c)));
 }
+constexpr int kPairsT = 128;
+static_assert(2 * kRntnMaxH + 1 <= kPairsT, "a thread for every row of x, and one for x itself");
 size_t images_bytes(const treelstm* ctx, int what) {     // forward image, backward image, chunk operands, leaves' weights
   const auto& s = ctx->trees.s;
   const size_t cta = sizeof(float) * (size_t)s.cs;
@@ -1347,7 +1362,8 @@ size_t plan_trees(treelstm* ctx) {
   // (TreeRNN: four CTAs at least from H = 64 on: 25 trees, H = 128, forward / backward on clusters of 1, 2, 4, 8 CTAs:
   // 58.6 / 142, 60.6 / 133, 56.0 / 124, 67.2 / 122 us)
   for (int cs = cell == kRnn && H >= 64 ? 4 : 1; cs <= 16 && !t.ok; cs *= 2) t.ok = shape_fits(cell, H, cs, s);
-  for (int back = 0; back < 2 && t.ok; ++back) {
+  const bool forward = ctx->precision == TREELSTM_FP32;     // (the bf16 forward has kernels of its own)
+  for (int back = forward ? 0 : 1; back < 2 && t.ok; ++back) {
     TreesKernel k = back ? backward_kernel(cell, s) : forward_kernel(cell);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at;
@@ -1362,35 +1378,38 @@ size_t plan_trees(treelstm* ctx) {
     (back ? t.clusters_bwd : t.clusters) = clusters;
   }
   if (!t.ok) { cudaGetLastError(); return 0; }
-  if (cell == kLstm && cudaFuncSetAttribute(k_leaves_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem) != cudaSuccess) {
+  if (forward && cell == kLstm && cudaFuncSetAttribute(k_leaves_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem) != cudaSuccess) {
     cudaGetLastError();
     t.ok = false;
     return 0;
   }
-  return images_bytes(ctx, 0) + images_bytes(ctx, 1) + images_bytes(ctx, 2) + images_bytes(ctx, 3);
+  return forward ? images_bytes(ctx, 0) + images_bytes(ctx, 2) + images_bytes(ctx, 3) : 0;
 }
+size_t tree_backward_bytes(const treelstm* ctx) { return ctx->trees.ok ? images_bytes(ctx, 1) : 0; }
 
 int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream) {
   auto& t = ctx->trees;
-  if (!t.ok) return TREELSTM_OK;
+  if (!t.ok || ctx->precision != TREELSTM_FP32) return TREELSTM_OK;
   t.Wf = reinterpret_cast<float*>(memory);
-  t.Wb = reinterpret_cast<float*>(memory + images_bytes(ctx, 0));
-  t.pairs = reinterpret_cast<ushort2*>(memory + images_bytes(ctx, 0) + images_bytes(ctx, 1));
-  t.Wx = reinterpret_cast<float*>(memory + images_bytes(ctx, 0) + images_bytes(ctx, 1) + images_bytes(ctx, 2));
-  if (ctx->cell == kRntn) k_trees_pairs<<<1, 1, 0, stream>>>(ctx->H, t.pairs);
+  t.pairs = reinterpret_cast<ushort2*>(memory + images_bytes(ctx, 0));
+  t.Wx = reinterpret_cast<float*>(memory + images_bytes(ctx, 0) + images_bytes(ctx, 2));
+  if (ctx->cell == kRntn) k_trees_pairs<<<1, kPairsT, 0, stream>>>(ctx->H, t.pairs);
   TL_CUDA(ctx, cudaGetLastError());
   return TREELSTM_OK;
 }
 
-int pack_trees(treelstm* ctx, cudaStream_t stream) {
+int pack_trees(treelstm* ctx, bool forward, bool backward, cudaStream_t stream) {
   const auto& t = ctx->trees;
-  const auto& s = t.s;
   if (!t.ok) return TREELSTM_OK;
-  const int H = ctx->H, E = ctx->E, cell = ctx->cell;
-  const float* src = cell == kLstm ? ctx->W : ctx->Wcat;
-  k_trees_pack<<<592, 256, 0, stream>>>(0, cell, H, E, fwd_words(cell), kFwdT, s, t.pairs, src, t.Wf);
-  k_trees_pack<<<592, 256, 0, stream>>>(1, cell, H, E, bwd_words(cell, s), s.bthreads, s, t.pairs, src, t.Wb);
-  if (cell == kLstm) k_leaves_pack<<<592, 256, 0, stream>>>(H, E, ctx->W, t.Wx);
+  PackParams p{};
+  p.cell = ctx->cell; p.H = ctx->H; p.E = ctx->E; p.s = t.s; p.pairs = t.pairs;
+  p.fwd_words = fwd_words(ctx->cell); p.bwd_words = bwd_words(ctx->cell, t.s);
+  p.src = ctx->cell == kLstm ? ctx->W : ctx->Wcat;
+  p.fwd = forward ? t.Wf : nullptr;
+  p.leaves = forward && ctx->cell == kLstm ? t.Wx : nullptr;
+  p.bwd = backward ? t.Wb : nullptr;
+  if (!p.fwd && !p.bwd) return TREELSTM_OK;
+  k_trees_pack<<<592, 256, 0, stream>>>(p);
   TL_CUDA(ctx, cudaGetLastError());
   return TREELSTM_OK;
 }

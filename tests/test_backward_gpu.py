@@ -253,3 +253,38 @@ def test_large_forests_on_either_way(H, shapes):
     res = _train_step(model, forest, labels, binding.PERSISTENT)
     assert util.max_abs(res["h"], ref["h"]) < util.TOL["fp32"]
     _compare(res, ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("precision,n_trees", [("fp32", 6), ("bf16", 6), ("fp32", 90), ("bf16", 90)])
+def test_weights_of_the_backward_come_with_the_classifier_and_follow_every_update(precision, n_trees):
+    """a context without a classifier keeps no weights in the layouts that only the backward reads; the classifier may come
+    between forward and backward; new weights reach every layout (tree clusters and wide wavefronts)"""
+    rng = np.random.default_rng(1100 + n_trees)
+    draw = lambda: fg.draw_params(rng, 256, 300, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.04, n_classes=3)
+    params, other = draw(), draw()
+    forest = fg.random_forest(rng, n_trees, 2, 30, 60)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    util.lib_ready()
+    arrs = [util.to_dev(a) for a in (forest.left, forest.right, forest.token, labels)]
+    weights = [[util.to_dev(a) for a in (p.emb, p.W, p.b, p.Wc, p.bc)] for p in (params, other)]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    model = binding.TreeLSTM(256, 300, 60, *weights[0][:3], binding.FP32 if precision == "fp32" else binding.BF16)
+    assert before - torch.cuda.mem_get_info()[0] <= 12 << 20      # W 4.2 MB and one image of it; with the backward's two: 16 and more
+    need = model.workspace_bytes(forest.n_nodes, True)
+    model.forward(*arrs[:3], flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+    model.set_classifier(*weights[0][3:])
+    assert model.workspace_bytes(forest.n_nodes, True) == need
+    for k, p in ((0, params), (1, other)):
+        if k:
+            model.update_weights(*weights[1][:3])
+            model.set_classifier(*weights[1][3:])
+            model.forward(*arrs[:3], flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+        res = {q: v.cpu().numpy() for q, v in model.backward(arrs[3], forest.n_leaves).items()}
+        ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, p.emb, p.W, p.b, p.Wc, p.bc, labels)
+        for q in ("dW", "db", "dWc", "dbc"):
+            assert util.max_abs(res[q], ref[q]) <= util.REL[precision] * float(np.abs(ref[q]).max()), q
+        n = int(res["n_touched"][0])
+        assert util.max_abs(res["dEmb_rows"][:n], ref["dEmb_rows"]) <= util.REL[precision] * float(np.abs(ref["dEmb_rows"]).max())
+    model.close()
