@@ -213,12 +213,16 @@ int finish_status(treelstm* ctx) {
   return st;
 }
 
-// Whether a kernel may write to host memory at `ptr` (pinned, at the same address on the device); NULL: nothing to write.
-bool gpu_writable(const void* ptr) {
-  if (!ptr) return true;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) { cudaGetLastError(); return false; }
-  return a.type == cudaMemoryTypeHost && a.devicePointer == ptr;
+// Whether a kernel may write to `bytes` bytes of host memory at `ptr` (pinned, at the same address on the device): the first
+// and the last of them are looked at, since a registered range may be shorter than what the caller says.  NULL: nothing to write.
+bool gpu_writable(const void* ptr, size_t bytes) {
+  if (!ptr || bytes == 0) return true;
+  for (const char* at : {static_cast<const char*>(ptr), static_cast<const char*>(ptr) + bytes - 1}) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, at) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (a.type != cudaMemoryTypeHost || a.devicePointer != at) return false;
+  }
+  return true;
 }
 
 // used by backward.cu
@@ -543,6 +547,7 @@ int treelstm_forward_host(treelstm_t* ctx, int n_nodes, const int32_t* left, con
   if (!ctx || n_nodes < 0 || max_roots < 0) return TREELSTM_ERR_INVALID_ARG;
   if (n_nodes > 0 && (!left || !right || !token)) return TREELSTM_ERR_INVALID_ARG;
   if (flags & TREELSTM_SAVE_FOR_BACKWARD) return TREELSTM_ERR_INVALID_ARG;
+  if (ctx->cell != 0) c = root_c = nullptr;   // these cells have no cell state
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (!on_own_device(ctx)) return TREELSTM_ERR_STATE;
   auto& p = ctx->hp;
@@ -608,7 +613,12 @@ int treelstm_forward_host(treelstm_t* ctx, int n_nodes, const int32_t* left, con
   p.root_c = p.root_h + (size_t)max_r * H;
   // Roots whose destinations are pinned are written there by the gathering kernel itself, and so is the control
   // block: two copies less behind it on the stream.
-  const bool direct = want_roots && max_r > 0 && gpu_writable(root_ids) && gpu_writable(root_h) && gpu_writable(root_c);
+  const size_t id_bytes = 4 * (size_t)max_r, row_bytes = id_bytes * H;
+  const bool one_range = root_ids && root_h == reinterpret_cast<float*>(root_ids + max_r) && root_c == root_h + (size_t)max_r * H;
+  const bool direct = want_roots && max_r > 0 &&
+                      (one_range ? gpu_writable(root_ids, id_bytes + 2 * row_bytes)
+                                 : gpu_writable(root_ids, id_bytes) && gpu_writable(root_h, row_bytes) &&
+                                       gpu_writable(root_c, row_bytes));
   if (want_roots) {
     rc = direct ? launch_gather_roots(ctx, max_r, root_ids, root_h, root_c, nullptr, ctx->host_status, s)
                 : launch_gather_roots(ctx, max_r, p.root_ids, p.root_h, p.root_c, p.n_roots, nullptr, s);
@@ -616,20 +626,19 @@ int treelstm_forward_host(treelstm_t* ctx, int n_nodes, const int32_t* left, con
   }
   if (n_nodes > 0) {
     if (h) TL_CUDA(ctx, cudaMemcpyAsync(h, p.h, nb * H, cudaMemcpyDeviceToHost, s));
-    if (c && ctx->cell == 0) TL_CUDA(ctx, cudaMemcpyAsync(c, p.c, nb * H, cudaMemcpyDeviceToHost, s));
+    if (c) TL_CUDA(ctx, cudaMemcpyAsync(c, p.c, nb * H, cudaMemcpyDeviceToHost, s));
     if (level) TL_CUDA(ctx, cudaMemcpyAsync(level, p.level, nb, cudaMemcpyDeviceToHost, s));
     if (order) TL_CUDA(ctx, cudaMemcpyAsync(order, p.order, nb, cudaMemcpyDeviceToHost, s));
   }
   if (want_roots && max_r > 0 && !direct) {
     // the number of roots is not known on the host yet: copy max_r rows (rows past n_roots are
     // unspecified) - callers pass the number of trees they submitted
-    if (root_ids && root_h && root_c && max_r == max_roots &&
-        root_h == reinterpret_cast<float*>(root_ids + max_r) && root_c == root_h + (size_t)max_r * H) {
-      TL_CUDA(ctx, cudaMemcpyAsync(root_ids, p.root_ids, (4 + 8 * H) * (size_t)max_r, cudaMemcpyDeviceToHost, s));
+    if (one_range && max_r == max_roots) {
+      TL_CUDA(ctx, cudaMemcpyAsync(root_ids, p.root_ids, id_bytes + 2 * row_bytes, cudaMemcpyDeviceToHost, s));
     } else {
-      if (root_ids) TL_CUDA(ctx, cudaMemcpyAsync(root_ids, p.root_ids, 4 * (size_t)max_r, cudaMemcpyDeviceToHost, s));
-      if (root_h) TL_CUDA(ctx, cudaMemcpyAsync(root_h, p.root_h, 4 * (size_t)max_r * H, cudaMemcpyDeviceToHost, s));
-      if (root_c) TL_CUDA(ctx, cudaMemcpyAsync(root_c, p.root_c, 4 * (size_t)max_r * H, cudaMemcpyDeviceToHost, s));
+      if (root_ids) TL_CUDA(ctx, cudaMemcpyAsync(root_ids, p.root_ids, id_bytes, cudaMemcpyDeviceToHost, s));
+      if (root_h) TL_CUDA(ctx, cudaMemcpyAsync(root_h, p.root_h, row_bytes, cudaMemcpyDeviceToHost, s));
+      if (root_c) TL_CUDA(ctx, cudaMemcpyAsync(root_c, p.root_c, row_bytes, cudaMemcpyDeviceToHost, s));
     }
   }
   // the level and root counts come back with the control block that the status read copies anyway

@@ -327,6 +327,7 @@ int launch_gather_roots(treelstm* ctx, int max_roots, int32_t* root_ids, float* 
     cudaError_t e_ = (expr);                                \
     if (e_ != cudaSuccess) {                                \
       (ctx)->cuda_error = (int)e_;                          \
+      cudaGetLastError(); /* reported: not the next call's */ \
       return TREELSTM_ERR_CUDA;                             \
     }                                                       \
   } while (0)

@@ -186,6 +186,38 @@ def test_host_buffer_forward():
     np.testing.assert_array_equal(out2["root_h"].numpy(), out["root_h"].numpy())
 
 
+def test_roots_into_memory_that_is_pinned_in_part():
+    """a registered range that ends before the last of max_roots rows: the kernel does not write there; the copy either
+    takes such memory or says that it does not, and the next call is not troubled by it"""
+    w = fg.make_workload("tiny8", 0)
+    f, H, m = w.forest, w.params.H, w.forest.n_nodes            # room for as many roots as there are nodes
+    model = util.make_model(w.params, "fp32")
+    host = [torch.from_numpy(a).pin_memory() for a in (f.left, f.right, f.token)]
+    good = model.forward_host(*host, max_roots=f.n_trees)
+    page = 4096
+    rows = (m * H * 4 + page - 1) // page + 1
+    raw = np.full((2 * rows + 2) * page, 7, np.uint8)
+    first = -raw.ctypes.data % page
+    root_h = torch.from_numpy(raw[first:first + m * H * 4].view(np.float32)).view(m, H)
+    root_c = torch.from_numpy(raw[first + rows * page:first + rows * page + m * H * 4].view(np.float32)).view(m, H)
+    assert m * H * 4 > page and root_h.data_ptr() % page == 0
+    out = dict(n_levels=torch.zeros(1, dtype=torch.int32, pin_memory=True), n_roots=torch.zeros(1, dtype=torch.int32, pin_memory=True),
+               root_ids=torch.zeros(m, dtype=torch.int32, pin_memory=True), root_h=root_h, root_c=root_c)
+    cudart = torch.cuda.cudart()
+    assert int(cudart.cudaHostRegister(root_h.data_ptr(), page, 0)) == 0
+    try:
+        model.forward_host(*host, max_roots=m, out=out)
+        assert int(out["n_roots"][0]) == f.n_trees
+        np.testing.assert_array_equal(root_h[:f.n_trees].numpy(), good["root_h"].numpy())
+    except binding.TreeLSTMError as err:
+        assert err.code == binding.ERR_CUDA
+    finally:
+        torch.cuda.synchronize()
+        assert int(cudart.cudaHostUnregister(root_h.data_ptr())) == 0
+    again = model.forward_host(*host, max_roots=f.n_trees)
+    np.testing.assert_array_equal(again["root_h"].numpy(), good["root_h"].numpy())
+
+
 def test_bounded_waits_time_out_cleanly():
     """failure detection without a fault: a wait on a flag that nothing sets ends by its cycle limit,
     the status word says TIMEOUT, and the context keeps working afterwards"""
