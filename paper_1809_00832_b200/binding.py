@@ -118,7 +118,7 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
 
 
 def _stream() -> int:
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())   # (no Stream object is made for it)
+    return torch.cuda.current_stream(torch.cuda.current_device()).cuda_stream
 
 
 STATIC_MAX_NODES = 16384

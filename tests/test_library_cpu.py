@@ -98,3 +98,11 @@ def test_tile_plan_invariants(lib):
     # a narrow wavefront gets small tiles (all SMs busy), a wide one fat tiles
     assert binding.tile_plan(123, 256, 300, 148, False)["rows_per_tile"] == 32
     assert binding.tile_plan(7240, 256, 300, 148, True)["groups_per_tile"] == 4
+
+
+def test_package_uses_public_torch_only():
+    """names that begin with an underscore may change with any release of torch"""
+    pkg = os.path.join(ROOT, "paper_1809_00832_b200")
+    for fn in sorted(os.listdir(pkg)):
+        if fn.endswith(".py"):
+            assert not re.search(r"\btorch\.(\w+\.)*_[a-zA-Z]", open(os.path.join(pkg, fn)).read()), fn
