@@ -275,7 +275,7 @@ def time_forward(model, forest, flags, steps, warmup, flush, kernel_every=16, ov
         return statistics.mean(ms)
 
     # the kernel of the timed steps, alone: the event in front of it makes it start when the scheduler has
-    # ended, its code and order of work (large bf16 forests: leaves first) stay those of the steps
+    # ended, its code and order of work stay those of the steps
     k_ms = kernel_pass()
     TIMINGS["kernel_ms_plain_order"] = None
     if overlap_launch is None or overlap_launch:
@@ -496,8 +496,6 @@ def main() -> int:
                     help="cell of the sweeps (the benchmark line itself is always TreeLSTM)")
     ap.add_argument("--tail-width", type=int, default=None,
                     help="sweeps only: widest wavefront handed to the one-cluster kernel (0 = never hand over)")
-    ap.add_argument("--leaves-first-min-nodes", type=int, default=None,
-                    help="headline run only: smallest forest whose leaf wavefront runs before the wait for the schedule")
     ap.add_argument("--overlap-launch", type=int, default=None, choices=[0, 1],
                     help="headline run only: 0 = plain stream order between the scheduler and the wavefront kernel")
     ap.add_argument("--sweep", default=None, choices=["shapes", "length", "all"],
@@ -539,8 +537,6 @@ def main() -> int:
     model = binding.TreeLSTM(p.H, p.E, p.vocab, _dev(p.emb), _dev(p.W), _dev(p.b), prec)
     if args.overlap_launch is not None:
         model.set_option(binding.OPT_OVERLAP_LAUNCH, args.overlap_launch)
-    if args.leaves_first_min_nodes is not None:
-        model.set_option(binding.OPT_LEAVES_FIRST_MIN_NODES, args.leaves_first_min_nodes)
     flags = {"persistent": binding.PERSISTENT, "per_level": binding.PER_LEVEL, "subforests": binding.SUBFORESTS}[args.mode]
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device="cuda")
 

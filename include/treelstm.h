@@ -124,11 +124,10 @@ typedef enum treelstm_status {
                                             /* itself; otherwise the bounded grid barrier ends the call    */
                                             /* with TREELSTM_ERR_TIMEOUT.  0: cooperative launch in plain  */
                                             /* stream order (residency guaranteed by the runtime)          */
-#define TREELSTM_OPT_LEAVES_FIRST_MIN_NODES 9 /* a kernel started that way evaluates the leaf wavefront    */
-                                            /* before it waits for the schedule if the forest has at least */
-                                            /* this many nodes (default 4096); smaller forests keep the    */
-                                            /* order of work of the cooperative launch: their scheduler    */
-                                            /* is too short to hide the two extra grid barriers            */
+#define TREELSTM_OPT_LEAVES_FIRST_MIN_NODES 9 /* accepted and without effect: an order of work that took   */
+                                            /* the leaves before the schedule was the slower one at every  */
+                                            /* size once forests from 4096 nodes on are scheduled by a     */
+                                            /* cluster                                                     */
 #define TREELSTM_OPT_DW_TENSOR_CORES 10     /* 1 (default): after a forward that kept its level table on   */
                                             /* the device, treelstm_backward forms dW, db, the input       */
                                             /* gradients of the leaves (dEmb_rows) and, in forests with    */

@@ -28,7 +28,6 @@ WsLayout ws_layout(const treelstm* ctx, int n, bool with_backward) {
     L.xin = take(2 * nn * (size_t)ctx->Ep);          // leaf embedding rows in ready order
     L.ain = take(2 * nn * 2 * (size_t)ctx->Hp);      // [h_l | h_r] of every position, bf16
     L.cin = take(4 * nn * 2 * (size_t)row_pitch(ctx->H));       // [c_l | c_r] of every position, fp32
-    L.pre = take(4 * 1024);                          // leaves per CTA (wavefront kernel started under the scheduler)
   }
   L.gates = L.dh = L.dc = L.dz = L.tok_slot = off;
   if (with_backward) {
@@ -385,8 +384,7 @@ int treelstm_set_option(treelstm_t* ctx, int key, long long value) {
       ctx->tail_skip = false;
       return TREELSTM_OK;
     case TREELSTM_OPT_LEAVES_FIRST_MIN_NODES:
-      ctx->opt.leaves_first_min_nodes = value > (1 << 30) ? (1 << 30) : (int)value;
-      return TREELSTM_OK;
+      return TREELSTM_OK;                    // (no effect any more)
     case TREELSTM_OPT_OVERLAP_LAUNCH:
       ctx->opt.overlap_launch = value != 0;
       return TREELSTM_OK;

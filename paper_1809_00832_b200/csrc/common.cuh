@@ -33,7 +33,7 @@ __host__ __device__ inline int row_pitch(int H) { return (H + 3) / 4 * 4; }
 
 struct WsLayout {
   size_t status, parent, pending, order_tmp, level_offset, roots, table, slot, part_order, part_offset,
-      part_spill, xin, ain, cin, gates, dh, dc, dz, tok_slot, trace, check, pre, img_dz, img_x0, img_x1, img_end, total;
+      part_spill, xin, ain, cin, gates, dh, dc, dz, tok_slot, trace, check, img_dz, img_x0, img_x1, img_end, total;
 };
 
 // Cycle stamps of the wavefront kernels (builds with -DTREELSTM_TRACE only): kTraceSlots stamps per
@@ -57,7 +57,6 @@ struct Options {
   int tail_width = 32;    // persistent bf16 forward: trailing wavefronts this narrow may run on one cluster (0: never)
   int tail_min_levels = 0; // > 0: hand them over if at least this many remain; 0: the device decides by its cost model
   int tail_max_nodes = 4096;   // forests with more nodes never launch the cluster kernel
-  int leaves_first_min_nodes = 4096;   // forests at least this large: leaf wavefront before the wait for the schedule
   int dw_tensor_cores = 1;     // one-launch backward: dW and db by split-bf16 tensor-core contraction
   int overlap_launch = 1;      // persistent bf16 forward: the wavefront kernel starts under the scheduler (programmatic dependent launch)
 };

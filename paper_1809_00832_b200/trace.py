@@ -148,14 +148,6 @@ def main() -> int:
               "starts known, placed = " + ", ".join(str(int(buf[8 + i])) for i in range(5)))
     for which, name in ((0, "grid-wide kernel"), (1, "cluster kernel")):
         t = read_trace(model, which)
-        if which == 0 and t[LEVELS - 1, 4] != 0:
-            ph = t[LEVELS - 1]
-            names = ("set up, own node ids read", "leaf counts of all CTAs known", "own leaves ranked, embedding rows copied",
-                     "all rows in place (leaf wavefront starts)", "leaf wavefront done everywhere", "scheduler ended, schedule read",
-                     "slots written, leaf states handed over", "first internal wavefront may start")
-            print("# grid-wide kernel started under the scheduler, first CTA, cycles since its start: " +
-                  ", ".join(f"{nm} {int(ph[i + 1] - ph[0])}" for i, nm in enumerate(names)))
-            t[LEVELS - 1] = 0
         rows = [l for l in range(min(len(widths), LEVELS)) if t[l, 0] != 0]
         if not rows:
             continue

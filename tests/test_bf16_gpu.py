@@ -286,9 +286,9 @@ def test_both_launch_forms_give_identical_states():
 
 
 def test_leaves_taken_first_on_small_grids_and_leaf_only_forests():
-    """the kernel started under the scheduler ranks the leaves itself (every CTA a share of the node
-    ids): same bits as the run in plain stream order on grids of 1, 5 and 40 CTAs (several node ids
-    per thread), on a forest of single-leaf trees only (one wavefront) and on a mixed one"""
+    """the kernel started under the scheduler: same bits as the run in plain stream order on grids of 1, 5
+    and 40 CTAs (several node ids per thread), on a forest of single-leaf trees only (one wavefront)
+    and on a mixed one; the option that once chose another order of work is still accepted"""
     rng = np.random.default_rng(50)
     params = fg.draw_params(rng, 128, 72, 400, emb_dist="normal", emb_scale=0.3, w_scale=0.15)
     forests = [fg.random_forest(rng, 37, 1, 1, 400),        # leaves only
@@ -302,7 +302,7 @@ def test_leaves_taken_first_on_small_grids_and_leaf_only_forests():
         h, c, _ = orc.forward_recursive(forest.left, forest.right, forest.token, params.emb, params.W, params.b)
         assert util.max_abs(ref["h"], h) < util.TOL["bf16"]
         model.set_option(binding.OPT_OVERLAP_LAUNCH, 1)
-        model.set_option(binding.OPT_LEAVES_FIRST_MIN_NODES, 0)     # these forests are below the default threshold
+        model.set_option(binding.OPT_LEAVES_FIRST_MIN_NODES, 0)
         for ctas in (0, 1, 5, 40):
             model.set_option(binding.OPT_MAX_CTAS, ctas)
             res = util.gpu_forward(model, forest, binding.PERSISTENT)
