@@ -117,8 +117,17 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
     return t
 
 
+def _public_raw_stream(device: int) -> int:
+    return torch.cuda.current_stream(device).cuda_stream
+
+
+# The handle alone, without a Stream object around it (0.3 us against 1.3, of a call of 70); a torch without it has the
+# public way.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", _public_raw_stream)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream(torch.cuda.current_device()).cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 STATIC_MAX_NODES = 16384

@@ -321,3 +321,10 @@ def test_fp32_leaves_at_the_limits_of_their_tiles(H, E, kind):
     res = util.gpu_forward(util.make_model(params, "fp32"), forest, binding.PERSISTENT)
     h, c, _ = orc.forward_recursive(forest.left, forest.right, forest.token, params.emb, params.W, params.b)
     assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
+
+
+def test_calls_go_to_the_current_stream():
+    device, other = torch.cuda.current_device(), torch.cuda.Stream()
+    assert binding._stream() == binding._public_raw_stream(device) == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(other):
+        assert binding._stream() == binding._public_raw_stream(device) == other.cuda_stream
