@@ -389,10 +389,10 @@ __device__ void trees_win(const TreesParams& p, const TreesSmem& s, float* sm, c
   }
 }
 // The tables of the forest, then what the cluster has to walk: nothing, if loads->win says that the forest is the next kernel's.
-__device__ __forceinline__ void deal_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, TreeLoads* loads, Walk* walk) {
+__device__ __forceinline__ void deal_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, bool choose, TreeLoads* loads, Walk* walk) {
   const int warp = (int)threadIdx.x >> 5;
   if (threadIdx.x == 0) loads->win = 1;
-  if (!p.choose) {
+  if (!choose) {
     load_kids(p, s, sm, nullptr);
     if (warp == 0) walk_trees(p, s, sm, part, parts, nullptr, walk);
     __syncthreads();
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   float w[RC * 4 * U];
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
-  deal_trees(p, s, sm, part, parts, &s_loads, &s_walk);
+  deal_trees(p, s, sm, part, parts, CELL != kLstm && p.choose, &s_loads, &s_walk);
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
@@ -457,9 +457,13 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     }
   }
   for (int e = tid; e < fwd_parts(CELL, p.s) * NT * outs; e += kFwdT) red[e] = 0.f;   // (sums beyond the segments stay zero)
-  if (CELL == kLstm) asm volatile("griddepcontrol.wait;" ::: "memory"); // the leaves' states come from the kernel ahead
+  int depths = walk.depths, leaves = walk.leaves;
+  if (CELL == kLstm) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the leaves' states come from the kernel ahead, and whose forest it is
+    if (p.choose && !ld_volatile(&p.st->trees_fwd)) depths = leaves = 0;
+  }
   cluster_sync(cs);                                      // every CTA of the cluster runs: its shared memory may be written
-  for (int q = warp; q < walk.leaves; q += kFwdT / 32) {
+  for (int q = warp; q < leaves; q += kFwdT / 32) {
     const int node = leaf[q];
     const unsigned code = leaf_par[q];
     const bool keep = resident && code != kNoCaller;
@@ -503,7 +507,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   const int parts_sum = fwd_parts(CELL, p.s);
   cluster_sync(cs);                                      // the leaves' states are in place
   TL_STAMP(trace, kTraceLevels - 1, 3);
-  for (int d = walk.depths - 1; d >= 0; --d) {
+  for (int d = depths - 1; d >= 0; --d) {
     for (int lo = start[d], hi = start[d + 1]; lo < hi; lo += NT) {
       const int cnt = min(NT, hi - lo);
       TL_STAMP(trace, d, 0);
@@ -638,7 +642,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   // what follows on the stream waits for this grid only: it must not end before the scheduler ahead of it has
   if (blockIdx.x == 0) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tid == 0) p.st->trees_fwd = s_loads.win;
+    if (CELL != kLstm && tid == 0) p.st->trees_fwd = s_loads.win;
   }
 }
 
@@ -662,6 +666,9 @@ struct LeafParams {
   float *h, *c, *gates;
   DevStatus* st;
   long long wait_limit;
+  int choose, parts;                       // 1: the first CTA says whether the clusters (so many) take the forest (trees_win)
+  const int* right;
+  WalkCosts costs;
 };
 // image of the input weights: [slice of 32 units][input unit][gate i, o, u][unit], zeros behind the last unit
 __host__ __device__ inline size_t leaf_image_words(int H, int E) { return (size_t)((H + kLeafU - 1) / kLeafU) * E * 3 * kLeafU; }
@@ -694,17 +701,36 @@ __device__ __forceinline__ void leaf_rows(const float* As, const float* Ws, int 
     }
   }
 }
-__global__ void __launch_bounds__(kLeafT) k_leaves_fp32(LeafParams p) {
+// The choice takes no time here: the clusters' kernel waits for the leaves anyhow, and one CTA more beside them is done before
+// they are.  (In the clusters' own kernel, beside the walk, it cost 2.5 us of 90.)
+constexpr int kLeafTableWords = kLeafSmem / 4;
+__host__ __device__ inline bool leaves_hold_tables(int n) { return n + 2 * (n / 32 + 1) + (n + 1) / 2 + 8 <= kLeafTableWords; }
+__device__ __forceinline__ void leaves_choose(const LeafParams& p, float* sm) {
+  __shared__ TreeLoads s_loads;
+  TreesParams q{};
+  q.n = p.n; q.vocab = p.vocab; q.left = p.left; q.right = p.right; q.token = p.token; q.costs = p.costs;
+  TreesSmem s{};
+  s.child = p.n;
+  const int words = (p.n + 1) / 2, at = s.child + p.n / 32 + 1;
+  const TreeLinks links{reinterpret_cast<unsigned short*>(sm + at), reinterpret_cast<int*>(sm + at + words), true};
+  if (threadIdx.x == 0) s_loads.win = 1;
+  if (!load_kids(q, s, sm, links.up) && threadIdx.x >= 32) trees_win(q, s, sm, links, p.parts, &s_loads);
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");     // the scheduler clears the control block at its start
+  if (threadIdx.x == 0) p.st->trees_fwd = s_loads.win;
+}
+__global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ LeafParams p) {
   extern __shared__ __align__(16) float leaf_smem[];
   float* const Ws = leaf_smem;                           // [kLeafK][3 gates][32 units]; then the second halves' sums
   float* const As = leaf_smem + kLeafK * 3 * kLeafU;     // [rows][pitch]
   __shared__ int s_node[kLeafIds], s_tok[kLeafIds], s_count, s_abort;
   __shared__ __align__(8) uint64_t s_bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = p.H, E = p.E;
-  const int tiles_u = (H + kLeafU - 1) / kLeafU, slice = (int)blockIdx.x % tiles_u;
-  const int id0 = (int)blockIdx.x / tiles_u * kLeafIds, u0 = slice * kLeafU;
+  const int tiles_u = (H + kLeafU - 1) / kLeafU, block = (int)blockIdx.x - p.choose, slice = block % tiles_u;
+  const int id0 = block / tiles_u * kLeafIds, u0 = slice * kLeafU;
   const uint32_t bar = smem_u32(&s_bar);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (p.choose && blockIdx.x == 0) { leaves_choose(p, leaf_smem); return; }
   auto ask = [&](int k0) {                               // one thread: the weights of the next kLeafK indices
     const uint32_t bytes = (uint32_t)min(kLeafK, E - k0) * 3 * kLeafU * 4;
     mbar_arrive_expect_tx(bar, bytes);
@@ -860,7 +886,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   if (CELL == kRntn)
     for (int e = tid; e < kND * 2 * Hp; e += nt) xs[e] = 0.f;
   TL_STAMP(trace, kTraceLevels - 1, 1);
-  deal_trees(p, s, sm, part, parts, &s_loads, &s_walk);
+  deal_trees(p, s, sm, part, parts, p.choose != 0, &s_loads, &s_walk);
 #pragma unroll
   for (int q = 0; q < kWords; ++q) asm volatile("" : "+f"(w[q]));       // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
@@ -1329,7 +1355,7 @@ WalkCosts walk_costs(int cell, int H, bool backward) {
     // a wavefront over the whole GPU: with the weights' slice resident in shared memory, or streamed (from H = 165 on)
     if (!backward)
       return {10.f, 0.35f + 0.0025f * fminf(h, 200.f), 1.9f, 1.5e-4f * h, 40.f, H <= 164 ? 3.2f + 0.0265f * h : 0.1f * h, fmaxf(0.f, 2.9e-4f * h - 0.0075f)};
-    return {66.f, 0.65f, 2.9f, 2e-4f * h, 105.f, 8.f, 1.5e-4f * h};
+    return {66.f, 0.65f, 2.9f, 2e-4f * h, H % 4 ? 150.f : 105.f, 8.f, 1.5e-4f * h};   // (rows that are no whole 16 bytes)
   }
   if (cell == kRnn) {
     const float unit = 0.3f + 0.0011f * h;
@@ -1417,7 +1443,7 @@ int pack_trees(treelstm* ctx, bool forward, bool backward, cudaStream_t stream) 
 // Forests whose tables fit shared memory; beyond that the level kernels are used.
 bool trees_take(const treelstm* ctx, int n) {
   const auto& s = ctx->trees.s;
-  return ctx->trees.ok && n >= 1 && n <= 32767 && trees_smem(n, fwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0 &&
+  return ctx->trees.ok && n >= 1 && n <= 32767 && leaves_hold_tables(n) && trees_smem(n, fwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0 &&
          trees_smem(n, bwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0;
 }
 
@@ -1439,12 +1465,13 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
   p.W = ctx->trees.Wf;
   p.costs = walk_costs(ctx->cell, ctx->H, false);
   p.choose = !trees_always_pay(ctx->cell, ctx->H, n, false);
+  const int parts = trees_parts(ctx, n, false, after_running);
   p.gates = save_gates ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
   if (ctx->cell == kLstm) {
     LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->trees.Wx, ctx->b, h, c, p.gates,
-                 p.st, ctx->opt.wait_limit_kcycles * 1024};
+                 p.st, ctx->opt.wait_limit_kcycles * 1024, p.choose, parts, right, p.costs};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((n + kLeafIds - 1) / kLeafIds * ((ctx->H + kLeafU - 1) / kLeafU));
+    cfg.gridDim = dim3((n + kLeafIds - 1) / kLeafIds * ((ctx->H + kLeafU - 1) / kLeafU) + p.choose);
     cfg.blockDim = dim3(kLeafT); cfg.dynamicSmemBytes = kLeafSmem; cfg.stream = stream;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1453,7 +1480,7 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
     TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_leaves_fp32, q));
     ctx->launches += 1;
   }
-  return launch_trees(ctx, forward_kernel(ctx->cell), p, kFwdT, trees_parts(ctx, n, false, after_running), after_running, stream);
+  return launch_trees(ctx, forward_kernel(ctx->cell), p, kFwdT, parts, after_running, stream);
 }
 
 int launch_backward_trees(treelstm* ctx, cudaStream_t stream) {
