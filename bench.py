@@ -32,8 +32,8 @@ L2_FLUSH_BYTES = 256 << 20          # larger than the 126 MB L2
 # committed ncu capture named beside it (a constant copied from that capture, not measured by this
 # run); None for workloads without a capture of the current kernel.
 NCU_TRAFFIC = {
-    "batch256_bf16": (6305536 + 8880896, "profiles/k_fwd_tc_batch256_bf16.md (static: ncu capture of one launch, not measured by this run)"),
-    "balanced1024_bf16": (10304000 + 77163520, "profiles/k_fwd_tc_balanced1024_bf16.md (static: ncu capture of one launch, not measured by this run)"),
+    "batch256_bf16": (6304768 + 5180160, "profiles/k_fwd_tc_batch256_bf16.md (static: ncu capture of one launch, not measured by this run)"),
+    "balanced1024_bf16": (10477824 + 73920256, "profiles/k_fwd_tc_balanced1024_bf16.md (static: ncu capture of one launch, not measured by this run)"),
 }
 MODES = ("persistent", "per_level", "subforests")
 TIMINGS = {}   # side results of the last time_forward call
@@ -79,7 +79,7 @@ def roofline_block(forest, p, precision: str, kernel_ms: float, step_ms: float, 
         head = {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"]}
     head.update({
         "traffic": traffic, "traffic_source": source, "peak_source": peaks["source"],
-        "kernel": "k_fwd_tc (persistent wavefront kernel)" if precision == "bf16" else "k_fwd_fp32_persistent",
+        "kernel": "k_fwd_tc (persistent wavefront kernel)" if precision == "bf16" else "k_leaves_fp32 and k_trees_forward (or k_fwd_fp32_persistent)",
         "kernel_timing": "the kernel of the timed steps run alone, between the library's event pair (the event keeps it "
                          "from starting under the scheduler as it does in the steps)",
         "kernel_ms_plain_order": TIMINGS.get("kernel_ms_plain_order"),
@@ -369,8 +369,8 @@ def train_step_time(peaks, flush, steps: int = 200, warmup: int = 5):
                          "fp32_tflops": flops / (mean * 1e-3) / 1e12,
                          "note": "whole step (forward + backward launches together); fp32 FMA pipes except the "
                                  "weight gradient, a split-bf16 tensor-core contraction"},
-            "note": "persistent forward + one-launch backward (wavefronts) + tensor-core dW/db kernel; the binding "
-                    "reads the status word back after each"}
+            "note": "forward and backward on tree clusters, tensor-core dW/db kernel, and the two kernels over the whole "
+                    "GPU that find the forest taken; the binding reads the status word back after each"}
 
 
 def run_sweeps(args):

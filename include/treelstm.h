@@ -67,8 +67,10 @@ typedef enum treelstm_status {
 /* flags of treelstm_forward (or-ed together) */
 #define TREELSTM_PER_LEVEL 0    /* one launch per wavefront; synchronises the stream once to read   */
                                 /* the level table, returns device-detected errors directly          */
-#define TREELSTM_PERSISTENT 1   /* one cooperative launch loops over the wavefronts with a bounded   */
-                                /* grid-wide barrier; fully asynchronous (see treelstm_status_sync)  */
+#define TREELSTM_PERSISTENT 1   /* no launch per wavefront: one kernel loops over the wavefronts with */
+                                /* a bounded grid-wide barrier, or (fp32) clusters walk whole trees,  */
+                                /* whichever suits the forest; fully asynchronous (see                */
+                                /* treelstm_status_sync)                                              */
 #define TREELSTM_SAVE_FOR_BACKWARD 2 /* keep every node's gate activations for treelstm_backward   */
 #define TREELSTM_SUBFORESTS 4   /* bf16 only: the trees are dealt out to as many sub-forests as      */
                                 /* thread-block clusters fit on the GPU; one cluster evaluates one   */
@@ -181,7 +183,9 @@ TREELSTM_API int treelstm_update_weights(treelstm_t* ctx, const float* emb, cons
 /*
  * treelstm_set_classifier - per-node softmax classifier used by treelstm_backward
  *   (Section 6.1: every node of every tree carries a label).
- *   Wc [H][C], bc [C]; copied; synchronises `stream`.  1 <= C <= 32.
+ *   Wc [H][C], bc [C]; copied; synchronises `stream`.  1 <= C <= 32.  The first call allocates room for the
+ *   classifier and for the weights in the layouts that only the backward reads (H = 256, E = 300: 10 MB), which
+ *   treelstm_update_weights keeps up to date from then on; a later call waits for the device.
  */
 TREELSTM_API int treelstm_set_classifier(treelstm_t* ctx, int C, const float* Wc, const float* bc, void* stream);
 
@@ -191,6 +195,9 @@ TREELSTM_API int treelstm_set_option(treelstm_t* ctx, int key, long long value);
  * treelstm_workspace_bytes - size of the caller-provided device scratch buffer that
  * treelstm_forward (and, if with_backward != 0, treelstm_backward) needs for forests of up to
  * max_nodes nodes.  Returns 0 on invalid arguments.  The buffer must be 256-byte aligned.
+ * With with_backward the bytes grow with every node's gates, dh, dc and dz (48 H bytes, fp32) and, from some hundred
+ * nodes on (H <= 512, E <= 1024), with dz and both cell inputs as three bf16 pieces, which doubles that: 14592 nodes,
+ * H = 256, E = 300, bf16 forward: 425 MB, 191 of them pieces.
  */
 TREELSTM_API size_t treelstm_workspace_bytes(const treelstm_t* ctx, int max_nodes, int with_backward);
 
@@ -278,9 +285,10 @@ TREELSTM_API int treelstm_backward(treelstm_t* ctx, const int32_t* labels, float
  *   dW [2H][H], db [H]  out;  dV [H][2H][2H] out (RNTN; may be NULL for TreeRNN);
  *   dEmb_rows [n_leaves][H] out: one summed row per touched id.
  * All device pointers; gradients are overwritten; fp32.  Up to H = 256 (TreeRNN) and H = 32 (RNTN), after a
- * TREELSTM_PERSISTENT forward, three launches without a host round trip; else the level table is read back
- * once (the call synchronises the stream of the forward), then one launch per phase and wavefront.  Errors: as treelstm_backward; TREELSTM_ERR_STATE on a TreeLSTM context
- * (and treelstm_backward returns it on a TreeRNN / RNTN context).
+ * TREELSTM_PERSISTENT forward, three launches without a host round trip, four for forests that may be walked
+ * faster wavefront by wavefront over the whole GPU; else the level table is read back once (the call synchronises
+ * the stream of the forward), then one launch per phase and wavefront.  Errors: as treelstm_backward;
+ * TREELSTM_ERR_STATE on a TreeLSTM context (and treelstm_backward returns it on a TreeRNN / RNTN context).
  */
 TREELSTM_API int treelstm_backward_recursive(treelstm_t* ctx, const int32_t* labels, float* loss, float* dW,
                                              float* db, float* dV, float* dWc, float* dbc, int32_t* touched_ids,

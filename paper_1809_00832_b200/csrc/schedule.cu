@@ -721,7 +721,7 @@ k_schedule_cluster(int n, const int* __restrict__ left, const int* __restrict__ 
       __syncthreads();
     }
     // rank of every item among the warp's items of its bin (and of every root among the warp's roots)
-    unsigned int ranks[kClGroups];                       // rank | bin << 16 | root rank << 22, per group of 32
+    unsigned int ranks[kClGroups];                       // rank | bin << 16 | root rank << 23, per group of 32
     int warp_roots = 0;
 #pragma unroll
     for (int g = 0; g < kClGroups; ++g) {

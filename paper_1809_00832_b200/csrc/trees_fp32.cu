@@ -21,7 +21,8 @@
 //
 // Order.  The schedule that callers see (level, order) is the scheduler's.  A cluster needs only "children
 // before parents"; deepest depth first is such an order with the same number of steps.  It finds roots and depths
-// itself, from the child arrays in shared memory, so nothing here waits for the scheduler before its end.  (A
+// itself, from the child arrays in shared memory, so nothing here waits for the scheduler before its end (TreeLSTM waits
+// for the leaves' kernel).  Forests that are faster wavefront by wavefront are left to the kernel behind (trees_win).  (A
 // malformed forest is the scheduler's to report; here every index is clamped and every list bounded, so that
 // whatever the arrays hold the walk ends.)  Clusters take roots q, q + Q, ... in id order.
 #include <math.h>
@@ -721,7 +722,7 @@ __device__ __forceinline__ void leaves_choose(const LeafParams& p, float* sm) {
 }
 __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ LeafParams p) {
   extern __shared__ __align__(16) float leaf_smem[];
-  float* const Ws = leaf_smem;                           // [kLeafK][3 gates][32 units]; then the second halves' sums
+  float* const Ws = leaf_smem;                           // [kLeafK][3 gates][32 units]; then the quarters' sums
   float* const As = leaf_smem + kLeafK * 3 * kLeafU;     // [rows][pitch]
   __shared__ int s_node[kLeafIds], s_tok[kLeafIds], s_count, s_abort;
   __shared__ __align__(8) uint64_t s_bar;

@@ -24,9 +24,7 @@ Cluster kernel of the narrow tail (k_fwd_tc_tail), stamps of different warps of 
   s9  older child cell states are in      s5  cell updates done
   s10 new h complete in shared memory     s11 every peer's prefetch has landed (pushes may go)
   s6  pushes issued
-One-launch backward (--train: train25_fp32, fp32 forward + k_bwd_persistent), first CTA, per wavefront in
-reverse: s0 start, s1 gate gradients done, s2 barrier, s3 input gradients done, s4 barrier; and the
-phases of the kernel.
+Training step (--train: train25_fp32): the tree kernels, depth by depth of the first cluster's trees.
 The sub-forest kernel (--mode subforests) uses s0 start, s1 first operand request, s2 first box seen by
 the MMA issuer, s3 last MMAs committed, s4 epilogue starts waiting, s5 last tile stored, s6 arrival at
 the cluster barrier, s7 barrier left.  The stamps cost a few cycles each; the normal build is a little
@@ -43,6 +41,7 @@ import torch
 from . import binding, build, forests as fg
 
 SLOTS, LEVELS = 16, 256
+CLUSTER_MIN_NODES = 4096   # forests from this size on are scheduled by one cluster
 
 
 def read_trace(model: binding.TreeLSTM, which: int) -> np.ndarray:
@@ -66,33 +65,26 @@ def trace_training_step() -> int:
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
     for i in range(4):
         flush.fill_(i)
-        out = model.forward(left, right, token, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+        model.forward(left, right, token, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+        torch.cuda.synchronize()
+        forward = read_trace(model, 0)                   # (the backward clears this table)
         model.backward(labels, f.n_leaves)
     torch.cuda.synchronize()
-    widths = np.diff(out["level_offset"].cpu().numpy()[:int(out["n_levels"].item()) + 1])
-    tf = read_trace(model, 1)
-    phf = tf[LEVELS - 1]
-    print(f"# fp32 persistent forward, first CTA, cycles since its start: weight slice fetched {int(phf[1] - phf[0])}, "
-          f"schedule there {int(phf[2] - phf[0])}, last stamp {int(tf[:LEVELS - 1].max() - phf[0])}")
-    print("level width tiles_done barrier_passed ids_resolved first_chunk contracted   (cycles since the wavefront's start; the last three: streaming tiles only)")
-    for l in range(len(widths)):
-        if tf[l, 0]:
-            print(f"{l:<5d} {int(widths[l]):<5d} " + " ".join(f"{(tf[l, k] - tf[l, 0]) if tf[l, k] else 0:<10d}" for k in (1, 2, 3, 4, 5)))
-    t = read_trace(model, 0)
-    ph = t[LEVELS - 1]
-    names = ("outputs and scratch cleared", "tokens marked", "own part of token scan / classifier done",
-             "classifier, loss, token scan done everywhere", "all wavefronts done", "dW from the leaves (own blocks)",
-             "dW from the internal nodes (own blocks)", "db done", "token scan: first warp has read its flags",
-             "token scan: all warps have", "classifier (second CTA): starts", "classifier: first warp's node done",
-             "classifier: all warps' nodes done", "classifier: partial sums sent")
-    print("# one-launch backward, first CTA, cycles since its start: " +
-          ", ".join(f"{nm} {int(ph[i + 1] - ph[0])}" for i, nm in enumerate(names) if ph[i + 1]))
-    print("level width gates_done barrier dinput_done barrier first_dz contracted own_blocks operands_landed request_begin indices_requested weights_requested   (cycles since the wavefront's start; "
-          "wavefronts run in reverse; the last three only where the gate gradients are formed inside the contraction)")
-    for l in range(len(widths) - 1, -1, -1):
-        if t[l, 0] == 0:
-            continue
-        print(f"{l:<5d} {int(widths[l]):<5d} " + " ".join(f"{(t[l, k] - t[l, 0]) if t[l, k] else 0:<10d}" for k in range(1, 12)))
+    for name, t, phases, columns in (
+            ("k_trees_forward", forward, {2: "tables and walk done", 3: "leaves' states in place"},
+             ("multiplied", "summed", "updated", "barrier")),
+            ("k_trees_backward", read_trace(model, 1), {1: "buffers cleared", 2: "tables and walk done", 3: "classifier's dh there", 4: "dh in place"},
+             ("gates", "products", "barrier", "added", "complete"))):
+        ph = t[LEVELS - 1]
+        print(f"# {name}, first CTA of the first cluster, cycles since its start: " +
+              ", ".join(f"{what} {int(ph[k] - ph[0])}" for k, what in phases.items()))
+        print("depth " + " ".join(f"{c:<10s}" for c in columns) + " (cycles since the start of the depth's last nodes)")
+        rows = [d for d in range(LEVELS - 1) if t[d, 0] > ph[0]]
+        for d in rows if name == "k_trees_backward" else rows[::-1]:
+            print(f"{d:<5d} " + " ".join(f"{(t[d, k + 1] - t[d, 0]) if t[d, k + 1] > t[d, 0] else 0:<10d}" for k in range(len(columns))))
+        print(f"# last stamp {int(t[:LEVELS - 1].max() - ph[0])}")
+    ph = read_trace(model, 0)[LEVELS - 1]
+    print(f"# k_bwd_begin, second CTA: classifier, all warps' nodes done {int(ph[13] - ph[11])} cycles after its start, partial sums sent {int(ph[14] - ph[11])}")
     return 0
 
 
@@ -104,7 +96,7 @@ def main() -> int:
     ap.add_argument("--tail-min-levels", type=int, default=None)
     ap.add_argument("--trees", type=int, default=None)
     ap.add_argument("--levels", default=None, help="A:B - print only wavefronts A..B-1")
-    ap.add_argument("--train", action="store_true", help="trace the one-launch backward of a training step on train25_fp32")
+    ap.add_argument("--train", action="store_true", help="trace the tree kernels of a training step on train25_fp32")
     ap.add_argument("--plain-order", action="store_true",
                     help="launch the grid-wide kernel cooperatively behind the scheduler instead of under it")
     args = ap.parse_args()
@@ -141,11 +133,12 @@ def main() -> int:
     fn.restype = ctypes.c_int
     fn.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int]
     if fn(model.handle, 2, ctypes.cast(buf, ctypes.c_void_p), 16) > 0:
-        names = ("cleared", "validated+linked", "links checked, leaves reported", "climbed", "levels written", "ordered")
-        print("# single-CTA scheduler, thread 0, cycles since its start: " +
-              ", ".join(f"{nm} {int(buf[i])}" for i, nm in enumerate(names)))
-        print("#   inside the few-levels placement (cycles since its start): counts cleared, counted, rows scanned, "
-              "starts known, placed = " + ", ".join(str(int(buf[8 + i])) for i in range(5)))
+        if f.n_nodes >= CLUSTER_MIN_NODES:
+            names = ("cleared", "validated+linked", "leaves reported", "own climbs ended", "climbed", "levels written", "counted", "places known",
+                     "staged", "ended")
+        else:
+            names = ("cleared", "validated+linked", "links checked, leaves reported", "climbed", "levels written", "ordered")
+        print("# scheduler, thread 0, cycles since its start: " + ", ".join(f"{nm} {int(buf[i])}" for i, nm in enumerate(names)))
     for which, name in ((0, "grid-wide kernel"), (1, "cluster kernel")):
         t = read_trace(model, which)
         rows = [l for l in range(min(len(widths), LEVELS)) if t[l, 0] != 0]
