@@ -350,7 +350,14 @@ int treelstm_set_classifier(treelstm_t* ctx, int C, const float* Wc, const float
   if (!ctx || !Wc || !bc || C < 1) return TREELSTM_ERR_INVALID_ARG;
   if (C > kMaxClasses) return TREELSTM_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (ctx->C > 0) TL_CUDA(ctx, cudaDeviceSynchronize());   // a backward on another stream may still read the old one
+  if (ctx->C > 0) {                      // a backward on another stream may still read the old one
+    int dev = -1;
+    TL_CUDA(ctx, cudaGetDevice(&dev));
+    if (dev != ctx->device) TL_CUDA(ctx, cudaSetDevice(ctx->device));
+    const cudaError_t e = cudaDeviceSynchronize();
+    if (dev != ctx->device) TL_CUDA(ctx, cudaSetDevice(dev));
+    TL_CUDA(ctx, e);
+  }
   ctx->C = 0;
   const int rc = ensure_backward_memory(ctx, s);
   if (rc != TREELSTM_OK) return rc;
