@@ -267,10 +267,12 @@ def test_weights_of_the_backward_come_with_the_classifier_and_follow_every_updat
     util.lib_ready()
     arrs = [util.to_dev(a) for a in (forest.left, forest.right, forest.token, labels)]
     weights = [[util.to_dev(a) for a in (p.emb, p.W, p.b, p.Wc, p.bc)] for p in (params, other)]
+    create = lambda: binding.TreeLSTM(256, 300, 60, *weights[0][:3], binding.FP32 if precision == "fp32" else binding.BF16)
+    create().close()                                              # the kernels that a create launches are on the device now
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     before = torch.cuda.mem_get_info()[0]
-    model = binding.TreeLSTM(256, 300, 60, *weights[0][:3], binding.FP32 if precision == "fp32" else binding.BF16)
+    model = create()
     assert before - torch.cuda.mem_get_info()[0] <= 12 << 20      # W 4.2 MB and one image of it; with the backward's two: 16 and more
     need = model.workspace_bytes(forest.n_nodes, True)
     model.forward(*arrs[:3], flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
