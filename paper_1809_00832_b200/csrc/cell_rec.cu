@@ -179,7 +179,7 @@ int launch_forward_rec(treelstm* ctx, int n, const int32_t* left, const int32_t*
                        const WsLayout& lay, cudaStream_t stream) {
   bool after_trees = false;
   if ((flags & TREELSTM_PERSISTENT) && trees_take(ctx, n)) {
-    const int rc = launch_forward_trees(ctx, n, left, right, token, h, nullptr, false, ws, lay,
+    const int rc = launch_forward_trees(ctx, n, left, right, token, h, nullptr, (flags & TREELSTM_SAVE_FOR_BACKWARD) != 0, ws, lay,
                                         ctx->opt.overlap_launch && scheduler_lets_start(ctx, n), stream);
     if (rc != TREELSTM_OK || trees_always_pay(ctx->cell, ctx->H, n, false)) return rc;
     after_trees = true;

@@ -33,7 +33,7 @@ __host__ __device__ inline int row_pitch(int H) { return (H + 3) / 4 * 4; }
 
 struct WsLayout {
   size_t status, parent, pending, order_tmp, level_offset, roots, table, slot, part_order, part_offset,
-      part_spill, xin, ain, cin, gates, dh, dc, dz, tok_slot, trace, check, img_dz, img_x0, img_x1, img_end, total;
+      part_spill, xin, ain, cin, gates, dh, dc, dz, tok_slot, walks, trace, check, img_dz, img_x0, img_x1, img_end, total;
 };
 
 // Cycle stamps of the wavefront kernels (builds with -DTREELSTM_TRACE only): kTraceSlots stamps per
@@ -107,7 +107,7 @@ struct TreesShape {
 
 // What the two fp32 ways through a forest cost in microseconds: trees dealt out to clusters (trees_fp32.cu), where the
 // fullest cluster sets the time, or every wavefront over the whole GPU (cell_fp32.cu, cell_rec.cu, backward.cu).  The host
-// knows the number of nodes only, so the tree kernel counts (trees_win) and leaves the forest to the kernel behind it, or
+// knows the number of nodes only, so the tree kernel counts (clusters_win) and leaves the forest to the kernel behind it, or
 // not; that one reads the outcome in the control block.
 struct WalkCosts {
   float tree0, node, depth, rest;   // clusters: fixed, per internal node and depth of the fullest one, per internal node of the forest
@@ -251,8 +251,9 @@ size_t tree_backward_bytes(const treelstm* ctx);         // and of the backward'
 int init_trees(treelstm* ctx, unsigned char* memory, cudaStream_t stream);
 int pack_trees(treelstm* ctx, bool forward, bool backward, cudaStream_t stream);   // after the weights have changed
 bool trees_take(const treelstm* ctx, int n);
+size_t saved_walks_bytes(const treelstm* ctx, int n);     // what a forward leaves for the backward pass
 int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
-                         float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
+                         float* c, bool save, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream);
 int launch_backward_trees(treelstm* ctx, cudaStream_t stream);   // dz of every node (TreeRNN / RNTN: and dh of the leaves) from dh
 int launch_rec_grads(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb_rows, const int* tok_slot, cudaStream_t stream);
 

@@ -21,25 +21,25 @@
 //
 // Order.  The schedule that callers see (level, order) is the scheduler's.  A cluster needs only "children
 // before parents"; deepest depth first is such an order with the same number of steps.  It finds roots and depths
-// itself, from the child arrays in shared memory, so nothing here waits for the scheduler before its end (TreeLSTM waits
-// for the leaves' kernel).  Forests that are faster wavefront by wavefront are left to the kernel behind (trees_win).  (A
-// malformed forest is the scheduler's to report; here every index is clamped and every list bounded, so that
-// whatever the arrays hold the walk ends.)  Clusters take roots q, q + Q, ... in id order.
+// itself, from the child arrays in shared memory (trees_plan.cuh), so nothing here waits for the scheduler before its end
+// (TreeLSTM waits for the leaves' kernel).  Forests that are faster wavefront by wavefront are left to the kernel behind
+// (clusters_win).  (A malformed forest is the scheduler's to report; here every index is clamped and every list bounded, so
+// that whatever the arrays hold the walk ends.)
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
 #include "split_tc.cuh"
+#include "trees_plan.cuh"
 
 namespace tl {
 namespace {
 
 constexpr int NT = 4;                     // nodes per pass of the forward
 constexpr int kFwdT = 512, kBwdT = 640;   // threads of a CTA (backward: at most)
-constexpr int kSmemMax = 224 * 1024;
 constexpr int kLstm = 0, kRnn = TREELSTM_CELL_TREERNN, kRntn = TREELSTM_CELL_RNTN;
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kND = 16;                   // backward: nodes between two cluster barriers at most
 constexpr int kRntnBC = 2, kRntnJS = 8, kRntnMaxH = 32, kRntnT = 512;   // RNTN backward: columns and units per thread
 constexpr int kRntnBwdWords = 4 * kRntnBC * kRntnJS + kRntnJS;
@@ -85,17 +85,17 @@ __device__ __forceinline__ void lane_sums4(float (&v)[4], int lane) {
 template <int LANES>
 __device__ __forceinline__ int value_of_lane(int lane) { return ((lane & (LANES / 2)) ? 2 : 0) + ((lane & (LANES / 4)) ? 1 : 0); }
 
-struct TreesParams {
-  int n, H, E, vocab;
+struct TreesParams : ForestIn {
+  int H, E;
   int Hp;                                 // H rounded up to 4: half an operand row in shared memory
   TreesShape s;
   int* chk_counts;
-  const int *left, *right, *token;
   const float *emb, *W, *b;               // W: register image [rank][word][thread]; b [G H]
   const ushort2* pairs;                   // RNTN: the two operands of every input chunk
   WalkCosts costs;
-  int choose;                             // 1: the forest may be left to the kernel behind this one (trees_win)
+  int choose;                             // 1: the forest may be left to the kernel behind this one (clusters_win)
   float *h, *c, *gates, *dh, *dc, *dz;
+  SavedWalks walks;                       // of the forward pass, for the backward one (at == nullptr: none)
   DevStatus* st;
   long long* trace;                       // cycle stamps of the first CTA (trace builds), else nullptr
 };
@@ -153,28 +153,6 @@ __host__ __device__ inline WeightAt bwd_weight(int cell, int H, int E, const Tre
   return cell == kLstm ? WeightAt{((long long)E + out) * 5 * H + (long long)gate * H + j, -1} : WeightAt{(long long)out * H + j, -1};
 }
 
-// ---- shared memory -------------------------------------------------------------------------------- //
-// Offsets in 4-byte words.  What is left behind `state` holds the states of the cluster's nodes, if they fit.
-struct TreesSmem {
-  int buf, kids, child, list, start, par, leaf, leaf_par, state, state_words;
-};
-__host__ __device__ inline TreesSmem trees_smem(int n, int buf_words) {
-  TreesSmem s{};
-  int off = 0;
-  auto take = [&](int words) { const int o = off; off += (words + 3) & ~3; return o; };
-  s.buf = take(buf_words);
-  s.kids = take(n);
-  s.child = take(n / 32 + 1);             // a bit per node: it has a caller
-  const int half = n / 4 + 8;             // uint16 entries for the internal nodes (fewer than n / 2)
-  s.list = take(half);
-  s.start = take(half);
-  s.par = take(half);
-  s.leaf = take(n / 2 + 8);               // (a forest of single-leaf trees has n leaves)
-  s.leaf_par = take(n / 2 + 8);
-  s.state = off;
-  s.state_words = kSmemMax / 4 - off;
-  return s;
-}
 // forward: partial sums [nseg][NT][outs], gate values [NT][outs], operand rows and cell states of a pass (states in L2)
 __host__ __device__ inline int fwd_outs(const TreesShape& s) { return s.U * s.JL; }
 __host__ __device__ inline int fwd_parts(int cell, const TreesShape& s) { return ((cell == kRntn ? kFwdT / 32 : s.nseg) + 7) & ~7; }
@@ -185,228 +163,6 @@ __host__ __device__ inline int fwd_buf_words(int cell, int H, const TreesShape& 
 __host__ __device__ inline int bwd_in_row(int cell, const TreesShape& s) { return cell == kRntn ? kRntnJS : 4 * s.bseg * s.BC; }
 __host__ __device__ inline int bwd_buf_words(int cell, int H, const TreesShape& s) {
   return kND * bwd_in_row(cell, s) + 2 * s.cs * kND * 2 * s.JS + (cell == kRntn ? kND * 2 * ((H + 3) & ~3) : 0);
-}
-
-// Child table entry of a node: left | right << 16 (ids below 32768), or the top bit and the token of a leaf.  Ids and
-// tokens are clamped: nothing has been validated yet.
-constexpr unsigned kLeafBit = 0x80000000u;
-__device__ __forceinline__ bool is_leaf(unsigned kids) { return (kids & kLeafBit) != 0; }
-// (up: if given, every node's caller, a root's itself.  Two callers of one child are no forest: which of them is found is a matter of timing, so
-// the answer is true then, the same in every CTA.)
-__device__ __forceinline__ bool load_kids(const TreesParams& p, const TreesSmem& s, float* sm, unsigned short* up) {
-  unsigned* kids = reinterpret_cast<unsigned*>(sm + s.kids);
-  unsigned* child = reinterpret_cast<unsigned*>(sm + s.child);
-  for (int k = threadIdx.x; k < p.n / 32 + 1; k += blockDim.x) child[k] = 0u;
-  if (up)
-    for (int k = threadIdx.x; k < p.n; k += blockDim.x) up[k] = (unsigned short)k;
-  __syncthreads();
-  bool twice = false;
-  for (int k = threadIdx.x; k < p.n; k += blockDim.x) {
-    const int l = p.left[k], r = p.right[k], t = p.token[k];
-    if (l < 0) {
-      kids[k] = kLeafBit | (unsigned)min(max(t, 0), p.vocab - 1);
-    } else {
-      const unsigned a = (unsigned)min(l, p.n - 1), b = (unsigned)min(max(r, 0), p.n - 1);
-      kids[k] = a | (b << 16);
-      if (up) {
-        up[a] = up[b] = (unsigned short)k;
-        const unsigned had_a = atomicOr(child + (a >> 5), 1u << (a & 31)), had_b = atomicOr(child + (b >> 5), 1u << (b & 31));
-        twice = twice || ((had_a >> (a & 31) | had_b >> (b & 31)) & 1u);
-      } else {
-        atomicOr(child + (a >> 5), 1u << (a & 31));
-        atomicOr(child + (b >> 5), 1u << (b & 31));
-      }
-    }
-  }
-  return __syncthreads_or(twice) != 0;
-}
-
-// The cluster's trees by depth: internal node number q is list[q], depth d is [start[d], start[d + 1]), the leaves are
-// in leaf[]; par[q] and leaf_par[] say whose child a node is: 2 x number of the caller + side, kNoCaller for a root.  One
-// warp; every CTA of the cluster gets the same lists.
-constexpr unsigned short kNoCaller = 0xFFFF;
-struct Walk { int depths, internal, leaves; };
-// `win`: if given, the walk may end where it reads zero.
-__device__ __forceinline__ void walk_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, const int* win, Walk* out) {
-  const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
-  const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
-  unsigned short* list = reinterpret_cast<unsigned short*>(sm + s.list);
-  unsigned short* start = reinterpret_cast<unsigned short*>(sm + s.start);
-  unsigned short* par = reinterpret_cast<unsigned short*>(sm + s.par);
-  unsigned short* leaf = reinterpret_cast<unsigned short*>(sm + s.leaf);
-  unsigned short* leaf_par = reinterpret_cast<unsigned short*>(sm + s.leaf_par);
-  const int lane = threadIdx.x & 31, n = p.n;
-  const unsigned below = (1u << lane) - 1u;
-  const int max_internal = n / 2, max_leaves = n;
-  int count = 0, leaves = 0, depth = 0, lo = 0, rank0 = 0;
-  auto scan = [&](int v) {                // inclusive over the lanes
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(kFull, v, d);
-      if (lane >= d) v += t;
-    }
-    return v;
-  };
-  for (int w0 = 0; w0 * 32 < n; w0 += 32) {   // roots: nodes without a caller, 32 words of 32 ids at a time
-    const int w = w0 + lane, base = w * 32;
-    unsigned m = base < n ? ~child[w] : 0u;
-    if (base < n && n - base < 32) m &= (1u << (n - base)) - 1u;
-    const int roots = __popc(m), incl = scan(roots);
-    int rank = rank0 + incl - roots, mi = 0, ml = 0;
-    rank0 += __shfl_sync(kFull, incl, 31);
-    for (unsigned b = m; b; b &= b - 1, ++rank)
-      if (rank % parts == part) (is_leaf(kids[base + __ffs(b) - 1]) ? ml : mi) += 1;
-    const int ii = scan(mi), il = scan(ml);
-    int ci = count + ii - mi, cl = leaves + il - ml;
-    rank = rank0 - __shfl_sync(kFull, incl, 31) + incl - roots;
-    for (unsigned b = m; b; b &= b - 1, ++rank)
-      if (rank % parts == part) {
-        const int node = base + __ffs(b) - 1;
-        if (is_leaf(kids[node])) { leaf[cl] = (unsigned short)node; leaf_par[cl++] = kNoCaller; }
-        else if (ci < max_internal) { list[ci] = (unsigned short)node; par[ci++] = kNoCaller; }
-      }
-    count = min(count + __shfl_sync(kFull, ii, 31), max_internal);
-    leaves += __shfl_sync(kFull, il, 31);
-  }
-  bool fits = true;
-  if (lane == 0) start[0] = 0;
-  __syncwarp();
-  while (lo < count && fits) {
-    const int hi = count;
-    if (win && hi - lo >= 512 && !__shfl_sync(kFull, *(const volatile int*)win, 0)) break;   // (narrow depths are not worth the look)
-    ++depth;
-    if (lane == 0) start[depth] = (unsigned short)hi;
-    for (int i0 = lo; i0 < hi; i0 += 32) {
-      const bool have = i0 + lane < hi;
-      const unsigned kd = have ? kids[list[i0 + lane]] : 0u;
-      const int l = (int)(kd & 0xFFFFu), r = (int)(kd >> 16);
-      const bool ll = is_leaf(kids[l]), lr = is_leaf(kids[r]);
-      const unsigned il = __ballot_sync(kFull, have && !ll), ir = __ballot_sync(kFull, have && !lr);
-      const unsigned fl = __ballot_sync(kFull, have && ll), fr = __ballot_sync(kFull, have && lr);
-      // only arrays that are no forest of trees can run over
-      if (count + __popc(il) + __popc(ir) > max_internal || leaves + __popc(fl) + __popc(fr) > max_leaves) { fits = false; break; }
-      if (have) {
-        const int al = ll ? leaves + __popc(fl & below) : count + __popc(il & below);
-        const int ar = lr ? leaves + __popc(fl) + __popc(fr & below) : count + __popc(il) + __popc(ir & below);
-        (ll ? leaf : list)[al] = (unsigned short)l;
-        (lr ? leaf : list)[ar] = (unsigned short)r;
-        (ll ? leaf_par : par)[al] = (unsigned short)(2 * (i0 + lane));
-        (lr ? leaf_par : par)[ar] = (unsigned short)(2 * (i0 + lane) + 1);
-      }
-      count += __popc(il) + __popc(ir);
-      leaves += __popc(fl) + __popc(fr);
-      __syncwarp();
-    }
-    lo = hi;
-  }
-  if (lane == 0) *out = fits ? Walk{depth, count, leaves} : Walk{0, 0, 0};
-}
-
-// Whether this forest is walked faster by clusters than wavefront by wavefront over the whole GPU.  (The average load of a
-// cluster says too little: one tree of 1024 leaves among 24 sentences, H = 150, was 4.5 times slower here than over the whole
-// GPU.)  Every node of a sample - all of them, if there are no more than kClimbs per thread - climbs to its root, which says
-// whose load it is; every CTA takes the same sample and comes to the same answer.  All warps but the first, which walks the
-// trees meanwhile: with all nodes' ancestors doubled by the whole CTA instead, 25 sentences (H = 150) took 104 us, not 92.
-constexpr int kMaxTreeClusters = 192, kClimbs = 3;
-struct TreeLoads { int nodes[kMaxTreeClusters], depth[kMaxTreeClusters], win; };
-// Callers by node id, then (32-bit words) the roots before each word of the bit map: behind the lists if there is room, else
-// in their place (`beside` false: then the walk comes afterwards).
-struct TreeLinks { unsigned short* up; int* before; bool beside; };
-__device__ __forceinline__ TreeLinks tree_links(const TreesSmem& s, float* sm, int n) {
-  const int words = (n + 1) / 2;
-  TreeLinks t;
-  t.beside = s.state_words >= words + n / 32 + 1;
-  float* at = sm + (t.beside ? s.state : s.list);
-  t.up = reinterpret_cast<unsigned short*>(at);
-  t.before = reinterpret_cast<int*>(at + words);
-  return t;
-}
-__device__ void trees_win(const TreesParams& p, const TreesSmem& s, float* sm, const TreeLinks& links, int parts, TreeLoads* out) {
-  const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
-  const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
-  const int tid = (int)threadIdx.x - 32, nt = (int)blockDim.x - 32, lane = tid & 31, n = p.n;
-  auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); };
-  for (int q = tid; q < parts; q += nt) out->nodes[q] = out->depth[q] = 0;
-  if (tid < 32) {
-    int sum = 0;
-    for (int w0 = 0; w0 * 32 < n; w0 += 32) {
-      const int w = w0 + lane, roots = w * 32 < n ? __popc(~child[w]) : 0;   // (ids beyond n come last: nobody counts them)
-      int incl = roots;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(kFull, incl, d);
-        if (lane >= d) incl += t;
-      }
-      if (w * 32 < n) links.before[w] = sum + incl - roots;
-      sum += __shfl_sync(kFull, incl, 31);
-    }
-  }
-  const int sample = min(n, nt * kClimbs);
-  int at[kClimbs], depth[kClimbs];
-  bool have[kClimbs];
-#pragma unroll
-  for (int q = 0; q < kClimbs; ++q) {
-    const int i = tid + q * nt;
-    have[q] = i < sample;
-    at[q] = have[q] ? (int)((long long)i * n / sample) : 0;
-    depth[q] = is_leaf(kids[at[q]]) ? 0 : 1;
-  }
-  for (int step = 0; step < n; ++step) {                     // (arrays that are no forest may hold a cycle)
-    bool any = false;
-#pragma unroll
-    for (int q = 0; q < kClimbs; ++q) {
-      const int up = links.up[at[q]];
-      if (up != at[q]) { ++depth[q]; any = true; }
-      at[q] = up;
-    }
-    if (!any) break;
-  }
-  sync();
-#pragma unroll
-  for (int q = 0; q < kClimbs; ++q) {
-    const int root = at[q], w = root >> 5;
-    const int part = have[q] ? (links.before[w] + __popc(~child[w] & ((1u << (root & 31)) - 1u))) % parts : -1;
-    const unsigned peers = __match_any_sync(kFull, part);
-    const int deepest = __reduce_max_sync(peers, depth[q]);
-    if (have[q] && lane == __ffs(peers) - 1) {
-      atomicAdd(&out->nodes[part], __popc(peers));
-      atomicMax(&out->depth[part], deepest);
-    }
-  }
-  sync();
-  if (tid < 32) {
-    const int roots = links.before[(n - 1) >> 5] + __popc(~child[(n - 1) >> 5] & (0xFFFFFFFFu >> (31 - ((n - 1) & 31))));
-    const float internal = (float)((n - roots) / 2), share = internal / (float)sample;
-    float cost = 0.f;
-    int waves = 0;
-    for (int q = lane; q < parts; q += 32) {
-      cost = fmaxf(cost, tree_cost(p.costs, share * (float)out->nodes[q], (float)out->depth[q], internal));
-      waves = max(waves, out->depth[q]);
-    }
-    waves = __reduce_max_sync(kFull, waves);
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) cost = fmaxf(cost, __shfl_xor_sync(kFull, cost, d));
-    if (lane == 0) *(volatile int*)&out->win = cost < grid_cost(p.costs, (float)waves, internal);
-  }
-}
-// The tables of the forest, then what the cluster has to walk: nothing, if loads->win says that the forest is the next kernel's.
-__device__ __forceinline__ void deal_trees(const TreesParams& p, const TreesSmem& s, float* sm, int part, int parts, bool choose, TreeLoads* loads, Walk* walk) {
-  const int warp = (int)threadIdx.x >> 5;
-  if (threadIdx.x == 0) loads->win = 1;
-  if (!choose) {
-    load_kids(p, s, sm, nullptr);
-    if (warp == 0) walk_trees(p, s, sm, part, parts, nullptr, walk);
-    __syncthreads();
-    return;
-  }
-  const TreeLinks links = tree_links(s, sm, p.n);
-  const bool forest = !load_kids(p, s, sm, links.up);    // (else: the scheduler reports it, and the walk is bounded)
-  if (forest && warp > 0) trees_win(p, s, sm, links, parts, loads);
-  if (!links.beside) __syncthreads();
-  if (warp == 0) walk_trees(p, s, sm, part, parts, &loads->win, walk);
-  __syncthreads();
-  if (threadIdx.x == 0 && !loads->win) *walk = Walk{0, 0, 0};
-  __syncthreads();
 }
 
 // ---- forward -------------------------------------------------------------------------------------- //
@@ -422,16 +178,19 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   const TreesSmem s = trees_smem(p.n, fwd_buf_words(CELL, H, p.s));
 #ifdef TREELSTM_TRACE
   long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;   // row d: depth d; last row: set-up
+#else
+  long long* const trace = nullptr;
 #endif
   TL_STAMP(trace, kTraceLevels - 1, 0);
   float w[RC * 4 * U];
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
-  deal_trees(p, s, sm, part, parts, CELL != kLstm && p.choose, &s_loads, &s_walk);
+  deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, &s_loads, &s_walk, trace);
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
   const Walk walk = s_walk;
+  if (p.walks.at && rank == 0) save_walk(p.walks, s, sm, part, parts, walk);
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
   const unsigned short* start = reinterpret_cast<const unsigned short*>(sm + s.start);
@@ -643,7 +402,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   // what follows on the stream waits for this grid only: it must not end before the scheduler ahead of it has
   if (blockIdx.x == 0) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (CELL != kLstm && tid == 0) p.st->trees_fwd = s_loads.win;
+    if (tid == 0 && (CELL != kLstm || !p.choose)) p.st->trees_fwd = s_loads.win;   // (TreeLSTM: else the leaves' kernel has said so)
   }
 }
 
@@ -667,7 +426,7 @@ struct LeafParams {
   float *h, *c, *gates;
   DevStatus* st;
   long long wait_limit;
-  int choose, parts;                       // 1: the first CTA says whether the clusters (so many) take the forest (trees_win)
+  int choose, parts;                       // 1: the first CTA says whether the clusters (so many) take the forest (clusters_win)
   const int* right;
   WalkCosts costs;
 };
@@ -705,17 +464,21 @@ __device__ __forceinline__ void leaf_rows(const float* As, const float* Ws, int 
 // The choice takes no time here: the clusters' kernel waits for the leaves anyhow, and one CTA more beside them is done before
 // they are.  (In the clusters' own kernel, beside the walk, it cost 2.5 us of 90.)
 constexpr int kLeafTableWords = kLeafSmem / 4;
-__host__ __device__ inline bool leaves_hold_tables(int n) { return n + 2 * (n / 32 + 1) + (n + 1) / 2 + 8 <= kLeafTableWords; }
+__host__ __device__ inline int leaves_tables_at(int n) { return (n + n / 32 + 4) / 4 * 4; }   // (16-byte boundary)
+__host__ __device__ inline bool leaves_hold_tables(int n) { return leaves_tables_at(n) + deal_words(n) <= kLeafTableWords; }
 __device__ __forceinline__ void leaves_choose(const LeafParams& p, float* sm) {
   __shared__ TreeLoads s_loads;
-  TreesParams q{};
-  q.n = p.n; q.vocab = p.vocab; q.left = p.left; q.right = p.right; q.token = p.token; q.costs = p.costs;
+  const ForestIn q{p.n, p.vocab, p.left, p.right, p.token};
   TreesSmem s{};
   s.child = p.n;
-  const int words = (p.n + 1) / 2, at = s.child + p.n / 32 + 1;
-  const TreeLinks links{reinterpret_cast<unsigned short*>(sm + at), reinterpret_cast<int*>(sm + at + words), true};
-  if (threadIdx.x == 0) s_loads.win = 1;
-  if (!load_kids(q, s, sm, links.up) && threadIdx.x >= 32) trees_win(q, s, sm, links, p.parts, &s_loads);
+  const TreeLinks links = tree_links(sm + leaves_tables_at(p.n), p.n);
+  const unsigned* kids = reinterpret_cast<const unsigned*>(sm);
+  const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
+  if (threadIdx.x == 0) { s_loads.win = 1; s_loads.internal = 0; }
+  const bool forest = !load_kids(q, s, sm, links.up, &s_loads.internal);   // (else the scheduler reports it)
+  if (threadIdx.x < 32) count_roots(links, child, p.n, threadIdx.x);
+  __syncthreads();
+  if (forest) deal_by_size(p.n, kids, child, links, p.costs, p.parts, deals_by_size(p.n, s_loads.internal, p.parts), true, 0, &s_loads);
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the scheduler clears the control block at its start
   if (threadIdx.x == 0) p.st->trees_fwd = s_loads.win;
@@ -861,6 +624,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   const TreesSmem s = trees_smem(p.n, bwd_buf_words(CELL, H, p.s));
 #ifdef TREELSTM_TRACE
   long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;
+#else
+  long long* const trace = nullptr;
 #endif
   TL_STAMP(trace, kTraceLevels - 1, 0);
   if (p.choose) {
@@ -877,9 +642,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
       return;
     }
   }
-  float w[kWords];
-#pragma unroll
-  for (int q = 0; q < kWords; ++q) w[q] = __ldg(p.W + ((size_t)rank * kWords + q) * nt + tid);
   float* const in = sm + s.buf;                          // [kND][in_row]
   float* const dx = in + kND * in_row;                   // [2][cs][kND][2 JS]
   float* const xs = dx + 2 * cs * kND * 2 * JS;          // RNTN: [kND][2 Hp]
@@ -887,7 +649,15 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   if (CELL == kRntn)
     for (int e = tid; e < kND * 2 * Hp; e += nt) xs[e] = 0.f;
   TL_STAMP(trace, kTraceLevels - 1, 1);
-  deal_trees(p, s, sm, part, parts, p.choose != 0, &s_loads, &s_walk);
+  if (!(p.walks.at && p.st->trees_fwd && load_walk(p.walks, p.costs, p.n, p.st->n_roots, s, sm, part, parts, p.choose != 0, &s_loads, &s_walk)))
+    deal_trees(p, p.costs, s, sm, part, parts, p.choose != 0, &s_loads, &s_walk, trace);
+  // The weights behind the lists: asked for before them, some were spilled, and read again in every round (25 sentences, H = 150,
+  // training step 224 us, this way 216).
+  const float* image = p.W + (size_t)rank * kWords * nt + tid;
+  asm volatile("" : "+l"(image));
+  float w[kWords];
+#pragma unroll
+  for (int q = 0; q < kWords; ++q) w[q] = __ldg(image + (size_t)q * nt);
 #pragma unroll
   for (int q = 0; q < kWords; ++q) asm volatile("" : "+f"(w[q]));       // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
@@ -1448,26 +1218,39 @@ bool trees_take(const treelstm* ctx, int n) {
          trees_smem(n, bwd_buf_words(ctx->cell, ctx->H, s)).state_words >= 0;
 }
 
-// clusters that a launch takes
-static int trees_parts(const treelstm* ctx, int n, bool backward, bool after_running) {
+// Clusters that a launch takes: the same number in both directions, so that the backward pass can walk what the forward pass has.
+static int most_parts(const treelstm* ctx) {
   const auto& t = ctx->trees;
-  int clusters = backward ? t.clusters_bwd : t.clusters;
-  if (after_running && !backward && (ctx->sm_count - 1) / t.s.cs < clusters) clusters = (ctx->sm_count - 1) / t.s.cs;   // a single scheduling CTA keeps its SM
-  if (ctx->opt.max_ctas > 0 && ctx->opt.max_ctas / t.s.cs < clusters) clusters = ctx->opt.max_ctas / t.s.cs;
-  if (clusters > kMaxTreeClusters) clusters = kMaxTreeClusters;
+  int clusters = t.clusters_bwd;
+  if (ctx->precision == TREELSTM_FP32) {
+    if (t.clusters < clusters) clusters = t.clusters;
+    if ((ctx->sm_count - 1) / t.s.cs < clusters) clusters = (ctx->sm_count - 1) / t.s.cs;   // a single scheduling CTA keeps its SM
+  }
+  return clusters < 1 ? 1 : (clusters > kMaxTreeClusters ? kMaxTreeClusters : clusters);
+}
+static int trees_parts(const treelstm* ctx, int n) {
+  int clusters = most_parts(ctx);
+  if (ctx->opt.max_ctas > 0 && ctx->opt.max_ctas / ctx->trees.s.cs < clusters) clusters = ctx->opt.max_ctas / ctx->trees.s.cs;
   if (clusters > n) clusters = n;                        // (a tree is a node at least)
   return clusters < 1 ? 1 : clusters;
 }
+// For any number of clusters, since TREELSTM_OPT_MAX_CTAS may change it, and no less for more nodes.
+size_t saved_walks_bytes(const treelstm* ctx, int n) {
+  if (ctx->precision != TREELSTM_FP32 || !ctx->trees.ok) return 0;
+  size_t most = 0;
+  for (int parts = most_parts(ctx); parts >= 1; --parts) most = std::max(most, parts * saved_block(saved_cap(n < 32767 ? n : 32767, parts)));
+  return most;
+}
 
 int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h,
-                         float* c, bool save_gates, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream) {
-  const auto& s = ctx->trees.s;
+                         float* c, bool save, void* ws, const WsLayout& lay, bool after_running, cudaStream_t stream) {
   TreesParams p = trees_params(ctx, n, left, right, token, h, c, ws, lay);
   p.W = ctx->trees.Wf;
   p.costs = walk_costs(ctx->cell, ctx->H, false);
   p.choose = !trees_always_pay(ctx->cell, ctx->H, n, false);
-  const int parts = trees_parts(ctx, n, false, after_running);
-  p.gates = save_gates ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
+  const int parts = trees_parts(ctx, n);
+  p.gates = save && ctx->cell == kLstm ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
+  if (save) p.walks = {reinterpret_cast<unsigned char*>(ws) + lay.walks, saved_cap(n, parts)};
   if (ctx->cell == kLstm) {
     LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->trees.Wx, ctx->b, h, c, p.gates,
                  p.st, ctx->opt.wait_limit_kcycles * 1024, p.choose, parts, right, p.costs};
@@ -1491,8 +1274,11 @@ int launch_backward_trees(treelstm* ctx, cudaStream_t stream) {
   p.costs = walk_costs(ctx->cell, ctx->H, true);
   p.choose = !trees_always_pay(ctx->cell, ctx->H, L.n, true);
   p.gates = reinterpret_cast<float*>(static_cast<char*>(L.ws) + L.lay.gates);
+  const int parts = trees_parts(ctx, L.n);
+  if (ctx->precision == TREELSTM_FP32 && L.mode == TREELSTM_PERSISTENT)
+    p.walks = {reinterpret_cast<unsigned char*>(L.ws) + L.lay.walks, saved_cap(L.n, parts)};
   if (p.trace) p.trace += kTraceSlots * kTraceLevels;
-  return launch_trees(ctx, backward_kernel(ctx->cell, p.s), p, p.s.bthreads, trees_parts(ctx, L.n, true, true), true, stream);
+  return launch_trees(ctx, backward_kernel(ctx->cell, p.s), p, p.s.bthreads, parts, true, stream);
 }
 
 int launch_rec_grads(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb_rows, const int* tok_slot, cudaStream_t stream) {

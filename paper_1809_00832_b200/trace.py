@@ -71,9 +71,9 @@ def trace_training_step() -> int:
         model.backward(labels, f.n_leaves)
     torch.cuda.synchronize()
     for name, t, phases, columns in (
-            ("k_trees_forward", forward, {2: "tables and walk done", 3: "leaves' states in place"},
+            ("k_trees_forward", forward, {5: "child table", 6: "dealt", 2: "lists done", 3: "leaves' states in place"},
              ("multiplied", "summed", "updated", "barrier")),
-            ("k_trees_backward", read_trace(model, 1), {1: "buffers cleared", 2: "tables and walk done", 3: "classifier's dh there", 4: "dh in place"},
+            ("k_trees_backward", read_trace(model, 1), {1: "buffers cleared", 5: "child table", 6: "dealt", 2: "lists done", 3: "classifier's dh there", 4: "dh in place"},
              ("gates", "products", "barrier", "added", "complete"))):
         ph = t[LEVELS - 1]
         print(f"# {name}, first CTA of the first cluster, cycles since its start: " +

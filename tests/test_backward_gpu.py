@@ -255,6 +255,24 @@ def test_large_forests_on_either_way(H, shapes):
     _compare(res, ref, util.TOL["fp32"])
 
 
+@pytest.mark.parametrize("H,n_trees", [(150, 15), (150, 16), (150, 61), (20, 147), (20, 148), (20, 512), (20, 513)])
+def test_trees_dealt_by_size(H, n_trees):
+    """as many trees as clusters (15 and 147 on 148 SMs), one more, as many as are dealt by size at most, one more; sizes far
+    apart, trees of one leaf among them, and one cluster whose lists are longer than what the forward keeps for the backward"""
+    rng = np.random.default_rng(1200 + H + n_trees)
+    params = fg.draw_params(rng, H, 24, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    shapes = [fg.left_chain_shape(90), fg.random_split_shape(rng, 50)] + [
+        None if t % 11 == 3 else fg.random_split_shape(rng, int(rng.integers(2, 4 if n_trees > 100 else 24))) for t in range(n_trees - 2)]
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes, rng, 60), rng)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    res = _train_step(model, forest, labels, binding.PERSISTENT)
+    assert util.max_abs(res["h"], ref["h"]) < util.TOL["fp32"]
+    _compare(res, ref, util.TOL["fp32"])
+
+
 @pytest.mark.parametrize("precision,n_trees", [("fp32", 6), ("bf16", 6), ("fp32", 90), ("bf16", 90)])
 def test_weights_of_the_backward_come_with_the_classifier_and_follow_every_update(precision, n_trees):
     """a context without a classifier keeps no weights in the layouts that only the backward reads; the classifier may come

@@ -217,20 +217,22 @@ def test_large_forests_on_either_way(cell, H, kind):
     _training_step(cell, p, forest, binding.PERSISTENT)
 
 
-@pytest.mark.parametrize("kind", ["two callers", "itself", "cycle"])
+@pytest.mark.parametrize("kind", ["two callers", "itself", "cycle", "same children"])
 def test_large_malformed_forests_return_errors(kind):
     """the ways are chosen from the arrays before anything has validated them"""
     rng = np.random.default_rng(950)
     p = fg.draw_recursive_params(rng, 20, 90, tensor=False, emb_scale=0.8, w_scale=0.2)
-    forest = fg.forest_from_shapes([fg.balanced_shape(1024)] * 2, rng, 90)
+    forest = fg.forest_from_shapes([fg.balanced_shape(256)] * 2 + [None] * 200 if kind == "same children" else [fg.balanced_shape(1024)] * 2, rng, 90)
     left, right = forest.left.copy(), forest.right.copy()
     inner = np.flatnonzero(left >= 0)
     if kind == "two callers":
         left[inner[7]] = left[inner[300]]
     elif kind == "itself":
         right[inner[40]] = inner[40]
-    else:                                       # a node below the root calls the root
+    elif kind == "cycle":                       # a node below the root calls the root
         left[inner[3]] = forest.roots[0]
+    else:                                       # 202 trees by the node count, six times as many nodes without a caller
+        left[inner], right[inner] = left[inner[0]], right[inner[0]]
     model = _model(binding.CELL_TREERNN, p)
     with pytest.raises(binding.TreeLSTMError) as err:
         model.forward(util.to_dev(left), util.to_dev(right), util.to_dev(forest.token), flags=binding.PERSISTENT)
