@@ -69,6 +69,7 @@ int copy_params(treelstm* ctx, const float* emb, const float* W, const float* b,
   TL_CUDA(ctx, cudaMemcpyAsync(ctx->b, b, sizeof(float) * 5 * H, cudaMemcpyDeviceToDevice, s));
   if (ctx->precision == TREELSTM_BF16) {
     int rc = pack_weights_bf16(ctx, s);
+    if (rc == TREELSTM_OK) rc = pack_trees_tc(ctx, s);
     if (rc != TREELSTM_OK) return rc;
   }
   int rc = pack_trees(ctx, true, true, s);
@@ -276,6 +277,7 @@ int treelstm_create(treelstm_t** out, int H, int E, int vocab, const float* emb,
       take(ctx->emb_bf, 2 * V * Ep);
       take(ctx->Wp_h, 2 * groups * 40 * 2 * Hp);
       take(ctx->Wp_x, 2 * groups * 24 * Ep);
+      take(ctx->Wp_t, trees_tc_bytes(ctx));
       take(ctx->bp_h, 4 * groups * 40);
       take(ctx->bp_x, 4 * groups * 24);
     }
@@ -293,6 +295,7 @@ int treelstm_create(treelstm_t** out, int H, int E, int vocab, const float* emb,
   if (rc != TREELSTM_OK) return fail(rc);
   ctx->sf = subforest_plan(ctx);
   ctx->tail_ok = ctx->sf.ok && init_tail_attributes(ctx) == TREELSTM_OK;
+  init_trees_tc(ctx);
   *out = ctx;
   return TREELSTM_OK;
 }
@@ -450,8 +453,11 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
                                                                              : kSchedPartMaxNodes;
   const bool subforests = (flags & TREELSTM_SUBFORESTS) && ctx->precision == TREELSTM_BF16 && ctx->sf.ok &&
                           n_nodes > 0 && n_nodes <= single_max;
-  int rc = launch_schedule(ctx, n_nodes, left, right, token, level, order, lvl_off, n_levels, workspace,
-                           lay, subforests ? ctx->sf.n_parts : 0, s);
+  int rc = launch_check_clear(ctx, n_nodes, workspace, lay, s);
+  if (rc != TREELSTM_OK) return rc;
+  rc = trees_tc_asked(ctx, n_nodes, flags)
+           ? launch_schedule_trees_tc(ctx, n_nodes, left, right, token, h, c, level, order, lvl_off, n_levels, save, workspace, lay, s)
+           : launch_schedule(ctx, n_nodes, left, right, token, level, order, lvl_off, n_levels, workspace, lay, subforests ? ctx->sf.n_parts : 0, s);
   if (rc != TREELSTM_OK) return rc;
   const bool persistent = (flags & (TREELSTM_PERSISTENT | TREELSTM_SUBFORESTS)) != 0;
   L.mode = subforests ? TREELSTM_SUBFORESTS : (persistent ? TREELSTM_PERSISTENT : TREELSTM_PER_LEVEL);
@@ -462,8 +468,6 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
     rc = read_levels(ctx);
     if (rc != TREELSTM_OK) { L.valid = false; return rc; }
   }
-  rc = launch_check_clear(ctx, n_nodes, workspace, lay, s);
-  if (rc != TREELSTM_OK) { L.valid = false; return rc; }
   ctx->ev_valid = false;
   if (ctx->opt.time_kernel) TL_CUDA(ctx, cudaEventRecord(ctx->ev_begin, s));
   if (ctx->cell != 0)

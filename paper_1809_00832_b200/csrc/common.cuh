@@ -152,6 +152,7 @@ struct treelstm {
   __nv_bfloat16* emb_bf = nullptr;  // [vocab][Ep]
   __nv_bfloat16* Wp_h = nullptr;    // [(Hp/8)*40][2*Hp]  packed recurrent weights, K contiguous
   __nv_bfloat16* Wp_x = nullptr;    // [(Hp/8)*24][Ep]    packed input weights (gates i, o, u)
+  __nv_bfloat16* Wp_t = nullptr;    // recurrent weights as tensor memory takes them (trees_tc.cu)
   float* bp_h = nullptr;            // [(Hp/8)*40] bias in packed column order
   float* bp_x = nullptr;            // [(Hp/8)*24]
   tl::TmapSet maps;                     // passed to the kernels by value
@@ -160,6 +161,7 @@ struct treelstm {
   int tmap_ws_rows = 0;
   bool have_tmaps = false;
   tl::SubforestPlan sf;                 // filled at create (bf16 only)
+  struct TreesTc { int parts = 0, max_nodes = 0; } ttc;   // trees_tc.cu: clusters beside the scheduler's (0: none), largest forest they are asked about
   bool tail_ok = false;                 // the tail kernel exists for this context's sizes
   int tc_resident_ctas = 0;             // CTAs of the grid-wide bf16 kernel the device holds at once
   bool tail_skip = false;               // the last forward whose control block was read back had no tail worth a hand-over
@@ -279,6 +281,14 @@ int init_tail_attributes(treelstm* ctx);
 int launch_forward_bf16_tail(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token,
                              float* h, float* c, const int32_t* order, const int32_t* level_offset_dev, int flags,
                              void* ws, const WsLayout& lay, cudaStream_t stream);
+
+// trees_tc.cu: the scheduler, and clusters that evaluate whole trees meanwhile
+size_t trees_tc_bytes(const treelstm* ctx);            // an image of the recurrent weights
+int pack_trees_tc(treelstm* ctx, cudaStream_t stream);
+void init_trees_tc(treelstm* ctx);
+bool trees_tc_asked(const treelstm* ctx, int n, int flags);
+int launch_schedule_trees_tc(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h, float* c, int32_t* level,
+                             int32_t* order, int32_t* level_offset, int32_t* n_levels_out, bool save_gates, void* ws, const WsLayout& lay, cudaStream_t stream);
 
 int launch_selftest_waits(treelstm* ctx, void* ws, int* result_dev, cudaStream_t stream);
 

@@ -210,6 +210,7 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
     n_levels = failed ? 0 : p.st->n_levels;
     const int tail_from = only_level < 0 ? tail_first_level(p.level_offset, n_levels, p.tail_width, p.tail_min_levels, s_stop) : n_levels;
     if (only_level < 0 && !failed && blockIdx.x == 0 && tid == 0) p.st->tail_from = tail_from;
+    if (ld_volatile(&p.st->trees_fwd) != 0) return;   // clusters evaluated the forest beside the scheduler (trees_tc.cu)
     lvl_end = only_level >= 0 ? only_level + 1 : (p.tail_launched ? tail_from : n_levels);
     for (int i = tid; i < kLevelCache && i <= n_levels; i += kThreads) s_level_offset[i] = p.level_offset[i];
   }

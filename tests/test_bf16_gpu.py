@@ -5,6 +5,7 @@ import dataclasses
 
 import numpy as np
 import pytest
+import torch
 
 from oracle import treelstm_oracle as orc
 from paper_1809_00832_b200 import binding, forests as fg
@@ -330,6 +331,60 @@ def test_bf16_deeper_than_the_level_cache():
             ref = res
         np.testing.assert_array_equal(res["h"], ref["h"])
         np.testing.assert_array_equal(res["c"], ref["c"])
+
+
+WHOLE_TREES = {
+    # (taken: whether the clusters beside the scheduler evaluate the forest; None: their choice)
+    "as wide as a buffer": (True, lambda rng: [fg.balanced_shape(128), fg.left_chain_shape(30), None]),
+    "wider": (False, lambda rng: [fg.balanced_shape(256), fg.left_chain_shape(30)]),
+    "as many nodes as a cluster takes": (True, lambda rng: [fg.left_chain_shape(1281), fg.left_chain_shape(2)]),
+    "one more": (False, lambda rng: [fg.left_chain_shape(1282)]),
+    "one tree": (True, lambda rng: [fg.random_split_shape(rng, 97)]),
+    "two nodes a depth in turns": (True, lambda rng: [fg.left_chain_shape(40), fg.left_chain_shape(41)]),
+    "trees dealt by size": (True, lambda rng: [fg.random_split_shape(rng, int(n)) for n in rng.integers(1, 50, size=45)]),
+    "more trees than are dealt by size": (None, lambda rng: [fg.left_chain_shape(60)] * 8 + [None if t % 3 else fg.random_split_shape(rng, 4) for t in range(530)]),
+    "looked at in a sample": (True, lambda rng: [fg.left_chain_shape(50)] * 60),
+}
+
+
+@pytest.mark.parametrize("kind", WHOLE_TREES)
+@pytest.mark.parametrize("H,E", [(64, 64), (101, 33), (150, 300), (193, 20), (256, 300)])
+def test_whole_trees_on_clusters_beside_the_scheduler(H, E, kind):
+    """narrow, deep forests go to clusters that take whole trees: every node's contraction runs over the same products in the
+    same order as in the grid-wide kernel, so the states have the same bits; also with gates kept, whose gradients are the same.
+    Depths as wide as an operand buffer, one tile of leaves and a bit, the most nodes a cluster has room for, trees of one leaf,
+    both ways of dealing the trees"""
+    taken, shapes = WHOLE_TREES[kind]
+    rng = np.random.default_rng(1300 + H)
+    params = fg.draw_params(rng, H, E, 300, emb_dist="normal", emb_scale=0.3, w_scale=0.08, n_classes=3)
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes(rng), rng, 300), rng)
+    plain = util.make_model(params, "bf16")
+    plain.set_option(binding.OPT_TAIL_WIDTH, 0)                 # every wavefront on the grid-wide kernel
+    model = util.make_model(params, "bf16")
+    dev = [util.to_dev(a) for a in (forest.left, forest.right, forest.token)]
+    labels = util.to_dev(rng.integers(0, 3, size=forest.n_nodes).astype(np.int32))
+    res = {}
+    for name, m in (("plain", plain), ("model", model)):
+        for flags in (binding.PERSISTENT, binding.PERSISTENT | binding.SAVE_FOR_BACKWARD):
+            out = m.forward(*dev, flags=flags)
+            word = 4 * 9                                         # trees_fwd in the control block at the workspace's start
+            at = (-m._ws.data_ptr()) % 256
+            took = int(m._ws[at + word:at + word + 4].clone().view(torch.int32).item())
+            if name == "plain":
+                assert took == 0
+            elif taken is not None:
+                assert took == int(taken)
+            res[name, flags] = {k: out[k].cpu().numpy() for k in ("h", "c", "level", "order", "n_levels")}
+        res[name, "grads"] = {k: v.cpu().numpy() for k, v in m.backward(labels, forest.n_leaves).items()}
+    for flags in (binding.PERSISTENT, binding.PERSISTENT | binding.SAVE_FOR_BACKWARD):
+        for k, v in res["plain", binding.PERSISTENT].items():
+            np.testing.assert_array_equal(res["model", flags][k], v)
+    # Sums of 32-bit numbers in the order of atomic adds.  A class's bias gradient is the sum of n terms (p - y) / n, magnitudes
+    # that add up to at most one but cancel: its error is a few units of 2^-24 of one, not of the sum.
+    for k in ("dW", "db", "dWc", "dbc", "loss"):
+        a, b = res["model", "grads"][k], res["plain", "grads"][k]
+        assert util.max_abs(a, b) <= 1e-5 * np.abs(b).max() + (2.0 ** -22 if k == "dbc" else 0.0)
+    model.close(); plain.close()
 
 
 def test_narrow_tails_are_handed_to_one_cluster():
