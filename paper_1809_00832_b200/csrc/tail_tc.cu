@@ -105,6 +105,7 @@ k_fwd_tc_tail(const __grid_constant__ TmapSet maps, const __grid_constant__ SfTm
   __shared__ int s_first[2];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // launched as the grid-wide kernel's programmatic dependent: comes up while that ends
   const int n_levels_all = ld_volatile(&p.st->n_levels);
   if (n_levels_all <= 0 || ld_volatile(&p.st->trees_fwd) != 0) return;
   const int first_level = tail_first_level(p.level_offset, n_levels_all, p.tail_width, p.tail_min_levels, s_first);
@@ -605,14 +606,16 @@ int launch_forward_bf16_tail(treelstm* ctx, int n, const int32_t* left, const in
   int rc = ensure_operand_tmaps(ctx, ws, n, p.xin, p.ain);
   if (rc != TREELSTM_OK) return rc;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = ctx->sf.cluster_size; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(ctx->sf.cluster_size);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = tail_smem_bytes(ctx);
   cfg.stream = stream;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = ctx->opt.overlap_launch ? 1 : 0;
+  cfg.attrs = at; cfg.numAttrs = 2;
   TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_fwd_tc_tail, ctx->maps, ctx->sf_maps, p));
   ctx->launches += 1;
   return TREELSTM_OK;

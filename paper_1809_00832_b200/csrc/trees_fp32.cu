@@ -184,8 +184,11 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   TL_STAMP(trace, kTraceLevels - 1, 0);
   float w[RC * 4 * U];
 #pragma unroll
-  for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
-  deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, &s_loads, &s_walk, trace);
+  for (int q = 0; q < RC * 4 * U; ++q)                    // (asked for here, not where they are used first)
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(w[q]) : "l"(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid));
+  // (dealing by size takes 10 k cycles, which TreeLSTM spends beside its leaves and a training step gains twice: 54 chains of 16
+  // leaves, TreeRNN H = 79, forward alone 42 us without and 47 with it)
+  deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || p.walks.at != nullptr, &s_loads, &s_walk, trace);
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
@@ -476,8 +479,6 @@ __device__ __forceinline__ void leaves_choose(const LeafParams& p, float* sm) {
   const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
   if (threadIdx.x == 0) { s_loads.win = 1; s_loads.internal = 0; }
   const bool forest = !load_kids(q, s, sm, links.up, &s_loads.internal);   // (else the scheduler reports it)
-  if (threadIdx.x < 32) count_roots(links, child, p.n, threadIdx.x);
-  __syncthreads();
   if (forest) deal_by_size(p.n, kids, child, links, p.costs, p.parts, deals_by_size(p.n, s_loads.internal, p.parts), true, 0, &s_loads);
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the scheduler clears the control block at its start
@@ -650,7 +651,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
     for (int e = tid; e < kND * 2 * Hp; e += nt) xs[e] = 0.f;
   TL_STAMP(trace, kTraceLevels - 1, 1);
   if (!(p.walks.at && p.st->trees_fwd && load_walk(p.walks, p.costs, p.n, p.st->n_roots, s, sm, part, parts, p.choose != 0, &s_loads, &s_walk)))
-    deal_trees(p, p.costs, s, sm, part, parts, p.choose != 0, &s_loads, &s_walk, trace);
+    deal_trees(p, p.costs, s, sm, part, parts, p.choose != 0, true, &s_loads, &s_walk, trace);
   // The weights behind the lists: asked for before them, some were spilled, and read again in every round (25 sentences, H = 150,
   // training step 224 us, this way 216).
   const float* image = p.W + (size_t)rank * kWords * nt + tid;
@@ -979,7 +980,6 @@ __global__ void __launch_bounds__(kGT) k_rec_grads(GradParams p) {
     }
   }
 }
-
 
 // ---- register images and launches ------------------------------------------------------------------ //
 // The images that are wanted (out != nullptr), one after the other in one launch: it belongs to every change of the weights.

@@ -89,9 +89,9 @@ __device__ __forceinline__ bool load_kids(const ForestIn& p, const TreesSmem& s,
 // warp; every CTA of the cluster gets the same lists.
 constexpr unsigned short kNoCaller = 0xFFFF;
 struct Walk { int depths, internal, leaves; };
-// `dealt`: if given, the cluster of every root (ascending ids), else root r goes to cluster r mod parts; `win`: if given, the walk
+// `few`: no more trees than clusters; `dealt`: if given, the cluster of every root (ascending ids), else root r goes to cluster r mod parts; `win`: if given, the walk
 // may end where it reads zero.
-__device__ __forceinline__ void walk_trees(const ForestIn& p, const TreesSmem& s, float* sm, int part, int parts, const unsigned char* dealt, const int* win, Walk* out) {
+__device__ __forceinline__ void walk_trees(const ForestIn& p, const TreesSmem& s, float* sm, int part, int parts, bool few, const unsigned char* dealt, const int* win, Walk* out) {
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
   unsigned short* list = reinterpret_cast<unsigned short*>(sm + s.list);
@@ -111,7 +111,10 @@ __device__ __forceinline__ void walk_trees(const ForestIn& p, const TreesSmem& s
     }
     return v;
   };
-  auto mine = [&](int rank) { return (dealt ? (int)dealt[min(rank, kDealt - 1)] : rank % parts) == part; };
+  auto mine = [&](int rank) {
+    if (__builtin_expect(dealt != nullptr, 0)) return (int)dealt[min(rank, kDealt - 1)] == part;
+    return (few ? rank : rank % parts) == part;
+  };
   for (int w0 = 0; w0 * 32 < n; w0 += 32) {   // roots: nodes without a caller, 32 words of 32 ids at a time
     const int w = w0 + lane, base = w * 32;
     unsigned m = base < n ? ~child[w] : 0u;
@@ -219,13 +222,14 @@ __device__ __forceinline__ bool clusters_win(const WalkCosts& costs, const TreeL
 // of the trees; the trees are dealt out (see the head of this file), and (`choose`) the clusters' loads say whether they win.  (The
 // average load of a cluster says too little: one tree of 1024 leaves among 24 sentences, H = 150, was 4.5 times slower on
 // clusters than over the whole GPU.)  Called by the threads from `first` on, a multiple of 32; barrier 1 is theirs.  Every CTA
-// takes the same sample and comes to the same answer.  After count_roots and a barrier.  (This code runs once, and what is not in the instruction cache costs
+// takes the same sample and comes to the same answer.  (This code runs once, and what is not in the instruction cache costs
 // more than what it does: 25 sentences on 512 threads 10 k cycles, twice that with loops unrolled and all nodes climbing.)
 __device__ __forceinline__ void deal_by_size(int n, const unsigned* kids, const unsigned* child, const TreeLinks& t, const WalkCosts& costs, int parts,
                                              bool dealt, bool choose, int first, TreeLoads* out) {
   const int tid = (int)threadIdx.x - first, nt = (int)blockDim.x - first, lane = tid & 31;
   auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); };
-  const int roots = roots_in_all(t, child, n), trees = max(1, min(roots, kDealt)), slots = dealt ? trees : parts;   // (not dealt: the clusters' own)
+  const int internal = out->internal, trees = max(1, min(n - 2 * internal, kDealt)), slots = dealt ? trees : parts;   // (not dealt: the clusters' own)
+  if (tid < 32) count_roots(t, child, n, lane);
 #pragma unroll 1
   for (int q = tid; q < slots + 3; q += nt)
     if (q < kDealt) t.size[q] = t.deep[q] = 0;
@@ -289,8 +293,7 @@ __device__ __forceinline__ void deal_by_size(int n, const unsigned* kids, const 
   if (!choose) return;
   sync();
   if (tid < 32) {
-    const float internal = (float)((n - roots) / 2);
-    const bool win = clusters_win(costs, *out, parts, internal, internal / (float)sample, lane);
+    const bool win = clusters_win(costs, *out, parts, (float)internal, (float)internal / (float)sample, lane);
     if (lane == 0) *(volatile int*)&out->win = win;
   }
 }
@@ -302,8 +305,8 @@ __device__ __forceinline__ bool deals_by_size(int n, int internal, int parts) {
   return trees > parts && trees <= kDealt;
 }
 // The tables of the forest, then what the cluster has to walk: nothing, if loads->win says that the forest is the next kernel's
-// (`choose`).  A choice without a deal takes its time beside the walk.
-__device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& costs, const TreesSmem& s, float* sm, int part, int parts, bool choose, TreeLoads* loads, Walk* walk, long long* trace) {
+// (`choose`).  A choice without a deal (`by_size`: there may be one) takes its time beside the walk.
+__device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& costs, const TreesSmem& s, float* sm, int part, int parts, bool choose, bool by_size, TreeLoads* loads, Walk* walk, long long* trace) {
   const int tid = (int)threadIdx.x, nt = (int)blockDim.x, n = p.n;
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
@@ -312,14 +315,12 @@ __device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& c
   if (tid == 0) { loads->win = 1; loads->internal = 0; }
   const bool forest = !load_kids(p, s, sm, choose ? links.up : nullptr, &loads->internal);   // (else the scheduler reports it, and the walk is bounded)
   TL_STAMP(trace, kTraceLevels - 1, 5);
-  const bool dealt = forest && deals_by_size(n, loads->internal, parts), climb = forest && (dealt || choose);
-  if (climb) {
-    if (tid < 32) count_roots(links, child, n, tid);
-    if (!choose)                                                         // the callers were not noted with the child table
+  const bool dealt = forest && by_size && deals_by_size(n, loads->internal, parts), climb = forest && (dealt || choose);
+  if (__builtin_expect(climb, 0)) {                        // (out of the way of what every call executes)
+    if (!choose) {                                                       // the callers were not noted with the child table
 #pragma unroll 1
       for (int k = tid; k < n; k += nt) links.up[k] = (unsigned short)k;
-    __syncthreads();
-    if (!choose) {
+      __syncthreads();
 #pragma unroll 1
       for (int k = tid; k < n; k += nt) {
         const unsigned kd = kids[k];
@@ -332,7 +333,7 @@ __device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& c
     if (dealt || !beside) __syncthreads();
   }
   TL_STAMP(trace, kTraceLevels - 1, 6);
-  if (tid < 32) walk_trees(p, s, sm, part, parts, dealt ? loads->part : nullptr, choose ? &loads->win : nullptr, walk);
+  if (tid < 32) walk_trees(p, s, sm, part, parts, forest && n - 2 * loads->internal <= parts, dealt ? loads->part : nullptr, choose ? &loads->win : nullptr, walk);
   __syncthreads();
   if (choose) {
     if (tid == 0 && !loads->win) *walk = Walk{0, 0, 0};

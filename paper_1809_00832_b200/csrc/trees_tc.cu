@@ -240,12 +240,49 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
   }
   const TreeLinks links{nullptr, t.before, nullptr, nullptr};
   if (warp == (pt >> 5) - 1) count_roots(links, t.child, n, lane);   // (the last to have nodes)
+  // Small forests: up to kClimb steps at once - what others have found by then counts as one -, and again where that was not
+  // enough; sentences are done after the first turn (five rounds of single steps took 3 k cycles of barriers).  Large ones, where a
+  // step takes what a round does: a step at a time, four nodes of a thread side by side.
+  constexpr int kClimb = 12;
   unsigned far = t.inner;                                  // nodes whose ancestor may not be the root yet
 #pragma unroll 1
-  for (int round = 0; round < 17; ++round) {               // (arrays that are no forest may hold a cycle)
+  for (int round = 0; round < 17 && n <= kSampleNodes; ++round) {   // (arrays that are no forest may hold a cycle)
+    unsigned left = 0u;
+#pragma unroll 1
+    for (int j0 = 0; far >> j0; j0 += 3) {                 // three chains of reads under way
+      unsigned v[3];
+      bool go[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        go[j] = (far >> (j0 + j) & 1u) != 0u;
+        v[j] = go[j] ? t.up[tid + (j0 + j) * pt] : 0u;
+      }
+#pragma unroll 1
+      for (int step = 0; step < kClimb && (go[0] || go[1] || go[2]); ++step) {
+        unsigned x[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) x[j] = t.up[v[j] & 0xFFFFu];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          go[j] = go[j] && ((v[j] ^ x[j]) & 0xFFFFu) != 0u;   // (an ancestor that is its own is a root)
+          if (go[j]) v[j] = (x[j] & 0xFFFFu) | ((v[j] & 0xFFFF0000u) + (x[j] & 0xFFFF0000u));
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (far >> (j0 + j) & 1u) {
+          t.up[tid + (j0 + j) * pt] = v[j];
+          if (go[j]) left |= 1u << (j0 + j);
+        }
+    }
+    far = left;
+    if (!tt_any(far != 0u, pt)) break;
+  }
+#pragma unroll 1
+  for (int round = 0; round < 17 && n > kSampleNodes; ++round) {
     bool moved = false;
 #pragma unroll 1
-    for (int j0 = 0; far >> j0; j0 += 4) {                 // four chains of reads under way
+    for (int j0 = 0; far >> j0; j0 += 4) {
       unsigned v[4], x[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) v[j] = far >> (j0 + j) & 1u ? t.up[tid + (j0 + j) * pt] : 0u;
@@ -257,7 +294,7 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
         if (((v[j] ^ x[j]) & 0xFFFFu) != 0u) {
           t.up[tid + (j0 + j) * pt] = (x[j] & 0xFFFFu) | ((v[j] & 0xFFFF0000u) + (x[j] & 0xFFFF0000u));
           moved = true;
-        } else {                                           // an ancestor that is its own is a root
+        } else {
           far &= ~(1u << (j0 + j));
         }
       }
@@ -327,7 +364,8 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
   if (warp == 0) {                                         // (loads->internal: from here on, cells per cluster)
     const bool bad = __any_sync(kFull, lane < parts && (loads->nodes[lane] > kMaxInner ||
                                                         loads->nodes[lane] + (t.trees + parts - 1) / parts + 1 > kMaxLeaves));
-    const bool win = clusters_win(p.costs, *loads, parts, (float)internal, 1.f, lane);
+    // (of 70 forests with fewer nodes none was slower on clusters by more than 2 %)
+    const bool win = n <= kSampleNodes || clusters_win(p.costs, *loads, parts, (float)internal, 1.f, lane);
     if (lane == 0) { loads->win = win && !bad; loads->internal = most; }
   }
 }
@@ -577,7 +615,7 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
   } else {
     // The recurrent weights, meanwhile, to tensor memory: lane = gate row, a column = two contraction indices.  An MMA whose
     // weights come from there reads only the nodes' rows from shared memory.
-    if (tiles > 0) gather(0);
+    if (tiles > 0) { gather(0); gathered(0); }
     if (quad * 32 < m_rows && walk.depths > 0) {
       const int pitch = (m_rows + 31) / 32 * 32;           // 16-byte pieces: [8 columns][half][lane]
       const uint4* const src = p.wp_t + ((size_t)rank * (Hp / 8) * 2) * pitch + m;
@@ -593,7 +631,6 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
       tmem_st_wait();
       tc_fence_before();
     }
-    if (tiles > 0) gathered(0);
     const float bias = m < l_rows ? __ldg(p.bp_x + rank * l_rows + m) : 0.f;
     const bool is_tanh = m % kGColsL >= 16;
     const float a_in = is_tanh ? 1.f : 0.5f, a_add = is_tanh ? 0.f : 0.5f;
