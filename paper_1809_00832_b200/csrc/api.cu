@@ -1,5 +1,7 @@
 // extern "C" entry points of libtreelstm_b200 (declared in include/treelstm.h): argument checks,
 // parameter copies, workspace layout and the launch sequence of one forward / backward call.
+#include <string.h>
+
 #include <new>
 #include <type_traits>
 
@@ -205,9 +207,9 @@ void learn_tail_hint(treelstm* ctx) {
 }
 
 // Waits for the stream of the last call, whose control block is then in ctx->host_status, and says what it holds.
-int finish_status(treelstm* ctx) {
+int finish_status(treelstm* ctx, bool waited = false) {
   auto& L = ctx->last;
-  TL_CUDA(ctx, cudaStreamSynchronize(L.stream));
+  if (!waited) TL_CUDA(ctx, cudaStreamSynchronize(L.stream));
   const int st = reinterpret_cast<const DevStatus*>(ctx->host_status)->status;
   if (st != 0) L.valid = false;
   else learn_tail_hint(ctx);
@@ -285,6 +287,7 @@ int treelstm_create(treelstm_t** out, int H, int E, int vocab, const float* emb,
     if (!pass && (cudaMalloc((void**)&ctx->memory, off) != cudaSuccess ||
                   cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess))
       return fail(TREELSTM_ERR_CUDA);
+    if (!pass) memset(ctx->host_status, 0, sizeof(DevStatus));
     if (pass && init_trees(ctx, images, s) != TREELSTM_OK) return fail(TREELSTM_ERR_CUDA);
   }
   int rc = init_schedule_attributes(ctx);
@@ -326,6 +329,7 @@ int treelstm_create_recursive(treelstm_t** out, int cell, int H, int vocab, cons
   if (cudaMalloc((void**)&ctx->memory, emb_bytes + w_bytes + b_bytes + trees) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess)
     return fail(TREELSTM_ERR_CUDA);
+  memset(ctx->host_status, 0, sizeof(DevStatus));
   ctx->emb = reinterpret_cast<float*>(ctx->memory);
   ctx->Wcat = reinterpret_cast<float*>(ctx->memory + emb_bytes);
   ctx->b = reinterpret_cast<float*>(ctx->memory + emb_bytes + w_bytes);
@@ -429,6 +433,7 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
   if (!ctx) return TREELSTM_ERR_INVALID_ARG;
   ctx->last.valid = false;
   ctx->launches = 0;
+  ctx->status_expected = 0;
   if (!on_own_device(ctx)) return TREELSTM_ERR_STATE;
   if (n_nodes < 0 || !n_levels || !workspace) return TREELSTM_ERR_INVALID_ARG;
   if (n_nodes > 0 && (!left || !right || !token || !h || (!c && ctx->cell == 0) || !level || !order))
@@ -507,6 +512,11 @@ int treelstm_status_sync(treelstm_t* ctx) {
   auto& L = ctx->last;
   if (!L.ws) return TREELSTM_ERR_STATE;
   char* base = static_cast<char*>(L.ws);
+  if (ctx->status_expected != 0 && ctx->status_stream == L.stream) {   // the last kernel of the backward pass writes it
+    TL_CUDA(ctx, cudaStreamSynchronize(L.stream));
+    const volatile DevStatus* hs = reinterpret_cast<const volatile DevStatus*>(ctx->host_status);
+    if (hs->seq == ctx->status_expected) return finish_status(ctx, true);
+  }
   TL_CUDA(ctx, cudaMemcpyAsync(ctx->host_status, base + L.lay.status, sizeof(DevStatus),
                                cudaMemcpyDeviceToHost, L.stream));
   return finish_status(ctx);
@@ -531,6 +541,7 @@ int treelstm_backward(treelstm_t* ctx, const int32_t* labels, float* loss, float
   if (ctx->cell != 0) return TREELSTM_ERR_STATE;   // TreeRNN / RNTN contexts: treelstm_backward_recursive
   if (!on_own_device(ctx)) return TREELSTM_ERR_STATE;
   ctx->launches = 0;
+  ctx->status_expected = 0;
   return launch_backward(ctx, labels, loss, dW, db, dWc, dbc, touched_ids, dEmb_rows, n_touched,
                          static_cast<cudaStream_t>(stream));
 }
@@ -546,6 +557,7 @@ int treelstm_backward_recursive(treelstm_t* ctx, const int32_t* labels, float* l
     return TREELSTM_ERR_STATE;
   if (!on_own_device(ctx)) return TREELSTM_ERR_STATE;
   ctx->launches = 0;
+  ctx->status_expected = 0;
   return launch_backward_rec(ctx, labels, loss, dW, db, dV, dWc, dbc, touched_ids, dEmb_rows, n_touched,
                              static_cast<cudaStream_t>(stream));
 }

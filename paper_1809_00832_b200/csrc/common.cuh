@@ -22,8 +22,10 @@ struct DevStatus {
   unsigned int barrier_bwd;  // arrival counter of the one-launch backward pass (cleared by its launch)
   unsigned int barrier_levels;  // the same of its wavefronts alone, behind k_bwd_begin
   int tail_from;         // persistent bf16 forward: first wavefront the cluster kernel takes (or would take), n_levels if none
-  int trees_fwd, trees_bwd;   // 1: the tree kernels (trees_fp32.cu) took this forest forward / backward
-  int pad[53];
+  int trees_fwd, trees_bwd;   // 1: the tree kernels (trees_fp32.cu, trees_tc.cu) took this forest forward / backward
+  unsigned int tickets;       // CTAs that are done (publish_status)
+  int pad[51];
+  int seq;                    // in the host's copy: the launch that wrote it
 };
 static_assert(sizeof(DevStatus) == 256, "control block is one 256-byte line group");
 
@@ -194,6 +196,8 @@ struct treelstm {
   int32_t* host_level_offset = nullptr;  // pinned, grows on demand
   int host_level_cap = 0;
   int* host_status = nullptr;            // pinned copy of DevStatus
+  int status_seq = 0, status_expected = 0;   // launches that write that copy; the one whose copy is to come (0: none)
+  cudaStream_t status_stream = nullptr;
 
   // buffers of treelstm_forward_host (library-owned, grown on demand)
   struct HostPath {
@@ -292,6 +296,14 @@ int launch_schedule_trees_tc(treelstm* ctx, int n, const int32_t* left, const in
 
 int launch_selftest_waits(treelstm* ctx, void* ws, int* result_dev, cudaStream_t stream);
 
+// For the last launch of a backward pass: where its copy of the control block goes.
+inline int expect_status(treelstm* ctx, cudaStream_t stream) {
+  ctx->status_seq = ctx->status_seq == 0x7FFFFFFF ? 1 : ctx->status_seq + 1;
+  ctx->status_expected = ctx->status_seq;
+  ctx->status_stream = stream;
+  return ctx->status_seq;
+}
+
 // backward.cu
 int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float* dW, float* db, float* dV,
                         float* dWc, float* dbc, int32_t* touched_ids, float* dEmb_rows, int32_t* n_touched,
@@ -347,6 +359,24 @@ int launch_gather_roots(treelstm* ctx, int max_roots, int32_t* root_ids, float* 
 __device__ __forceinline__ void report(DevStatus* st, int code) { atomicMin(&st->status, code); }
 
 __device__ __forceinline__ int ld_volatile(const int* p) { return *(const volatile int*)p; }
+
+// The last kernel of a backward pass leaves the control block in pinned host memory itself: a copy behind it would be 3 us of
+// a step that ends with the host waiting for it.  Every CTA's threads call this last; whichever CTA is the last writes.
+struct StatusOut { int* host; int seq; };
+__device__ __forceinline__ void publish_status(DevStatus* st, const StatusOut& out) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(&st->tickets, 1u) == gridDim.x * gridDim.y * gridDim.z - 1u;
+  }
+  __syncthreads();
+  constexpr int kWords = (int)(sizeof(DevStatus) / sizeof(int));
+  if (!s_last || threadIdx.x >= 32) return;
+  __threadfence();
+  for (int k = threadIdx.x; k < kWords; k += 32) out.host[k] = k == kWords - 1 ? out.seq : reinterpret_cast<volatile int*>(st)[k];
+  if (threadIdx.x == 0) st->tickets = 0u;                  // (a backward pass may be repeated)
+}
 
 // Checked build (-DTREELSTM_CHECKED; compute-sanitizer's stand-in where that tool is not available):
 // every index that a kernel reads from the caller's arrays or from the schedule passes through

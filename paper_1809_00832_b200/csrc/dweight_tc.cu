@@ -42,6 +42,7 @@ struct DwParams {
   const int* tok_slot;          // row of every token in dEmb_rows (third kind of work item only)
   float *dW, *db, *dEmb_rows;   // dEmb_rows == nullptr: the leaves' input gradients are not formed here
   DevStatus* st;
+  StatusOut out;
   long long wait_limit;
   BwdImages img;                // operands split beforehand (forests that went to the grid-wide wavefront kernel)
   int after_trees;              // the tree kernels took the forest if the control block says so, and img holds nothing
@@ -265,13 +266,13 @@ __device__ void dw_from_images(const DwParams& p, int n_leaves, unsigned char* t
   }
 }
 
-__global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
+__device__ __forceinline__ void dweight(DwParams& p) {
   extern __shared__ unsigned char dw_dyn[];
   __shared__ int s_node[kDwMaxRun * kDwBlock], s_ia[kDwMaxRun * kDwBlock], s_ib[kDwMaxRun * kDwBlock];
   __shared__ __align__(8) uint64_t s_bars[2 * kDwStages + 2];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  if (ld_volatile(&p.st->status) != 0) return;   // the passes before failed: nothing here may be trusted
+  if (__syncthreads_or(ld_volatile(&p.st->status) != 0)) return;   // the passes before failed: nothing here may be trusted
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* tiles = dw_dyn + ((1024u - (smem_u32(dw_dyn) & 1023u)) & 1023u);
   const uint32_t tiles_addr = smem_u32(tiles);
@@ -449,6 +450,11 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
     tmem_dealloc(tmem_base, kSpTmemCols);
   }
 }
+__global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  dweight(p);
+  publish_status(p.st, p.out);
+}
 
 }  // namespace
 
@@ -500,6 +506,7 @@ int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t*
   p.tok_slot = tok_slot; p.dEmb_rows = dEmb_rows;
   p.wait_limit = ctx->opt.wait_limit_kcycles * 1024;
   if (n == 0) return TREELSTM_OK;
+  p.out = {ctx->host_status, expect_status(ctx, stream)};
   // The host does not know how the nodes divide into leaves and internal nodes (the level table stayed on the
   // device), so the kernel sizes its work items itself from the grid it finds: one CTA per SM unless even
   // single-block items are fewer (counted for the division that gives the most).
@@ -510,8 +517,13 @@ int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t*
     if (c > items) items = c;
   }
   const int grid = items < ctx->sm_count ? items : ctx->sm_count;
-  k_bwd_dweight_tc<<<grid, kDwThreads, kDwSmemBytes, stream>>>(p);
-  TL_CUDA(ctx, cudaGetLastError());
+  // (as the programmatic dependent of whatever is ahead: it comes up while that ends)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kDwThreads); cfg.dynamicSmemBytes = kDwSmemBytes; cfg.stream = stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization; at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_bwd_dweight_tc, p));
   ctx->launches += 1;
   return TREELSTM_OK;
 }

@@ -892,17 +892,17 @@ struct GradParams {
   const float *h, *dh, *dz;
   float *dW, *db, *dV, *dEmb_rows;
   DevStatus* st;
+  StatusOut out;
 };
-__global__ void __launch_bounds__(kGT) k_rec_grads(GradParams p) {
+__device__ __forceinline__ void rec_grads(const GradParams& p) {
   __shared__ float As[GN][GR];
   __shared__ __align__(16) float Ds[GN][GU];
   __shared__ int s_node[GN], s_l[GN], s_r[GN];
   __shared__ int s_a[GR], s_b[GR];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = p.H, K = p.K;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   // On any error the kernels ahead may have stopped half way: with a label out of range some CTAs of k_bwd_begin give up at
   // their last barrier, and the tokens they would have placed still hold the mark 1, which is no row of dEmb_rows.
-  if (ld_volatile(&p.st->status) != 0 || p.st->n_levels < 1) return;
+  if (__syncthreads_or(ld_volatile(&p.st->status) != 0 || p.st->n_levels < 1)) return;
   const int n_leaves = p.level_offset[1];
   const int grad_ctas = p.tiles * p.splits;
   if ((int)blockIdx.x >= grad_ctas) {
@@ -980,6 +980,12 @@ __global__ void __launch_bounds__(kGT) k_rec_grads(GradParams p) {
     }
   }
 }
+__global__ void __launch_bounds__(kGT) k_rec_grads(const __grid_constant__ GradParams p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  rec_grads(p);
+  publish_status(p.st, p.out);
+}
+
 
 // ---- register images and launches ------------------------------------------------------------------ //
 // The images that are wanted (out != nullptr), one after the other in one launch: it belongs to every change of the weights.
@@ -1298,8 +1304,13 @@ int launch_rec_grads(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb
   if (g.splits > most) g.splits = most;
   if (g.splits < 1) g.splits = 1;
   const int leaf_ctas = L.n / 16 < 64 ? L.n / 16 + 1 : 64;
-  k_rec_grads<<<g.tiles * g.splits + leaf_ctas, kGT, 0, stream>>>(g);
-  TL_CUDA(ctx, cudaGetLastError());
+  g.out = {ctx->host_status, expect_status(ctx, stream)};
+  cudaLaunchConfig_t cfg = {};                            // (the programmatic dependent of whatever is ahead: it comes up while that ends)
+  cfg.gridDim = dim3(g.tiles * g.splits + leaf_ctas); cfg.blockDim = dim3(kGT); cfg.stream = stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization; at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_rec_grads, g));
   ctx->launches += 1;
   return TREELSTM_OK;
 }
