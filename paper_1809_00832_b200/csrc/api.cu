@@ -434,6 +434,7 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
   ctx->last.valid = false;
   ctx->launches = 0;
   ctx->status_expected = 0;
+  ctx->bwd_counters_clear = false;
   if (!on_own_device(ctx)) return TREELSTM_ERR_STATE;
   if (n_nodes < 0 || !n_levels || !workspace) return TREELSTM_ERR_INVALID_ARG;
   if (n_nodes > 0 && (!left || !right || !token || !h || (!c && ctx->cell == 0) || !level || !order))
@@ -467,6 +468,7 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
   const bool persistent = (flags & (TREELSTM_PERSISTENT | TREELSTM_SUBFORESTS)) != 0;
   L.mode = subforests ? TREELSTM_SUBFORESTS : (persistent ? TREELSTM_PERSISTENT : TREELSTM_PER_LEVEL);
   L.valid = true;
+  ctx->bwd_counters_clear = true;                          // with the whole control block
   if (n_nodes == 0) return TREELSTM_OK;
 
   if (!persistent) {

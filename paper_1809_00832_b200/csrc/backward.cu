@@ -1240,6 +1240,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   __shared__ int s_abort, s_flag;
   __shared__ int s_node[kSpTile], s_da[kSpTile], s_db[kSpTile];
   __shared__ int s_off[kWideOffCache];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (ld_volatile(&p.st->status) != 0 || (a.after_trees && p.st->trees_bwd)) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grid = (int)gridDim.x;
   unsigned char* const tiles = wide_dyn + ((1024u - (smem_u32(wide_dyn) & 1023u)) & 1023u);
@@ -1518,7 +1519,9 @@ int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, in
   if (per_sm < 1) return TREELSTM_ERR_UNSUPPORTED;
   int grid = ctx->sm_count * (per_sm < 2 ? per_sm : 2);
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
-  TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, 2 * sizeof(unsigned int), stream));   // and barrier_levels behind it
+  if (!ctx->bwd_counters_clear)          // (2 us of a training step between its forward and its backward)
+    TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, 2 * sizeof(unsigned int), stream));   // and barrier_levels behind it
+  ctx->bwd_counters_clear = false;       // until the pass's last kernel is launched
   const int* lvl_off = ctx->last.level_offset;
   long long wait_limit = ctx->opt.wait_limit_kcycles * 1024;
   void* args[] = {&p, &dV, &sizes, &lvl_off, &wait_limit, &wide};
@@ -1550,8 +1553,20 @@ static int launch_bwd_wide(treelstm* ctx, BwdParams& p, const BwdImages& img, in
   int grid = ctx->sm_count;
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
   WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, after_trees, img};
-  void* args[] = {&p, &a};
-  TL_CUDA(ctx, cudaLaunchCooperativeKernel((void*)k_bwd_wide, dim3(grid), dim3(kWideThreads), args, kWideSmem, stream));
+  // A grid barrier, so every CTA has to be resident: one per SM, as a programmatic dependent that comes up while the tree kernel
+  // ends (and mostly exits: 3 us), or cooperatively (see launch_forward_bf16 for the two ways).
+  int per_sm = 0;
+  TL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_wide, kWideThreads, kWideSmem));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kWideThreads); cfg.dynamicSmemBytes = kWideSmem; cfg.stream = stream;
+  cudaLaunchAttribute at;
+  if (ctx->opt.overlap_launch && per_sm >= 1) {
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization; at.val.programmaticStreamSerializationAllowed = 1;
+  } else {
+    at.id = cudaLaunchAttributeCooperative; at.val.cooperative = 1;
+  }
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_bwd_wide, p, a));
   ctx->launches += 1;
   return TREELSTM_OK;
 }
@@ -1621,6 +1636,7 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
                                                         p.tok_slot, dEmb_rows, p.st, &img, trees, stream);
     }
     TL_CUDA(ctx, cudaMemsetAsync(&p.st->barrier_bwd, 0, sizeof(unsigned int), stream));
+    ctx->bwd_counters_clear = false;
     const int with_dweight = ctx->opt.dw_tensor_cores ? 0 : 1;
     const int rc = launch_bwd_persistent(ctx, p, cls_smem, with_dweight, 0, stream);
     if (rc != TREELSTM_OK) return rc;

@@ -19,7 +19,7 @@ struct DevStatus {
   int max_level;         // scratch of the multi-CTA level assignment
   unsigned int barrier;  // arrival counter of the persistent kernels' grid barrier
   int n_touched;         // distinct leaf tokens (backward)
-  unsigned int barrier_bwd;  // arrival counter of the one-launch backward pass (cleared by its launch)
+  unsigned int barrier_bwd;  // arrival counter of k_bwd_begin or the one-launch backward pass
   unsigned int barrier_levels;  // the same of its wavefronts alone, behind k_bwd_begin
   int tail_from;         // persistent bf16 forward: first wavefront the cluster kernel takes (or would take), n_levels if none
   int trees_fwd, trees_bwd;   // 1: the tree kernels (trees_fp32.cu, trees_tc.cu) took this forest forward / backward
@@ -198,6 +198,7 @@ struct treelstm {
   int* host_status = nullptr;            // pinned copy of DevStatus
   int status_seq = 0, status_expected = 0;   // launches that write that copy; the one whose copy is to come (0: none)
   cudaStream_t status_stream = nullptr;
+  bool bwd_counters_clear = false;       // the backward's arrival counters, in stream order: by the forward, and by the kernel that publishes the status
 
   // buffers of treelstm_forward_host (library-owned, grown on demand)
   struct HostPath {
@@ -301,6 +302,7 @@ inline int expect_status(treelstm* ctx, cudaStream_t stream) {
   ctx->status_seq = ctx->status_seq == 0x7FFFFFFF ? 1 : ctx->status_seq + 1;
   ctx->status_expected = ctx->status_seq;
   ctx->status_stream = stream;
+  ctx->bwd_counters_clear = true;
   return ctx->status_seq;
 }
 
@@ -375,7 +377,7 @@ __device__ __forceinline__ void publish_status(DevStatus* st, const StatusOut& o
   if (!s_last || threadIdx.x >= 32) return;
   __threadfence();
   for (int k = threadIdx.x; k < kWords; k += 32) out.host[k] = k == kWords - 1 ? out.seq : reinterpret_cast<volatile int*>(st)[k];
-  if (threadIdx.x == 0) st->tickets = 0u;                  // (a backward pass may be repeated)
+  if (threadIdx.x == 0) st->tickets = st->barrier_bwd = st->barrier_levels = 0u;   // (a backward pass may be repeated)
 }
 
 // Checked build (-DTREELSTM_CHECKED; compute-sanitizer's stand-in where that tool is not available):
