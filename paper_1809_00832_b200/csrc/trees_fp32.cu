@@ -188,7 +188,16 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(w[q]) : "l"(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid));
   // (dealing by size takes 10 k cycles, which TreeLSTM spends beside its leaves and a training step gains twice: 54 chains of 16
   // leaves, TreeRNN H = 79, forward alone 42 us without and 47 with it)
-  deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || p.walks.at != nullptr, &s_loads, &s_walk, trace);
+  // Of a forest so large that the leaves' kernel takes its turns on the SMs, its choice is known when this kernel gets there: 29
+  // balanced trees of 256 leaves, H = 177, spent 60 us of 523 on lists that nobody walked.  (Some CTAs of a cluster may see it
+  // and others not: the lists alone are left out.)
+  const bool left = CELL == kLstm && p.choose && __syncthreads_or(tid == 0 && ld_volatile(&p.st->trees_left) != 0);
+  if (left) {
+    if (tid == 0) s_walk = Walk{0, 0, 0};
+    __syncthreads();
+  } else {
+    deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || p.walks.at != nullptr, &s_loads, &s_walk, trace);
+  }
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
@@ -482,7 +491,10 @@ __device__ __forceinline__ void leaves_choose(const LeafParams& p, float* sm) {
   if (forest) deal_by_size(p.n, kids, child, links, p.costs, p.parts, deals_by_size(p.n, s_loads.internal, p.parts), true, 0, &s_loads);
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the scheduler clears the control block at its start
-  if (threadIdx.x == 0) p.st->trees_fwd = s_loads.win;
+  if (threadIdx.x == 0) {
+    p.st->trees_fwd = s_loads.win;
+    p.st->trees_left = !s_loads.win;
+  }
 }
 __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ LeafParams p) {
   extern __shared__ __align__(16) float leaf_smem[];
