@@ -195,25 +195,11 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
     if (lane == 0 && own) atomicAdd(&loads->internal, own);
   }
   tt_sync(pt);
-  // a node's word says whose child it is now: a child that two callers claim has one of them (no atomics: the bits of 32
-  // neighbours are one word)
-  bool twice = false;
-#pragma unroll 1
-  for (int j = 0; j * pt + warp * 32 < n; ++j) {
-    const int k = tid + j * pt;
-    const unsigned m = __ballot_sync(kFull, k < n && t.up[min(k, n - 1)] >> 16 != 0u);
-    if (lane == 0) t.child[k >> 5] = m;
-    if (t.inner >> j & 1u) {
-      const unsigned kd = t.kids[k], a = kd & 0xFFFFu, b = kd >> 16;
-      twice = twice || a == b || (t.up[a] & 0xFFFFu) != (unsigned)k || (t.up[b] & 0xFFFFu) != (unsigned)k;
-    }
-  }
-  if (tt_any(twice, pt)) return;
   const int internal = loads->internal;
   if (internal > parts * kMaxInner) return;
-  TL_STAMP(trace, kTraceLevels - 1, 1);
   if (n > kSampleNodes) {
-    // Before the work that grows with the forest, a look at a sample: if most of its nodes lie at a depth that must be wider than
+    // Before most of the work that grows with the forest, a look at a sample (of arrays that are no forest the CTAs may see different
+    // things here; those that go on find that below): if most of its nodes lie at a depth that must be wider than
     // the buffers, or if not even an equal deal would win, the forest is left here (the scheduler takes 30 k cycles, and what the
     // plan takes beyond that the grid-wide kernel waits for: 140 sentences, H = 256, 107 us and not 101).
     constexpr int kDepths = 64;
@@ -238,6 +224,21 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
     const bool over = tid < kDepths - 1 && share * (float)t.wide[tid] > (float)R;   // (the last holds all that are deeper)
     if (tt_any(over || 0.8f * tree_cost(p.costs, nodes, depth, (float)internal) > grid_cost(p.costs, depth, (float)internal), pt)) return;
   }
+  // a node's word says whose child it is now: a child that two callers claim has one of them (no atomics: the bits of 32
+  // neighbours are one word)
+  bool twice = false;
+#pragma unroll 1
+  for (int j = 0; j * pt + warp * 32 < n; ++j) {
+    const int k = tid + j * pt;
+    const unsigned m = __ballot_sync(kFull, k < n && t.up[min(k, n - 1)] >> 16 != 0u);
+    if (lane == 0) t.child[k >> 5] = m;
+    if (t.inner >> j & 1u) {
+      const unsigned kd = t.kids[k], a = kd & 0xFFFFu, b = kd >> 16;
+      twice = twice || a == b || (t.up[a] & 0xFFFFu) != (unsigned)k || (t.up[b] & 0xFFFFu) != (unsigned)k;
+    }
+  }
+  if (tt_any(twice, pt)) return;
+  TL_STAMP(trace, kTraceLevels - 1, 1);
   const TreeLinks links{nullptr, t.before, nullptr, nullptr};
   if (warp == (pt >> 5) - 1) count_roots(links, t.child, n, lane);   // (the last to have nodes)
   // Small forests: up to kClimb steps at once - what others have found by then counts as one -, and again where that was not
