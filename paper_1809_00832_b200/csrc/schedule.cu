@@ -210,6 +210,7 @@ __global__ void k_sched_offsets(int n, const int* level, const int* order, int* 
 __global__ void k_gather_roots(int max_roots, int H, const int* roots, const float* h,
                                const float* c, int* root_ids, float* root_h, float* root_c,
                                int* n_roots_out, const DevStatus* st, int* status_out) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // (comes up while the kernel ahead ends)
   const int n_roots = st->status == 0 ? min(st->n_roots, max_roots) : 0;
   if (blockIdx.x == 0 && threadIdx.x == 0 && n_roots_out) *n_roots_out = n_roots;
   // the control block to pinned host memory (the destinations may lie there as well): no copy behind this kernel
@@ -218,9 +219,17 @@ __global__ void k_gather_roots(int max_roots, int H, const int* roots, const flo
   for (int t = blockIdx.x; t < n_roots; t += gridDim.x) {
     const int node = roots[t];   // written by the scheduler from ids below n
     if (threadIdx.x == 0 && root_ids) root_ids[t] = node;
-    for (int j = threadIdx.x; j < H; j += blockDim.x) {
-      if (root_h) root_h[(size_t)t * H + j] = h[(size_t)node * H + j];
-      if (root_c) root_c[(size_t)t * H + j] = c[(size_t)node * H + j];
+    // Half of the threads take h, the others c; 16 bytes each where every row starts on such a boundary (host memory behind PCIe:
+    // the size of the pieces matters).
+    const int half = (int)blockDim.x / 2, side = (int)threadIdx.x >= half, at = (int)threadIdx.x - side * half;
+    float* const to = side ? root_c : root_h;
+    const float* const from = side ? c : h;
+    if (!to) continue;
+    const size_t src = (size_t)node * H, dst = (size_t)t * H;
+    if (H % 4 == 0 && ((reinterpret_cast<uintptr_t>(to) | reinterpret_cast<uintptr_t>(from)) & 15) == 0) {
+      for (int j = at; j < H / 4; j += half) reinterpret_cast<float4*>(to + dst)[j] = reinterpret_cast<const float4*>(from + src)[j];
+    } else {
+      for (int j = at; j < H; j += half) to[dst + j] = from[src + j];
     }
   }
 }
@@ -389,10 +398,14 @@ int launch_gather_roots(treelstm* ctx, int max_roots, int32_t* root_ids, float* 
   const DevStatus* st = reinterpret_cast<const DevStatus*>(base + L.lay.status);
   const int* roots = reinterpret_cast<const int*>(base + L.lay.roots);
   int blocks = max_roots < 1 ? 1 : (max_roots < 1184 ? max_roots : 1184);
-  k_gather_roots<<<blocks, 128, 0, stream>>>(max_roots, ctx->H, roots, L.h, L.c, root_ids, root_h,
-                                             L.c ? root_c : nullptr, n_roots, st, status_out);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks); cfg.blockDim = dim3(128); cfg.stream = stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization; at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_gather_roots, max_roots, ctx->H, (const int*)roots, (const float*)L.h, (const float*)L.c, (int*)root_ids, root_h,
+                                  L.c ? root_c : nullptr, (int*)n_roots, (const DevStatus*)st, status_out));
   ctx->launches += 1;
-  TL_CUDA(ctx, cudaGetLastError());
   return TREELSTM_OK;
 }
 
