@@ -184,8 +184,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   TL_STAMP(trace, kTraceLevels - 1, 0);
   float w[RC * 4 * U];
 #pragma unroll
-  for (int q = 0; q < RC * 4 * U; ++q)                    // (asked for here, not where they are used first)
-    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(w[q]) : "l"(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid));
+  for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
   // (dealing by size takes 10 k cycles, which TreeLSTM spends beside its leaves and a training step gains twice: 54 chains of 16
   // leaves, TreeRNN H = 79, forward alone 42 us without and 47 with it)
   // Of a forest so large that the leaves' kernel takes its turns on the SMs, its choice is known when this kernel gets there: 29

@@ -51,7 +51,7 @@ __host__ __device__ inline TreesSmem trees_smem(int n, int buf_words) {
 constexpr unsigned kLeafBit = 0x80000000u;
 __device__ __forceinline__ bool is_leaf(unsigned kids) { return (kids & kLeafBit) != 0; }
 // (up: if given, every node's caller, a root's itself.  Two callers of one child are no forest: which of them is found is a matter of timing, so
-// the answer is true then, the same in every CTA.  internal: zero before; how many nodes have children.)
+// the answer is true then, the same in every CTA.  internal: if given, zero before; how many nodes have children.)
 __device__ __forceinline__ bool load_kids(const ForestIn& p, const TreesSmem& s, float* sm, unsigned short* up, int* internal) {
   unsigned* kids = reinterpret_cast<unsigned*>(sm + s.kids);
   unsigned* child = reinterpret_cast<unsigned*>(sm + s.child);
@@ -79,8 +79,10 @@ __device__ __forceinline__ bool load_kids(const ForestIn& p, const TreesSmem& s,
       }
     }
   }
-  own = __reduce_add_sync(kFull, own);
-  if ((threadIdx.x & 31) == 0) atomicAdd(internal, own);
+  if (internal) {
+    own = __reduce_add_sync(kFull, own);
+    if ((threadIdx.x & 31) == 0) atomicAdd(internal, own);
+  }
   return __syncthreads_or(twice) != 0;
 }
 
@@ -313,7 +315,7 @@ __device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& c
   const bool beside = s.state_words >= deal_words(n);
   const TreeLinks links = tree_links(sm + (beside ? s.state : s.list), n);
   if (tid == 0) { loads->win = 1; loads->internal = 0; }
-  const bool forest = !load_kids(p, s, sm, choose ? links.up : nullptr, &loads->internal);   // (else the scheduler reports it, and the walk is bounded)
+  const bool forest = !load_kids(p, s, sm, choose ? links.up : nullptr, choose || by_size ? &loads->internal : nullptr);   // (else the scheduler reports it, and the walk is bounded)
   TL_STAMP(trace, kTraceLevels - 1, 5);
   const bool dealt = forest && by_size && deals_by_size(n, loads->internal, parts), climb = forest && (dealt || choose);
   if (__builtin_expect(climb, 0)) {                        // (out of the way of what every call executes)
@@ -333,7 +335,7 @@ __device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& c
     if (dealt || !beside) __syncthreads();
   }
   TL_STAMP(trace, kTraceLevels - 1, 6);
-  if (tid < 32) walk_trees(p, s, sm, part, parts, forest && n - 2 * loads->internal <= parts, dealt ? loads->part : nullptr, choose ? &loads->win : nullptr, walk);
+  if (tid < 32) walk_trees(p, s, sm, part, parts, by_size && forest && n - 2 * loads->internal <= parts, dealt ? loads->part : nullptr, choose ? &loads->win : nullptr, walk);
   __syncthreads();
   if (choose) {
     if (tid == 0 && !loads->win) *walk = Walk{0, 0, 0};
