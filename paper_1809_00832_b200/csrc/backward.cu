@@ -174,6 +174,63 @@ __device__ __forceinline__ void scan_place_groups(const BwdParams& p, const int*
     }
   }
 }
+// The same without flags in memory, behind a single grid barrier: a CTA finds the leaf tokens of its own run of groups in the
+// forest itself, every owner reading all of it, and keeps them as bits in shared memory.  The flags need two grid barriers more (cleared |
+// set | counted | placed).
+struct OwnTokens {
+  int g0, g1;                                            // groups of 128 ids
+  __device__ OwnTokens(int vocab) {
+    const int n_groups = (vocab + 127) / 128, per = (n_groups + (int)gridDim.x - 1) / (int)gridDim.x;
+    g0 = min(n_groups, (int)(gridDim.x - 1 - blockIdx.x) * per);
+    g1 = min(n_groups, g0 + per);
+  }
+};
+__device__ __forceinline__ void own_tokens_count(const BwdParams& p, const OwnTokens& t, unsigned int* s_mask, int* group_count) {
+  if (t.g0 == t.g1) return;
+  const int tid = threadIdx.x, words = 4 * (t.g1 - t.g0);
+  for (int w = tid; w < words; w += blockDim.x) s_mask[w] = 0u;
+  __syncthreads();
+  constexpr int kBatch = 8;
+  for (int i0 = tid; i0 < p.n; i0 += kBatch * (int)blockDim.x) {
+    int left[kBatch], token[kBatch];
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const int i = min(i0 + b * (int)blockDim.x, p.n - 1);      // (the last node more than once: the same bit)
+      left[b] = __ldg(p.left + i);
+      token[b] = __ldg(p.token + i);
+    }
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const unsigned int at = (unsigned int)(token[b] - 128 * t.g0);
+      if (left[b] < 0 && at < 32u * (unsigned int)words) atomicOr(s_mask + (at >> 5), 1u << (at & 31u));
+    }
+  }
+  __syncthreads();
+  for (int g = t.g0 + tid; g < t.g1; g += blockDim.x) {
+    const uint4 m = reinterpret_cast<const uint4*>(s_mask)[g - t.g0];
+    group_count[g] = __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);
+  }
+}
+__device__ __forceinline__ void own_tokens_place(const BwdParams& p, const OwnTokens& t, const unsigned int* s_mask, const int* group_count) {
+  if (threadIdx.x >= 32 || t.g0 == t.g1) return;
+  const int lane = threadIdx.x, n_groups = (p.vocab + 127) / 128;
+  int base = 0;
+  for (int q = lane; q < t.g0; q += 32) base += ld_volatile(group_count + q);
+  base = __reduce_add_sync(kFull, base);
+  for (int g = t.g0; g < t.g1; ++g) {
+    const unsigned int* m = s_mask + 4 * (g - t.g0);
+    const unsigned int mine = m[lane >> 3], shift = 4u * (lane & 7u);
+    int e = base + __popc(mine & ((1u << shift) - 1u));  // rows before this lane's four ids
+    for (int w = 0; w < lane >> 3; ++w) e += __popc(m[w]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int id = 128 * g + 4 * lane + k;
+      if ((mine >> (shift + k)) & 1u) { p.tok_slot[id] = e; p.touched_ids[e] = id; ++e; }
+    }
+    base += __popc(m[0]) + __popc(m[1]) + __popc(m[2]) + __popc(m[3]);
+  }
+  if (t.g1 == n_groups && lane == 0) { *p.n_touched = base; p.st->n_touched = base; }
+}
 constexpr int kScanMaskWords = 8192;
 __global__ void __launch_bounds__(1024) k_bwd_scan_tokens(BwdParams p) {
   __shared__ __align__(16) unsigned int s_mask[kScanMaskWords];
@@ -1458,13 +1515,19 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   }
 }
 
-// What precedes the walk over the trees (trees_fp32.cu), in one cooperative launch: outputs cleared | leaf tokens
-// marked | tokens counted beside the classifier | tokens placed.  The level table stays on the device.
+// What precedes the walk over the trees (trees_fp32.cu), in one cooperative launch: outputs cleared beside the count of every run of
+// token ids | classifier, tokens placed; large forests: outputs cleared | leaf tokens marked | tokens counted beside the classifier | tokens
+// placed.  Bound by the latency of its grid barriers and of the classifier's chain.  The level table stays on the device.
 struct GradSizes { size_t dW, db, dV; };   // floats
+constexpr int kBeginMaskWords = 1024;
+// Leaf tokens found by the CTA that numbers them rather than flagged in memory: every owner reads the whole forest, two grid barriers and the
+// clearing of the flags are saved.  Backward passes, H = 64, 20 000 words, own | flags, us: 106 nodes 105.7 | 110.9, 1.4 k 133.6 | 139.4, 15 k
+// 282.5 | 285.5, 30 k 337.8 | 336.8, 60 k 472 | 460; 200 000 words 108 | 117, 136 | 145, 284 | 291, 341 | 345, 475 | 469.
+constexpr int kOwnTokensMaxNodes = 20000;
 __global__ void __launch_bounds__(256, 2)
 k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, long long wait_limit, int wide) {
   extern __shared__ float s_cls[];
-  __shared__ __align__(16) unsigned int s_mask[1024];
+  __shared__ __align__(16) unsigned int s_mask[kBeginMaskWords];
   __shared__ int s_flag;
   // the kernel behind this one may set itself up: it waits for this grid before it reads dh
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1483,11 +1546,15 @@ k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, lo
   zero_range(dV, sizes.dV, gtid, gthreads);
   zero_range(p.dWc, (size_t)H * C, gtid, gthreads);
   zero_range(p.dbc, (size_t)C, gtid, gthreads);
-  zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
+  const OwnTokens own_tokens(p.vocab);
+  const bool own = gridDim.x > 1 && p.n <= kOwnTokensMaxNodes && 4 * (((p.vocab + 127) / 128 + (int)gridDim.x - 1) / (int)gridDim.x) <= kBeginMaskWords;
+  if (!own) zero_range(p.tok_slot, (size_t)p.vocab + 1, gtid, gthreads);
   zero_range(p.dEmb_rows, (size_t)p.n_leaves * p.E, gtid, gthreads);
   if (wide) zero_range(p.dc, (size_t)p.n * H, gtid, gthreads);   // k_bwd_wide may follow: dc of the roots
-  if (!barrier()) return;
-  for (size_t r = gtid; r < (size_t)(wide ? p.n : p.n_leaves); r += gthreads) {
+  int* const group_count = p.tok_slot + p.vocab + 4;
+  if (own) own_tokens_count(p, own_tokens, s_mask, group_count);
+  else if (!barrier()) return;
+  for (size_t r = own ? (size_t)p.n_leaves + gtid : gtid; r < (size_t)(wide ? p.n : p.n_leaves); r += gthreads) {
     const int node = chk(p.st, p.order[r], p.n);
     if (r < (size_t)p.n_leaves) {
       p.tok_slot[chk(p.st, p.token[node], p.vocab)] = 1;
@@ -1497,9 +1564,11 @@ k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, lo
     }
   }
   if (!barrier()) return;
-  int* const group_count = p.tok_slot + p.vocab + 4;
-  if (gridDim.x == 1) {
-    scan_tokens(p, s_mask, 1024);
+  if (own) {
+    classifier_groups(p, blockIdx.x, gridDim.x, s_cls);
+    own_tokens_place(p, own_tokens, s_mask, group_count);
+  } else if (gridDim.x == 1) {
+    scan_tokens(p, s_mask, kBeginMaskWords);
     classifier_groups(p, 0, 1, s_cls);
   } else {
     scan_count_groups(p, group_count);

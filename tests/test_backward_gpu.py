@@ -273,6 +273,32 @@ def test_trees_dealt_by_size(H, n_trees):
     _compare(res, ref, util.TOL["fp32"])
 
 
+@pytest.mark.parametrize("vocab,trees,ctas", [
+    (1, (3, 2), 0), (2, (5, 1), 0), (127, (40, 5), 0), (128, (40, 5), 0), (129, (40, 5), 0), (37888, (60, 9), 0), (37889, (60, 9), 0),
+    (65536, (60, 9), 2), (65537, (60, 9), 2), (300, (6000, 2000), 0), (300, (6001, 1998), 0)])
+def test_touched_tokens_and_their_rows(vocab, trees, ctas):
+    """one id, groups of 128 ids with a partial one, one and two groups a CTA on 148 SMs, as many ids as two CTAs keep and one more; the
+    largest forest whose tokens are found by the CTAs that number them (20000 nodes) and one of 20001.  First and last id are in use"""
+    rng = np.random.default_rng(vocab + trees[0])
+    H, E = 8, 8
+    params = fg.draw_params(rng, H, E, vocab, emb_dist="normal", emb_scale=0.3, w_scale=0.25, n_classes=3)
+    shapes = [fg.balanced_shape(2)] * trees[0] + [None] * trees[1]
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes, rng, vocab), rng)
+    leaves = np.flatnonzero(forest.left < 0)
+    forest.token[leaves[0]], forest.token[leaves[-1]] = 0, vocab - 1
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    if ctas:
+        model.set_option(binding.OPT_MAX_CTAS, ctas)
+    res = _train_step(model, forest, labels, binding.PERSISTENT)
+    m = int(res["n_touched"][0])
+    assert m == len(ref["touched_ids"])
+    assert np.array_equal(res["touched_ids"][:m], ref["touched_ids"])
+    _compare(res, ref, util.TOL["fp32"])
+
+
 @pytest.mark.parametrize("precision,n_trees", [("fp32", 6), ("bf16", 6), ("fp32", 90), ("bf16", 90)])
 def test_weights_of_the_backward_come_with_the_classifier_and_follow_every_update(precision, n_trees):
     """a context without a classifier keeps no weights in the layouts that only the backward reads; the classifier may come
