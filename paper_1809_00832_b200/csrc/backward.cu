@@ -331,14 +331,18 @@ __device__ __forceinline__ void classifier_nodes(const BwdParams& p, int warp_fi
     for (int k = 0; k < kClsRegC; ++k)
       if (lane + 32 * t < H && k < C) atomicAdd(&s_dWc[(lane + 32 * t) * C + k], acc[t][k]);
   if (lane < C) atomicAdd(&s_dWc[H * C + lane], acc_b);
-  if (lane == 0 && loss != 0.f) atomicAdd(p.loss, loss * inv_n);
+  if (lane == 0 && loss != 0.f) atomicAdd(&s_dWc[H * C + C], loss * inv_n);
 }
 
 // The CTA takes the node groups vb_first, vb_first + vb_step, ...; s_dWc [H][C] + [C] collects its partial sums.
-__device__ void classifier_groups(const BwdParams& p, int vb_first, int vb_step, float* s_dWc) {
+struct AlreadyCleared { __device__ bool operator()() const { return true; } };
+// (s_dWc: the CTA's sums of dWc, dbc and the loss, H C + C + 1 words.  They are added to the outputs behind `cleared`, which says whether
+// to go on; the nodes' dh need not wait for that.)
+template <typename Cleared>
+__device__ bool classifier_groups(const BwdParams& p, int vb_first, int vb_step, float* s_dWc, Cleared cleared) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int H = p.H, C = p.C;
-  for (int i = tid; i < H * C + C; i += blockDim.x) s_dWc[i] = 0.f;
+  for (int i = tid; i < H * C + C + 1; i += blockDim.x) s_dWc[i] = 0.f;
   __syncthreads();
 #ifdef TREELSTM_TRACE
   long long* const ctrace = blockIdx.x == 1 && tid == 0 ? p.trace : nullptr;   // the first CTA with nodes to classify
@@ -378,7 +382,7 @@ __device__ void classifier_groups(const BwdParams& p, int vb_first, int vb_step,
     if (!y_ok && lane == 0) report(p.st, TREELSTM_ERR_LABEL_OUT_OF_RANGE);
     const float lse = m + logf(sum);
     const float logit_y = __shfl_sync(kFull, logit, y_ok ? y : 0);
-    if (lane == 0 && y_ok) atomicAdd(p.loss, (lse - logit_y) * inv_n);
+    if (lane == 0 && y_ok) atomicAdd(&s_dWc[H * C + C], (lse - logit_y) * inv_n);
     const float dlogit = lane < C ? (e / sum - (lane == y ? 1.f : 0.f)) * inv_n : 0.f;
     if (lane < C) atomicAdd(&s_dWc[H * C + lane], dlogit);
     for (int j0 = 0; j0 < H; j0 += 32) {
@@ -399,14 +403,17 @@ __device__ void classifier_groups(const BwdParams& p, int vb_first, int vb_step,
   }
   __syncthreads();
   TL_STAMP(ctrace, kTraceLevels - 1, 13);     // all warps: nodes done
-  if (vb_first >= n_groups) return;   // a CTA without a group has nothing to add (and 300 CTAs adding zeros to the same H x C words queue up)
+  if (!cleared()) return false;
+  if (vb_first >= n_groups) return true;   // a CTA without a group has nothing to add (and 300 CTAs adding zeros to the same H x C words queue up)
   for (int i = tid; i < H * C; i += blockDim.x) atomicAdd(&p.dWc[i], s_dWc[i]);
   for (int i = tid; i < C; i += blockDim.x) atomicAdd(&p.dbc[i], s_dWc[H * C + i]);
+  if (tid == 0) atomicAdd(p.loss, s_dWc[H * C + C]);
   TL_STAMP(ctrace, kTraceLevels - 1, 14);     // partial sums sent
+  return true;
 }
 __global__ void __launch_bounds__(kClsWarps * 32) k_bwd_classifier(BwdParams p) {
   extern __shared__ float s_dyn[];
-  classifier_groups(p, blockIdx.x, gridDim.x, s_dyn);
+  classifier_groups(p, blockIdx.x, gridDim.x, s_dyn, AlreadyCleared{});
 }
 
 // ---- gate gradients of one wavefront -------------------------------------------------------- //
@@ -953,10 +960,10 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
   if (after_begin) {
   } else if (gridDim.x == 1) {
     scan_tokens(p, s_mask, mask_cap);
-    classifier_groups(p, 0, 1, s_cls);
+    classifier_groups(p, 0, 1, s_cls, AlreadyCleared{});
   } else {
     scan_count_groups(p, group_count);
-    classifier_groups(p, blockIdx.x, gridDim.x, s_cls);
+    classifier_groups(p, blockIdx.x, gridDim.x, s_cls, AlreadyCleared{});
   }
   TL_STAMP(trace, kTraceLevels - 1, 3);   // this CTA's part (the first one: the token scan) done
   if (!after_begin && !barrier()) return;
@@ -1563,24 +1570,28 @@ k_bwd_begin(BwdParams p, float* dV, GradSizes sizes, const int* level_offset, lo
       p.pos_right[r] = p.right[node];
     }
   }
+  if (own) {                               // the barrier in two halves: by the time the nodes are classified everybody has arrived
+    __syncthreads();
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&p.st->barrier_bwd) : "memory");
+    if (classifier_groups(p, blockIdx.x, gridDim.x, s_cls, [&]() { return grid_barrier(p.st, gridDim.x, wait_limit, &s_flag, false, &p.st->barrier_bwd); }))
+      own_tokens_place(p, own_tokens, s_mask, group_count);
+    return;
+  }
   if (!barrier()) return;
-  if (own) {
-    classifier_groups(p, blockIdx.x, gridDim.x, s_cls);
-    own_tokens_place(p, own_tokens, s_mask, group_count);
-  } else if (gridDim.x == 1) {
+  if (gridDim.x == 1) {
     scan_tokens(p, s_mask, kBeginMaskWords);
-    classifier_groups(p, 0, 1, s_cls);
+    classifier_groups(p, 0, 1, s_cls, AlreadyCleared{});
   } else {
     scan_count_groups(p, group_count);
-    classifier_groups(p, blockIdx.x, gridDim.x, s_cls);
+    classifier_groups(p, blockIdx.x, gridDim.x, s_cls, AlreadyCleared{});
     if (!barrier()) return;
     scan_place_groups(p, group_count);
   }
 }
 
 int launch_bwd_begin(treelstm* ctx, BwdParams& p, float* dV, GradSizes sizes, int wide, cudaStream_t stream) {
-  const size_t smem = sizeof(float) * ((size_t)p.H * p.C + p.C);
-  if (smem > 160 * 1024) return TREELSTM_ERR_UNSUPPORTED;
+  const size_t smem = sizeof(float) * ((size_t)p.H * p.C + p.C + 1);
+  if (smem > 160 * 1024 + sizeof(float)) return TREELSTM_ERR_UNSUPPORTED;
   if (smem > 40 * 1024)
     TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_begin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
@@ -1675,8 +1686,8 @@ int launch_backward(treelstm* ctx, const int32_t* labels, float* loss, float* dW
 #endif
 
   const size_t J = 5 * (size_t)H;
-  const size_t cls_smem = sizeof(float) * ((size_t)H * C + C);
-  if (cls_smem > 160 * 1024) return TREELSTM_ERR_UNSUPPORTED;
+  const size_t cls_smem = sizeof(float) * ((size_t)H * C + C + 1);
+  if (cls_smem > 160 * 1024 + sizeof(float)) return TREELSTM_ERR_UNSUPPORTED;
   if (one_launch) {
     if (n == 0) {
       TL_CUDA(ctx, cudaMemsetAsync(loss, 0, sizeof(float), stream));
@@ -1991,8 +2002,8 @@ int launch_backward_rec(treelstm* ctx, const int32_t* labels, float* loss, float
   p.tok_slot = reinterpret_cast<int*>(base + L.lay.tok_slot);
   p.touched_ids = touched_ids; p.n_touched = n_touched;
   p.st = reinterpret_cast<DevStatus*>(base + L.lay.status);
-  const size_t cls_smem = sizeof(float) * ((size_t)H * C + C);
-  if (cls_smem > 160 * 1024) return TREELSTM_ERR_UNSUPPORTED;
+  const size_t cls_smem = sizeof(float) * ((size_t)H * C + C + 1);
+  if (cls_smem > 160 * 1024 + sizeof(float)) return TREELSTM_ERR_UNSUPPORTED;
   TL_CUDA(ctx, cudaMemsetAsync(p.tok_slot, 0, sizeof(int) * ((size_t)ctx->vocab + 1), stream));
   TL_CUDA(ctx, cudaMemsetAsync(dEmb_rows, 0, sizeof(float) * (size_t)n_leaves * H, stream));
   k_bwd_mark_tokens<<<(n_leaves + 255) / 256, 256, 0, stream>>>(p);
