@@ -68,7 +68,8 @@ typedef enum treelstm_status {
 #define TREELSTM_PER_LEVEL 0    /* one launch per wavefront; synchronises the stream once to read   */
                                 /* the level table, returns device-detected errors directly          */
 #define TREELSTM_PERSISTENT 1   /* no launch per wavefront: one kernel loops over the wavefronts with */
-                                /* a bounded grid-wide barrier, or (fp32) clusters walk whole trees,  */
+                                /* a bounded grid-wide barrier, or clusters walk whole trees (bf16:   */
+                                /* in the scheduler's launch, H padded to <= 256, up to 16384 nodes), */
                                 /* whichever suits the forest; fully asynchronous (see                */
                                 /* treelstm_status_sync)                                              */
 #define TREELSTM_SAVE_FOR_BACKWARD 2 /* keep every node's gate activations for treelstm_backward   */
@@ -89,7 +90,8 @@ typedef enum treelstm_status {
                                             /* 1024 SM clock cycles                                  */
 #define TREELSTM_OPT_MAX_CTAS 3             /* cap on the persistent grid (0 = all co-resident CTAs) */
 #define TREELSTM_OPT_TIME_WAVEFRONT_KERNEL 4 /* 1: bracket the wavefront kernel launch(es) of each  */
-                                            /* forward with CUDA events (treelstm_last_kernel_ms)    */
+                                            /* forward with CUDA events (treelstm_last_kernel_ms);   */
+                                            /* bf16 forests then all go to those                     */
 #define TREELSTM_OPT_TAIL_WIDTH 5           /* TREELSTM_PERSISTENT, bf16, H padded to <= 256: the last    */
                                             /* wavefronts of a forest, once every remaining one has at    */
                                             /* most this many nodes (default 32, largest value 64), may   */
@@ -98,13 +100,13 @@ typedef enum treelstm_status {
                                             /* from child to caller through distributed shared memory.     */
                                             /* Decided by the library on the device (see below), same      */
                                             /* results bit for bit; 0 keeps every wavefront on the         */
-                                            /* grid-wide kernel                                            */
+                                            /* grid-wide kernel (no clusters that take whole trees either)  */
 #define TREELSTM_OPT_TAIL_MIN_LEVELS 6      /* 0 (default): the hand-over happens if a cost model fitted   */
                                             /* to cycle traces says that the narrow wavefronts save more   */
                                             /* than the second launch costs (deep, narrow forests: yes; a  */
                                             /* few narrow wavefronts on top of a wide forest: no).         */
                                             /* > 0: it happens whenever at least this many wavefronts      */
-                                            /* remain                                                      */
+                                            /* remain, and no clusters take whole trees                    */
 #define TREELSTM_OPT_TAIL_MAX_NODES 7       /* forests with more nodes than this (default 4096) never      */
                                             /* launch the cluster kernel: the host knows the node count    */
                                             /* only, and a large forest has nothing to gain.  The second   */

@@ -141,6 +141,18 @@ def main() -> int:
         print("# scheduler, thread 0, cycles since its start: " + ", ".join(f"{nm} {int(buf[i])}" for i, nm in enumerate(names)))
     for which, name in ((0, "grid-wide kernel"), (1, "cluster kernel")):
         t = read_trace(model, which)
+        ph = t[LEVELS - 1]
+        if which == 1 and ph[6] > ph[0] > 0:             # whole trees on clusters beside the scheduler
+            print("# clusters that take whole trees, first CTA, cycles since its start: " + ", ".join(
+                f"{what} {int(ph[k] - ph[0])}" for k, what in enumerate(
+                    ("children linked", "trees dealt", "decided", "lists", "leaves", "leaves' states exchanged"), 1)))
+            print("step  issued  retired gates   pushed  next (cycles since the depth's operands were complete; deepest depth first)")
+            for i in range(LEVELS - 1):
+                if t[i, 0] <= ph[0]:
+                    break
+                nxt = t[i + 1, 0] - t[i, 0] if t[i + 1, 0] > t[i, 0] and i + 2 < LEVELS else 0
+                print(f"{i:<5d} " + " ".join(f"{t[i, k] - t[i, 0]:<7d}" for k in range(1, 5)) + f" {nxt}")
+            continue
         rows = [l for l in range(min(len(widths), LEVELS)) if t[l, 0] != 0]
         if not rows:
             continue
