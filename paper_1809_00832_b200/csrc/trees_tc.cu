@@ -6,7 +6,7 @@
 // global memory, grid barrier, operand rows back through TMA, MMAs, cell update.  A cluster that has all of a tree needs none of
 // the first three: the new bf16 h goes straight into the shared memory of the CTAs that multiply with it next.  And nothing waits
 // for the schedule: a cluster needs only "children before parents", so it walks its trees by distance from the root, deepest
-// first, which it finds from the child arrays itself (tt_plan).  The launch is the scheduler's: its first cluster
+// first, which it finds from the child arrays itself (tt_decide, tt_lists).  The launch is the scheduler's: its first cluster
 // schedules, the others evaluate meanwhile, or leave the forest to the grid-wide kernel behind (DevStatus::trees_fwd).
 //
 // One depth.  CTA r of a cluster owns hidden units [r U, (r + 1) U), U = 8 gpc, and keeps the packed recurrent weights of those
@@ -20,13 +20,13 @@
 // depth d (the argument is the same for the gate values, which take the buffer of the depth being finished).  There is no other
 // signal between CTAs.  Cell states stay with the units' owner.
 //
-// Leaves first: tiles of 64 leaves of the cluster's trees, every CTA its own units, the same orientation (weights M, leaves N).
+// Leaves first: tiles of 96 leaves of the cluster's trees, every CTA its own units, the same orientation (weights M, leaves N).
 //
 // Measured (H = 256, 11 nodes a depth): a depth takes 3.6 k cycles - 32 MMAs 1.1 k (34 cycles each whatever their width; 43 with the
 // weights in shared memory), their retirement seen 0.35 k, gate values to shared memory 0.5 k, cell updates, pushes and their way
 // 1.7 k (the interconnect moves about 8 bytes a cycle and CTA) - where the grid-wide kernel takes 7.8 k: 64 chains of 64 leaves
-// 308 -> 180 us, 25 sentences (H = 150) 82 -> 48.  The plan takes 13 k cycles for one sentence and 49 k for the 64 chains, a tile of
-// leaves 5 k.
+// 308 -> 180 us, 25 sentences (H = 150) 80 -> 43, one sentence from and to host arrays 70 -> 52.  Before the first depth: 23 k cycles for
+// one sentence (trees and loads 8 k, lists 4.5 k, leaves 6 k, exchange 2 k), 30 k for the 25, 96 k for the 64 chains (41 k, 9 k, 39 k).
 //
 // Warp roles (1024 threads, as the scheduler's): warps 0-23 epilogue (warp w reads tensor-memory lane quadrant w mod 4), 24-30
 // filling warps, 31 MMA issuer and tensor-memory owner; all of them gather and finish leaves.
@@ -221,7 +221,10 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
     tt_sync(pt);
     const float share = (float)internal / (float)(parts * max(t.wide[kDepths], 1));   // of one cluster, for a node of the sample
     const float nodes = share * (float)t.wide[kDepths], depth = (float)t.wide[kDepths + 1];
-    const bool over = tid < kDepths - 1 && share * (float)t.wide[tid] > (float)R;   // (the last holds all that are deeper)
+    // (a cluster's nodes of a depth scatter by about their root around the mean, and the widest counts: 180 sentences, H = 156, with 60 of 64
+    // in the mean, were left only after the plan, 128 us; now at once. The last word holds all depths that are deeper.)
+    const float seen = tid < kDepths - 1 ? (float)t.wide[tid] : 0.f, mean = share * (seen + 0.5f * sqrtf(seen));   // (what is seen scatters, too)
+    const bool over = mean + sqrtf(mean) > (float)R;
     if (tt_any(over || 0.8f * tree_cost(p.costs, nodes, depth, (float)internal) > grid_cost(p.costs, depth, (float)internal), pt)) return;
   }
   // a node's word says whose child it is now: a child that two callers claim has one of them (no atomics: the bits of 32
