@@ -77,7 +77,7 @@ def trace_training_step() -> int:
              ("gates", "products", "barrier", "added", "complete"))):
         ph = t[LEVELS - 1]
         print(f"# {name}, first CTA of the first cluster, cycles since its start: " +
-              ", ".join(f"{what} {int(ph[k] - ph[0])}" for k, what in phases.items()))
+              ", ".join(f"{what} {int(ph[k] - ph[0])}" for k, what in phases.items() if ph[k] > ph[0]))
         print("depth " + " ".join(f"{c:<10s}" for c in columns) + " (cycles since the start of the depth's last nodes)")
         rows = [d for d in range(LEVELS - 1) if t[d, 0] > ph[0]]
         for d in rows if name == "k_trees_backward" else rows[::-1]:
