@@ -197,23 +197,29 @@ int read_levels(treelstm* ctx) {
 
 }  // namespace
 
-// What a control block that has just been read back says about the hand-over to the cluster kernel.
-void learn_tail_hint(treelstm* ctx) {
-  const DevStatus* hs = reinterpret_cast<const DevStatus*>(ctx->host_status);
-  const auto& L = ctx->last;
-  if (!ctx->tail_ok || ctx->precision != TREELSTM_BF16 || L.mode != TREELSTM_PERSISTENT || hs->status != 0 || hs->n_levels <= 0)
-    return;
-  ctx->tail_skip = hs->tail_from >= hs->n_levels;
+// What the stream of the last call, which the caller has waited for, left behind: the status, and a hint about the hand-over to
+// the cluster kernel.
+int settle(treelstm* ctx, int status, int hint) {
+  auto& L = ctx->last;
+  if (status != 0) L.valid = false;
+  else if (hint != kTailUnknown && ctx->tail_ok && ctx->precision == TREELSTM_BF16 && L.mode == TREELSTM_PERSISTENT) ctx->tail_skip = hint == kNoTail;
+  return status;
 }
 
 // Waits for the stream of the last call, whose control block is then in ctx->host_status, and says what it holds.
-int finish_status(treelstm* ctx, bool waited = false) {
-  auto& L = ctx->last;
-  if (!waited) TL_CUDA(ctx, cudaStreamSynchronize(L.stream));
-  const int st = reinterpret_cast<const DevStatus*>(ctx->host_status)->status;
-  if (st != 0) L.valid = false;
-  else learn_tail_hint(ctx);
-  return st;
+int finish_status(treelstm* ctx) {
+  TL_CUDA(ctx, cudaStreamSynchronize(ctx->last.stream));
+  const DevStatus* hs = reinterpret_cast<const DevStatus*>(ctx->host_status);
+  return settle(ctx, hs->status, tail_hint(hs->status, hs->n_levels, hs->tail_from));
+}
+
+// Pinned host memory of a context: a copy of the control block and, on a line of its own, the word that backward passes write.
+int make_host_status(treelstm* ctx) {
+  const size_t bytes = round_up_sz(sizeof(DevStatus), 256) + 256;
+  TL_CUDA(ctx, cudaMallocHost((void**)&ctx->host_status, bytes));
+  memset(ctx->host_status, 0, bytes);
+  ctx->bwd_status = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ctx->host_status) + bytes - 256);
+  return TREELSTM_OK;
 }
 
 // Whether a kernel may write to `bytes` bytes of host memory at `ptr` (pinned, at the same address on the device): the first
@@ -284,10 +290,8 @@ int treelstm_create(treelstm_t** out, int H, int E, int vocab, const float* emb,
       take(ctx->bp_x, 4 * groups * 24);
     }
     take(images, trees);
-    if (!pass && (cudaMalloc((void**)&ctx->memory, off) != cudaSuccess ||
-                  cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess))
+    if (!pass && (cudaMalloc((void**)&ctx->memory, off) != cudaSuccess || make_host_status(ctx) != TREELSTM_OK))
       return fail(TREELSTM_ERR_CUDA);
-    if (!pass) memset(ctx->host_status, 0, sizeof(DevStatus));
     if (pass && init_trees(ctx, images, s) != TREELSTM_OK) return fail(TREELSTM_ERR_CUDA);
   }
   int rc = init_schedule_attributes(ctx);
@@ -326,10 +330,8 @@ int treelstm_create_recursive(treelstm_t** out, int cell, int H, int vocab, cons
   auto fail = [&](int rc) { treelstm_destroy(ctx); return rc; };
   const size_t trees = plan_trees(ctx), emb_bytes = round_up_sz(sizeof(float) * V_ * Hs, 256),
                w_bytes = round_up_sz(sizeof(float) * (KQ + K2) * Hs, 256), b_bytes = round_up_sz(sizeof(float) * Hs, 256);
-  if (cudaMalloc((void**)&ctx->memory, emb_bytes + w_bytes + b_bytes + trees) != cudaSuccess ||
-      cudaMallocHost((void**)&ctx->host_status, sizeof(DevStatus)) != cudaSuccess)
+  if (cudaMalloc((void**)&ctx->memory, emb_bytes + w_bytes + b_bytes + trees) != cudaSuccess || make_host_status(ctx) != TREELSTM_OK)
     return fail(TREELSTM_ERR_CUDA);
-  memset(ctx->host_status, 0, sizeof(DevStatus));
   ctx->emb = reinterpret_cast<float*>(ctx->memory);
   ctx->Wcat = reinterpret_cast<float*>(ctx->memory + emb_bytes);
   ctx->b = reinterpret_cast<float*>(ctx->memory + emb_bytes + w_bytes);
@@ -516,8 +518,9 @@ int treelstm_status_sync(treelstm_t* ctx) {
   char* base = static_cast<char*>(L.ws);
   if (ctx->status_expected != 0 && ctx->status_stream == L.stream) {   // the last kernel of the backward pass writes it
     TL_CUDA(ctx, cudaStreamSynchronize(L.stream));
-    const volatile DevStatus* hs = reinterpret_cast<const volatile DevStatus*>(ctx->host_status);
-    if (hs->seq == ctx->status_expected) return finish_status(ctx, true);
+    const unsigned long long word = *const_cast<const volatile unsigned long long*>(ctx->bwd_status);
+    if ((int)(word >> 32) == ctx->status_expected) return settle(ctx, -(int)(word & 0xFFFFu), (int)(word >> 16 & 0xFFFFu));
+    // (a backward pass on another stream has written it since: the control block itself says it)
   }
   TL_CUDA(ctx, cudaMemcpyAsync(ctx->host_status, base + L.lay.status, sizeof(DevStatus),
                                cudaMemcpyDeviceToHost, L.stream));

@@ -25,8 +25,7 @@ struct DevStatus {
   int trees_fwd, trees_bwd;   // 1: the tree kernels (trees_fp32.cu, trees_tc.cu) took this forest forward / backward
   unsigned int tickets;       // CTAs that are done (publish_status)
   int trees_left;             // 1: the leaves' kernel (trees_fp32.cu) has said that the tree kernel behind it leaves this forest
-  int pad[50];
-  int seq;                    // in the host's copy: the launch that wrote it
+  int pad[51];
 };
 static_assert(sizeof(DevStatus) == 256, "control block is one 256-byte line group");
 
@@ -196,8 +195,9 @@ struct treelstm {
   } last;
   int32_t* host_level_offset = nullptr;  // pinned, grows on demand
   int host_level_cap = 0;
-  int* host_status = nullptr;            // pinned copy of DevStatus
-  int status_seq = 0, status_expected = 0;   // launches that write that copy; the one whose copy is to come (0: none)
+  int* host_status = nullptr;            // pinned copy of DevStatus: written on the stream of a call that then waits for it, never later
+  unsigned long long* bwd_status = nullptr;   // pinned, behind it: what the last kernel of a backward pass says, whenever that ends (StatusOut)
+  int status_seq = 0, status_expected = 0;   // launches that write that word; the one whose word is to come (0: none)
   cudaStream_t status_stream = nullptr;
   bool bwd_counters_clear = false;       // the backward's arrival counters, in stream order: by the forward, and by the kernel that publishes the status
 
@@ -298,7 +298,7 @@ int launch_schedule_trees_tc(treelstm* ctx, int n, const int32_t* left, const in
 
 int launch_selftest_waits(treelstm* ctx, void* ws, int* result_dev, cudaStream_t stream);
 
-// For the last launch of a backward pass: where its copy of the control block goes.
+// For the last launch of a backward pass: the number that its status word will have.
 inline int expect_status(treelstm* ctx, cudaStream_t stream) {
   ctx->status_seq = ctx->status_seq == 0x7FFFFFFF ? 1 : ctx->status_seq + 1;
   ctx->status_expected = ctx->status_seq;
@@ -357,28 +357,34 @@ int launch_gather_roots(treelstm* ctx, int max_roots, int32_t* root_ids, float* 
     }                                                       \
   } while (0)
 
+// The word that a backward pass leaves on the host: launch number | what the forward's kernel said about a tail (tail_hint) | -status.
+enum TailHint { kTailUnknown = 0, kTailWorthIt = 1, kNoTail = 2 };
+__host__ __device__ inline int tail_hint(int status, int n_levels, int tail_from) {
+  return status != 0 || n_levels <= 0 ? kTailUnknown : (tail_from >= n_levels ? kNoTail : kTailWorthIt);
+}
+__host__ __device__ inline unsigned long long status_word(int seq, int status, int n_levels, int tail_from) {
+  return (unsigned long long)(unsigned)seq << 32 | (unsigned long long)tail_hint(status, n_levels, tail_from) << 16 | (unsigned)(-status & 0xFFFF);
+}
+
 #ifdef __CUDACC__
 // Record an error in the control block; the most negative code wins.
 __device__ __forceinline__ void report(DevStatus* st, int code) { atomicMin(&st->status, code); }
 
 __device__ __forceinline__ int ld_volatile(const int* p) { return *(const volatile int*)p; }
 
-// The last kernel of a backward pass leaves the control block in pinned host memory itself: a copy behind it would be 3 us of
-// a step that ends with the host waiting for it.  Every CTA's threads call this last; whichever CTA is the last writes.
-struct StatusOut { int* host; int seq; };
+// The last kernel of a backward pass leaves its status in pinned host memory itself: a copy of the control block behind it would
+// be 3 us of a step that ends with the host waiting for it.  Every CTA's threads call this last; whichever CTA is the last writes.
+// The word is written whenever that kernel ends, beside calls on other streams that wait for their own answers, so
+// nothing else is read from it or written to it, and it is one store: launch number and status cannot be of two launches.
+struct StatusOut { unsigned long long* host; int seq; };
 __device__ __forceinline__ void publish_status(DevStatus* st, const StatusOut& out) {
-  __shared__ int s_last;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = atomicAdd(&st->tickets, 1u) == gridDim.x * gridDim.y * gridDim.z - 1u;
-  }
-  __syncthreads();
-  constexpr int kWords = (int)(sizeof(DevStatus) / sizeof(int));
-  if (!s_last || threadIdx.x >= 32) return;
+  if (threadIdx.x != 0) return;
   __threadfence();
-  for (int k = threadIdx.x; k < kWords; k += 32) out.host[k] = k == kWords - 1 ? out.seq : reinterpret_cast<volatile int*>(st)[k];
-  if (threadIdx.x == 0) st->tickets = st->barrier_bwd = st->barrier_levels = 0u;   // (a backward pass may be repeated)
+  if (atomicAdd(&st->tickets, 1u) != gridDim.x * gridDim.y * gridDim.z - 1u) return;
+  __threadfence();
+  *(volatile unsigned long long*)out.host = status_word(out.seq, ld_volatile(&st->status), ld_volatile(&st->n_levels), ld_volatile(&st->tail_from));
+  st->tickets = st->barrier_bwd = st->barrier_levels = 0u;   // (a backward pass may be repeated)
 }
 
 // Checked build (-DTREELSTM_CHECKED; compute-sanitizer's stand-in where that tool is not available):

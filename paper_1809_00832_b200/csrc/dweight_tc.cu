@@ -506,7 +506,7 @@ int launch_dweight_tc(treelstm* ctx, int n, const int32_t* order, const int32_t*
   p.tok_slot = tok_slot; p.dEmb_rows = dEmb_rows;
   p.wait_limit = ctx->opt.wait_limit_kcycles * 1024;
   if (n == 0) return TREELSTM_OK;
-  p.out = {ctx->host_status, expect_status(ctx, stream)};
+  p.out = {ctx->bwd_status, expect_status(ctx, stream)};
   // The host does not know how the nodes divide into leaves and internal nodes (the level table stayed on the
   // device), so the kernel sizes its work items itself from the grid it finds: one CTA per SM unless even
   // single-block items are fewer (counted for the division that gives the most).

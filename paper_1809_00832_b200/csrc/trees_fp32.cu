@@ -1315,7 +1315,7 @@ int launch_rec_grads(treelstm* ctx, float* dW, float* db, float* dV, float* dEmb
   if (g.splits > most) g.splits = most;
   if (g.splits < 1) g.splits = 1;
   const int leaf_ctas = L.n / 16 < 64 ? L.n / 16 + 1 : 64;
-  g.out = {ctx->host_status, expect_status(ctx, stream)};
+  g.out = {ctx->bwd_status, expect_status(ctx, stream)};
   cudaLaunchConfig_t cfg = {};                            // (the programmatic dependent of whatever is ahead: it comes up while that ends)
   cfg.gridDim = dim3(g.tiles * g.splits + leaf_ctas); cfg.blockDim = dim3(kGT); cfg.stream = stream;
   cudaLaunchAttribute at;

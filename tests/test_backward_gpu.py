@@ -334,3 +334,103 @@ def test_weights_of_the_backward_come_with_the_classifier_and_follow_every_updat
         n = int(res["n_touched"][0])
         assert util.max_abs(res["dEmb_rows"][:n], ref["dEmb_rows"]) <= util.REL[precision] * float(np.abs(ref["dEmb_rows"]).max())
     model.close()
+
+
+class _RawStep:
+    """forward that keeps its activations and backward as a C caller enqueues them, with a workspace of their own, on the current
+    stream; nothing waits for the device"""
+
+    def __init__(self, model, forest, labels):
+        f32, i32 = dict(dtype=torch.float32, device="cuda"), dict(dtype=torch.int32, device="cuda")
+        n, H, E, C = forest.n_nodes, model.H, model.E, model.C
+        self.model, self.n = model, n
+        self.forest = [util.to_dev(a) for a in (forest.left, forest.right, forest.token)]
+        self.labels = util.to_dev(labels)
+        self.states = [torch.empty((n, H), **f32), torch.empty((n, H), **f32), torch.empty(n, **i32), torch.empty(n, **i32),
+                       torch.empty(n + 2, **i32), torch.empty(1, **i32)]
+        self.grads = dict(loss=torch.empty(1, **f32), dW=torch.empty((E + 2 * H, 5 * H), **f32), db=torch.empty(5 * H, **f32),
+                          dWc=torch.empty((H, C), **f32), dbc=torch.empty(C, **f32), touched_ids=torch.empty(forest.n_leaves, **i32),
+                          dEmb_rows=torch.empty((forest.n_leaves, E), **f32), n_touched=torch.empty(1, **i32))
+        need = model.workspace_bytes(n, True)
+        self.ws = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+        self.at, self.ws_bytes = self.ws.data_ptr() + (-self.ws.data_ptr()) % 256, need
+
+    def forward(self):
+        rc = self.model.lib.treelstm_forward(self.model.handle, self.n, *(t.data_ptr() for t in self.forest + self.states),
+                                             binding.PERSISTENT | binding.SAVE_FOR_BACKWARD, self.at, self.ws_bytes,
+                                             torch.cuda.current_stream().cuda_stream)
+        assert rc == binding.OK
+
+    def backward(self):
+        rc = self.model.lib.treelstm_backward(self.model.handle, self.labels.data_ptr(), *(t.data_ptr() for t in self.grads.values()),
+                                              torch.cuda.current_stream().cuda_stream)
+        assert rc == binding.OK
+
+
+@pytest.mark.parametrize("call", ["forward_host", "per_level"])
+def test_backward_that_ends_beside_another_call_leaves_its_answer_alone(call):
+    """a backward pass (one whose labels are bad) is left on its stream while a call on another stream waits for its own level and
+    root counts and status; the backward ends before, within and behind that call"""
+    rng = np.random.default_rng(1400)
+    params = fg.draw_params(rng, 20, 12, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.3, n_classes=3)
+    model = util.make_model(params, "fp32")
+    model.set_option(binding.OPT_MAX_CTAS, 16)                   # the kernels of both streams fit the device together
+    one = fg.forest_from_shapes([fg.left_chain_shape(30), None], rng, 60)
+    other = fg.forest_from_shapes([fg.balanced_shape(4)] * 5, rng, 60)
+    labels = rng.integers(0, 3, size=one.n_nodes).astype(np.int32)
+    labels[3] = 3
+    step = _RawStep(model, one, labels)
+    host = binding.pack_forest_host(other.left, other.right, other.token)
+    dev = [util.to_dev(a) for a in (other.left, other.right, other.token)]
+    want = {k: v.cpu().numpy() for k, v in model.forward(*dev, flags=binding.PER_LEVEL).items()}
+    roots = model.forward_host(*host, max_roots=8)["root_h"].numpy().copy()
+    out, levels = model.forward_host(*host, max_roots=8), model.forward(*dev, flags=binding.PER_LEVEL)
+    behind, beside = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for wait in range(0, 400):
+        with torch.cuda.stream(behind):
+            step.forward()
+            torch.cuda._sleep(500 * wait)                        # cycles: up to 100 us
+            step.backward()
+        with torch.cuda.stream(beside):
+            if call == "forward_host":
+                model.forward_host(*host, max_roots=8, out=out)
+                assert int(out["n_levels"]) == 3 and int(out["n_roots"]) == 5
+                np.testing.assert_array_equal(out["root_h"].numpy()[:5], roots[:5])
+            else:
+                model.forward(*dev, flags=binding.PER_LEVEL, out=levels)   # one launch a level, as many as the host has read
+                np.testing.assert_array_equal(levels["h"].cpu().numpy(), want["h"])
+        behind.synchronize()
+
+
+def test_status_of_the_last_backward_when_one_on_another_stream_ends_later():
+    """two backward passes on two streams with a workspace each: treelstm_status_sync speaks of the last call, whichever of them
+    is the last to end"""
+    rng = np.random.default_rng(1401)
+    params = fg.draw_params(rng, 20, 12, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.3, n_classes=3)
+    model = util.make_model(params, "fp32")
+    model.set_option(binding.OPT_MAX_CTAS, 16)
+    forest = fg.forest_from_shapes([fg.left_chain_shape(30), fg.balanced_shape(4)], rng, 60)
+    good = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    bad = good.copy()
+    bad[5] = 3
+    steps = {binding.OK: _RawStep(model, forest, good), binding.ERR_LABEL_OUT_OF_RANGE: _RawStep(model, forest, bad)}
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for last, first in ((binding.OK, binding.ERR_LABEL_OUT_OF_RANGE), (binding.ERR_LABEL_OUT_OF_RANGE, binding.OK)):
+        for first_ends_later in (False, True):
+            torch.cuda.synchronize()
+            with torch.cuda.stream(streams[0]):
+                steps[first].forward()
+                torch.cuda._sleep(20_000_000 if first_ends_later else 1)      # 10 ms
+                steps[first].backward()
+            if not first_ends_later:
+                streams[0].synchronize()
+            with torch.cuda.stream(streams[1]):
+                steps[last].forward()
+                steps[last].backward()
+            assert model.status_sync() == last
+            torch.cuda.synchronize()
+            assert model.status_sync() == last                   # the other one's word lies there now
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, good)
+    _compare({k: v.cpu().numpy() for k, v in steps[binding.OK].grads.items()}, ref, util.TOL["fp32"])
