@@ -127,7 +127,9 @@ typedef enum treelstm_status {
                                             /* library checks) and on the stream having the device to      */
                                             /* itself; otherwise the bounded grid barrier ends the call    */
                                             /* with TREELSTM_ERR_TIMEOUT.  0: cooperative launch in plain  */
-                                            /* stream order (residency guaranteed by the runtime)          */
+                                            /* stream order (residency guaranteed by the runtime).  Of a   */
+                                            /* backward pass the kernels with a grid barrier are always    */
+                                            /* cooperative: it may share the device                        */
 #define TREELSTM_OPT_LEAVES_FIRST_MIN_NODES 9 /* accepted and without effect: an order of work that took   */
                                             /* the leaves before the schedule was the slower one at every  */
                                             /* size once forests from 4096 nodes on are scheduled by a     */

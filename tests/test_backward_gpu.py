@@ -434,3 +434,55 @@ def test_status_of_the_last_backward_when_one_on_another_stream_ends_later():
     ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
                                  params.bc, good)
     _compare({k: v.cpu().numpy() for k, v in steps[binding.OK].grads.items()}, ref, util.TOL["fp32"])
+
+
+REPEATED = {
+    "tree clusters": (150, lambda rng: [fg.random_split_shape(rng, int(n)) for n in rng.integers(2, 40, size=20)]),
+    "wide wavefronts": (40, lambda rng: [fg.balanced_shape(512)] * 2 + [None] * 3),
+    "beyond the tree kernels": (300, lambda rng: [fg.balanced_shape(64)] * 2),
+}
+
+
+@pytest.mark.parametrize("overlap", [0, 1])
+@pytest.mark.parametrize("kind", REPEATED)
+def test_a_backward_pass_may_be_repeated(kind, overlap):
+    """two backward passes behind one forward, on every way through the forest and with either launch form of the forward: the second
+    finds the counters of its grid barriers as the first one did"""
+    H, shapes = REPEATED[kind]
+    rng = np.random.default_rng(1500 + H)
+    params = fg.draw_params(rng, H, 30, 70, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes(rng), rng, 70), rng)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    model.set_option(binding.OPT_OVERLAP_LAUNCH, overlap)
+    arrs = [util.to_dev(a) for a in (forest.left, forest.right, forest.token, labels)]
+    model.forward(*arrs[:3], flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+    for _ in range(2):
+        _compare({k: v.cpu().numpy() for k, v in model.backward(arrs[3], forest.n_leaves).items()}, ref, util.TOL["fp32"])
+
+
+def test_backward_passes_side_by_side_share_the_device():
+    """two contexts' backward passes of wide forests, each with a grid barrier over the whole device, enqueued on two streams at once"""
+    rng = np.random.default_rng(1600)
+    params = fg.draw_params(rng, 40, 30, 70, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(40), n_classes=3)
+    forest = fg.forest_from_shapes([fg.balanced_shape(512)] * 4, rng, 70)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    models = [util.make_model(params, "fp32") for _ in range(2)]
+    steps = [_RawStep(m, forest, labels) for m in models]
+    streams = [torch.cuda.Stream() for _ in models]
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for step in steps:                                        # (one after the other: a forward has the device to itself)
+            step.forward()
+            torch.cuda.synchronize()
+        for step, stream in zip(steps, streams):
+            with torch.cuda.stream(stream):
+                torch.cuda._sleep(100_000)                        # both are enqueued by the time either starts
+                step.backward()
+        assert [m.status_sync() for m in models] == [binding.OK] * 2
+    for step in steps:
+        _compare({k: v.cpu().numpy() for k, v in step.grads.items()}, ref, util.TOL["fp32"])

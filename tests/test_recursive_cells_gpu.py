@@ -273,3 +273,25 @@ def test_label_out_of_range_reaches_no_gradient(cell, n_trees, hi):
     model.forward(*arrs, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
     assert np.isfinite(model.backward_recursive(util.to_dev(labels), leaves)["loss"].item())
     model.close()
+
+
+@pytest.mark.parametrize("overlap", [0, 1])
+@pytest.mark.parametrize("kind", ["sentences", "one large tree"])
+def test_a_backward_pass_may_be_repeated(kind, overlap):
+    """two backward passes behind one forward, on tree clusters and over the whole GPU"""
+    rng = np.random.default_rng(960)
+    p = fg.draw_recursive_params(rng, 20, 90, tensor=False, emb_scale=0.8, w_scale=0.2)
+    shapes = [fg.random_split_shape(rng, 20) for _ in range(8)] if kind == "sentences" else [fg.balanced_shape(1024)] * 2
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes, rng, 90), rng)
+    Wc, bc = rng.uniform(-0.3, 0.3, size=(20, 3)).astype(np.float32), rng.uniform(-0.1, 0.1, size=3).astype(np.float32)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = rc.loss_and_gradients(KIND[binding.CELL_TREERNN], forest.left, forest.right, forest.token, p.emb, p.W, p.b, Wc, bc, labels, p.V)
+    model = _model(binding.CELL_TREERNN, p)
+    model.set_option(binding.OPT_OVERLAP_LAUNCH, overlap)
+    model.set_classifier(util.to_dev(Wc), util.to_dev(bc))
+    arrs = [util.to_dev(a) for a in (forest.left, forest.right, forest.token, labels)]
+    model.forward(*arrs[:3], flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+    for _ in range(2):
+        g = {k: v.cpu().numpy() for k, v in model.backward_recursive(arrs[3], forest.n_leaves).items()}
+        util.compare_training_step(g, ref, util.TOL["fp32"], util.REL["fp32"], loss_rel=1e-5)
+    model.close()
