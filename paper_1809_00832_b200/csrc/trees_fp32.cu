@@ -166,7 +166,10 @@ __host__ __device__ inline int bwd_buf_words(int cell, int H, const TreesShape& 
 }
 
 // ---- forward -------------------------------------------------------------------------------------- //
-template <int CELL, int U, int RC>
+// SAVE: a backward pass follows (trees of all cells dealt by size, the cluster's lists kept for it).  An instantiation of its own,
+// because what runs once costs as code, run or not: with one for both, TreeRNN H = 128, forward alone, 10 sentences of 2 to 20
+// words took 26.7 us and not 24.7, 100 of 2 to 12 words 28.7 and not 26.7; RNTN H = 32, the same 10, 34.2 and not 32.9.
+template <int CELL, int U, int RC, bool SAVE>
 __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constant__ TreesParams p) {
   extern __shared__ __align__(16) float sm[];
   __shared__ Walk s_walk;
@@ -195,13 +198,13 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     if (tid == 0) s_walk = Walk{0, 0, 0};
     __syncthreads();
   } else {
-    deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || p.walks.at != nullptr, &s_loads, &s_walk, trace);
+    deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || SAVE, &s_loads, &s_walk, trace);
   }
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
   const Walk walk = s_walk;
-  if (p.walks.at && rank == 0) save_walk(p.walks, s, sm, part, parts, walk);
+  if (SAVE && rank == 0) save_walk(p.walks, s, sm, part, parts, walk);
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
   const unsigned short* start = reinterpret_cast<const unsigned short*>(sm + s.start);
@@ -1063,9 +1066,11 @@ bool shape_fits(int cell, int H, int cs, TreesShape& s) {
 }
 
 using TreesKernel = void (*)(const TreesParams);
-TreesKernel forward_kernel(int cell) {
-  return cell == kRntn ? k_trees_forward<kRntn, 4, kRntnRC> : (cell == kRnn ? k_trees_forward<kRnn, 4, kRnnRC> : k_trees_forward<kLstm, 5, kLstmRC>);
+template <bool SAVE>
+TreesKernel forward_kernel_of(int cell) {
+  return cell == kRntn ? k_trees_forward<kRntn, 4, kRntnRC, SAVE> : (cell == kRnn ? k_trees_forward<kRnn, 4, kRnnRC, SAVE> : k_trees_forward<kLstm, 5, kLstmRC, SAVE>);
 }
+TreesKernel forward_kernel(int cell, bool save) { return save ? forward_kernel_of<true>(cell) : forward_kernel_of<false>(cell); }
 TreesKernel backward_kernel(int cell, const TreesShape& s) {
   if (cell == kRntn) return k_trees_backward<kRntn, 8, 1, kRntnT>;
   if (cell == kRnn) return s.bseg == 8 ? k_trees_backward<kRnn, 8, 4, kBwdT> : k_trees_backward<kRnn, 4, 4, 512>;
@@ -1177,8 +1182,9 @@ size_t plan_trees(treelstm* ctx) {
   // 58.6 / 142, 60.6 / 133, 56.0 / 124, 67.2 / 122 us)
   for (int cs = cell == kRnn && H >= 64 ? 4 : 1; cs <= 16 && !t.ok; cs *= 2) t.ok = shape_fits(cell, H, cs, s);
   const bool forward = ctx->precision == TREELSTM_FP32;     // (the bf16 forward has kernels of its own)
-  for (int back = forward ? 0 : 1; back < 2 && t.ok; ++back) {
-    TreesKernel k = back ? backward_kernel(cell, s) : forward_kernel(cell);
+  for (int kind = forward ? 0 : 2; kind < 3 && t.ok; ++kind) {   // forward, the same with lists kept for the backward, backward
+    const bool back = kind == 2;
+    TreesKernel k = back ? backward_kernel(cell, s) : forward_kernel(cell, kind == 1);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
@@ -1189,7 +1195,8 @@ size_t plan_trees(treelstm* ctx) {
     t.ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) == cudaSuccess &&
            (s.cs <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
            cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) == cudaSuccess && clusters >= 1;
-    (back ? t.clusters_bwd : t.clusters) = clusters;
+    if (back) t.clusters_bwd = clusters;
+    else t.clusters = kind == 0 ? clusters : std::min(t.clusters, clusters);
   }
   if (!t.ok) { cudaGetLastError(); return 0; }
   if (forward && cell == kLstm && cudaFuncSetAttribute(k_leaves_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem) != cudaSuccess) {
@@ -1281,7 +1288,7 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
     TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_leaves_fp32, q));
     ctx->launches += 1;
   }
-  return launch_trees(ctx, forward_kernel(ctx->cell), p, kFwdT, parts, after_running, stream);
+  return launch_trees(ctx, forward_kernel(ctx->cell, save), p, kFwdT, parts, after_running, stream);
 }
 
 int launch_backward_trees(treelstm* ctx, cudaStream_t stream) {

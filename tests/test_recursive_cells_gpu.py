@@ -295,3 +295,22 @@ def test_a_backward_pass_may_be_repeated(kind, overlap):
         g = {k: v.cpu().numpy() for k, v in model.backward_recursive(arrs[3], forest.n_leaves).items()}
         util.compare_training_step(g, ref, util.TOL["fp32"], util.REL["fp32"], loss_rel=1e-5)
     model.close()
+
+
+@pytest.mark.parametrize("cell,H", [(binding.CELL_TREERNN, 128), (binding.CELL_TREERNN, 20), (binding.CELL_RNTN, 32)])
+@pytest.mark.parametrize("kind", ["one leaf", "few trees", "more trees than clusters", "left to the whole GPU"])
+def test_states_are_the_same_with_and_without_a_backward_to_come(kind, cell, H):
+    """two instantiations of the tree kernel: trees dealt by id, or by size with the lists kept; whose cluster a tree is changes no
+    bit of its nodes' states (where both leave the forest to the whole GPU: neither)"""
+    rng = np.random.default_rng(970 + H)
+    p = fg.draw_recursive_params(rng, H, 90, tensor=cell == binding.CELL_RNTN, emb_scale=0.8, w_scale=1.0 / np.sqrt(2 * H), v_scale=1.0 / (2 * H))
+    shapes = {"one leaf": [None], "few trees": [fg.random_split_shape(rng, int(n)) for n in rng.integers(2, 30, size=9)],
+              "more trees than clusters": [None if t % 9 == 4 else fg.random_split_shape(rng, int(rng.integers(2, 6))) for t in range(160)],
+              "left to the whole GPU": [fg.balanced_shape(1024 if H > 32 else 256)] * 2}[kind]
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes, rng, 90), rng)
+    model = _model(cell, p)
+    arrs = [util.to_dev(a) for a in (forest.left, forest.right, forest.token)]
+    alone = model.forward(*arrs, flags=binding.PERSISTENT)["h"].cpu().numpy()
+    saved = model.forward(*arrs, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)["h"].cpu().numpy()
+    np.testing.assert_array_equal(alone, saved)
+    model.close()
