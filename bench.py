@@ -61,11 +61,15 @@ def algorithmic_work(forest: fg.Forest, H: int, E: int, weight_bytes_per_elem: i
     return flops, bytes_
 
 
-def roofline_block(forest, p, precision: str, kernel_ms: float, step_ms: float, peaks, workload: str):
+def roofline_block(forest, p, precision: str, kernel_ms, step_ms: float, peaks, workload: str):
     """Achieved fraction of the slower of the two ceilings: algorithmic bytes at the measured HBM copy
     bandwidth, gate flops at the measured tensor peak (bf16 path; the fp32 path runs on the FP32
     pipes and is reported against HBM only).  `frac` uses the wavefront kernel's own duration,
-    `frac_of_step` the whole forward call (scheduler included)."""
+    `frac_of_step` the whole forward call (scheduler included).  Without a kernel time (clusters evaluate the
+    forest in the scheduler's launch) both are those of the whole call."""
+    alone = kernel_ms is not None
+    if not alone:
+        kernel_ms = step_ms
     flops, abytes = algorithmic_work(forest, p.H, p.E, 2 if precision == "bf16" else 4)
     t_hbm = abytes / (peaks["hbm_gbs"] * 1e9)
     t_tensor = flops / (peaks["bf16_tflops_sustained"] * 1e12) if precision == "bf16" else 0.0
@@ -79,11 +83,13 @@ def roofline_block(forest, p, precision: str, kernel_ms: float, step_ms: float, 
         head = {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"]}
     head.update({
         "traffic": traffic, "traffic_source": source, "peak_source": peaks["source"],
-        "kernel": "k_fwd_tc (persistent wavefront kernel)" if precision == "bf16" else "k_leaves_fp32 and k_trees_forward (or k_fwd_fp32_persistent)",
+        "kernel": "k_leaves_fp32 and k_trees_forward (or k_fwd_fp32_persistent)" if precision != "bf16" else
+                  ("k_fwd_tc (persistent wavefront kernel)" if alone else "k_schedule_trees_tc (whole trees on clusters, in the scheduler's launch)"),
         "kernel_timing": "the kernel of the timed steps run alone, between the library's event pair (the event keeps it "
-                         "from starting under the scheduler as it does in the steps)",
+                         "from starting under the scheduler as it does in the steps)" if alone else
+                         "whole calls: no kernel behind the scheduler evaluates this forest",
         "kernel_ms_plain_order": TIMINGS.get("kernel_ms_plain_order"),
-        "kernel_ms": kernel_ms, "algorithmic_bytes": abytes, "algorithmic_flops": flops,
+        "kernel_ms": kernel_ms if alone else None, "algorithmic_bytes": abytes, "algorithmic_flops": flops,
         "frac_of_step": head["frac"] * kernel_ms / step_ms,
         "hbm_gbs": gbs, "hbm_frac": gbs / peaks["hbm_gbs"],
         "tensor_tflops": tfl, "tensor_frac_of_sustained": tfl / peaks["bf16_tflops_sustained"],
@@ -235,13 +241,23 @@ def _dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-def time_forward(model, forest, flags, steps, warmup, flush, kernel_every=16, overlap_launch=None):
+def clusters_took(model) -> bool:
+    """Whether the last forward's forest was evaluated by clusters in the scheduler's launch (a word of the control block, which
+    lies at the first 256-byte boundary of the handle's workspace)."""
+    import torch
+    from paper_1809_00832_b200 import binding
+    at = (-model._ws.data_ptr()) % 256 + 4 * 9
+    return model.precision == binding.BF16 and bool(model._ws[at:at + 4].clone().view(torch.int32).item())
+
+
+def time_forward(model, forest, flags, steps, warmup, flush, kernel_every=16, overlap_launch=None, always_kernel=False):
     """`steps` forward calls on a device-resident forest, L2 flushed before each (untimed), CUDA events
     on the launching stream around every call.  The wavefront kernel's own device time is taken in a
     second pass (same flushing, read on every kernel_every-th call): the library's event pair around
     that kernel sits between the scheduler and the wavefront kernel on the stream and keeps the
-    latter from starting under the former, so it stays out of the timed steps.
-    Returns (per-step ms list, mean kernel ms, launches, outputs)."""
+    latter from starting under the former, so it stays out of the timed steps.  With the pair the library gives every
+    bf16 forest to that kernel, so a forest that clusters take in the steps has no kernel time of its own.
+    Returns (per-step ms list, mean kernel ms or None, launches, outputs)."""
     import torch
     from paper_1809_00832_b200 import binding
     left, right, token = _dev(forest.left), _dev(forest.right), _dev(forest.token)
@@ -263,6 +279,10 @@ def time_forward(model, forest, flags, steps, warmup, flush, kernel_every=16, ov
     status = model.status_sync()
     if status != 0:
         raise RuntimeError(f"device status {status} after the timed region")
+    step_ms = [a.elapsed_time(b) for a, b in ev]
+    TIMINGS["kernel_ms_plain_order"] = None
+    if clusters_took(model) and not always_kernel:
+        return step_ms, None, launches, out
     model.set_option(binding.OPT_TIME_WAVEFRONT_KERNEL, 1)
 
     def kernel_pass():
@@ -277,14 +297,13 @@ def time_forward(model, forest, flags, steps, warmup, flush, kernel_every=16, ov
     # the kernel of the timed steps, alone: the event in front of it makes it start when the scheduler has
     # ended, its code and order of work stay those of the steps
     k_ms = kernel_pass()
-    TIMINGS["kernel_ms_plain_order"] = None
     if overlap_launch is None or overlap_launch:
         # for the record: the form the library uses in plain stream order (cooperative launch)
         model.set_option(binding.OPT_OVERLAP_LAUNCH, 0)
         TIMINGS["kernel_ms_plain_order"] = kernel_pass()
     model.set_option(binding.OPT_TIME_WAVEFRONT_KERNEL, 0)
     model.set_option(binding.OPT_OVERLAP_LAUNCH, 1 if overlap_launch is None else overlap_launch)
-    return [a.elapsed_time(b) for a, b in ev], k_ms, launches, out
+    return step_ms, k_ms, launches, out
 
 
 def extra_forward(name, n_trees, peaks, flush, steps=200, warmup=5):
@@ -309,20 +328,21 @@ def extra_forward(name, n_trees, peaks, flush, steps=200, warmup=5):
 
 def wavefront_latency_floor(peaks, flush, levels_of_headline, steps=100, warmup=5):
     """Third, non-judged line: what the dependency depth alone costs.  A single left chain of 64
-    leaves has 64 wavefronts of one or two nodes each: its kernel time / 64 is the latency of an
-    (almost) empty wavefront; times the headline workload's level count = the floor no amount of
-    bandwidth or tensor throughput removes."""
+    leaves has 64 wavefronts of one or two nodes each: the time of the wavefront kernels on it / 64 is the latency of
+    an (almost) empty wavefront (in a call without the event pair the library gives this chain to clusters in the
+    scheduler's launch); times the headline workload's level count = the floor no amount of bandwidth or tensor
+    throughput removes."""
     import torch
     from paper_1809_00832_b200 import binding
     rng = np.random.default_rng(0)
     p = fg.draw_params(rng, 256, 300, 20000, emb_dist="normal", emb_scale=0.1, w_scale=0.05)
     forest = fg.forest_from_shapes([fg.left_chain_shape(64)], rng, p.vocab)
     model = binding.TreeLSTM(p.H, p.E, p.vocab, _dev(p.emb), _dev(p.W), _dev(p.b), binding.BF16)
-    step_ms, k_ms, _, out = time_forward(model, forest, binding.PERSISTENT, steps, warmup, flush, kernel_every=4)
+    step_ms, k_ms, _, out = time_forward(model, forest, binding.PERSISTENT, steps, warmup, flush, kernel_every=4, always_kernel=True)
     levels = int(out["n_levels"].item())
     per = k_ms / levels
     model.close()
-    return {"probe": "one left chain of 64 leaves, H=256, E=300, bf16", "probe_levels": levels, "probe_kernel_ms": k_ms,
+    return {"probe": "one left chain of 64 leaves, H=256, E=300, bf16", "probe_levels": levels, "probe_kernel": "k_fwd_tc, one cluster for narrow wavefronts (k_fwd_tc_tail)", "probe_kernel_ms": k_ms,
             "ms_per_empty_wavefront": per, "levels": levels_of_headline, "floor_ms": per * levels_of_headline}
 
 
