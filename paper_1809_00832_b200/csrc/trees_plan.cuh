@@ -1,5 +1,5 @@
 // Which trees a cluster takes and in which order it walks them: the pieces that every kernel whose clusters evaluate whole
-// trees shares (trees_fp32.cu).
+// trees shares (trees_fp32.cu; trees_tc.cu has a plan of its own and takes the tables, the ranking and the choice from here).
 //
 // A cluster needs the internal nodes of its trees by depth, deepest last, and for every node the row of its caller.  All
 // CTAs of all clusters work that out for themselves from the child arrays - no launch ahead, no exchange -, each the same
@@ -207,6 +207,20 @@ __device__ __forceinline__ void count_roots(const TreeLinks& t, const unsigned* 
     sum += __shfl_sync(kFull, incl, 31);
   }
 }
+// The cluster of tree `q` when trees are dealt by size there and back (equal ones in the order of their ids; the sizes, a multiple of
+// four of them, are zero behind the last tree).
+__device__ __forceinline__ int dealt_to(const int* size, int slots, int q, int parts) {
+  const int mine = size[q];
+  int rank = 0;
+#pragma unroll 1
+  for (int s0 = 0; s0 < slots; s0 += 4) {
+    const int4 v = *reinterpret_cast<const int4*>(size + s0);
+    rank += (v.x > mine || (v.x == mine && s0 < q)) + (v.y > mine || (v.y == mine && s0 + 1 < q)) +
+            (v.z > mine || (v.z == mine && s0 + 2 < q)) + (v.w > mine || (v.w == mine && s0 + 3 < q));
+  }
+  const int turn = rank / parts, in_turn = rank - turn * parts;
+  return turn & 1 ? parts - 1 - in_turn : in_turn;
+}
 // one warp: the outcome, from the clusters' loads (counts of a sample: `share` internal nodes for each)
 __device__ __forceinline__ bool clusters_win(const WalkCosts& costs, const TreeLoads& loads, int parts, float internal, float share, int lane) {
   float cost = 0.f;
@@ -276,15 +290,7 @@ __device__ __forceinline__ void deal_by_size(int n, const unsigned* kids, const 
     const int mine = t.size[q];
     int part = q;
     if (dealt) {
-      int rank = 0;
-#pragma unroll 1
-      for (int s0 = 0; s0 < slots; s0 += 4) {                // (zero behind the last tree)
-        const int4 v = *reinterpret_cast<const int4*>(t.size + s0);
-        rank += (v.x > mine || (v.x == mine && s0 < q)) + (v.y > mine || (v.y == mine && s0 + 1 < q)) +
-                (v.z > mine || (v.z == mine && s0 + 2 < q)) + (v.w > mine || (v.w == mine && s0 + 3 < q));
-      }
-      const int turn = rank / parts, in_turn = rank - turn * parts;
-      part = turn & 1 ? parts - 1 - in_turn : in_turn;
+      part = dealt_to(t.size, slots, q, parts);
       out->part[q] = (unsigned char)part;
     }
     if (choose && mine) {

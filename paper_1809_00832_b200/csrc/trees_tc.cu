@@ -327,19 +327,7 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
   const int slots = t.dealt ? t.trees : parts;
 #pragma unroll 1
   for (int q = tid; q < slots; q += pt) {
-    const int mine = t.size[q];
-    int to = q;
-    if (t.dealt) {
-      int at = 0;
-#pragma unroll 1
-      for (int s0 = 0; s0 < slots; s0 += 4) {              // (zero behind the last tree)
-        const int4 v = *reinterpret_cast<const int4*>(t.size + s0);
-        at += (v.x > mine || (v.x == mine && s0 < q)) + (v.y > mine || (v.y == mine && s0 + 1 < q)) +
-              (v.z > mine || (v.z == mine && s0 + 2 < q)) + (v.w > mine || (v.w == mine && s0 + 3 < q));
-      }
-      const int turn = at / parts, in_turn = at - turn * parts;
-      to = turn & 1 ? parts - 1 - in_turn : in_turn;
-    }
+    const int mine = t.size[q], to = t.dealt ? dealt_to(t.size, slots, q, parts) : q;
     loads->part[q] = (unsigned char)to;
     if (mine) atomicAdd(&loads->nodes[to], mine);
   }
