@@ -31,7 +31,9 @@ WsLayout ws_layout(const treelstm* ctx, int n, bool with_backward) {
     L.ain = take(2 * nn * 2 * (size_t)ctx->Hp);      // [h_l | h_r] of every position, bf16
     L.cin = take(4 * nn * 2 * (size_t)row_pitch(ctx->H));       // [c_l | c_r] of every position, fp32
   }
-  L.gates = L.dh = L.dc = L.dz = L.tok_slot = L.walks = off;
+  L.walks = off;
+  if (with_backward || ctx->cell == 0) L.walks = take(saved_walks_bytes(ctx, (int)nn));
+  L.gates = L.dh = L.dc = L.dz = L.tok_slot = off;
   if (with_backward) {
     const size_t H = (size_t)ctx->H;
     L.gates = take(4 * nn * 5 * (size_t)row_pitch(ctx->H));
@@ -40,7 +42,6 @@ WsLayout ws_layout(const treelstm* ctx, int n, bool with_backward) {
     L.dz = take(4 * nn * 5 * H);
     L.tok_slot = take(4 * ((size_t)ctx->vocab + 4 + ((size_t)ctx->vocab + 127) / 128));   // vocab + 1 entries in use, the scan
                                                                    // reads whole quads; then one count per 128 ids
-    L.walks = take(saved_walks_bytes(ctx, (int)nn));
   }
   L.img_dz = L.img_x0 = L.img_x1 = L.img_end = off;
   // forests that the tree kernels may be too slow for: operands of the backward pass split into bf16 pieces

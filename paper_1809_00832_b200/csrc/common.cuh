@@ -24,8 +24,7 @@ struct DevStatus {
   int tail_from;         // persistent bf16 forward: first wavefront the cluster kernel takes (or would take), n_levels if none
   int trees_fwd, trees_bwd;   // 1: the tree kernels (trees_fp32.cu, trees_tc.cu) took this forest forward / backward
   unsigned int tickets;       // CTAs that are done (publish_status)
-  int trees_left;             // 1: the leaves' kernel (trees_fp32.cu) has said that the tree kernel behind it leaves this forest
-  int pad[51];
+  int pad[52];
 };
 static_assert(sizeof(DevStatus) == 256, "control block is one 256-byte line group");
 

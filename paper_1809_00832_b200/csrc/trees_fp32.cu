@@ -70,6 +70,15 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t smem_addr, uint32_t rank)
 __device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
+// A row of n floats to shared memory, by one warp, in pieces of 1, 2 or 4 of them (both ends aligned to a piece, n a multiple); waits for nothing.
+__device__ __forceinline__ void copy_row(uint32_t dst, const float* src, int n, int piece, int lane) {
+  if (piece == 4)
+    for (int k = 4 * lane; k < n; k += 128) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 4u * k), "l"(src + k) : "memory");
+  else if (piece == 2)
+    for (int k = 2 * lane; k < n; k += 64) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + 4u * k), "l"(src + k) : "memory");
+  else
+    for (int k = lane; k < n; k += 32) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * k), "l"(src + k) : "memory");
+}
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Four sums over each group of LANES lanes: v[0] of a lane becomes the sum of value value_of_lane(lane) - every
@@ -180,7 +189,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   const int cs = p.s.cs, rank = cs > 1 ? (int)cta_rank() : 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int part = blockIdx.x / cs, parts = gridDim.x / cs;
-  const int H = p.H, Hp = p.Hp, JS = p.s.JS, JS4 = (JS + 3) & ~3, JL = p.s.JL, outs = U * JL, j0 = rank * JS;
+  const int H = p.H, Hp = p.Hp, JS = p.s.JS, JS4 = (JS + 3) & ~3, JL = p.s.JL, outs = U * JL, j0 = rank * JS, jn = min(JS, H - j0);   // (jn may be below one: a CTA without units)
   const TreesSmem s = trees_smem(p.n, fwd_buf_words(CELL, H, p.s));
 #ifdef TREELSTM_TRACE
   long long* const trace = blockIdx.x == 0 && tid == 0 ? p.trace : nullptr;   // row d: depth d; last row: set-up
@@ -191,18 +200,17 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   float w[RC * 4 * U];
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
+  float* const red = sm + s.buf;
+  for (int e = tid; e < fwd_parts(CELL, p.s) * NT * outs; e += kFwdT) red[e] = 0.f;   // (sums beyond the segments stay zero)
   // (dealing by size takes 10 k cycles, which TreeLSTM spends beside its leaves and a training step gains twice: 54 chains of 16
   // leaves, TreeRNN H = 79, forward alone 42 us without and 47 with it)
-  // Of a forest so large that the leaves' kernel takes its turns on the SMs, its choice is known when this kernel gets there: 29
-  // balanced trees of 256 leaves, H = 177, spent 60 us of 523 on lists that nobody walked.  (Some CTAs of a cluster may see it
-  // and others not: the lists alone are left out.)
-  const bool left = CELL == kLstm && p.choose && __syncthreads_or(tid == 0 && ld_volatile(&p.st->trees_left) != 0);
-  if (left) {
-    if (tid == 0) s_walk = Walk{0, 0, 0};
-    __syncthreads();
-  } else {
-    deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || SAVE, &s_loads, &s_walk, trace);
+  bool planned = false;
+  if constexpr (CELL == kLstm) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the leaves' states and the lists come from the kernel ahead, and whose forest it is
+    if (p.choose && !ld_volatile(&p.st->trees_fwd)) return;
+    planned = load_walk(p.walks, p.costs, p.n, 0, s, sm, part, parts, false, &s_loads, &s_walk);
   }
+  if (!planned) deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || SAVE, &s_loads, &s_walk, trace);
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
@@ -218,7 +226,6 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   // CTA's own units
   const int row = CELL == kRntn ? 2 * Hp : 4 * p.s.nseg * RC, crow = CELL == kLstm ? 2 * JS4 : 0;
   const bool resident = (long long)walk.internal * (row + crow) <= s.state_words;
-  float* const red = sm + s.buf;
   float* const act = red + fwd_parts(CELL, p.s) * NT * outs;
   float* const xrow = act + NT * outs;                   // states in L2: operand rows and cell states of a pass
   float* const state = resident ? sm + s.state : xrow;
@@ -233,33 +240,31 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
       xrow[e] = 0.f;
     }
   }
-  for (int e = tid; e < fwd_parts(CELL, p.s) * NT * outs; e += kFwdT) red[e] = 0.f;   // (sums beyond the segments stay zero)
-  int depths = walk.depths, leaves = walk.leaves;
-  if (CELL == kLstm) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // the leaves' states come from the kernel ahead, and whose forest it is
-    if (p.choose && !ld_volatile(&p.st->trees_fwd)) depths = leaves = 0;
-  }
-  cluster_sync(cs);                                      // every CTA of the cluster runs: its shared memory may be written
-  for (int q = warp; q < leaves; q += kFwdT / 32) {
+  const int depths = walk.depths, leaves = walk.leaves;
+  // A leaf per warp and turn, as copies that need no registers, so that all of a warp's leaves are under way at once (one leaf
+  // after the other through registers took 10 k cycles for the 60 of two sentences, pairs of leaves 8 k, this way 4 k).
+  const float* const leaf_rows = CELL == kLstm ? p.h : p.emb;
+  const int piece = H % 4 == 0 && (reinterpret_cast<uintptr_t>(leaf_rows) & 15) == 0 ? 4 : (H % 2 == 0 && (reinterpret_cast<uintptr_t>(leaf_rows) & 7) == 0 ? 2 : 1);
+  const uint32_t cstate_addr = smem_u32(cstate);
+#pragma unroll 1
+  for (int q = warp; q < leaves && resident; q += kFwdT / 32) {
     const int node = leaf[q];
     const unsigned code = leaf_par[q];
-    const bool keep = resident && code != kNoCaller;
-    const float* src = CELL == kLstm ? p.h + (size_t)node * H : p.emb + (size_t)(kids[node] & ~kLeafBit) * H;
-    float* dst = state + (code >> 1) * row + (code & 1) * Hp;
-    const bool copy = CELL != kLstm && q % cs == rank;   // a leaf's state is its word vector
-    if (keep || copy)
-      for (int k = lane; k < H; k += 32) {
-        const float v = CELL == kLstm ? __ldcg(src + k) : __ldg(src + k);
-        if (keep) dst[k] = v;
-        if (copy) {
-          p.h[(size_t)node * H + k] = v;
-          count_write(p.chk_counts, node, 1);
-        }
-      }
-    if (CELL == kLstm && keep)
-      for (int u = lane; u < JS && j0 + u < H; u += 32)
-        cstate[(code >> 1) * crow + (code & 1) * JS4 + u] = __ldcg(p.c + (size_t)node * H + j0 + u);
+    if (code == kNoCaller) continue;
+    copy_row(state_addr + 4u * ((code >> 1) * row + (code & 1) * Hp), leaf_rows + (size_t)(CELL == kLstm ? node : (int)(kids[node] & ~kLeafBit)) * H, H, piece, lane);
+    if (CELL == kLstm && jn > 0)
+      copy_row(cstate_addr + 4u * ((code >> 1) * crow + (code & 1) * JS4), p.c + (size_t)node * H + j0, jn, 1, lane);
   }
+  if (CELL != kLstm)                                     // a leaf's state is its word vector
+    for (int q = rank + cs * warp; q < leaves; q += cs * (kFwdT / 32)) {
+      const int node = leaf[q];
+      const float* const src = p.emb + (size_t)(kids[node] & ~kLeafBit) * H;
+      for (int k = lane; k < H; k += 32) {
+        p.h[(size_t)node * H + k] = __ldg(src + k);
+        count_write(p.chk_counts, node, 1);
+      }
+    }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   // the thread's first chunk, or (RNTN) its chunks' operands: b in bits 8.., a below, 255: the linear part
   const int lane_out = tid % JL, seg = tid / JL;
   const bool works = seg < p.s.nseg;
@@ -282,7 +287,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   const int cell_i = cell_q / JS, cell_u = cell_q - cell_i * JS;
   (void)cell_i; (void)cell_u; (void)sets;
   const int parts_sum = fwd_parts(CELL, p.s);
-  cluster_sync(cs);                                      // the leaves' states are in place
+  cluster_sync(cs);                                      // the leaves' states are in place; every CTA of the cluster runs: its shared memory may be written
   TL_STAMP(trace, kTraceLevels - 1, 3);
   for (int d = depths - 1; d >= 0; --d) {
     for (int lo = start[d], hi = start[d + 1]; lo < hi; lo += NT) {
@@ -437,9 +442,9 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     TL_STAMP(trace, d, 4);
   }
   // what follows on the stream waits for this grid only: it must not end before the scheduler ahead of it has
-  if (blockIdx.x == 0) {
+  if (CELL != kLstm && blockIdx.x == 0) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tid == 0 && (CELL != kLstm || !p.choose)) p.st->trees_fwd = s_loads.win;   // (TreeLSTM: else the leaves' kernel has said so)
+    if (tid == 0) p.st->trees_fwd = s_loads.win;         // (TreeLSTM: the leaves' kernel has said so)
   }
 }
 
@@ -466,6 +471,7 @@ struct LeafParams {
   int choose, parts;                       // 1: the first CTA says whether the clusters (so many) take the forest (clusters_win)
   const int* right;
   WalkCosts costs;
+  SavedWalks walks;                        // where it leaves what each of them walks
 };
 // image of the input weights: [slice of 32 units][input unit][gate i, o, u][unit], zeros behind the last unit
 __host__ __device__ inline size_t leaf_image_words(int H, int E) { return (size_t)((H + kLeafU - 1) / kLeafU) * E * 3 * kLeafU; }
@@ -498,28 +504,30 @@ __device__ __forceinline__ void leaf_rows(const float* As, const float* Ws, int 
     }
   }
 }
-// The choice takes no time here: the clusters' kernel waits for the leaves anyhow, and one CTA more beside them is done before
-// they are.  (In the clusters' own kernel, beside the walk, it cost 2.5 us of 90.)
+// The first CTA plans for the clusters' kernel, which waits for the leaves anyhow: whether it takes the forest, and what each cluster walks.  The
+// leaves' kernel is no longer for it (14.5 us, 25 sentences), and the clusters' kernel reads its lists in 2 k cycles where it made them in 23 k (H = 150, with
+// the leaves' copies there: forward 71 -> 60 us, training step 199 -> 184).
 constexpr int kLeafTableWords = kLeafSmem / 4;
 __host__ __device__ inline int leaves_tables_at(int n) { return (n + n / 32 + 4) / 4 * 4; }   // (16-byte boundary)
 __host__ __device__ inline bool leaves_hold_tables(int n) { return leaves_tables_at(n) + deal_words(n) <= kLeafTableWords; }
-__device__ __forceinline__ void leaves_choose(const LeafParams& p, float* sm) {
+__device__ __forceinline__ void leaves_plan(const LeafParams& p, float* sm) {
   __shared__ TreeLoads s_loads;
   const ForestIn q{p.n, p.vocab, p.left, p.right, p.token};
   TreesSmem s{};
   s.child = p.n;
-  const TreeLinks links = tree_links(sm + leaves_tables_at(p.n), p.n);
+  const int tables = leaves_tables_at(p.n), used = tables + deal_words(p.n);
+  const TreeLinks links = tree_links(sm + tables, p.n);
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm);
   const unsigned* child = reinterpret_cast<const unsigned*>(sm + s.child);
   if (threadIdx.x == 0) { s_loads.win = 1; s_loads.internal = 0; }
   const bool forest = !load_kids(q, s, sm, links.up, &s_loads.internal);   // (else the scheduler reports it)
-  if (forest) deal_by_size(p.n, kids, child, links, p.costs, p.parts, deals_by_size(p.n, s_loads.internal, p.parts), true, 0, &s_loads);
+  const bool dealt = forest && deals_by_size(p.n, s_loads.internal, p.parts);
+  if (forest) deal_by_size(p.n, kids, child, links, p.costs, p.parts, dealt, p.choose != 0, 0, &s_loads);
   __syncthreads();
+  const int win = s_loads.win;
+  plan_walks(p.n, kids, child, links, win != 0, forest, dealt, p.parts, reinterpret_cast<int*>(sm + used), kLeafTableWords - used, p.walks, &s_loads);
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the scheduler clears the control block at its start
-  if (threadIdx.x == 0) {
-    p.st->trees_fwd = s_loads.win;
-    p.st->trees_left = !s_loads.win;
-  }
+  if (threadIdx.x == 0) p.st->trees_fwd = win;
 }
 __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ LeafParams p) {
   extern __shared__ __align__(16) float leaf_smem[];
@@ -528,11 +536,11 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
   __shared__ int s_node[kLeafIds], s_tok[kLeafIds], s_count, s_abort;
   __shared__ __align__(8) uint64_t s_bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = p.H, E = p.E;
-  const int tiles_u = (H + kLeafU - 1) / kLeafU, block = (int)blockIdx.x - p.choose, slice = block % tiles_u;
+  const int tiles_u = (H + kLeafU - 1) / kLeafU, block = (int)blockIdx.x - 1, slice = block % tiles_u;
   const int id0 = block / tiles_u * kLeafIds, u0 = slice * kLeafU;
   const uint32_t bar = smem_u32(&s_bar);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (p.choose && blockIdx.x == 0) { leaves_choose(p, leaf_smem); return; }
+  if (blockIdx.x == 0) { leaves_plan(p, leaf_smem); return; }
   auto ask = [&](int k0) {                               // one thread: the weights of the next kLeafK indices
     const uint32_t bytes = (uint32_t)min(kLeafK, E - k0) * 3 * kLeafU * 4;
     mbar_arrive_expect_tx(bar, bytes);
@@ -601,7 +609,6 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
   if (__syncthreads_or(!ok)) {                           // a wait expired: what was asked for gets a bounded time to land
     if (tid == 32) { mbar_drain(bar, 0); mbar_drain(bar, 1); }
     __syncthreads();
-    if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
   float* const red = Ws;                                 // [quarter][row][gate][unit]
@@ -633,9 +640,8 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
       }
     }
   }
-  // the kernel behind this one waits for this grid only: it must not end before the scheduler ahead of it has (one CTA
-  // is enough for that; the others make room for that kernel)
-  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // (The kernel behind this one waits for this grid only, which must not end before the scheduler ahead of it has: the first CTA waits
+  // for that, the others make room for that kernel.)
 }
 
 
@@ -1091,7 +1097,7 @@ bool shape_fits(int cell, int H, int cs, TreesShape& s) {
 using TreesKernel = void (*)(const TreesParams);
 template <bool SAVE>
 TreesKernel forward_kernel_of(int cell) {
-  return cell == kRntn ? k_trees_forward<kRntn, 4, kRntnRC, SAVE> : (cell == kRnn ? k_trees_forward<kRnn, 4, kRnnRC, SAVE> : k_trees_forward<kLstm, 5, kLstmRC, SAVE>);
+  return cell == kRntn ? k_trees_forward<kRntn, 4, kRntnRC, SAVE> : (cell == kRnn ? k_trees_forward<kRnn, 4, kRnnRC, SAVE> : k_trees_forward<kLstm, 5, kLstmRC, false>);
 }
 TreesKernel forward_kernel(int cell, bool save) { return save ? forward_kernel_of<true>(cell) : forward_kernel_of<false>(cell); }
 TreesKernel backward_kernel(int cell, const TreesShape& s) {
@@ -1297,12 +1303,12 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
   p.choose = !trees_always_pay(ctx->cell, ctx->H, n, false);
   const int parts = trees_parts(ctx, n);
   p.gates = save && ctx->cell == kLstm ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
-  if (save) p.walks = {reinterpret_cast<unsigned char*>(ws) + lay.walks, saved_cap(n, parts)};
+  if (save || ctx->cell == kLstm) p.walks = {reinterpret_cast<unsigned char*>(ws) + lay.walks, saved_cap(n, parts)};
   if (ctx->cell == kLstm) {
     LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->trees.Wx, ctx->b, h, c, p.gates,
-                 p.st, ctx->opt.wait_limit_kcycles * 1024, p.choose, parts, right, p.costs};
+                 p.st, ctx->opt.wait_limit_kcycles * 1024, p.choose, parts, right, p.costs, p.walks};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((n + kLeafIds - 1) / kLeafIds * ((ctx->H + kLeafU - 1) / kLeafU) + p.choose);
+    cfg.gridDim = dim3((n + kLeafIds - 1) / kLeafIds * ((ctx->H + kLeafU - 1) / kLeafU) + 1);
     cfg.blockDim = dim3(kLeafT); cfg.dynamicSmemBytes = kLeafSmem; cfg.stream = stream;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

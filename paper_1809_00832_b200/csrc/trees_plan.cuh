@@ -397,9 +397,139 @@ __device__ __forceinline__ void save_walk(const SavedWalks& w, const TreesSmem& 
     }
   }
 }
+// The same from one CTA for all clusters, ahead of the kernel that walks (TreeLSTM forward: beside the leaves).  Behind deal_by_size, whose tables and
+// outcome it takes; all threads.  `at`: what the tables leave of the CTA's shared memory, `words` of it.  Every node climbs to its root; internal
+// nodes are counted by cluster and depth and take their places there (which one of a depth does not matter), then look up their callers' places.  Arrays
+// that are no forest get empty lists (the scheduler reports them); lists that are not wanted or not to be had say so in their headers.
+__device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const unsigned* child, const TreeLinks& t, bool wanted, bool forest, bool dealt, int parts, int* at, int words,
+                                           const SavedWalks& w, TreeLoads* loads) {
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  unsigned* const where = reinterpret_cast<unsigned*>(at);   // cluster | depth << 8, then place | cluster << 16
+  int* const next = at + n;
+  const bool room = n + parts <= words;                      // (as many depths as there is room for: below)
+  constexpr unsigned kNone = 0xFFFFFFFFu;
+  __syncthreads();
+  for (int q = tid; q < parts; q += nt) loads->nodes[q] = loads->depth[q] = 0;   // internal nodes, leaves
+  if (tid == 0) loads->internal = 0;                         // deepest
+  __syncthreads();
+  bool fits = wanted && forest && room && parts < 256;
+  if (fits) {
+    int deepest = 0;
+#pragma unroll 1
+    for (int k0 = tid; k0 < n; k0 += kClimbs * nt) {
+      int up[kClimbs], depth[kClimbs];
+#pragma unroll
+      for (int j = 0; j < kClimbs; ++j) { up[j] = min(k0 + j * nt, n - 1); depth[j] = 0; }
+#pragma unroll 1
+      for (int step = 0; step < n; ++step) {                 // (arrays that are no forest may hold a cycle)
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < kClimbs; ++j) {
+          const int x = t.up[up[j]];
+          if (x != up[j]) { ++depth[j]; any = true; }
+          up[j] = x;
+        }
+        if (!any) break;
+      }
+#pragma unroll
+      for (int j = 0; j < kClimbs; ++j) {
+        const int k = k0 + j * nt;
+        if (k >= n) continue;
+        const int rank = t.before[up[j] >> 5] + __popc(~child[up[j] >> 5] & ((1u << (up[j] & 31)) - 1u));
+        const bool tree = !(child[up[j] >> 5] >> (up[j] & 31) & 1u);
+        const unsigned part = dealt ? loads->part[min(rank, kDealt - 1)] : (unsigned)(rank % parts);
+        where[k] = tree ? part | (unsigned)depth[j] << 8 : kNone;
+        if (tree && !is_leaf(kids[k])) deepest = max(deepest, depth[j] + 1);
+      }
+    }
+    deepest = __reduce_max_sync(kFull, deepest);
+    if (lane == 0) atomicMax(&loads->internal, deepest);
+  }
+  __syncthreads();
+  const int depths = loads->internal;
+  fits = fits && n + parts * depths <= words;
+  if (fits) {
+    for (int q = tid; q < parts * depths; q += nt) next[q] = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int k = tid; k < n; k += nt) {
+      const unsigned v = where[k];
+      if (v != kNone && !is_leaf(kids[k])) atomicAdd(next + (v & 255u) * depths + (v >> 8), 1);
+    }
+    __syncthreads();
+    for (int part = tid >> 5; part < parts; part += nt >> 5) {
+      const SavedBlock b = saved_at(w, part);
+      int sum = 0, deep = 0;
+      for (int d0 = 0; d0 < depths; d0 += 32) {
+        const int d = d0 + lane, v = d < depths ? next[part * depths + d] : 0;
+        int incl = v;
+#pragma unroll
+        for (int e = 1; e < 32; e <<= 1) {
+          const int x = __shfl_up_sync(kFull, incl, e);
+          if (lane >= e) incl += x;
+        }
+        if (d < depths) next[part * depths + d] = sum + incl - v;
+        if (v && d <= w.cap) b.start[d] = (unsigned short)(sum + incl - v);
+        sum += __shfl_sync(kFull, incl, 31);
+        deep += __popc(__ballot_sync(kFull, v != 0));        // (depths have no gaps)
+      }
+      if (lane == 0) {
+        if (deep <= w.cap) b.start[deep] = (unsigned short)sum;
+        loads->nodes[part] = sum | deep << 16;
+      }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int k = tid; k < n; k += nt) {
+      const unsigned v = where[k], kd = kids[k];
+      if (v == kNone || is_leaf(kd)) continue;
+      const unsigned part = v & 255u;
+      const int q = atomicAdd(next + part * depths + (v >> 8), 1);
+      where[k] = (unsigned)q | part << 16;
+      if (q >= w.cap) continue;
+      const SavedBlock b = saved_at(w, (int)part);
+      b.list[q] = (unsigned short)k;
+      b.kids[q] = kd;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int k0 = 0; k0 < n; k0 += nt) {
+      const int k = min(k0 + tid, n - 1);
+      const bool have = k0 + tid < n && where[k] != kNone, lf = is_leaf(kids[k]);
+      const int part = have ? (int)(lf ? where[k] & 255u : where[k] >> 16) : -1, up = t.up[k];
+      unsigned code = kNoCaller;
+      if (up != k && have) code = 2u * (where[up] & 0xFFFFu) + (unsigned)((kids[up] & 0xFFFFu) != (unsigned)k);
+      const unsigned peers = __match_any_sync(kFull, have && lf ? part : -1);
+      int place = 0;
+      if (have && lf && lane == __ffs(peers) - 1) place = atomicAdd(&loads->depth[part], __popc(peers));
+      place = __shfl_sync(kFull, place, __ffs(peers) - 1) + __popc(peers & ((1u << lane) - 1u));
+      if (!have) continue;
+      const SavedBlock b = saved_at(w, part);
+      if (lf) {
+        if (place < 2 * w.cap) { b.leaf[place] = (unsigned short)k; b.leaf_par[place] = (unsigned short)code; }
+      } else if ((int)(where[k] & 0xFFFFu) < w.cap) {
+        b.par[where[k] & 0xFFFFu] = (unsigned short)code;
+      }
+    }
+    __syncthreads();
+  }
+  for (int part = tid; part < parts; part += nt) {
+    const int internal = loads->nodes[part] & 0xFFFF, deep = loads->nodes[part] >> 16, leaves = loads->depth[part];
+    const bool good = forest ? fits && internal <= w.cap && leaves <= 2 * w.cap : true;
+    *saved_at(w, part).head = good ? make_int4(deep, internal, leaves, parts) : make_int4(0, 0, 0, 0);
+  }
+}
 // All threads (of a small block each looks at several headers); false: there is nothing to load.  Of the child table only the entries of the cluster's internal nodes are filled.
+// (The first entries are asked for together with the headers.)
 __device__ __forceinline__ bool load_walk(const SavedWalks& w, const WalkCosts& costs, int n, int n_roots, const TreesSmem& s, float* sm, int part, int parts,
                                           bool choose, TreeLoads* loads, Walk* walk) {
+  const SavedBlock b = saved_at(w, part);
+  struct Entry { unsigned kids; unsigned short list, par, start, leaf, leaf_par; };
+  auto read = [&](int q) {
+    const int i = min(q, w.cap - 1), l = min(q, 2 * w.cap - 1);
+    return Entry{b.kids[i], b.list[i], b.par[i], b.start[min(q, w.cap)], b.leaf[l], b.leaf_par[l]};
+  };
+  Entry e = read(threadIdx.x);
   bool ok = true;
 #pragma unroll 1
   for (int q = threadIdx.x; q < parts; q += blockDim.x) {
@@ -421,21 +551,21 @@ __device__ __forceinline__ bool load_walk(const SavedWalks& w, const WalkCosts& 
     }
     __syncthreads();
   }
-  const SavedBlock b = saved_at(w, part);
   const Walk have = *walk;
 #pragma unroll 1
-  for (int q = threadIdx.x; q < have.leaves || q <= have.internal; q += blockDim.x) {
+  for (int q = threadIdx.x; q < have.leaves || q <= have.internal;) {
     if (q < have.internal) {
-      const int node = b.list[q];
-      reinterpret_cast<unsigned*>(sm + s.kids)[node] = b.kids[q];
-      reinterpret_cast<unsigned short*>(sm + s.list)[q] = (unsigned short)node;
-      reinterpret_cast<unsigned short*>(sm + s.par)[q] = b.par[q];
+      reinterpret_cast<unsigned*>(sm + s.kids)[e.list] = e.kids;
+      reinterpret_cast<unsigned short*>(sm + s.list)[q] = e.list;
+      reinterpret_cast<unsigned short*>(sm + s.par)[q] = e.par;
     }
-    if (q <= have.depths) reinterpret_cast<unsigned short*>(sm + s.start)[q] = b.start[q];
+    if (q <= have.depths) reinterpret_cast<unsigned short*>(sm + s.start)[q] = e.start;
     if (q < have.leaves) {
-      reinterpret_cast<unsigned short*>(sm + s.leaf)[q] = b.leaf[q];
-      reinterpret_cast<unsigned short*>(sm + s.leaf_par)[q] = b.leaf_par[q];
+      reinterpret_cast<unsigned short*>(sm + s.leaf)[q] = e.leaf;
+      reinterpret_cast<unsigned short*>(sm + s.leaf_par)[q] = e.leaf_par;
     }
+    q += blockDim.x;
+    e = read(q);
   }
   __syncthreads();
   return true;

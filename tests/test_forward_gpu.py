@@ -323,6 +323,28 @@ def test_fp32_leaves_at_the_limits_of_their_tiles(H, E, kind):
     assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
 
 
+@pytest.mark.parametrize("kind", ["one node", "one climb each", "one node more", "longer than a cluster's lists", "deeper than the tables"])
+def test_fp32_lists_from_the_leaves_kernel(kind):
+    """the clusters' lists, planned beside the leaves: a lone leaf, as many nodes as the planning CTA climbs from at once (3 x 512) and one
+    tree more, lists that are longer than a cluster's share of the workspace and more depths than the tables hold (the clusters then plan
+    for themselves); ids in no order, the same states twice"""
+    rng = np.random.default_rng(14)
+    params = fg.draw_params(rng, 20, 9, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.1)
+    sentences = [fg.random_split_shape(rng, int(k)) for k in rng.integers(2, 40, size=30)]
+    base = fg.forest_from_shapes(sentences, rng, 60).n_nodes
+    shapes = {"one node": [None], "one climb each": sentences + [None] * (1536 - base), "one node more": sentences + [None] * (1537 - base),
+              "longer than a cluster's lists": sentences[:5] + [fg.left_chain_shape(600)] + [None] * 400,
+              "deeper than the tables": [fg.left_chain_shape(1500)] + [fg.left_chain_shape(3)] * 200}[kind]
+    forest = fg.forest_from_shapes(shapes, rng, 60)
+    forest, _ = fg.permute_node_ids(forest, rng)
+    order = orc.schedule(forest.left, forest.right)[3]
+    h, c, _ = orc.forward_iterative(forest.left, forest.right, forest.token, params.emb, params.W, params.b, order)
+    model = util.make_model(params, "fp32")
+    first, again = (util.gpu_forward(model, forest, binding.PERSISTENT) for _ in range(2))
+    assert util.max_abs(first["h"], h) < util.TOL["fp32"] and util.max_abs(first["c"], c) < util.TOL["fp32"]
+    assert np.array_equal(first["h"], again["h"]) and np.array_equal(first["c"], again["c"])
+
+
 def test_calls_go_to_the_current_stream():
     device, other = torch.cuda.current_device(), torch.cuda.Stream()
     assert binding._stream() == binding._public_raw_stream(device) == torch.cuda.current_stream().cuda_stream
