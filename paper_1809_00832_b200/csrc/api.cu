@@ -203,7 +203,7 @@ int read_levels(treelstm* ctx) {
 int settle(treelstm* ctx, int status, int hint) {
   auto& L = ctx->last;
   if (status != 0) L.valid = false;
-  else if (hint != kTailUnknown && ctx->tail_ok && ctx->precision == TREELSTM_BF16 && L.mode == TREELSTM_PERSISTENT) ctx->tail_skip = hint == kNoTail;
+  else if (hint != kTailUnknown && L.says_tail && ctx->tail_ok && ctx->precision == TREELSTM_BF16 && L.mode == TREELSTM_PERSISTENT) ctx->tail_skip = hint == kNoTail;
   return status;
 }
 
@@ -454,7 +454,7 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
   auto& L = ctx->last;
   L.n = n_nodes; L.flags = flags; L.left = left; L.right = right; L.token = token;
   L.h = h; L.c = c; L.level = level; L.order = order; L.level_offset = lvl_off;
-  L.ws = workspace; L.lay = lay; L.stream = s; L.host_levels_valid = false; L.n_levels = 0;
+  L.ws = workspace; L.lay = lay; L.stream = s; L.host_levels_valid = false; L.n_levels = 0; L.says_tail = true;
 
   // Sub-forest mode needs the cluster plan of this context and a forest the single-CTA scheduler
   // can deal out; anything else runs the grid-wide persistent kernel instead.
@@ -464,7 +464,8 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
                           n_nodes > 0 && n_nodes <= single_max;
   int rc = launch_check_clear(ctx, n_nodes, workspace, lay, s);
   if (rc != TREELSTM_OK) return rc;
-  rc = trees_tc_asked(ctx, n_nodes, flags)
+  const bool asked = trees_tc_asked(ctx, n_nodes, flags);
+  rc = asked
            ? launch_schedule_trees_tc(ctx, n_nodes, left, right, token, h, c, level, order, lvl_off, n_levels, save, workspace, lay, s)
            : launch_schedule(ctx, n_nodes, left, right, token, level, order, lvl_off, n_levels, workspace, lay, subforests ? ctx->sf.n_parts : 0, s);
   if (rc != TREELSTM_OK) return rc;
@@ -473,12 +474,18 @@ int treelstm_forward(treelstm_t* ctx, int n_nodes, const int32_t* left, const in
   L.valid = true;
   ctx->bwd_counters_clear = true;                          // with the whole control block
   if (n_nodes == 0) return TREELSTM_OK;
+  ctx->ev_valid = false;
+  if (asked && trees_tc_always_take(ctx, n_nodes)) {
+    L.says_tail = false;
+    rc = launch_check_counts(ctx, n_nodes, order, left, workspace, lay, s);
+    if (rc != TREELSTM_OK) L.valid = false;
+    return rc;
+  }
 
   if (!persistent) {
     rc = read_levels(ctx);
     if (rc != TREELSTM_OK) { L.valid = false; return rc; }
   }
-  ctx->ev_valid = false;
   if (ctx->opt.time_kernel) TL_CUDA(ctx, cudaEventRecord(ctx->ev_begin, s));
   if (ctx->cell != 0)
     rc = launch_forward_rec(ctx, n_nodes, left, right, token, h, order, lvl_off, ctx->host_level_offset, L.n_levels,

@@ -186,7 +186,8 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
 #else
 #define TL_ROLE_STAMP(slot_first, slot_second) do { } while (0)
 #endif
-  if (only_level < 0) {
+  // (A CTA that comes up when clusters beside the scheduler have already taken the forest only looks and exits; read again behind the wait.)
+  if (only_level < 0 && ld_volatile(&p.st->trees_fwd) == 0) {
     // Every CTA reads the packed weights and biases in every wavefront, but they may have left L2 since
     // the last call: all CTAs ask for a share of them now, and for the tensor maps, so that the first
     // tiles do not wait for memory.
@@ -206,11 +207,13 @@ k_fwd_tc(const __grid_constant__ TmapSet maps, TcParams p, int only_level) {
   // is still worked out and left in the control block for the host to learn from).
   {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    const bool taken = ld_volatile(&p.st->trees_fwd) != 0;   // clusters evaluated the forest beside the scheduler (trees_tc.cu)
+    if (taken && blockIdx.x != 0) return;
     failed = ld_volatile(&p.st->status) != 0;      // schedule failed: nothing to evaluate
     n_levels = failed ? 0 : p.st->n_levels;
     const int tail_from = only_level < 0 ? tail_first_level(p.level_offset, n_levels, p.tail_width, p.tail_min_levels, s_stop) : n_levels;
     if (only_level < 0 && !failed && blockIdx.x == 0 && tid == 0) p.st->tail_from = tail_from;
-    if (ld_volatile(&p.st->trees_fwd) != 0) return;   // clusters evaluated the forest beside the scheduler (trees_tc.cu)
+    if (taken) return;
     lvl_end = only_level >= 0 ? only_level + 1 : (p.tail_launched ? tail_from : n_levels);
     for (int i = tid; i < kLevelCache && i <= n_levels; i += kThreads) s_level_offset[i] = p.level_offset[i];
   }

@@ -16,19 +16,21 @@ namespace tl {
 namespace {
 
 __global__ void __launch_bounds__(kSingleThreads, 1)
-k_schedule_single(int n, const int* __restrict__ left, const int* __restrict__ right,
-                  const int* __restrict__ token, int vocab, int* parent, int* level, int* order,
+k_schedule_single(int n, const int* left, const int* right, const int* token,
+                  int vocab, int* parent, int* level, int* order,
                   int* order_tmp, int* level_offset, int* roots, int* n_levels_out, DevStatus* st,
                   int n_parts, int* part_order, int* part_offset, int* slot, int cache_children) {
   extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_last(left, right, token);
   schedule_single(smem, false, n, left, right, token, vocab, parent, level, order, order_tmp, level_offset, roots, n_levels_out, st, n_parts,
                   part_order, part_offset, slot, cache_children);
 }
 __global__ void __launch_bounds__(kSingleThreads, 1)
-k_schedule_cluster(int n, const int* __restrict__ left, const int* __restrict__ right, const int* __restrict__ token,
+k_schedule_cluster(int n, const int* left, const int* right, const int* token,
                    int vocab, int* level, int* order, int* order_tmp, int* level_offset, int* roots, int* n_levels_out,
                    DevStatus* st, int sh) {
   extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_last(left, right, token);
   schedule_cluster(smem, false, n, left, right, token, vocab, level, order, order_tmp, level_offset, roots, n_levels_out, st, sh);
 }
 
@@ -287,11 +289,12 @@ int launch_schedule(treelstm* ctx, int n, const int32_t* left, const int32_t* ri
   if (n > 0 && n_parts == 0 && schedules_on_cluster(ctx, n)) {
     const int cs = ctx->sched_cluster;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cs; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1] = behind_last(ctx, stream);
     cfg.gridDim = dim3(cs); cfg.blockDim = dim3(kSingleThreads); cfg.dynamicSmemBytes = cl_smem_bytes(cl_shift(n, cs)); cfg.stream = stream;
-    cfg.attrs = &at; cfg.numAttrs = 1;
+    cfg.attrs = at; cfg.numAttrs = 2;
     TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_schedule_cluster, n, left, right, token, ctx->vocab, level, order, order_tmp,
                                     level_offset, roots, n_levels_out, st, cl_shift(n, cs)));
     ctx->launches += 1;
@@ -301,12 +304,14 @@ int launch_schedule(treelstm* ctx, int n, const int32_t* left, const int32_t* ri
     // the kernel clears the control block itself and writes the level count to the caller
     const bool parts = n_parts > 0 && n <= kSchedPartMaxNodes;
     const bool cache = single_caches_children(n, parts);
-    k_schedule_single<<<1, kSingleThreads, single_smem_bytes(n, parts) + (cache ? (size_t)n * 4 + 16 : 0), stream>>>(
-        n, left, right, token, ctx->vocab, parent, level, order, order_tmp, level_offset, roots, n_levels_out,
-        st, parts ? n_parts : 0, reinterpret_cast<int*>(base + lay.part_order),
-        reinterpret_cast<int*>(base + lay.part_offset), reinterpret_cast<int*>(base + lay.slot), cache ? 1 : 0);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = behind_last(ctx, stream);
+    cfg.gridDim = dim3(1); cfg.blockDim = dim3(kSingleThreads); cfg.dynamicSmemBytes = single_smem_bytes(n, parts) + (cache ? (size_t)n * 4 + 16 : 0); cfg.stream = stream;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_schedule_single, n, left, right, token, ctx->vocab, parent, level, order, order_tmp, level_offset, roots,
+                                    n_levels_out, st, parts ? n_parts : 0, reinterpret_cast<int*>(base + lay.part_order),
+                                    reinterpret_cast<int*>(base + lay.part_offset), reinterpret_cast<int*>(base + lay.slot), cache ? 1 : 0));
     ctx->launches += 1;
-    TL_CUDA(ctx, cudaGetLastError());
     return TREELSTM_OK;
   }
 

@@ -293,6 +293,12 @@ __device__ int place_few_levels(int n, int n_levels, const unsigned short* lv16,
   return s_root_total;
 }
 
+// A scheduler is a programmatic dependent of whatever is ahead of it on the stream (behind_last): it comes up while that ends, and reads, writes
+// and lets go nothing before.  (The pointers pass through, so that no load of constant data moves ahead of the wait.)
+__device__ __forceinline__ void wait_for_last(const int*& left, const int*& right, const int*& token) {
+  asm volatile("griddepcontrol.wait;" : "+l"(left), "+l"(right), "+l"(token) :: "memory");
+}
+
 __device__ __forceinline__ void clear_status(DevStatus* st, bool keep_choice) {
   const int word = (int)threadIdx.x;
   if (word < (int)(sizeof(DevStatus) / sizeof(int)) && !(keep_choice && word == (int)(offsetof(DevStatus, trees_fwd) / sizeof(int))))

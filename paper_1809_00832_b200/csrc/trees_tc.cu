@@ -156,7 +156,7 @@ struct TtPlan {
 // CTA of every cluster comes to the same answer: they all count all nodes.
 // Trees and depths come from pointer jumping (in place: a word holds an ancestor and its distance, whichever it is): 64 chains of
 // 64 leaves took 107 k cycles with climbs.
-__device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, int wide_words, TreeLoads* loads, long long* trace) {
+__device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, const ForestIn& f, int R, int wide_words, TreeLoads* loads, long long* trace) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = t.n, pt = t.pt, parts = t.parts;
 #pragma unroll 1
   for (int k = tid; k < n; k += pt) t.up[k] = (unsigned)k;
@@ -173,8 +173,8 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int k = tid + (j0 + j) * pt;
-      l[j] = k < n ? __ldg(p.f.left + k) : -1;
-      r[j] = k < n ? __ldg(p.f.right + k) : -1;
+      l[j] = k < n ? __ldg(f.left + k) : -1;
+      r[j] = k < n ? __ldg(f.right + k) : -1;
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -364,7 +364,7 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, int R, i
 // The cluster's lists: internal nodes by depth, their callers' rows and children, the leaves.  The place of a node among those of
 // its depth does not matter, but all CTAs must agree on it (it is an address in all of them): the first one gives the places out,
 // the others read its list.  All threads of the CTA; those behind the first pt only take part in the cluster's barrier.
-__device__ __forceinline__ void tt_lists(const TtPlan& t, float* sm, const TtLayout& L, int part, int rank, const TtParams& p, TreeLoads* loads, Walk* walk) {
+__device__ __forceinline__ void tt_lists(const TtPlan& t, float* sm, const TtLayout& L, int part, int rank, const ForestIn& f, TreeLoads* loads, Walk* walk) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = t.n, pt = t.pt;
   unsigned char* const base = reinterpret_cast<unsigned char*>(sm);
   unsigned short* const list = reinterpret_cast<unsigned short*>(base + L.list);
@@ -448,7 +448,7 @@ __device__ __forceinline__ void tt_lists(const TtPlan& t, float* sm, const TtLay
   const int leaves = loads->internal;
   unsigned* const ltok = reinterpret_cast<unsigned*>(base + L.ltok);
 #pragma unroll 1
-  for (int e = tid; e < leaves; e += pt) ltok[e] = (unsigned)min(max(__ldg(p.f.token + leaf[e]), 0), p.f.vocab - 1);
+  for (int e = tid; e < leaves; e += pt) ltok[e] = (unsigned)min(max(__ldg(f.token + leaf[e]), 0), f.vocab - 1);
   if (tid == 0) *walk = Walk{depths, mine, leaves};
 }
 
@@ -457,8 +457,9 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
   __shared__ Walk s_walk;
   __shared__ TreeLoads s_loads;
   const int cs = (int)cluster_size();
+  ForestIn f = p.f;
+  wait_for_last(f.left, f.right, f.token);
   if ((int)blockIdx.x < cs) {
-    const ForestIn& f = p.f;
     if (q.on_cluster)
       schedule_cluster(smem_raw, true, f.n, f.left, f.right, f.token, f.vocab, q.level, q.order, q.order_tmp, q.level_offset, q.roots, q.n_levels_out, p.st, q.sh);
     else if (blockIdx.x == 0)
@@ -468,10 +469,14 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     return;
   }
+  if ((int)blockIdx.x == cs && threadIdx.x == 0) {         // (nothing decided: the kernel behind, which comes up with what it needs unless it reads otherwise)
+    p.st->trees_fwd = 0;
+    __threadfence();
+  }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int rank = (int)cluster_rank(), part = (int)blockIdx.x / cs - 1, parts = (int)gridDim.x / cs - 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = p.f.n, H = p.H, Hp = p.Hp, Ep = p.Ep, gpc = p.gpc, U = 8 * gpc, U0 = rank * U;
+  const int n = f.n, H = p.H, Hp = p.Hp, Ep = p.Ep, gpc = p.gpc, U = 8 * gpc, U0 = rank * U;
   const TtLayout L = tt_layout(Hp, Ep, gpc);
   const uint32_t raw_addr = smem_u32(smem_raw), base = (raw_addr + 1023u) & ~1023u;
   unsigned char* const base_ptr = smem_raw + (base - raw_addr);
@@ -484,10 +489,10 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
 #endif
   TL_STAMP(trace, kTraceLevels - 1, 0);
   TtPlan t(sm, n, parts);
-  if (tid < t.pt) tt_decide(t, p, L.R, (int)L.rk / 4 - tt_tables(n).wide, &s_loads, trace);
+  if (tid < t.pt) tt_decide(t, p, f, L.R, (int)L.rk / 4 - tt_tables(n).wide, &s_loads, trace);
   __syncthreads();
   const bool taken = s_loads.win != 0;
-  if (part == 0 && rank == 0 && tid == 0) p.st->trees_fwd = taken ? 1 : 0;
+  if (part == 0 && rank == 0 && tid == 0 && taken) p.st->trees_fwd = 1;
   if (!taken) return;
   TL_STAMP(trace, kTraceLevels - 1, 3);
   uint64_t* const bars = reinterpret_cast<uint64_t*>(base_ptr + L.bars);
@@ -516,7 +521,7 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
   }
   __syncwarp();
   if (warp == kMmaWarp) tmem_alloc(smem_u32(s_tmem), 512);
-  tt_lists(t, sm, L, part, rank, p, &s_loads, &s_walk);
+  tt_lists(t, sm, L, part, rank, f, &s_loads, &s_walk);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -939,6 +944,11 @@ bool trees_tc_asked(const treelstm* ctx, int n, int flags) {
          ctx->opt.max_ctas == 0 && !ctx->opt.time_kernel && n >= 1 && n <= ctx->ttc.max_nodes && ctx->opt.sched_single_cta_max >= kSchedSingleMaxNodes;
 }
 
+// A forest that the clusters leave has a depth of more than R nodes, or more nodes than their lists hold.  One of no more than R nodes has neither whatever
+// its shape, and the kernels behind, which would look and exit, are not launched: one sentence of 30 words from and to host arrays, H = 256, 53.0 -> 50.2 us
+// (45.9 with the scheduler's early start).
+bool trees_tc_always_take(const treelstm* ctx, int n) { return n <= tt_layout(ctx->Hp, ctx->Ep, ctx->sf.groups_per_cta).R; }
+
 int launch_schedule_trees_tc(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h, float* c, int32_t* level,
                              int32_t* order, int32_t* level_offset, int32_t* n_levels_out, bool save_gates, void* ws, const WsLayout& lay, cudaStream_t stream) {
   char* base = static_cast<char*>(ws);
@@ -966,11 +976,12 @@ int launch_schedule_trees_tc(treelstm* ctx, int n, const int32_t* left, const in
   q.level = level; q.order = order; q.order_tmp = reinterpret_cast<int*>(base + lay.order_tmp);
   q.level_offset = level_offset; q.roots = reinterpret_cast<int*>(base + lay.roots); q.n_levels_out = n_levels_out;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cs; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1] = behind_last(ctx, stream);
   cfg.gridDim = dim3(cs * (1 + ctx->ttc.parts)); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = kSmemDynamic; cfg.stream = stream;
-  cfg.attrs = &at; cfg.numAttrs = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
   TL_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_schedule_trees_tc, ctx->sf_maps.wx[0], p, q));
   ctx->launches += 1;
   return TREELSTM_OK;

@@ -478,3 +478,29 @@ def test_cluster_launch_is_left_out_while_forests_have_no_tail():
         np.testing.assert_array_equal(res["h"], ref["h"])
         np.testing.assert_array_equal(res["c"], ref["c"])
     assert seen == [3, 2, 2, 3, 3, 2]
+
+
+@pytest.mark.parametrize("H", [40, 150, 256])
+@pytest.mark.parametrize("shapes", [[None], [None] * 64, [None] * 65, "chain 32", "chain 33", "balanced 32", "pairs"])
+def test_forests_that_only_clusters_can_take(H, shapes):
+    """up to 64 nodes one launch evaluates the forest and nothing follows it, whatever the shape; the first larger ones have the kernels behind it;
+    back to back without a host's look between them, each call starts while the last one ends"""
+    rng = np.random.default_rng(79)
+    params = fg.draw_params(rng, H, 24, 100, emb_dist="normal", emb_scale=0.3, w_scale=0.08)
+    if isinstance(shapes, str):
+        kind, _, k = shapes.partition(" ")
+        shapes = [fg.left_chain_shape(2)] * 21 if kind == "pairs" else [(fg.left_chain_shape if kind == "chain" else fg.balanced_shape)(int(k))]
+    forest = fg.forest_from_shapes(shapes, rng, 100)
+    forest, _ = fg.permute_node_ids(forest, rng)
+    model = util.make_model(params, "bf16")
+    arrays = [util.to_dev(a) for a in (forest.left, forest.right, forest.token)]
+    first, again = (model.forward(*arrays, check=False) for _ in range(2))
+    assert model.status_sync() == binding.OK
+    assert (model.last_launch_count() == 1) == (forest.n_nodes <= 64)
+    h, c, _ = orc.forward_recursive(forest.left, forest.right, forest.token, params.emb, params.W, params.b, operand_round=orc.round_to_bf16)
+    for out in (first, again):
+        assert util.max_abs(out["h"].cpu().numpy(), h) < TIGHT and util.max_abs(out["c"].cpu().numpy(), c) < TIGHT
+    arrays[0][int(np.flatnonzero(forest.left < 0)[0])] = 0              # a leaf with one child
+    with pytest.raises(binding.TreeLSTMError) as err:
+        model.forward(*arrays)
+    assert err.value.code == binding.ERR_INVALID_FOREST
