@@ -96,29 +96,66 @@ __device__ __forceinline__ void tile_store(const DwParams& p, unsigned char* til
 }
 
 // The third kind of work item, dEmb_rows += dz_leaves W_x^T, contracts over the gate columns, which are
-// contiguous in both operands (a leaf's dz row, a row of W): no transposition, a thread takes eight
-// consecutive columns of one row - one 16-byte piece - for two rows.  row_ptr(r): start of tile row r in
-// global memory or nullptr; j0: first column of the block; J: columns in a row.
+// contiguous in both operands (a leaf's dz row, a row of W): no transposition, a thread takes four
+// consecutive columns - half of a 16-byte piece - of four rows, sixteen lanes a row's whole block (eight columns a thread, one after
+// the other, had a warp touch 32 sectors with every load: 7.3 k cycles a block, this way 6.6 k).  row_ptr(r): start of tile row r in
+// global memory; j0: first column of the block; J: columns in a row; pairs: rows are even and start on 8-byte boundaries.
 template <class RowFn>
-__device__ __forceinline__ void rows_load(RowFn row_ptr, int j0, int J, float (&v)[2][8]) {
-  const int c = threadIdx.x & 7;
+__device__ __forceinline__ void rows_load(RowFn row_ptr, int j0, int J, bool pairs, float (&v)[2][8]) {
+  const int j = j0 + 4 * (threadIdx.x & 15);
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const float* row = row_ptr((threadIdx.x >> 3) + 64 * i);
+  for (int i = 0; i < 4; ++i) {
+    const float* row = row_ptr((threadIdx.x >> 4) + 32 * i);
+    float* x = &v[i >> 1][4 * (i & 1)];
+    if (pairs) {
+      const float2 a = *reinterpret_cast<const float2*>(row + min(j, J - 2)), b = *reinterpret_cast<const float2*>(row + min(j + 2, J - 2));
+      x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
+    } else {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[i][e] = row[min(j0 + 8 * c + e, J - 1)];
+      for (int e = 0; e < 4; ++e) x[e] = row[min(j + e, J - 1)];
+    }
   }
 }
 __device__ __forceinline__ void rows_store(unsigned char* tile, int rows_valid, int j0, int J, const float (&v)[2][8]) {
-  const int c = threadIdx.x & 7;
+  const int c = threadIdx.x & 15;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int r = (threadIdx.x >> 3) + 64 * i;
-    float x[8];
+  for (int i = 0; i < 4; ++i) {
+    const int r = (threadIdx.x >> 4) + 32 * i;
+    float x[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) x[e] = r < rows_valid && j0 + 8 * c + e < J ? v[i][e] : 0.f;
-    split_store8(tile, r, c, x);
+    for (int e = 0; e < 4; ++e) x[e] = r < rows_valid && j0 + 4 * c + e < J ? v[i >> 1][4 * (i & 1) + e] : 0.f;
+    uint32_t w0[2], w1[2], w2[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) split3_pair(x[2 * e], x[2 * e + 1], w0[e], w1[e], w2[e]);
+    unsigned char* dst = tile + swz_piece(r, c >> 1) + 8 * (c & 1);
+    *reinterpret_cast<uint2*>(dst) = make_uint2(w0[0], w0[1]);
+    *reinterpret_cast<uint2*>(dst + kSpTileBytes) = make_uint2(w1[0], w1[1]);
+    *reinterpret_cast<uint2*>(dst + 2 * kSpTileBytes) = make_uint2(w2[0], w2[1]);
   }
+}
+// A finished tile from its copy in shared memory to the outputs: rows [0, rows) of `cols` columns, row r to out_of(r), in adds of V floats
+// (5.5 to 6.5 k cycles one by one, H = 150, 4.2 to 5.5 k in pairs).
+template <int V, class OutFn>
+__device__ __forceinline__ void add_rows(const float* staged, int stride, int rows, int cols, OutFn out_of) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r = warp; r < rows; r += kDwThreads / 32) {
+    float* out = out_of(r);
+#pragma unroll
+    for (int i = 0; i < kDwTile / (32 * V); ++i) {
+      const int c = V * (lane + 32 * i);
+      if (c >= cols) continue;                               // (cols is a multiple of V)
+      const float* x = staged + (size_t)r * stride + c;
+      if constexpr (V == 4) atomicAdd(reinterpret_cast<float4*>(out + c), *reinterpret_cast<const float4*>(x));
+      else if constexpr (V == 2) atomicAdd(reinterpret_cast<float2*>(out + c), *reinterpret_cast<const float2*>(x));
+      else atomicAdd(out + c, *x);
+    }
+  }
+}
+template <class OutFn>
+__device__ __forceinline__ void add_rows(const float* staged, int stride, int rows, int cols, int width, uintptr_t address, OutFn out_of) {   // `width` floats a row of the output
+  if (width % 4 == 0 && address % 16 == 0) add_rows<4>(staged, stride, rows, cols, out_of);
+  else if (width % 2 == 0 && address % 8 == 0) add_rows<2>(staged, stride, rows, cols, out_of);
+  else add_rows<1>(staged, stride, rows, cols, out_of);
 }
 
 struct DwShape {
@@ -150,14 +187,11 @@ __host__ __device__ inline DwShape dw_shape(int n, int n_leaves, int H, int E, i
   s.items[2] = leaf_dinput ? s.leaf_tiles * s.e_tiles * s.runs2 : 0;
   return s;
 }
-// The number of 64-wide blocks per work item: as few as give every CTA of the grid at most one item.
-__host__ __device__ inline int dw_run(int n, int n_leaves, int H, int E, bool leaf_dinput, int ctas) {
-  int run = 1;
-  for (; run < kDwMaxRun; ++run) {
-    const DwShape s = dw_shape(n, n_leaves, H, E, run, leaf_dinput);
-    if (s.items[0] + s.items[1] + s.items[2] <= ctas) break;
-  }
-  return run;
+// The number of 64-wide blocks per work item: as few as give every CTA of the grid at most one item.  A whole warp, a lane per number.
+__device__ __forceinline__ int dw_run(int n, int n_leaves, int H, int E, bool leaf_dinput, int ctas) {
+  const DwShape s = dw_shape(n, n_leaves, H, E, min((int)(threadIdx.x & 31) + 1, kDwMaxRun), leaf_dinput);
+  const unsigned fits = __ballot_sync(0xffffffffu, s.items[0] + s.items[1] + s.items[2] <= ctas);
+  return min(fits ? __ffs(fits) : kDwMaxRun, kDwMaxRun);
 }
 
 // The sums over the nodes where the wavefront kernel has left both operands split (BwdImages): no thread touches a
@@ -272,7 +306,12 @@ __device__ __forceinline__ void dweight(DwParams& p) {
   __shared__ __align__(8) uint64_t s_bars[2 * kDwStages + 2];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  if (__syncthreads_or(ld_volatile(&p.st->status) != 0)) return;   // the passes before failed: nothing here may be trusted
+  // What the forward has left (status, level table, order) is final before this kernel comes up; the kernel ahead is waited for behind the first item's
+  // tables.  (Up to there 6 k cycles, beside the tree kernel's last clusters.  With the wider loads and adds: training step of 25 sentences 184.0 -> 180.1 us.)
+  if (__syncthreads_or(ld_volatile(&p.st->status) != 0)) {   // the forward failed: nothing here may be trusted
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* tiles = dw_dyn + ((1024u - (smem_u32(dw_dyn) & 1023u)) & 1023u);
   const uint32_t tiles_addr = smem_u32(tiles);
@@ -293,31 +332,22 @@ __device__ __forceinline__ void dweight(DwParams& p) {
   const uint32_t tmem_base = s_tmem;
   const int H = p.H, E = p.E, J = 5 * H;
   const int n_leaves = p.st->n_levels > 0 ? min(p.n, max(0, p.level_offset[1])) : 0;
-  if (p.img.dz != nullptr && !(p.after_trees && p.st->trees_bwd)) {
-    dw_from_images(p, n_leaves, tiles, stage_bar0, smem_u32(&s_bars[kDwStages + 2]), acc_bar, tmem_base, &s_abort);
-    tc_fence_before();
-    __syncthreads();
-    if (s_abort) {                         // what was asked for gets a bounded time to land, the MMAs a bounded time to retire
-      if (warp == 1 && elect_one()) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
-      if (tid == 0) for (int s = 0; s < kDwStages; ++s) mbar_drain(stage_bar0 + 8 * s, 0);
-      __syncthreads();
-    }
-    if (warp == 0) {
-      tc_fence_after();
-      tmem_dealloc(tmem_base, kSpTmemCols);
-    }
-    return;
-  }
   const bool leaf_dinput = p.dEmb_rows != nullptr;
-  const int run = dw_run(p.n, n_leaves, H, E, leaf_dinput, (int)gridDim.x);   // the host does not know the number of leaves
-  const DwShape sh = dw_shape(p.n, n_leaves, H, E, run, leaf_dinput);
+  // (Where the host knows that the operands are split, nothing is set up here: it would be behind the kernel ahead, 2 us of a step of 256 sentences.)
+  const bool images = p.img.dz != nullptr && !p.after_trees;
+  int run = 1;                           // the host does not know the number of leaves
+  DwShape sh{};
+  if (!images) {
+    run = dw_run(p.n, n_leaves, H, E, leaf_dinput, (int)gridDim.x);
+    sh = dw_shape(p.n, n_leaves, H, E, run, leaf_dinput);
+  }
   const uint32_t idesc = umma_idesc(kDwTile);
-  uint32_t built = 0, items_done = 0;   // blocks built / items finished by this CTA so far (barrier phases)
-  bool failed = false;
-  for (int item = blockIdx.x; item < sh.items[0] + sh.items[1] + sh.items[2] && !failed; item += gridDim.x) {
-    const int part = item < sh.items[0] ? 0 : (item < sh.items[0] + sh.items[1] ? 1 : 2);
+  const int n_items = sh.items[0] + sh.items[1] + sh.items[2];
+  int part = 0, m0 = 0, j0 = 0, pos0 = 0, pos_end = 0, nblk = 0, kb0 = 0, rows_here = 0;   // of the CTA's item
+  auto take = [&](int item) {            // its place and its tables
+    part = item < sh.items[0] ? 0 : (item < sh.items[0] + sh.items[1] ? 1 : 2);
     int it = item - (part > 0 ? sh.items[0] : 0) - (part > 1 ? sh.items[1] : 0);
-    int m0, j0, pos0 = 0, pos_end = 0, nblk, kb0 = 0, rows_here = 0;
+    pos0 = pos_end = kb0 = rows_here = 0;
     if (part < 2) {
       const int nt = it % sh.n_tiles; it /= sh.n_tiles;
       const int mt = it % sh.m_tiles[part], ri = it / sh.m_tiles[part];
@@ -353,6 +383,29 @@ __device__ __forceinline__ void dweight(DwParams& p) {
         s_node[t] = node; s_ia[t] = slot;
       }
     }
+  };
+  if ((int)blockIdx.x < n_items) take(blockIdx.x);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const bool stop = __syncthreads_or(ld_volatile(&p.st->status) != 0) != 0;   // (a label out of range)
+  if (!stop && (images || (p.img.dz != nullptr && !p.st->trees_bwd))) {
+    dw_from_images(p, n_leaves, tiles, stage_bar0, smem_u32(&s_bars[kDwStages + 2]), acc_bar, tmem_base, &s_abort);
+    tc_fence_before();
+    __syncthreads();
+    if (s_abort) {                         // what was asked for gets a bounded time to land, the MMAs a bounded time to retire
+      if (warp == 1 && elect_one()) { umma_commit(drain_bar); mbar_drain(drain_bar, 0); }
+      if (tid == 0) for (int s = 0; s < kDwStages; ++s) mbar_drain(stage_bar0 + 8 * s, 0);
+      __syncthreads();
+    }
+    if (warp == 0) {
+      tc_fence_after();
+      tmem_dealloc(tmem_base, kSpTmemCols);
+    }
+    return;
+  }
+  uint32_t built = 0, items_done = 0;   // blocks built / items finished by this CTA so far (barrier phases)
+  bool failed = false;
+  for (int item = blockIdx.x; item < n_items && !failed && !stop; item += gridDim.x) {
+    if (item != (int)blockIdx.x) take(item);
     __syncthreads();
     // The fp32 values of block b + 1 are on their way into registers while block b is split, stored and multiplied.
     auto block_col = [&](int b) {        // part 2: first gate column of the block
@@ -363,9 +416,9 @@ __device__ __forceinline__ void dweight(DwParams& p) {
     auto load_block = [&](int b) {
       if (part == 0) tile_load<0>(p, m0, s_node, s_ia, s_ib, b, na);
       else if (part == 1) tile_load<1>(p, m0, s_node, s_ia, s_ib, b, na);
-      else rows_load([&](int r) { return p.dz + (size_t)s_node[r] * J; }, block_col(b), J, na);
+      else rows_load([&](int r) { return p.dz + (size_t)s_node[r] * J; }, block_col(b), J, J % 2 == 0, na);   // (dz and W: the library's, on 256-byte boundaries)
       if (part < 2) tile_load<2>(p, j0, s_node, s_ia, s_ib, b, nb);
-      else rows_load([&](int r) { return p.W + (size_t)min(j0 + r, E - 1) * J; }, block_col(b), J, nb);
+      else rows_load([&](int r) { return p.W + (size_t)min(j0 + r, E - 1) * J; }, block_col(b), J, J % 2 == 0, nb);
     };
     load_block(0);
     for (int b = 0; b < nblk; ++b, ++built) {
@@ -421,20 +474,12 @@ __device__ __forceinline__ void dweight(DwParams& p) {
     __syncthreads();
     const int rows_valid = part < 2 ? min(kDwTile, sh.rows[part] + 1 - m0) : rows_here;
     const int cols_valid = part < 2 ? min(kDwTile, J - j0) : min(kDwTile, E - j0);
-    for (int r = warp; r < rows_valid; r += kDwThreads / 32) {
-      float* out;
-      if (part < 2) {
-        const int f = m0 + r;
-        out = f == sh.rows[part] ? p.db + j0 : p.dW + (size_t)((part ? E : 0) + f) * J + j0;
-      } else {
-        out = p.dEmb_rows + (size_t)s_ia[r] * E + j0;   // leaves with the same token share a row
-      }
-#pragma unroll
-      for (int i = 0; i < kDwTile / 32; ++i) {
-        const int c = lane + 32 * i;
-        if (c < cols_valid) atomicAdd(out + c, stage_out[(size_t)r * kRowStride + c]);
-      }
-    }
+    if (part < 2)
+      add_rows(stage_out, kRowStride, rows_valid, cols_valid, J, reinterpret_cast<uintptr_t>(p.dW) | reinterpret_cast<uintptr_t>(p.db),
+               [&](int r) { return m0 + r == sh.rows[part] ? p.db + j0 : p.dW + (size_t)((part ? E : 0) + m0 + r) * J + j0; });
+    else                                                     // leaves with the same token share a row
+      add_rows(stage_out, kRowStride, rows_valid, cols_valid, E, reinterpret_cast<uintptr_t>(p.dEmb_rows),
+               [&](int r) { return p.dEmb_rows + (size_t)s_ia[r] * E + j0; });
     __syncthreads();   // the next item overwrites the index tables, the stages and the accumulator
   }
   // teardown: MMAs still in flight after a failed wait get a bounded time to retire before tensor memory goes back
@@ -451,7 +496,6 @@ __device__ __forceinline__ void dweight(DwParams& p) {
   }
 }
 __global__ void __launch_bounds__(kDwThreads, 1) k_bwd_dweight_tc(DwParams p) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   dweight(p);
   publish_status(p.st, p.out);
 }

@@ -758,6 +758,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_trees_backward(const __grid_constan
   const uint32_t send_turn = 4u * (uint32_t)(cs * kND * 2 * JS), send_node = 4u * (uint32_t)(2 * JS);
   const int sum_i0 = tid / (2 * JS), sum_k0 = tid - sum_i0 * 2 * JS, sum_di = nt / (2 * JS), sum_dk = nt - sum_di * 2 * JS;
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  // All that is ahead of this grid has ended: the weight gradient's kernel may read it while it sets itself up.  (k_rec_grads, whose CTAs are small, would
+  // come up eight to an SM on the few SMs without a cluster and stay there: RNTN step 160 -> 174 us.)
+  if (CELL == kLstm) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   TL_STAMP(trace, kTraceLevels - 1, 3);
   if (resident)
     for (int e = tid; e < walk.internal * 2 * JS; e += nt) {
