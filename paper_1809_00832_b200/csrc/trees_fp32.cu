@@ -37,7 +37,10 @@
 namespace tl {
 namespace {
 
-constexpr int NT = 4;                     // nodes per pass of the forward
+constexpr int NT = 4;                     // nodes that are multiplied side by side in the forward
+// Nodes per pass.  A pass ends with sums, activations, stores to the callers' rows and a barrier, 1.2 k cycles whatever their number; RNTN, whose
+// pass has few of them, takes eight (25 sentences, H = 32, training step 163.9 -> 161.4 us; TreeRNN, H = 128, 116.2 -> 121).
+__host__ __device__ constexpr int pass_nodes(int cell) { return cell == TREELSTM_CELL_RNTN ? 2 * NT : NT; }
 constexpr int kFwdT = 512, kBwdT = 640;   // threads of a CTA (backward: at most)
 constexpr int kLstm = 0, kRnn = TREELSTM_CELL_TREERNN, kRntn = TREELSTM_CELL_RNTN;
 constexpr int kND = 16;                   // backward: nodes between two cluster barriers at most
@@ -165,11 +168,11 @@ __host__ __device__ inline WeightAt bwd_weight(int cell, int H, int E, const Tre
   return cell == kLstm ? WeightAt{((long long)E + out) * 5 * H + (long long)gate * H + j, -1} : WeightAt{(long long)out * H + j, -1};
 }
 
-// forward: partial sums [nseg][NT][outs], gate values [NT][outs], operand rows and cell states of a pass (states in L2)
+// forward: partial sums [nseg][pass][outs], gate values [pass][outs], operand rows and cell states of a pass (states in L2)
 __host__ __device__ inline int fwd_outs(const TreesShape& s) { return s.U * s.JL; }
 __host__ __device__ inline int fwd_parts(int cell, const TreesShape& s) { return ((cell == kRntn ? kFwdT / 32 : s.nseg) + 7) & ~7; }
 __host__ __device__ inline int fwd_buf_words(int cell, int H, const TreesShape& s) {
-  return (fwd_parts(cell, s) + 1) * NT * fwd_outs(s) + NT * (2 * ((H + 3) & ~3) + 2 * ((s.JS + 3) & ~3));
+  return (fwd_parts(cell, s) + 1) * pass_nodes(cell) * fwd_outs(s) + pass_nodes(cell) * (2 * ((H + 3) & ~3) + 2 * ((s.JS + 3) & ~3));
 }
 // backward: gate gradients of a round [kND][in_row], then the sums that came in [2][cs][kND][2 JS] (RNTN: and x)
 __host__ __device__ inline int bwd_in_row(int cell, const TreesShape& s) { return cell == kRntn ? kRntnJS : 4 * s.bseg * s.BC; }
@@ -186,6 +189,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   extern __shared__ __align__(16) float sm[];
   __shared__ Walk s_walk;
   __shared__ TreeLoads s_loads;
+  constexpr int kPass = pass_nodes(CELL);
   const int cs = p.s.cs, rank = cs > 1 ? (int)cta_rank() : 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int part = blockIdx.x / cs, parts = gridDim.x / cs;
@@ -201,7 +205,8 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) w[q] = __ldg(p.W + ((size_t)rank * (RC * 4 * U) + q) * kFwdT + tid);
   float* const red = sm + s.buf;
-  for (int e = tid; e < fwd_parts(CELL, p.s) * NT * outs; e += kFwdT) red[e] = 0.f;   // (sums beyond the segments stay zero)
+  if (CELL == kLstm)                                       // (sums beyond the segments stay zero; here beside the leaves' kernel)
+    for (int e = tid; e < fwd_parts(CELL, p.s) * kPass * outs; e += kFwdT) red[e] = 0.f;
   // (dealing by size takes 10 k cycles, which TreeLSTM spends beside its leaves and a training step gains twice: 54 chains of 16
   // leaves, TreeRNN H = 79, forward alone 42 us without and 47 with it)
   bool planned = false;
@@ -226,13 +231,13 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   // CTA's own units
   const int row = CELL == kRntn ? 2 * Hp : 4 * p.s.nseg * RC, crow = CELL == kLstm ? 2 * JS4 : 0;
   const bool resident = (long long)walk.internal * (row + crow) <= s.state_words;
-  float* const act = red + fwd_parts(CELL, p.s) * NT * outs;
-  float* const xrow = act + NT * outs;                   // states in L2: operand rows and cell states of a pass
+  float* const act = red + fwd_parts(CELL, p.s) * kPass * outs;
+  float* const xrow = act + kPass * outs;                   // states in L2: operand rows and cell states of a pass
   float* const state = resident ? sm + s.state : xrow;
-  float* const cstate = state + (resident ? walk.internal * row : NT * 2 * Hp);
+  float* const cstate = state + (resident ? walk.internal * row : kPass * 2 * Hp);
   const uint32_t state_addr = smem_u32(state);
   const int xstride = resident ? row : 2 * Hp;           // (the padding behind an L2 row is the next row: finite, times zero)
-  for (int e = tid; e < (resident ? walk.internal * (row - 2 * H) : NT * (2 * Hp + 2 * JS4)); e += kFwdT) {
+  for (int e = tid; e < (resident ? walk.internal * (row - 2 * H) : kPass * (2 * Hp + 2 * JS4)); e += kFwdT) {
     if (resident) {
       const int q = e / (row - 2 * H), k = e - q * (row - 2 * H);
       state[q * row + (k < Hp - H ? H + k : H + k + H)] = 0.f;
@@ -240,6 +245,8 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
       xrow[e] = 0.f;
     }
   }
+  if (CELL != kLstm)
+    for (int e = tid; e < fwd_parts(CELL, p.s) * kPass * outs; e += kFwdT) red[e] = 0.f;
   const int depths = walk.depths, leaves = walk.leaves;
   // A leaf per warp and turn, as copies that need no registers, so that all of a warp's leaves are under way at once (one leaf
   // after the other through registers took 10 k cycles for the 60 of two sentences, pairs of leaves 8 k, this way 4 k).
@@ -290,8 +297,8 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
   cluster_sync(cs);                                      // the leaves' states are in place; every CTA of the cluster runs: its shared memory may be written
   TL_STAMP(trace, kTraceLevels - 1, 3);
   for (int d = depths - 1; d >= 0; --d) {
-    for (int lo = start[d], hi = start[d + 1]; lo < hi; lo += NT) {
-      const int cnt = min(NT, hi - lo);
+    for (int lo = start[d], hi = start[d + 1]; lo < hi; lo += kPass) {
+      const int cnt = min(kPass, hi - lo);
       TL_STAMP(trace, d, 0);
       if (!resident) {
         // the children's states from L2 (a leaf of TreeRNN / RNTN: from the table itself)
@@ -309,13 +316,13 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
         __syncthreads();
       }
       const float* const x0 = state + (resident ? lo * row : 0);
-      auto multiply = [&](auto n_const) {
+      auto multiply = [&](auto n_const, int first) {       // nodes `first` .. of the pass
         constexpr int N = decltype(n_const)::value;
         float acc[N][U];
         const float* xb[N];
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-          xb[i] = x0 + min(i, cnt - 1) * xstride + (CELL == kRntn ? 0 : ops[0]);
+          xb[i] = x0 + min(first + i, cnt - 1) * xstride + (CELL == kRntn ? 0 : ops[0]);
 #pragma unroll
           for (int u = 0; u < U; ++u) acc[i][u] = 0.f;
         }
@@ -350,15 +357,18 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
             if constexpr (CELL == kRntn) {               // JL is a power of two: a warp adds its own segments first
               float v = acc[i][u];
               for (int dd = JL; dd < 32; dd <<= 1) v += __shfl_xor_sync(kFull, v, dd);
-              if (lane < JL) red[(warp * NT + i) * outs + u * JL + lane_out] = v;
+              if (lane < JL) red[(warp * kPass + first + i) * outs + u * JL + lane_out] = v;
             } else if (works) {
-              red[(seg * NT + i) * outs + u * JL + lane_out] = acc[i][u];
+              red[(seg * kPass + first + i) * outs + u * JL + lane_out] = acc[i][u];
             }
           }
       };
-      if (cnt == 1) multiply(std::integral_constant<int, 1>{});
-      else if (cnt == 2) multiply(std::integral_constant<int, 2>{});
-      else multiply(std::integral_constant<int, NT>{});
+#pragma unroll 1
+      for (int first = 0; first < (kPass > NT ? cnt : 1); first += NT) {
+        if (cnt - first == 1) multiply(std::integral_constant<int, 1>{}, first);
+        else if (cnt - first == 2) multiply(std::integral_constant<int, 2>{}, first);
+        else multiply(std::integral_constant<int, NT>{}, first);
+      }
       __syncthreads();
       TL_STAMP(trace, d, 1);
       auto put_h = [&](int q, int unit, float hv, int first, int by) {   // into the caller's row, in every CTA (or every by-th)
@@ -372,7 +382,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
       // States of the last nodes of a depth go to global memory behind the arrival at the cluster's barrier, which otherwise
       // waits until L2 has them (a release covers them too; nobody in the cluster reads them there if the rows are resident):
       // 25 sentences, TreeLSTM H = 150, forward 73.6 -> 71.3 us; training step TreeRNN H = 128 118.3 -> 115.9, RNTN H = 32 162.3 -> 160.4
-      const bool early = resident && lo + NT >= hi;
+      const bool early = resident && lo + kPass >= hi;
       float* h_to = nullptr;
       float h_kept = 0.f;
       for (int i = red_i, o = red_o; i < cnt;) {
@@ -380,10 +390,10 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
         const int g = CELL == kLstm ? (own ? red_g : o / JS) : 0, u = CELL == kLstm ? (own ? red_u : o - g * JS) : o;
         float z = own ? red_bias : __ldg(p.b + min(g, 4) * H + min(j0 + u, H - 1));
         const float* r = red + i * outs + o;
-        for (int q = 0; q < parts_sum; q += 8, r += 8 * NT * outs) {   // eight reads in flight (the sums are padded to eights)
+        for (int q = 0; q < parts_sum; q += 8, r += 8 * kPass * outs) {   // eight reads in flight (the sums are padded to eights)
           float v[8];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) v[k] = r[k * NT * outs];
+          for (int k = 0; k < 8; ++k) v[k] = r[k * kPass * outs];
           z += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
         }
         if constexpr (CELL == kLstm) {
@@ -434,7 +444,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
           p.c[h_to - p.h] = c_kept;
         }
       }
-      if (CELL != kLstm && lo + NT < hi) __syncthreads();   // the next pass's partial sums overwrite these
+      if (CELL != kLstm && lo + kPass < hi) __syncthreads();   // the next pass's partial sums overwrite these
       TL_STAMP(trace, d, 3);
     }
     if (!resident) cluster_arrive(cs);
