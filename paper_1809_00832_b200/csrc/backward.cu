@@ -1070,7 +1070,10 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
 // gradient.  What is left is latency: 10 - 14 k cycles of a narrow wavefront (3.3 k grid barrier, 3.5 k gate gradients, 2.5 k MMAs, 4 k
 // adds), 30 k of one of 300 nodes, 70 k of one of 2.5 k; 340 us in all (ncu, cold caches) for 14.6 k nodes, 19 wavefronts.
 constexpr int kWideSmem = 2 * kSpStageBytes + 1024, kWideThreads = 512;
-constexpr int kDirectRows = 256, kWideOffCache = 512;
+// A wavefront of up to kDirectRows nodes, one tile of them, forms its gate gradients where the tensor core reads them.  Two tiles have more blocks than
+// there are CTAs, and a CTA forms two, 17 k cycles where gradients through the images and a barrier take 12 k: wavefronts of 129 to 256 nodes 33 k -> 27 k
+// (H = 256; step of 256 sentences 598 -> 592 us).
+constexpr int kDirectRows = 128, kWideOffCache = 512;
 struct WideArgs {
   const int* level_offset;
   long long wait_limit;
@@ -1333,11 +1336,16 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
 #endif
   TL_STAMP(trace, kTraceLevels - 1, 0);
   unsigned int arrivals = 0;
+  bool arrived = false;                                  // at the next barrier already
   auto barrier = [&]() {
     arrivals += gridDim.x;
-    return grid_barrier(p.st, arrivals, a.wait_limit, &s_flag, true, &p.st->barrier_levels);
+    const bool arrive = !arrived;
+    arrived = false;
+    return grid_barrier(p.st, arrivals, a.wait_limit, &s_flag, arrive, &p.st->barrier_levels);
   };
-  // The inputs' images are for the kernel behind this one: CTAs without a share of a wavefront write them.
+  // The inputs' images are for the kernel behind this one: CTAs without a share of a wavefront write them.  They have nothing to tell the others, and
+  // arrive at the wavefront's barrier before: 64 rows take 10 k cycles, about as long as a narrow wavefront, and three of those had
+  // taken 21 k and not 11 k (training step, 256 sentences bf16: 605.1 -> 598.3 us).
   const int rows0 = (n_leaves + 63) / 64 * 64, chunks = rows0 / 64 + (n > n_leaves ? (n + 63) / 64 - n_leaves / 64 : 0);
   int chunks_done = 0;
   auto input_chunk = [&](int chunk) {
@@ -1349,7 +1357,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
     for (int q = (int)blockIdx.x * kWideThreads + tid; q < ((n + 63) / 64 * 64 - n) * ju * 8; q += grid * kWideThreads)
       split_store8_unit(dz_unit(a.img, n, q % (ju * 8) >> 3, ju), (n + q / (ju * 8)) & 63, q & 7, zero);
   }
-  bool ok = true, fetched = false;
+  bool ok = true, fetched = false, tables = false;       // of the next tile: tables read and blocks asked for; tables alone
   uint32_t blk = 0, asked = 0, done = 0;                 // blocks multiplied; asked for (thread 0); tiles
   auto read_tables = [&](const WidePlan& w, int pos0) {  // the nodes of a tile and where its rows go
     if (tid >= kSpTile) return;
@@ -1366,16 +1374,25 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
     }
     s_node[tid] = node; s_da[tid] = da; s_db[tid] = db;
   };
-  // thread 0: blocks k0 .. k0 + nk - 1 of a tile -> the ring
-  auto ask = [&](const WidePlan& w, int pos0, int ot, int k0, int nk) {
-    const unsigned char* wt = a.img.w + (size_t)((w.leaf ? 0 : wsp_tiles_x(E)) + ot) * wsp_kb * kSpOperandBytes;
+  // thread 0: blocks k0 .. k0 + nk - 1 of a tile -> the ring; the weights of the first `early` of them have been asked for ahead (ask_weights)
+  auto weights_at = [&](const WidePlan& w, int ot, int k) {
+    const int kb = k < w.skip_first ? k : k + w.skip;
+    return a.img.w + ((size_t)((w.leaf ? 0 : wsp_tiles_x(E)) + ot) * wsp_kb + kb) * kSpOperandBytes;
+  };
+  auto ask_weights = [&](const WidePlan& w, int ot, int k, uint32_t at) {   // at: the block's number in the ring
+    const uint32_t stage = at & 1u, bar = full0 + 8 * stage;
+    if (at >= 2 && !mbar_wait(empty0 + 8 * stage, ((at >> 1) - 1) & 1u, &s_abort, a.wait_limit, p.st)) return false;
+    mbar_arrive_expect_tx(bar, w.direct ? kSpOperandBytes : kSpStageBytes);
+    bulk_load(tiles_addr + stage * kSpStageBytes + kSpOperandBytes, weights_at(w, ot, k), kSpOperandBytes, bar);
+    return true;
+  };
+  auto ask = [&](const WidePlan& w, int pos0, int ot, int k0, int nk, uint32_t early) {
     for (int k = 0; k < nk; ++k) {
       const uint32_t stage = asked & 1u, dst = tiles_addr + stage * kSpStageBytes, bar = full0 + 8 * stage;
-      if (asked >= 2 && !mbar_wait(empty0 + 8 * stage, ((asked >> 1) - 1) & 1u, &s_abort, a.wait_limit, p.st)) return false;
+      if (k >= (int)early && !ask_weights(w, ot, k0 + k, asked)) return false;
       ++asked;
-      const int kk = k0 + k, kb = kk < w.skip_first ? kk : kk + w.skip;
-      mbar_arrive_expect_tx(bar, w.direct ? kSpOperandBytes : kSpStageBytes);
       if (!w.direct) {
+        const int kk = k0 + k, kb = kk < w.skip_first ? kk : kk + w.skip;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -1383,7 +1400,6 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
             bulk_load(dst + q * kSpTileBytes + h * kUnitPieceBytes, dz_unit(a.img, pos0 + 64 * h, kb, ju) + q * kUnitPieceBytes,
                       kUnitPieceBytes, bar);
       }
-      bulk_load(dst + kSpOperandBytes, wt + (size_t)kb * kSpOperandBytes, kSpOperandBytes, bar);
     }
     return true;
   };
@@ -1391,12 +1407,30 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   if (n_levels > 0) w = wide_plan(level_begin(n_levels - 1), level_begin(n_levels), n_levels == 1, H, E, grid);
   for (int lvl = n_levels - 1; lvl >= 0 && ok; --lvl) {
     TL_STAMP(trace, lvl, 0);
+    uint32_t early = 0;                                  // (thread 0)
     if (!w.direct) {
+      // What of this CTA's first tile does not depend on the gate gradients: its tables, the weights of two blocks (595 -> 590 us).
+      const int lo = blockIdx.x * w.per;
+      if (lo < w.total) {
+        const int tile = lo / w.span, k0 = lo - tile * w.span, nk = min(min(w.per, w.span - k0), w.kbs - k0);
+        if (nk > 0) {
+          if (tid == 0)
+            while (ok && early < 2u && (int)early < nk) {
+              ok = ask_weights(w, tile % w.to, k0 + (int)early, asked + early);
+              if (ok) ++early;
+            }
+          read_tables(w, w.base + tile / w.to * kSpTile);
+          tables = true;
+        }
+      }
       if (vec_h) wide_gates<true>(p, a.img, w);
       else wide_gates<false>(p, a.img, w);
       TL_STAMP(trace, lvl, 1);              // own gate gradients stored
       asm volatile("fence.proxy.async;" ::: "memory");   // the image is read by bulk copies
-      if (!(ok = barrier())) break;
+      if (!(ok = barrier())) {
+        asked += early;                                  // (under way)
+        break;
+      }
       asm volatile("fence.proxy.async;" ::: "memory");
       TL_STAMP(trace, lvl, 2);
     }
@@ -1406,8 +1440,10 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
         const int nk = min(len, w.kbs - k0), ot = tile % w.to, pos0 = w.base + tile / w.to * kSpTile;
         at += len;
         if (nk <= 0) continue;
-        if (!fetched) read_tables(w, pos0);
-        if (tid == 0 && !fetched) ok = ask(w, pos0, ot, k0, nk);
+        if (tid == 0 && !fetched) ok = ask(w, pos0, ot, k0, nk, early);
+        if (!fetched && !tables) read_tables(w, pos0);
+        tables = false;
+        early = 0;
         if (w.direct) {
           if (!fetched) __syncthreads();
           for (int k = 0; k < nk; ++k) {
@@ -1482,7 +1518,14 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
     if (!ok) break;
     const int busy = (w.total + w.per - 1) / w.per;
     if (busy < grid) {
-      if ((int)blockIdx.x >= busy && chunks_done + (int)blockIdx.x - busy < chunks) input_chunk(chunks_done + blockIdx.x - busy);
+      if ((int)blockIdx.x >= busy && chunks_done + (int)blockIdx.x - busy < chunks) {
+        if (lvl > 0) {
+          arrived = true;
+          __syncthreads();
+          if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&p.st->barrier_levels) : "memory");
+        }
+        input_chunk(chunks_done + blockIdx.x - busy);
+      }
       chunks_done += grid - busy;
     }
     if (lvl == 0) break;
@@ -1493,7 +1536,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
         const int tile = lo / w.span, k0 = lo - tile * w.span, nk = min(w.per, w.kbs - k0), pos0 = w.base + tile / w.to * kSpTile;
         if (nk > 0) {
           read_tables(w, pos0);
-          if (tid == 0) ask(w, pos0, tile % w.to, k0, nk);
+          if (tid == 0) ask(w, pos0, tile % w.to, k0, nk, 0);
           fetched = true;
         }
       }
