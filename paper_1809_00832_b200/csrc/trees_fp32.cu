@@ -482,6 +482,7 @@ struct LeafParams {
   const int* right;
   WalkCosts costs;
   SavedWalks walks;                        // where it leaves what each of them walks
+  int ids;                                 // consecutive node ids of a CTA
 };
 // image of the input weights: [slice of 32 units][input unit][gate i, o, u][unit], zeros behind the last unit
 __host__ __device__ inline size_t leaf_image_words(int H, int E) { return (size_t)((H + kLeafU - 1) / kLeafU) * E * 3 * kLeafU; }
@@ -532,10 +533,12 @@ __device__ __forceinline__ void leaves_plan(const LeafParams& p, float* sm) {
   if (threadIdx.x == 0) { s_loads.win = 1; s_loads.internal = 0; }
   const bool forest = !load_kids(q, s, sm, links.up, &s_loads.internal);   // (else the scheduler reports it)
   const bool dealt = forest && deals_by_size(p.n, s_loads.internal, p.parts);
-  if (forest) deal_by_size(p.n, kids, child, links, p.costs, p.parts, dealt, p.choose != 0, 0, &s_loads);
+  const bool climbed = p.n <= kLeafT * kClimbs && used + p.n <= kLeafTableWords;
+  if (forest)
+    deal_by_size(p.n, kids, child, links, p.costs, p.parts, dealt, p.choose != 0, 0, &s_loads, climbed ? reinterpret_cast<unsigned*>(sm + used) : nullptr);
   __syncthreads();
   const int win = s_loads.win;
-  plan_walks(p.n, kids, child, links, win != 0, forest, dealt, p.parts, reinterpret_cast<int*>(sm + used), kLeafTableWords - used, p.walks, &s_loads);
+  plan_walks(p.n, kids, child, links, win != 0, forest, dealt, climbed, p.parts, reinterpret_cast<int*>(sm + used), kLeafTableWords - used, p.walks, &s_loads);
   asm volatile("griddepcontrol.wait;" ::: "memory");     // the scheduler clears the control block at its start
   if (threadIdx.x == 0) p.st->trees_fwd = win;
 }
@@ -547,7 +550,7 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
   __shared__ __align__(8) uint64_t s_bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = p.H, E = p.E;
   const int tiles_u = (H + kLeafU - 1) / kLeafU, block = (int)blockIdx.x - 1, slice = block % tiles_u;
-  const int id0 = block / tiles_u * kLeafIds, u0 = slice * kLeafU;
+  const int id0 = block / tiles_u * p.ids, u0 = slice * kLeafU;
   const uint32_t bar = smem_u32(&s_bar);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (blockIdx.x == 0) { leaves_plan(p, leaf_smem); return; }
@@ -567,7 +570,7 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
 #pragma unroll
     for (int q = 0; q < kLeafIds / 32; ++q) {
       const int k = id0 + 32 * q + tid;
-      const bool lf = k < p.n && p.left[min(k, p.n - 1)] < 0;
+      const bool lf = k < min(p.n, id0 + p.ids) && p.left[min(k, p.n - 1)] < 0;
       const unsigned m = __ballot_sync(0xffffffffu, lf);
       if (lf) {
         const int at = count + __popc(m & ((1u << tid) - 1u));
@@ -580,7 +583,7 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
   }
   __syncthreads();
   const int count = s_count, quarter = warp >> 2;
-  const int rpt = count <= 32 ? 8 : (count <= 40 ? 10 : (count <= 48 ? 12 : 16)), row0 = (warp & 3) * rpt;
+  const int rpt = count <= 16 ? 4 : (count <= 28 ? 7 : (count <= 32 ? 8 : (count <= 40 ? 10 : (count <= 48 ? 12 : 16)))), row0 = (warp & 3) * rpt;
   const int u = min(u0 + lane, H - 1);
   const float bi = __ldg(p.b + u), bo = __ldg(p.b + 3 * H + u), bu = __ldg(p.b + 4 * H + u);
   float acc[16][3] = {};
@@ -610,7 +613,9 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
       for (int e = tid; e < (pitch - nk) * 3 * kLeafU; e += kLeafT) Ws[nk * 3 * kLeafU + e] = 0.f;
     if (__syncthreads_or(!ok)) { ok = false; break; }
     if (row0 < count) {
-      if (rpt == 8) leaf_rows<8>(As, Ws, pitch, nk, row0, quarter, lane, acc);
+      if (rpt == 4) leaf_rows<4>(As, Ws, pitch, nk, row0, quarter, lane, acc);
+      else if (rpt == 7) leaf_rows<7>(As, Ws, pitch, nk, row0, quarter, lane, acc);
+      else if (rpt == 8) leaf_rows<8>(As, Ws, pitch, nk, row0, quarter, lane, acc);
       else if (rpt == 10) leaf_rows<10>(As, Ws, pitch, nk, row0, quarter, lane, acc);
       else if (rpt == 12) leaf_rows<12>(As, Ws, pitch, nk, row0, quarter, lane, acc);
       else leaf_rows<16>(As, Ws, pitch, nk, row0, quarter, lane, acc);
@@ -1322,10 +1327,14 @@ int launch_forward_trees(treelstm* ctx, int n, const int32_t* left, const int32_
   p.gates = save && ctx->cell == kLstm ? reinterpret_cast<float*>(static_cast<char*>(ws) + lay.gates) : nullptr;
   if (save || ctx->cell == kLstm) p.walks = {reinterpret_cast<unsigned char*>(ws) + lay.walks, saved_cap(n, parts)};
   if (ctx->cell == kLstm) {
+    // As many CTAs as there are SMs, if that leaves each of them 32 ids or more: 25 sentences, H = 150, on 145 and not 115 of them 28 leaves and not 40 at most
+    // (with the planning CTA's shorter climbs: forward 58.7 -> 57.8 us).
+    const int slices = (ctx->H + kLeafU - 1) / kLeafU, blocks = std::max(1, (ctx->sm_count - 1) / slices);
+    const int ids = std::min(kLeafIds, std::max(32, (n + blocks - 1) / blocks));
     LeafParams q{n, ctx->H, ctx->E, ctx->vocab, p.chk_counts, left, token, ctx->emb, ctx->trees.Wx, ctx->b, h, c, p.gates,
-                 p.st, ctx->opt.wait_limit_kcycles * 1024, p.choose, parts, right, p.costs, p.walks};
+                 p.st, ctx->opt.wait_limit_kcycles * 1024, p.choose, parts, right, p.costs, p.walks, ids};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((n + kLeafIds - 1) / kLeafIds * ((ctx->H + kLeafU - 1) / kLeafU) + 1);
+    cfg.gridDim = dim3((n + ids - 1) / ids * slices + 1);
     cfg.blockDim = dim3(kLeafT); cfg.dynamicSmemBytes = kLeafSmem; cfg.stream = stream;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
