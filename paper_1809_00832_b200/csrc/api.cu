@@ -637,8 +637,10 @@ int treelstm_forward_host(treelstm_t* ctx, int n_nodes, const int32_t* left, con
       TL_CUDA(ctx, cudaMemcpyAsync(p.token, token, nb, cudaMemcpyHostToDevice, s));
     }
   }
+  ctx->behind_copy = true;
   int rc = treelstm_forward(ctx, n_nodes, p.left, p.right, p.token, p.h, p.c, p.level, p.order, nullptr,
                             p.n_levels, flags, p.ws, p.ws_bytes, s);
+  ctx->behind_copy = false;
   if (rc != TREELSTM_OK) return rc;
   const int launches_fwd = ctx->launches;
   const bool want_roots = root_ids || root_h || root_c || n_roots;

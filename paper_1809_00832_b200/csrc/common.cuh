@@ -199,6 +199,7 @@ struct treelstm {
   unsigned long long* bwd_status = nullptr;   // pinned, behind it: what the last kernel of a backward pass says, whenever that ends (StatusOut)
   int status_seq = 0, status_expected = 0;   // launches that write that word; the one whose word is to come (0: none)
   cudaStream_t status_stream = nullptr;
+  bool behind_copy = false;              // what is ahead on the stream is a copy of treelstm_forward_host's: nothing for the scheduler to come up beside
   bool bwd_counters_clear = false;       // the backward's arrival counters, in stream order: by the forward, and by the kernel that publishes the status
 
   // buffers of treelstm_forward_host (library-owned, grown on demand)
@@ -243,8 +244,8 @@ int launch_schedule(treelstm* ctx, int n, const int32_t* left, const int32_t* ri
 // (Not in a capture, whose nodes ahead may be of any kind.)  Calls that follow one another, with what the kernel behind clusters that took the forest no longer
 // does (gemm_tc.cu): 25 sentences bf16 42.9 -> 40.2 us, 256 sentences 119.7 -> 117.8, 64 chains 180.2 -> 177.6, 25 sentences fp32 60.1 -> 58.1.
 inline cudaLaunchAttribute behind_last(const treelstm* ctx, cudaStream_t stream) {
-  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) { cudaGetLastError(); capturing = cudaStreamCaptureStatusActive; }
+  cudaStreamCaptureStatus capturing = ctx->behind_copy ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  if (!ctx->behind_copy && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) { cudaGetLastError(); capturing = cudaStreamCaptureStatusActive; }
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = ctx->opt.overlap_launch && capturing == cudaStreamCaptureStatusNone ? 1 : 0;

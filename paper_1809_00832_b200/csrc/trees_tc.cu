@@ -80,7 +80,7 @@ __host__ __device__ inline TtLayout tt_layout(int Hp, int Ep, int gpc) {
   L.gates = L.rows + 2u * L.rows_bytes;
   return L;
 }
-// The plan's tables, offsets in 4-byte words: children by node (left | right << 16, or the top bit of a leaf), for every node an
+// The plan's tables, offsets in 4-byte words: children by node (left | right << 16, or the top bit and the token of a leaf), for every node an
 // ancestor and its distance (later tree | depth << 16, later the row), a bit for every node that has a caller, roots before each
 // word of those, sizes of the trees; behind them, nodes of every cluster's depths.
 struct TtTables { int kids, up, child, before, size, wide; };
@@ -169,19 +169,20 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, const Fo
   tt_sync(pt);
 #pragma unroll 1
   for (int j0 = 0; j0 * pt + tid < n; j0 += 4) {           // ids are clamped: nothing has been validated yet
-    int l[4], r[4];
+    int l[4], r[4], w[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int k = tid + (j0 + j) * pt;
       l[j] = k < n ? __ldg(f.left + k) : -1;
       r[j] = k < n ? __ldg(f.right + k) : -1;
+      w[j] = k < n ? __ldg(f.token + k) : 0;
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int k = tid + (j0 + j) * pt;
       if (k >= n) break;
       if (l[j] < 0) {
-        t.kids[k] = kLeafBit;
+        t.kids[k] = kLeafBit | (unsigned)min(max(w[j], 0), f.vocab - 1);   // (its token: no trip to memory behind the lists; 25 sentences 40.6 -> 40.2 us)
       } else {
         const unsigned a = (unsigned)min(l[j], n - 1), b = (unsigned)min(max(r[j], 0), n - 1);
         t.kids[k] = a | (b << 16);
@@ -364,7 +365,7 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, const Fo
 // The cluster's lists: internal nodes by depth, their callers' rows and children, the leaves.  The place of a node among those of
 // its depth does not matter, but all CTAs must agree on it (it is an address in all of them): the first one gives the places out,
 // the others read its list.  All threads of the CTA; those behind the first pt only take part in the cluster's barrier.
-__device__ __forceinline__ void tt_lists(const TtPlan& t, float* sm, const TtLayout& L, int part, int rank, const ForestIn& f, TreeLoads* loads, Walk* walk) {
+__device__ __forceinline__ void tt_lists(const TtPlan& t, float* sm, const TtLayout& L, int part, int rank, TreeLoads* loads, Walk* walk) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = t.n, pt = t.pt;
   unsigned char* const base = reinterpret_cast<unsigned char*>(sm);
   unsigned short* const list = reinterpret_cast<unsigned short*>(base + L.list);
@@ -448,7 +449,7 @@ __device__ __forceinline__ void tt_lists(const TtPlan& t, float* sm, const TtLay
   const int leaves = loads->internal;
   unsigned* const ltok = reinterpret_cast<unsigned*>(base + L.ltok);
 #pragma unroll 1
-  for (int e = tid; e < leaves; e += pt) ltok[e] = (unsigned)min(max(__ldg(f.token + leaf[e]), 0), f.vocab - 1);
+  for (int e = tid; e < leaves; e += pt) ltok[e] = t.kids[leaf[e]] & ~kLeafBit;
   if (tid == 0) *walk = Walk{depths, mine, leaves};
 }
 
@@ -521,7 +522,7 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
   }
   __syncwarp();
   if (warp == kMmaWarp) tmem_alloc(smem_u32(s_tmem), 512);
-  tt_lists(t, sm, L, part, rank, f, &s_loads, &s_walk);
+  tt_lists(t, sm, L, part, rank, &s_loads, &s_walk);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
