@@ -129,7 +129,10 @@ typedef enum treelstm_status {
                                             /* with TREELSTM_ERR_TIMEOUT.  0: cooperative launch in plain  */
                                             /* stream order (residency guaranteed by the runtime).  Of a   */
                                             /* backward pass the kernels with a grid barrier are always    */
-                                            /* cooperative: it may share the device                        */
+                                            /* cooperative: it may share the device.  With 1 the ready-set */
+                                            /* construction itself comes up while the launch ahead of it   */
+                                            /* on the stream ends (not in a stream capture); it waits for  */
+                                            /* that launch before it reads or writes anything              */
 #define TREELSTM_OPT_LEAVES_FIRST_MIN_NODES 9 /* accepted and without effect: an order of work that took   */
                                             /* the leaves before the schedule was the slower one at every  */
                                             /* size once forests from 4096 nodes on are scheduled by a     */
@@ -201,7 +204,8 @@ TREELSTM_API int treelstm_set_option(treelstm_t* ctx, int key, long long value);
  * max_nodes nodes.  Returns 0 on invalid arguments.  The buffer must be 256-byte aligned.
  * With with_backward the bytes grow with every node's gates, dh, dc and dz (48 H bytes, fp32) and, from some hundred
  * nodes on (H <= 512, E <= 1024), with dz and both cell inputs as three bf16 pieces, which doubles that: 14592 nodes,
- * H = 256, E = 300, bf16 forward: 425 MB, 191 of them pieces.
+ * H = 256, E = 300, bf16 forward: 425 MB, 191 of them pieces.  An fp32 TreeLSTM forward leaves its clusters' lists there (up to 36 bytes a node,
+ * at least 1 KB per cluster) whether or not a backward pass follows.
  */
 TREELSTM_API size_t treelstm_workspace_bytes(const treelstm_t* ctx, int max_nodes, int with_backward);
 
