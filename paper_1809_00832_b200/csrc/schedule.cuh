@@ -294,7 +294,8 @@ __device__ int place_few_levels(int n, int n_levels, const unsigned short* lv16,
 }
 
 // A scheduler is a programmatic dependent of whatever is ahead of it on the stream (behind_last): it comes up while that ends, and reads, writes
-// and lets go nothing before.  (The pointers pass through, so that no load of constant data moves ahead of the wait.)
+// and lets go nothing before.  (The pointers pass through, so that no load moves ahead of the wait; and the arrays, which the kernel ahead may still write when
+// this one has started, are not read as constant data.)
 __device__ __forceinline__ void wait_for_last(const int*& left, const int*& right, const int*& token) {
   asm volatile("griddepcontrol.wait;" : "+l"(left), "+l"(right), "+l"(token) :: "memory");
 }
@@ -324,8 +325,8 @@ __device__ __forceinline__ void clear_status(DevStatus* st, bool keep_choice) {
 //
 // Called by all kSingleThreads threads of one CTA.  keep_choice: the control block's word trees_fwd is another CTA's to write.
 __device__ __forceinline__ void
-schedule_single(unsigned char* smem, bool keep_choice, int n, const int* __restrict__ left, const int* __restrict__ right,
-                  const int* __restrict__ token, int vocab, int* parent, int* level, int* order,
+schedule_single(unsigned char* smem, bool keep_choice, int n, const int* left, const int* right, const int* token,
+                  int vocab, int* parent, int* level, int* order,
                   int* order_tmp, int* level_offset, int* roots, int* n_levels_out, DevStatus* st,
                   int n_parts, int* part_order, int* part_offset, int* slot, int cache_children) {
   const size_t w_bytes = (size_t)n * 4 > kSingleScratch ? (((size_t)n * 4 + 15) & ~(size_t)15) : kSingleScratch;
@@ -604,7 +605,7 @@ __device__ __forceinline__ void cl_sync() {
 
 // Called by all threads of all CTAs of one cluster.
 __device__ __forceinline__ void
-schedule_cluster(unsigned char* cl_smem, bool keep_choice, int n, const int* __restrict__ left, const int* __restrict__ right, const int* __restrict__ token,
+schedule_cluster(unsigned char* cl_smem, bool keep_choice, int n, const int* left, const int* right, const int* token,
                    int vocab, int* level, int* order, int* order_tmp, int* level_offset, int* roots, int* n_levels_out,
                    DevStatus* st, int sh) {
   ClSmem& sm = *reinterpret_cast<ClSmem*>(cl_smem);

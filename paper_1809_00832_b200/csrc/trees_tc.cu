@@ -173,9 +173,9 @@ __device__ __forceinline__ void tt_decide(TtPlan& t, const TtParams& p, const Fo
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int k = tid + (j0 + j) * pt;
-      l[j] = k < n ? __ldg(f.left + k) : -1;
-      r[j] = k < n ? __ldg(f.right + k) : -1;
-      w[j] = k < n ? __ldg(f.token + k) : 0;
+      l[j] = k < n ? __ldcg(f.left + k) : -1;
+      r[j] = k < n ? __ldcg(f.right + k) : -1;
+      w[j] = k < n ? __ldcg(f.token + k) : 0;
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {

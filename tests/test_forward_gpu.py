@@ -345,6 +345,30 @@ def test_fp32_lists_from_the_leaves_kernel(kind):
     assert np.array_equal(first["h"], again["h"]) and np.array_equal(first["c"], again["c"])
 
 
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+@pytest.mark.parametrize("n_trees", [1, 30, 300])
+def test_forests_that_kernels_ahead_of_the_call_write(precision, n_trees):
+    """the scheduler comes up while the launch ahead of it ends, here kernels that overwrite the forest's arrays in place (one forest, then
+    another of the same size) with no wait by the host: every call sees its own forest; schedulers of one CTA, of a cluster, beside tree clusters"""
+    rng = np.random.default_rng(15)
+    params = fg.draw_params(rng, 40, 24, 100, emb_dist="normal", emb_scale=0.3, w_scale=0.1)
+    sizes = rng.integers(2, 40, size=n_trees)
+    forests = [fg.forest_from_shapes([fg.random_split_shape(rng, int(k)) for k in sizes], rng, 100) for _ in range(2)]
+    model = util.make_model(params, precision)
+    refs = [util.gpu_forward(model, f, binding.PERSISTENT) for f in forests]
+    sources = [[util.to_dev(a) for a in (f.left, f.right, f.token)] for f in forests]
+    arrays = [torch.zeros_like(a) for a in sources[0]]
+    results = []
+    for call in range(12):
+        for to, a in zip(arrays, sources[call % 2]):
+            torch.mul(a, 1, out=to)
+        results.append(model.forward(*arrays, check=False))
+    assert model.status_sync() == binding.OK
+    for call, out in enumerate(results):
+        for key in ("h", "c", "level", "order"):
+            np.testing.assert_array_equal(out[key].cpu().numpy(), refs[call % 2][key])
+
+
 def test_calls_go_to_the_current_stream():
     device, other = torch.cuda.current_device(), torch.cuda.Stream()
     assert binding._stream() == binding._public_raw_stream(device) == torch.cuda.current_stream().cuda_stream
