@@ -306,8 +306,7 @@ __device__ __forceinline__ void dweight(DwParams& p) {
   __shared__ __align__(8) uint64_t s_bars[2 * kDwStages + 2];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  // What the forward has left (status, level table, order) is final before this kernel comes up; the kernel ahead is waited for behind the first item's
-  // tables.  (Up to there 6 k cycles, beside the tree kernel's last clusters.  With the wider loads and adds: training step of 25 sentences 184.0 -> 180.1 us.)
+  // What the forward has left (status, level table, order) is final before this kernel comes up.
   if (__syncthreads_or(ld_volatile(&p.st->status) != 0)) {   // the forward failed: nothing here may be trusted
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
@@ -384,6 +383,10 @@ __device__ __forceinline__ void dweight(DwParams& p) {
       }
     }
   };
+  // The first item's tables hold rows of the embedding gradient (tok_slot), which k_bwd_begin or, where that is the kernel ahead, k_bwd_persistent numbers.
+  // Behind the tree kernels they are read ahead of the wait: k_bwd_begin has ended when k_trees_backward lets this kernel come up, and a kernel between
+  // those two lets go at its end only and leaves the rows alone.  Else the kernel ahead is waited for first.
+  if (!p.after_trees) asm volatile("griddepcontrol.wait;" ::: "memory");
   if ((int)blockIdx.x < n_items) take(blockIdx.x);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const bool stop = __syncthreads_or(ld_volatile(&p.st->status) != 0) != 0;   // (a label out of range)

@@ -486,3 +486,21 @@ def test_backward_passes_side_by_side_share_the_device():
         assert [m.status_sync() for m in models] == [binding.OK] * 2
     for step in steps:
         _compare({k: v.cpu().numpy() for k, v in step.grads.items()}, ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("H,trees", [(300, 40), (300, 150), (520, 40), (520, 700)])
+def test_rows_that_the_kernel_ahead_numbers(H, trees):
+    """hidden sizes without tree kernels, where the launch ahead of the weight gradient numbers the embedding gradient's rows: forests of single leaves,
+    whose pass ends with that numbering; other words from step to step in the same memory, so that rows of the step before are never the right ones"""
+    rng = np.random.default_rng(H + trees)
+    vocab, E = 3000, 20
+    params = fg.draw_params(rng, H, E, vocab, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    model = util.make_model(params, "fp32")
+    for step in range(4):
+        forest = fg.forest_from_shapes([None] * trees, rng, vocab)
+        words = rng.choice(vocab, size=5 + 40 * step, replace=False).astype(np.int32)       # each of them several times, in any order
+        forest.token[:] = words[rng.integers(0, len(words), size=trees)]
+        labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+        ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                     params.bc, labels)
+        _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
