@@ -414,8 +414,10 @@ __device__ __forceinline__ void save_walk(const SavedWalks& w, const TreesSmem& 
   }
 }
 // The same from one CTA for all clusters, ahead of the kernel that walks (TreeLSTM forward: beside the leaves).  Behind deal_by_size, whose tables and
-// outcome it takes (`climbed`: what its climbs found is where the places go, `at`); all threads.  `at`: what the tables leave of the CTA's shared memory, `words` of it.  Every node climbs to its root; internal
-// nodes are counted by cluster and depth and take their places there (which one of a depth does not matter), then look up their callers' places.  Arrays
+// outcome it takes (`climbed`: what its climbs found is where the places go, `at`); all threads.  `at`: what the tables leave of the CTA's shared memory, `words` of it.
+// Every node finds its root and its distance from it by pointer jumping (in place: a word holds an ancestor and its distance, whichever it is; a step at a
+// time, a chain of 8192 leaves took millions of cycles).  Internal nodes are counted by cluster and depth and take their places there (which one of a depth does
+// not matter), then look up their callers' places.  Arrays
 // that are no forest get empty lists (the scheduler reports them); lists that are not wanted or not to be had say so in their headers.
 __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const unsigned* child, const TreeLinks& t, bool wanted, bool forest, bool dealt, bool climbed, int parts, int* at, int words,
                                            const SavedWalks& w, TreeLoads* loads) {
@@ -430,40 +432,46 @@ __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const un
   __syncthreads();
   bool fits = wanted && forest && room && parts < 256;
   if (fits) {
+    if (!climbed) {                                          // root | distance << 16, as the climbs leave them
+      for (int k = tid; k < n; k += nt) where[k] = (unsigned)t.up[k] | (t.up[k] != k ? 1u << 16 : 0u);
+      __syncthreads();
+      constexpr int kAhead = 4;
+#pragma unroll 1
+      for (int round = 0; round < 16; ++round) {             // (n < 2^15; arrays that are no forest may hold a cycle)
+        bool any = false;
+#pragma unroll 1
+        for (int k0 = tid; k0 < n; k0 += kAhead * nt) {
+          unsigned v[kAhead], u[kAhead];
+#pragma unroll
+          for (int j = 0; j < kAhead; ++j) v[j] = where[min(k0 + j * nt, n - 1)];
+#pragma unroll
+          for (int j = 0; j < kAhead; ++j) u[j] = where[v[j] & 0xFFFFu];
+#pragma unroll
+          for (int j = 0; j < kAhead; ++j)
+            if (k0 + j * nt < n && (u[j] & 0xFFFFu) != (v[j] & 0xFFFFu)) {
+              where[k0 + j * nt] = (u[j] & 0xFFFFu) | ((v[j] >> 16) + (u[j] >> 16)) << 16;
+              any = true;
+            }
+        }
+        if (!__syncthreads_or(any)) break;
+      }
+    }
     int deepest = 0;
 #pragma unroll 1
     for (int k0 = tid; k0 < n; k0 += kClimbs * nt) {
-      int up[kClimbs], depth[kClimbs];
+      unsigned v[kClimbs];
 #pragma unroll
-      for (int j = 0; j < kClimbs; ++j) {
-        up[j] = min(k0 + j * nt, n - 1);
-        depth[j] = 0;
-        if (climbed) {
-          const unsigned v = where[up[j]];
-          up[j] = (int)(v & 0xFFFFu);
-          depth[j] = (int)(v >> 16);
-        }
-      }
-#pragma unroll 1
-      for (int step = climbed ? n : 0; step < n; ++step) {   // (arrays that are no forest may hold a cycle)
-        bool any = false;
-#pragma unroll
-        for (int j = 0; j < kClimbs; ++j) {
-          const int x = t.up[up[j]];
-          if (x != up[j]) { ++depth[j]; any = true; }
-          up[j] = x;
-        }
-        if (!any) break;
-      }
+      for (int j = 0; j < kClimbs; ++j) v[j] = where[min(k0 + j * nt, n - 1)];
 #pragma unroll
       for (int j = 0; j < kClimbs; ++j) {
         const int k = k0 + j * nt;
         if (k >= n) continue;
-        const int rank = t.before[up[j] >> 5] + __popc(~child[up[j] >> 5] & ((1u << (up[j] & 31)) - 1u));
-        const bool tree = !(child[up[j] >> 5] >> (up[j] & 31) & 1u);
+        const int root = (int)(v[j] & 0xFFFFu), depth = (int)(v[j] >> 16);
+        const int rank = t.before[root >> 5] + __popc(~child[root >> 5] & ((1u << (root & 31)) - 1u));
+        const bool tree = !(child[root >> 5] >> (root & 31) & 1u);
         const unsigned part = dealt ? loads->part[min(rank, kDealt - 1)] : (unsigned)(rank % parts);
-        where[k] = tree ? part | (unsigned)depth[j] << 8 : kNone;
-        if (tree && !is_leaf(kids[k])) deepest = max(deepest, depth[j] + 1);
+        where[k] = tree ? part | (unsigned)depth << 8 : kNone;
+        if (tree && !is_leaf(kids[k])) deepest = max(deepest, depth + 1);
       }
     }
     deepest = __reduce_max_sync(kFull, deepest);

@@ -374,3 +374,17 @@ def test_calls_go_to_the_current_stream():
     assert binding._stream() == binding._public_raw_stream(device) == torch.cuda.current_stream().cuda_stream
     with torch.cuda.stream(other):
         assert binding._stream() == binding._public_raw_stream(device) == other.cuda_stream
+
+
+@pytest.mark.parametrize("shapes", ["two chains", "a chain among sentences", "single leaves"])
+def test_fp32_lists_of_more_nodes_than_climb_at_once(shapes):
+    """forests beyond the 1536 nodes that the planning CTA climbs from: depths and roots by pointer jumping, ids in no order"""
+    rng = np.random.default_rng(15)
+    params = fg.draw_params(rng, 20, 9, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.15, n_classes=0)
+    shapes = {"two chains": [fg.left_chain_shape(1025), fg.left_chain_shape(1000)], "single leaves": [None] * 1700,
+              "a chain among sentences": [fg.left_chain_shape(200)] + [fg.random_split_shape(rng, int(k)) for k in rng.integers(2, 40, size=60)]}[shapes]
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes, rng, 60), rng)
+    order = orc.schedule(forest.left, forest.right)[3]
+    h, c, _ = orc.forward_iterative(forest.left, forest.right, forest.token, params.emb, params.W, params.b, order)
+    res = util.gpu_forward(util.make_model(params, "fp32"), forest, binding.PERSISTENT)
+    assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
