@@ -204,8 +204,8 @@ TREELSTM_API int treelstm_set_option(treelstm_t* ctx, int key, long long value);
  * max_nodes nodes.  Returns 0 on invalid arguments.  The buffer must be 256-byte aligned.
  * With with_backward the bytes grow with every node's gates, dh, dc and dz (48 H bytes, fp32) and, from some hundred
  * nodes on (H <= 512, E <= 1024), with dz and both cell inputs as three bf16 pieces, which doubles that: 14592 nodes,
- * H = 256, E = 300, bf16 forward: 425 MB, 191 of them pieces.  An fp32 TreeLSTM forward leaves its clusters' lists there (up to 36 bytes a node,
- * at least 1 KB per cluster) whether or not a backward pass follows.
+ * H = 256, E = 300, bf16 forward: 425 MB, 191 of them pieces.  An fp32 TreeLSTM forward leaves its clusters' lists
+ * there whether or not a backward pass follows: 54 bytes a node and 1.3 KB for each cluster at most (H = 150: 15 clusters).
  */
 TREELSTM_API size_t treelstm_workspace_bytes(const treelstm_t* ctx, int max_nodes, int with_backward);
 

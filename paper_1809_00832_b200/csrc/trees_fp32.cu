@@ -215,12 +215,15 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     if (p.choose && !ld_volatile(&p.st->trees_fwd)) return;
     planned = load_walk(p.walks, p.costs, p.n, 0, s, sm, part, parts, false, &s_loads, &s_walk);
   }
-  if (!planned) deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || SAVE, &s_loads, &s_walk, trace);
+  if (!planned) {
+    deal_trees(p, p.costs, s, sm, part, parts, CELL != kLstm && p.choose, CELL == kLstm || SAVE, &s_loads, &s_walk, trace);
+    if (CELL == kLstm && SAVE && tid == 0) s_loads.longer = -1;   // (lists to be kept: below)
+  }
 #pragma unroll
   for (int q = 0; q < RC * 4 * U; ++q) asm volatile("" : "+f"(w[q]));   // held in registers: not to be loaded again where it is used
   TL_STAMP(trace, kTraceLevels - 1, 2);
   const Walk walk = s_walk;
-  if (SAVE && rank == 0) save_walk(p.walks, s, sm, part, parts, walk);
+  if (CELL != kLstm && SAVE && rank == 0) save_walk(p.walks, s, sm, part, parts, walk);
   const unsigned* kids = reinterpret_cast<const unsigned*>(sm + s.kids);
   const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
   const unsigned short* start = reinterpret_cast<const unsigned short*>(sm + s.start);
@@ -451,6 +454,9 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
     cluster_wait(cs);                                    // the depth's states are in place (and no CTA leaves while a peer still writes to it)
     TL_STAMP(trace, d, 4);
   }
+  // (TreeLSTM: not before all CTAs of the cluster have looked at the header, which says that there is nothing; and behind the walk, which the weights in
+  // registers leave no room for it beside: spilled, 25 sentences, training step 185 -> 187 us.)
+  if (CELL == kLstm && SAVE && rank == 0 && s_loads.longer < 0) save_walk(p.walks, trees_smem(p.n, fwd_buf_words(CELL, p.H, p.s)), sm, part, parts, s_walk);
   // what follows on the stream waits for this grid only: it must not end before the scheduler ahead of it has
   if (CELL != kLstm && blockIdx.x == 0) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1119,7 +1125,7 @@ bool shape_fits(int cell, int H, int cs, TreesShape& s) {
 using TreesKernel = void (*)(const TreesParams);
 template <bool SAVE>
 TreesKernel forward_kernel_of(int cell) {
-  return cell == kRntn ? k_trees_forward<kRntn, 4, kRntnRC, SAVE> : (cell == kRnn ? k_trees_forward<kRnn, 4, kRnnRC, SAVE> : k_trees_forward<kLstm, 5, kLstmRC, false>);
+  return cell == kRntn ? k_trees_forward<kRntn, 4, kRntnRC, SAVE> : (cell == kRnn ? k_trees_forward<kRnn, 4, kRnnRC, SAVE> : k_trees_forward<kLstm, 5, kLstmRC, SAVE>);
 }
 TreesKernel forward_kernel(int cell, bool save) { return save ? forward_kernel_of<true>(cell) : forward_kernel_of<false>(cell); }
 TreesKernel backward_kernel(int cell, const TreesShape& s) {
@@ -1313,7 +1319,8 @@ static int trees_parts(const treelstm* ctx, int n) {
 size_t saved_walks_bytes(const treelstm* ctx, int n) {
   if (ctx->precision != TREELSTM_FP32 || !ctx->trees.ok) return 0;
   size_t most = 0;
-  for (int parts = most_parts(ctx); parts >= 1; --parts) most = std::max(most, parts * saved_block(saved_cap(n < 32767 ? n : 32767, parts)));
+  n = std::min(n, 32767);
+  for (int parts = most_parts(ctx); parts >= 1; --parts) most = std::max(most, parts * saved_block(saved_cap(n, parts)) + (ctx->cell == kLstm ? longer_bytes(n, parts) : 0));
   return most;
 }
 

@@ -188,7 +188,7 @@ __device__ __forceinline__ void walk_trees(const ForestIn& p, const TreesSmem& s
 // What the clusters would have to walk, and (`win`) whether that is faster than wavefront by wavefront over the whole GPU;
 // of up to kDealt trees, the cluster that each goes to.
 constexpr int kMaxTreeClusters = 192, kClimbs = 3;
-struct TreeLoads { int nodes[kMaxTreeClusters], depth[kMaxTreeClusters], win, internal; unsigned char part[kDealt]; };
+struct TreeLoads { int nodes[kMaxTreeClusters], depth[kMaxTreeClusters], win, internal, longer; unsigned char part[kDealt]; };
 // Tables that are needed until the trees are dealt: callers by node id, roots before each word of the bit map, size and depth
 // of the trees.  Behind the lists (where the states go afterwards) if there is room, else in their place.
 struct TreeLinks { unsigned short* up; int *before, *size, *deep; };
@@ -372,25 +372,32 @@ __device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& c
   }
 }
 
-// What the clusters of a forward walked, kept in the workspace for the backward pass of the same forest, whose clusters
-// would otherwise work it out again beside k_bwd_begin (34 k cycles there for 25 sentences, H = 150).  One block per cluster:
-// header, then children, node and caller of every row, starts of the depths, leaves and their callers.  A cluster whose lists are
-// longer than `cap` says so, and the backward pass deals anew.
+// What the clusters of a forward walk, in the workspace: planned ahead of them by one CTA (plan_walks), or kept by them for the backward pass of the same forest,
+// whose clusters would otherwise work it out again beside k_bwd_begin (34 k cycles there for 25 sentences, H = 150).  One block per cluster:
+// header, then children, node and caller of every row, starts of the depths, leaves and their callers.  A block has room for four times the average
+// (`cap`).  One tree's lists are one cluster's, whatever their length: the planning CTA, which knows all of them, puts longer ones behind the blocks, one after
+// the other, and the header says where.  (Left to the clusters themselves, behind the leaves, the plan of one chain of 200 leaves
+// had its forward take 656 us and not 604, H = 150, and 321 and not 270, H = 24.)  A cluster that keeps its own lists says that it has none if they are longer, and the backward pass deals anew.
 struct SavedWalks { unsigned char* at; int cap; };
 __host__ __device__ inline int saved_cap(int n, int parts) { return min(n / 2 + 2, 4 * (n / 2 / parts) + 64); }
 __host__ __device__ inline size_t saved_block(int cap) { return (size_t)(16 + 18 * cap + 4 + 15) / 16 * 16; }
+__host__ __device__ inline size_t longer_bytes(int n, int parts) { return 18 * (size_t)n + 48 * (size_t)parts; }   // of all longer blocks: each has room for as many rows as the cluster has leaves
 struct SavedBlock { int4* head; unsigned* kids; unsigned short *list, *par, *start, *leaf, *leaf_par; };
-__device__ __forceinline__ SavedBlock saved_at(const SavedWalks& w, int part) {
-  unsigned char* at = w.at + saved_block(w.cap) * part;
+__device__ __forceinline__ SavedBlock saved_at(unsigned char* at, int cap) {
   SavedBlock b;
   b.head = reinterpret_cast<int4*>(at);
   b.kids = reinterpret_cast<unsigned*>(at + 16);
-  b.list = reinterpret_cast<unsigned short*>(b.kids + w.cap);
-  b.par = b.list + w.cap;
-  b.leaf = b.par + w.cap;
-  b.leaf_par = b.leaf + 2 * w.cap;
-  b.start = b.leaf_par + 2 * w.cap;
+  b.list = reinterpret_cast<unsigned short*>(b.kids + cap);
+  b.par = b.list + cap;
+  b.leaf = b.par + cap;
+  b.leaf_par = b.leaf + 2 * cap;
+  b.start = b.leaf_par + 2 * cap;
   return b;
+}
+__device__ __forceinline__ SavedBlock saved_at(const SavedWalks& w, int part) { return saved_at(w.at + saved_block(w.cap) * part, w.cap); }
+// `where`: 16-byte units behind the blocks, plus one
+__device__ __forceinline__ SavedBlock longer_at(const SavedWalks& w, int parts, int where, int leaves) {
+  return saved_at(w.at + saved_block(w.cap) * parts + 16 * (size_t)(where - 1), leaves);
 }
 // All threads, with the cluster's lists in shared memory.
 __device__ __forceinline__ void save_walk(const SavedWalks& w, const TreesSmem& s, const float* sm, int part, int parts, const Walk& walk) {
@@ -417,20 +424,20 @@ __device__ __forceinline__ void save_walk(const SavedWalks& w, const TreesSmem& 
 // outcome it takes (`climbed`: what its climbs found is where the places go, `at`); all threads.  `at`: what the tables leave of the CTA's shared memory, `words` of it.
 // Every node finds its root and its distance from it by pointer jumping (in place: a word holds an ancestor and its distance, whichever it is; a step at a
 // time, a chain of 8192 leaves took millions of cycles).  Internal nodes are counted by cluster and depth and take their places there (which one of a depth does
-// not matter), then look up their callers' places.  Arrays
-// that are no forest get empty lists (the scheduler reports them); lists that are not wanted or not to be had say so in their headers.
+// not matter), then look up their callers' places.  Clusters without a tree have no counts: one tree's depths fit whatever their number.  Arrays
+// that are no forest get empty lists (the scheduler reports them); lists that are not wanted or not to be had say so in all headers.
 __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const unsigned* child, const TreeLinks& t, bool wanted, bool forest, bool dealt, bool climbed, int parts, int* at, int words,
                                            const SavedWalks& w, TreeLoads* loads) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-  unsigned* const where = reinterpret_cast<unsigned*>(at);   // cluster | depth << 8, then place | cluster << 16
+  unsigned* const where = reinterpret_cast<unsigned*>(at);   // cluster | depth << 8; then a leaf's cluster | place << 8, an internal node's place | cluster << 16
   int* const next = at + n;
-  const bool room = n + parts <= words;                      // (as many depths as there is room for: below)
+  const int busy = max(1, min(parts, n - 2 * loads->internal));   // clusters with a tree
   constexpr unsigned kNone = 0xFFFFFFFFu;
   __syncthreads();
-  for (int q = tid; q < parts; q += nt) loads->nodes[q] = loads->depth[q] = 0;   // internal nodes, leaves
-  if (tid == 0) loads->internal = 0;                         // deepest
+  for (int q = tid; q < parts; q += nt) loads->nodes[q] = loads->depth[q] = 0;   // internal nodes | place behind the blocks << 16; leaves | depths << 16
+  if (tid == 0) loads->internal = loads->longer = 0;         // deepest; 16-byte units in use behind the blocks
   __syncthreads();
-  bool fits = wanted && forest && room && parts < 256;
+  bool fits = wanted && forest && n + busy <= words && parts < 256;   // (as many depths as there is room for: below)
   if (fits) {
     if (!climbed) {                                          // root | distance << 16, as the climbs leave them
       for (int k = tid; k < n; k += nt) where[k] = (unsigned)t.up[k] | (t.up[k] != k ? 1u << 16 : 0u);
@@ -479,18 +486,35 @@ __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const un
   }
   __syncthreads();
   const int depths = loads->internal;
-  fits = fits && n + parts * depths <= words;
+  fits = fits && n + busy * depths <= words;
   if (fits) {
-    for (int q = tid; q < parts * depths; q += nt) next[q] = 0;
+    for (int q = tid; q < busy * depths; q += nt) next[q] = 0;
     __syncthreads();
 #pragma unroll 1
-    for (int k = tid; k < n; k += nt) {
-      const unsigned v = where[k];
-      if (v != kNone && !is_leaf(kids[k])) atomicAdd(next + (v & 255u) * depths + (v >> 8), 1);
+    for (int k0 = 0; k0 < n; k0 += nt) {                     // (leaves take their places)
+      const int k = min(k0 + tid, n - 1);
+      const unsigned v = k0 + tid < n ? where[k] : kNone;
+      const bool lf = v != kNone && is_leaf(kids[k]);
+      if (v != kNone && !lf) atomicAdd(next + (v & 255u) * depths + (v >> 8), 1);
+      const unsigned peers = __match_any_sync(kFull, lf ? (int)(v & 255u) : -1);
+      int place = 0;
+      if (lf && lane == __ffs(peers) - 1) place = atomicAdd(loads->depth + (v & 255u), __popc(peers));
+      place = __shfl_sync(kFull, place, __ffs(peers) - 1) + __popc(peers & ((1u << lane) - 1u));
+      if (lf) where[k] = (v & 255u) | (unsigned)place << 8;
     }
     __syncthreads();
-    for (int part = tid >> 5; part < parts; part += nt >> 5) {
-      const SavedBlock b = saved_at(w, part);
+    for (int part = tid; part < busy; part += nt) {          // lists that may be longer than a block (a tree has one more leaf than internal nodes)
+      const int leaves = loads->depth[part];
+      if (leaves > w.cap) loads->nodes[part] = (atomicAdd(&loads->longer, (int)(saved_block(leaves) / 16)) + 1) << 16;
+    }
+    __syncthreads();
+    const bool longer = loads->longer != 0;
+    auto block_of = [&](int part) {
+      const int place = longer ? loads->nodes[part] >> 16 : 0;
+      return place ? longer_at(w, parts, place, loads->depth[part] & 0xFFFF) : saved_at(w, part);
+    };
+    for (int part = tid >> 5; part < busy; part += nt >> 5) {
+      const SavedBlock b = block_of(part);
       int sum = 0, deep = 0;
       for (int d0 = 0; d0 < depths; d0 += 32) {
         const int d = d0 + lane, v = d < depths ? next[part * depths + d] : 0;
@@ -501,13 +525,14 @@ __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const un
           if (lane >= e) incl += x;
         }
         if (d < depths) next[part * depths + d] = sum + incl - v;
-        if (v && d <= w.cap) b.start[d] = (unsigned short)(sum + incl - v);
+        if (v) b.start[d] = (unsigned short)(sum + incl - v);
         sum += __shfl_sync(kFull, incl, 31);
         deep += __popc(__ballot_sync(kFull, v != 0));        // (depths have no gaps)
       }
       if (lane == 0) {
-        if (deep <= w.cap) b.start[deep] = (unsigned short)sum;
-        loads->nodes[part] = sum | deep << 16;
+        b.start[deep] = (unsigned short)sum;
+        loads->depth[part] |= deep << 16;
+        loads->nodes[part] |= sum;
       }
     }
     __syncthreads();
@@ -518,58 +543,54 @@ __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const un
       const unsigned part = v & 255u;
       const int q = atomicAdd(next + part * depths + (v >> 8), 1);
       where[k] = (unsigned)q | part << 16;
-      if (q >= w.cap) continue;
-      const SavedBlock b = saved_at(w, (int)part);
+      const SavedBlock b = block_of((int)part);
       b.list[q] = (unsigned short)k;
       b.kids[q] = kd;
     }
     __syncthreads();
 #pragma unroll 1
-    for (int k0 = 0; k0 < n; k0 += nt) {
-      const int k = min(k0 + tid, n - 1);
-      const bool have = k0 + tid < n && where[k] != kNone, lf = is_leaf(kids[k]);
-      const int part = have ? (int)(lf ? where[k] & 255u : where[k] >> 16) : -1, up = t.up[k];
+    for (int k = tid; k < n; k += nt) {
+      const unsigned v = where[k];
+      if (v == kNone) continue;
+      const bool lf = is_leaf(kids[k]);
+      const int up = t.up[k];
       unsigned code = kNoCaller;
-      if (up != k && have) code = 2u * (where[up] & 0xFFFFu) + (unsigned)((kids[up] & 0xFFFFu) != (unsigned)k);
-      const unsigned peers = __match_any_sync(kFull, have && lf ? part : -1);
-      int place = 0;
-      if (have && lf && lane == __ffs(peers) - 1) place = atomicAdd(&loads->depth[part], __popc(peers));
-      place = __shfl_sync(kFull, place, __ffs(peers) - 1) + __popc(peers & ((1u << lane) - 1u));
-      if (!have) continue;
-      const SavedBlock b = saved_at(w, part);
+      if (up != k) code = 2u * (where[up] & 0xFFFFu) + (unsigned)((kids[up] & 0xFFFFu) != (unsigned)k);
+      const SavedBlock b = block_of((int)(lf ? v & 255u : v >> 16));
       if (lf) {
-        if (place < 2 * w.cap) { b.leaf[place] = (unsigned short)k; b.leaf_par[place] = (unsigned short)code; }
-      } else if ((int)(where[k] & 0xFFFFu) < w.cap) {
-        b.par[where[k] & 0xFFFFu] = (unsigned short)code;
+        b.leaf[v >> 8] = (unsigned short)k;
+        b.leaf_par[v >> 8] = (unsigned short)code;
+      } else {
+        b.par[v & 0xFFFFu] = (unsigned short)code;
       }
     }
-    __syncthreads();
   }
+  // (All clusters' or none: one that deals anew keeps its lists where these would be.)
   for (int part = tid; part < parts; part += nt) {
-    const int internal = loads->nodes[part] & 0xFFFF, deep = loads->nodes[part] >> 16, leaves = loads->depth[part];
-    const bool good = forest ? fits && internal <= w.cap && leaves <= 2 * w.cap : true;
-    *saved_at(w, part).head = good ? make_int4(deep, internal, leaves, parts) : make_int4(0, 0, 0, 0);
+    const int nodes = loads->nodes[part], depth = loads->depth[part];
+    *saved_at(w, part).head = !forest || fits ? make_int4(depth >> 16, nodes & 0xFFFF, depth & 0xFFFF, parts | nodes >> 16 << 8) : make_int4(0, 0, 0, 0);
   }
 }
 // All threads (of a small block each looks at several headers); false: there is nothing to load.  Of the child table only the entries of the cluster's internal nodes are filled.
 // (The first entries are asked for together with the headers.)
 __device__ __forceinline__ bool load_walk(const SavedWalks& w, const WalkCosts& costs, int n, int n_roots, const TreesSmem& s, float* sm, int part, int parts,
                                           bool choose, TreeLoads* loads, Walk* walk) {
-  const SavedBlock b = saved_at(w, part);
+  SavedBlock b = saved_at(w, part);
+  int cap = w.cap;
   struct Entry { unsigned kids; unsigned short list, par, start, leaf, leaf_par; };
   auto read = [&](int q) {
-    const int i = min(q, w.cap - 1), l = min(q, 2 * w.cap - 1);
-    return Entry{b.kids[i], b.list[i], b.par[i], b.start[min(q, w.cap)], b.leaf[l], b.leaf_par[l]};
+    const int i = min(q, cap - 1), l = min(q, 2 * cap - 1);
+    return Entry{b.kids[i], b.list[i], b.par[i], b.start[min(q, cap)], b.leaf[l], b.leaf_par[l]};
   };
   Entry e = read(threadIdx.x);
   bool ok = true;
 #pragma unroll 1
   for (int q = threadIdx.x; q < parts; q += blockDim.x) {
     const int4 head = *saved_at(w, q).head;
-    ok = ok && head.w == parts;
+    ok = ok && (head.w & 255) == parts;
     loads->nodes[q] = head.y;
     loads->depth[q] = head.x;
-    if (q == part) { *walk = Walk{head.x, head.y, head.z}; loads->win = 1; }
+    if (q == part) { *walk = Walk{head.x, head.y, head.z}; loads->win = 1; loads->longer = head.w >> 8; }
   }
   if (!__syncthreads_and(ok)) return false;
   if (choose) {
@@ -584,6 +605,11 @@ __device__ __forceinline__ bool load_walk(const SavedWalks& w, const WalkCosts& 
     __syncthreads();
   }
   const Walk have = *walk;
+  if (__builtin_expect(loads->longer != 0 && have.leaves > 0, 0)) {   // (none: the outcome is the whole GPU)
+    b = longer_at(w, parts, loads->longer, have.leaves);
+    cap = have.leaves;
+    e = read(threadIdx.x);
+  }
 #pragma unroll 1
   for (int q = threadIdx.x; q < have.leaves || q <= have.internal;) {
     if (q < have.internal) {

@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import treelstm_oracle as orc
-from paper_1809_00832_b200 import binding, forests as fg
+from paper_1809_00832_b200 import binding, forests as fg, trace
 from tests import util
 
 pytestmark = pytest.mark.gpu
@@ -504,3 +504,24 @@ def test_rows_that_the_kernel_ahead_numbers(H, trees):
         ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
                                      params.bc, labels)
         _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("H,kind,kept", [(150, "planned", True), (150, "one tree", True), (20, "one tree", True), (20, "more nodes than are planned ahead", True),
+                                         (20, "more depths than are planned ahead", False)])
+def test_lists_of_the_forward_are_kept_for_the_backward(H, kind, kept):
+    """planned beside the leaves, behind the clusters' own blocks where one cluster has all of them, and by the clusters themselves where the planning CTA has no
+    room: the backward plans nothing itself (trace build: that would leave a stamp), unless lists that clusters have planned are longer than their blocks"""
+    rng = np.random.default_rng(301)
+    params = fg.draw_params(rng, H, 12, 40, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    shapes = {"planned": [fg.random_split_shape(rng, int(k)) for k in range(2, 40)], "one tree": [fg.left_chain_shape(300)],
+              "more nodes than are planned ahead": [fg.left_chain_shape(29)] * 300,
+              "more depths than are planned ahead": [fg.left_chain_shape(400)] + [fg.left_chain_shape(2)] * 200}[kind]
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes, rng, 40), rng)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32", variant="trace")
+    model._workspace(forest.n_nodes, True).zero_()
+    _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
+    setup = trace.read_trace(model, 1)[trace.LEVELS - 1]
+    assert setup[3] > 0 and (setup[6] == 0) == kept                       # (dealt; depth 255 of a chain shares this row's first six slots)

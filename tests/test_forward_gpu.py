@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from oracle import treelstm_oracle as orc
-from paper_1809_00832_b200 import binding, forests as fg
+from paper_1809_00832_b200 import binding, forests as fg, trace
 from tests import util
 
 pytestmark = pytest.mark.gpu
@@ -387,4 +387,25 @@ def test_fp32_lists_of_more_nodes_than_climb_at_once(shapes):
     order = orc.schedule(forest.left, forest.right)[3]
     h, c, _ = orc.forward_iterative(forest.left, forest.right, forest.token, params.emb, params.W, params.b, order)
     res = util.gpu_forward(util.make_model(params, "fp32"), forest, binding.PERSISTENT)
+    assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
+
+
+@pytest.mark.parametrize("save", [0, binding.SAVE_FOR_BACKWARD])
+@pytest.mark.parametrize("H,kind", [(150, "chain 86"), (150, "chain 200"), (256, "balanced 256"), (24, "random 120"), (24, "chain 1100"), (20, "chain 8192"), (64, "three long")])
+def test_fp32_lists_of_one_or_a_few_longer_trees_are_planned_ahead(H, kind, save):
+    """one cluster's lists may hold the whole forest, and one tree's depths are all there are: no cluster plans for itself behind the leaves
+    (trace build: that would leave a stamp), and the states are the oracle's"""
+    rng = np.random.default_rng(16)
+    params = fg.draw_params(rng, H, 9, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    shape, _, k = kind.partition(" ")
+    shapes = {"chain": lambda: [fg.left_chain_shape(int(k))], "balanced": lambda: [fg.balanced_shape(int(k))], "random": lambda: [fg.random_split_shape(rng, int(k))],
+              "three": lambda: [None, fg.left_chain_shape(150), fg.random_split_shape(rng, 200), fg.random_split_shape(rng, 3)]}[shape]()
+    forest, _ = fg.permute_node_ids(fg.forest_from_shapes(shapes, rng, 60), rng)
+    model = util.make_model(params, "fp32", variant="trace")
+    model._workspace(forest.n_nodes, bool(save)).zero_()
+    res = util.gpu_forward(model, forest, binding.PERSISTENT | save)
+    setup = trace.read_trace(model, 0)[trace.LEVELS - 1]
+    assert setup[2] > 0 and setup[5] == 0                                 # (lists there; no child table of the cluster's own)
+    order = orc.schedule(forest.left, forest.right)[3]
+    h, c, _ = orc.forward_iterative(forest.left, forest.right, forest.token, params.emb, params.W, params.b, order)
     assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
