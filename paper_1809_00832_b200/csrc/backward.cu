@@ -1070,10 +1070,9 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
 // gradient.  What is left is latency: 10 - 14 k cycles of a narrow wavefront (3.3 k grid barrier, 3.5 k gate gradients, 2.5 k MMAs, 4 k
 // adds), 30 k of one of 300 nodes, 70 k of one of 2.5 k; 340 us in all (ncu, cold caches) for 14.6 k nodes, 19 wavefronts.
 constexpr int kWideSmem = 2 * kSpStageBytes + 1024, kWideThreads = 512;
-// A wavefront of up to kDirectRows nodes, one tile of them, forms its gate gradients where the tensor core reads them.  Two tiles have more blocks than
-// there are CTAs, and a CTA forms two, 17 k cycles where gradients through the images and a barrier take 12 k: wavefronts of 129 to 256 nodes 33 k -> 27 k
-// (H = 256; step of 256 sentences 598 -> 592 us).
-constexpr int kDirectRows = 128, kWideOffCache = 512;
+// A wavefront of one tile of nodes forms its gate gradients where the tensor core reads them, which saves the images and a grid barrier; every tile of outputs
+// forms them again.  Two tiles of nodes: wide_direct_rows.  Where a CTA has two blocks of them (H > 224) it does not pay: 33 k cycles, through the images 27 k.
+constexpr int kWideOffCache = 512;
 struct WideArgs {
   const int* level_offset;
   long long wait_limit;
@@ -1086,10 +1085,19 @@ struct WideArgs {
 struct WidePlan {
   int begin, end, base, leaf, direct, to, kbs, span, per, total, skip_first, skip;
 };
-__device__ __forceinline__ WidePlan wide_plan(int begin, int end, int leaf, int H, int E, int grid) {
+// The widest wavefront that is formed in place: two tiles of nodes if no CTA has two blocks, loads are of 16 bytes, and rows are whole lines of 128 bytes, so that what is formed
+// again reads no parts of more lines, or so short that there is little to it.  Backward passes with 14 wavefronts of 190 to 200 nodes, in place | through the images, us:
+// whole lines H = 96 361 | 372, 128 367 | 379, 160 393 | 412, 192 434 | 458, 224 463 | 480 (64, one tile of outputs and few CTAs either way, 334 | 332); short ones
+// H = 8 402 | 412, 16 360 | 377, 32 353 | 365; others H = 40 380 | 376, 100 483 | 466, 120 409 | 394, 144 410 | 408, 168 434 | 423, 176 418 | 421, 200 479 | 466,
+// 208 474 | 480; loads of 4 bytes H = 30 401 | 394, 150 557 | 468; two blocks a CTA H = 232 575 | 494, 256 518 | 485.  With 130 and 256 nodes the same, 1 to 5 % either way.
+__device__ __forceinline__ int wide_direct_rows(int H, int grid, bool vec_h) {
+  const int to = (2 * H + 127) / 128;
+  return vec_h && (H <= 32 || (H % 32 == 0 && to > 1)) && 2 * to * wsp_kblocks(H) <= grid ? 2 * kSpTile : kSpTile;
+}
+__device__ __forceinline__ WidePlan wide_plan(int begin, int end, int leaf, int H, int E, int grid, int direct_rows) {
   WidePlan w;
   w.begin = begin; w.end = end; w.leaf = leaf;
-  w.direct = !leaf && end - begin <= kDirectRows;
+  w.direct = !leaf && end - begin <= direct_rows;
   w.base = w.direct ? begin : begin & ~63;
   w.to = ((leaf ? E : 2 * H) + 127) / 128;
   const int tiles = (end - w.base + 127) / 128 * w.to, gp = gate_pitch(H);
@@ -1329,6 +1337,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   const int n_leaves = p.n_leaves, wsp_kb = wsp_kblocks(H);
   // 16-byte accesses to rows of H (and E): whether every row starts on a 16-byte boundary
   const bool vec_h = H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.h) | reinterpret_cast<uintptr_t>(p.c)) & 15) == 0;
+  const int direct_rows = wide_direct_rows(H, grid, vec_h);
   const bool vec_e = E % 4 == 0 && (reinterpret_cast<uintptr_t>(p.dEmb_rows) & 15) == 0;
   const bool vec_x = vec_h && E % 4 == 0 && (reinterpret_cast<uintptr_t>(p.emb) & 15) == 0;
 #ifdef TREELSTM_TRACE
@@ -1404,7 +1413,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
     return true;
   };
   WidePlan w;
-  if (n_levels > 0) w = wide_plan(level_begin(n_levels - 1), level_begin(n_levels), n_levels == 1, H, E, grid);
+  if (n_levels > 0) w = wide_plan(level_begin(n_levels - 1), level_begin(n_levels), n_levels == 1, H, E, grid, direct_rows);
   for (int lvl = n_levels - 1; lvl >= 0 && ok; --lvl) {
     TL_STAMP(trace, lvl, 0);
     uint32_t early = 0;                                  // (thread 0)
@@ -1529,7 +1538,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
       chunks_done += grid - busy;
     }
     if (lvl == 0) break;
-    w = wide_plan(level_begin(lvl - 1), level_begin(lvl), lvl == 1, H, E, grid);
+    w = wide_plan(level_begin(lvl - 1), level_begin(lvl), lvl == 1, H, E, grid, direct_rows);
     if (w.direct) {                                      // what does not depend on the wavefront above, while the barrier is pending
       const int lo = blockIdx.x * w.per;
       if (lo < w.total) {

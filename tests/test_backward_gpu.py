@@ -525,3 +525,17 @@ def test_lists_of_the_forward_are_kept_for_the_backward(H, kind, kept):
     _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
     setup = trace.read_trace(model, 1)[trace.LEVELS - 1]
     assert setup[3] > 0 and (setup[6] == 0) == kept                       # (dealt; depth 255 of a chain shares this row's first six slots)
+
+
+@pytest.mark.parametrize("H,chains", [(64, 128), (96, 129), (150, 128), (224, 128), (224, 129), (256, 129)])
+def test_wavefronts_of_one_and_two_tiles(H, chains):
+    """wavefronts of 128, 129 to 192, 256 and 257 nodes in a forest that the tree kernels leave: operands formed at the tensor core (one tile; two, where the
+    rows are whole lines and no CTA forms two blocks) or stored first"""
+    rng = np.random.default_rng(400 + H + chains)
+    params = fg.draw_params(rng, H, 20, 50, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    forest = fg.forest_from_shapes([fg.left_chain_shape(12)] * chains + [fg.balanced_shape(1024)], rng, 50)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
