@@ -470,11 +470,14 @@ __global__ void __launch_bounds__(kT, 1) k_schedule_trees_tc(const __grid_consta
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     return;
   }
-  if ((int)blockIdx.x == cs && threadIdx.x == 0) {         // (nothing decided: the kernel behind, which comes up with what it needs unless it reads otherwise)
-    p.st->trees_fwd = 0;
-    __threadfence();
+  // (Nothing decided: the kernel behind, which comes up with what it needs unless it reads otherwise.  One thread speaks for its CTA, behind what it has stored.)
+  if (threadIdx.x == 0) {
+    if ((int)blockIdx.x == cs) {
+      p.st->trees_fwd = 0;
+      __threadfence();
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int rank = (int)cluster_rank(), part = (int)blockIdx.x / cs - 1, parts = (int)gridDim.x / cs - 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = f.n, H = p.H, Hp = p.Hp, Ep = p.Ep, gpc = p.gpc, U = 8 * gpc, U0 = rank * U;
