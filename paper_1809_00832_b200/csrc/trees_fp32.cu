@@ -465,12 +465,12 @@ __global__ void __launch_bounds__(kFwdT, 1) k_trees_forward(const __grid_constan
 }
 
 // ---- TreeLSTM leaves ------------------------------------------------------------------------------ //
-// Their states need no schedule, so this kernel runs beside the scheduler, over the whole GPU.  A CTA takes 64 consecutive node
-// ids, the leaves among them (about half), and 32 hidden units x the three gates a leaf has.  All operands of
+// Their states need no schedule, so this kernel runs beside the scheduler, over the whole GPU.  A CTA takes 32 to 64 consecutive node
+// ids (as few as give every SM some), the leaves among them (about half), and 32 hidden units x the three gates a leaf has.  All operands of
 // kLeafK contraction indices are asked for at once - the weights as one bulk copy out of an image kept for it, the
 // embedding rows through registers - because the kernel is bound by the latency of its loads: in chunks of 32 indices,
 // each a round trip behind the one before, 25 trees (H = 150, E = 300) took 43 us with cold caches, this way 17.
-// A warp takes a quarter of the rows (8, 10, 12 or 16) and a quarter of the contraction: rows read as broadcasts, weights one
+// A warp takes a quarter of the rows (4, 5, 7, 8, 10, 12 or 16) and a quarter of the contraction: rows read as broadcasts, weights one
 // word per lane, 96 multiply-adds per 20 reads.  (Half of the rows and twice the quarters of the contraction, 48 per 16 reads,
 // was bound by shared memory: 15 k cycles for 32 leaves.)  The quarters meet in shared memory, every warp finishes some rows.
 constexpr int kLeafT = 512, kLeafU = 32, kLeafIds = 64, kLeafK = 320;
@@ -589,7 +589,9 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
   }
   __syncthreads();
   const int count = s_count, quarter = warp >> 2;
-  const int rpt = count <= 16 ? 4 : (count <= 28 ? 7 : (count <= 32 ? 8 : (count <= 40 ? 10 : (count <= 48 ? 12 : 16)))), row0 = (warp & 3) * rpt;
+  // Rows of a warp.  32 ids, what a CTA takes of a small forest, hold 16 leaves and a few more or less.  A size is code of its own that each SM fetches once: with one for 24
+  // leaves as well, 25 sentences, H = 150, took 57.1 us and not 56.4; without the one for 20, one sentence 36.5 and not 35.4, five 50.5 and not 49.5.
+  const int rpt = count <= 16 ? 4 : (count <= 20 ? 5 : (count <= 28 ? 7 : (count <= 32 ? 8 : (count <= 40 ? 10 : (count <= 48 ? 12 : 16))))), row0 = (warp & 3) * rpt;
   const int u = min(u0 + lane, H - 1);
   const float bi = __ldg(p.b + u), bo = __ldg(p.b + 3 * H + u), bu = __ldg(p.b + 4 * H + u);
   float acc[16][3] = {};
@@ -620,6 +622,7 @@ __global__ void __launch_bounds__(kLeafT) k_leaves_fp32(const __grid_constant__ 
     if (__syncthreads_or(!ok)) { ok = false; break; }
     if (row0 < count) {
       if (rpt == 4) leaf_rows<4>(As, Ws, pitch, nk, row0, quarter, lane, acc);
+      else if (rpt == 5) leaf_rows<5>(As, Ws, pitch, nk, row0, quarter, lane, acc);
       else if (rpt == 7) leaf_rows<7>(As, Ws, pitch, nk, row0, quarter, lane, acc);
       else if (rpt == 8) leaf_rows<8>(As, Ws, pitch, nk, row0, quarter, lane, acc);
       else if (rpt == 10) leaf_rows<10>(As, Ws, pitch, nk, row0, quarter, lane, acc);

@@ -409,3 +409,14 @@ def test_fp32_lists_of_one_or_a_few_longer_trees_are_planned_ahead(H, kind, save
     order = orc.schedule(forest.left, forest.right)[3]
     h, c, _ = orc.forward_iterative(forest.left, forest.right, forest.token, params.emb, params.W, params.b, order)
     assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
+
+
+@pytest.mark.parametrize("leaves", [16, 17, 20, 21, 28, 29, 32, 33])
+def test_fp32_leaves_of_one_cta(leaves):
+    """as many leaves as a warp's rows hold, and one more"""
+    rng = np.random.default_rng(17)
+    params = fg.draw_params(rng, 33, 321, 60, emb_dist="normal", emb_scale=0.3, w_scale=0.1)
+    forest = fg.forest_from_shapes([None] * leaves, rng, 60)
+    h, c, _ = orc.forward_recursive(forest.left, forest.right, forest.token, params.emb, params.W, params.b)
+    res = util.gpu_forward(util.make_model(params, "fp32"), forest, binding.PERSISTENT)
+    assert util.max_abs(res["h"], h) < util.TOL["fp32"] and util.max_abs(res["c"], c) < util.TOL["fp32"]
