@@ -1,6 +1,8 @@
 """Parity of the CUDA training step (forward + backward through structure, via the C ABI) against
 the fp64 oracle: loss and every gradient group within 1e-4 max-abs and within 2e-5 of the group's
 own largest entry (several groups of the full-size workload lie below 1e-4 altogether)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -539,3 +541,35 @@ def test_wavefronts_of_one_and_two_tiles(H, chains):
                                  params.bc, labels)
     model = util.make_model(params, "fp32")
     _compare(_train_step(model, forest, labels, binding.PERSISTENT), ref, util.TOL["fp32"])
+
+
+@pytest.mark.parametrize("words", [1, 2, 3])
+@pytest.mark.parametrize("H,E,shapes", [(40, 24, "sentences"), (42, 26, "sentences"), (33, 23, "sentences"), (40, 24, "wide"), (300, 20, "sentences")])
+def test_gradients_in_memory_of_any_alignment(H, E, shapes, words):
+    """outputs that start 4, 8 and 12 bytes behind a 16-byte boundary (rows added in pieces of one, two and four floats, by the address and the
+    width): behind the tree kernels, from the images of a wide forest, and where neither applies; what lies around them stays"""
+    rng = np.random.default_rng(500 + H)
+    params = fg.draw_params(rng, H, E, 70, emb_dist="normal", emb_scale=0.3, w_scale=0.7 / np.sqrt(H), n_classes=3)
+    forest = fg.forest_from_shapes([fg.balanced_shape(512)] * 2 if shapes == "wide" else [fg.random_split_shape(rng, k) for k in (20, 9, 1, 14)], rng, 70)
+    labels = rng.integers(0, 3, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc,
+                                 params.bc, labels)
+    model = util.make_model(params, "fp32")
+    arrays = [util.to_dev(a) for a in (forest.left, forest.right, forest.token)]
+    on_device = util.to_dev(labels)
+    out = model.forward(*arrays, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+    shape = dict(dW=(E + 2 * H, 5 * H), db=(5 * H,), dWc=(H, 3), dbc=(3,), dEmb_rows=(forest.n_leaves, E))
+    whole = {k: torch.full((int(np.prod(v)) + 8,), 7.0, device="cuda") for k, v in shape.items()}
+    at = {k: v[words:words + int(np.prod(shape[k]))] for k, v in whole.items()}
+    loss, touched, count = torch.empty(1, device="cuda"), *(torch.empty(k, dtype=torch.int32, device="cuda") for k in (forest.n_leaves, 1))
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    rc = model.lib.treelstm_backward(model.handle, ptr(on_device), ptr(loss), ptr(at["dW"]), ptr(at["db"]), ptr(at["dWc"]), ptr(at["dbc"]), ptr(touched),
+                                     ptr(at["dEmb_rows"]), ptr(count), binding._stream())
+    assert rc == binding.OK and model.status_sync() == binding.OK
+    for k, v in whole.items():
+        v = v.cpu().numpy()
+        assert (v[:words] == 7.0).all() and (v[words + int(np.prod(shape[k])):] == 7.0).all(), k
+    res = {k: v.cpu().numpy().reshape(shape[k]) for k, v in at.items()}
+    res.update(loss=loss.cpu().numpy(), touched_ids=touched.cpu().numpy(), n_touched=count.cpu().numpy())
+    _compare(res, ref, util.TOL["fp32"])
+    del out

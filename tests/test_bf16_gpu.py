@@ -504,3 +504,62 @@ def test_forests_that_only_clusters_can_take(H, shapes):
     with pytest.raises(binding.TreeLSTMError) as err:
         model.forward(*arrays)
     assert err.value.code == binding.ERR_INVALID_FOREST
+
+
+@pytest.mark.parametrize("H", [40, 150, 256])
+@pytest.mark.parametrize("shapes", [[None], [2, 30], [12, 1, 19], [31, None, 1, 1], [33]])
+def test_training_step_behind_a_forward_of_one_launch(H, shapes):
+    """up to 64 nodes nothing follows the scheduler's launch, and the backward's first kernel is the next on the stream (33 leaves: 65 nodes)"""
+    rng = np.random.default_rng(83)
+    params = fg.draw_params(rng, H, 24, 100, emb_dist="normal", emb_scale=0.3, w_scale=0.08, n_classes=5)
+    forest = fg.forest_from_shapes([k if k is None else fg.random_split_shape(rng, k) for k in shapes], rng, 100)
+    forest, _ = fg.permute_node_ids(forest, rng)
+    labels = rng.integers(0, 5, size=forest.n_nodes).astype(np.int32)
+    ref = orc.loss_and_gradients(forest.left, forest.right, forest.token, params.emb, params.W, params.b, params.Wc, params.bc, labels)
+    model = util.make_model(params, "bf16")
+    arrays = [util.to_dev(a) for a in (forest.left, forest.right, forest.token)]
+    for _ in range(2):
+        model.forward(*arrays, flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD, check=False)
+        assert (model.last_launch_count() == 1) == (forest.n_nodes <= 64)
+        grads = model.backward(util.to_dev(labels), forest.n_leaves)
+        torch.cuda.synchronize()
+        util.compare_training_step({k: v.cpu().numpy() for k, v in grads.items()}, ref, util.TOL["bf16"], util.REL["bf16"])
+
+
+@pytest.mark.parametrize("H", [64, 150, 256])
+def test_calls_that_start_while_the_last_one_runs(H):
+    """forests of up to 64 nodes let the next call's scheduler come up at once: different forests in turn, small and large, forward alone and with a backward, in one
+    context and workspace with no wait by the host, so that a control block, level table or order written too early would be another forest's"""
+    rng = np.random.default_rng(89)
+    params = fg.draw_params(rng, H, 24, 100, emb_dist="normal", emb_scale=0.3, w_scale=0.08, n_classes=5)
+    kinds = [[fg.left_chain_shape(30)], [fg.balanced_shape(16), None], [fg.random_split_shape(rng, 40) for _ in range(60)],
+             [fg.random_split_shape(rng, 3) for _ in range(9)], [fg.random_split_shape(rng, 30) for _ in range(300)], [None] * 5]
+    forests = [fg.permute_node_ids(fg.forest_from_shapes(k, rng, 100), rng)[0] for k in kinds]
+    refs = [util.gpu_forward(util.make_model(params, "bf16"), f, binding.PERSISTENT) for f in forests]
+    model = util.make_model(params, "bf16")
+    arrays = [[util.to_dev(a) for a in (f.left, f.right, f.token)] for f in forests]
+    labels = [util.to_dev(rng.integers(0, 5, size=f.n_nodes).astype(np.int32)) for f in forests]
+    model._workspace(max(f.n_nodes for f in forests), True)              # (one for all: none is replaced while a call runs)
+    grad_refs = {}
+    for k in (0, 1, 3):
+        model.forward(*arrays[k], flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD)
+        grad_refs[k] = model.backward(labels[k], forests[k].n_leaves)
+    turns = [0, 1, 0, 3, 1, 5, 2, 0, 4, 1, 3, 5, 0, 2, 2, 1, 4, 4, 3, 0]
+    results = [(k, model.forward(*arrays[k], check=False)) for k in turns]
+    grads = []
+    for k in (0, 1, 3, 1, 0):                                            # forward, then backward (which waits), a forward of another forest ahead of them
+        results.append((3, model.forward(*arrays[3], check=False)))
+        results.append((k, model.forward(*arrays[k], flags=binding.PERSISTENT | binding.SAVE_FOR_BACKWARD, check=False)))
+        grads.append((k, model.backward(labels[k], forests[k].n_leaves)))
+    assert model.status_sync() == binding.OK
+    for k, out in results:
+        levels = int(out["n_levels"].item())
+        assert levels == refs[k]["n_levels"]
+        for key in ("h", "c", "level", "order"):
+            np.testing.assert_array_equal(out[key].cpu().numpy(), refs[k][key])
+        np.testing.assert_array_equal(out["level_offset"].cpu().numpy()[:levels + 1], refs[k]["level_offset"][:levels + 1])
+    for k, got in grads:
+        want = {key: v.cpu().numpy() for key, v in grad_refs[k].items()}
+        util.compare_training_step({key: v.cpu().numpy() for key, v in got.items()}, dict(
+            want, loss=float(want["loss"][0]), touched_ids=want["touched_ids"][:int(want["n_touched"][0])],
+            dEmb_rows=want["dEmb_rows"][:int(want["n_touched"][0])]), util.TOL["fp32"], util.REL["fp32"])
