@@ -374,50 +374,35 @@ __device__ __forceinline__ void deal_trees(const ForestIn& p, const WalkCosts& c
 
 // What the clusters of a forward walk, in the workspace: planned ahead of them by one CTA (plan_walks), or kept by them for the backward pass of the same forest,
 // whose clusters would otherwise work it out again beside k_bwd_begin (34 k cycles there for 25 sentences, H = 150).  One block per cluster:
-// header, then children, node and caller of every row, starts of the depths, leaves and their callers.  A block has room for four times the average
-// (`cap`).  One tree's lists are one cluster's, whatever their length: the planning CTA, which knows all of them, puts longer ones behind the blocks, one after
+// header, then children, node and caller of every row, leaves and their callers, starts of the depths.  A block has room for four times the average
+// (`cap` rows).  One tree's lists are one cluster's, whatever their length: the planning CTA, which knows all of them, puts longer ones behind the blocks, one after
 // the other, and the header says where.  (Left to the clusters themselves, behind the leaves, the plan of one chain of 200 leaves
 // had its forward take 656 us and not 604, H = 150, and 321 and not 270, H = 24.)  A cluster that keeps its own lists says that it has none if they are longer, and the backward pass deals anew.
 struct SavedWalks { unsigned char* at; int cap; };
 __host__ __device__ inline int saved_cap(int n, int parts) { return min(n / 2 + 2, 4 * (n / 2 / parts) + 64); }
 __host__ __device__ inline size_t saved_block(int cap) { return (size_t)(16 + 18 * cap + 4 + 15) / 16 * 16; }
 __host__ __device__ inline size_t longer_bytes(int n, int parts) { return 18 * (size_t)n + 48 * (size_t)parts; }   // of all longer blocks: each has room for as many rows as the cluster has leaves
-struct SavedBlock { int4* head; unsigned* kids; unsigned short *list, *par, *start, *leaf, *leaf_par; };
-__device__ __forceinline__ SavedBlock saved_at(unsigned char* at, int cap) {
-  SavedBlock b;
-  b.head = reinterpret_cast<int4*>(at);
-  b.kids = reinterpret_cast<unsigned*>(at + 16);
-  b.list = reinterpret_cast<unsigned short*>(b.kids + cap);
-  b.par = b.list + cap;
-  b.leaf = b.par + cap;
-  b.leaf_par = b.leaf + 2 * cap;
-  b.start = b.leaf_par + 2 * cap;
-  return b;
-}
-__device__ __forceinline__ SavedBlock saved_at(const SavedWalks& w, int part) { return saved_at(w.at + saved_block(w.cap) * part, w.cap); }
-// `where`: 16-byte units behind the blocks, plus one
-__device__ __forceinline__ SavedBlock longer_at(const SavedWalks& w, int parts, int where, int leaves) {
-  return saved_at(w.at + saved_block(w.cap) * parts + 16 * (size_t)(where - 1), leaves);
-}
+struct SavedBlock {
+  unsigned char* at;
+  int cap;
+  __device__ __forceinline__ int4* head() const { return reinterpret_cast<int4*>(at); }   // depths, rows, leaves, clusters | 16-byte units to where the rest is << 8 (zero: here)
+  __device__ __forceinline__ uint2* row(int q) const { return reinterpret_cast<uint2*>(at + 16) + q; }   // children, node | caller << 16
+  __device__ __forceinline__ unsigned* leaf(int q) const { return reinterpret_cast<unsigned*>(at + 16 + 8 * (size_t)cap) + q; }   // node | caller << 16
+  __device__ __forceinline__ unsigned short* start(int d) const { return reinterpret_cast<unsigned short*>(at + 16 + 16 * (size_t)cap) + d; }
+};
+__device__ __forceinline__ SavedBlock saved_at(const SavedWalks& w, int part) { return {w.at + saved_block(w.cap) * part, w.cap}; }
 // All threads, with the cluster's lists in shared memory.
 __device__ __forceinline__ void save_walk(const SavedWalks& w, const TreesSmem& s, const float* sm, int part, int parts, const Walk& walk) {
   const SavedBlock b = saved_at(w, part);
   const bool fits = walk.internal <= w.cap && walk.leaves <= 2 * w.cap;
-  if (threadIdx.x == 0) *b.head = make_int4(walk.depths, walk.internal, walk.leaves, fits ? parts : 0);
+  if (threadIdx.x == 0) *b.head() = make_int4(walk.depths, walk.internal, walk.leaves, fits ? parts : 0);
   if (!fits) return;
   const unsigned short* list = reinterpret_cast<const unsigned short*>(sm + s.list);
 #pragma unroll 1
   for (int q = threadIdx.x; q < walk.leaves || q <= walk.internal; q += blockDim.x) {
-    if (q < walk.internal) {
-      b.kids[q] = reinterpret_cast<const unsigned*>(sm + s.kids)[list[q]];
-      b.list[q] = list[q];
-      b.par[q] = reinterpret_cast<const unsigned short*>(sm + s.par)[q];
-    }
-    if (q <= walk.depths) b.start[q] = reinterpret_cast<const unsigned short*>(sm + s.start)[q];
-    if (q < walk.leaves) {
-      b.leaf[q] = reinterpret_cast<const unsigned short*>(sm + s.leaf)[q];
-      b.leaf_par[q] = reinterpret_cast<const unsigned short*>(sm + s.leaf_par)[q];
-    }
+    if (q < walk.internal) *b.row(q) = make_uint2(reinterpret_cast<const unsigned*>(sm + s.kids)[list[q]], list[q] | (unsigned)reinterpret_cast<const unsigned short*>(sm + s.par)[q] << 16);
+    if (q <= walk.depths) *b.start(q) = reinterpret_cast<const unsigned short*>(sm + s.start)[q];
+    if (q < walk.leaves) *b.leaf(q) = reinterpret_cast<const unsigned short*>(sm + s.leaf)[q] | (unsigned)reinterpret_cast<const unsigned short*>(sm + s.leaf_par)[q] << 16;
   }
 }
 // The same from one CTA for all clusters, ahead of the kernel that walks (TreeLSTM forward: beside the leaves).  Behind deal_by_size, whose tables and
@@ -434,7 +419,7 @@ __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const un
   const int busy = max(1, min(parts, n - 2 * loads->internal));   // clusters with a tree
   constexpr unsigned kNone = 0xFFFFFFFFu;
   __syncthreads();
-  for (int q = tid; q < parts; q += nt) loads->nodes[q] = loads->depth[q] = 0;   // internal nodes | place behind the blocks << 16; leaves | depths << 16
+  for (int q = tid; q < parts; q += nt) loads->nodes[q] = loads->depth[q] = 0;   // 16-byte units to the lists, leaves
   if (tid == 0) loads->internal = loads->longer = 0;         // deepest; 16-byte units in use behind the blocks
   __syncthreads();
   bool fits = wanted && forest && n + busy <= words && parts < 256;   // (as many depths as there is room for: below)
@@ -503,16 +488,14 @@ __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const un
       if (lf) where[k] = (v & 255u) | (unsigned)place << 8;
     }
     __syncthreads();
-    for (int part = tid; part < busy; part += nt) {          // lists that may be longer than a block (a tree has one more leaf than internal nodes)
+    // (a tree has one more leaf than rows)
+    const int units = (int)(saved_block(w.cap) / 16);
+    for (int part = tid; part < parts; part += nt) {
       const int leaves = loads->depth[part];
-      if (leaves > w.cap) loads->nodes[part] = (atomicAdd(&loads->longer, (int)(saved_block(leaves) / 16)) + 1) << 16;
+      loads->nodes[part] = leaves > w.cap ? parts * units + atomicAdd(&loads->longer, (int)(saved_block(leaves) / 16)) : part * units;
     }
     __syncthreads();
-    const bool longer = loads->longer != 0;
-    auto block_of = [&](int part) {
-      const int place = longer ? loads->nodes[part] >> 16 : 0;
-      return place ? longer_at(w, parts, place, loads->depth[part] & 0xFFFF) : saved_at(w, part);
-    };
+    auto block_of = [&](int part) { return SavedBlock{w.at + 16 * (size_t)loads->nodes[part], max(w.cap, loads->depth[part])}; };
     for (int part = tid >> 5; part < busy; part += nt >> 5) {
       const SavedBlock b = block_of(part);
       int sum = 0, deep = 0;
@@ -525,68 +508,52 @@ __device__ __forceinline__ void plan_walks(int n, const unsigned* kids, const un
           if (lane >= e) incl += x;
         }
         if (d < depths) next[part * depths + d] = sum + incl - v;
-        if (v) b.start[d] = (unsigned short)(sum + incl - v);
+        if (v) *b.start(d) = (unsigned short)(sum + incl - v);
         sum += __shfl_sync(kFull, incl, 31);
         deep += __popc(__ballot_sync(kFull, v != 0));        // (depths have no gaps)
       }
       if (lane == 0) {
-        b.start[deep] = (unsigned short)sum;
-        loads->depth[part] |= deep << 16;
-        loads->nodes[part] |= sum;
+        *b.start(deep) = (unsigned short)sum;
+        const int at = loads->nodes[part];
+        *saved_at(w, part).head() = make_int4(deep, sum, loads->depth[part], parts | (at == part * units ? 0 : at) << 8);
       }
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int k = tid; k < n; k += nt) {
-      const unsigned v = where[k], kd = kids[k];
-      if (v == kNone || is_leaf(kd)) continue;
-      const unsigned part = v & 255u;
-      const int q = atomicAdd(next + part * depths + (v >> 8), 1);
-      where[k] = (unsigned)q | part << 16;
-      const SavedBlock b = block_of((int)part);
-      b.list[q] = (unsigned short)k;
-      b.kids[q] = kd;
     }
     __syncthreads();
 #pragma unroll 1
     for (int k = tid; k < n; k += nt) {
       const unsigned v = where[k];
+      if (v == kNone || is_leaf(kids[k])) continue;
+      const unsigned part = v & 255u;
+      where[k] = (unsigned)atomicAdd(next + part * depths + (v >> 8), 1) | part << 16;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int k = tid; k < n; k += nt) {
+      const unsigned v = where[k], kd = kids[k];
       if (v == kNone) continue;
-      const bool lf = is_leaf(kids[k]);
       const int up = t.up[k];
       unsigned code = kNoCaller;
       if (up != k) code = 2u * (where[up] & 0xFFFFu) + (unsigned)((kids[up] & 0xFFFFu) != (unsigned)k);
-      const SavedBlock b = block_of((int)(lf ? v & 255u : v >> 16));
-      if (lf) {
-        b.leaf[v >> 8] = (unsigned short)k;
-        b.leaf_par[v >> 8] = (unsigned short)code;
-      } else {
-        b.par[v & 0xFFFFu] = (unsigned short)code;
-      }
+      const SavedBlock b = block_of((int)(is_leaf(kd) ? v & 255u : v >> 16));
+      if (is_leaf(kd)) *b.leaf((int)(v >> 8)) = (unsigned)k | code << 16;
+      else *b.row((int)(v & 0xFFFFu)) = make_uint2(kd, (unsigned)k | code << 16);
     }
   }
   // (All clusters' or none: one that deals anew keeps its lists where these would be.)
-  for (int part = tid; part < parts; part += nt) {
-    const int nodes = loads->nodes[part], depth = loads->depth[part];
-    *saved_at(w, part).head = !forest || fits ? make_int4(depth >> 16, nodes & 0xFFFF, depth & 0xFFFF, parts | nodes >> 16 << 8) : make_int4(0, 0, 0, 0);
-  }
+  for (int part = fits ? busy + tid : tid; part < parts; part += nt) *saved_at(w, part).head() = make_int4(0, 0, 0, !forest || fits ? parts : 0);
 }
 // All threads (of a small block each looks at several headers); false: there is nothing to load.  Of the child table only the entries of the cluster's internal nodes are filled.
 // (The first entries are asked for together with the headers.)
 __device__ __forceinline__ bool load_walk(const SavedWalks& w, const WalkCosts& costs, int n, int n_roots, const TreesSmem& s, float* sm, int part, int parts,
                                           bool choose, TreeLoads* loads, Walk* walk) {
   SavedBlock b = saved_at(w, part);
-  int cap = w.cap;
-  struct Entry { unsigned kids; unsigned short list, par, start, leaf, leaf_par; };
-  auto read = [&](int q) {
-    const int i = min(q, cap - 1), l = min(q, 2 * cap - 1);
-    return Entry{b.kids[i], b.list[i], b.par[i], b.start[min(q, cap)], b.leaf[l], b.leaf_par[l]};
-  };
+  struct Entry { uint2 row; unsigned leaf; unsigned short start; };
+  auto read = [&](int q) { return Entry{*b.row(min(q, b.cap - 1)), *b.leaf(min(q, 2 * b.cap - 1)), *b.start(min(q, b.cap))}; };
   Entry e = read(threadIdx.x);
   bool ok = true;
 #pragma unroll 1
   for (int q = threadIdx.x; q < parts; q += blockDim.x) {
-    const int4 head = *saved_at(w, q).head;
+    const int4 head = *saved_at(w, q).head();
     ok = ok && (head.w & 255) == parts;
     loads->nodes[q] = head.y;
     loads->depth[q] = head.x;
@@ -606,21 +573,20 @@ __device__ __forceinline__ bool load_walk(const SavedWalks& w, const WalkCosts& 
   }
   const Walk have = *walk;
   if (__builtin_expect(loads->longer != 0 && have.leaves > 0, 0)) {   // (none: the outcome is the whole GPU)
-    b = longer_at(w, parts, loads->longer, have.leaves);
-    cap = have.leaves;
+    b = {w.at + 16 * (size_t)loads->longer, have.leaves};
     e = read(threadIdx.x);
   }
 #pragma unroll 1
   for (int q = threadIdx.x; q < have.leaves || q <= have.internal;) {
     if (q < have.internal) {
-      reinterpret_cast<unsigned*>(sm + s.kids)[e.list] = e.kids;
-      reinterpret_cast<unsigned short*>(sm + s.list)[q] = e.list;
-      reinterpret_cast<unsigned short*>(sm + s.par)[q] = e.par;
+      reinterpret_cast<unsigned*>(sm + s.kids)[e.row.y & 0xFFFFu] = e.row.x;
+      reinterpret_cast<unsigned short*>(sm + s.list)[q] = (unsigned short)e.row.y;
+      reinterpret_cast<unsigned short*>(sm + s.par)[q] = (unsigned short)(e.row.y >> 16);
     }
     if (q <= have.depths) reinterpret_cast<unsigned short*>(sm + s.start)[q] = e.start;
     if (q < have.leaves) {
-      reinterpret_cast<unsigned short*>(sm + s.leaf)[q] = e.leaf;
-      reinterpret_cast<unsigned short*>(sm + s.leaf_par)[q] = e.leaf_par;
+      reinterpret_cast<unsigned short*>(sm + s.leaf)[q] = (unsigned short)e.leaf;
+      reinterpret_cast<unsigned short*>(sm + s.leaf_par)[q] = (unsigned short)(e.leaf >> 16);
     }
     q += blockDim.x;
     e = read(q);
