@@ -1067,8 +1067,8 @@ k_bwd_persistent(BwdParams p, const int* level_offset, long long wait_limit, int
 // (BwdImages, the layout the tensor core reads), and tiles of 128 positions x 128 outputs are multiplied with W split once
 // per set of weights: one thread asks for blocks (plain bulk copies of whole tiles), one issues the MMAs, sixteen warps
 // add the tile to the children's dh.  The leaves' dIn (their rows of dEmb) is one more such wavefront.  The images stay for the weight
-// gradient.  What is left is latency: 10 - 14 k cycles of a narrow wavefront (3.3 k grid barrier, 3.5 k gate gradients, 2.5 k MMAs, 4 k
-// adds), 30 k of one of 300 nodes, 70 k of one of 2.5 k; 340 us in all (ncu, cold caches) for 14.6 k nodes, 19 wavefronts.
+// gradient.  What is left is latency.  Cycles of a wavefront, H = 256, 14.3 k nodes: 15 - 20 k of one of 11 to 83 nodes (4 - 9 k gate gradients, 2.5 k MMAs, 1.2 k read
+// back, 4 k adds, 3.2 k grid barrier), 27 - 32 k of 130 to 460, 37 k of 960, 71 k of 2.4 k; 318 us in all (ncu, 19 wavefronts).
 constexpr int kWideSmem = 2 * kSpStageBytes + 1024, kWideThreads = 512;
 // A wavefront of one tile of nodes forms its gate gradients where the tensor core reads them, which saves the images and a grid barrier; every tile of outputs
 // forms them again.  Two tiles of nodes: wide_direct_rows.  Where a CTA has two blocks of them (H > 224) it does not pay: 33 k cycles, through the images 27 k.

@@ -1201,7 +1201,9 @@ int launch_trees(treelstm* ctx, TreesKernel kernel, const TreesParams& p, int th
 // among 24 sentences; TreeLSTM H = 64 to 256, TreeRNN 64 to 256, RNTN 16 and 32).  Forward / backward in us, clusters against
 // whole GPU: TreeLSTM H = 150, 25 sentences 100 / 163 against 170 / 298, chain of 1024 leaves 3 410 / 3 870 against 7 450 / 8 530,
 // balanced tree of 1024 leaves 945 / 848 against 166 / 240; TreeRNN H = 128, 25 sentences 51 / 112 against 351 / 361, balanced
-// tree of 8192 leaves 3 080 / 3 320 against 590 / 1 330.
+// tree of 8192 leaves 3 080 / 3 320 against 590 / 1 330.  Both ways have become faster since (TreeLSTM H = 150, 25 sentences 69 / 127 against 138 / 252, chain 3 220 / 3 820
+// against 7 340 / 8 890, balanced tree 908 / 768 against 151 / 212) and the constants are those of the fit: of 420 calls (TreeLSTM H = 64 to 256, TreeRNN 128, RNTN 32,
+// both directions, many of them near the border) 27 take more than 5 % longer than the better way, at most 24 %.
 WalkCosts walk_costs(int cell, int H, bool backward) {
   const float h = (float)H;
   if (cell == kLstm) {

@@ -1,9 +1,11 @@
 // Which trees a cluster takes and in which order it walks them: the pieces that every kernel whose clusters evaluate whole
 // trees shares (trees_fp32.cu; trees_tc.cu has a plan of its own and takes the tables, the ranking and the choice from here).
 //
-// A cluster needs the internal nodes of its trees by depth, deepest last, and for every node the row of its caller.  All
-// CTAs of all clusters work that out for themselves from the child arrays - no launch ahead, no exchange -, each the same
-// way, since the rows of a cluster's lists are addresses in the shared memory of all its CTAs:
+// A cluster needs the internal nodes of its trees by depth, deepest last, and for every node the row of its caller.  For a TreeLSTM forward one CTA of
+// the launch ahead works that out for all clusters, beside the leaves (plan_walks: 1 and 2 below, then nodes counted by cluster and depth), and a
+// backward pass reads what its forward has walked (load_walk).  Everywhere else, and where that CTA's tables do not hold the forest, all CTAs of all
+// clusters work it out for themselves from the child arrays, each the same way, since the rows of a cluster's lists are addresses in the shared
+// memory of all its CTAs:
 //   1. child table, caller of every node, a bit for every node that has a caller           (load_kids)
 //   2. every internal node climbs to its root; trees ranked by size and dealt out to the clusters there and back (0 .. Q-1,
 //      Q-1 .. 0, ...): the fullest cluster sets the time, and of 25 sentences on 15 clusters it held 85 to 96 nodes when trees

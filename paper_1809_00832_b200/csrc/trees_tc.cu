@@ -949,8 +949,7 @@ bool trees_tc_asked(const treelstm* ctx, int n, int flags) {
 }
 
 // A forest that the clusters leave has a depth of more than R nodes, or more nodes than their lists hold.  One of no more than R nodes has neither whatever
-// its shape, and the kernels behind, which would look and exit, are not launched: one sentence of 30 words from and to host arrays, H = 256, 53.0 -> 50.2 us
-// (45.9 with the scheduler's early start).
+// its shape, and the kernels behind, which would look and exit, are not launched: one sentence of 30 words from and to host arrays, H = 256, 53.0 -> 50.2 us.
 bool trees_tc_always_take(const treelstm* ctx, int n) { return n <= tt_layout(ctx->Hp, ctx->Ep, ctx->sf.groups_per_cta).R; }
 
 int launch_schedule_trees_tc(treelstm* ctx, int n, const int32_t* left, const int32_t* right, const int32_t* token, float* h, float* c, int32_t* level,
