@@ -1076,7 +1076,7 @@ constexpr int kWideOffCache = 512;
 struct WideArgs {
   const int* level_offset;
   long long wait_limit;
-  int after_trees;
+  int after_trees, direct_rows;
   BwdImages img;
 };
 
@@ -1090,7 +1090,7 @@ struct WidePlan {
 // whole lines H = 96 361 | 372, 128 367 | 379, 160 393 | 412, 192 434 | 458, 224 463 | 480 (64, one tile of outputs and few CTAs either way, 334 | 332); short ones
 // H = 8 402 | 412, 16 360 | 377, 32 353 | 365; others H = 40 380 | 376, 100 483 | 466, 120 409 | 394, 144 410 | 408, 168 434 | 423, 176 418 | 421, 200 479 | 466,
 // 208 474 | 480; loads of 4 bytes H = 30 401 | 394, 150 557 | 468; two blocks a CTA H = 232 575 | 494, 256 518 | 485.  With 130 and 256 nodes the same, 1 to 5 % either way.
-__device__ __forceinline__ int wide_direct_rows(int H, int grid, bool vec_h) {
+inline int wide_direct_rows(int H, int grid, bool vec_h) {
   const int to = (2 * H + 127) / 128;
   return vec_h && (H <= 32 || (H % 32 == 0 && to > 1)) && 2 * to * wsp_kblocks(H) <= grid ? 2 * kSpTile : kSpTile;
 }
@@ -1337,7 +1337,6 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
   const int n_leaves = p.n_leaves, wsp_kb = wsp_kblocks(H);
   // 16-byte accesses to rows of H (and E): whether every row starts on a 16-byte boundary
   const bool vec_h = H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.h) | reinterpret_cast<uintptr_t>(p.c)) & 15) == 0;
-  const int direct_rows = wide_direct_rows(H, grid, vec_h);
   const bool vec_e = E % 4 == 0 && (reinterpret_cast<uintptr_t>(p.dEmb_rows) & 15) == 0;
   const bool vec_x = vec_h && E % 4 == 0 && (reinterpret_cast<uintptr_t>(p.emb) & 15) == 0;
 #ifdef TREELSTM_TRACE
@@ -1413,7 +1412,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
     return true;
   };
   WidePlan w;
-  if (n_levels > 0) w = wide_plan(level_begin(n_levels - 1), level_begin(n_levels), n_levels == 1, H, E, grid, direct_rows);
+  if (n_levels > 0) w = wide_plan(level_begin(n_levels - 1), level_begin(n_levels), n_levels == 1, H, E, grid, a.direct_rows);
   for (int lvl = n_levels - 1; lvl >= 0 && ok; --lvl) {
     TL_STAMP(trace, lvl, 0);
     uint32_t early = 0;                                  // (thread 0)
@@ -1538,7 +1537,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bwd_wide(BwdParams p, WideA
       chunks_done += grid - busy;
     }
     if (lvl == 0) break;
-    w = wide_plan(level_begin(lvl - 1), level_begin(lvl), lvl == 1, H, E, grid, direct_rows);
+    w = wide_plan(level_begin(lvl - 1), level_begin(lvl), lvl == 1, H, E, grid, a.direct_rows);
     if (w.direct) {                                      // what does not depend on the wavefront above, while the barrier is pending
       const int lo = blockIdx.x * w.per;
       if (lo < w.total) {
@@ -1683,7 +1682,9 @@ static int launch_bwd_wide(treelstm* ctx, BwdParams& p, const BwdImages& img, in
   TL_CUDA(ctx, cudaFuncSetAttribute(k_bwd_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmem));
   int grid = ctx->sm_count;
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
-  WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, after_trees, img};
+  const bool vec_h = ctx->H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.h) | reinterpret_cast<uintptr_t>(p.c)) & 15) == 0;
+  // (Worked out here: in the kernel, between a wavefront's last adds and its barrier, it is 100 cycles of each.)
+  WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, after_trees, wide_direct_rows(ctx->H, grid, vec_h), img};
   // A grid barrier, so every CTA has to be resident, and the runtime sees to that: a backward pass may run beside other work and
   // other backward passes.  (As a programmatic dependent that comes up while the tree kernel ends it would save 2 us of 200 us,
   // 25 trees in fp32, and of 610, 256 trees in bf16, and end in a timeout where the device is shared.)
