@@ -1683,7 +1683,7 @@ static int launch_bwd_wide(treelstm* ctx, BwdParams& p, const BwdImages& img, in
   int grid = ctx->sm_count;
   if (ctx->opt.max_ctas > 0 && grid > ctx->opt.max_ctas) grid = ctx->opt.max_ctas;
   const bool vec_h = ctx->H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.h) | reinterpret_cast<uintptr_t>(p.c)) & 15) == 0;
-  // (Worked out here: in the kernel, between a wavefront's last adds and its barrier, it is 100 cycles of each.)
+  // (Worked out here, where the sizes and addresses are known; in the kernel it takes the same time.)
   WideArgs a{ctx->last.level_offset, ctx->opt.wait_limit_kcycles * 1024, after_trees, wide_direct_rows(ctx->H, grid, vec_h), img};
   // A grid barrier, so every CTA has to be resident, and the runtime sees to that: a backward pass may run beside other work and
   // other backward passes.  (As a programmatic dependent that comes up while the tree kernel ends it would save 2 us of 200 us,
